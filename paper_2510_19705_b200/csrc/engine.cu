@@ -8,12 +8,16 @@
 #include <new>
 #include <vector>
 
+#include "attn_prompt.cuh"
 #include "forward.cuh"
 #include "fwd_persist.cuh"
+#include "gemm_big.cuh"
 #include "gemm_tc.cuh"
 #include "sampling_api.cuh"
 
 using namespace hsd;
+
+#define HSD_TRY(e) do { int st__ = (e); if (st__) return st__; } while (0)
 
 namespace {
 
@@ -24,6 +28,8 @@ constexpr int kMaxSplits = 64;
 constexpr int kTcAttnMinKeys = 2048;           // = the kernel's thresholds for the tensor-memory attention path:
 constexpr int kTcAttnMinVectors = 8;          //   keys of a work item, query vectors of an attention item
 constexpr int kPrefillRows = 128;              // rows of one prompt chunk: the largest pass the one-launch forward takes
+constexpr int kPromptRows = 2304;              // rows of one prompt chunk on the tensor-bound path (forward_prompt): nine 256-row tiles,
+                                               //   which with 4096-wide outputs make 1.95 rounds of the 74 CTA pairs (eight make 1.73)
 constexpr uint32_t kTraceMagic = 0x48534454u;
 
 constexpr size_t kTcCtrlBytes = 16384 + 256;    // status word (first 256 bytes) + per-tile counters
@@ -53,6 +59,7 @@ struct Layout {
   std::vector<int> slots;
   std::vector<ModelLayout> model;
   int max_rows, pages_per_seq, n_pages, max_logit_rows;
+  int base_rows;                                            // rows of the largest pass outside forward_prompt
   size_t ring_slot;
 };
 
@@ -94,6 +101,13 @@ bool valid_models(const hsd_model_desc *ms, int n_levels, const int32_t *T) {
   return true;
 }
 
+// What forward_prompt's kernels take (besides a model on the persistent forward).
+bool prompt_path_dims(const hsd_model_desc *m) {
+  const int page = m->page_size ? m->page_size : 16;
+  return m->dtype == HSD_BF16 && (m->head_dim == 64 || m->head_dim == 128) && m->d_model % 256 == 0 && m->d_ff % kTcBlockK == 0 &&
+         (m->n_q_heads * m->head_dim) % 128 == 0 && (m->n_kv_heads * m->head_dim) % 128 == 0 && page >= 16 && (page & (page - 1)) == 0;
+}
+
 Layout make_layout(const hsd_model_desc *models, int n_models, int n_levels, const int32_t *T) {
   Layout L;
   const hsd_model_desc *m0 = &models[0];
@@ -109,7 +123,10 @@ Layout make_layout(const hsd_model_desc *models, int n_models, int n_levels, con
   if (n_levels == 1) L.slots[0] = 1;
   // rows of one forward: drafts of the level below + catch-up rows (<= n_levels), per sequence
   int decode_rows = B * (sumT + n_levels + 1);
-  L.max_rows = std::max(kPrefillRows, decode_rows);
+  L.base_rows = std::max(kPrefillRows, decode_rows);
+  bool prompt_path = true;
+  for (int mi = 0; mi < n_models; ++mi) prompt_path = prompt_path && prompt_path_dims(&models[mi]);
+  L.max_rows = prompt_path ? (int)std::max<long long>(L.base_rows, std::min<long long>(kPromptRows, (long long)B * m0->max_seq)) : L.base_rows;
   L.pages_per_seq = (m0->max_seq + page - 1) / page;
   L.n_pages = B * L.pages_per_seq;
   size_t off = 0;
@@ -124,7 +141,9 @@ Layout make_layout(const hsd_model_desc *models, int n_models, int n_levels, con
   }
   L.vscratch = take(verify_scratch_bytes(B, sumT + 1));
   L.n_acc = take((size_t)B * 4);
-  L.ring_slot = align_up((size_t)L.max_rows * 40 + (size_t)B * 96 + 1024, 256);
+  // a slot holds one pass's descriptors: <= 40 bytes a row, or a prompt chunk's row lists (8 bytes a row) and one 16-byte
+  // item per 32 rows of a sequence (8 heads to a KV group, at most) and per sequence
+  L.ring_slot = align_up(std::max((size_t)L.base_rows * 40 + (size_t)B * 96, (size_t)L.max_rows * 8 + (size_t)(L.max_rows / 32 + B) * 16) + 1024, 256);
   L.ring = take(L.ring_slot * kRingSlots);
   L.grid_counter = take(256);
   L.model.resize(n_models);
@@ -132,8 +151,8 @@ Layout make_layout(const hsd_model_desc *models, int n_models, int n_levels, con
     const hsd_model_desc *m = &models[mi];
     ModelLayout &M = L.model[mi];
     const int d = m->d_model, hd = m->head_dim, nq = m->n_q_heads, nkv = m->n_kv_heads;
-    M.partial_rows = std::max(L.max_rows + kAttnRows * kAttnBlocksTarget / nkv + kAttnRows * kMaxSplits,
-                              L.max_rows * 20);   // the persistent forward may cut every row's keys into up to 20 splits
+    M.partial_rows = std::max(L.base_rows + kAttnRows * kAttnBlocksTarget / nkv + kAttnRows * kMaxSplits,
+                              L.base_rows * 20);   // the persistent forward may cut every row's keys into up to 20 splits
     M.cos_tab = take((size_t)m->max_seq * (hd / 2) * 4);
     M.sin_tab = take((size_t)m->max_seq * (hd / 2) * 4);
     M.pool_layer_stride = align_up((size_t)L.n_pages * nkv * page * hd * es, 256);
@@ -141,7 +160,7 @@ Layout make_layout(const hsd_model_desc *models, int n_models, int n_levels, con
     M.v_pool = take(M.pool_layer_stride * m->n_layers);
     M.x = take((size_t)L.max_rows * d * 4);
     M.h = take((size_t)L.max_rows * d * es);
-    M.qkv = take((size_t)L.max_rows * (nq + 2 * nkv) * hd * 4);
+    M.qkv = take((size_t)L.base_rows * (nq + 2 * nkv) * hd * 4);
     M.q = take((size_t)L.max_rows * nq * hd * es);
     M.att = take((size_t)L.max_rows * nq * hd * es);
     M.act = take((size_t)L.max_rows * m->d_ff * es);
@@ -194,6 +213,8 @@ struct Model {
   bool use_tc = false, use_persist = false;   // tensor-core GEMMs / the one-launch persistent forward (bf16 models)
   std::vector<CUtensorMap> wmaps;             // [n_layers * 7 + kHeadMaps]: wq wk wv wo wg wu wd per layer, then the levels' heads, the shared head
   CUtensorMap amaps[4][5];                    // activation buffers {h, att, act, hf} x row padding {16, 32, 64, 128, 256}
+  bool use_prompt = false;                    // long prompts run forward_prompt
+  std::vector<CUtensorMap> kvmaps;            // [n_layers][2]: K and V pools of each layer, for the prompt attention
   CUtensorMap amaps_rows[4][16];              // the same buffers with a box of exactly 1..16 rows (persistent forward, few rows)
 };
 
@@ -370,7 +391,7 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     if (st) return st;
   }
   if (R == 0) return HSD_OK;
-  if (R > L.max_rows) return HSD_E_INVALID_ARG;
+  if (R > L.base_rows) return HSD_E_INVALID_ARG;
   char *host, *devp;
   int st = ring_acquire(c, &host, &devp);
   if (st) return st;
@@ -572,7 +593,6 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
   void *h = c->dev<void>(ML.h), *q = c->dev<void>(ML.q), *att = c->dev<void>(ML.att), *act = c->dev<void>(ML.act);
   float *qkv = c->dev<float>(ML.qkv);
   const int *pt = c->dev<int>(L.page_table);
-#define HSD_TRY(e) do { int st__ = (e); if (st__) return st__; } while (0)
   HSD_TRY(launch_embed(md, M.embed, c->dev<int>(L.tokens), rb, x, s));
   for (int l = 0; l < c->exits[level]; ++l) {
     const void *const *w = &M.lw[(size_t)l * 9];
@@ -612,6 +632,88 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
   c->stats[level].forwards++;
   c->stats[level].rows += R;
   mark_valid();
+  return HSD_OK;
+}
+
+// A prompt chunk of many rows (no logits): one launch per operation, every projection a tensor-bound GEMM over all rows
+// (weights read once per chunk instead of once per 128 rows) with its finish in the epilogue, attention on tensor memory.
+// The chunk only fills the cache, so the last layer ends with its keys and values.
+int forward_prompt(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
+  Model &M = c->model_of(level);
+  const ModelDims &md = M.md;
+  const Layout &L = c->lay;
+  const ModelLayout &ML = M.lay;
+  const int tokens2 = 2 * prompt_attn_tokens(md.nq / md.nkv);       // tokens of one attention item
+  int R = 0, n_items = 0;
+  for (const SeqWork &w : work) {
+    const int rows = w.end - w.start;
+    if (rows <= 0 || w.start < 0 || w.end > md.max_seq || w.logit_first >= 0) return HSD_E_INVALID_ARG;
+    R += rows;
+    n_items += (rows + tokens2 - 1) / tokens2;
+    HSD_TRY(ensure_pages(c, w.b, w.end));
+  }
+  if (R == 0) return HSD_OK;
+  if (R > L.max_rows) return HSD_E_INVALID_ARG;
+  char *host, *devp;
+  HSD_TRY(ring_acquire(c, &host, &devp));
+  const size_t o_pos = align_up((size_t)R * 4, 16), o_items = align_up(o_pos + (size_t)R * 4, 16), bytes = o_items + (size_t)n_items * 16;
+  if (bytes > L.ring_slot) return HSD_E_INVALID_ARG;
+  int *row_seq = (int *)host, *row_pos = (int *)(host + o_pos);
+  int4 *items = (int4 *)(host + o_items);
+  int r = 0, ii = 0;
+  for (const SeqWork &w : work) {
+    for (int p = w.start; p < w.end; p += tokens2) items[ii++] = make_int4(r + (p - w.start), std::min(tokens2, w.end - p), w.b, p);
+    for (int p = w.start; p < w.end; ++p, ++r) { row_seq[r] = w.b; row_pos[r] = p; }
+  }
+  std::stable_sort(items, items + n_items, [](const int4 &x, const int4 &y) { return x.w + x.y > y.w + y.y; });   // longest key range first
+  HSD_CUDA_OK(cudaMemcpyAsync(devp, host, bytes, cudaMemcpyHostToDevice, c->stream));
+  HSD_TRY(upload_page_tables(c));
+  RowBatch rb = {};
+  rb.R = R; rb.row_seq = (const int *)devp; rb.row_pos = (const int *)(devp + o_pos);
+  cudaStream_t s = c->stream;
+  float *x = c->dev<float>(ML.x);
+  void *h = c->dev<void>(ML.h);
+  BigGemmArgs g = {};
+  g.R = R;
+  g.row_seq = rb.row_seq; g.row_pos = rb.row_pos; g.page_table = c->dev<int>(L.page_table);
+  g.cos_tab = c->dev<float>(ML.cos_tab); g.sin_tab = c->dev<float>(ML.sin_tab);
+  g.q = c->dev<__nv_bfloat16>(ML.q);
+  g.nq = md.nq; g.nkv = md.nkv; g.hd = md.hd; g.page = md.page; g.pages_per_seq = md.pages_per_seq; g.n_pages = md.n_pages;
+  g.status = (int *)(c->ws + c->status_off);
+  PromptAttnArgs pa = {};
+  pa.q = g.q; pa.att = c->dev<__nv_bfloat16>(ML.att);
+  pa.items = (const int4 *)(devp + o_items); pa.n_items = n_items; pa.page_table = g.page_table;
+  pa.nq = md.nq; pa.nkv = md.nkv; pa.hd = md.hd; pa.pages_per_seq = md.pages_per_seq; pa.n_pages = md.n_pages;
+  while ((1 << pa.page_shift) < md.page) ++pa.page_shift;
+  pa.status = g.status;
+  auto product = [&](int abuf, int K, int wmap0, int n_maps, int mode, int n, void *out, int ldo) {
+    g.a = M.amaps[abuf][3];
+    for (int i = 0; i < n_maps; ++i) g.w[i] = M.wmaps[(size_t)wmap0 + i];
+    g.mode = mode; g.K = K; g.seg_n[0] = n; g.ldo = ldo;
+    g.out_f32 = (float *)out; g.out_bf16 = (__nv_bfloat16 *)out;
+    return launch_gemm_big(g, c->sm_count, s);
+  };
+  HSD_TRY(launch_embed(md, M.embed, c->dev<int>(L.tokens), rb, x, s));
+  const int nqd = md.nq * md.hd, nkvd = md.nkv * md.hd, n_run = c->exits[level];
+  for (int l = 0; l < n_run; ++l) {
+    const void *const *w = &M.lw[(size_t)l * 9];
+    const bool last = l == n_run - 1;
+    HSD_TRY(launch_rmsnorm(md, x, w[0], nullptr, R, h, s));
+    g.k_pool = (__nv_bfloat16 *)(c->ws + ML.k_pool + ML.pool_layer_stride * l);
+    g.v_pool = (__nv_bfloat16 *)(c->ws + ML.v_pool + ML.pool_layer_stride * l);
+    g.seg_n[1] = g.seg_n[2] = nkvd;
+    g.skip_cols = last ? nqd / 256 * 256 : 0;
+    HSD_TRY(product(0, md.d, l * 7, 3, BIG_QKV, nqd, nullptr, 0));
+    if (last) break;
+    pa.k = M.kvmaps[2 * l]; pa.v = M.kvmaps[2 * l + 1];
+    HSD_TRY(launch_prompt_attention(pa, s));
+    HSD_TRY(product(1, nqd, l * 7 + 3, 1, BIG_ADD_F32, md.d, x, md.d));
+    HSD_TRY(launch_rmsnorm(md, x, w[5], nullptr, R, h, s));
+    HSD_TRY(product(0, md.d, l * 7 + 4, 2, BIG_SWIGLU, md.ff, c->dev<void>(ML.act), md.ff));
+    HSD_TRY(product(2, md.ff, l * 7 + 6, 1, BIG_ADD_F32, md.d, x, md.d));
+  }
+  for (const SeqWork &w : work)
+    for (int k = c->shared_cache ? 0 : level; k <= level; ++k) c->len_g[w.b][k] = w.end;
   return HSD_OK;
 }
 
@@ -782,9 +884,12 @@ int prefill(hsd_ctx *c, int batch, int prompt_len) {
   const int K = c->n_levels - 1;
   int end = prompt_len - 1;
   std::vector<int> done(batch, 0);
+  bool prompt_path = true;
+  for (const Model &M : c->models) prompt_path = prompt_path && M.use_prompt;
   for (;;) {
     std::vector<SeqWork> work;
-    int budget = kPrefillRows;
+    int budget = prompt_path ? c->lay.max_rows : kPrefillRows;
+    const int budget0 = budget;
     for (int b = 0; b < batch && budget > 0; ++b) {
       if (done[b] >= end) continue;
       int rows = std::min(budget, end - done[b]);
@@ -794,7 +899,8 @@ int prefill(hsd_ctx *c, int batch, int prompt_len) {
     }
     if (work.empty()) break;
     // early exits: the target's pass fills the one cache; separate models: each fills its own
-    for (int lvl = c->shared_cache ? K : 0; lvl <= K; ++lvl) HSD_TRY(forward(c, lvl, work));
+    for (int lvl = c->shared_cache ? K : 0; lvl <= K; ++lvl)
+      HSD_TRY(budget0 - budget > kPrefillRows ? forward_prompt(c, lvl, work) : forward(c, lvl, work));
   }
   return HSD_OK;
 }
@@ -863,7 +969,16 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   M.use_persist = coop != 0 && fwd_persist_supported(md.hd, md.nq / md.nkv) && md.d % 256 == 0 && md.d <= 4096 &&
                   (md.d / kTcBlockM) * 2 <= c->sm_count && md.n_layers <= 64 && (md.page & (md.page - 1)) == 0 && md.page >= 16;
-  return HSD_OK;
+  M.use_prompt = M.use_persist && prompt_path_dims(model) && lay.max_rows > kPrefillRows;
+  if (M.use_prompt) {
+    M.kvmaps.resize((size_t)md.n_layers * 2);
+    const long long rows = (long long)md.nkv * md.n_pages * md.page;
+    for (int l = 0; l < md.n_layers && !st; ++l) {
+      st = prompt_attn_map(&M.kvmaps[2 * l], ld[l].k_pool, rows, md.hd);
+      if (!st) st = prompt_attn_map(&M.kvmaps[2 * l + 1], ld[l].v_pool, rows, md.hd);
+    }
+  }
+  return st;
 }
 
 bool supported_dims(const hsd_model_desc *model) {
@@ -1052,7 +1167,7 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
   const ModelDims &md = M.md;
   const Layout &L = c->lay;
   const ModelLayout &ML = M.lay;
-  if (n_tokens > L.max_rows || n_tokens > md.max_seq || n_tokens > 128) return HSD_E_INVALID_ARG;
+  if (n_tokens > L.base_rows || n_tokens > md.max_seq || n_tokens > 128) return HSD_E_INVALID_ARG;
   for (int i = 0; i < n_layers_sel; ++i)
     if (layers[i] < 1 || layers[i] > md.n_layers || (i > 0 && layers[i] <= layers[i - 1])) return HSD_E_INVALID_ARG;
   c->stream = (cudaStream_t)stream;

@@ -37,6 +37,40 @@ __global__ void rmsnorm_kernel(const float *__restrict__ x, const T *__restrict_
   for (int k = threadIdx.x; k < d; k += blockDim.x) out[(size_t)i * d + k] = from_f32<T>(row[k] * inv * to_f32(gain[k]));
 }
 
+// bf16 rows of d = 4 x 256 x NV values or fewer: a row stays in registers between the two passes, 16-byte loads.
+template <int NV>
+__global__ void __launch_bounds__(256) rmsnorm_vec_kernel(const float *__restrict__ x, const __nv_bfloat16 *__restrict__ gain,
+                                                          const int *__restrict__ src, int d, float eps, __nv_bfloat16 *__restrict__ out) {
+  __shared__ float sh[8];
+  const int i = blockIdx.x, n4 = d >> 2;
+  const float4 *row = reinterpret_cast<const float4 *>(x + (size_t)(src ? src[i] : i) * d);
+  float4 v[NV];
+  float ss = 0.f;
+#pragma unroll
+  for (int j = 0; j < NV; ++j) {
+    const int k = threadIdx.x + 256 * j;
+    v[j] = k < n4 ? __ldcg(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+#pragma unroll
+  for (int j = 0; j < NV; ++j) ss += (v[j].x * v[j].x + v[j].y * v[j].y) + (v[j].z * v[j].z + v[j].w * v[j].w);
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) tot += sh[w];
+  const float inv = rsqrtf(tot / (float)d + eps);
+#pragma unroll
+  for (int j = 0; j < NV; ++j) {
+    const int k = threadIdx.x + 256 * j;
+    if (k >= n4) continue;
+    const uint2 graw = __ldg(reinterpret_cast<const uint2 *>(gain) + k);
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v[j].x * inv * __uint_as_float(graw.x << 16), v[j].y * inv * __uint_as_float(graw.x & 0xFFFF0000u));
+    const __nv_bfloat162 b = __floats2bfloat162_rn(v[j].z * inv * __uint_as_float(graw.y << 16), v[j].w * inv * __uint_as_float(graw.y & 0xFFFF0000u));
+    reinterpret_cast<uint2 *>(out + (size_t)i * d)[k] = make_uint2(*reinterpret_cast<const unsigned *>(&a), *reinterpret_cast<const unsigned *>(&b));
+  }
+}
+
 // ------------------------------------------------------------------------------ SIMT skinny GEMM
 // Each warp owns CPW output columns and streams their weight rows once with 16-byte loads; the
 // activation rows are staged through shared memory in K-chunks.  acc[r][c] in fp32.
@@ -385,7 +419,15 @@ int launch_embed(const ModelDims &md, const void *embed, const int *tokens, cons
 
 int launch_rmsnorm(const ModelDims &md, const float *x, const void *gain, const int *src, int rows, void *out, cudaStream_t s) {
   if (rows == 0) return HSD_OK;
-  if (md.dtype == HSD_BF16)
+  // the vector form wants 8-byte-aligned gains and rows it can hold: 2 / 4 / 8 float4 per thread
+  const bool vec = md.dtype == HSD_BF16 && md.d % 4 == 0 && md.d <= 8192 && ((uintptr_t)gain & 7) == 0 && ((uintptr_t)out & 7) == 0 &&
+                   ((uintptr_t)x & 15) == 0;
+  if (vec) {
+    const __nv_bfloat16 *g = (const __nv_bfloat16 *)gain;
+    if (md.d <= 2048) rmsnorm_vec_kernel<2><<<rows, 256, 0, s>>>(x, g, src, md.d, md.eps, (__nv_bfloat16 *)out);
+    else if (md.d <= 4096) rmsnorm_vec_kernel<4><<<rows, 256, 0, s>>>(x, g, src, md.d, md.eps, (__nv_bfloat16 *)out);
+    else rmsnorm_vec_kernel<8><<<rows, 256, 0, s>>>(x, g, src, md.d, md.eps, (__nv_bfloat16 *)out);
+  } else if (md.dtype == HSD_BF16)
     rmsnorm_kernel<__nv_bfloat16><<<rows, 256, 0, s>>>(x, (const __nv_bfloat16 *)gain, src, md.d, md.eps, (__nv_bfloat16 *)out);
   else
     rmsnorm_kernel<float><<<rows, 256, 0, s>>>(x, (const float *)gain, src, md.d, md.eps, (float *)out);

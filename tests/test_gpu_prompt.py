@@ -1,0 +1,54 @@
+"""Long prompts: the many-row chunk path (tensor-bound GEMMs on CTA pairs, attention on tensor memory) against the
+oracle, at the sizes where its tiles, items, pages and chunks end."""
+import os
+import tempfile
+
+import numpy as np
+import pytest
+import torch
+
+from oracle.transformer import Transformer
+from paper_2510_19705_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+
+# head size, query heads, KV heads, page, batch, prompt length.  Rows of a chunk = prompt - 1 per sequence.
+CASES = [
+    (128, 4, 1, 16, 1, 130),       # 129 rows: the shortest chunk of this path, one row in the second A half
+    (128, 4, 1, 16, 1, 257),       # 256 rows: exactly one token tile
+    (128, 4, 1, 32, 3, 150),       # several sequences in one chunk, items that end inside a tile
+    (128, 8, 8, 16, 2, 300),       # no grouped heads: 128 tokens per query tile
+    (128, 8, 1, 64, 1, 210),       # eight heads to a group
+    (128, 6, 2, 16, 1, 345),       # group of three: two rows of every query tile unused
+    (64, 8, 4, 16, 1, 391),        # head size 64: two heads per accumulator half
+    (64, 4, 2, 32, 2, 1300),       # 2598 rows: two chunks, the second starting inside a sequence
+    (128, 4, 1, 16, 1, 2433),      # 2432 rows: a full chunk and 128 rows left for the one-launch pass
+]
+
+
+@pytest.mark.parametrize("hd,nq,nkv,page,batch,prompt", CASES)
+def test_prompt_chunks_match_oracle(hd, nq, nkv, page, batch, prompt):
+    # 704 = 11 x 64 feed-forward columns: a half-empty last gate / up tile
+    cfg = inputs.model_cfg(3, 256, nq, nkv, 704, 1024, "bf16", head_dim=hd)
+    w = inputs.make_weights(cfg, 11)
+    for layer in w["layers"]:          # scores of unit size: the softmax is not flat
+        layer["wq"].mul_(3.0)
+        layer["wk"].mul_(3.0)
+    w_gpu = {k: (v.cuda() if k != "layers" else [{a: t.cuda() for a, t in l.items()} for l in v]) for k, v in w.items()}
+    prompts = inputs.make_prompts(cfg["vocab"], batch, prompt, 3)
+    eng = binding.Hsd(cfg, w_gpu, (1, 3), (2,), max_batch=batch, max_seq=prompt + 32, page_size=page)
+    with tempfile.TemporaryDirectory() as tmp:
+        path = os.path.join(tmp, "trace.bin")
+        eng.set_trace(path, logit_calls=2 * batch)
+        eng.generate(prompts.cuda(), 2, 5)
+        eng.set_trace(None)
+        recs = binding.read_trace(path)
+    eng.close()
+    om = Transformer(cfg, inputs.weights_to_numpy(w), (1, 3))
+    for b in range(batch):
+        rec = next(r for r in recs if r["level"] == 1 and r["seq"] == b)
+        om.reset()
+        om.rows(1, prompts[b].tolist(), rec["tokens"][:-1].tolist())
+        # the bound of the other bf16 parity tests: 2e-2 on logits of standard deviation 0.02 sqrt(256) = 0.32
+        err = float(np.abs(om.last_logits64 - rec["logits"]).max())
+        assert err < 2e-2, (b, err)
