@@ -2,13 +2,13 @@
 // under every verifier j; Section 2: alpha = 1 - TV(p_i, p_j) = sum_x min(p_i(x), p_j(x))).  Given the logits of
 // L models (exit layers) at the same R positions, the kernels below produce the L x L matrix of the rates
 // averaged over the positions.
-//   1. alpha_stats_kernel:   per (model, position): row maximum and sum of exp (fp32, fixed reduction order)
-//   2. alpha_pairs_kernel:   per (position, 1024-token chunk): the L probabilities of the chunk in shared
-//                            memory, every pair's sum of minima over the chunk -> one partial per pair
-//   3. alpha_reduce_kernel:  per pair: the partials of all positions and chunks added in fixed order in fp64
+//   1. alpha_stats_kernel:   per (model, position): reference exponent and sum of exp (fp32, fixed order, one read of the row)
+//   2. alpha_pairs_kernel:   per (position, <= 4096-token unit): every pair's sum of minima over the unit -> one partial per pair
+//   3. alpha_reduce_kernel:  per pair: the partials of all positions and units added in fixed order in fp64
 // Deterministic (no atomics).  Model pairs are enumerated i < j, pair index = i L - i (i + 1) / 2 + (j - i - 1).
 #include <cuda_bf16.h>
 #include <math.h>
+#include <type_traits>
 
 #include "../../include/hsd.h"
 #include "common.cuh"
@@ -17,73 +17,261 @@ namespace hsd {
 namespace {
 
 constexpr int kAlphaThreads = 256;
-constexpr int kAlphaChunk = 1024;      // tokens per block of the pair kernel
+constexpr int kAlphaTile = 256;        // tokens staged at a time
+constexpr int kAlphaUnit = 4096;       // tokens per partial at most: 128 per lane, all added in fp32
 constexpr int kAlphaMaxModels = 32;
+constexpr int kAlphaStride = kAlphaTile + 8;   // floats between the models of a staged tile
 
-template <typename T>
+template <typename T> struct AlphaVec;         // 16 bytes of logits
+template <> struct AlphaVec<__nv_bfloat16> {
+  static constexpr int N = 8;
+  __device__ static void unpack(const uint4 &v, float *f) {
+    f[0] = __uint_as_float(v.x << 16); f[1] = __uint_as_float(v.x & 0xFFFF0000u);
+    f[2] = __uint_as_float(v.y << 16); f[3] = __uint_as_float(v.y & 0xFFFF0000u);
+    f[4] = __uint_as_float(v.z << 16); f[5] = __uint_as_float(v.z & 0xFFFF0000u);
+    f[6] = __uint_as_float(v.w << 16); f[7] = __uint_as_float(v.w & 0xFFFF0000u);
+  }
+};
+template <> struct AlphaVec<float> {
+  static constexpr int N = 4;
+  __device__ static void unpack(const uint4 &v, float *f) {
+    f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y); f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
+  }
+};
+
+constexpr float kLog2e = 1.4426950408889634f;
+__device__ __forceinline__ float alpha_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// Weight of a logit relative to 2^n, n a whole number: exp(x) 2^-n.  Numerators and sums use the same expression, so
+// the approximation's own bias cancels in their quotient.
+__device__ __forceinline__ float alpha_weight(float x, float n) { return alpha_ex2(fmaf(x, kLog2e, -n)); }
+
+// Online sum of exp of a thread, relative to 2^n with 2^n at or above the largest exp so far: a larger n rescales the
+// sum by a power of two, exactly.
+struct RefSum {
+  float n = -INFINITY, s = 0.f;
+  __device__ void raise(float n2) {
+    if (n2 > n) {
+      s *= n > -INFINITY ? __int_as_float((int)(fmaxf(n - n2, -126.f) + 127.f) << 23) : 0.f;
+      n = n2;
+    }
+  }
+  __device__ void merge(float n2, float s2) {
+    RefSum o;
+    o.n = n2; o.s = s2;
+    const float nn = fmaxf(n, n2);
+    raise(nn);
+    o.raise(nn);
+    s += o.s;
+  }
+};
+
+// Bound by HBM: 16-byte loads when VEC (rows on 16-byte boundaries), four in flight per thread.
+template <typename T, bool VEC>
 __global__ void __launch_bounds__(kAlphaThreads)
 alpha_stats_kernel(const T *__restrict__ logits, long long model_stride, int R, int V, float2 *__restrict__ stats) {
-  __shared__ float sh[kAlphaThreads / 32];
+  __shared__ float shm[kAlphaThreads / 32], shs[kAlphaThreads / 32];
   const int r = blockIdx.x, l = blockIdx.y;
   const T *row = logits + (size_t)l * model_stride + (size_t)r * V;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float m = -INFINITY;
-  for (int k = threadIdx.x; k < V; k += kAlphaThreads) m = fmaxf(m, to_f32(row[k]));
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-  if (lane == 0) sh[warp] = m;
-  __syncthreads();
-  m = sh[0];
-  for (int w = 1; w < kAlphaThreads / 32; ++w) m = fmaxf(m, sh[w]);
-  __syncthreads();
-  float s = 0.f;
-  for (int k = threadIdx.x; k < V; k += kAlphaThreads) s += __expf(to_f32(row[k]) - m);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-  if (lane == 0) sh[warp] = s;
+  constexpr int N = VEC ? AlphaVec<T>::N : 1, U = 4;
+  RefSum ms;
+  const int nv = V / N;
+  for (int k0 = threadIdx.x; k0 < nv; k0 += kAlphaThreads * U) {
+    float f[U][N];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = k0 + u * kAlphaThreads;
+#pragma unroll
+      for (int e = 0; e < N; ++e) f[u][e] = -INFINITY;
+      if (k < nv) {
+        if constexpr (VEC) AlphaVec<T>::unpack(__ldg(reinterpret_cast<const uint4 *>(row) + k), f[u]);
+        else f[u][0] = to_f32(row[k]);
+      }
+    }
+    float mx = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < N; ++e) mx = fmaxf(mx, f[u][e]);
+    ms.raise(ceilf(mx * kLog2e));
+    if (ms.n > -INFINITY) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int e = 0; e < N; ++e) ms.s += alpha_weight(f[u][e], ms.n);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) ms.merge(__shfl_xor_sync(0xFFFFFFFFu, ms.n, o), __shfl_xor_sync(0xFFFFFFFFu, ms.s, o));
+  if (lane == 0) { shm[warp] = ms.n; shs[warp] = ms.s; }
   __syncthreads();
   if (threadIdx.x == 0) {
-    float tot = 0.f;
-    for (int w = 0; w < kAlphaThreads / 32; ++w) tot += sh[w];
-    stats[(size_t)l * R + r] = make_float2(m, tot);
+    RefSum t;
+    for (int w = 0; w < kAlphaThreads / 32; ++w) t.merge(shm[w], shs[w]);
+    stats[(size_t)l * R + r] = make_float2(t.n, t.s);
   }
 }
 
-// grid (R, n_chunks).  Shared memory: prob[chunk token][L] (model index fastest: lanes that work on different
-// pairs read different banks or the same word), then per-warp partials [8][n_pairs].
-template <typename T>
-__global__ void __launch_bounds__(kAlphaThreads)
-alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, int R, int V,
+// Sum over the lanes of 64 values per lane: lane i returns the sums of values 2 i and 2 i + 1 (fixed order).
+__device__ __forceinline__ float2 warp_sum64(float *v, int lane) {
+  // each step halves the values: a lane keeps the half its bit selects and gives the other to its partner
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < 2 * o; ++i) {
+      const float keep = up ? v[2 * o + i] : v[i], give = up ? v[i] : v[2 * o + i];
+      v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+    }
+  }
+  return make_float2(v[0], v[1]);
+}
+__device__ __forceinline__ int pair_index(int i, int j, int L) { return i * L - i * (i + 1) / 2 + (j - i - 1); }
+
+// Sums of minima of a block of eight models against another (KIND 0), or of the pairs i < j of one block (KIND 1, 2),
+// over the lane's tokens of one staged tile.  acc[i][jj] = the pairs (i, 2 jj) and (i, 2 jj + 1).  A diagonal block uses
+// the entries i <= 2 jj; a second one (KIND 2) is kept in the other half, entry (i, jj) at [7 - i][3 - jj].
+// Bound by instruction issue: a minimum per pair and token, one packed add per two pairs; 16 shared-memory loads feed
+// 64 pairs.
+template <int KIND>
+__device__ __forceinline__ void alpha_block(const float *pi, const float *pj, int step, float2 (*acc)[4]) {
+  for (int k = 0; k < kAlphaTile; k += step) {
+    float a[8], b[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) a[i] = pi[i * kAlphaStride + k];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) b[j] = KIND ? a[j] : pj[j * kAlphaStride + k];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj) {
+        if (KIND && i > 2 * jj) continue;
+        float2 &to = KIND == 2 ? acc[7 - i][3 - jj] : acc[i][jj];
+        to = __fadd2_rn(to, make_float2(fminf(a[i], b[2 * jj]), fminf(a[i], b[2 * jj + 1])));
+      }
+  }
+}
+
+// grid (units, R).  The unit's tokens go through shared memory 256 at a time as probabilities [model][token]
+// (double-buffered: the next tile's logits are fetched under this tile's minima).  A warp owns one pair of 8-model
+// blocks, or two diagonal blocks (about as much work), and the tokens lane + 32 slice, ...; with fewer blocks than
+// warps the warps share a pair and split the tokens.
+// 32 models x 256 positions x 32000 tokens: 478 us here + 97 us of statistics; one pair per lane, two shared-memory loads
+// per pair and token, took 5021 + 176 us.
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(kAlphaThreads, 2)
+alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, int R, int V, int unit,
                    const float2 *__restrict__ stats, float *__restrict__ partials) {
   extern __shared__ float sm[];
-  const int r = blockIdx.x, chunk = blockIdx.y, n_chunks = gridDim.y;
-  const int v0 = chunk * kAlphaChunk, nv = min(kAlphaChunk, V - v0);
+  __shared__ float2 st[kAlphaMaxModels];
+  const int r = blockIdx.y, u0 = blockIdx.x * unit, nt = min(unit, V - u0);
+  const int nb = (L + 7) >> 3, lpad = nb * 8, n_off = nb * (nb - 1) / 2, n_task = n_off + (nb + 1) / 2;
+  const int slices = max(1, 8 / n_task);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float *buf[2] = {sm, sm + (size_t)lpad * kAlphaStride};
+  float *wsum = sm + 2 * (size_t)lpad * kAlphaStride;                 // [slice][task][64]
   const int n_pairs = L * (L - 1) / 2;
-  float *prob = sm;                                   // [kAlphaChunk][L]
-  float *wpart = sm + (size_t)kAlphaChunk * L;        // [8][n_pairs]
-  for (int idx = threadIdx.x; idx < L * kAlphaChunk; idx += kAlphaThreads) {
-    const int l = idx / kAlphaChunk, k = idx - l * kAlphaChunk;      // consecutive threads: consecutive tokens of one model
-    float p = 0.f;
-    if (k < nv) {
-      const float2 st = stats[(size_t)l * R + r];
-      p = __expf(to_f32(logits[(size_t)l * model_stride + (size_t)r * V + v0 + k]) - st.x) / st.y;
+  if (tid < lpad) {
+    const float2 v = tid < L ? stats[(size_t)tid * R + r] : make_float2(0.f, 0.f);
+    st[tid] = make_float2(v.x, tid < L ? 1.f / v.y : 0.f);
+  }
+  __syncthreads();
+  // staging: 8 threads per model, 32 models at a time; vector i of a thread = tokens (8 i + tid % 8) N ..
+  constexpr int N = VEC ? AlphaVec<T>::N : 1, NV = kAlphaTile / 8 / N;
+  const int sm_model = tid >> 3, sv = tid & 7;
+  const bool stager = sm_model < lpad, in_use = sm_model < L;
+  const T *row = logits + (size_t)(in_use ? sm_model : 0) * model_stride + (size_t)r * V + u0;
+  typename std::conditional<VEC, uint4, T>::type raw[NV];
+  auto fetch = [&](int t0) {
+    if (!in_use) return;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int k = t0 + (8 * i + sv) * N;
+      if (k < nt) {
+        if constexpr (VEC) raw[i] = __ldg(reinterpret_cast<const uint4 *>(row + k));
+        else raw[i] = row[k];
+      }
     }
-    prob[(size_t)k * L + l] = p;
-  }
+  };
+  auto convert = [&](int t0, float *dst) {
+    if (!stager) return;
+    const float n = st[sm_model].x, inv = st[sm_model].y;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int at = (8 * i + sv) * N;
+      float f[N];
+#pragma unroll
+      for (int e = 0; e < N; ++e) f[e] = 0.f;
+      if (in_use && t0 + at < nt) {
+        if constexpr (VEC) AlphaVec<T>::unpack(raw[i], f);
+        else f[0] = to_f32(raw[i]);
+#pragma unroll
+        for (int e = 0; e < N; ++e) f[e] = alpha_weight(f[e], n) * inv;
+      }
+      float *d = dst + sm_model * kAlphaStride + at;
+      if constexpr (VEC) {
+#pragma unroll
+        for (int e = 0; e < N; e += 4) *reinterpret_cast<float4 *>(d + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
+      } else d[0] = f[0];
+    }
+  };
+  // this warp's task
+  const int task = warp % n_task, slice = warp / n_task;
+  const bool busy = slice < slices;
+  int bi = 0, bj = 0;
+  const bool diag = task >= n_off;
+  if (diag) { bi = 2 * (task - n_off); bj = bi + 1; }                // two diagonal blocks (the second may not exist)
+  else { int t = task; while (t >= nb - 1 - bi) { t -= nb - 1 - bi; ++bi; } bj = bi + 1 + t; }
+  const bool two = bj < nb;
+  float2 acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  fetch(0);
+  convert(0, buf[0]);
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int k0 = warp * (kAlphaChunk / 8);            // this warp's 128 tokens
-  for (int pr = lane; pr < n_pairs; pr += 32) {
-    int i = 0, rem = pr;                              // pair index -> (i, j)
-    while (rem >= L - 1 - i) { rem -= L - 1 - i; ++i; }
-    const int j = i + 1 + rem;
-    float s = 0.f;
-    for (int k = k0; k < k0 + kAlphaChunk / 8; ++k) s += fminf(prob[(size_t)k * L + i], prob[(size_t)k * L + j]);
-    wpart[warp * n_pairs + pr] = s;
+  for (int t0 = 0, b = 0; t0 < nt; t0 += kAlphaTile, b ^= 1) {
+    const bool more = t0 + kAlphaTile < nt;
+    if (more) fetch(t0 + kAlphaTile);
+    if (busy) {
+      const float *p = buf[b] + slice * 32 + lane;
+      if (!diag) alpha_block<0>(p + bi * 8 * kAlphaStride, p + bj * 8 * kAlphaStride, 32 * slices, acc);
+      else {
+        alpha_block<1>(p + bi * 8 * kAlphaStride, nullptr, 32 * slices, acc);
+        if (two) alpha_block<2>(p + bj * 8 * kAlphaStride, nullptr, 32 * slices, acc);
+      }
+    }
+    if (more) convert(t0 + kAlphaTile, buf[b ^ 1]);
+    __syncthreads();
   }
+  // lane sums; the slices of a task are added in slice order
+  float *out = partials + ((size_t)r * gridDim.x + blockIdx.x) * n_pairs;
+  float v[64];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { v[i * 8 + 2 * j] = acc[i][j].x; v[i * 8 + 2 * j + 1] = acc[i][j].y; }
+  const float2 lane_sum = warp_sum64(v, lane);
+  if (busy) *reinterpret_cast<float2 *>(wsum + (slice * n_task + task) * 64 + 2 * lane) = lane_sum;
   __syncthreads();
-  for (int pr = threadIdx.x; pr < n_pairs; pr += kAlphaThreads) {
-    float s = 0.f;
-    for (int w = 0; w < 8; ++w) s += wpart[w * n_pairs + pr];
-    partials[((size_t)r * n_chunks + chunk) * n_pairs + pr] = s;
+  if (!busy || slice != 0) return;
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const int ai = lane / 4, ajj = lane % 4;                          // the accumulator entry of values 2 lane, 2 lane + 1
+    int ib = bi, jb = bj, i = ai, j = 2 * ajj + e;
+    if (diag) {
+      if (ai <= 2 * ajj) jb = bi;
+      else { if (!two) continue; ib = bj; i = 7 - ai; j = 2 * (3 - ajj) + e; }
+    }
+    i += ib * 8; j += jb * 8;
+    if (i >= j || j >= L) continue;
+    float t = 0.f;
+    for (int sl = 0; sl < slices; ++sl) t += wsum[(sl * n_task + task) * 64 + 2 * lane + e];
+    out[pair_index(i, j, L)] = t;
   }
 }
 
@@ -113,37 +301,49 @@ alpha_reduce_kernel(const float *__restrict__ partials, int L, int n_blocks, int
   if (blockIdx.x == 0 && (int)threadIdx.x < L) alpha[(size_t)threadIdx.x * L + threadIdx.x] = 1.0;
 }
 
-struct AlphaPlan { int n_chunks, n_pairs; size_t stats_off, partials_off, total; };
+struct AlphaPlan { int unit, n_units, n_pairs; size_t stats_off, partials_off, total; };
 AlphaPlan alpha_plan(int L, int R, int V) {
   AlphaPlan p;
-  p.n_chunks = (V + kAlphaChunk - 1) / kAlphaChunk;
+  // equal units of a multiple of the tile; shorter ones when the positions alone would not fill the SMs
+  int n = (V + kAlphaUnit - 1) / kAlphaUnit;
+  while ((long long)n * R < 148 * 4 && (V + n - 1) / n > 2 * kAlphaTile) n *= 2;
+  p.unit = ((V + n - 1) / n + kAlphaTile - 1) / kAlphaTile * kAlphaTile;
+  p.n_units = (V + p.unit - 1) / p.unit;
   p.n_pairs = L * (L - 1) / 2;
   p.stats_off = 0;
   p.partials_off = ((size_t)L * R * sizeof(float2) + 255) / 256 * 256;
-  p.total = p.partials_off + (size_t)R * p.n_chunks * (p.n_pairs > 0 ? p.n_pairs : 1) * sizeof(float);
+  p.total = p.partials_off + (size_t)R * p.n_units * (p.n_pairs > 0 ? p.n_pairs : 1) * sizeof(float);
   return p;
+}
+
+template <typename T, bool VEC>
+int launch_alpha_t(const void *logits, long long model_stride, int L, int R, int V, void *ws, double *alpha, cudaStream_t s) {
+  const AlphaPlan p = alpha_plan(L, R, V);
+  float2 *stats = (float2 *)((char *)ws + p.stats_off);
+  float *partials = (float *)((char *)ws + p.partials_off);
+  alpha_stats_kernel<T, VEC><<<dim3(R, L), kAlphaThreads, 0, s>>>((const T *)logits, model_stride, R, V, stats);
+  if (p.n_pairs > 0) {
+    const int lpad = (L + 7) / 8 * 8;
+    const size_t smem = (2 * (size_t)lpad * kAlphaStride + 8 * 64) * sizeof(float);
+    static bool attr_set = false;
+    if (!attr_set) {
+      if (cudaFuncSetAttribute(alpha_pairs_kernel<T, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) != cudaSuccess) return HSD_E_CUDA;
+      attr_set = true;
+    }
+    alpha_pairs_kernel<T, VEC><<<dim3(p.n_units, R), kAlphaThreads, smem, s>>>((const T *)logits, model_stride, L, R, V, p.unit, stats, partials);
+  }
+  alpha_reduce_kernel<<<p.n_pairs > 0 ? min(p.n_pairs, 592) : 1, kAlphaThreads, 0, s>>>(partials, L, R * p.n_units, R, alpha);
+  hsd_count_launches(p.n_pairs > 0 ? 3 : 2);
+  return hsd_launch_status();
 }
 
 template <typename T>
 int launch_alpha(const void *logits, long long model_stride, int L, int R, int V, void *ws, double *alpha, cudaStream_t s) {
-  const AlphaPlan p = alpha_plan(L, R, V);
-  float2 *stats = (float2 *)((char *)ws + p.stats_off);
-  float *partials = (float *)((char *)ws + p.partials_off);
-  alpha_stats_kernel<T><<<dim3(R, L), kAlphaThreads, 0, s>>>((const T *)logits, model_stride, R, V, stats);
-  if (p.n_pairs > 0) {
-    const size_t smem = ((size_t)kAlphaChunk * L + 8 * (size_t)p.n_pairs) * sizeof(float);
-    if (smem > 48 * 1024) {
-      static bool attr_set = false;
-      if (!attr_set) {
-        if (cudaFuncSetAttribute(alpha_pairs_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) return HSD_E_CUDA;
-        attr_set = true;
-      }
-    }
-    alpha_pairs_kernel<T><<<dim3(R, p.n_chunks), kAlphaThreads, smem, s>>>((const T *)logits, model_stride, L, R, V, stats, partials);
-  }
-  alpha_reduce_kernel<<<p.n_pairs > 0 ? min(p.n_pairs, 148) : 1, kAlphaThreads, 0, s>>>(partials, L, R * p.n_chunks, R, alpha);
-  hsd_count_launches(p.n_pairs > 0 ? 3 : 2);
-  return hsd_launch_status();
+  // 16-byte loads need every row on a 16-byte boundary and no partial vector at a row's end
+  constexpr int N = AlphaVec<T>::N;
+  const bool vec = V % N == 0 && model_stride % N == 0 && ((uintptr_t)logits & 15) == 0;
+  return vec ? launch_alpha_t<T, true>(logits, model_stride, L, R, V, ws, alpha, s)
+             : launch_alpha_t<T, false>(logits, model_stride, L, R, V, ws, alpha, s);
 }
 
 }  // namespace
@@ -163,8 +363,6 @@ int hsd_pairwise_alpha(const void *logits, int dtype, int n_models, int n_rows, 
   if (n_models < 1 || n_models > hsd::kAlphaMaxModels || n_rows < 1 || vocab < 1) return HSD_E_INVALID_ARG;
   if (model_stride < (long long)n_rows * vocab) return HSD_E_INVALID_ARG;
   if (((uintptr_t)workspace & 255) != 0 || workspace_bytes < hsd::alpha_plan(n_models, n_rows, vocab).total) return HSD_E_INVALID_ARG;
-  if (((size_t)hsd::kAlphaChunk * n_models + 8 * (size_t)(n_models * (n_models - 1) / 2)) * sizeof(float) > 200 * 1024)
-    return HSD_E_TOO_LARGE;
   cudaStream_t s = (cudaStream_t)stream;
   return dtype == HSD_BF16
              ? hsd::launch_alpha<__nv_bfloat16>(logits, model_stride, n_models, n_rows, vocab, workspace, alpha, s)

@@ -95,3 +95,19 @@ def test_calibrate_then_search_end_to_end(lib):
     lat, sigma, T = binding.hsd_search_hierarchy(costs, alpha.tolist(), 8)
     assert sigma[-1] == len(layers) - 1 and lat <= costs[-1] and len(T) == len(sigma) - 1
     assert abs(lat - __import__("oracle.latency", fromlist=["x"]).search_hierarchy(costs, alpha.tolist(), 8)[0]) <= 1e-12 * lat
+
+
+@pytest.mark.parametrize("L,R,V,dtype", [(9, 2, 4104, torch.bfloat16),      # two 8-model blocks, a unit of one 8-token vector
+                                         (17, 3, 9001, torch.float32),       # three blocks, rows off the 16-byte grid
+                                         (24, 2, 5000, torch.float32), (32, 2, 8200, torch.bfloat16), (32, 1, 255, torch.bfloat16)])
+def test_pairwise_alpha_block_edges(lib, L, R, V, dtype):
+    """Model counts at the ends of the 8-model blocks and vocabularies at the ends of tiles and units."""
+    g = torch.Generator().manual_seed(L + V)
+    base = torch.randn(R, V, generator=g) * 2.5
+    logits = torch.stack([base + 0.1 * (m + 1) * torch.randn(R, V, generator=g) for m in range(L)]).to(dtype)
+    logits[0, 0, : V // 2] = -float("inf")                                   # a masked half: weight exactly zero
+    got = lib.hsd_pairwise_alpha(logits.cuda()).cpu().numpy()
+    p = torch.softmax(logits.double(), -1)
+    want = torch.stack([torch.minimum(p[i:i + 1], p).sum(-1).mean(-1) for i in range(L)]).numpy()
+    # fp32 sums of at most 128 terms per lane and 8 per warp and slice: about 2^-24 x 136 of a rate, 1e-5 at most
+    assert np.array_equal(got, got.T) and np.abs(got - want).max() < 1e-5, np.abs(got - want).max()
