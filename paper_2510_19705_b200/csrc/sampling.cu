@@ -588,6 +588,405 @@ __global__ void __launch_bounds__(kFusedThreads, 1) verify_fused_kernel(const __
   }
 }
 
+// ------------------------------------------------------------------------------ one cluster per sequence
+// Algorithm 2's decision, or level 0's draw (no drafts: the rule's final draw from the one row), for few sequences: a
+// cluster of C CTAs takes a sequence's 2 t + 1 rows, each CTA the same V / C consecutive tokens of every row.  Bound by
+// latency, not by bytes (t = 3 rows of 32000 bf16 tokens are 0.4 MB): the rows are read once into shared memory, the row
+// maxima and then the integer totals cross the cluster in one exchange each, every CTA takes the accept tests by itself,
+// and a rejection costs one more exchange for the residual's totals.  No scratch in global memory, nothing to clear.
+// A warp owns consecutive tokens; lane and unit index are interleaved (unit = 4 bytes: a bf16 pair or an fp32 value;
+// 2 bytes when rows of odd length leave bf16 pairs unaligned), so loads are whole lines whatever the row's alignment.
+constexpr int kClThreads = 512, kClWarps = kClThreads / 32, kClMaxRows = 63, kClMaxC = 8;
+
+template <typename T, int PER> struct ClUnit;              // PER tokens of one load
+template <> struct ClUnit<float, 1> {
+  typedef float raw;
+  __device__ static void get(float r, float *f) { f[0] = r; }
+};
+template <> struct ClUnit<__nv_bfloat16, 1> {
+  typedef unsigned short raw;
+  __device__ static void get(unsigned short r, float *f) { f[0] = __uint_as_float((u32)r << 16); }
+};
+template <> struct ClUnit<__nv_bfloat16, 2> {
+  typedef u32 raw;
+  __device__ static void get(u32 r, float *f) { f[0] = __uint_as_float(r << 16); f[1] = __uint_as_float(r & 0xFFFF0000u); }
+};
+
+struct ClusterArgs {
+  const void *p, *q;
+  int32_t *tokens;
+  int V, t_max, seg;             // seg: tokens per CTA, a multiple of 64
+  int staged;                    // rows kept in shared memory; 0: they do not fit and are read again where they are needed
+  int purpose;                   // PURPOSE_FINAL, or PURPOSE_DRAFT: level-0 draws
+  const VerifySeq *desc;         // verification: per sequence, or null (regular)
+  const SampleRow *rows;         // draws: per row, or null (regular)
+  int regular_t;                 // draws: rows per sequence
+  u32 regular_serial, regular_level;
+  u64 seed;
+  int32_t *out_tokens, *out_n;
+  int write_in_place;
+  u32 coin24;
+};
+
+__device__ __forceinline__ u32 cl_rank() { u32 r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ u32 cl_size() { u32 r; asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ u32 cl_id() { u32 r; asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cl_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ u32 cl_map(const void *p, u32 rank) {
+  u32 r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((u32)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cl_store(u32 addr, u32 v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ void cl_store(u32 addr, u64 v) { asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory"); }
+// fp32 (no NaN) -> signed integer in the same order, and back
+__device__ __forceinline__ int order_key(float f) { const int b = __float_as_int(f); return b ^ ((b >> 31) & 0x7FFFFFFF); }
+__device__ __forceinline__ float order_value(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7FFFFFFF)); }
+// Sum over a warp of values below 2^54.
+__device__ __forceinline__ u64 warp_sum54(u64 v) {
+  const u32 lo = __reduce_add_sync(0xFFFFFFFFu, (u32)v & 0x7FFFFFFu), hi = __reduce_add_sync(0xFFFFFFFFu, (u32)(v >> 27));
+  return ((u64)hi << 27) + lo;
+}
+
+// Shared memory (dynamic): raw units [rows][NU][threads] | wmax int [rows][warps] | wsum u64 [rows + 1][warps]
+template <typename T, int PER, int NT>
+__global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __grid_constant__ ClusterArgs a) {
+  typedef typename ClUnit<T, PER>::raw raw_t;
+  constexpr int NU = NT / PER;                                     // units per thread and row
+  extern __shared__ __align__(16) unsigned char cl_smem[];
+  __shared__ int cmax[kClMaxRows][kClMaxC];                        // row maxima of every CTA of the cluster (order keys)
+  __shared__ u64 csum[kClMaxRows + 1][kClMaxC];                    // row totals; the last entry: the residual
+  __shared__ float row_m[kClMaxRows];
+  __shared__ u64 row_S[kClMaxRows];
+  __shared__ int sh_n;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const u32 rank = cl_rank(), C = cl_size();
+  const int b = (int)cl_id();
+  VerifySeq d;
+  long long out_index = 0;
+  u32 uj = 0;
+  if (a.purpose == PURPOSE_DRAFT) {
+    SampleRow s;
+    if (a.rows) s = a.rows[b];
+    else { s.logit_row = b; s.out_index = b; s.j = b % a.regular_t; s.seq = b / a.regular_t; s.serial = a.regular_serial; s.level = 0; }
+    d.p_row0 = s.logit_row; d.q_row0 = 0; d.tok_off = 0; d.t = 0; d.serial = s.serial; d.seq = s.seq; d.level = s.level;
+    out_index = s.out_index; uj = s.j;
+  } else if (a.desc) d = a.desc[b];
+  else {
+    d.t = a.regular_t; d.p_row0 = (long long)b * (a.regular_t + 1); d.q_row0 = (long long)b * a.regular_t;
+    d.tok_off = (long long)b * a.regular_t; d.serial = a.regular_serial; d.seq = b; d.level = a.regular_level;
+  }
+  const int t = d.t, n_rows = 2 * t + 1;                           // rows 0..t: p; t + 1 + j: q_j
+  raw_t *stage = reinterpret_cast<raw_t *>(cl_smem);
+  const size_t max_rows = 2 * (size_t)a.t_max + 1;
+  u64 *wsum = reinterpret_cast<u64 *>(cl_smem + (a.staged ? max_rows * NU * kClThreads * sizeof(raw_t) : 0));   // [rows + 1][warps]
+  int *wmax = reinterpret_cast<int *>(wsum + (max_rows + 1) * kClWarps);
+  auto row_ptr = [&](int r) {
+    return r <= t ? reinterpret_cast<const T *>(a.p) + (size_t)(d.p_row0 + r) * a.V
+                  : reinterpret_cast<const T *>(a.q) + (size_t)(d.q_row0 + r - t - 1) * a.V;
+  };
+  const int tok0 = (int)rank * a.seg, tok_end = min(a.V, tok0 + a.seg);
+  const int k_lane = tok0 + warp * (32 * NT) + lane * PER;         // first token of unit i: k_lane + 32 PER i
+  // the drafted tokens' logits (every CTA takes the accept tests for itself)
+  float lp = 0.f, lq = 0.f;
+  int tok = -1;
+  if (tid < t) {
+    tok = a.tokens[d.tok_off + tid];
+    if (tok >= 0 && tok < a.V) { lp = to_f32(row_ptr(tid)[tok]); lq = to_f32(row_ptr(t + 1 + tid)[tok]); }
+  }
+  auto unit_of = [&](int r, int i) -> raw_t {                      // a unit of this thread, once more
+    if (a.staged) return stage[((size_t)r * NU + i) * kClThreads + tid];
+    const int k = k_lane + 32 * PER * i;
+    return k < tok_end ? __ldg(reinterpret_cast<const raw_t *>(row_ptr(r) + k)) : raw_t(0);
+  };
+  // weights of a row's units against the row maximum, two tokens j, j + 1 at a time (0 past the CTA's tokens)
+  auto weights_of = [&](const raw_t *v, float m, auto &&take) {
+    float f[NT];
+#pragma unroll
+    for (int i = 0; i < NU; ++i) ClUnit<T, PER>::get(v[i], f + i * PER);
+#pragma unroll
+    for (int j = 0; j < NT; j += 2) {
+      u32 e0, e1;
+      exp_weight2(f[j], f[j + 1], m, e0, e1);
+      take(j, k_lane + 32 * PER * (j / PER) < tok_end ? e0 : 0u, k_lane + 32 * PER * ((j + 1) / PER) < tok_end ? e1 : 0u);
+    }
+  };
+  // ---- rows into shared memory (own slots: no barrier between the write and the later reads) and the row maxima
+  constexpr int RB = NU <= 4 ? 8 : (NU <= 8 ? 4 : (NU <= 16 ? 2 : 1));   // rows fetched at a time
+  for (int r0 = 0; r0 < n_rows; r0 += RB) {
+    raw_t v[RB][NU];
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr) {
+      const T *row = row_ptr(min(r0 + rr, n_rows - 1));
+#pragma unroll
+      for (int i = 0; i < NU; ++i) {
+        const int k = k_lane + 32 * PER * i;
+        v[rr][i] = k < tok_end ? __ldg(reinterpret_cast<const raw_t *>(row + k)) : raw_t(0);
+      }
+    }
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr) {
+      if (r0 + rr >= n_rows) break;
+      float m = -INFINITY;
+#pragma unroll
+      for (int i = 0; i < NU; ++i) {
+        const int k = k_lane + 32 * PER * i;
+        float f[PER];
+        ClUnit<T, PER>::get(v[rr][i], f);
+        if (k < tok_end) {                                         // (PER = 2: V is even)
+#pragma unroll
+          for (int e = 0; e < PER; ++e) m = fmaxf(m, f[e]);
+        }
+        if (a.staged) stage[((size_t)(r0 + rr) * NU + i) * kClThreads + tid] = v[rr][i];
+      }
+      const int key = __reduce_max_sync(0xFFFFFFFFu, order_key(m));
+      if (lane == 0) wmax[(r0 + rr) * kClWarps + warp] = key;
+    }
+  }
+  __syncthreads();
+  for (int r = warp; r < n_rows; r += kClWarps) {
+    const int key = __reduce_max_sync(0xFFFFFFFFu, wmax[r * kClWarps + (lane & (kClWarps - 1))]);
+    if (lane < (int)C) cl_store(cl_map(&cmax[r][rank], (u32)lane), (u32)key);
+  }
+  cl_sync();
+  if (tid < n_rows) {
+    int key = cmax[tid][0];
+    for (u32 c = 1; c < C; ++c) key = max(key, cmax[tid][c]);
+    row_m[tid] = order_value(key);
+  }
+  __syncthreads();
+  // ---- integer totals
+  for (int r0 = 0; r0 < n_rows; r0 += RB) {
+    raw_t v[RB][NU];
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr)
+#pragma unroll
+      for (int i = 0; i < NU; ++i) v[rr][i] = unit_of(min(r0 + rr, n_rows - 1), i);
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr) {
+      if (r0 + rr >= n_rows) break;
+      const float m = row_m[r0 + rr];
+      u64 local = 0;
+      weights_of(v[rr], m, [&](int, u32 e0, u32 e1) { local += (u64)e0 + (u64)e1; });
+      const u64 s = warp_sum54(local);
+      if (lane == 0) wsum[(r0 + rr) * kClWarps + warp] = s;
+    }
+  }
+  __syncthreads();
+  auto publish = [&](int r) {                                      // a warp: total of wsum row r -> every CTA's csum
+    u64 s = lane < kClWarps ? wsum[r * kClWarps + lane] : 0ull;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    if (lane < (int)C) cl_store(cl_map(&csum[r][rank], (u32)lane), s);
+  };
+  for (int r = warp; r < n_rows; r += kClWarps) publish(r);
+  cl_sync();
+  if (tid < n_rows) {
+    u64 S = 0;
+    for (u32 c = 0; c < C; ++c) S += csum[tid][c];
+    row_S[tid] = S;
+  }
+  __syncthreads();
+  // ---- accept tests (t <= 31: one warp), n = first rejection
+  if (warp == 0) {
+    bool ok = true;
+    if (lane < t) {
+      const u32 ep = (tok >= 0 && tok < a.V) ? exp_weight(lp, row_m[lane]) : 0u, eq = (tok >= 0 && tok < a.V) ? exp_weight(lq, row_m[t + 1 + lane]) : 0u;
+      const u64 Pp = fixed_prob(ep, prob_scale(row_S[lane])), Pq = fixed_prob(eq, prob_scale(row_S[t + 1 + lane]));
+      const u32 U = uniform24(a.seed, lane, d.serial, d.level, PURPOSE_ACCEPT, d.seq);
+      ok = (((u64)U * Pq) >> 24) < Pp;                             // u < p(x) / q(x)
+      if (a.coin24 != kNoCoin) ok = U < a.coin24;                  // ablation: IID acceptance with a fixed probability
+    }
+    const unsigned rejected = __ballot_sync(0xFFFFFFFFu, !ok);
+    if (lane == 0) sh_n = rejected ? __ffs(rejected) - 1 : t;
+  }
+  __syncthreads();
+  const int n = sh_n;
+  // ---- the final draw's weights: the residual of row n, or row t itself
+  u64 w[NT];
+  int src = n;                                                     // row of wsum / csum that holds the totals of w
+  u64 total = row_S[n];
+  const float mp = row_m[n];
+  auto row_weights = [&]() {
+    raw_t v[NU];
+#pragma unroll
+    for (int i = 0; i < NU; ++i) v[i] = unit_of(n, i);
+    weights_of(v, mp, [&](int j, u32 e0, u32 e1) { w[j] = e0; w[j + 1] = e1; });
+  };
+  if (n < t) {
+    const float mq = row_m[t + 1 + n];
+    const ProbScale psp = prob_scale(row_S[n]), psq = prob_scale(row_S[t + 1 + n]);
+    u64 local = 0;
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      const int k = k_lane + 32 * PER * i;
+      float fp[PER], fq[PER];
+      ClUnit<T, PER>::get(unit_of(n, i), fp);
+      ClUnit<T, PER>::get(unit_of(t + 1 + n, i), fq);
+#pragma unroll
+      for (int e = 0; e < PER; ++e) {
+        u32 ep, eq;
+        exp_weight2m(fp[e], fq[e], mp, mq, ep, eq);
+        const u64 Pp = fixed_prob(ep, psp), Pq = fixed_prob(eq, psq);
+        w[i * PER + e] = (k < tok_end && Pp > Pq) ? Pp - Pq : 0ull;
+        local += w[i * PER + e];
+      }
+    }
+    const u64 s = warp_sum54(local);
+    if (lane == 0) wsum[n_rows * kClWarps + warp] = s;
+    __syncthreads();
+    if (warp == 0) publish(n_rows);
+    cl_sync();
+    total = 0;
+    for (u32 c = 0; c < C; ++c) total += csum[n_rows][c];
+    if (total != 0) src = n_rows;
+    else total = row_S[n];                                         // an all-zero residual: draw from the verifier's own row
+  }
+  if (src == n) row_weights();
+  // ---- inverse CDF: the CTA, then the warp, then the unit, then the token whose inclusive sum passes the threshold
+  const u32 U = uniform24(a.seed, uj, d.serial, d.level, a.purpose, d.seq);
+  const u64 tau = cdf_threshold(U, total);
+  u64 before = 0;
+  for (u32 c = 0; c < rank; ++c) before += csum[src][c];
+  if (total == 0) {                                                // non-finite logits: no token
+    if (rank == 0 && tid == 0) {
+      if (a.purpose == PURPOSE_DRAFT) a.out_tokens[out_index] = -1;
+      else {
+        if (a.write_in_place) a.tokens[d.tok_off + n] = -1;
+        if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = -1;
+      }
+    }
+  } else if (tau >= before && tau < before + csum[src][rank]) {
+    u64 mine = lane < kClWarps ? wsum[src * kClWarps + lane] : 0ull;   // every warp finds the owning one for itself
+    u64 incl = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+      const u64 v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const int owner = __ffs(__ballot_sync(0xFFFFFFFFu, before + incl > tau)) - 1;
+    if (warp == owner) {
+      u64 base = before + __shfl_sync(0xFFFFFFFFu, incl - mine, owner);
+      u64 tot[NU];
+#pragma unroll
+      for (int i = 0; i < NU; ++i) {
+        u64 s = 0;
+#pragma unroll
+        for (int e = 0; e < PER; ++e) s += w[i * PER + e];
+        tot[i] = warp_sum54(s);
+      }
+      bool done = false;
+#pragma unroll
+      for (int i = 0; i < NU; ++i) {
+        if (!done && base + tot[i] > tau) {                        // uniform over the warp
+          done = true;
+          u64 s = 0;
+#pragma unroll
+          for (int e = 0; e < PER; ++e) s += w[i * PER + e];
+          u64 c = s;
+          for (int o = 1; o < 32; o <<= 1) {
+            const u64 v = __shfl_up_sync(0xFFFFFFFFu, c, o);
+            if (lane >= o) c += v;
+          }
+          const int l = __ffs(__ballot_sync(0xFFFFFFFFu, base + c > tau)) - 1;
+          if (lane == l) {
+            u64 run = base + c - s;
+            int k = k_lane + 32 * PER * i;
+#pragma unroll
+            for (int e = 0; e < PER; ++e) {
+              run += w[i * PER + e];
+              if (run > tau) break;
+              ++k;
+            }
+            if (a.purpose == PURPOSE_DRAFT) a.out_tokens[out_index] = k;
+            else {
+              if (a.write_in_place) a.tokens[d.tok_off + n] = k;
+              if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = k;
+            }
+          }
+        } else if (!done) base += tot[i];
+      }
+    }
+  }
+  if (a.purpose != PURPOSE_DRAFT && rank == 0) {
+    if (tid == 0) a.out_n[b] = n;
+    if (a.out_tokens && tid <= a.t_max && tid != n) a.out_tokens[(size_t)b * (a.t_max + 1) + tid] = tid < n ? tok : -1;
+  }
+}
+
+// Cluster size, tokens per thread and shared memory of a call with n sequences of at most `rows` rows; false if the rows
+// are too long or too many for this path.
+struct ClusterPlan { int C, NT, per, staged, seg; size_t smem; };
+constexpr size_t kClMaxSmem = 216 * 1024;
+static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, int rows, ClusterPlan *pl) {
+  if (rows > kClMaxRows) return false;
+  pl->per = (dtype == HSD_BF16 && V % 2 == 0 && ((uintptr_t)p & 3) == 0 && ((uintptr_t)q & 3) == 0) ? 2 : 1;
+  // as many CTAs as run at once, of at least 4096 tokens (eight a thread) each: clusters of eight do not fit all 148 SMs
+  // (16 of them took two rounds), clusters of four and two do
+  int C = 1;
+  while (C < kClMaxC && V > C * 4096 && 2 * C * n <= (C == 4 ? 112 : 148)) C *= 2;
+  while (C < kClMaxC && ceil_div(V, C) > 32 * kClThreads - 64) C *= 2;
+  const int seg = ceil_div(ceil_div(V, C), 64) * 64;
+  if (seg > 32 * kClThreads) return false;
+  pl->C = C;
+  pl->seg = seg;
+  pl->NT = seg <= 8 * kClThreads ? 8 : seg <= 16 * kClThreads ? 16 : 32;
+  const size_t extra = (size_t)(rows + 1) * kClWarps * 8 + (size_t)rows * kClWarps * 4;
+  const size_t stage = (size_t)rows * pl->NT * kClThreads * (dtype == HSD_BF16 ? 2 : 4);
+  pl->staged = stage + extra <= kClMaxSmem;
+  pl->smem = extra + (pl->staged ? stage : 0);
+  return true;
+}
+// Where the cluster path is the faster one (us a call on an idle GPU, cluster / other path).  Its time grows with the
+// tokens a CTA goes through, rows x seg; the other paths give every row a CTA of its own.
+//   verification, rows the fused kernel takes (V = 32000 bf16): t = 3: 1 to 8 sequences 12 / 25, 32: 17 / 30, 64 (112k
+//     tokens a CTA): 38 / 35; t = 8: 8 sequences (68k) 19 / 26, 16 (136k): 36 / 30.
+//   other rows: statistics and decision kernels, each row read twice by one CTA.  fp32, V = 32001: t = 3 14 / 58, t = 8
+//     30 / 58; V = 9001: t = 3 14 / 15, t = 8 29 / 15; V = 2048: t = 3 11 / 7.  bf16 of odd length, 49999: t = 3 21 / 50, t = 8 55 / 50.
+//   draws: bf16 32000: 1 row 6.8 / 12.5, 64 rows 11.2 / 12.5; 16000: 100 rows (no split) 10.8 / 10.1; fp32 9001: 7.1 / 6.0,
+//     16001: 7.2 / 11.7, 50000: 64 rows 27 / 24.
+static bool cluster_pays_verify(const ClusterPlan &pl, int dtype, int V, int rows, bool fused) {
+  const long long work = (long long)pl.seg * rows;
+  if (fused) return work <= 100000;
+  if (dtype == HSD_BF16) return work * 5 <= 8ll * V;
+  return V > 20000 ? work <= 4ll * V : work * 5 <= 11ll * V;
+}
+static bool cluster_pays_draw(const ClusterPlan &pl, int dtype, int V, int n, bool chunked) {
+  if (pl.seg > 4096 && (pl.seg > 16384 || pl.C * n > 148)) return false;     // (256 rows of 32000: 39 / 25)
+  if (dtype == HSD_BF16 && chunked) return pl.seg <= 4096 || pl.C > 1;
+  return V > 12000 && pl.C > 1;
+}
+
+template <typename T, int PER, int NT>
+static int launch_cluster_t(const ClusterArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
+  static bool attr_set = false;
+  if (!attr_set) {
+    HSD_CUDA_OK(cudaFuncSetAttribute(cluster_sample_kernel<T, PER, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClMaxSmem));
+    attr_set = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n * pl.C); cfg.blockDim = dim3(kClThreads); cfg.dynamicSmemBytes = pl.smem; cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = pl.C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  HSD_CUDA_OK(cudaLaunchKernelEx(&cfg, cluster_sample_kernel<T, PER, NT>, a));
+  hsd_count_launches(1);
+  return hsd_launch_status();
+}
+template <typename T, int PER>
+static int launch_cluster_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
+  if (pl.NT == 8) return launch_cluster_t<T, PER, 8>(a, pl, n, s);
+  if (pl.NT == 16) return launch_cluster_t<T, PER, 16>(a, pl, n, s);
+  return launch_cluster_t<T, PER, 32>(a, pl, n, s);
+}
+static int launch_cluster(ClusterArgs a, const ClusterPlan &pl, int dtype, int n, cudaStream_t s) {
+  a.seg = pl.seg;
+  a.staged = pl.staged;
+  if (dtype == HSD_F32) return launch_cluster_nt<float, 1>(a, pl, n, s);
+  return pl.per == 2 ? launch_cluster_nt<__nv_bfloat16, 2>(a, pl, n, s) : launch_cluster_nt<__nv_bfloat16, 1>(a, pl, n, s);
+}
+
 // ------------------------------------------------------------------------------ host launchers
 // Scratch of one verification call: [counter per sequence (fused kernel)] [RowStat per logits row].
 static size_t verify_counter_bytes(int batch) { return ((size_t)(2 * batch + 2) * 4 + 255) / 256 * 256; }
@@ -606,6 +1005,14 @@ static int launch_draft_sample_t(const void *logits, int V, const SampleRow *des
 int launch_draft_sample(const void *logits, int dtype, int V, const SampleRow *desc, int n_rows, int regular_rows,
                         u32 regular_serial, u64 seed, int32_t *out, cudaStream_t s) {
   if (n_rows == 0) return HSD_OK;
+  ClusterPlan pl;
+  if (cluster_plan(logits, nullptr, dtype, V, n_rows, 1, &pl) &&
+      cluster_pays_draw(pl, dtype, V, n_rows, V % 8 == 0 && V <= kSampleThreads * kChunkTokens && ((uintptr_t)logits & 15) == 0)) {
+    ClusterArgs a = {};
+    a.p = logits; a.V = V; a.t_max = 0; a.purpose = PURPOSE_DRAFT; a.rows = desc; a.regular_t = regular_rows;
+    a.regular_serial = regular_serial; a.seed = seed; a.out_tokens = out; a.coin24 = kNoCoin;
+    return launch_cluster(a, pl, dtype, n_rows, s);
+  }
   return dtype == HSD_BF16
              ? launch_draft_sample_t<__nv_bfloat16>(logits, V, desc, n_rows, regular_rows, regular_serial, seed, out, s)
              : launch_draft_sample_t<float>(logits, V, desc, n_rows, regular_rows, regular_serial, seed, out, s);
@@ -652,6 +1059,14 @@ int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int 
   const size_t slot = ((size_t)V * 2 + 127) / 128 * 128, smem = kFusedSlots * slot + 2 * kFusedSlots * 8 + 128;
   const bool fused = dtype == HSD_BF16 && V % 8 == 0 && V <= kFusedMaxV && smem <= 220 * 1024 && ((uintptr_t)p & 15) == 0 &&
                      (q == nullptr || ((uintptr_t)q & 15) == 0) && t_max < kFusedConsumers;
+  ClusterPlan pl;
+  if (cluster_plan(p, q, dtype, V, batch, 2 * t_max + 1, &pl) && cluster_pays_verify(pl, dtype, V, 2 * t_max + 1, fused)) {
+    ClusterArgs a = {};
+    a.p = p; a.q = q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.purpose = PURPOSE_FINAL; a.desc = desc; a.regular_t = regular_t;
+    a.regular_serial = regular_serial; a.regular_level = regular_level; a.seed = seed; a.out_tokens = out_tokens; a.out_n = out_n;
+    a.write_in_place = write_in_place; a.coin24 = coin24;
+    return launch_cluster(a, pl, dtype, batch, s);
+  }
   if (fused) {
     static bool attr_set = false;
     if (!attr_set) {

@@ -114,3 +114,23 @@ def test_bad_arguments_are_rejected(lib):
         lib.hsd_verify_level(1, p, q, x, 0, 0, workspace=small)
     with pytest.raises(lib.HsdError, match="invalid argument"):
         lib.hsd_verify_level(300, p, q, x, 0, 0)
+
+
+@pytest.mark.parametrize("dtype,V,B,t", [("bf16", 4096, 3, 3),       # one CTA a sequence, every thread's eight tokens used
+                                         ("bf16", 4098, 2, 2),       # two CTAs, the second with an odd tail of pairs
+                                         ("bf16", 32000, 14, 2), ("bf16", 32000, 15, 2),    # clusters of eight / of four
+                                         ("bf16", 65538, 1, 1),      # 32 tokens a thread
+                                         ("bf16", 1536, 2, 31),      # the most rows a sequence can have here; read twice, not staged
+                                         ("bf16", 30001, 2, 1), ("fp32", 32769, 1, 8), ("fp32", 24001, 40, 1), ("bf16", 9000, 2, 0)])
+def test_cluster_decisions_match_oracle(lib, dtype, V, B, t):
+    p, q = inputs.make_accept_logits(B, t, V, seed=V + 7 * t, device="cuda", dtype=dtype)
+    p[0, :, V // 2:] = -float("inf")                                  # a mask over half the vocabulary
+    x = lib.hsd_draft_sample(q, 5, 0) if t else None
+    p_np, q_np = inputs.logits_to_numpy(p), inputs.logits_to_numpy(q)
+    x_np = x.cpu().numpy() if t else np.zeros((B, 0), np.int32)
+    if t:
+        assert np.array_equal(x_np, _oracle_draft(q_np, 5, 0))
+    for serial in range(3):
+        out, n = lib.hsd_verify_level(1, p, q, x, 17, serial)
+        want_out, want_n = _oracle_verify(1, p_np, q_np, x_np, 17, serial)
+        assert np.array_equal(n.cpu().numpy(), want_n) and np.array_equal(out.cpu().numpy(), want_out)
