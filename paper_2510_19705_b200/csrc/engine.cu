@@ -334,9 +334,9 @@ int upload_page_tables(hsd_ctx *c) {
 
 // Matrix product of the forward pass: tensor cores for bf16 models, CUDA cores otherwise.
 // abuf names the activation buffer A lives in (0 = h, 1 = att, 2 = act, 3 = hf); wmap0 the index of
-// the first segment's tensor map.
+// the first segment's tensor map; qkv: destinations of the q / k / v projection (tensor cores only).
 int gemm(hsd_ctx *c, Model &M, int abuf, const void *A, int R, int K, const GemmSegs &segs, int wmap0, int mode, float *out_f32,
-         void *out_t, const long long *dst) {
+         void *out_t, const long long *dst, const TcQkv *qkv = nullptr) {
   if (!M.use_tc) return launch_gemm_simt(M.md, A, R, K, segs, mode, out_f32, out_t, dst, c->stream);
   TcGemmArgs a;
   int total = 0;
@@ -353,17 +353,33 @@ int gemm(hsd_ctx *c, Model &M, int abuf, const void *A, int R, int K, const Gemm
   a.dst = dst;
   a.ldo = (mode == GEMM_SWIGLU_T) ? segs.n[0] : total;
   a.status = (int *)(c->ws + c->status_off);
-  a.counters = (int *)(c->ws + M.lay.tc_scratch + 256);
-  a.pieces = (float *)(c->ws + M.lay.tc_scratch + kTcCtrlBytes);
+  a.stream_weights = 1;
+  if (qkv) a.qkv = *qkv;
   for (int r0 = 0; r0 < R; r0 += 256) {
     a.R = std::min(256, R - r0);
     a.row0 = r0;
-    int np = tc_npad(a.R);
-    a.a = M.amaps[abuf][np == 16 ? 0 : np == 32 ? 1 : np == 64 ? 2 : np == 128 ? 3 : 4];
+    const int np = tc_npad(a.R);
+    a.a_box_rows = a.R <= 16 ? a.R : np;
+    a.a = a.R <= 16 ? M.amaps_rows[abuf][a.R - 1] : M.amaps[abuf][np == 32 ? 1 : np == 64 ? 2 : np == 128 ? 3 : 4];
     int st = launch_gemm_tc(a, c->sm_count, c->stream);
     if (st) return st;
   }
   return HSD_OK;
+}
+// q / k / v of a pass's rows: on tensor cores the projection itself rotates and stores them, otherwise a kernel after it.
+int project_qkv(hsd_ctx *c, Model &M, int layer, const RowBatch &rb, const void *h, float *qkv, const int *pt, void *kp, void *vp, void *q) {
+  const ModelDims &md = M.md;
+  const ModelLayout &ML = M.lay;
+  const void *const *w = &M.lw[(size_t)layer * 9];
+  const GemmSegs segs = {{w[1], w[2], w[3]}, {md.nq * md.hd, md.nkv * md.hd, md.nkv * md.hd}, 3};
+  const float *cs = c->dev<float>(ML.cos_tab), *sn = c->dev<float>(ML.sin_tab);
+  if (M.use_tc) {
+    const TcQkv to = {rb.row_seq, rb.row_pos, pt, cs, sn, (__nv_bfloat16 *)q, (__nv_bfloat16 *)kp, (__nv_bfloat16 *)vp,
+                      md.nq, md.hd, md.page, md.pages_per_seq, md.n_pages};
+    return gemm(c, M, 0, h, rb.R, md.d, segs, layer * 7, GEMM_QKV_T, nullptr, nullptr, nullptr, &to);
+  }
+  HSD_TRY(gemm(c, M, 0, h, rb.R, md.d, segs, layer * 7, GEMM_STORE_F32, qkv, nullptr, nullptr));
+  return launch_rope_kv(md, qkv, rb, cs, sn, pt, kp, vp, q, c->stream);
 }
 
 // One forward pass of level `level` (layers 1..exit) over the given rows; logits of the wanted
@@ -598,9 +614,7 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     const void *const *w = &M.lw[(size_t)l * 9];
     void *kp = c->ws + ML.k_pool + ML.pool_layer_stride * l, *vp = c->ws + ML.v_pool + ML.pool_layer_stride * l;
     HSD_TRY(launch_rmsnorm(md, x, w[0], nullptr, R, h, s));
-    GemmSegs qkv_segs = {{w[1], w[2], w[3]}, {md.nq * md.hd, md.nkv * md.hd, md.nkv * md.hd}, 3};
-    HSD_TRY(gemm(c, M, 0, h, R, md.d, qkv_segs, l * 7 + 0, GEMM_STORE_F32, qkv, nullptr, nullptr));
-    HSD_TRY(launch_rope_kv(md, qkv, rb, c->dev<float>(ML.cos_tab), c->dev<float>(ML.sin_tab), pt, kp, vp, q, s));
+    HSD_TRY(project_qkv(c, M, l, rb, h, qkv, pt, kp, vp, q));
     if (big_pass) {                                       // tensor-core attention of the persistent forward, as a launch of its own
       FwdArgs fa = {};
       fa.d = md.d; fa.nq = md.nq; fa.nkv = md.nkv; fa.hd = md.hd; fa.ff = md.ff; fa.V = md.V; fa.max_seq = md.max_seq; fa.page = md.page;
@@ -1213,9 +1227,7 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
     const void *const *w = &M.lw[(size_t)l * 9];
     void *kp = c->ws + ML.k_pool + ML.pool_layer_stride * l, *vp = c->ws + ML.v_pool + ML.pool_layer_stride * l;
     HSD_TRY(launch_rmsnorm(md, x, w[0], nullptr, R, h, s));
-    GemmSegs qkv_segs = {{w[1], w[2], w[3]}, {md.nq * md.hd, md.nkv * md.hd, md.nkv * md.hd}, 3};
-    HSD_TRY(gemm(c, M, 0, h, R, md.d, qkv_segs, l * 7 + 0, GEMM_STORE_F32, qkv, nullptr, nullptr));
-    HSD_TRY(launch_rope_kv(md, qkv, rb, c->dev<float>(ML.cos_tab), c->dev<float>(ML.sin_tab), pt, kp, vp, q, s));
+    HSD_TRY(project_qkv(c, M, l, rb, h, qkv, pt, kp, vp, q));
     HSD_TRY(launch_attention(md, q, rb, pt, kp, vp, c->dev<float>(ML.partials), keys_per_split, n_splits, att, s));
     GemmSegs o_segs = {{w[4], nullptr, nullptr}, {md.d, 0, 0}, 1};
     HSD_TRY(gemm(c, M, 1, att, R, md.nq * md.hd, o_segs, l * 7 + 3, GEMM_ADD_F32, x, nullptr, nullptr));
@@ -1282,8 +1294,7 @@ int hsd_set_trace(hsd_ctx *c, const char *path, int logit_calls) {
 
 size_t hsd_gemm_workspace_bytes(int R, int N, int K) {
   if (R < 1 || R > 256 || N < 1 || K < kTcBlockK || K % kTcBlockK) return 0;
-  int seg[3] = {N, 0, 0};
-  return kTcCtrlBytes + tc_plan(seg, 1, GEMM_STORE_F32, K, tc_npad(R), device_sm_count()).scratch_bytes;
+  return 256;                                   // the status word
 }
 
 int hsd_gemm_bf16(const void *A, int R, int K, const void *W, int N, float *out, void *workspace, size_t workspace_bytes,
@@ -1295,17 +1306,18 @@ int hsd_gemm_bf16(const void *A, int R, int K, const void *W, int N, float *out,
   int st = tc_init();
   if (st) return st;
   TcGemmArgs a;
-  st = tc_make_map(&a.w[0], W, N, K, kTcBoxRows);
-  if (!st) st = tc_make_map(&a.a, A, R, K, tc_npad(R));
+  const int sms = device_sm_count();
+  a.tile_rows = a.w_box_rows = tc_tile_rows(N, sms);
+  a.a_box_rows = R;
+  st = tc_make_map(&a.w[0], W, N, K, a.w_box_rows);
+  if (!st) st = tc_make_map(&a.a, A, R, K, R);
   if (st) return st;
   a.seg_n[0] = N; a.seg_n[1] = a.seg_n[2] = 0; a.n_segs = 1;
   a.K = K; a.R = R; a.row0 = 0; a.mode = GEMM_STORE_F32;
   a.out_f32 = out; a.out_bf16 = nullptr; a.dst = nullptr; a.ldo = N;
   a.status = (int *)workspace;
-  a.counters = (int *)((char *)workspace + 256);
-  a.pieces = (float *)((char *)workspace + kTcCtrlBytes);
-  HSD_CUDA_OK(cudaMemsetAsync(workspace, 0, kTcCtrlBytes, (cudaStream_t)stream));
-  return launch_gemm_tc(a, device_sm_count(), (cudaStream_t)stream);
+  a.reset_status = 1;
+  return launch_gemm_tc(a, sms, (cudaStream_t)stream);
 }
 
 int hsd_gemm_status(void *workspace, void *stream) {

@@ -38,7 +38,7 @@ struct GemmSegs {
   int n[3];
   int count;
 };
-enum GemmMode { GEMM_STORE_F32 = 0, GEMM_ADD_F32 = 1, GEMM_STORE_T_SCATTER = 2, GEMM_SWIGLU_T = 3 };
+enum GemmMode { GEMM_STORE_F32 = 0, GEMM_ADD_F32 = 1, GEMM_STORE_T_SCATTER = 2, GEMM_SWIGLU_T = 3, GEMM_QKV_T = 4 };
 
 int launch_embed(const ModelDims &md, const void *embed, const int *tokens, const RowBatch &rb, float *x, cudaStream_t s);
 // out[i, :] = T(rmsnorm(x[src ? src[i] : i, :]) * gain)

@@ -1,11 +1,20 @@
-// tcgen05 / TMEM / TMA weight-streaming GEMM (see gemm_tc.cuh).
+// Weight-streaming GEMM for up to 256 token rows (see gemm_tc.cuh).
 //
-// One CTA per SM, 192 threads: warp 0 = TMA producer (one lane), warp 1 = TMEM owner + MMA issuer
-// (one lane), warps 2..5 = epilogue (each reads its own 32-lane quarter of TMEM).  Shared-memory
-// ring of STAGES x (128x64 weight tile + NPADx64 activation tile), both K-major with the 128-byte
-// swizzle TMA writes and the UMMA descriptors read.  Two TMEM accumulators so the epilogue of one
-// tile overlaps the MMAs of the next.  Every wait is bounded by wall time; a wait that gives up
-// raises a flag, every role leaves its loop, TMEM is freed and a status word tells the host.
+// Bound by HBM: W is read once.  A tile is up to 128 weight rows on the MMA's M side, the token rows (padded to 16..256)
+// on its N side.  With few tiles the k-blocks of a tile are divided over a cluster of CTAs, whose partial sums stay in
+// shared memory and are added across the cluster in rank order (bit-reproducible): no pieces in global memory, no
+// counters.  With enough tiles to occupy the GPU a CTA takes whole tiles, and the next tile's weights stream in under a tile's finish.
+// A stream-K split over all SMs with pieces in global memory took 29.5 us for 14336 x 4096 at 24 rows (117 MB); whole tiles of 104 rows
+// on 138 CTAs take 25.6 us; 4096 x 4096 at 256 rows 49 -> 20 us.
+//
+// 192 threads: warp 0 = TMA producer (one lane), warp 1 = TMEM owner + MMA issuer (one lane), warps 2..5 = epilogue
+// (each reads its own 32-lane quarter of TMEM).  Shared-memory ring of (128 x 64 weight tile + NPAD x 64 activation
+// tile), both K-major with the 128-byte swizzle TMA writes and the UMMA descriptors read.  A CTA's k-blocks are summed in
+// two halves with a TMEM accumulator each, added in fp32 at the end: the tensor core's fp32 accumulation loses about as
+// much as its chain is long (relative error against fp64 at K = 4096: 4.4e-6 in one chain, 2.1e-6 in two).  Every
+// wait is bounded by wall time; a wait that gives up raises a flag, every role leaves its loop, TMEM is freed and a
+// status word tells the host.
+#include <algorithm>
 #include "gemm_tc.cuh"
 #include "tc_ptx.cuh"
 
@@ -16,17 +25,20 @@ using namespace ptx;
 
 constexpr int kThreads = 192;
 constexpr int kStageWBytes = kTcBlockM * kTcBlockK * 2;       // 16 KiB
-constexpr int kBoxBytes = kTcBoxRows * kTcBlockK * 2;         // 8 KiB
-constexpr int kSmemBudget = 232448 - 1024;                    // 227 KiB minus alignment slack
+constexpr int kSmemTotal = 232448;                            // 227 KiB
+constexpr int kLd = kTcBlockM + 4;                            // floats per token row of a staged tile (16-byte rows)
 
 template <int NPAD> struct TcCfg {
   static constexpr int kStageBytes = kStageWBytes + NPAD * kTcBlockK * 2;
-  static constexpr int kChunk = NPAD < 32 ? NPAD : 32;        // accumulator columns (token rows) the epilogue handles at a time
-  static constexpr int kStagingBytes = kTcBlockM * (kChunk + 1) * 4;
+  static constexpr int kChunk = NPAD < 32 ? NPAD : 32;        // token rows the epilogue stages at a time (whole tiles)
+  static constexpr int kStagingBytes = kChunk * kLd * 4;
   static constexpr int kCtrlBytes = 1024;
-  static constexpr int kStages = (kSmemBudget - kCtrlBytes - kStagingBytes) / kStageBytes;
+  static constexpr int kFit = (kSmemTotal - 1024 - kCtrlBytes - kStagingBytes) / kStageBytes;
+  static constexpr int kStages = kFit < 12 ? kFit : 12;       // 12 x 16 KiB of weights in flight per SM cover HBM's latency twice
   static constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + kCtrlBytes + 1024;
-  static constexpr int kTmemCols = (2 * NPAD < 32) ? 32 : 2 * NPAD;
+  static constexpr int kBufs = NPAD == 256 ? 1 : 2;           // tiles whose accumulators exist at a time, two accumulators each
+  static constexpr int kTmemCols = 2 * kBufs * NPAD;
+  static_assert(NPAD * kLd * 4 <= kStages * kStageBytes, "a cluster's partial sums must fit the ring");
 };
 
 struct TileInfo { int seg, row0, col0; };
@@ -35,25 +47,102 @@ __device__ __forceinline__ TileInfo tile_info(const TcGemmArgs &a, int tile) {
   if (a.mode == GEMM_SWIGLU_T) { ti.seg = 0; ti.row0 = tile * kTcBoxRows; ti.col0 = 0; return ti; }
   int t = tile, col0 = 0;
   for (int s = 0; s < a.n_segs; ++s) {
-    int nt = (a.seg_n[s] + kTcBlockM - 1) / kTcBlockM;
-    if (t < nt || s == a.n_segs - 1) { ti.seg = s; ti.row0 = t * kTcBlockM; ti.col0 = col0; return ti; }
+    int nt = (a.seg_n[s] + a.tile_rows - 1) / a.tile_rows;
+    if (t < nt || s == a.n_segs - 1) { ti.seg = s; ti.row0 = t * a.tile_rows; ti.col0 = col0; return ti; }
     t -= nt;
     col0 += a.seg_n[s];
   }
   ti.seg = 0; ti.row0 = 0; ti.col0 = 0;
   return ti;
 }
-__device__ __forceinline__ long long cta_begin(long long U, int G, int c) { return (U * c) / G; }
-__device__ __forceinline__ int unit_owner(long long U, int G, long long u) {
-  int c = (int)((u * G) / U);
-  while (c + 1 < G && cta_begin(U, G, c + 1) <= u) ++c;
-  while (c > 0 && cta_begin(U, G, c) > u) --c;
-  return c;
+__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr, uint32_t rank) {
+  uint32_t a;
+  float4 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint2 pack_bf16x4(const float4 &v) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+  return make_uint2(*reinterpret_cast<const unsigned *>(&a), *reinterpret_cast<const unsigned *>(&b));
+}
+
+// Token row r (of the pass), weight rows m .. m + 3 of the tile and, for SWIGLU / QKV, their partners (the up rows; the
+// second half of the head) -> the projection's output.
+template <int MODE>
+__device__ __forceinline__ void finish4(const TcGemmArgs &a, const TileInfo &ti, int r, int m, const float4 &v, const float4 &w) {
+  const int n = ti.row0 + m, left = a.seg_n[ti.seg] - n;
+  if (left <= 0) return;
+  const int row = a.row0 + r;
+  if (MODE == GEMM_SWIGLU_T) {                               // ff is a multiple of 64: whole groups of four
+    const float4 o = make_float4(silu_mul(v.x, w.x), silu_mul(v.y, w.y), silu_mul(v.z, w.z), silu_mul(v.w, w.w));
+    *reinterpret_cast<uint2 *>(a.out_bf16 + (size_t)row * a.ldo + n) = pack_bf16x4(o);
+  } else if (MODE == GEMM_QKV_T) {
+    const TcQkv &k = a.qkv;
+    const int half = k.hd >> 1, head = n / k.hd, c = n - head * k.hd;
+    const int pos = k.row_pos[row];
+    __nv_bfloat16 *dst;
+    if (ti.seg == 0) dst = k.q + ((size_t)row * k.nq + head) * k.hd + c;
+    else {
+      const int pg = k.page_table[(size_t)k.row_seq[row] * k.pages_per_seq + pos / k.page];
+      dst = (ti.seg == 1 ? k.k_pool : k.v_pool) + (((size_t)head * k.n_pages + pg) * k.page + pos % k.page) * k.hd + c;
+    }
+    float4 lo = v, hi = w;
+    if (ti.seg < 2) {
+      const float4 cs = __ldg(reinterpret_cast<const float4 *>(k.cos_tab + (size_t)pos * half + c));
+      const float4 sn = __ldg(reinterpret_cast<const float4 *>(k.sin_tab + (size_t)pos * half + c));
+      lo = make_float4(v.x * cs.x - w.x * sn.x, v.y * cs.y - w.y * sn.y, v.z * cs.z - w.z * sn.z, v.w * cs.w - w.w * sn.w);
+      hi = make_float4(w.x * cs.x + v.x * sn.x, w.y * cs.y + v.y * sn.y, w.z * cs.z + v.z * sn.z, w.w * cs.w + v.w * sn.w);
+    }
+    *reinterpret_cast<uint2 *>(dst) = pack_bf16x4(lo);
+    *reinterpret_cast<uint2 *>(dst + half) = pack_bf16x4(hi);
+  } else if (MODE == GEMM_STORE_T_SCATTER) {
+    __nv_bfloat16 *dst = a.out_bf16 + (size_t)a.dst[row] * a.ldo + ti.col0 + n;
+    if (left >= 4 && (a.ldo & 3) == 0) *reinterpret_cast<uint2 *>(dst) = pack_bf16x4(v);
+    else {
+      const float e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (i < left) dst[i] = __float2bfloat16_rn(e[i]);
+    }
+  } else {
+    float *dst = a.out_f32 + (size_t)row * a.ldo + ti.col0 + n;
+    float4 o = v;
+    if (left >= 4 && (a.ldo & 3) == 0 && ((uintptr_t)a.out_f32 & 15) == 0) {
+      if (MODE == GEMM_ADD_F32) {
+        const float4 old = __ldcg(reinterpret_cast<const float4 *>(dst));
+        o = make_float4(old.x + v.x, old.y + v.y, old.z + v.z, old.w + v.w);
+      }
+      *reinterpret_cast<float4 *>(dst) = o;
+    } else {
+      const float e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (i < left) dst[i] = MODE == GEMM_ADD_F32 ? __ldcg(dst + i) + e[i] : e[i];
+    }
+  }
+}
+
+// Items of one staged token row: groups of four weight rows (SWIGLU, QKV: of the first halves only).
+template <int MODE> __device__ __forceinline__ int items_of(const TcGemmArgs &a) {
+  return (MODE == GEMM_SWIGLU_T || MODE == GEMM_QKV_T) ? kTcBlockM / 8 : (a.tile_rows + 3) / 4;
+}
+template <int MODE> __device__ __forceinline__ void item_at(const TcGemmArgs &a, int i, int &m, int &partner) {
+  m = i * 4; partner = m;
+  if (MODE == GEMM_SWIGLU_T) partner = m + kTcBoxRows;
+  if (MODE == GEMM_QKV_T) {
+    const int half = a.qkv.hd >> 1, head = m / half;
+    m += head * half;
+    partner = m + half;
+  }
 }
 
 template <int NPAD, int MODE>
-__global__ void __launch_bounds__(kThreads, 1)
-gemm_tc_kernel(const __grid_constant__ TcGemmArgs args, int n_tiles, int KB, int pieces_max) {
+__global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_constant__ TcGemmArgs args, int n_tiles, int KB, int S) {
   using Cfg = TcCfg<NPAD>;
   constexpr int STAGES = Cfg::kStages;
   extern __shared__ uint8_t smem_raw[];
@@ -64,232 +153,186 @@ gemm_tc_kernel(const __grid_constant__ TcGemmArgs args, int n_tiles, int KB, int
   // bars: full[STAGES] | empty[STAGES] | acc_full[2] | acc_empty[2]
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * STAGES + 4);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-  volatile int *last_flag = reinterpret_cast<volatile int *>(tmem_slot + 2);
-  volatile int *wait_ok = reinterpret_cast<volatile int *>(tmem_slot + 4);      // [2], alternating per tile
+  volatile int *wait_ok = reinterpret_cast<volatile int *>(tmem_slot + 2);      // [2], alternating per tile
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
   auto accf_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + b); };
   auto acce_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + 2 + b); };
-
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int G = gridDim.x, c = blockIdx.x;
-  const long long U = (long long)n_tiles * KB;
-  const long long u0 = cta_begin(U, G, c), u1 = cta_begin(U, G, c + 1);
+  // S > 1: the cluster's CTAs share tile blockIdx.x / S; S = 1: tiles blockIdx.x, + gridDim.x, ...
+  const int rank = S > 1 ? (int)cluster_rank() : 0;
+  const int tile0 = S > 1 ? (int)blockIdx.x / S : (int)blockIdx.x, step = S > 1 ? n_tiles : (int)gridDim.x;
+  const int kb0 = KB * rank / S, kb1 = KB * (rank + 1) / S;
+  const int kb_half = kb1 - kb0 > 1 ? (kb0 + kb1) / 2 : kb1;     // the second accumulator's first k-block
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), 4); }
     *abort_flag = 0;
-    *last_flag = 0;
+    // a wait gives up after two seconds, long after every CTA (one per SM) has started
+    if (args.reset_status && blockIdx.x == 0) *args.status = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(Cfg::kTmemCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::);
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (warp == 1) tmem_alloc(smem_u32(tmem_slot), Cfg::kTmemCols);
+  tc_fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      long long issued = 0;
+      const uint64_t policy = l2_policy_evict_first();
+      int s = 0, issued = 0;
+      uint32_t ph = 0;
       bool ok = true;
-      for (long long u = u0; u < u1 && ok;) {
-        const int tile = (int)(u / KB), kb0 = (int)(u % KB);
-        const int kb1 = (int)min((long long)KB, kb0 + (u1 - u));
+      const uint32_t box_bytes = (uint32_t)args.w_box_rows * kTcBlockK * 2;
+      for (int tile = tile0; tile < n_tiles && ok; tile += step) {
         const TileInfo ti = tile_info(args, tile);
-        const bool second = (MODE == GEMM_SWIGLU_T) || (ti.row0 + kTcBoxRows < args.seg_n[ti.seg]);
-        const uint32_t bytes = (second ? 2 : 1) * kBoxBytes + NPAD * kTcBlockK * 2;
+        const bool second = MODE == GEMM_SWIGLU_T || (args.w_box_rows < args.tile_rows && ti.row0 + args.w_box_rows < args.seg_n[ti.seg]);
+        const CUtensorMap *w0 = &args.w[ti.seg], *w1 = MODE == GEMM_SWIGLU_T ? &args.w[1] : w0;
+        const int row1 = MODE == GEMM_SWIGLU_T ? ti.row0 : ti.row0 + args.w_box_rows;
+        const uint32_t bytes = (second ? 2 : 1) * box_bytes + (uint32_t)args.a_box_rows * kTcBlockK * 2;
         for (int kb = kb0; kb < kb1; ++kb, ++issued) {
-          const int s = (int)(issued % STAGES);
-          const uint32_t ph = (uint32_t)((issued / STAGES) & 1);
           if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
           const uint32_t dst = smem_u32(ring + (size_t)s * Cfg::kStageBytes);
           mbar_expect_tx(full_bar(s), bytes);
-          if (MODE == GEMM_SWIGLU_T) {
-            tma_load_2d(dst, &args.w[0], kb * kTcBlockK, ti.row0, full_bar(s));
-            tma_load_2d(dst + kBoxBytes, &args.w[1], kb * kTcBlockK, ti.row0, full_bar(s));
+          if (args.stream_weights) {
+            tma_load_2d_hint(dst, w0, kb * kTcBlockK, ti.row0, full_bar(s), policy);
+            if (second) tma_load_2d_hint(dst + box_bytes, w1, kb * kTcBlockK, row1, full_bar(s), policy);
           } else {
-            tma_load_2d(dst, &args.w[ti.seg], kb * kTcBlockK, ti.row0, full_bar(s));
-            if (second) tma_load_2d(dst + kBoxBytes, &args.w[ti.seg], kb * kTcBlockK, ti.row0 + kTcBoxRows, full_bar(s));
+            tma_load_2d(dst, w0, kb * kTcBlockK, ti.row0, full_bar(s));
+            if (second) tma_load_2d(dst + box_bytes, w1, kb * kTcBlockK, row1, full_bar(s));
           }
           tma_load_2d(dst + kStageWBytes, &args.a, kb * kTcBlockK, args.row0, full_bar(s));
+          if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
-        u += kb1 - kb0;
       }
-      if (!ok) {
-        // wait (bounded) for the copies still in flight before the CTA's shared memory goes away
-        long long first = issued > STAGES ? issued - STAGES : 0;
-        for (long long i = first; i < issued; ++i) {
-          unsigned long long t0 = globaltimer_ns();
-          while (!mbar_try_wait(full_bar((int)(i % STAGES)), (uint32_t)((i / STAGES) & 1)))
-            if (globaltimer_ns() - t0 > kWaitLimitNs) break;
-        }
+      if (!ok) {                                   // copies in flight land before the shared memory goes away
+        const unsigned long long t0 = globaltimer_ns();
+        while (globaltimer_ns() - t0 < 200000ull) {}
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     if (lane == 0) {
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NPAD >> 3) << 17) | ((uint32_t)(kTcBlockM >> 4) << 24);
-      long long consumed = 0;
-      int seg_idx = 0;
+      const uint32_t idesc = umma_idesc_bf16(NPAD);
+      int s = 0, ti = 0;
+      uint32_t ph = 0;
       bool ok = true;
-      for (long long u = u0; u < u1 && ok; ++seg_idx) {
-        const int kb0 = (int)(u % KB);
-        const int kb1 = (int)min((long long)KB, kb0 + (u1 - u));
-        const int ab = seg_idx & 1;
-        const uint32_t aph = (uint32_t)((seg_idx >> 1) & 1);
-        if (!mbar_wait(acce_bar(ab), aph ^ 1u, abort_flag)) { ok = false; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d_tmem = tmem_base + (uint32_t)(ab * NPAD);
-        for (int kb = kb0; kb < kb1; ++kb, ++consumed) {
-          const int s = (int)(consumed % STAGES);
-          const uint32_t ph = (uint32_t)((consumed / STAGES) & 1);
+      for (int tile = tile0; tile < n_tiles && ok; tile += step, ++ti) {
+        const int ab = ti % Cfg::kBufs;
+        if (!mbar_wait(acce_bar(ab), (uint32_t)((ti / Cfg::kBufs) & 1) ^ 1u, abort_flag)) break;
+        tc_fence_after();
+        uint32_t d_tmem = tmem_base + (uint32_t)(ab * 2 * NPAD), acc = 0u;
+        for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(full_bar(s), ph, abort_flag)) { ok = false; break; }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t wa = smem_u32(ring + (size_t)s * Cfg::kStageBytes);
           const uint64_t da = umma_desc(wa), db = umma_desc(wa + kStageWBytes);
+          if (kb == kb_half) { d_tmem += NPAD; acc = 0u; }
 #pragma unroll
-          for (int k = 0; k < kTcBlockK / 16; ++k)
-            umma_bf16(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+          for (int k = 0; k < kTcBlockK / 16; ++k) {
+            umma_bf16(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, acc);
+            acc = 1u;
+          }
           umma_commit(empty_bar(s));            // the stage is free once these MMAs have read it
+          if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
         if (ok) umma_commit(accf_bar(ab));      // accumulator complete
-        u += kb1 - kb0;
       }
     }
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..5)
     const int q = warp & 3;                     // TMEM lane quarter this warp may read
-    const int m = q * 32 + lane;                // row of the tile held by this thread
+    const int m = q * 32 + lane;                // weight row of the tile held by this thread
     const int et = threadIdx.x - 64;            // 0..127 among the epilogue threads
-    int seg_idx = 0;
-    bool ok = true;
-    for (long long u = u0; u < u1 && ok; ++seg_idx) {
-      const int tile = (int)(u / KB), kb0 = (int)(u % KB);
-      const int kb1 = (int)min((long long)KB, kb0 + (u1 - u));
-      const int ab = seg_idx & 1;
-      const uint32_t aph = (uint32_t)((seg_idx >> 1) & 1);
+    const int n_items = items_of<MODE>(args);
+    int ti = 0;
+    for (int tile = tile0; tile < n_tiles; tile += step, ++ti) {
+      const int ab = ti % Cfg::kBufs;
       // one thread waits, all 128 take the same decision (a bail-out must not split the group)
-      if (et == 0) wait_ok[seg_idx & 1] = mbar_wait(accf_bar(ab), aph, abort_flag) ? 1 : 0;
+      if (et == 0) wait_ok[ti & 1] = mbar_wait(accf_bar(ab), (uint32_t)((ti / Cfg::kBufs) & 1), abort_flag) ? 1 : 0;
       asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (!wait_ok[seg_idx & 1]) { ok = false; break; }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (!wait_ok[ti & 1]) break;
+      tc_fence_after();
       constexpr int CH = Cfg::kChunk;
-      const TileInfo ti = tile_info(args, tile);
-      const bool whole = (kb0 == 0 && kb1 == KB);
-      const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * NPAD);
-      int n_pieces = 1, piece = 0;
-      if (!whole) {
-        const int first_owner = unit_owner(U, G, (long long)tile * KB);
-        const int last_owner = unit_owner(U, G, (long long)tile * KB + KB - 1);
-        n_pieces = last_owner - first_owner + 1;
-        piece = c - first_owner;
-      }
-      // values of the tile's row m for token rows c0 .. c0 + CH - 1 -> the projection's output
-      auto finish_chunk = [&](int c0, float *v) {
-        if (MODE == GEMM_SWIGLU_T) {
-#pragma unroll
-          for (int r = 0; r < CH; ++r) staging[m * (CH + 1) + r] = v[r];
-          asm volatile("bar.sync 1, 128;" ::: "memory");
-          for (int i = et; i < kTcBoxRows * CH; i += 128) {
-            const int cc = i % kTcBoxRows, r = c0 + i / kTcBoxRows;
-            const int col = ti.row0 + cc;
-            if (r < args.R && col < args.seg_n[0]) {
-              const float g = staging[cc * (CH + 1) + (r - c0)], up = staging[(cc + kTcBoxRows) * (CH + 1) + (r - c0)];
-              args.out_bf16[(size_t)(args.row0 + r) * args.ldo + col] = __float2bfloat16_rn(ptx::silu_mul(g, up));
-            }
-          }
-          asm volatile("bar.sync 1, 128;" ::: "memory");
-        } else {
-          const int n = ti.row0 + m;
-          if (n < args.seg_n[ti.seg]) {
-            const int col = ti.col0 + n;
-            if (MODE == GEMM_ADD_F32) {
-              // residual add: all of the chunk's old values are fetched before the first store (a read-modify-write
-              // per row would be one dependent round trip per row)
-              float old[CH];
-#pragma unroll
-              for (int i = 0; i < CH; ++i)
-                old[i] = c0 + i < args.R ? __ldcg(args.out_f32 + (size_t)(args.row0 + c0 + i) * args.ldo + col) : 0.f;
-#pragma unroll
-              for (int i = 0; i < CH; ++i)
-                if (c0 + i < args.R) args.out_f32[(size_t)(args.row0 + c0 + i) * args.ldo + col] = old[i] + v[i];
-            } else {
-#pragma unroll
-              for (int i = 0; i < CH; ++i) {
-                const int r = c0 + i;
-                if (r < args.R) {
-                  if (MODE == GEMM_STORE_F32) args.out_f32[(size_t)(args.row0 + r) * args.ldo + col] = v[i];
-                  else args.out_bf16[(size_t)args.dst[args.row0 + r] * args.ldo + col] = __float2bfloat16_rn(v[i]);
-                }
-              }
-            }
-          }
-        }
-      };
-      float *mine = args.pieces + ((size_t)tile * pieces_max + piece) * NPAD * kTcBlockM;
+      const TileInfo info = tile_info(args, tile);
+      const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * 2 * NPAD);
+      float *part = S > 1 ? reinterpret_cast<float *>(ring) : staging;       // S > 1: every load of the CTA has been consumed
 #pragma unroll 1
-      for (int c0 = 0; c0 < NPAD; c0 += CH) {
-        float v[CH];
+      for (int c0 = 0; c0 < NPAD && c0 < args.R; c0 += CH) {
+        float v[CH], v2[CH];
 #pragma unroll
         for (int j = 0; j < CH / 16; ++j) tmem_ld16(tbase + (uint32_t)(c0 + j * 16), v + j * 16);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (c0 + CH >= NPAD) {                     // accumulator fully read: hand it back to the MMA warp
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(acce_bar(ab));
-        }
-        if (c0 >= args.R) continue;                // padding rows: nothing to write
-        if (whole) finish_chunk(c0, v);
-        else {
+        if (kb_half < kb1) {
 #pragma unroll
-          for (int i = 0; i < CH; ++i) mine[(c0 + i) * kTcBlockM + m] = v[i];
+          for (int j = 0; j < CH / 16; ++j) tmem_ld16(tbase + (uint32_t)(NPAD + c0 + j * 16), v2 + j * 16);
         }
-      }
-      if (!whole) {
-        // split tile: this piece is published; the last arriver sums all pieces in piece order
-        __threadfence();
+        tmem_ld_wait();
+        if (kb_half < kb1) {
+#pragma unroll
+          for (int r = 0; r < CH; ++r) v[r] += v2[r];
+        }
+        float *to = part + (S > 1 ? c0 * kLd : 0);
+#pragma unroll
+        for (int r = 0; r < CH; ++r) to[r * kLd + m] = v[r];
+        if (S > 1) continue;
         asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (et == 0) {
-          int prev = atomicAdd(&args.counters[tile], 1);
-          int last = (prev == n_pieces - 1);
-          if (last) args.counters[tile] = 0;
-          *last_flag = last;
-          __threadfence();
+        const int rows = min(CH, args.R - c0);
+        for (int i = et; i < rows * n_items; i += 128) {
+          const int r = i / n_items;
+          int mm, pp;
+          item_at<MODE>(args, i - r * n_items, mm, pp);
+          const float4 a4 = *reinterpret_cast<const float4 *>(to + r * kLd + mm), b4 = *reinterpret_cast<const float4 *>(to + r * kLd + pp);
+          finish4<MODE>(args, info, c0 + r, mm, a4, b4);
         }
         asm volatile("bar.sync 1, 128;" ::: "memory");
-        const bool finish = (*last_flag != 0);
-        asm volatile("bar.sync 1, 128;" ::: "memory");   // last_flag may be rewritten by the next tile
-        if (finish) {
-#pragma unroll 1
-          for (int c0 = 0; c0 < NPAD && c0 < args.R; c0 += CH) {
-            float v[CH];
-#pragma unroll
-            for (int i = 0; i < CH; ++i) v[i] = 0.f;
-            for (int p = 0; p < n_pieces; ++p) {
-              const float *src = args.pieces + ((size_t)tile * pieces_max + p) * NPAD * kTcBlockM;
-#pragma unroll
-              for (int i = 0; i < CH; ++i) v[i] += __ldcg(src + (c0 + i) * kTcBlockM + m);
-            }
-            finish_chunk(c0, v);
-          }
-        }
       }
-      u += kb1 - kb0;
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acce_bar(ab));
     }
   }
-  // ------------------------------------------------------------------ teardown
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == 1) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(Cfg::kTmemCols));
+  __syncwarp();
+  if (S > 1) {
+    // ------------------------------------------------------------------ sums across the cluster, in rank order
+    __syncthreads();
+    cluster_sync();
+    const TileInfo info = tile_info(args, tile0);
+    const int r0 = args.R * rank / S, r1 = args.R * (rank + 1) / S, n_items = items_of<MODE>(args);
+    const uint32_t base = smem_u32(ring);
+    const bool ok = !*abort_flag;
+    for (int i = threadIdx.x; i < (r1 - r0) * n_items && ok; i += kThreads) {
+      const int r = r0 + i / n_items;
+      int mm, pp;
+      item_at<MODE>(args, i % n_items, mm, pp);
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+      for (int p0 = 0; p0 < S; p0 += 4) {                         // up to four ranks' loads in flight
+        float4 xs[4], ys[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          if (p0 + p >= S) continue;
+          xs[p] = ld_cluster4(base + (uint32_t)(r * kLd + mm) * 4u, (uint32_t)(p0 + p));
+          if (MODE == GEMM_SWIGLU_T || MODE == GEMM_QKV_T) ys[p] = ld_cluster4(base + (uint32_t)(r * kLd + pp) * 4u, (uint32_t)(p0 + p));
+        }
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          if (p0 + p >= S) continue;
+          x.x += xs[p].x; x.y += xs[p].y; x.z += xs[p].z; x.w += xs[p].w;
+          if (MODE == GEMM_SWIGLU_T || MODE == GEMM_QKV_T) { y.x += ys[p].x; y.y += ys[p].y; y.z += ys[p].z; y.w += ys[p].w; }
+        }
+      }
+      finish4<MODE>(args, info, r, mm, x, y);
+    }
+    __syncwarp();
+    cluster_sync();                             // nobody leaves while its partial sums are being read
   }
+  // ------------------------------------------------------------------ teardown
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) tmem_dealloc(tmem_base, Cfg::kTmemCols);
   if (threadIdx.x == 0 && *abort_flag) atomicExch(args.status, 1);
 }
 
@@ -299,25 +342,32 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 EncodeTiledFn g_encode = nullptr;
 
 template <int NPAD, int MODE>
-int launch_t(const TcGemmArgs &args, const TcGemmPlan &plan, cudaStream_t s) {
+int launch_t(const TcGemmArgs &args, int n_tiles, int S, int grid, cudaStream_t s) {
   using Cfg = TcCfg<NPAD>;
   static bool attr_set = false;
   if (!attr_set) {
     HSD_CUDA_OK(cudaFuncSetAttribute(gemm_tc_kernel<NPAD, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
     attr_set = true;
   }
-  gemm_tc_kernel<NPAD, MODE><<<plan.grid, kThreads, Cfg::kSmemBytes, s>>>(args, plan.n_tiles, plan.kb, plan.pieces_max);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = Cfg::kSmemBytes; cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = S; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  HSD_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<NPAD, MODE>, args, n_tiles, args.K / kTcBlockK, S));
   hsd_count_launches(1);
   return hsd_launch_status();
 }
 
 template <int NPAD>
-int launch_mode(const TcGemmArgs &args, const TcGemmPlan &plan, cudaStream_t s) {
+int launch_mode(const TcGemmArgs &args, int n_tiles, int S, int grid, cudaStream_t s) {
   switch (args.mode) {
-    case GEMM_STORE_F32: return launch_t<NPAD, GEMM_STORE_F32>(args, plan, s);
-    case GEMM_ADD_F32: return launch_t<NPAD, GEMM_ADD_F32>(args, plan, s);
-    case GEMM_STORE_T_SCATTER: return launch_t<NPAD, GEMM_STORE_T_SCATTER>(args, plan, s);
-    case GEMM_SWIGLU_T: return launch_t<NPAD, GEMM_SWIGLU_T>(args, plan, s);
+    case GEMM_STORE_F32: return launch_t<NPAD, GEMM_STORE_F32>(args, n_tiles, S, grid, s);
+    case GEMM_ADD_F32: return launch_t<NPAD, GEMM_ADD_F32>(args, n_tiles, S, grid, s);
+    case GEMM_STORE_T_SCATTER: return launch_t<NPAD, GEMM_STORE_T_SCATTER>(args, n_tiles, S, grid, s);
+    case GEMM_SWIGLU_T: return launch_t<NPAD, GEMM_SWIGLU_T>(args, n_tiles, S, grid, s);
+    case GEMM_QKV_T: return launch_t<NPAD, GEMM_QKV_T>(args, n_tiles, S, grid, s);
     default: return HSD_E_INVALID_ARG;
   }
 }
@@ -365,16 +415,31 @@ TcGemmPlan tc_plan(const int *seg_n, int n_segs, int mode, int K, int npad, int 
   return p;
 }
 
+// Rows of a tile of one matrix on its own: 128, or as many fewer as spread the rows evenly over the rounds the SMs need.
+int tc_tile_rows(int N, int sm_count) {
+  if (ceil_div(N, kTcBlockM) * 2 <= sm_count) return kTcBlockM;       // k-blocks are divided: full tiles
+  const int rounds = ceil_div(N, kTcBlockM * sm_count);
+  return std::min(kTcBlockM, ceil_div(ceil_div(N, rounds * sm_count), 8) * 8);
+}
+
 int launch_gemm_tc(const TcGemmArgs &args, int sm_count, cudaStream_t s) {
-  if (args.R < 1 || args.R > 256 || args.K % kTcBlockK != 0) return HSD_E_UNSUPPORTED;
-  const int npad = tc_npad(args.R);
-  TcGemmPlan plan = tc_plan(args.seg_n, args.n_segs, args.mode, args.K, npad, sm_count);
-  switch (npad) {
-    case 16: return launch_mode<16>(args, plan, s);
-    case 32: return launch_mode<32>(args, plan, s);
-    case 64: return launch_mode<64>(args, plan, s);
-    case 128: return launch_mode<128>(args, plan, s);
-    default: return launch_mode<256>(args, plan, s);
+  if (args.R < 1 || args.R > 256 || args.K < kTcBlockK || args.K % kTcBlockK != 0) return HSD_E_UNSUPPORTED;
+  int n_tiles = 0;
+  if (args.mode == GEMM_SWIGLU_T) n_tiles = ceil_div(args.seg_n[0], kTcBoxRows);
+  else
+    for (int i = 0; i < args.n_segs; ++i) n_tiles += ceil_div(args.seg_n[i], args.tile_rows);
+  // k-blocks divided over at most eight CTAs (a portable cluster) while the tiles alone leave half the SMs idle; the
+  // division does not depend on the number of rows, so neither does a row's result.  Clusters of more than four are
+  // not scheduled on all SMs at once (see the clusters of eight in sampling.cu): four at most from 16 tiles on.
+  int S = std::max(1, std::min(sm_count / n_tiles, args.K / kTcBlockK));
+  S = std::min(S, n_tiles >= 16 ? 4 : 8);
+  const int grid = S > 1 ? n_tiles * S : std::min(n_tiles, sm_count);
+  switch (tc_npad(args.R)) {
+    case 16: return launch_mode<16>(args, n_tiles, S, grid, s);
+    case 32: return launch_mode<32>(args, n_tiles, S, grid, s);
+    case 64: return launch_mode<64>(args, n_tiles, S, grid, s);
+    case 128: return launch_mode<128>(args, n_tiles, S, grid, s);
+    default: return launch_mode<256>(args, n_tiles, S, grid, s);
   }
 }
 

@@ -1,9 +1,7 @@
 // Weight-streaming skinny GEMM on the 5th-generation tensor cores (tcgen05 + TMEM), operands fed
-// by TMA.  out[r, n] = sum_k A[r, k] * W[n, k]: the weight rows sit on the MMA's M side (128 per
-// tile), the token rows on its N side (padded to 16..128), so every weight byte is read from HBM
-// exactly once per pass whatever the row count.  The k-blocks of all tiles are split evenly over a
-// persistent grid (stream-K); tiles cut by a split are finished by whichever CTA arrives last,
-// summing the pieces in a fixed order (bit-reproducible, no CTA ever waits for another).
+// by TMA.  out[r, n] = sum_k A[r, k] * W[n, k]: the weight rows sit on the MMA's M side (up to 128 per
+// tile), the token rows on its N side (padded to 16..256), so every weight byte is read from HBM
+// exactly once per pass whatever the row count.
 #pragma once
 #include <cuda.h>
 #include "common.cuh"
@@ -20,17 +18,29 @@ int tc_init();                     // HSD_OK when the tensor-map encoder is avai
 // 2-D bf16 tensor map over a row-major [rows, cols] matrix, box = [box_rows, 64], 128-byte swizzle.
 int tc_make_map(CUtensorMap *map, const void *base, long long rows, long long cols, int box_rows);
 
+// Split of a projection's (tile, k-block) units over the CTAs of the one-launch forward, and the scratch its pieces take.
 struct TcGemmPlan {
   int n_tiles, kb, grid, pieces_max;
-  size_t scratch_bytes;            // split pieces + per-tile counters
+  size_t scratch_bytes;
 };
-// Decomposition for a GEMM with the given segment sizes (mode as in GemmMode), K, row padding.
 TcGemmPlan tc_plan(const int *seg_n, int n_segs, int mode, int K, int npad, int sm_count);
 int tc_npad(int rows);             // 16, 32, 64 or 128 (rows <= 128)
 
+// Where the q / k / v projection's rows go (GEMM_QKV_T): q rotated -> q; k rotated, v -> their cache pages.
+struct TcQkv {
+  const int *row_seq, *row_pos, *page_table;
+  const float *cos_tab, *sin_tab;
+  __nv_bfloat16 *q, *k_pool, *v_pool;
+  int nq, hd, page, pages_per_seq, n_pages;
+};
 struct TcGemmArgs {
-  CUtensorMap w[3];                // weight maps (box rows 64)
-  CUtensorMap a;                   // activation map (box rows = npad), covers the whole buffer
+  CUtensorMap w[3];                // weight maps
+  CUtensorMap a;                   // activation map, covers the whole buffer
+  int tile_rows = kTcBlockM, w_box_rows = kTcBoxRows;   // weight rows of a tile (<= 128; SWIGLU: 64 gate + 64 up) and of one box of their maps
+  int a_box_rows;                  // rows of one box of the activation map (R .. row padding)
+  int stream_weights = 0;          // 1: the weights will not be read again soon (evict-first in L2)
+  int reset_status = 0;            // 1: the kernel clears the status word first
+  TcQkv qkv;
   int seg_n[3], n_segs;
   int K, R, row0;                  // R rows of A starting at buffer row row0
   int mode;                        // GemmMode
@@ -38,10 +48,9 @@ struct TcGemmArgs {
   __nv_bfloat16 *out_bf16;         // STORE_T_SCATTER: [dst[row], ldo];  SWIGLU_T: [row, ldo]
   const long long *dst;
   int ldo;
-  float *pieces;                   // scratch: split pieces
-  int *counters;                   // scratch: per-tile arrival counters (zero on entry, zero on exit)
   int *status;                     // device word: set non-zero if a bounded wait gave up
 };
+int tc_tile_rows(int N, int sm_count);
 int launch_gemm_tc(const TcGemmArgs &args, int sm_count, cudaStream_t s);
 
 }  // namespace hsd

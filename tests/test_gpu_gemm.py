@@ -42,3 +42,19 @@ def test_gemm_rejects_bad_shapes(lib):
     W = torch.zeros(64, 100, dtype=torch.bfloat16, device="cuda")
     with pytest.raises(lib.HsdError):
         lib.hsd_gemm_bf16(A, W)          # K not a multiple of 64
+
+
+@pytest.mark.parametrize("R,N,K", [(24, 14257, 256),     # whole tiles of 104 rows, the last one of 9
+                                   (256, 2048, 5632),    # k-blocks over a cluster of four, one accumulator buffer
+                                   (5, 100, 64),         # one k-block: no split, no second accumulator
+                                   (17, 1000, 192),      # three k-blocks over a cluster of three
+                                   (33, 19100, 128)])    # more tiles than SMs: a CTA's second tile
+def test_gemm_tile_and_cluster_edges(lib, R, N, K):
+    g = torch.Generator().manual_seed(R + N + K)
+    A = torch.randn(R, K, generator=g).to(torch.bfloat16).cuda()
+    W = (torch.randn(N, K, generator=g) * 0.05).to(torch.bfloat16).cuda()
+    out = lib.hsd_gemm_bf16(A, W).double()
+    ref = A.double() @ W.double().T
+    # fp32 accumulation: 2^-23 per addition of a chain of K / 32 partial sums of this size, at most
+    bound = 2.0 ** -23 * (K / 32) * (A.double().abs() @ W.double().abs().T) + 1e-7
+    assert bool(((out - ref).abs() < bound).all())
