@@ -983,7 +983,7 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   M.use_persist = coop != 0 && fwd_persist_supported(md.hd, md.nq / md.nkv) && md.d % 256 == 0 && md.d <= 4096 &&
                   (md.d / kTcBlockM) * 2 <= c->sm_count && md.n_layers <= 64 && (md.page & (md.page - 1)) == 0 && md.page >= 16;
-  M.use_prompt = M.use_persist && prompt_path_dims(model) && lay.max_rows > kPrefillRows;
+  M.use_prompt = M.use_persist && prompt_path_dims(model);
   if (M.use_prompt) {
     M.kvmaps.resize((size_t)md.n_layers * 2);
     const long long rows = (long long)md.nkv * md.n_pages * md.page;
@@ -1195,7 +1195,11 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
   for (int p = L.n_pages - 1; p >= 0; --p) c->free_pages.push_back(p);
   HSD_CUDA_OK(cudaMemcpyAsync(c->dev<int>(L.tokens), token_ids, (size_t)n_tokens * 4, cudaMemcpyDeviceToDevice, s));
   HSD_TRY(ensure_pages(c, 0, n_tokens));
-  const int R = n_tokens, n_attn = (R + kAttnRows - 1) / kAttnRows;
+  // Attention on tensor memory where the model allows it (one query tile per item); the normalised rows of the chosen
+  // layers then collect in the buffer of the split attention's partials, idle here, so that the head's weights are read
+  // once for all of them instead of once per layer.
+  const bool tm = M.use_prompt;
+  const int R = n_tokens, per_item = tm ? prompt_attn_tokens(md.nq / md.nkv) : kAttnRows, n_attn = (R + per_item - 1) / per_item;
   char *host, *devp;
   HSD_TRY(ring_acquire(c, &host, &devp));
   size_t o_seq = 0, o_pos = align_up(o_seq + (size_t)R * 4, 16), o_attn = align_up(o_pos + (size_t)R * 4, 16),
@@ -1206,7 +1210,7 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
   int4 *attn = (int4 *)(host + o_attn);
   long long *ldst = (long long *)(host + o_dst);
   for (int r = 0; r < R; ++r) { row_seq[r] = 0; row_pos[r] = r; lsrc[r] = r; ldst[r] = r; }
-  for (int i = 0; i < n_attn; ++i) attn[i] = make_int4(i * kAttnRows, std::min(kAttnRows, R - i * kAttnRows), 0, i * kAttnRows);
+  for (int i = 0; i < n_attn; ++i) attn[i] = make_int4(i * per_item, std::min(per_item, R - i * per_item), 0, i * per_item);
   HSD_CUDA_OK(cudaMemcpyAsync(devp, host, bytes, cudaMemcpyHostToDevice, s));
   HSD_TRY(upload_page_tables(c));
   RowBatch rb;
@@ -1221,14 +1225,37 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
   float *qkv = c->dev<float>(ML.qkv);
   const int *pt = c->dev<int>(L.page_table);
   const size_t es = elem_size(md.dtype);
+  PromptAttnArgs pa = {};
+  pa.q = (const __nv_bfloat16 *)q; pa.att = (__nv_bfloat16 *)att; pa.items = rb.attn; pa.n_items = n_attn; pa.page_table = pt;
+  pa.nq = md.nq; pa.nkv = md.nkv; pa.hd = md.hd; pa.pages_per_seq = md.pages_per_seq; pa.n_pages = md.n_pages;
+  while ((1 << pa.page_shift) < md.page) ++pa.page_shift;
+  pa.status = (int *)(c->ws + c->status_off);
+  char *rows_buf = c->dev<char>(ML.partials);
+  const size_t row_bytes = (size_t)md.d * es, rows_cap = (size_t)ML.partial_rows * md.nq * (md.hd + 2) * 4 / row_bytes;
+  const int layers_cap = tm ? (int)std::min<size_t>(rows_cap / R, (size_t)n_layers_sel) : 0;     // layers whose rows fit the buffer
+  int held = 0, next = 0;                                 // layers in the buffer; layers normalised so far
+  auto flush = [&]() -> int {                             // logits of the layers held: next - held ..
+    void *out = (char *)out_logits + (size_t)(next - held) * R * md.V * es;
+    BigGemmArgs g = {};
+    g.R = held * R; g.K = md.d; g.mode = BIG_LOGITS; g.seg_n[0] = md.V; g.ldo = md.V;
+    g.out_bf16 = (__nv_bfloat16 *)out; g.status = pa.status;
+    g.w[0] = M.wmaps[(size_t)md.n_layers * 7 + kHeadMaps - 1];
+    held = 0;
+    int st = tc_make_map(&g.a, rows_buf, g.R, md.d, kBigBoxRowsA);
+    return st ? st : launch_gemm_big(g, c->sm_count, s);
+  };
   HSD_TRY(launch_embed(md, M.embed, c->dev<int>(L.tokens), rb, x, s));
-  int next = 0;
   for (int l = 0; l < md.n_layers && next < n_layers_sel; ++l) {
     const void *const *w = &M.lw[(size_t)l * 9];
     void *kp = c->ws + ML.k_pool + ML.pool_layer_stride * l, *vp = c->ws + ML.v_pool + ML.pool_layer_stride * l;
     HSD_TRY(launch_rmsnorm(md, x, w[0], nullptr, R, h, s));
     HSD_TRY(project_qkv(c, M, l, rb, h, qkv, pt, kp, vp, q));
-    HSD_TRY(launch_attention(md, q, rb, pt, kp, vp, c->dev<float>(ML.partials), keys_per_split, n_splits, att, s));
+    if (tm) {
+      pa.k = M.kvmaps[2 * l]; pa.v = M.kvmaps[2 * l + 1];
+      HSD_TRY(launch_prompt_attention(pa, s));
+    } else {
+      HSD_TRY(launch_attention(md, q, rb, pt, kp, vp, c->dev<float>(ML.partials), keys_per_split, n_splits, att, s));
+    }
     GemmSegs o_segs = {{w[4], nullptr, nullptr}, {md.d, 0, 0}, 1};
     HSD_TRY(gemm(c, M, 1, att, R, md.nq * md.hd, o_segs, l * 7 + 3, GEMM_ADD_F32, x, nullptr, nullptr));
     HSD_TRY(launch_rmsnorm(md, x, w[5], nullptr, R, h, s));
@@ -1236,15 +1263,21 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
     HSD_TRY(gemm(c, M, 0, h, R, md.d, gu_segs, l * 7 + 4, GEMM_SWIGLU_T, nullptr, act, nullptr));
     GemmSegs d_segs = {{w[8], nullptr, nullptr}, {md.d, 0, 0}, 1};
     HSD_TRY(gemm(c, M, 2, act, R, md.ff, d_segs, l * 7 + 6, GEMM_ADD_F32, x, nullptr, nullptr));
-    if (layers[next] == l + 1) {                         // exit after layer l + 1: shared final norm + head on every row
-      // (the normalised rows go to the h buffer, free between two layers and large enough for every row; the
-      // buffer of the generation path's final norm holds the few logit rows of a verification only)
-      HSD_TRY(launch_rmsnorm(md, x, M.final_norm, rb.lrow_src, R, h, s));
-      GemmSegs lm_segs = {{M.lm_head, nullptr, nullptr}, {md.V, 0, 0}, 1};
-      HSD_TRY(gemm(c, M, 0, h, R, md.d, lm_segs, md.n_layers * 7 + kHeadMaps - 1, GEMM_STORE_T_SCATTER, nullptr,
-                   (char *)out_logits + (size_t)next * R * md.V * es, rb.lrow_dst));
+    if (layers[next] != l + 1) continue;
+    // exit after layer l + 1: shared final norm + head on every row
+    if (layers_cap > 0) {
+      HSD_TRY(launch_rmsnorm(md, x, M.final_norm, rb.lrow_src, R, rows_buf + (size_t)held * R * row_bytes, s));
       ++next;
+      if (++held == layers_cap || next == n_layers_sel) HSD_TRY(flush());
+      continue;
     }
+    // (the normalised rows go to the h buffer, free between two layers and large enough for every row; the
+    // buffer of the generation path's final norm holds the few logit rows of a verification only)
+    HSD_TRY(launch_rmsnorm(md, x, M.final_norm, rb.lrow_src, R, h, s));
+    GemmSegs lm_segs = {{M.lm_head, nullptr, nullptr}, {md.V, 0, 0}, 1};
+    HSD_TRY(gemm(c, M, 0, h, R, md.d, lm_segs, md.n_layers * 7 + kHeadMaps - 1, GEMM_STORE_T_SCATTER, nullptr,
+                 (char *)out_logits + (size_t)next * R * md.V * es, rb.lrow_dst));
+    ++next;
   }
   return sync_stream(c);
 }

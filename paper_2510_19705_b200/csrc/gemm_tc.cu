@@ -428,11 +428,11 @@ int launch_gemm_tc(const TcGemmArgs &args, int sm_count, cudaStream_t s) {
   if (args.mode == GEMM_SWIGLU_T) n_tiles = ceil_div(args.seg_n[0], kTcBoxRows);
   else
     for (int i = 0; i < args.n_segs; ++i) n_tiles += ceil_div(args.seg_n[i], args.tile_rows);
-  // k-blocks divided over at most eight CTAs (a portable cluster) while the tiles alone leave half the SMs idle; the
-  // division does not depend on the number of rows, so neither does a row's result.  Clusters of more than four are
-  // not scheduled on all SMs at once (see the clusters of eight in sampling.cu): four at most from 16 tiles on.
-  int S = std::max(1, std::min(sm_count / n_tiles, args.K / kTcBlockK));
-  S = std::min(S, n_tiles >= 16 ? 4 : 8);
+  // k-blocks divided over 2, 4 or (few tiles) 8 CTAs while the tiles alone leave half the SMs idle; the division does not
+  // depend on the number of rows, so neither does a row's result.  48 clusters of three or 16 of eight do not run at
+  // once (6144 x 4096 at 128 rows: 36 us in threes, 25 us in pairs), 74 of two and 32 of four do.
+  int S = 1;
+  while (S < (n_tiles <= 14 ? 8 : 4) && n_tiles * S * 2 <= sm_count && S * 2 <= args.K / kTcBlockK) S *= 2;
   const int grid = S > 1 ? n_tiles * S : std::min(n_tiles, sm_count);
   switch (tc_npad(args.R)) {
     case 16: return launch_mode<16>(args, n_tiles, S, grid, s);
