@@ -214,7 +214,7 @@ struct Model {
   std::vector<CUtensorMap> wmaps;             // [n_layers * 7 + kHeadMaps]: wq wk wv wo wg wu wd per layer, then the levels' heads, the shared head
   CUtensorMap amaps[4][5];                    // activation buffers {h, att, act, hf} x row padding {16, 32, 64, 128, 256}
   bool use_prompt = false;                    // long prompts run forward_prompt
-  std::vector<CUtensorMap> kvmaps;            // [n_layers][2]: K and V pools of each layer, for the prompt attention
+  std::vector<CUtensorMap> kvmaps;            // [n_layers][4]: K and V pools of each layer, two box heights each, for the prompt attention
   CUtensorMap amaps_rows[4][16];              // the same buffers with a box of exactly 1..16 rows (persistent forward, few rows)
 };
 
@@ -719,7 +719,7 @@ int forward_prompt(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     g.skip_cols = last ? nqd / 256 * 256 : 0;
     HSD_TRY(product(0, md.d, l * 7, 3, BIG_QKV, nqd, nullptr, 0));
     if (last) break;
-    pa.k = M.kvmaps[2 * l]; pa.v = M.kvmaps[2 * l + 1];
+    pa.k = M.kvmaps[4 * l]; pa.k_run = M.kvmaps[4 * l + 1]; pa.v = M.kvmaps[4 * l + 2]; pa.v_run = M.kvmaps[4 * l + 3];
     HSD_TRY(launch_prompt_attention(pa, s));
     HSD_TRY(product(1, nqd, l * 7 + 3, 1, BIG_ADD_F32, md.d, x, md.d));
     HSD_TRY(launch_rmsnorm(md, x, w[5], nullptr, R, h, s));
@@ -985,11 +985,11 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
                   (md.d / kTcBlockM) * 2 <= c->sm_count && md.n_layers <= 64 && (md.page & (md.page - 1)) == 0 && md.page >= 16;
   M.use_prompt = M.use_persist && prompt_path_dims(model);
   if (M.use_prompt) {
-    M.kvmaps.resize((size_t)md.n_layers * 2);
+    M.kvmaps.resize((size_t)md.n_layers * 4);
     const long long rows = (long long)md.nkv * md.n_pages * md.page;
     for (int l = 0; l < md.n_layers && !st; ++l) {
-      st = prompt_attn_map(&M.kvmaps[2 * l], ld[l].k_pool, rows, md.hd);
-      if (!st) st = prompt_attn_map(&M.kvmaps[2 * l + 1], ld[l].v_pool, rows, md.hd);
+      st = prompt_attn_maps(&M.kvmaps[4 * l], ld[l].k_pool, rows, md.hd);
+      if (!st) st = prompt_attn_maps(&M.kvmaps[4 * l + 2], ld[l].v_pool, rows, md.hd);
     }
   }
   return st;
@@ -1251,7 +1251,7 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
     HSD_TRY(launch_rmsnorm(md, x, w[0], nullptr, R, h, s));
     HSD_TRY(project_qkv(c, M, l, rb, h, qkv, pt, kp, vp, q));
     if (tm) {
-      pa.k = M.kvmaps[2 * l]; pa.v = M.kvmaps[2 * l + 1];
+      pa.k = M.kvmaps[4 * l]; pa.k_run = M.kvmaps[4 * l + 1]; pa.v = M.kvmaps[4 * l + 2]; pa.v_run = M.kvmaps[4 * l + 3];
       HSD_TRY(launch_prompt_attention(pa, s));
     } else {
       HSD_TRY(launch_attention(md, q, rb, pt, kp, vp, c->dev<float>(ML.partials), keys_per_split, n_splits, att, s));
