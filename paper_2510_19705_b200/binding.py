@@ -28,6 +28,7 @@ def library():
                            "(there is no fallback path)")
         lib = ctypes.CDLL(LIB_PATH)
         _declare(lib)
+        _declare_engine(lib)
         _lib = lib
     return _lib
 
@@ -48,7 +49,7 @@ def _declare(lib):
 
 
 def _check(status):
-    if status != 0:
+    if status:
         raise HsdError("hsd call failed: %s (%d)" % (library().hsd_strerror(status).decode(), status))
 
 
@@ -63,11 +64,13 @@ def _dtype_code(t):
 def _dev(t):
     if not (t.is_cuda and t.is_contiguous()):
         raise HsdError("expected a contiguous CUDA tensor")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current device's current stream.  (The raw handle: a call's stream object, pointer objects and prototype
+    set-up took longer on the host, 12 us, than its kernel on the GPU.)"""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def hsd_draft_sample(logits, seed, call_serial, out_tokens=None):
@@ -222,7 +225,6 @@ class Hsd:
 
     def __init__(self, cfg, weights, exits, T, max_batch, max_seq, page_size=16):
         lib = library()
-        _declare_engine(lib)
         self._lib = lib
         self.T = list(T)
         self.weights = weights                      # keep the device buffers alive
@@ -357,7 +359,6 @@ def read_trace(path):
 def hsd_expected_latency(costs, alphas, T):
     """Theorem 3.2 for the chain with costs c_0..c_K, alphas[i] = rate level i -> i+1, parameters T."""
     lib = library()
-    _declare_engine(lib)
     n = len(costs)
     out = ctypes.c_double()
     _check(lib.hsd_expected_latency((ctypes.c_double * n)(*costs), (ctypes.c_double * max(1, n - 1))(*(alphas or [0])), n,
@@ -368,7 +369,6 @@ def hsd_expected_latency(costs, alphas, T):
 def hsd_expected_latency_literal(costs, alphas, T):
     """Expected cost per token of Algorithm 1 as printed (verifiers see everything the level below collected)."""
     lib = library()
-    _declare_engine(lib)
     n = len(costs)
     out = ctypes.c_double()
     _check(lib.hsd_expected_latency_literal((ctypes.c_double * n)(*costs), (ctypes.c_double * max(1, n - 1))(*(alphas or [0])),
@@ -379,7 +379,6 @@ def hsd_expected_latency_literal(costs, alphas, T):
 def hsd_search_T(costs, alphas, T_max=15, monotone=True):
     """argmin over T in [1, T_max]^K of the expected latency -> (T tuple, latency)."""
     lib = library()
-    _declare_engine(lib)
     n = len(costs)
     out_T = (ctypes.c_int32 * max(1, n - 1))()
     out = ctypes.c_double()
@@ -393,7 +392,6 @@ def hsd_pairwise_alpha(logits):
     """logits: CUDA tensor [n_models, n_rows, vocab] (fp32 or bf16) -> float64 CUDA tensor [n_models, n_models] of the
     acceptance rates alpha[i][j] = mean over rows of sum_x min(p_i(x), p_j(x))."""
     lib = library()
-    _declare_engine(lib)
     L, R, V = logits.shape
     logits = logits.contiguous()
     need = lib.hsd_pairwise_alpha_workspace_bytes(L, R, V)
@@ -415,7 +413,6 @@ def hsd_search_hierarchy(costs, alpha, T_max=15):
     costs: c_0..c_K; alpha[i][j]: acceptance rate of drafter i under verifier j (i < j).
     -> (latency, sigma tuple, T tuple)."""
     lib = library()
-    _declare_engine(lib)
     n = len(costs)
     flat = [0.0] * (n * n)
     for i in range(n):
@@ -434,7 +431,6 @@ def hsd_stream_read_gbs(n_bytes=4 << 30, repeats=5):
     """Read-only streaming rate of this GPU's HBM in GB/s (hsd_stream_read over a buffer far larger than L2, best of
     `repeats` after one warm-up, CUDA events on the current stream)."""
     lib = library()
-    _declare_engine(lib)
     buf = torch.empty(n_bytes, dtype=torch.uint8, device="cuda")
     buf.zero_()
     best = 0.0
@@ -452,20 +448,17 @@ def hsd_stream_read_gbs(n_bytes=4 << 30, repeats=5):
 
 def hsd_kernel_launches():
     lib = library()
-    _declare_engine(lib)
     return int(lib.hsd_kernel_launches())
 
 
 def hsd_gemm_workspace_bytes(R, N, K):
     lib = library()
-    _declare_engine(lib)
     return int(lib.hsd_gemm_workspace_bytes(R, N, K))
 
 
 def hsd_gemm_bf16(A, W, out=None, workspace=None, check=True):
     """A bf16 [R, K], W bf16 [N, K] (CUDA) -> fp32 [R, N] = A @ W^T on the tensor cores."""
     lib = library()
-    _declare_engine(lib)
     R, K = A.shape
     N = W.shape[0]
     need = hsd_gemm_workspace_bytes(R, N, K)
