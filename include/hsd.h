@@ -188,7 +188,8 @@ int hsd_set_phase_folding(hsd_ctx *ctx, int fold_qkv, int fold_gate_up, int earl
  * head size 128, an item with 8 or more query vectors whose key range has 2048 keys or more runs on the
  * fifth-generation tensor cores with its scores and outputs in tensor memory; enabled = 0: every item runs on the warp-level path.  Both paths compute the
  * same attention (softmax weights rounded to bf16 before the P V product on the tensor-memory path, to bf16 hi + lo
- * on the other), so results agree to rounding, not bit for bit.  enabled = 2 additionally keeps the key splits of
+ * on the other), so results agree to rounding, not bit for bit.  (Prompt chunks of more than 128 rows
+ * have an attention kernel of their own, which this does not affect.)  enabled = 2 additionally keeps the key splits of
  * long contexts at 2048 keys or more, so that small test models reach that path too.  A test hook and a tuning knob.
  * Errors: INVALID_ARG. */
 int hsd_set_tensor_attention(hsd_ctx *ctx, int enabled);
@@ -301,13 +302,13 @@ int hsd_layer_logits(hsd_ctx *ctx, const int32_t *token_ids, int n_tokens, const
  * From the logits of n_models models (exit layers) at the same n_rows positions, the n_models x n_models
  * matrix of the rates averaged over the positions: alpha[i][j] = mean_r sum_x min(softmax(l_i[r])(x),
  * softmax(l_j[r])(x)); symmetric, diagonal 1.  fp32 softmax (exp by the hardware approximation), sums in
- * fixed order (fp32 per 128 tokens, fp64 across), no atomics: repeatable bit for bit.
+ * fixed order (fp32 within 4096 tokens at most, 128 in a row, fp64 across), no atomics: repeatable bit for bit.
  *   logits device: model m's rows at logits + m * model_stride elements, each [n_rows, vocab] row-major,
  *     dtype HSD_F32 or HSD_BF16; model_stride >= n_rows * vocab;
  *   workspace device, 256-byte aligned, at least hsd_pairwise_alpha_workspace_bytes(...) (0 = bad sizes);
  *   alpha device [n_models * n_models] doubles, row-major, written by the call (asynchronously on stream).
  * The caller owns every buffer.  n_models <= 32.  Errors: INVALID_ARG (null, sizes, alignment, workspace too
- * small), TOO_LARGE (n_models beyond what one block's shared memory holds), CUDA. */
+ * small), CUDA. */
 size_t hsd_pairwise_alpha_workspace_bytes(int n_models, int n_rows, int vocab);
 int hsd_pairwise_alpha(const void *logits, int dtype, int n_models, int n_rows, int vocab, long long model_stride,
                        void *workspace, size_t workspace_bytes, double *alpha, void *stream);
