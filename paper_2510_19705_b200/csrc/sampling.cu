@@ -617,7 +617,6 @@ struct ClusterArgs {
   int32_t *tokens;
   int V, t_max, seg;             // seg: tokens per CTA, a multiple of 64
   int staged;                    // rows kept in shared memory; 0: they do not fit and are read again where they are needed
-  int purpose;                   // PURPOSE_FINAL, or PURPOSE_DRAFT: level-0 draws
   const VerifySeq *desc;         // verification: per sequence, or null (regular)
   const SampleRow *rows;         // draws: per row, or null (regular)
   int regular_t;                 // draws: rows per sequence
@@ -651,8 +650,11 @@ __device__ __forceinline__ u64 warp_sum54(u64 v) {
 }
 
 // Shared memory (dynamic): raw units [rows][NU][threads] | wmax int [rows][warps] | wsum u64 [rows + 1][warps]
-template <typename T, int PER, int NT>
-__global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __grid_constant__ ClusterArgs a) {
+// DRAW: one row, 32-bit weights, two CTAs per SM.
+template <bool DRAW> struct ClWeight { typedef u64 type; };
+template <> struct ClWeight<true> { typedef u32 type; };
+template <typename T, int PER, int NT, bool DRAW>
+__global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kernel(const __grid_constant__ ClusterArgs a) {
   typedef typename ClUnit<T, PER>::raw raw_t;
   constexpr int NU = NT / PER;                                     // units per thread and row
   extern __shared__ __align__(16) unsigned char cl_smem[];
@@ -667,7 +669,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __g
   VerifySeq d;
   long long out_index = 0;
   u32 uj = 0;
-  if (a.purpose == PURPOSE_DRAFT) {
+  if (DRAW) {
     SampleRow s;
     if (a.rows) s = a.rows[b];
     else { s.logit_row = b; s.out_index = b; s.j = b % a.regular_t; s.seq = b / a.regular_t; s.serial = a.regular_serial; s.level = 0; }
@@ -678,7 +680,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __g
     d.t = a.regular_t; d.p_row0 = (long long)b * (a.regular_t + 1); d.q_row0 = (long long)b * a.regular_t;
     d.tok_off = (long long)b * a.regular_t; d.serial = a.regular_serial; d.seq = b; d.level = a.regular_level;
   }
-  const int t = d.t, n_rows = 2 * t + 1;                           // rows 0..t: p; t + 1 + j: q_j
+  const int t = DRAW ? 0 : d.t, n_rows = 2 * t + 1;                           // rows 0..t: p; t + 1 + j: q_j
   raw_t *stage = reinterpret_cast<raw_t *>(cl_smem);
   const size_t max_rows = 2 * (size_t)a.t_max + 1;
   u64 *wsum = reinterpret_cast<u64 *>(cl_smem + (a.staged ? max_rows * NU * kClThreads * sizeof(raw_t) : 0));   // [rows + 1][warps]
@@ -789,7 +791,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __g
   }
   __syncthreads();
   // ---- accept tests (t <= 31: one warp), n = first rejection
-  if (warp == 0) {
+  if (!DRAW && warp == 0) {
     bool ok = true;
     if (lane < t) {
       const u32 ep = (tok >= 0 && tok < a.V) ? exp_weight(lp, row_m[lane]) : 0u, eq = (tok >= 0 && tok < a.V) ? exp_weight(lq, row_m[t + 1 + lane]) : 0u;
@@ -801,10 +803,10 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __g
     const unsigned rejected = __ballot_sync(0xFFFFFFFFu, !ok);
     if (lane == 0) sh_n = rejected ? __ffs(rejected) - 1 : t;
   }
-  __syncthreads();
-  const int n = sh_n;
+  if (!DRAW) __syncthreads();
+  const int n = DRAW ? 0 : sh_n;
   // ---- the final draw's weights: the residual of row n, or row t itself
-  u64 w[NT];
+  typename ClWeight<DRAW>::type w[NT];
   int src = n;                                                     // row of wsum / csum that holds the totals of w
   u64 total = row_S[n];
   const float mp = row_m[n];
@@ -814,7 +816,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __g
     for (int i = 0; i < NU; ++i) v[i] = unit_of(n, i);
     weights_of(v, mp, [&](int j, u32 e0, u32 e1) { w[j] = e0; w[j + 1] = e1; });
   };
-  if (n < t) {
+  if (!DRAW && n < t) {
     const float mq = row_m[t + 1 + n];
     const ProbScale psp = prob_scale(row_S[n]), psq = prob_scale(row_S[t + 1 + n]);
     u64 local = 0;
@@ -843,15 +845,15 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __g
     if (total != 0) src = n_rows;
     else total = row_S[n];                                         // an all-zero residual: draw from the verifier's own row
   }
-  if (src == n) row_weights();
+  if (DRAW || src == n) row_weights();
   // ---- inverse CDF: the CTA, then the warp, then the unit, then the token whose inclusive sum passes the threshold
-  const u32 U = uniform24(a.seed, uj, d.serial, d.level, a.purpose, d.seq);
+  const u32 U = uniform24(a.seed, uj, d.serial, d.level, DRAW ? PURPOSE_DRAFT : PURPOSE_FINAL, d.seq);
   const u64 tau = cdf_threshold(U, total);
   u64 before = 0;
   for (u32 c = 0; c < rank; ++c) before += csum[src][c];
   if (total == 0) {                                                // non-finite logits: no token
     if (rank == 0 && tid == 0) {
-      if (a.purpose == PURPOSE_DRAFT) a.out_tokens[out_index] = -1;
+      if (DRAW) a.out_tokens[out_index] = -1;
       else {
         if (a.write_in_place) a.tokens[d.tok_off + n] = -1;
         if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = -1;
@@ -898,7 +900,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __g
               if (run > tau) break;
               ++k;
             }
-            if (a.purpose == PURPOSE_DRAFT) a.out_tokens[out_index] = k;
+            if (DRAW) a.out_tokens[out_index] = k;
             else {
               if (a.write_in_place) a.tokens[d.tok_off + n] = k;
               if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = k;
@@ -908,7 +910,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __g
       }
     }
   }
-  if (a.purpose != PURPOSE_DRAFT && rank == 0) {
+  if (!DRAW && rank == 0) {
     if (tid == 0) a.out_n[b] = n;
     if (a.out_tokens && tid <= a.t_max && tid != n) a.out_tokens[(size_t)b * (a.t_max + 1) + tid] = tid < n ? tok : -1;
   }
@@ -918,16 +920,17 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_sample_kernel(const __g
 // are too long or too many for this path.
 struct ClusterPlan { int C, NT, per, staged, seg; size_t smem; };
 constexpr size_t kClMaxSmem = 216 * 1024;
-static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, int rows, ClusterPlan *pl) {
+static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, int rows, bool draw, ClusterPlan *pl) {
   if (rows > kClMaxRows) return false;
   pl->per = (dtype == HSD_BF16 && V % 2 == 0 && ((uintptr_t)p & 3) == 0 && ((uintptr_t)q & 3) == 0) ? 2 : 1;
-  // as many CTAs as run at once, of at least 4096 tokens (eight a thread) each: clusters of eight do not fit all 148 SMs
+  // as many CTAs as run at once (draws: two per SM), of at least 4096 tokens (eight a thread) each: clusters of eight do not fit all 148 SMs
   // (16 of them took two rounds), clusters of four and two do
   int C = 1;
-  while (C < kClMaxC && V > C * 4096 && 2 * C * n <= (C == 4 ? 112 : 148)) C *= 2;
-  while (C < kClMaxC && ceil_div(V, C) > 32 * kClThreads - 64) C *= 2;
+  while (C < kClMaxC && V > C * 4096 && 2 * C * n <= (C == 4 ? 112 : draw ? 296 : 148)) C *= 2;
+  const int most = (draw ? 16 : 32) * kClThreads;
+  while (C < kClMaxC && ceil_div(V, C) > most - 64) C *= 2;
   const int seg = ceil_div(ceil_div(V, C), 64) * 64;
-  if (seg > 32 * kClThreads) return false;
+  if (seg > most) return false;
   pl->C = C;
   pl->seg = seg;
   pl->NT = seg <= 8 * kClThreads ? 8 : seg <= 16 * kClThreads ? 16 : 32;
@@ -943,8 +946,9 @@ static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, 
 //     tokens a CTA): 38 / 35; t = 8: 8 sequences (68k) 19 / 26, 16 (136k): 36 / 30.
 //   other rows: statistics and decision kernels, each row read twice by one CTA.  fp32, V = 32001: t = 3 14 / 58, t = 8
 //     30 / 58; V = 9001: t = 3 14 / 15, t = 8 29 / 15; V = 2048: t = 3 11 / 7.  bf16 of odd length, 49999: t = 3 21 / 50, t = 8 55 / 50.
-//   draws: bf16 32000: 1 row 6.8 / 12.5, 64 rows 11.2 / 12.5; 16000: 100 rows (no split) 10.8 / 10.1; fp32 9001: 7.1 / 6.0,
-//     16001: 7.2 / 11.7, 50000: 64 rows 27 / 24.
+//   draws (two CTAs per SM, 16 tokens a thread at most): bf16 32000: 1 row 4.4 / 10.6, 64 rows 6.7 / 11.3 (one CTA per
+//     SM, 32 tokens a thread: 11.2), 100 rows would take a second round; fp32 32000: 1 row 5.7 / 28, 64 rows 8.6 / 28; 16001:
+//     5.2 / 10.8; 9001 (two CTAs a row): 6.9 / 6.2, 2048: 6.8 / 3.9; bf16 2048 (one CTA): 6.7 / 9.8.
 static bool cluster_pays_verify(const ClusterPlan &pl, int dtype, int V, int rows, bool fused) {
   const long long work = (long long)pl.seg * rows;
   if (fused) return work <= 100000;
@@ -952,16 +956,16 @@ static bool cluster_pays_verify(const ClusterPlan &pl, int dtype, int V, int row
   return V > 20000 ? work <= 4ll * V : work * 5 <= 11ll * V;
 }
 static bool cluster_pays_draw(const ClusterPlan &pl, int dtype, int V, int n, bool chunked) {
-  if (pl.seg > 4096 && (pl.seg > 16384 || pl.C * n > 148)) return false;     // (256 rows of 32000: 39 / 25)
+  if (pl.seg > 4096 && pl.C * n > 296) return false;
   if (dtype == HSD_BF16 && chunked) return pl.seg <= 4096 || pl.C > 1;
   return V > 12000 && pl.C > 1;
 }
 
-template <typename T, int PER, int NT>
+template <typename T, int PER, int NT, bool DRAW>
 static int launch_cluster_t(const ClusterArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
   static bool attr_set = false;
   if (!attr_set) {
-    HSD_CUDA_OK(cudaFuncSetAttribute(cluster_sample_kernel<T, PER, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClMaxSmem));
+    HSD_CUDA_OK(cudaFuncSetAttribute(cluster_sample_kernel<T, PER, NT, DRAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(DRAW ? kClMaxSmem / 2 : kClMaxSmem)));
     attr_set = true;
   }
   cudaLaunchConfig_t cfg = {};
@@ -970,21 +974,23 @@ static int launch_cluster_t(const ClusterArgs &a, const ClusterPlan &pl, int n, 
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = pl.C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = 1;
-  HSD_CUDA_OK(cudaLaunchKernelEx(&cfg, cluster_sample_kernel<T, PER, NT>, a));
+  HSD_CUDA_OK(cudaLaunchKernelEx(&cfg, cluster_sample_kernel<T, PER, NT, DRAW>, a));
   hsd_count_launches(1);
   return hsd_launch_status();
 }
-template <typename T, int PER>
+template <typename T, int PER, bool DRAW>
 static int launch_cluster_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
-  if (pl.NT == 8) return launch_cluster_t<T, PER, 8>(a, pl, n, s);
-  if (pl.NT == 16) return launch_cluster_t<T, PER, 16>(a, pl, n, s);
-  return launch_cluster_t<T, PER, 32>(a, pl, n, s);
+  if (pl.NT == 8) return launch_cluster_t<T, PER, 8, DRAW>(a, pl, n, s);
+  if (pl.NT == 16) return launch_cluster_t<T, PER, 16, DRAW>(a, pl, n, s);
+  if constexpr (!DRAW) return launch_cluster_t<T, PER, 32, DRAW>(a, pl, n, s);
+  return HSD_E_UNSUPPORTED;
 }
+template <bool DRAW>
 static int launch_cluster(ClusterArgs a, const ClusterPlan &pl, int dtype, int n, cudaStream_t s) {
   a.seg = pl.seg;
   a.staged = pl.staged;
-  if (dtype == HSD_F32) return launch_cluster_nt<float, 1>(a, pl, n, s);
-  return pl.per == 2 ? launch_cluster_nt<__nv_bfloat16, 2>(a, pl, n, s) : launch_cluster_nt<__nv_bfloat16, 1>(a, pl, n, s);
+  if (dtype == HSD_F32) return launch_cluster_nt<float, 1, DRAW>(a, pl, n, s);
+  return pl.per == 2 ? launch_cluster_nt<__nv_bfloat16, 2, DRAW>(a, pl, n, s) : launch_cluster_nt<__nv_bfloat16, 1, DRAW>(a, pl, n, s);
 }
 
 // ------------------------------------------------------------------------------ host launchers
@@ -1006,12 +1012,12 @@ int launch_draft_sample(const void *logits, int dtype, int V, const SampleRow *d
                         u32 regular_serial, u64 seed, int32_t *out, cudaStream_t s) {
   if (n_rows == 0) return HSD_OK;
   ClusterPlan pl;
-  if (cluster_plan(logits, nullptr, dtype, V, n_rows, 1, &pl) &&
+  if (cluster_plan(logits, nullptr, dtype, V, n_rows, 1, true, &pl) &&
       cluster_pays_draw(pl, dtype, V, n_rows, V % 8 == 0 && V <= kSampleThreads * kChunkTokens && ((uintptr_t)logits & 15) == 0)) {
     ClusterArgs a = {};
-    a.p = logits; a.V = V; a.t_max = 0; a.purpose = PURPOSE_DRAFT; a.rows = desc; a.regular_t = regular_rows;
+    a.p = logits; a.V = V; a.t_max = 0; a.rows = desc; a.regular_t = regular_rows;
     a.regular_serial = regular_serial; a.seed = seed; a.out_tokens = out; a.coin24 = kNoCoin;
-    return launch_cluster(a, pl, dtype, n_rows, s);
+    return launch_cluster<true>(a, pl, dtype, n_rows, s);
   }
   return dtype == HSD_BF16
              ? launch_draft_sample_t<__nv_bfloat16>(logits, V, desc, n_rows, regular_rows, regular_serial, seed, out, s)
@@ -1060,12 +1066,12 @@ int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int 
   const bool fused = dtype == HSD_BF16 && V % 8 == 0 && V <= kFusedMaxV && smem <= 220 * 1024 && ((uintptr_t)p & 15) == 0 &&
                      (q == nullptr || ((uintptr_t)q & 15) == 0) && t_max < kFusedConsumers;
   ClusterPlan pl;
-  if (cluster_plan(p, q, dtype, V, batch, 2 * t_max + 1, &pl) && cluster_pays_verify(pl, dtype, V, 2 * t_max + 1, fused)) {
+  if (cluster_plan(p, q, dtype, V, batch, 2 * t_max + 1, false, &pl) && cluster_pays_verify(pl, dtype, V, 2 * t_max + 1, fused)) {
     ClusterArgs a = {};
-    a.p = p; a.q = q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.purpose = PURPOSE_FINAL; a.desc = desc; a.regular_t = regular_t;
+    a.p = p; a.q = q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.desc = desc; a.regular_t = regular_t;
     a.regular_serial = regular_serial; a.regular_level = regular_level; a.seed = seed; a.out_tokens = out_tokens; a.out_n = out_n;
     a.write_in_place = write_in_place; a.coin24 = coin24;
-    return launch_cluster(a, pl, dtype, batch, s);
+    return launch_cluster<false>(a, pl, dtype, batch, s);
   }
   if (fused) {
     static bool attr_set = false;
