@@ -11,6 +11,7 @@
 #include "attn_prompt.cuh"
 #include "forward.cuh"
 #include "fwd_persist.cuh"
+#include "fwd_small.cuh"
 #include "gemm_big.cuh"
 #include "gemm_tc.cuh"
 #include "sampling_api.cuh"
@@ -50,7 +51,7 @@ size_t elem_size(int dtype) { return dtype == HSD_BF16 ? 2 : 4; }
 // page table, per-level logits rows, decision scratch, descriptor ring).
 struct ModelLayout {
   size_t cos_tab, sin_tab, k_pool, v_pool, pool_layer_stride, x, h, qkv, q, att, act, partials, hf, tc_scratch,
-      tc_pieces_bytes, tc_pieces2, wmaps_dev, layers_dev, attn_counters, prof;
+      tc_pieces_bytes, tc_pieces2, wmaps_dev, layers_dev, small_layers, attn_counters, prof;
   int partial_rows;
 };
 struct Layout {
@@ -186,6 +187,7 @@ Layout make_layout(const hsd_model_desc *models, int n_models, int n_levels, con
     M.tc_pieces2 = take(M.tc_pieces_bytes);       // second piece buffer (down projection of passes with few rows)
     M.wmaps_dev = take(((size_t)m->n_layers * 7 + kHeadMaps) * sizeof(CUtensorMap));
     M.layers_dev = take((size_t)m->n_layers * sizeof(FwdLayerDev));
+    M.small_layers = take(m->dtype == HSD_F32 ? (size_t)m->n_layers * sizeof(SmallLayerDev) : 0);
     M.attn_counters = take(16384);
     M.prof = take((size_t)device_sm_count() * kFwdProfEvents * 8);
   }
@@ -213,6 +215,8 @@ struct Model {
   bool use_tc = false, use_persist = false;   // tensor-core GEMMs / the one-launch persistent forward (bf16 models)
   std::vector<CUtensorMap> wmaps;             // [n_layers * 7 + kHeadMaps]: wq wk wv wo wg wu wd per layer, then the levels' heads, the shared head
   CUtensorMap amaps[4][5];                    // activation buffers {h, att, act, hf} x row padding {16, 32, 64, 128, 256}
+  bool use_small = false;                     // passes of few rows of a small fp32 model: one launch (fwd_small)
+  int small_grid = 1;
   bool use_prompt = false;                    // long prompts run forward_prompt
   std::vector<CUtensorMap> kvmaps;            // [n_layers][4]: K and V pools of each layer, two box heights each, for the prompt attention
   CUtensorMap amaps_rows[4][16];              // the same buffers with a box of exactly 1..16 rows (persistent forward, few rows)
@@ -249,7 +253,8 @@ struct hsd_ctx {
   int trace_logit_calls, trace_records;
   cudaStream_t stream;
   uint64_t seed;
-  bool any_tc = false;                        // some model runs the tensor-core kernels (their status word is polled)
+  unsigned small_base = 0;                    // barrier arrivals of all one-launch fp32 passes so far
+  bool any_tc = false;                        // some model runs kernels with bounded waits (their status word is polled)
   bool no_fuse_qkv = false;                   // keep the QKV finish phase in every pass (hsd_set_phase_folding)
   bool no_fuse_gu = false;                    // keep the gate / up finish phase in every pass
   bool no_early_norm = false;                 // keep the grid barrier between a residual projection and its norm
@@ -605,6 +610,31 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     mark_valid();
     return HSD_OK;
   }
+  // (a level's own head or norm gain may lie on any 4-byte boundary: such a level keeps the launches per operation)
+  const bool heads_aligned = (((uintptr_t)c->level_head[level] | (uintptr_t)c->level_norm[level]) & 15) == 0;
+  if (M.use_small && R <= kSmallRows && n_logit <= kSmallRows && heads_aligned) {
+    SmallFwdArgs a;
+    a.d = md.d; a.nq = md.nq; a.nkv = md.nkv; a.hd = md.hd; a.ff = md.ff; a.V = md.V; a.n_run = c->exits[level]; a.max_seq = md.max_seq;
+    a.page = md.page; a.pages_per_seq = md.pages_per_seq; a.n_pages = md.n_pages; a.eps = md.eps;
+    a.layers = c->dev<SmallLayerDev>(ML.small_layers);
+    a.embed = (const float *)M.embed; a.final_norm = (const float *)c->level_norm[level]; a.lm_head = (const float *)c->level_head[level];
+    a.cos_tab = c->dev<float>(ML.cos_tab); a.sin_tab = c->dev<float>(ML.sin_tab);
+    a.R = R; a.L = n_logit;
+    a.tokens = c->dev<int>(L.tokens); a.page_table = c->dev<int>(L.page_table);
+    a.row_seq = rb.row_seq; a.row_pos = rb.row_pos; a.lrow_src = rb.lrow_src; a.lrow_dst = rb.lrow_dst;
+    a.x = c->dev<float>(ML.x); a.q = c->dev<float>(ML.q); a.att = c->dev<float>(ML.att); a.act = c->dev<float>(ML.act);
+    a.logits = (float *)(c->ws + L.logits[level]);
+    a.counter = c->dev<unsigned>(L.grid_counter) + 48;        // behind the words the bf16 forward clears
+    a.base = c->small_base;
+    a.status = (int *)(c->ws + c->status_off);
+    HSD_TRY(launch_forward_small(a, M.small_grid, s));
+    c->small_base += fwd_small_arrivals(a.n_run, a.L, M.small_grid);
+    if (tp) cudaEventRecord(tp->b, s);
+    c->stats[level].forwards++;
+    c->stats[level].rows += R;
+    mark_valid();
+    return HSD_OK;
+  }
   float *x = c->dev<float>(ML.x);
   void *h = c->dev<void>(ML.h), *q = c->dev<void>(ML.q), *att = c->dev<void>(ML.att), *act = c->dev<void>(ML.act);
   float *qkv = c->dev<float>(ML.qkv);
@@ -919,6 +949,13 @@ int prefill(hsd_ctx *c, int batch, int prompt_len) {
   return HSD_OK;
 }
 
+bool coop_launch_supported() {
+  int coop = 0, dev = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  return coop != 0;
+}
+
 // Sets up one model of a context: rotary tables, tensor maps, device-side tables.  `head_levels`: the levels whose
 // output-head tensor map slots are (re)built for this model.
 int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLayout &ml) {
@@ -942,6 +979,21 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
     if (cudaMemcpy(c->ws + ml.cos_tab, cs.data(), cs.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->ws + ml.sin_tab, sn.data(), sn.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess)
       return HSD_E_CUDA;
+  }
+  M.use_small = fwd_small_supported(md) && coop_launch_supported();
+  if (M.use_small) {
+    M.small_grid = fwd_small_grid(md, c->sm_count);
+    std::vector<SmallLayerDev> sl(md.n_layers);
+    for (int l = 0; l < md.n_layers; ++l) {
+      for (int k = 0; k < 9; ++k) {
+        sl[l].w[k] = (const float *)M.lw[(size_t)l * 9 + k];
+        M.use_small = M.use_small && ((uintptr_t)sl[l].w[k] & 15) == 0;      // 16-byte loads
+      }
+      sl[l].k_pool = (float *)(c->ws + ml.k_pool + ml.pool_layer_stride * l);
+      sl[l].v_pool = (float *)(c->ws + ml.v_pool + ml.pool_layer_stride * l);
+    }
+    M.use_small = M.use_small && ((uintptr_t)M.embed & 15) == 0;
+    if (cudaMemcpy(c->ws + ml.small_layers, sl.data(), sl.size() * sizeof(SmallLayerDev), cudaMemcpyHostToDevice) != cudaSuccess) return HSD_E_CUDA;
   }
   // tensor-core path: bf16 model whose contraction sizes are multiples of the 64-element k-block
   M.use_tc = model->dtype == HSD_BF16 && model->d_model % kTcBlockK == 0 && model->d_ff % kTcBlockK == 0 &&
@@ -978,10 +1030,7 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
       cudaMemcpy(c->ws + ml.layers_dev, ld.data(), ld.size() * sizeof(FwdLayerDev), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(c->ws + ml.attn_counters, 0, 16384) != cudaSuccess)
     return HSD_E_CUDA;
-  int coop = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-  M.use_persist = coop != 0 && fwd_persist_supported(md.hd, md.nq / md.nkv) && md.d % 256 == 0 && md.d <= 4096 &&
+  M.use_persist = coop_launch_supported() && fwd_persist_supported(md.hd, md.nq / md.nkv) && md.d % 256 == 0 && md.d <= 4096 &&
                   (md.d / kTcBlockM) * 2 <= c->sm_count && md.n_layers <= 64 && (md.page & (md.page - 1)) == 0 && md.page >= 16;
   M.use_prompt = M.use_persist && prompt_path_dims(model);
   if (M.use_prompt) {
@@ -1048,7 +1097,7 @@ int create_ctx(const hsd_model_desc *models, int n_models, const int32_t *exit_l
   c->models.resize(n_models);
   for (int mi = 0; mi < n_models && !st; ++mi) {
     st = init_model(c, c->models[mi], &models[mi], lay.model[mi]);
-    c->any_tc = c->any_tc || c->models[mi].use_tc;
+    c->any_tc = c->any_tc || c->models[mi].use_tc || c->models[mi].use_small;
   }
   if (st) {
     hsd_destroy(c);
