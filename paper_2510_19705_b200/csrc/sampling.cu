@@ -633,6 +633,9 @@ __device__ __forceinline__ u32 cl_id() { u32 r; asm volatile("mov.u32 %0, %%clus
 __device__ __forceinline__ void cl_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// "This CTA runs": a CTA may touch another's shared memory once every CTA of the cluster has arrived here.
+__device__ __forceinline__ void cl_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ u32 cl_map(const void *p, u32 rank) {
   u32 r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((u32)__cvta_generic_to_shared(p)), "r"(rank));
@@ -666,6 +669,7 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const u32 rank = cl_rank(), C = cl_size();
   const int b = (int)cl_id();
+  cl_arrive();                                                     // (the wait is in front of the first store to a peer)
   VerifySeq d;
   long long out_index = 0;
   u32 uj = 0;
@@ -748,6 +752,7 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
     }
   }
   __syncthreads();
+  cl_wait();                                                       // every CTA of the cluster has started
   for (int r = warp; r < n_rows; r += kClWarps) {
     const int key = __reduce_max_sync(0xFFFFFFFFu, wmax[r * kClWarps + (lane & (kClWarps - 1))]);
     if (lane < (int)C) cl_store(cl_map(&cmax[r][rank], (u32)lane), (u32)key);

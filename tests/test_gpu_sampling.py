@@ -134,3 +134,22 @@ def test_cluster_decisions_match_oracle(lib, dtype, V, B, t):
         out, n = lib.hsd_verify_level(1, p, q, x, 17, serial)
         want_out, want_n = _oracle_verify(1, p_np, q_np, x_np, 17, serial)
         assert np.array_equal(n.cpu().numpy(), want_n) and np.array_equal(out.cpu().numpy(), want_out)
+
+
+@pytest.mark.parametrize("dtype,V,B", [("bf16", 32000, 2), ("bf16", 32000, 37), ("fp32", 32001, 18), ("bf16", 9000, 70)])
+def test_cluster_draws_on_a_busy_gpu(lib, dtype, V, B):
+    # clusters of eight, four and two whose CTAs start while another stream's kernels occupy SMs and shared memory: the
+    # first exchange of a draw needs every CTA of its cluster on the GPU
+    _, q = inputs.make_accept_logits(B, 1, V, seed=V + B, device="cuda", dtype=dtype)
+    _, other = inputs.make_accept_logits(64, 4, 32000, seed=1, device="cuda", dtype="bf16")
+    want = [_oracle_draft(inputs.logits_to_numpy(q), 31, s) for s in range(4)]
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    got = []
+    for i in range(64):
+        with torch.cuda.stream(side):
+            lib.hsd_draft_sample(other, 8, i)
+        got.append(lib.hsd_draft_sample(q, 31, i % 4))
+    torch.cuda.synchronize()
+    for i, x in enumerate(got):
+        assert np.array_equal(x.cpu().numpy(), want[i % 4]), i
