@@ -290,7 +290,8 @@ int hsd_search_hierarchy(const double *costs, const double *alpha, int n_models,
  *     resets its sequences and KV cache as a generation does, so it must not overlap one;
  *   token_ids device [n_tokens], 1 <= n_tokens <= 128 (and <= max_seq);
  *   layers host [n_sel]: exit layers, strictly ascending, each in 1 .. n_layers (n_layers = the full model);
- *   out_logits device [n_sel, n_tokens, vocab] in the model's storage dtype, written by the call;
+ *   out_logits device [n_sel, n_tokens, vocab] in the model's storage dtype, at any address that dtype allows (bf16 at
+ *     16-byte boundaries is the faster one), written by the call;
  *   stream: the call returns after its work on the stream has completed.
  * Errors: INVALID_ARG, OUT_OF_PAGES, CUDA, DEVICE_TIMEOUT. */
 int hsd_layer_logits(hsd_ctx *ctx, const int32_t *token_ids, int n_tokens, const int32_t *layers, int n_sel,

@@ -221,7 +221,7 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
         const long long dr = on ? (args.dst ? args.dst[r] : (long long)r) : 0;
         __nv_bfloat16 *row = args.out_bf16 + (size_t)dr * args.ldo + nt * kBN;
         const int left = args.seg_n[0] - nt * kBN;
-        const bool vec = (args.ldo & 7) == 0;
+        const bool vec = (args.ldo & 7) == 0 && ((uintptr_t)args.out_bf16 & 15) == 0;     // (the caller's buffer: any element's address)
 #pragma unroll 1
         for (int c = 0; c < kBN; c += 16) {
           float v[16];

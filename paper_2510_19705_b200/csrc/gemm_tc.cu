@@ -102,7 +102,7 @@ __device__ __forceinline__ void finish4(const TcGemmArgs &a, const TileInfo &ti,
     *reinterpret_cast<uint2 *>(dst + half) = pack_bf16x4(hi);
   } else if (MODE == GEMM_STORE_T_SCATTER) {
     __nv_bfloat16 *dst = a.out_bf16 + (size_t)a.dst[row] * a.ldo + ti.col0 + n;
-    if (left >= 4 && (a.ldo & 3) == 0) *reinterpret_cast<uint2 *>(dst) = pack_bf16x4(v);
+    if (left >= 4 && (a.ldo & 3) == 0 && ((uintptr_t)a.out_bf16 & 7) == 0) *reinterpret_cast<uint2 *>(dst) = pack_bf16x4(v);
     else {
       const float e[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll

@@ -111,3 +111,24 @@ def test_pairwise_alpha_block_edges(lib, L, R, V, dtype):
     want = torch.stack([torch.minimum(p[i:i + 1], p).sum(-1).mean(-1) for i in range(L)]).numpy()
     # fp32 sums of at most 128 terms per lane and 8 per warp and slice: about 2^-24 x 136 of a rate, 1e-5 at most
     assert np.array_equal(got, got.T) and np.abs(got - want).max() < 1e-5, np.abs(got - want).max()
+
+
+@pytest.mark.parametrize("d,nq,nkv,V", [(256, 4, 2, 1000), (256, 4, 2, 1004), (192, 3, 1, 1000)])     # head in one product over all layers / a product per layer
+def test_layer_logits_into_any_element_address(lib, d, nq, nkv, V):
+    """The output needs the alignment of its elements only, whatever the vocabulary's divisors."""
+    import ctypes
+    from paper_2510_19705_b200 import inputs
+    cfg = inputs.model_cfg(2, d, nq, nkv, 256, V, "bf16", head_dim=64)
+    w = inputs.make_weights(cfg, 5)
+    w = {k: (v.cuda() if k != "layers" else [{n: t.cuda() for n, t in l.items()} for l in v]) for k, v in w.items()}
+    eng = lib.Hsd(cfg, w, (1, 2), (1,), max_batch=1, max_seq=64, page_size=16)
+    toks = inputs.make_prompts(V, 1, 21, 3)[0].cuda()
+    want = eng.layer_logits(toks, [1, 2])
+    for off in (1, 2, 3, 4):
+        buf = torch.full((want.numel() + 8,), 7.0, dtype=torch.bfloat16, device="cuda")
+        st = lib.library().hsd_layer_logits(eng._ctx, toks.data_ptr(), 21, (ctypes.c_int32 * 2)(1, 2), 2, buf.data_ptr() + 2 * off,
+                                            torch.cuda.current_stream().cuda_stream)
+        assert st == 0
+        assert torch.equal(buf[off:off + want.numel()].view(want.shape), want)
+        assert (buf[:off] == 7.0).all() and (buf[off + want.numel():] == 7.0).all()
+    eng.close()
