@@ -155,7 +155,7 @@ __device__ __forceinline__ void alpha_block(const float *pi, const float *pj, in
   }
 }
 
-// grid (units, R).  The unit's tokens go through shared memory 256 at a time as probabilities [model][token]
+// Block r x units + u = unit u of position r (one dimension: any number of positions).  The unit's tokens go through shared memory 256 at a time as probabilities [model][token]
 // (double-buffered: the next tile's logits are fetched under this tile's minima).  A warp owns one pair of 8-model
 // blocks, or two diagonal blocks (about as much work), and the tokens lane + 32 slice, ...; with fewer blocks than
 // warps the warps share a pair and split the tokens.
@@ -163,11 +163,11 @@ __device__ __forceinline__ void alpha_block(const float *pi, const float *pj, in
 // per pair and token, took 5021 + 176 us.
 template <typename T, bool VEC>
 __global__ void __launch_bounds__(kAlphaThreads, 2)
-alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, int R, int V, int unit,
+alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, int R, int V, int unit, int n_units,
                    const float2 *__restrict__ stats, float *__restrict__ partials) {
   extern __shared__ float sm[];
   __shared__ float2 st[kAlphaMaxModels];
-  const int r = blockIdx.y, u0 = blockIdx.x * unit, nt = min(unit, V - u0);
+  const int r = blockIdx.x / n_units, u0 = (blockIdx.x - r * n_units) * unit, nt = min(unit, V - u0);
   const int nb = (L + 7) >> 3, lpad = nb * 8, n_off = nb * (nb - 1) / 2, n_task = n_off + (nb + 1) / 2;
   const int slices = max(1, 8 / n_task);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -249,7 +249,7 @@ alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, 
     __syncthreads();
   }
   // lane sums; the slices of a task are added in slice order
-  float *out = partials + ((size_t)r * gridDim.x + blockIdx.x) * n_pairs;
+  float *out = partials + (size_t)blockIdx.x * n_pairs;
   float v[64];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
@@ -330,7 +330,7 @@ int launch_alpha_t(const void *logits, long long model_stride, int L, int R, int
       if (cudaFuncSetAttribute(alpha_pairs_kernel<T, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) != cudaSuccess) return HSD_E_CUDA;
       attr_set = true;
     }
-    alpha_pairs_kernel<T, VEC><<<dim3(p.n_units, R), kAlphaThreads, smem, s>>>((const T *)logits, model_stride, L, R, V, p.unit, stats, partials);
+    alpha_pairs_kernel<T, VEC><<<p.n_units * R, kAlphaThreads, smem, s>>>((const T *)logits, model_stride, L, R, V, p.unit, p.n_units, stats, partials);
   }
   alpha_reduce_kernel<<<p.n_pairs > 0 ? min(p.n_pairs, 592) : 1, kAlphaThreads, 0, s>>>(partials, L, R * p.n_units, R, alpha);
   hsd_count_launches(p.n_pairs > 0 ? 3 : 2);

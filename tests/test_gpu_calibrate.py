@@ -132,3 +132,14 @@ def test_layer_logits_into_any_element_address(lib, d, nq, nkv, V):
         assert torch.equal(buf[off:off + want.numel()].view(want.shape), want)
         assert (buf[:off] == 7.0).all() and (buf[off + want.numel():] == 7.0).all()
     eng.close()
+
+
+@pytest.mark.parametrize("R", [65535, 65536, 65600])
+def test_pairwise_alpha_of_many_positions(lib, R):
+    """More positions than a grid's second and third dimensions hold."""
+    g = torch.Generator().manual_seed(R)
+    logits = torch.randn(3, R, 8, generator=g) * 2.0
+    got = lib.hsd_pairwise_alpha(logits.cuda()).cpu()
+    p = torch.softmax(logits.double(), -1)
+    want = torch.stack([torch.minimum(p[i:i + 1], p).sum(-1).mean(-1) for i in range(3)])
+    assert torch.equal(got, got.T) and (got - want).abs().max() < 1e-5
