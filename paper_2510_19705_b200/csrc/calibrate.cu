@@ -47,7 +47,11 @@ __device__ __forceinline__ float alpha_ex2(float x) {
 }
 // Weight of a logit relative to 2^n, n a whole number: exp(x) 2^-n.  Numerators and sums use the same expression, so
 // the approximation's own bias cancels in their quotient.
-__device__ __forceinline__ float alpha_weight(float x, float n) { return alpha_ex2(fmaf(x, kLog2e, -n)); }
+__device__ __forceinline__ float alpha_weight(float x, float n, float scale = kLog2e) { return alpha_ex2(fmaf(x, scale, -n)); }
+// The reference n is off by half its last bit, 2^32 in the weights at |n| = 2^30, which fp32 holds.  Past that (and in a row
+// of nothing but its type's lowest value, n = -inf) a logit below the maximum is below it by 32 or more: those rows take
+// scale 1 and the maximum itself as n, exactly 1 at the maximum and 2^-32 at most elsewhere.  Their sums carry the sign bit.
+constexpr float kAlphaFar = 1073741824.f;
 
 // Online sum of exp of a thread, relative to 2^n with 2^n at or above the largest exp so far: a larger n rescales the
 // sum by a power of two, exactly.
@@ -108,10 +112,27 @@ alpha_stats_kernel(const T *__restrict__ logits, long long model_stride, int R, 
   for (int o = 16; o > 0; o >>= 1) ms.merge(__shfl_xor_sync(0xFFFFFFFFu, ms.n, o), __shfl_xor_sync(0xFFFFFFFFu, ms.s, o));
   if (lane == 0) { shm[warp] = ms.n; shs[warp] = ms.s; }
   __syncthreads();
+  RefSum t;
+  for (int w = 0; w < kAlphaThreads / 32; ++w) t.merge(shm[w], shs[w]);     // the same in every thread
+  if (fabsf(t.n) <= kAlphaFar) {
+    if (threadIdx.x == 0) stats[(size_t)l * R + r] = make_float2(t.n, t.s);
+    return;
+  }
+  __syncthreads();
+  float m = -INFINITY, s = 0.f;
+  for (int k = threadIdx.x; k < V; k += kAlphaThreads) m = fmaxf(m, to_f32(row[k]));
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+  if (lane == 0) shm[warp] = m;
+  __syncthreads();
+  for (int w = 0; w < kAlphaThreads / 32; ++w) m = fmaxf(m, shm[w]);
+  for (int k = threadIdx.x; k < V; k += kAlphaThreads) s += alpha_weight(to_f32(row[k]), m, 1.f);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  if (lane == 0) shs[warp] = s;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    RefSum t;
-    for (int w = 0; w < kAlphaThreads / 32; ++w) t.merge(shm[w], shs[w]);
-    stats[(size_t)l * R + r] = make_float2(t.n, t.s);
+    float tot = 0.f;
+    for (int w = 0; w < kAlphaThreads / 32; ++w) tot += shs[w];
+    stats[(size_t)l * R + r] = make_float2(m, __int_as_float(__float_as_int(tot) | (int)0x80000000));
   }
 }
 
@@ -166,7 +187,7 @@ __global__ void __launch_bounds__(kAlphaThreads, 2)
 alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, int R, int V, int unit, int n_units,
                    const float2 *__restrict__ stats, float *__restrict__ partials) {
   extern __shared__ float sm[];
-  __shared__ float2 st[kAlphaMaxModels];
+  __shared__ float4 st[kAlphaMaxModels];
   const int r = blockIdx.x / n_units, u0 = (blockIdx.x - r * n_units) * unit, nt = min(unit, V - u0);
   const int nb = (L + 7) >> 3, lpad = nb * 8, n_off = nb * (nb - 1) / 2, n_task = n_off + (nb + 1) / 2;
   const int slices = max(1, 8 / n_task);
@@ -174,9 +195,10 @@ alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, 
   float *buf[2] = {sm, sm + (size_t)lpad * kAlphaStride};
   float *wsum = sm + 2 * (size_t)lpad * kAlphaStride;                 // [slice][task][64]
   const int n_pairs = L * (L - 1) / 2;
-  if (tid < lpad) {
+  if (tid < lpad) {                                                   // (scale, reference exponent, 1 / sum)
     const float2 v = tid < L ? stats[(size_t)tid * R + r] : make_float2(0.f, 0.f);
-    st[tid] = make_float2(v.x, tid < L ? 1.f / v.y : 0.f);
+    const bool far = __float_as_int(v.y) < 0;
+    st[tid] = make_float4(far ? 1.f : kLog2e, v.x, tid < L ? 1.f / fabsf(v.y) : 0.f, 0.f);
   }
   __syncthreads();
   // staging: 8 threads per model, 32 models at a time; vector i of a thread = tokens (8 i + tid % 8) N ..
@@ -198,7 +220,7 @@ alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, 
   };
   auto convert = [&](int t0, float *dst) {
     if (!stager) return;
-    const float n = st[sm_model].x, inv = st[sm_model].y;
+    const float4 st4 = st[sm_model];
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
       const int at = (8 * i + sv) * N;
@@ -209,7 +231,7 @@ alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, 
         if constexpr (VEC) AlphaVec<T>::unpack(raw[i], f);
         else f[0] = to_f32(raw[i]);
 #pragma unroll
-        for (int e = 0; e < N; ++e) f[e] = alpha_weight(f[e], n) * inv;
+        for (int e = 0; e < N; ++e) f[e] = alpha_weight(f[e], st4.y, st4.x) * st4.z;
       }
       float *d = dst + sm_model * kAlphaStride + at;
       if constexpr (VEC) {

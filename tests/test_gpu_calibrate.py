@@ -143,3 +143,25 @@ def test_pairwise_alpha_of_many_positions(lib, R):
     p = torch.softmax(logits.double(), -1)
     want = torch.stack([torch.minimum(p[i:i + 1], p).sum(-1).mean(-1) for i in range(3)])
     assert torch.equal(got, got.T) and (got - want).abs().max() < 1e-5
+
+
+@pytest.mark.parametrize("V,dtype", [(2048, torch.bfloat16), (2047, torch.bfloat16), (1000, torch.float32), (1001, torch.float32)])
+def test_pairwise_alpha_of_extreme_logits(lib, V, dtype):
+    """Rows far from zero, of the type's lowest value only, and half at the highest: what the softmax of the rows gives."""
+    g = torch.Generator().manual_seed(V)
+    x = torch.randn(4, 9, V, generator=g, dtype=torch.float64) * 2.0
+    fi = torch.finfo(dtype)
+    x[:, 1] += 3e4
+    x[:, 2] = x[:, 2] * 1e9 + 3e12
+    x[:, 3] = x[:, 3] * 1e31 - 2e34
+    x[:, 4] = fi.min                                     # a fully masked row: uniform
+    x[:, 5] = x[:, 5].sign() * 3.0e38
+    x[1:, 6] = fi.min                                    # masked under some models only
+    x[:, 7, V // 3:] = fi.min
+    x[:, 8, ::2] = -float("inf")
+    logits = x.to(dtype)
+    got = lib.hsd_pairwise_alpha(logits.cuda()).cpu()
+    z = logits.double()
+    p = torch.softmax(z - z.max(-1, keepdim=True).values, -1)
+    want = torch.stack([torch.minimum(p[i:i + 1], p).sum(-1).mean(-1) for i in range(4)])
+    assert torch.equal(got, got.T) and (got - want).abs().max() < 1e-5, (got, want)
