@@ -17,10 +17,9 @@ namespace hsd {
 namespace {
 
 constexpr int kAlphaThreads = 256;
-constexpr int kAlphaTile = 256;        // tokens staged at a time
+constexpr int kAlphaTile = 256;        // units are multiples of this many tokens
 constexpr int kAlphaUnit = 4096;       // tokens per partial at most: 128 per lane, all added in fp32
 constexpr int kAlphaMaxModels = 32;
-constexpr int kAlphaStride = kAlphaTile + 8;   // floats between the models of a staged tile
 
 template <typename T> struct AlphaVec;         // 16 bytes of logits
 template <> struct AlphaVec<__nv_bfloat16> {
@@ -157,14 +156,14 @@ __device__ __forceinline__ int pair_index(int i, int j, int L) { return i * L - 
 // the entries i <= 2 jj; a second one (KIND 2) is kept in the other half, entry (i, jj) at [7 - i][3 - jj].
 // Bound by instruction issue: a minimum per pair and token, one packed add per two pairs; 16 shared-memory loads feed
 // 64 pairs.
-template <int KIND>
-__device__ __forceinline__ void alpha_block(const float *pi, const float *pj, int step, float2 (*acc)[4]) {
-  for (int k = 0; k < kAlphaTile; k += step) {
+template <int KIND, int STRIDE>
+__device__ __forceinline__ void alpha_block(const float *pi, const float *pj, int tokens, int step, float2 (*acc)[4]) {
+  for (int k = 0; k < tokens; k += step) {
     float a[8], b[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) a[i] = pi[i * kAlphaStride + k];
+    for (int i = 0; i < 8; ++i) a[i] = pi[i * STRIDE + k];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) b[j] = KIND ? a[j] : pj[j * kAlphaStride + k];
+    for (int j = 0; j < 8; ++j) b[j] = KIND ? a[j] : pj[j * STRIDE + k];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
@@ -176,24 +175,27 @@ __device__ __forceinline__ void alpha_block(const float *pi, const float *pj, in
   }
 }
 
-// Block r x units + u = unit u of position r (one dimension: any number of positions).  The unit's tokens go through shared memory 256 at a time as probabilities [model][token]
-// (double-buffered: the next tile's logits are fetched under this tile's minima).  A warp owns one pair of 8-model
-// blocks, or two diagonal blocks (about as much work), and the tokens lane + 32 slice, ...; with fewer blocks than
-// warps the warps share a pair and split the tokens.
+// Block r x units + u = unit u of position r (one dimension: any number of positions).  The unit's tokens go through
+// shared memory TILE at a time as probabilities [model][token] (double-buffered: the next tile's logits are fetched under
+// this tile's minima).  A warp owns one pair of 8-model blocks, or two diagonal blocks (about as much work), and the tokens
+// lane + 32 slice, ...; with fewer blocks than warps the warps share a pair and split the tokens.
 // 32 models x 256 positions x 32000 tokens: 478 us here + 97 us of statistics; one pair per lane, two shared-memory loads
 // per pair and token, took 5021 + 176 us.
-template <typename T, bool VEC>
-__global__ void __launch_bounds__(kAlphaThreads, 2)
+// All 256 threads stage, so TILE x models is constant: 256 tokens of up to 32 models, 512 of 16, 1024 of 8.  (256 tokens of
+// two models keep 16 threads busy: 2 x 256 x 32000 in fp32 153 us, this way 70.)
+template <typename T, bool VEC, int TILE>
+__global__ void __launch_bounds__(kAlphaThreads, TILE == 1024 && VEC && sizeof(T) == 2 ? 3 : 2)
 alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, int R, int V, int unit, int n_units,
                    const float2 *__restrict__ stats, float *__restrict__ partials) {
+  constexpr int STRIDE = TILE + 8;                                    // floats between the models of a staged tile
   extern __shared__ float sm[];
   __shared__ float4 st[kAlphaMaxModels];
   const int r = blockIdx.x / n_units, u0 = (blockIdx.x - r * n_units) * unit, nt = min(unit, V - u0);
   const int nb = (L + 7) >> 3, lpad = nb * 8, n_off = nb * (nb - 1) / 2, n_task = n_off + (nb + 1) / 2;
   const int slices = max(1, 8 / n_task);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float *buf[2] = {sm, sm + (size_t)lpad * kAlphaStride};
-  float *wsum = sm + 2 * (size_t)lpad * kAlphaStride;                 // [slice][task][64]
+  float *buf[2] = {sm, sm + (size_t)lpad * STRIDE};
+  float *wsum = sm + 2 * (size_t)lpad * STRIDE;                 // [slice][task][64]
   const int n_pairs = L * (L - 1) / 2;
   if (tid < lpad) {                                                   // (scale, reference exponent, 1 / sum)
     const float2 v = tid < L ? stats[(size_t)tid * R + r] : make_float2(0.f, 0.f);
@@ -201,9 +203,9 @@ alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, 
     st[tid] = make_float4(far ? 1.f : kLog2e, v.x, tid < L ? 1.f / fabsf(v.y) : 0.f, 0.f);
   }
   __syncthreads();
-  // staging: 8 threads per model, 32 models at a time; vector i of a thread = tokens (8 i + tid % 8) N ..
-  constexpr int N = VEC ? AlphaVec<T>::N : 1, NV = kAlphaTile / 8 / N;
-  const int sm_model = tid >> 3, sv = tid & 7;
+  // staging: TPM threads per model; vector i of a thread = tokens (TPM i + tid % TPM) N ..
+  constexpr int N = VEC ? AlphaVec<T>::N : 1, TPM = TILE / 32, NV = 32 / N;
+  const int sm_model = tid / TPM, sv = tid % TPM;
   const bool stager = sm_model < lpad, in_use = sm_model < L;
   const T *row = logits + (size_t)(in_use ? sm_model : 0) * model_stride + (size_t)r * V + u0;
   typename std::conditional<VEC, uint4, T>::type raw[NV];
@@ -211,7 +213,7 @@ alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, 
     if (!in_use) return;
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      const int k = t0 + (8 * i + sv) * N;
+      const int k = t0 + (TPM * i + sv) * N;
       if (k < nt) {
         if constexpr (VEC) raw[i] = __ldg(reinterpret_cast<const uint4 *>(row + k));
         else raw[i] = row[k];
@@ -223,7 +225,7 @@ alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, 
     const float4 st4 = st[sm_model];
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      const int at = (8 * i + sv) * N;
+      const int at = (TPM * i + sv) * N;
       float f[N];
 #pragma unroll
       for (int e = 0; e < N; ++e) f[e] = 0.f;
@@ -233,7 +235,7 @@ alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, 
 #pragma unroll
         for (int e = 0; e < N; ++e) f[e] = alpha_weight(f[e], st4.y, st4.x) * st4.z;
       }
-      float *d = dst + sm_model * kAlphaStride + at;
+      float *d = dst + sm_model * STRIDE + at;
       if constexpr (VEC) {
 #pragma unroll
         for (int e = 0; e < N; e += 4) *reinterpret_cast<float4 *>(d + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
@@ -256,18 +258,20 @@ alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, 
   fetch(0);
   convert(0, buf[0]);
   __syncthreads();
-  for (int t0 = 0, b = 0; t0 < nt; t0 += kAlphaTile, b ^= 1) {
-    const bool more = t0 + kAlphaTile < nt;
-    if (more) fetch(t0 + kAlphaTile);
+  for (int t0 = 0, b = 0; t0 < nt; t0 += TILE, b ^= 1) {
+    const bool more = t0 + TILE < nt;
+    if (more) fetch(t0 + TILE);
     if (busy) {
       const float *p = buf[b] + slice * 32 + lane;
-      if (!diag) alpha_block<0>(p + bi * 8 * kAlphaStride, p + bj * 8 * kAlphaStride, 32 * slices, acc);
+      const int tokens = TILE == 1024 ? min(TILE, nt - t0) - slice * 32 : TILE, step = 32 * slices;   // (the tile is zero past the unit's tokens)
+      if (TILE == 1024) alpha_block<1, STRIDE>(p, nullptr, tokens, step, acc);    // one block of eight models
+      else if (!diag) alpha_block<0, STRIDE>(p + bi * 8 * STRIDE, p + bj * 8 * STRIDE, tokens, step, acc);
       else {
-        alpha_block<1>(p + bi * 8 * kAlphaStride, nullptr, 32 * slices, acc);
-        if (two) alpha_block<2>(p + bj * 8 * kAlphaStride, nullptr, 32 * slices, acc);
+        alpha_block<1, STRIDE>(p + bi * 8 * STRIDE, nullptr, tokens, step, acc);
+        if (two) alpha_block<2, STRIDE>(p + bj * 8 * STRIDE, nullptr, tokens, step, acc);
       }
     }
-    if (more) convert(t0 + kAlphaTile, buf[b ^ 1]);
+    if (more) convert(t0 + TILE, buf[b ^ 1]);
     __syncthreads();
   }
   // lane sums; the slices of a task are added in slice order
@@ -338,22 +342,31 @@ AlphaPlan alpha_plan(int L, int R, int V) {
   return p;
 }
 
+template <typename T, bool VEC, int TILE>
+int launch_pairs(const T *logits, long long model_stride, int L, int R, int V, const AlphaPlan &p, const float2 *stats, float *partials, cudaStream_t s) {
+  const int lpad = (L + 7) / 8 * 8;
+  const size_t smem = (2 * (size_t)lpad * (TILE + 8) + 8 * 64) * sizeof(float);
+  static bool attr_set = false;
+  if (!attr_set) {
+    HSD_CUDA_OK(cudaFuncSetAttribute(alpha_pairs_kernel<T, VEC, TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+    attr_set = true;
+  }
+  alpha_pairs_kernel<T, VEC, TILE><<<p.n_units * R, kAlphaThreads, smem, s>>>(logits, model_stride, L, R, V, p.unit, p.n_units, stats, partials);
+  return HSD_OK;
+}
+
 template <typename T, bool VEC>
-int launch_alpha_t(const void *logits, long long model_stride, int L, int R, int V, void *ws, double *alpha, cudaStream_t s) {
+int launch_alpha_t(const T *logits, long long model_stride, int L, int R, int V, void *ws, double *alpha, cudaStream_t s) {
   const AlphaPlan p = alpha_plan(L, R, V);
   float2 *stats = (float2 *)((char *)ws + p.stats_off);
   float *partials = (float *)((char *)ws + p.partials_off);
-  alpha_stats_kernel<T, VEC><<<dim3(R, L), kAlphaThreads, 0, s>>>((const T *)logits, model_stride, R, V, stats);
-  if (p.n_pairs > 0) {
-    const int lpad = (L + 7) / 8 * 8;
-    const size_t smem = (2 * (size_t)lpad * kAlphaStride + 8 * 64) * sizeof(float);
-    static bool attr_set = false;
-    if (!attr_set) {
-      if (cudaFuncSetAttribute(alpha_pairs_kernel<T, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) != cudaSuccess) return HSD_E_CUDA;
-      attr_set = true;
-    }
-    alpha_pairs_kernel<T, VEC><<<p.n_units * R, kAlphaThreads, smem, s>>>((const T *)logits, model_stride, L, R, V, p.unit, p.n_units, stats, partials);
-  }
+  alpha_stats_kernel<T, VEC><<<dim3(R, L), kAlphaThreads, 0, s>>>(logits, model_stride, R, V, stats);
+  int st = HSD_OK;
+  if (p.n_pairs > 0)
+    st = L <= 8    ? launch_pairs<T, VEC, 1024>(logits, model_stride, L, R, V, p, stats, partials, s)
+         : L <= 16 ? launch_pairs<T, VEC, 512>(logits, model_stride, L, R, V, p, stats, partials, s)
+                   : launch_pairs<T, VEC, 256>(logits, model_stride, L, R, V, p, stats, partials, s);
+  if (st) return st;
   alpha_reduce_kernel<<<p.n_pairs > 0 ? min(p.n_pairs, 592) : 1, kAlphaThreads, 0, s>>>(partials, L, R * p.n_units, R, alpha);
   hsd_count_launches(p.n_pairs > 0 ? 3 : 2);
   return hsd_launch_status();
@@ -364,8 +377,8 @@ int launch_alpha(const void *logits, long long model_stride, int L, int R, int V
   // 16-byte loads need every row on a 16-byte boundary and no partial vector at a row's end
   constexpr int N = AlphaVec<T>::N;
   const bool vec = V % N == 0 && model_stride % N == 0 && ((uintptr_t)logits & 15) == 0;
-  return vec ? launch_alpha_t<T, true>(logits, model_stride, L, R, V, ws, alpha, s)
-             : launch_alpha_t<T, false>(logits, model_stride, L, R, V, ws, alpha, s);
+  return vec ? launch_alpha_t<T, true>((const T *)logits, model_stride, L, R, V, ws, alpha, s)
+             : launch_alpha_t<T, false>((const T *)logits, model_stride, L, R, V, ws, alpha, s);
 }
 
 }  // namespace

@@ -99,7 +99,9 @@ def test_calibrate_then_search_end_to_end(lib):
 
 @pytest.mark.parametrize("L,R,V,dtype", [(9, 2, 4104, torch.bfloat16),      # two 8-model blocks, a unit of one 8-token vector
                                          (17, 3, 9001, torch.float32),       # three blocks, rows off the 16-byte grid
-                                         (24, 2, 5000, torch.float32), (32, 2, 8200, torch.bfloat16), (32, 1, 255, torch.bfloat16)])
+                                         (24, 2, 5000, torch.float32), (32, 2, 8200, torch.bfloat16), (32, 1, 255, torch.bfloat16),
+                                         # up to eight models: 1024-token tiles, a last one of 904 and of 1 token; up to sixteen: 512
+                                         (2, 40, 5000, torch.bfloat16), (8, 3, 3073, torch.float32), (3, 700, 24, torch.float32), (16, 2, 4608, torch.bfloat16)])
 def test_pairwise_alpha_block_edges(lib, L, R, V, dtype):
     """Model counts at the ends of the 8-model blocks and vocabularies at the ends of tiles and units."""
     g = torch.Generator().manual_seed(L + V)
