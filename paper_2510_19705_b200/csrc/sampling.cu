@@ -925,13 +925,14 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
 // are too long or too many for this path.
 struct ClusterPlan { int C, NT, per, staged, seg; size_t smem; };
 constexpr size_t kClMaxSmem = 216 * 1024;
+constexpr int kClSMs = 148, kClEights = 14;       // SMs of the GPU; clusters of eight that run at once (one CTA per SM)
 static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, int rows, bool draw, ClusterPlan *pl) {
   if (rows > kClMaxRows) return false;
   pl->per = (dtype == HSD_BF16 && V % 2 == 0 && ((uintptr_t)p & 3) == 0 && ((uintptr_t)q & 3) == 0) ? 2 : 1;
-  // as many CTAs as run at once (draws: two per SM), of at least 4096 tokens (eight a thread) each: clusters of eight do not fit all 148 SMs
+  // as many CTAs as run at once (draws: two per SM), of at least 4096 tokens (eight a thread) each: clusters of eight do not fit all SMs
   // (16 of them took two rounds), clusters of four and two do
   int C = 1;
-  while (C < kClMaxC && V > C * 4096 && 2 * C * n <= (C == 4 ? 112 : draw ? 296 : 148)) C *= 2;
+  while (C < kClMaxC && V > C * 4096 && 2 * C * n <= (C == 4 ? 8 * kClEights : draw ? 2 * kClSMs : kClSMs)) C *= 2;
   const int most = (draw ? 16 : 32) * kClThreads;
   while (C < kClMaxC && ceil_div(V, C) > most - 64) C *= 2;
   const int seg = ceil_div(ceil_div(V, C), 64) * 64;
@@ -946,24 +947,35 @@ static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, 
   return true;
 }
 // Where the cluster path is the faster one (us a call on an idle GPU, cluster / other path).  Its time grows with the
-// tokens a CTA goes through, rows x seg; the other paths give every row a CTA of its own.
-//   verification, rows the fused kernel takes (V = 32000 bf16): t = 3: 1 to 8 sequences 12 / 25, 32: 17 / 30, 64 (112k
-//     tokens a CTA): 38 / 35; t = 8: 8 sequences (68k) 19 / 26, 16 (136k): 36 / 30.
+// tokens a CTA goes through, rows x 512 NT, and with the rounds its clusters need; the other paths give every row a CTA
+// of its own.
+//   verification, rows the fused kernel takes: both times from their fits (within 10 % of 140 measured calls: V 64 to
+//     32000, 1 to 128 sequences, t 1 to 16), the cluster path where its own is the smaller by 15 %.  V = 32000
+//     bf16, t = 3: 1 to 8 sequences 12 / 25, 32: 17 / 30, 64: 38 / 35; t = 8: 8 sequences 19 / 26, 16: 36 / 30.  V = 2048,
+//     t = 16: 16 sequences 37 / 25, 64: 37 / 51; t = 8: 4 sequences 21 / 19, 32: 21 / 25.
 //   other rows: statistics and decision kernels, each row read twice by one CTA.  fp32, V = 32001: t = 3 14 / 58, t = 8
-//     30 / 58; V = 9001: t = 3 14 / 15, t = 8 29 / 15; V = 2048: t = 3 11 / 7.  bf16 of odd length, 49999: t = 3 21 / 50, t = 8 55 / 50.
+//     30 / 58; V = 9001: t = 3 14 / 15, t = 8 29 / 15; V = 2048: t = 3 11 / 7.  bf16 of odd length, 49999: t = 3 21 / 50, t = 8 55 / 50;
+//     128 sequences at t = 1 (four rounds) 98 / 79, fp32 97 / 82; rows of more than 50000 tokens take the other path so much
+//     longer that rounds do not matter (65536, 128 sequences: 88 / 142).
 //   draws (two CTAs per SM, 16 tokens a thread at most): bf16 32000: 1 row 4.4 / 10.6, 64 rows 6.7 / 11.3 (one CTA per
 //     SM, 32 tokens a thread: 11.2), 100 rows would take a second round; fp32 32000: 1 row 5.7 / 28, 64 rows 8.6 / 28; 16001:
-//     5.2 / 10.8; 9001 (two CTAs a row): 6.9 / 6.2, 2048: 6.8 / 3.9; bf16 2048 (one CTA): 6.7 / 9.8.
-static bool cluster_pays_verify(const ClusterPlan &pl, int dtype, int V, int rows, bool fused) {
+//     5.2 / 10.8; 9001 (two CTAs a row): 6.9 / 6.2, 12289 (two) 10.4 / 9.5, (four) 6.3 / 9.5, 2048: 6.8 / 3.9; bf16 2048 (one CTA): 6.7 / 9.8.
+static bool cluster_pays_verify(const ClusterPlan &pl, int dtype, int V, int batch, int rows, bool fused) {
   const long long work = (long long)pl.seg * rows;
-  if (fused) return work <= 100000;
+  if (fused) {
+    const double tokens = 512.0 * pl.NT * rows, rounds = ceil_div(pl.C * batch, kClSMs);
+    const double cluster_us = rounds * (7.5 + tokens * (pl.NT == 32 ? 2.7e-4 : 2.05e-4));
+    const double fused_us = 17.5 + V * 2.4e-4 + (double)batch * rows * (0.0155 + V * 4e-7);
+    return cluster_us * 1.15 < fused_us;
+  }
+  if (pl.C * batch > 2 * kClSMs && V <= 50000) return false;
   if (dtype == HSD_BF16) return work * 5 <= 8ll * V;
   return V > 20000 ? work <= 4ll * V : work * 5 <= 11ll * V;
 }
 static bool cluster_pays_draw(const ClusterPlan &pl, int dtype, int V, int n, bool chunked) {
-  if (pl.seg > 4096 && pl.C * n > 296) return false;
+  if (pl.seg > 4096 && pl.C * n > 2 * kClSMs) return false;
   if (dtype == HSD_BF16 && chunked) return pl.seg <= 4096 || pl.C > 1;
-  return V > 12000 && pl.C > 1;
+  return V > (pl.C > 2 ? 12000 : 13000) && pl.C > 1;
 }
 
 template <typename T, int PER, int NT, bool DRAW>
@@ -1071,7 +1083,7 @@ int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int 
   const bool fused = dtype == HSD_BF16 && V % 8 == 0 && V <= kFusedMaxV && smem <= 220 * 1024 && ((uintptr_t)p & 15) == 0 &&
                      (q == nullptr || ((uintptr_t)q & 15) == 0) && t_max < kFusedConsumers;
   ClusterPlan pl;
-  if (cluster_plan(p, q, dtype, V, batch, 2 * t_max + 1, false, &pl) && cluster_pays_verify(pl, dtype, V, 2 * t_max + 1, fused)) {
+  if (cluster_plan(p, q, dtype, V, batch, 2 * t_max + 1, false, &pl) && cluster_pays_verify(pl, dtype, V, batch, 2 * t_max + 1, fused)) {
     ClusterArgs a = {};
     a.p = p; a.q = q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.desc = desc; a.regular_t = regular_t;
     a.regular_serial = regular_serial; a.regular_level = regular_level; a.seed = seed; a.out_tokens = out_tokens; a.out_n = out_n;

@@ -120,7 +120,9 @@ def test_bad_arguments_are_rejected(lib):
                                          ("bf16", 4098, 2, 2),       # two CTAs, the second with an odd tail of pairs
                                          ("bf16", 32000, 14, 2), ("bf16", 32000, 15, 2),    # clusters of eight / of four
                                          ("bf16", 65538, 1, 1),      # 32 tokens a thread
-                                         ("bf16", 1536, 2, 31),      # the most rows a sequence can have here; read twice, not staged
+                                         ("bf16", 1536, 2, 31),      # the most rows a sequence can have here
+                                         ("bf16", 512, 128, 16),     # one CTA a sequence, its 33 rows read twice, not staged
+                                         ("bf16", 2048, 16, 16), ("bf16", 2048, 64, 8),     # the fused kernel's side of the line, the clusters'
                                          ("bf16", 30001, 2, 1), ("fp32", 32769, 1, 8), ("fp32", 24001, 40, 1), ("bf16", 9000, 2, 0)])
 def test_cluster_decisions_match_oracle(lib, dtype, V, B, t):
     p, q = inputs.make_accept_logits(B, t, V, seed=V + 7 * t, device="cuda", dtype=dtype)
