@@ -37,6 +37,9 @@ template <int NPAD> struct TcCfg {
   static constexpr int kStages = kFit < 12 ? kFit : 12;       // 12 x 16 KiB of weights in flight per SM cover HBM's latency twice
   static constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + kCtrlBytes + 1024;
   static constexpr int kBufs = NPAD == 256 ? 1 : 2;           // tiles whose accumulators exist at a time, two accumulators each
+  // one tile at a time: the epilogue adds the first accumulator to the second, and the next tile's first half runs under
+  // the finish from there (128256 x 4096 at 256 rows: 322 -> 255 us)
+  static constexpr bool kFold = kBufs == 1;
   static constexpr int kTmemCols = 2 * kBufs * NPAD;
   static_assert(NPAD * kLd * 4 <= kStages * kStageBytes, "a cluster's partial sums must fit the ring");
 };
@@ -230,7 +233,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           if (!mbar_wait(full_bar(s), ph, abort_flag)) { ok = false; break; }
           const uint32_t wa = smem_u32(ring + (size_t)s * Cfg::kStageBytes);
           const uint64_t da = umma_desc(wa), db = umma_desc(wa + kStageWBytes);
-          if (kb == kb_half) { d_tmem += NPAD; acc = 0u; }
+          if (kb == kb_half) {
+            if (Cfg::kFold) {
+              if (!mbar_wait(acce_bar(1), (uint32_t)(ti & 1) ^ 1u, abort_flag)) { ok = false; break; }
+              tc_fence_after();
+            }
+            d_tmem += NPAD; acc = 0u;
+          }
 #pragma unroll
           for (int k = 0; k < kTcBlockK / 16; ++k) {
             umma_bf16(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, acc);
@@ -260,17 +269,38 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       const TileInfo info = tile_info(args, tile);
       const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * 2 * NPAD);
       float *part = S > 1 ? reinterpret_cast<float *>(ring) : staging;       // S > 1: every load of the CTA has been consumed
+      const bool fold = Cfg::kFold && S == 1 && kb_half < kb1;
+      if (fold) {
+#pragma unroll 1
+        for (int c0 = 0; c0 < NPAD && c0 < args.R; c0 += CH) {
+          float v[CH], v2[CH];
+#pragma unroll
+          for (int j = 0; j < CH / 16; ++j) {
+            tmem_ld16(tbase + (uint32_t)(c0 + j * 16), v + j * 16);
+            tmem_ld16(tbase + (uint32_t)(NPAD + c0 + j * 16), v2 + j * 16);
+          }
+          tmem_ld_wait();
+#pragma unroll
+          for (int r = 0; r < CH; ++r) v[r] += v2[r];
+#pragma unroll
+          for (int j = 0; j < CH / 16; ++j) tmem_st16u(tbase + (uint32_t)(NPAD + c0 + j * 16), reinterpret_cast<const unsigned *>(v + j * 16));
+        }
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acce_bar(0));
+      }
 #pragma unroll 1
       for (int c0 = 0; c0 < NPAD && c0 < args.R; c0 += CH) {
         float v[CH], v2[CH];
 #pragma unroll
-        for (int j = 0; j < CH / 16; ++j) tmem_ld16(tbase + (uint32_t)(c0 + j * 16), v + j * 16);
-        if (kb_half < kb1) {
+        for (int j = 0; j < CH / 16; ++j) tmem_ld16(tbase + (uint32_t)((fold ? NPAD : 0) + c0 + j * 16), v + j * 16);
+        if (kb_half < kb1 && !fold) {
 #pragma unroll
           for (int j = 0; j < CH / 16; ++j) tmem_ld16(tbase + (uint32_t)(NPAD + c0 + j * 16), v2 + j * 16);
         }
         tmem_ld_wait();
-        if (kb_half < kb1) {
+        if (kb_half < kb1 && !fold) {
 #pragma unroll
           for (int r = 0; r < CH; ++r) v[r] += v2[r];
         }
@@ -291,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(acce_bar(ab));
+      if (lane == 0) mbar_arrive(acce_bar(fold ? 1 : ab));
     }
   }
   __syncwarp();

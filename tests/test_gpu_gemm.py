@@ -47,8 +47,9 @@ def test_gemm_rejects_bad_shapes(lib):
 @pytest.mark.parametrize("R,N,K", [(24, 14257, 256),     # whole tiles of 104 rows, the last one of 9
                                    (256, 2048, 5632),    # k-blocks over a cluster of four, one accumulator buffer
                                    (5, 100, 64),         # one k-block: no split, no second accumulator
-                                   (17, 1000, 192),      # three k-blocks over a cluster of three
-                                   (33, 19100, 128)])    # more tiles than SMs: a CTA's second tile
+                                   (17, 1000, 192),      # three k-blocks over a cluster of two: one and two
+                                   (33, 19100, 128),     # more tiles than SMs: a CTA's second tile
+                                   (200, 19100, 192), (256, 57000, 128), (129, 38000, 64)])   # ... with room for one tile's accumulators
 def test_gemm_tile_and_cluster_edges(lib, R, N, K):
     g = torch.Generator().manual_seed(R + N + K)
     A = torch.randn(R, K, generator=g).to(torch.bfloat16).cuda()
