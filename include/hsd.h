@@ -188,8 +188,8 @@ int hsd_set_phase_folding(hsd_ctx *ctx, int fold_qkv, int fold_gate_up, int earl
  * head size 128, an item with 8 or more query vectors whose key range has 2048 keys or more runs on the
  * fifth-generation tensor cores with its scores and outputs in tensor memory; enabled = 0: every item runs on the warp-level path.  Both paths compute the
  * same attention (softmax weights rounded to bf16 before the P V product on the tensor-memory path, to bf16 hi + lo
- * on the other), so results agree to rounding, not bit for bit.  (Prompt chunks of more than 128 rows
- * have an attention kernel of their own, which this does not affect.)  enabled = 2 additionally keeps the key splits of
+ * on the other), so results agree to rounding, not bit for bit.  (Prompts on the many-row
+ * path have an attention kernel of their own, with hi + lo weights at every length, which this does not affect.)  enabled = 2 additionally keeps the key splits of
  * long contexts at 2048 keys or more, so that small test models reach that path too.  A test hook and a tuning knob.
  * Errors: INVALID_ARG. */
 int hsd_set_tensor_attention(hsd_ctx *ctx, int enabled);

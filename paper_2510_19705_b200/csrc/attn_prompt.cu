@@ -4,7 +4,7 @@
 // KV group), over all keys up to the last of them, in tiles of 64 keys.  Per key tile and query tile
 //   S[128 x 64]   = Q K^T                      both operands in shared memory
 //   P             = exp2((S - m_ref) scale log2 e), thread = query vector, split into bf16 hi + lo halves that overwrite
-//                   S (the P V product keeps about 16 bits of P); with 2048 keys or more one bf16, as in the decode passes
+//                   S (the P V product keeps about 16 bits of P, at every length)
 //   O[128 x hd]  += P_hi V + P_lo V            A operand from tensor memory, V as it lies in the cache (MN-major)
 // m_ref moves only when a row maximum passes it by a factor 256; then O is rescaled.  Two query tiles share every K
 // and V tile.  S has two buffers per query tile: the scores of the next key tile are ready when the weights of this one
@@ -30,7 +30,6 @@ constexpr int TK = 64;                                   // keys per tile
 constexpr int kQBlk = 128 * 128;                         // [128 query vectors][64 bf16] block, 128-byte swizzle
 constexpr int kBlk = TK * 128;                           // [64 keys][64 bf16] block
 constexpr int kStages = 4;
-constexpr int kBf16WeightKeys = 2048;                    // as in the decode passes: from here on the weights are one bf16 each
 
 template <int HD> struct Cfg {
   static constexpr int NB = HD / 64;                     // 64-column blocks
@@ -94,7 +93,6 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
   const int kv_len = pos0 + ntok;
   const int nA = (pos0 + tokA + TK - 1) / TK, nB = tokB > 0 ? (kv_len + TK - 1) / TK : 0;
   const int n = max(nA, nB);
-  const bool hilo = kv_len < kBf16WeightKeys;
 
   if (threadIdx.x == 0) {
     for (int b = 0; b < kStages; ++b) { mbar_init(k_full(b), 1); mbar_init(k_free(b), 1); mbar_init(v_full(b), 1); mbar_init(v_free(b), 1); }
@@ -210,10 +208,8 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
           const uint32_t d = tO(x), p = tS(x) + (uint32_t)((j & 1) * TK);
 #pragma unroll
           for (int ks = 0; ks < TK / 16; ++ks) umma_ts(d, p + ks * 16, vb + ks * 128, id2, ks > 0 ? 1u : (j > 0 ? 1u : 0u));
-          if (hilo) {
 #pragma unroll
-            for (int ks = 0; ks < TK / 16; ++ks) umma_ts(d, p + ks * 16 + 8, vb + ks * 128, id2, 1u);
-          }
+          for (int ks = 0; ks < TK / 16; ++ks) umma_ts(d, p + ks * 16 + 8, vb + ks * 128, id2, 1u);
           umma_commit(pv_done(x));
           if (j + 2 < nx) issue_s(x, j + 2);                         // over P(j), after the products that read it
           if (j + 1 == nx) umma_commit(o_done(x));
@@ -295,14 +291,12 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
           else l2a = __fadd2_rn(l2a, p);
           const __nv_bfloat162 h2 = __floats2bfloat162_rn(p.x, p.y);
           hi[e] = *reinterpret_cast<const unsigned *>(&h2);
-          if (hilo) {
-            const float2 r = __ffma2_rn(make_float2(__uint_as_float(hi[e] << 16), __uint_as_float(hi[e] & 0xFFFF0000u)), make_float2(-1.f, -1.f), p);
-            const __nv_bfloat162 lw = __floats2bfloat162_rn(r.x, r.y);
-            lo[e] = *reinterpret_cast<const unsigned *>(&lw);
-          }
+          const float2 r = __ffma2_rn(make_float2(__uint_as_float(hi[e] << 16), __uint_as_float(hi[e] & 0xFFFF0000u)), make_float2(-1.f, -1.f), p);
+          const __nv_bfloat162 lw = __floats2bfloat162_rn(r.x, r.y);
+          lo[e] = *reinterpret_cast<const unsigned *>(&lw);
         }
         tmem_st8u(S + (uint32_t)c, hi);
-        if (hilo) tmem_st8u(S + (uint32_t)(c + 8), lo);
+        tmem_st8u(S + (uint32_t)(c + 8), lo);
       }
       l += (l2a.x + l2a.y) + (l2b.x + l2b.y);
       tmem_st_wait();

@@ -52,3 +52,24 @@ def test_prompt_chunks_match_oracle(hd, nq, nkv, page, batch, prompt):
         # the bound of the other bf16 parity tests: 2e-2 on logits of standard deviation 0.02 sqrt(256) = 0.32
         err = float(np.abs(om.last_logits64 - rec["logits"]).max())
         assert err < 2e-2, (b, err)
+
+
+@pytest.mark.parametrize("hd,nq,nkv,batch,prompt", [
+    (64, 8, 4, 2, 2100),           # the second sequence starts in the middle of a chunk: other items, other key ranges
+    (128, 4, 1, 2, 2100)])
+def test_a_prompt_does_not_depend_on_its_place_in_the_batch(hd, nq, nkv, batch, prompt):
+    # the same prompt as every sequence of a batch: the chunks cut each of them somewhere else
+    cfg = inputs.model_cfg(3, 256, nq, nkv, 704, 1024, "bf16", head_dim=hd)
+    w = inputs.make_weights(cfg, 11, device="cuda")
+    prompts = inputs.make_prompts(cfg["vocab"], 1, prompt, 3).repeat(batch, 1)
+    eng = binding.Hsd(cfg, w, (1, 3), (2,), max_batch=batch, max_seq=prompt + 32)
+    with tempfile.TemporaryDirectory() as tmp:
+        path = os.path.join(tmp, "trace.bin")
+        eng.set_trace(path, logit_calls=2 * batch)
+        eng.generate(prompts.cuda(), 2, 5)
+        eng.set_trace(None)
+        recs = binding.read_trace(path)
+    eng.close()
+    rows = [next(r for r in recs if r["level"] == 1 and r["seq"] == b)["logits"][0] for b in range(batch)]
+    for b in range(1, batch):
+        assert np.array_equal(rows[b], rows[0]), b
