@@ -218,8 +218,12 @@ int hsd_set_exit_heads(hsd_ctx *ctx, const void *const *final_norms, const void 
 int hsd_set_iid_acceptance(hsd_ctx *ctx, const double *alphas);
 
 /* Generate n_new tokens per sequence with Algorithm 1 called at idx = K until enough tokens exist
- * (the first n_new are returned).  Sequence b produces exactly the tokens it would produce alone
- * with the same seed (uniforms are keyed by b).
+ * (the first n_new are returned).  Sequence b produces the tokens it would produce alone with the same seed
+ * (uniforms are keyed by b): exactly, by construction, for the small fp32 models whose passes are one launch (at
+ * most 8 MB of weights a layer and 64 MB of output head, head size 32 / 64 / 128, 16-byte-aligned weights), whose rows do
+ * not depend on the rest of a pass.  In other models the division of a long key range among CTAs, and with bf16 the path of a
+ * prompt, follow the rows of a pass: logits agree to rounding, and a token can differ where a uniform falls
+ * between two such roundings.
  *   prompt_ids  device int32 [batch, prompt_len], prompt_len >= 1
  *   out_tokens  device int32 [batch, n_new]
  *   stats       host [n_levels] or NULL; overwritten

@@ -215,7 +215,7 @@ struct Model {
   bool use_tc = false, use_persist = false;   // tensor-core GEMMs / the one-launch persistent forward (bf16 models)
   std::vector<CUtensorMap> wmaps;             // [n_layers * 7 + kHeadMaps]: wq wk wv wo wg wu wd per layer, then the levels' heads, the shared head
   CUtensorMap amaps[4][5];                    // activation buffers {h, att, act, hf} x row padding {16, 32, 64, 128, 256}
-  bool use_small = false;                     // passes of few rows of a small fp32 model: one launch (fwd_small)
+  bool use_small = false;                     // a small fp32 model: fwd_small runs its passes
   int small_grid = 1;
   bool use_prompt = false;                    // long prompts run forward_prompt
   std::vector<CUtensorMap> kvmaps;            // [n_layers][4]: K and V pools of each layer, two box heights each, for the prompt attention
@@ -424,6 +424,10 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
   int *row_seq = (int *)(host + o_seq), *row_pos = (int *)(host + o_pos), *lsrc = (int *)(host + o_src);
   int4 *attn = (int4 *)(host + o_attn);
   long long *ldst = (long long *)(host + o_dst);
+  // Every pass of a small fp32 model runs fwd_small, whatever its rows: a row's sums then do not depend on the rest of the
+  // pass.  (A level's own head or norm gain may lie on any 4-byte boundary: such a level keeps the launches per operation.)
+  const bool small = M.use_small && (((uintptr_t)c->level_head[level] | (uintptr_t)c->level_norm[level]) & 15) == 0;
+  std::vector<int> group_logits(small ? ceil_div(R, kSmallRows) : 0, 0);     // logit rows of each launch
   int r = 0, ia = 0, il = 0;
   for (const SeqWork &w : work) {
     for (int p0 = w.start; p0 < w.end; p0 += arows) {
@@ -434,7 +438,8 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
       row_seq[r] = w.b;
       row_pos[r] = p;
       if (w.logit_first >= 0 && p >= w.logit_first) {
-        lsrc[il] = r;
+        lsrc[il] = small ? r % kSmallRows : r;
+        if (small) ++group_logits[r / kSmallRows];
         ldst[il] = (long long)w.b * L.slots[level] + w.slot0 + (p - w.logit_first);
         if (w.slot0 + (p - w.logit_first) >= L.slots[level]) return HSD_E_INVALID_ARG;
         ++il;
@@ -610,25 +615,26 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     mark_valid();
     return HSD_OK;
   }
-  // (a level's own head or norm gain may lie on any 4-byte boundary: such a level keeps the launches per operation)
-  const bool heads_aligned = (((uintptr_t)c->level_head[level] | (uintptr_t)c->level_norm[level]) & 15) == 0;
-  if (M.use_small && R <= kSmallRows && n_logit <= kSmallRows && heads_aligned) {
+  if (small) {
     SmallFwdArgs a;
     a.d = md.d; a.nq = md.nq; a.nkv = md.nkv; a.hd = md.hd; a.ff = md.ff; a.V = md.V; a.n_run = c->exits[level]; a.max_seq = md.max_seq;
     a.page = md.page; a.pages_per_seq = md.pages_per_seq; a.n_pages = md.n_pages; a.eps = md.eps;
     a.layers = c->dev<SmallLayerDev>(ML.small_layers);
     a.embed = (const float *)M.embed; a.final_norm = (const float *)c->level_norm[level]; a.lm_head = (const float *)c->level_head[level];
     a.cos_tab = c->dev<float>(ML.cos_tab); a.sin_tab = c->dev<float>(ML.sin_tab);
-    a.R = R; a.L = n_logit;
     a.tokens = c->dev<int>(L.tokens); a.page_table = c->dev<int>(L.page_table);
-    a.row_seq = rb.row_seq; a.row_pos = rb.row_pos; a.lrow_src = rb.lrow_src; a.lrow_dst = rb.lrow_dst;
     a.x = c->dev<float>(ML.x); a.q = c->dev<float>(ML.q); a.att = c->dev<float>(ML.att); a.act = c->dev<float>(ML.act);
     a.logits = (float *)(c->ws + L.logits[level]);
     a.counter = c->dev<unsigned>(L.grid_counter) + 48;        // behind the words the bf16 forward clears
-    a.base = c->small_base;
     a.status = (int *)(c->ws + c->status_off);
-    HSD_TRY(launch_forward_small(a, M.small_grid, s));
-    c->small_base += fwd_small_arrivals(a.n_run, a.L, M.small_grid);
+    for (int g = 0, l0 = 0; g * kSmallRows < R; l0 += a.L, ++g) {       // (a sequence's rows ascend: its earlier keys are there)
+      a.R = std::min(kSmallRows, R - g * kSmallRows); a.L = group_logits[g];
+      a.row_seq = rb.row_seq + g * kSmallRows; a.row_pos = rb.row_pos + g * kSmallRows;
+      a.lrow_src = rb.lrow_src + l0; a.lrow_dst = rb.lrow_dst + l0;
+      a.base = c->small_base;
+      HSD_TRY(launch_forward_small(a, M.small_grid, s));
+      c->small_base += fwd_small_arrivals(a.n_run, a.L, M.small_grid);
+    }
     if (tp) cudaEventRecord(tp->b, s);
     c->stats[level].forwards++;
     c->stats[level].rows += R;

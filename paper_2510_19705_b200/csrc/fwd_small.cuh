@@ -1,4 +1,4 @@
-// One-launch verifier forward of small fp32 models (passes of a few rows).
+// One-launch verifier forward of small fp32 models.
 #pragma once
 #include "common.cuh"
 #include "forward.cuh"
@@ -21,7 +21,7 @@ struct SmallFwdArgs {
   int *status;                       // set non-zero when a bounded wait gave up
 };
 
-constexpr int kSmallRows = 32;
+constexpr int kSmallRows = 128;          // rows of one launch; longer passes are several, in row order
 bool fwd_small_supported(const ModelDims &md);
 int fwd_small_grid(const ModelDims &md, int sm_count);
 // Barrier arrivals of one launch (added to the counter).

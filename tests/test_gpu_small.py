@@ -1,4 +1,4 @@
-"""Small fp32 models: passes of up to 32 rows in one launch, against the oracle, where the row tiles, staged chunks,
+"""Small fp32 models: a pass in one launch per 128 rows, against the oracle, where the row tiles, staged chunks,
 head sizes and the vocabulary end."""
 import os
 import tempfile
@@ -38,3 +38,27 @@ def test_small_fp32_passes_match_oracle(d, nq, nkv, hd, ff, V, page, batch, prom
         om.rows(1, prompts[b].tolist(), rec["tokens"][:-1].tolist())
         err = float(np.abs(om.last_logits64 - rec["logits"]).max())
         assert err < 1e-5, (b, err)                # the bound of the other fp32 parity tests
+
+
+@pytest.mark.parametrize("d,nq,nkv,hd,ff,V,prompt", [(128, 4, 4, 32, 512, 512, 16), (256, 4, 2, 64, 700, 1001, 70)])
+def test_small_fp32_rows_do_not_depend_on_the_batch(d, nq, nkv, hd, ff, V, prompt):
+    """Sequence 0 alone, in a batch whose passes have more than 32 rows, and in one whose passes have more than 128: the
+    same logits bit for bit in every pass."""
+    cfg = inputs.model_cfg(3, d, nq, nkv, ff, V, "fp32", head_dim=hd)
+    w = inputs.make_weights(cfg, 13, device="cuda")
+    prompts = inputs.make_prompts(V, 40, prompt, 4)
+    seen = []
+    for batch in (1, 9, 40):
+        eng = binding.Hsd(cfg, w, (1, 3), (4,), max_batch=batch, max_seq=prompt + 40)
+        with tempfile.TemporaryDirectory() as tmp:
+            path = os.path.join(tmp, "trace.bin")
+            eng.set_trace(path, logit_calls=10 ** 6)
+            toks, _, _ = eng.generate(prompts[:batch].cuda(), 8, 5)
+            eng.set_trace(None)
+            recs = [r for r in binding.read_trace(path) if r["seq"] == 0]
+        eng.close()
+        seen.append((toks[0].cpu().numpy(), [(r["level"], r["logits"]) for r in recs]))
+    for toks, recs in seen[1:]:
+        assert np.array_equal(toks, seen[0][0]) and len(recs) == len(seen[0][1])
+        for (level, a), (want_level, b) in zip(recs, seen[0][1]):
+            assert level == want_level and np.array_equal(a, b)
