@@ -934,12 +934,14 @@ int prefill(hsd_ctx *c, int batch, int prompt_len) {
   const int K = c->n_levels - 1;
   int end = prompt_len - 1;
   std::vector<int> done(batch, 0);
-  bool prompt_path = true;
+  // One path for a whole call: a sequence's rows, up to its last ones, take the same kernels wherever the chunks cut it.
+  // (forward_prompt takes as long for 33 rows as for 200: 8.0 ms on the 8B shape, 2.2 ms on the 1B shape, a 128-row chunk of
+  // the one-launch forward 4.3 and 1.1 ms: it pays from two of them on.)
+  bool prompt_path = (long long)batch * end > kPrefillRows;
   for (const Model &M : c->models) prompt_path = prompt_path && M.use_prompt;
   for (;;) {
     std::vector<SeqWork> work;
     int budget = prompt_path ? c->lay.max_rows : kPrefillRows;
-    const int budget0 = budget;
     for (int b = 0; b < batch && budget > 0; ++b) {
       if (done[b] >= end) continue;
       int rows = std::min(budget, end - done[b]);
@@ -950,7 +952,7 @@ int prefill(hsd_ctx *c, int batch, int prompt_len) {
     if (work.empty()) break;
     // early exits: the target's pass fills the one cache; separate models: each fills its own
     for (int lvl = c->shared_cache ? K : 0; lvl <= K; ++lvl)
-      HSD_TRY(budget0 - budget > kPrefillRows ? forward_prompt(c, lvl, work) : forward(c, lvl, work));
+      HSD_TRY(prompt_path ? forward_prompt(c, lvl, work) : forward(c, lvl, work));
   }
   return HSD_OK;
 }

@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 # head size, query heads, KV heads, page, batch, prompt length.  Rows of a chunk = prompt - 1 per sequence.
 CASES = [
-    (128, 4, 1, 16, 1, 130),       # 129 rows: the shortest chunk of this path, one row in the second A half
+    (128, 4, 1, 16, 1, 130),       # 129 rows: the fewest of this path, one row in the second A half
     (128, 4, 1, 16, 1, 257),       # 256 rows: exactly one token tile
     (128, 4, 1, 32, 3, 150),       # several sequences in one chunk, items that end inside a tile
     (128, 8, 8, 16, 2, 300),       # no grouped heads: 128 tokens per query tile
@@ -22,7 +22,8 @@ CASES = [
     (128, 6, 2, 16, 1, 345),       # group of three: two rows of every query tile unused
     (64, 8, 4, 16, 1, 391),        # head size 64: two heads per accumulator half
     (64, 4, 2, 32, 2, 1300),       # 2598 rows: two chunks, the second starting inside a sequence
-    (128, 4, 1, 16, 1, 2433),      # 2432 rows: a full chunk and 128 rows left for the one-launch pass
+    (128, 4, 1, 16, 1, 2433),      # 2432 rows: a full chunk and one of 128 rows
+    (128, 4, 1, 16, 9, 16),        # 135 rows of nine short prompts
 ]
 
 
@@ -55,6 +56,7 @@ def test_prompt_chunks_match_oracle(hd, nq, nkv, page, batch, prompt):
 
 
 @pytest.mark.parametrize("hd,nq,nkv,batch,prompt", [
+    (128, 4, 1, 8, 300),           # 2392 rows: the last 88 of the last sequence are a chunk of their own
     (64, 8, 4, 2, 2100),           # the second sequence starts in the middle of a chunk: other items, other key ranges
     (128, 4, 1, 2, 2100)])
 def test_a_prompt_does_not_depend_on_its_place_in_the_batch(hd, nq, nkv, batch, prompt):
