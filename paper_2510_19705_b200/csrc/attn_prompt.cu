@@ -336,11 +336,9 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
 
 template <int HD>
 int launch_t(const PromptAttnArgs &a, cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    HSD_CUDA_OK(cudaFuncSetAttribute(prompt_attn_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<HD>::kSmem));
-    attr_set = true;
-  }
+  static std::atomic<u64> limits{0};
+  const int limit = hsd_smem_limit((const void *)prompt_attn_kernel<HD>, Cfg<HD>::kSmem, limits);
+  if (limit) return limit;
   prompt_attn_kernel<HD><<<a.n_items * a.nkv, kThreads, Cfg<HD>::kSmem, s>>>(a);
   hsd_count_launches(1);
   return hsd_launch_status();

@@ -346,11 +346,9 @@ template <typename T, bool VEC, int TILE>
 int launch_pairs(const T *logits, long long model_stride, int L, int R, int V, const AlphaPlan &p, const float2 *stats, float *partials, cudaStream_t s) {
   const int lpad = (L + 7) / 8 * 8;
   const size_t smem = (2 * (size_t)lpad * (TILE + 8) + 8 * 64) * sizeof(float);
-  static bool attr_set = false;
-  if (!attr_set) {
-    HSD_CUDA_OK(cudaFuncSetAttribute(alpha_pairs_kernel<T, VEC, TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
-    attr_set = true;
-  }
+  static std::atomic<u64> limits{0};
+  const int limit = hsd_smem_limit((const void *)alpha_pairs_kernel<T, VEC, TILE>, 100 * 1024, limits);
+  if (limit) return limit;
   alpha_pairs_kernel<T, VEC, TILE><<<p.n_units * R, kAlphaThreads, smem, s>>>(logits, model_stride, L, R, V, p.unit, p.n_units, stats, partials);
   return HSD_OK;
 }

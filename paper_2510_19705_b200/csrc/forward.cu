@@ -391,11 +391,9 @@ static int attention_t(const ModelDims &md, const void *q, const RowBatch &rb, c
                        const void *v_pool, float *partials, int keys_per_split, int n_splits, void *att_out, cudaStream_t s) {
   int group = md.nq / md.nkv;
   size_t smem = attn_smem_bytes(group, HD, sizeof(T));
-  static bool attr_set = false;
-  if (!attr_set) {
-    HSD_CUDA_OK(cudaFuncSetAttribute(attn_split_kernel<T, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    attr_set = true;
-  }
+  static std::atomic<u64> limits{0};
+  const int limit = hsd_smem_limit((const void *)attn_split_kernel<T, HD>, 200 * 1024, limits);
+  if (limit) return limit;
   dim3 grid(n_splits, md.nkv, rb.n_attn);
   attn_split_kernel<T, HD><<<grid, kAttnThreads, smem, s>>>((const T *)q, rb.attn, page_table, (const T *)k_pool,
                                                            (const T *)v_pool, partials, md.nq, md.nkv, md.page,

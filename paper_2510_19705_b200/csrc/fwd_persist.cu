@@ -1791,12 +1791,10 @@ __global__ void __launch_bounds__(256, 2) attn_tiles_kernel(const __grid_constan
 
 template <int HD>
 int launch_attn_tiles_t(const FwdArgs &a, __nv_bfloat16 *k_pool, __nv_bfloat16 *v_pool, int sm_count, cudaStream_t s) {
-  static bool attr_set = false;
+  static std::atomic<u64> limits{0};
   const int smem = kScratchBytes + 1024;
-  if (!attr_set) {
-    HSD_CUDA_OK(cudaFuncSetAttribute(attn_tiles_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    attr_set = true;
-  }
+  const int limit = hsd_smem_limit((const void *)attn_tiles_kernel<HD>, smem, limits);
+  if (limit) return limit;
   const int n_work = a.n_attn * a.nkv * a.n_splits;
   attn_tiles_kernel<HD><<<std::min(n_work, 2 * sm_count), 256, smem, s>>>(a, k_pool, v_pool);
   hsd_count_launches(1);
@@ -1806,11 +1804,9 @@ int launch_attn_tiles_t(const FwdArgs &a, __nv_bfloat16 *k_pool, __nv_bfloat16 *
 template <int NPAD, int HD, bool TC>
 int launch_t(const FwdArgs &args, int sm_count, cudaStream_t s) {
   using Cfg = PCfg<NPAD>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    HSD_CUDA_OK(cudaFuncSetAttribute(fwd_persistent_kernel<NPAD, HD, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
-    attr_set = true;
-  }
+  static std::atomic<u64> limits{0};
+  const int limit = hsd_smem_limit((const void *)fwd_persistent_kernel<NPAD, HD, TC>, Cfg::kSmemBytes, limits);
+  if (limit) return limit;
   void *params[1] = {const_cast<FwdArgs *>(&args)};
   HSD_CUDA_OK(cudaLaunchCooperativeKernel((const void *)fwd_persistent_kernel<NPAD, HD, TC>, dim3(sm_count), dim3(kFwdThreads), params,
                                           (size_t)Cfg::kSmemBytes, s));

@@ -296,11 +296,9 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
 
 template <int MODE, int HD>
 int launch_t(const BigGemmArgs &a, int n_tiles, int m_tiles, int sm_count, cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    HSD_CUDA_OK(cudaFuncSetAttribute(gemm_big_kernel<MODE, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-    attr_set = true;
-  }
+  static std::atomic<u64> limits{0};
+  const int limit = hsd_smem_limit((const void *)gemm_big_kernel<MODE, HD>, kSmemBytes, limits);
+  if (limit) return limit;
   const int pairs = std::min(sm_count / 2, n_tiles);
   gemm_big_kernel<MODE, HD><<<2 * pairs, kThreads, kSmemBytes, s>>>(a, n_tiles, m_tiles, a.K / kBK);
   hsd_count_launches(1);

@@ -374,11 +374,9 @@ EncodeTiledFn g_encode = nullptr;
 template <int NPAD, int MODE>
 int launch_t(const TcGemmArgs &args, int n_tiles, int S, int grid, cudaStream_t s) {
   using Cfg = TcCfg<NPAD>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    HSD_CUDA_OK(cudaFuncSetAttribute(gemm_tc_kernel<NPAD, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
-    attr_set = true;
-  }
+  static std::atomic<u64> limits{0};
+  const int limit = hsd_smem_limit((const void *)gemm_tc_kernel<NPAD, MODE>, Cfg::kSmemBytes, limits);
+  if (limit) return limit;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = Cfg::kSmemBytes; cfg.stream = s;
   cudaLaunchAttribute at[1];

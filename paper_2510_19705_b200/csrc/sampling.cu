@@ -980,11 +980,9 @@ static bool cluster_pays_draw(const ClusterPlan &pl, int dtype, int V, int n, bo
 
 template <typename T, int PER, int NT, bool DRAW>
 static int launch_cluster_t(const ClusterArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    HSD_CUDA_OK(cudaFuncSetAttribute(cluster_sample_kernel<T, PER, NT, DRAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(DRAW ? kClMaxSmem / 2 : kClMaxSmem)));
-    attr_set = true;
-  }
+  static std::atomic<u64> limits{0};
+  const int limit = hsd_smem_limit((const void *)cluster_sample_kernel<T, PER, NT, DRAW>, (int)(DRAW ? kClMaxSmem / 2 : kClMaxSmem), limits);
+  if (limit) return limit;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n * pl.C); cfg.blockDim = dim3(kClThreads); cfg.dynamicSmemBytes = pl.smem; cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -1091,11 +1089,9 @@ int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int 
     return launch_cluster<false>(a, pl, dtype, batch, s);
   }
   if (fused) {
-    static bool attr_set = false;
-    if (!attr_set) {
-      HSD_CUDA_OK(cudaFuncSetAttribute(verify_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-      attr_set = true;
-    }
+    static std::atomic<u64> limits{0};
+    const int limit = hsd_smem_limit((const void *)verify_fused_kernel, 220 * 1024, limits);
+    if (limit) return limit;
     HSD_CUDA_OK(cudaMemsetAsync(counters, 0, verify_counter_bytes(batch), s));
     FusedArgs a;
     a.p = (const __nv_bfloat16 *)p; a.q = (const __nv_bfloat16 *)q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.batch = batch;
