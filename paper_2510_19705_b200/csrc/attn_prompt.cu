@@ -12,9 +12,8 @@
 // Bound by that chain: 2304 rows of the 8B shape behind 4608 cached keys 354 us with one S buffer and 128-key tiles
 // (which put the products into the chain; sixteen softmax warps, or the tiles' exponentials in turns, changed nothing),
 // 284 us this way.
-// 320 threads: warps 0-3 / 4-7 = softmax of tile A / B, warp 8 = K / V loader (TMA: a tile per copy and column block where
-// its pages follow one another in the pool, else 16 keys of one page per copy), warp 9 = MMA issue (one lane).  Items
-// come longest first.  Every wait is bounded.
+// 320 threads: warps 0-3 / 4-7 = softmax of tile A / B, warp 8 = K / V loader (TMA: a tile per copy and column block;
+// the pages of a tile follow one another in the pool), warp 9 = MMA issue (one lane).  Items come longest first.  Every wait is bounded.
 #include <algorithm>
 #include "attn_prompt.cuh"
 #include "gemm_tc.cuh"
@@ -125,29 +124,19 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
   if (warp == kLoaderWarp) {
     // ------------------------------------------------------------------ loader
     const int *pt = a.page_table + (size_t)seq * a.pages_per_seq;
-    constexpr int kCopies = TK / 16 * C::NB;                               // per operand and tile: (16-key group, column block)
-    const int grp = lane & (TK / 16 - 1), blk = (lane / (TK / 16)) & (C::NB - 1);
-    const int last_group = (kv_len - 1) >> 4;
     bool ok = true;
     for (int j = 0; j < n && ok; ++j) {
-      const int b = j % kStages;
-      const uint32_t ph = (uint32_t)((j / kStages) & 1);
-      // a group past the last key has no page: the last group again (its scores are masked, its V rows zeroed below)
-      const int key = min(j * (TK / 16) + grp, last_group) * 16;
-      const int pg = pt[key >> a.page_shift];
-      const int row = ((kvh * a.n_pages + pg) << a.page_shift) + (key & ((1 << a.page_shift) - 1));
-      // pages that follow one another in the pool (a prompt's nearly always do) come in one copy per column block
-      const int row_first = __shfl_sync(0xFFFFFFFFu, row, 0);
-      const bool run = __all_sync(0xFFFFFFFFu, row - row_first == key - j * TK);
-      const uint32_t off = (uint32_t)(run ? lane * kBlk : blk * kBlk + grp * 2048);
-      const int copies = run ? C::NB : kCopies, x0 = (run ? lane : blk) * 64, y0 = run ? row_first : row;
+      const int b = j % kStages, key = j * TK;
+      const uint32_t ph = (uint32_t)((j / kStages) & 1), off = (uint32_t)(lane * kBlk);
+      // (rows past the last key belong to nobody: their scores are masked, their V rows zeroed below)
+      const int row = ((kvh * a.n_pages + pt[key >> a.page_shift]) << a.page_shift) + (key & ((1 << a.page_shift) - 1));
       if (lane == 0) {
         ok = mbar_wait(k_free(b), ph ^ 1u, abort_flag);
         if (ok) mbar_expect_tx(k_full(b), C::kTile);
       }
       ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
-      if (lane < copies) tma_load_2d(s0 + C::kOffK + b * C::kTile + off, run ? &a.k_run : &a.k, x0, y0, k_full(b));
+      if (lane < C::NB) tma_load_2d(s0 + C::kOffK + b * C::kTile + off, &a.k, lane * 64, row, k_full(b));
       const bool tail = (j + 1) * TK > kv_len;
       if (lane == 0) {
         ok = mbar_wait(v_free(b), ph ^ 1u, abort_flag);
@@ -155,7 +144,7 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
       }
       ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
-      if (lane < copies) tma_load_2d(s0 + C::kOffV + b * C::kTile + off, run ? &a.v_run : &a.v, x0, y0, tail ? v_land : v_full(b));
+      if (lane < C::NB) tma_load_2d(s0 + C::kOffV + b * C::kTile + off, &a.v, lane * 64, row, tail ? v_land : v_full(b));
       if (tail) {                                                    // the last tile: V rows past the last key must be finite (P is 0 there)
         if (lane == 0) ok = mbar_wait(v_land, 0u, abort_flag);
         ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
@@ -346,9 +335,12 @@ int launch_t(const PromptAttnArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-int prompt_attn_maps(CUtensorMap *maps, const void *pool, long long rows, int hd) {
-  const int st = tc_make_map(&maps[0], pool, rows, hd, kPromptBoxRows);
-  return st ? st : tc_make_map(&maps[1], pool, rows, hd, TK);
+int prompt_attn_map(CUtensorMap *map, const void *pool, long long rows, int hd) { return tc_make_map(map, pool, rows, hd, TK); }
+
+bool prompt_attn_pages(const int *pages, int n_pages, int page) {
+  for (int i = 1; i < n_pages; ++i)
+    if (i * page % TK != 0 && pages[i] != pages[i - 1] + 1) return false;
+  return true;
 }
 
 int launch_prompt_attention(const PromptAttnArgs &a, cudaStream_t s) {

@@ -6,7 +6,7 @@
 namespace hsd {
 
 struct PromptAttnArgs {
-  CUtensorMap k, v, k_run, v_run;    // one layer's pools as [nkv * n_pages * page, hd], box 16 / 64 rows x 64 columns, 128-byte swizzle
+  CUtensorMap k, v;                  // one layer's pools as [nkv * n_pages * page, hd], box 64 rows x 64 columns, 128-byte swizzle
   const __nv_bfloat16 *q;            // [R, nq, hd]
   __nv_bfloat16 *att;                // [R, nq, hd]
   const int4 *items;                 // (first packed row, tokens <= 2 * prompt_attn_tokens, sequence, position of the first)
@@ -16,10 +16,12 @@ struct PromptAttnArgs {
   int *status;                       // set non-zero if a bounded wait gave up
 };
 
-constexpr int kPromptBoxRows = 16;   // keys of one copy: pages hold a multiple of 16 tokens
 // tokens of one 128-row query tile: the heads of a KV group sit side by side in it
 inline int prompt_attn_tokens(int group) { return 128 / group; }
-int prompt_attn_maps(CUtensorMap *maps /*[2]: 16-row, 64-row boxes*/, const void *pool, long long rows, int hd);
+int prompt_attn_map(CUtensorMap *map, const void *pool, long long rows, int hd);
+// A 64-key tile is one copy: the pages within it must follow one another in the pool.  (A prompt's do: prompts are read
+// from a full free list in ascending order, a sequence's pages in one run.)
+bool prompt_attn_pages(const int *pages, int n_pages, int page);
 int launch_prompt_attention(const PromptAttnArgs &args, cudaStream_t s);
 
 }  // namespace hsd

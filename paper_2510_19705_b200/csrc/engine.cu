@@ -218,7 +218,7 @@ struct Model {
   bool use_small = false;                     // a small fp32 model: fwd_small runs its passes
   int small_grid = 1;
   bool use_prompt = false;                    // long prompts run forward_prompt
-  std::vector<CUtensorMap> kvmaps;            // [n_layers][4]: K and V pools of each layer, two box heights each, for the prompt attention
+  std::vector<CUtensorMap> kvmaps;            // [n_layers][2]: K and V pools of each layer, for the prompt attention
   CUtensorMap amaps_rows[4][16];              // the same buffers with a box of exactly 1..16 rows (persistent forward, few rows)
 };
 
@@ -701,6 +701,7 @@ int forward_prompt(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     R += rows;
     n_items += (rows + tokens2 - 1) / tokens2;
     HSD_TRY(ensure_pages(c, w.b, w.end));
+    if (!prompt_attn_pages(c->page_table_host + (size_t)w.b * md.pages_per_seq, c->n_pages_of[w.b], md.page)) return HSD_E_UNSUPPORTED;
   }
   if (R == 0) return HSD_OK;
   if (R > L.max_rows) return HSD_E_INVALID_ARG;
@@ -755,7 +756,7 @@ int forward_prompt(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     g.skip_cols = last ? nqd / 256 * 256 : 0;
     HSD_TRY(product(0, md.d, l * 7, 3, BIG_QKV, nqd, nullptr, 0));
     if (last) break;
-    pa.k = M.kvmaps[4 * l]; pa.k_run = M.kvmaps[4 * l + 1]; pa.v = M.kvmaps[4 * l + 2]; pa.v_run = M.kvmaps[4 * l + 3];
+    pa.k = M.kvmaps[2 * l]; pa.v = M.kvmaps[2 * l + 1];
     HSD_TRY(launch_prompt_attention(pa, s));
     HSD_TRY(product(1, nqd, l * 7 + 3, 1, BIG_ADD_F32, md.d, x, md.d));
     HSD_TRY(launch_rmsnorm(md, x, w[5], nullptr, R, h, s));
@@ -1042,11 +1043,11 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
                   (md.d / kTcBlockM) * 2 <= c->sm_count && md.n_layers <= 64 && (md.page & (md.page - 1)) == 0 && md.page >= 16;
   M.use_prompt = M.use_persist && prompt_path_dims(model);
   if (M.use_prompt) {
-    M.kvmaps.resize((size_t)md.n_layers * 4);
+    M.kvmaps.resize((size_t)md.n_layers * 2);
     const long long rows = (long long)md.nkv * md.n_pages * md.page;
     for (int l = 0; l < md.n_layers && !st; ++l) {
-      st = prompt_attn_maps(&M.kvmaps[4 * l], ld[l].k_pool, rows, md.hd);
-      if (!st) st = prompt_attn_maps(&M.kvmaps[4 * l + 2], ld[l].v_pool, rows, md.hd);
+      st = prompt_attn_map(&M.kvmaps[2 * l], ld[l].k_pool, rows, md.hd);
+      if (!st) st = prompt_attn_map(&M.kvmaps[2 * l + 1], ld[l].v_pool, rows, md.hd);
     }
   }
   return st;
@@ -1255,7 +1256,7 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
   // Attention on tensor memory where the model allows it (one query tile per item); the normalised rows of the chosen
   // layers then collect in the buffer of the split attention's partials, idle here, so that the head's weights are read
   // once for all of them instead of once per layer.
-  const bool tm = M.use_prompt;
+  const bool tm = M.use_prompt && prompt_attn_pages(c->page_table_host, c->n_pages_of[0], md.page);
   const int R = n_tokens, per_item = tm ? prompt_attn_tokens(md.nq / md.nkv) : kAttnRows, n_attn = (R + per_item - 1) / per_item;
   char *host, *devp;
   HSD_TRY(ring_acquire(c, &host, &devp));
@@ -1308,7 +1309,7 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
     HSD_TRY(launch_rmsnorm(md, x, w[0], nullptr, R, h, s));
     HSD_TRY(project_qkv(c, M, l, rb, h, qkv, pt, kp, vp, q));
     if (tm) {
-      pa.k = M.kvmaps[4 * l]; pa.k_run = M.kvmaps[4 * l + 1]; pa.v = M.kvmaps[4 * l + 2]; pa.v_run = M.kvmaps[4 * l + 3];
+      pa.k = M.kvmaps[2 * l]; pa.v = M.kvmaps[2 * l + 1];
       HSD_TRY(launch_prompt_attention(pa, s));
     } else {
       HSD_TRY(launch_attention(md, q, rb, pt, kp, vp, c->dev<float>(ML.partials), keys_per_split, n_splits, att, s));
