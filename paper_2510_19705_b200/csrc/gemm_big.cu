@@ -3,14 +3,18 @@
 // Bound by the tensor pipe: a 256 x 256 tile per CTA pair takes about 512 cycles per 64-wide k-block, in which each CTA
 // takes 32 KiB of operands from L2 and reads them from shared memory once (its 128 A rows and its 128 of the 256 B
 // rows); a 128 x 256 tile per single CTA would take half as much again of both.  One CTA of the pair issues the MMAs;
-// both load their own operands and signal the issuing CTA's barrier.  192 threads: warp 0 = TMA producer, warp 1 = TMEM owner and (leader) MMA issuer, warps
-// 2..5 = epilogue; six stages; two 256-column accumulators (all of tensor memory), so a tile's epilogue runs under
-// the next tile's MMAs.  Tiles are dealt round-robin with the token tile fastest: the pairs that work at the same
+// both load their own operands and signal the issuing CTA's barrier.  Warp 0 = TMA producer, warp 1 = TMEM owner and
+// (leader) MMA issuer, then the epilogue; six stages; two 256-column accumulators (all of tensor memory), so a tile's epilogue
+// runs under the next tile's MMAs.  Tiles are dealt round-robin with the token tile fastest: the pairs that work at the same
 // time share weight rows, so a weight tile comes from HBM once.  Every wait is bounded.
+// The tensor core's fp32 accumulation loses about as much as its chain is long.  Products for the fp32 residual stream cut K
+// into chains (chain_blocks): the accumulators take turns, eight epilogue warps add each chain's sum to their registers under
+// the next chain's MMAs and put the whole sum back into tensor memory for the finish (a finish straight from the 128
+// registers: 1.5 % of a prompt pass slower; reads of 16 columns instead of 32: O 90 us instead of 86).
 //
-// Measured on the 8B shape, 2304 rows: gate / up 346 us (1564 TFLOP/s, 0.96 of cuBLAS's 8192^3 rate), down 190 us, O 72 us,
-// QKV 88 us (the last three lose a part of their second round of 74 tiles).  A 1023-row prompt pass: 37.3 ms in 128-row
-// chunks of the one-launch forward, 12.9 ms this way; eight such prompts 300 -> 96 ms.
+// Measured on the 8B shape, 2304 rows: gate / up 317 us (1.7 PFLOP/s), down 199 us, O 86 us, QKV 87 us (the last three lose a
+// part of their second round of 74 tiles).  A 1023-row prompt pass: 37.3 ms in 128-row chunks of the one-launch forward, 13.0 ms
+// this way; eight such prompts 300 -> 99 ms.
 #include <algorithm>
 #include "gemm_big.cuh"
 #include "tc_ptx.cuh"
@@ -20,7 +24,6 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 192;
 constexpr int kBM = 256, kBN = 256, kBK = 64;
 constexpr int kStages = 6;
 constexpr int kABytes = 128 * kBK * 2, kBBytes = 128 * kBK * 2;      // per CTA and stage
@@ -87,9 +90,13 @@ __device__ __forceinline__ void store_bf16x16(__nv_bfloat16 *dst, const float *v
   reinterpret_cast<uint4 *>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
+// Threads: a TMA and an MMA warp, four epilogue warps, or eight where the epilogue sums chains (a thread then holds half a row).
+template <int MODE> constexpr int threads_of() { return MODE == BIG_ADD_F32 ? 320 : 192; }
+
 template <int MODE, int HD>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_tiles, int KB) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of<MODE>(), 1)
+gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_tiles, int KB, int chain) {
+  constexpr bool CHAINS = MODE == BIG_ADD_F32;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes);
@@ -108,7 +115,7 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), 8); }
+    for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), CHAINS ? 16 : 8); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -151,27 +158,92 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
     // ------------------------------------------------------------------ MMA issuer (one lane of the leader)
     if (lane == 0 && rank == 0) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-      int s = 0, ti = 0;
+      int s = 0, ci = 0;
       uint32_t ph = 0;
       bool ok = true;
-      for (int t = pair; t < n_tiles && ok; t += pairs, ++ti) {
-        const int ab = ti & 1;
-        if (!mbar_wait(acce_bar(ab), (uint32_t)((ti >> 1) & 1) ^ 1u, abort_flag)) break;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(ab * kBN);
-        for (int kb = 0; kb < KB; ++kb) {
-          if (!mbar_wait(full_bar(s), ph, abort_flag)) { ok = false; break; }
+      for (int t = pair; t < n_tiles && ok; t += pairs) {
+        for (int k0 = 0; k0 < KB && ok; k0 += chain, ++ci) {
+          const int ab = ci & 1, k1 = min(KB, k0 + chain);
+          ok = mbar_wait(acce_bar(ab), (uint32_t)((ci >> 1) & 1) ^ 1u, abort_flag);
+          if (!ok) break;
           tc_fence_after();
-          const uint32_t wa = s0 + (uint32_t)(s * kStageBytes);
-          const uint64_t da = umma_desc(wa), db = umma_desc(wa + kABytes);
+          const uint32_t d_tmem = tmem_base + (uint32_t)(ab * kBN);
+          for (int kb = k0; kb < k1; ++kb) {
+            if (!mbar_wait(full_bar(s), ph, abort_flag)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t wa = s0 + (uint32_t)(s * kStageBytes);
+            const uint64_t da = umma_desc(wa), db = umma_desc(wa + kABytes);
 #pragma unroll
-          for (int k = 0; k < kBK / 16; ++k)
-            umma_bf16_pair(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (kb > 0 || k > 0) ? 1u : 0u);
-          umma_commit_pair(empty_bar(s));
-          if (++s == kStages) { s = 0; ph ^= 1u; }
+            for (int k = 0; k < kBK / 16; ++k)
+              umma_bf16_pair(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (kb > k0 || k > 0) ? 1u : 0u);
+            umma_commit_pair(empty_bar(s));
+            if (++s == kStages) { s = 0; ph ^= 1u; }
+          }
+          if (ok) umma_commit_pair(accf_bar(ab));
         }
-        if (ok) umma_commit_pair(accf_bar(ab));
       }
+    }
+  } else if constexpr (CHAINS) {
+    // ------------------------------------------------------------------ epilogue (warps 2..9): thread = token row and half
+    // of the tile's columns
+    const int q = warp & 3, hw = (warp - 2) >> 2;                       // TMEM lane quarter, column half
+    int ci = 0;
+    bool ok = true;
+    for (int t = pair; t < n_tiles; t += pairs) {
+      uint32_t tb = 0, acce = 0;
+      float acc[128];                                                   // sum of the tile's chains so far
+#pragma unroll
+      for (int i = 0; i < 128; ++i) acc[i] = 0.f;
+      for (int k0 = 0; k0 < KB; k0 += chain, ++ci) {
+        const int ab = ci & 1;
+        if (lane == 0) ok = mbar_wait(accf_bar(ab), (uint32_t)((ci >> 1) & 1), abort_flag);
+        ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
+        if (!ok) break;
+        tc_fence_after();
+        tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * kBN + hw * 128);
+        acce = map_to_rank(acce_bar(ab), 0);
+        if (chain >= KB) continue;                                      // one chain: the finish reads it where it lies
+#pragma unroll
+        for (int c = 0; c < 128; c += 32) {
+          float v[32];
+          tmem_ld32(tb + c, v);
+          tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 32; ++e) acc[c + e] += v[e];
+        }
+        if (k0 + chain < KB) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) remote_arrive(acce);
+        } else {                                                        // the finish reads the sum where the last chain lay
+#pragma unroll
+          for (int c = 0; c < 128; c += 16) tmem_st16u(tb + c, reinterpret_cast<const unsigned *>(acc + c));
+          tmem_st_wait();
+        }
+      }
+      if (!ok) break;
+      const int mt = t % m_tiles, nt = t / m_tiles;
+      const int r = mt * kBM + (int)rank * 128 + q * 32 + lane;
+      const bool on = r < args.R;
+      float *row = args.out_f32 + (size_t)r * args.ldo + nt * kBN + hw * 128;
+#pragma unroll 1
+      for (int c = 0; c < 128; c += 32) {
+        float v[32];
+        tmem_ld32(tb + c, v);
+        float4 old[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) old[e] = on ? __ldcg(reinterpret_cast<const float4 *>(row + c) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+        tmem_ld_wait();
+        if (on) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            __stcg(reinterpret_cast<float4 *>(row + c) + e, make_float4(old[e].x + v[4 * e], old[e].y + v[4 * e + 1],
+                                                                        old[e].z + v[4 * e + 2], old[e].w + v[4 * e + 3]));
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) remote_arrive(acce);
     }
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..5): thread = token row
@@ -187,25 +259,7 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
       const int r = mt * kBM + (int)rank * 128 + q * 32 + lane;
       const bool on = r < args.R;
       const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * kBN);
-      if (MODE == BIG_ADD_F32) {
-        float *row = args.out_f32 + (size_t)r * args.ldo + nt * kBN;
-#pragma unroll 1
-        for (int c = 0; c < kBN; c += 32) {
-          float v[32];
-          tmem_ld16(tb + c, v);
-          tmem_ld16(tb + c + 16, v + 16);
-          float4 old[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) old[e] = on ? __ldcg(reinterpret_cast<const float4 *>(row + c) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-          tmem_ld_wait();
-          if (on) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-              __stcg(reinterpret_cast<float4 *>(row + c) + e, make_float4(old[e].x + v[4 * e], old[e].y + v[4 * e + 1],
-                                                                          old[e].z + v[4 * e + 2], old[e].w + v[4 * e + 3]));
-          }
-        }
-      } else if (MODE == BIG_SWIGLU) {
+      if (MODE == BIG_SWIGLU) {
         __nv_bfloat16 *row = args.out_bf16 + (size_t)r * args.ldo + nt * 128;
 #pragma unroll 1
         for (int c = 0; c < 128; c += 16) {
@@ -294,13 +348,28 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
   if (threadIdx.x == 0 && *abort_flag) atomicExch(args.status, 1);
 }
 
+// k-blocks of a chain.  Products that go to the fp32 residual stream: as many as a CTA of the one-launch forward (passes of
+// up to 128 rows) sums in a row for the same product: a quarter of K while four CTAs to a 128-row tile fit the SMs, and at
+// least kMinChain (a shorter chain is over before a tile's finish has given the other accumulator back).  Products whose result
+// is rounded to bf16 at once: all of K (4e-6 at 4096 columns against the rounding's 2e-3).  A chain's sum holds the MMAs up
+// while it is read; 2304 rows of the 8B shape in one chain / four: O 72 / 86 us, down 190 / 199; chains in QKV and gate / up
+// too: 90 / 99 and 322 / 349.
+constexpr int kMinChain = 16;
+int chain_blocks(const BigGemmArgs &a, int KB, int sm_count) {
+  if (a.mode != BIG_ADD_F32) return KB;
+  const int tiles = ceil_div(a.seg_n[0], 128);
+  const int blocks = tiles * 2 <= sm_count ? ceil_div(KB, std::min(4, sm_count / tiles))
+                                           : (int)std::min<long long>(KB, ((long long)tiles * KB + sm_count - 1) / sm_count);
+  return std::min(KB, std::max(blocks, kMinChain));
+}
+
 template <int MODE, int HD>
 int launch_t(const BigGemmArgs &a, int n_tiles, int m_tiles, int sm_count, cudaStream_t s) {
   static std::atomic<u64> limits{0};
   const int limit = hsd_smem_limit((const void *)gemm_big_kernel<MODE, HD>, kSmemBytes, limits);
   if (limit) return limit;
-  const int pairs = std::min(sm_count / 2, n_tiles);
-  gemm_big_kernel<MODE, HD><<<2 * pairs, kThreads, kSmemBytes, s>>>(a, n_tiles, m_tiles, a.K / kBK);
+  const int pairs = std::min(sm_count / 2, n_tiles), KB = a.K / kBK;
+  gemm_big_kernel<MODE, HD><<<2 * pairs, threads_of<MODE>(), kSmemBytes, s>>>(a, n_tiles, m_tiles, KB, chain_blocks(a, KB, sm_count));
   hsd_count_launches(1);
   return hsd_launch_status();
 }
