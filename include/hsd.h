@@ -148,7 +148,8 @@ typedef struct {
 } hsd_level_stats;
 
 /* Device workspace needed by hsd_create for this model / hierarchy (KV pages, token buffers,
- * per-level logits rows, activations, scratch).  0 on invalid arguments. */
+ * per-level logits rows, activations, scratch).  bf16 models on the many-row prompt path hold the activations of up to
+ * 2304 rows (or max_batch * max_seq, if that is less): about 150 MB for an 8B shape.  0 on invalid arguments. */
 size_t hsd_workspace_bytes(const hsd_model_desc *model, const int32_t *exit_layers, int n_levels, const int32_t *T);
 
 /* Build a context.  exit_layers [n_levels] ascending, last == n_layers; T [n_levels - 1], each >= 1

@@ -67,10 +67,13 @@ def _dev(t):
     return t.data_ptr()
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)       # not public: a torch without it takes the stream object
+
+
 def _stream():
     """The current device's current stream.  (The raw handle: a call's stream object, pointer objects and prototype
     set-up took longer on the host, 12 us, than its kernel on the GPU.)"""
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return _raw_stream(torch.cuda.current_device()) if _raw_stream else torch.cuda.current_stream().cuda_stream
 
 
 def hsd_draft_sample(logits, seed, call_serial, out_tokens=None):

@@ -11,7 +11,7 @@
 // are, so a tile's chain is load - maximum - exponentials - store and the products run beside it.
 // Bound by that chain: 2304 rows of the 8B shape behind 4608 cached keys 354 us with one S buffer and 128-key tiles
 // (which put the products into the chain; sixteen softmax warps, or the tiles' exponentials in turns, changed nothing),
-// 284 us this way.
+// 284 us this way with one bf16 per weight, 326 us with hi + lo.
 // 320 threads: warps 0-3 / 4-7 = softmax of tile A / B, warp 8 = K / V loader (TMA: a tile per copy and column block;
 // the pages of a tile follow one another in the pool), warp 9 = MMA issue (one lane).  Items come longest first.  Every wait is bounded.
 #include <algorithm>

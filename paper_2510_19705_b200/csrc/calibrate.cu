@@ -332,7 +332,7 @@ AlphaPlan alpha_plan(int L, int R, int V) {
   AlphaPlan p;
   // equal units of a multiple of the tile; shorter ones when the positions alone would not fill the SMs
   int n = (V + kAlphaUnit - 1) / kAlphaUnit;
-  while ((long long)n * R < 148 * 4 && (V + n - 1) / n > 2 * kAlphaTile) n *= 2;
+  while ((long long)n * R < 4 * kMeasuredSMs && (V + n - 1) / n > 2 * kAlphaTile) n *= 2;
   p.unit = ((V + n - 1) / n + kAlphaTile - 1) / kAlphaTile * kAlphaTile;
   p.n_units = (V + p.unit - 1) / p.unit;
   p.n_pairs = L * (L - 1) / 2;
@@ -365,7 +365,7 @@ int launch_alpha_t(const T *logits, long long model_stride, int L, int R, int V,
          : L <= 16 ? launch_pairs<T, VEC, 512>(logits, model_stride, L, R, V, p, stats, partials, s)
                    : launch_pairs<T, VEC, 256>(logits, model_stride, L, R, V, p, stats, partials, s);
   if (st) return st;
-  alpha_reduce_kernel<<<p.n_pairs > 0 ? min(p.n_pairs, 592) : 1, kAlphaThreads, 0, s>>>(partials, L, R * p.n_units, R, alpha);
+  alpha_reduce_kernel<<<p.n_pairs > 0 ? min(p.n_pairs, 4 * kMeasuredSMs) : 1, kAlphaThreads, 0, s>>>(partials, L, R * p.n_units, R, alpha);
   hsd_count_launches(p.n_pairs > 0 ? 3 : 2);
   return hsd_launch_status();
 }

@@ -35,6 +35,9 @@ static inline int hsd_smem_limit(const void *kernel, int bytes, std::atomic<u64>
   return HSD_OK;
 }
 
+// SMs of the GPU that measured lines (path choices, unit sizes) refer to; launches ask the device.
+constexpr int kMeasuredSMs = 148;
+
 __host__ __device__ static inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 // Stored value -> fp32 (bf16 widens exactly).

@@ -24,7 +24,7 @@ struct TcGemmPlan {
   size_t scratch_bytes;
 };
 TcGemmPlan tc_plan(const int *seg_n, int n_segs, int mode, int K, int npad, int sm_count);
-int tc_npad(int rows);             // 16, 32, 64 or 128 (rows <= 128)
+int tc_npad(int rows);             // 16, 32, 64, 128 or 256 (rows <= 256)
 
 // Where the q / k / v projection's rows go (GEMM_QKV_T): q rotated -> q; k rotated, v -> their cache pages.
 struct TcQkv {

@@ -925,14 +925,14 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
 // are too long or too many for this path.
 struct ClusterPlan { int C, NT, per, staged, seg; size_t smem; };
 constexpr size_t kClMaxSmem = 216 * 1024;
-constexpr int kClSMs = 148, kClEights = 14;       // SMs of the GPU; clusters of eight that run at once (one CTA per SM)
+constexpr int kClEights = 14;                     // clusters of eight that run at once (one CTA per SM)
 static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, int rows, bool draw, ClusterPlan *pl) {
   if (rows > kClMaxRows) return false;
   pl->per = (dtype == HSD_BF16 && V % 2 == 0 && ((uintptr_t)p & 3) == 0 && ((uintptr_t)q & 3) == 0) ? 2 : 1;
   // as many CTAs as run at once (draws: two per SM), of at least 4096 tokens (eight a thread) each: clusters of eight do not fit all SMs
   // (16 of them took two rounds), clusters of four and two do
   int C = 1;
-  while (C < kClMaxC && V > C * 4096 && 2 * C * n <= (C == 4 ? 8 * kClEights : draw ? 2 * kClSMs : kClSMs)) C *= 2;
+  while (C < kClMaxC && V > C * 4096 && 2 * C * n <= (C == 4 ? 8 * kClEights : draw ? 2 * kMeasuredSMs : kMeasuredSMs)) C *= 2;
   const int most = (draw ? 16 : 32) * kClThreads;
   while (C < kClMaxC && ceil_div(V, C) > most - 64) C *= 2;
   const int seg = ceil_div(ceil_div(V, C), 64) * 64;
@@ -963,17 +963,17 @@ static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, 
 static bool cluster_pays_verify(const ClusterPlan &pl, int dtype, int V, int batch, int rows, bool fused) {
   const long long work = (long long)pl.seg * rows;
   if (fused) {
-    const double tokens = 512.0 * pl.NT * rows, rounds = ceil_div(pl.C * batch, kClSMs);
+    const double tokens = 512.0 * pl.NT * rows, rounds = ceil_div(pl.C * batch, kMeasuredSMs);
     const double cluster_us = rounds * (7.5 + tokens * (pl.NT == 32 ? 2.7e-4 : 2.05e-4));
     const double fused_us = 17.5 + V * 2.4e-4 + (double)batch * rows * (0.0155 + V * 4e-7);
     return cluster_us * 1.15 < fused_us;
   }
-  if (pl.C * batch > 2 * kClSMs && V <= 50000) return false;
+  if (pl.C * batch > 2 * kMeasuredSMs && V <= 50000) return false;
   if (dtype == HSD_BF16) return work * 5 <= 8ll * V;
   return V > 20000 ? work <= 4ll * V : work * 5 <= 11ll * V;
 }
 static bool cluster_pays_draw(const ClusterPlan &pl, int dtype, int V, int n, bool chunked) {
-  if (pl.seg > 4096 && pl.C * n > 2 * kClSMs) return false;
+  if (pl.seg > 4096 && pl.C * n > 2 * kMeasuredSMs) return false;
   if (dtype == HSD_BF16 && chunked) return pl.seg <= 4096 || pl.C > 1;
   return V > (pl.C > 2 ? 12000 : 13000) && pl.C > 1;
 }
