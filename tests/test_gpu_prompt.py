@@ -22,6 +22,7 @@ CASES = [
     (128, 6, 2, 16, 1, 345),       # group of three: two rows of every query tile unused
     (64, 8, 4, 16, 1, 391),        # head size 64: two heads per accumulator half
     (64, 4, 2, 32, 2, 1300),       # 2598 rows: two chunks, the second starting inside a sequence
+    (64, 4, 2, 16, 1, 2600),       # head size 64 well past 2048 keys
     (128, 4, 1, 16, 1, 2433),      # 2432 rows: a full chunk and one of 128 rows
     (128, 4, 1, 16, 9, 16),        # 135 rows of nine short prompts
 ]
