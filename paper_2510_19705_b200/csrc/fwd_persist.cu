@@ -1486,7 +1486,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
   auto ready_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + 4 + b); };
   const uint32_t attn_done_bar = smem_u32(dbg_cy + 15);         // the last counter slot (laps use 0..14)
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int G = gridDim.x, c = blockIdx.x;
   const int n_phases = 4 * a.n_run + (a.L > 0 ? 1 : 0);
 
@@ -1508,122 +1508,120 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  // The three pipeline roles below are single threads: a lone thread runs ~5 cycles per dependent
-  // instruction, and with whole-tile GEMMs one SM has to sustain up to twice its fair share of the
-  // weight stream (~90 GB/s = one 16 KiB stage per 180 ns).  So they keep wrapped slot counters and
-  // parities in registers instead of dividing a stage count, ring slots are handed back in pairs (a
-  // tcgen05.commit costs the tensor pipe as much as three MMAs of this shape), and
-  // tcgen05.fence::after_thread_sync (~0.1 us while MMAs are in flight) is issued only where another
-  // thread's tcgen05 operations must come first (accumulator reuse), not after the wait on TMA data.
-  constexpr int WGS = 1;                                          // landing slots handed back together
+  // The three pipeline roles below are a warp each, of which one lane issues (elect_one).  They are bound by their own
+  // instruction chain wherever the data is there already: the ring's eight stages at the start of every phase, and
+  // phases whose CTA streams more than its share.  So they keep wrapped slot counters and parities in registers instead of
+  // dividing a stage count, and tcgen05.fence::after_thread_sync (~0.1 us while MMAs are in flight) is issued only where
+  // another thread's tcgen05 operations must come first (accumulator reuse), not after the wait on TMA data.  A role that
+  // gives up leaves its loops lane by lane: nothing inside them synchronises the warp.
   if (warp == 0) {
     // ------------------------------------------------------------ weight-tile producer (runs ahead)
-    if (lane == 0) {
-      int s = 0, n_issued = 0;
-      uint32_t par = 1;                                  // parity to wait for on the slot group's empty barrier
-      const uint64_t w_policy = l2_policy_evict_first();  // weights are read once per pass: first out of L2
-      bool ok = true;
-      for (int p = 0; p < n_phases && ok; ++p) {
-        const Gemm g = make_gemm(a, p);
-        SegIter it = seg_begin(g, G, c);
-        Seg sg;
-        // the tensor-memory attention phase uses the ring's memory: the O projection's tiles wait until it is over
-        // (one completion per layer, waited for in every layer, so the parity never is ambiguous)
-        if (TC && (p & 3) == 1 && p < 4 * a.n_run && !mbar_wait(attn_done_bar, (uint32_t)((p >> 2) & 1), abort_flag)) { ok = false; break; }
-        if (built_down(a, p)) ring_pos_sh[(p >> 2) & 15] = (unsigned)s | (par << 8) | ((unsigned)p << 16);   // where the builders' tiles go
-        while (ok && seg_next(g, it, sg)) {
-          const Tile ti = tile_of(g, sg.tile);
-          const bool second = (g.mode == MODE_SWIGLU) || (ti.row0 + kTcBoxRows < g.seg_n[ti.seg]);
-          const CUtensorMap *m0 = g.mode == MODE_SWIGLU ? g.w[0] : g.w[ti.seg];
-          const CUtensorMap *m1 = g.mode == MODE_SWIGLU ? g.w[1] : m0;
-          const int row1 = g.mode == MODE_SWIGLU ? ti.row0 : ti.row0 + kTcBoxRows;
-          const uint32_t tx = (second ? 2 : 1) * kBoxBytes;
-          for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-            if (s % WGS == 0 && !mbar_wait(empty_bar(s / WGS), par, abort_flag)) { ok = false; break; }
+    const bool issuer = elect_one();
+    int s = 0, n_issued = 0;
+    uint32_t par = 1;                                    // parity to wait for on the slot's empty barrier
+    const uint64_t w_policy = l2_policy_evict_first();   // weights are read once per pass: first out of L2
+    bool ok = true;
+    for (int p = 0; p < n_phases && ok; ++p) {
+      const Gemm g = make_gemm(a, p);
+      SegIter it = seg_begin(g, G, c);
+      Seg sg;
+      // the tensor-memory attention phase uses the ring's memory: the O projection's tiles wait until it is over
+      // (one completion per layer, waited for in every layer, so the parity never is ambiguous)
+      if (TC && (p & 3) == 1 && p < 4 * a.n_run && !mbar_wait(attn_done_bar, (uint32_t)((p >> 2) & 1), abort_flag)) { ok = false; break; }
+      if (issuer && built_down(a, p)) ring_pos_sh[(p >> 2) & 15] = (unsigned)s | (par << 8) | ((unsigned)p << 16);   // where the builders' tiles go
+      while (ok && seg_next(g, it, sg)) {
+        const Tile ti = tile_of(g, sg.tile);
+        const bool second = (g.mode == MODE_SWIGLU) || (ti.row0 + kTcBoxRows < g.seg_n[ti.seg]);
+        const CUtensorMap *m0 = g.mode == MODE_SWIGLU ? g.w[0] : g.w[ti.seg];
+        const CUtensorMap *m1 = g.mode == MODE_SWIGLU ? g.w[1] : m0;
+        const int row1 = g.mode == MODE_SWIGLU ? ti.row0 : ti.row0 + kTcBoxRows;
+        const uint32_t tx = (second ? 2 : 1) * kBoxBytes;
+        for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
+          if (!mbar_wait(empty_bar(s), par, abort_flag)) { ok = false; break; }
+          if (issuer) {
             const uint32_t dst = smem_u32(ring) + (uint32_t)(s * Cfg::kStageBytes);
             mbar_expect_tx(full_bar(s), tx);
             tma_load_2d_hint(dst, m0, kb * kTcBlockK, ti.row0, full_bar(s), w_policy);
             if (second) tma_load_2d_hint(dst + kBoxBytes, m1, kb * kTcBlockK, row1, full_bar(s), w_policy);
-            ++n_issued;
-            if (++s == STAGES) { s = 0; par ^= 1u; }
           }
+          ++n_issued;
+          if (++s == STAGES) { s = 0; par ^= 1u; }
         }
       }
-      if (!ok) {
-        atomicExch(a.status, 1);
-        // let copies in flight land (bounded): the last min(n_issued, STAGES) slots, newest first
-        uint32_t fpar = par ^ 1u;                        // full-barrier parity of the current round
-        for (int i = 0, sl = s; i < STAGES && i < n_issued; ++i) {
-          if (--sl < 0) { sl = STAGES - 1; fpar ^= 1u; }
-          unsigned long long t0 = globaltimer_ns();
-          while (!mbar_try_wait(full_bar(sl), fpar))
-            if (globaltimer_ns() - t0 > kWaitLimitNs / 4) break;
-        }
+    }
+    if (!ok && issuer) {
+      atomicExch(a.status, 1);
+      // let copies in flight land (bounded): the last min(n_issued, STAGES) slots, newest first
+      uint32_t fpar = par ^ 1u;                          // full-barrier parity of the current round
+      for (int i = 0, sl = s; i < STAGES && i < n_issued; ++i) {
+        if (--sl < 0) { sl = STAGES - 1; fpar ^= 1u; }
+        unsigned long long t0 = globaltimer_ns();
+        while (!mbar_try_wait(full_bar(sl), fpar))
+          if (globaltimer_ns() - t0 > kWaitLimitNs / 4) break;
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ activation-tile producer
-    if (lane == 0) {
-      int s = 0;
-      uint32_t par = 1;
-      bool ok = true;
-      const uint32_t a_bytes = (uint32_t)a.a_box_rows * kTcBlockK * 2;
-      for (int p = 0; p < n_phases && ok; ++p) {
-        const Gemm g = make_gemm(a, p);
-        SegIter it = seg_begin(g, G, c);
-        Seg sg;
-        bool have = seg_next(g, it, sg);
-        // the operand of phase p is complete once the workers have passed the barrier before it
-        if (!mbar_wait(ready_bar(p & 1), (uint32_t)((p >> 1) & 1), abort_flag)) { ok = false; break; }
-        const bool built = built_down(a, p);
-        while (ok && have) {
-          for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-            if (s % WGS == 0 && !mbar_wait(empty_bar(s / WGS), par, abort_flag)) { ok = false; break; }
-            const uint32_t dst = smem_u32(ring) + (uint32_t)(s * Cfg::kStageBytes) + kWBytes;
-            if (!built) {                                // built down projection: the workers fill the tile and arrive
-              mbar_expect_tx(full_bar(s), a_bytes);
-              tma_load_2d(dst, g.amap, kb * kTcBlockK, 0, full_bar(s));
-            }
-            if (++s == STAGES) { s = 0; par ^= 1u; }
+    const bool issuer = elect_one();
+    int s = 0;
+    uint32_t par = 1;
+    bool ok = true;
+    const uint32_t a_bytes = (uint32_t)a.a_box_rows * kTcBlockK * 2;
+    for (int p = 0; p < n_phases && ok; ++p) {
+      const Gemm g = make_gemm(a, p);
+      SegIter it = seg_begin(g, G, c);
+      Seg sg;
+      bool have = seg_next(g, it, sg);
+      // the operand of phase p is complete once the workers have passed the barrier before it
+      if (!mbar_wait(ready_bar(p & 1), (uint32_t)((p >> 1) & 1), abort_flag)) { ok = false; break; }
+      const bool built = built_down(a, p);
+      while (ok && have) {
+        for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
+          if (!mbar_wait(empty_bar(s), par, abort_flag)) { ok = false; break; }
+          if (issuer && !built) {                        // built down projection: the workers fill the tile and arrive
+            mbar_expect_tx(full_bar(s), a_bytes);
+            tma_load_2d(smem_u32(ring) + (uint32_t)(s * Cfg::kStageBytes) + kWBytes, g.amap, kb * kTcBlockK, 0, full_bar(s));
           }
-          have = seg_next(g, it, sg);
+          if (++s == STAGES) { s = 0; par ^= 1u; }
         }
+        have = seg_next(g, it, sg);
       }
-      if (!ok) atomicExch(a.status, 1);
     }
+    if (!ok && issuer) atomicExch(a.status, 1);
   } else if (warp == 2) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(NPAD);
-      const uint64_t da0 = umma_desc(smem_u32(ring));
-      int s = 0, seg_idx = 0;
-      uint32_t par = 0;
-      bool ok = true;
-      for (int p = 0; p < n_phases && ok; ++p) {
-        const Gemm g = make_gemm(a, p);
-        SegIter it = seg_begin(g, G, c);
-        Seg sg;
-        for (; ok && seg_next(g, it, sg); ++seg_idx) {
-          const int ab = seg_idx & 1;
-          if (!mbar_wait(acce_bar(ab), (uint32_t)(((seg_idx >> 1) & 1) ^ 1), abort_flag)) { ok = false; break; }
-          tc_fence_after();                              // the epilogue's tcgen05.ld of this accumulator come first
-          const uint32_t d_tmem = tmem_base + (uint32_t)(ab * NPAD);
-          uint32_t acc = 0u;
-          for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-            if (!mbar_wait(full_bar(s), par, abort_flag)) { ok = false; break; }
-            const uint64_t da = da0 + (uint64_t)(s * (Cfg::kStageBytes >> 4)), db = da + (uint64_t)(kWBytes >> 4);
+    const bool issuer = elect_one();
+    const uint32_t idesc = umma_idesc_bf16(NPAD);
+    const uint64_t da0 = umma_desc(smem_u32(ring));
+    int s = 0, seg_idx = 0;
+    uint32_t par = 0;
+    bool ok = true;
+    for (int p = 0; p < n_phases && ok; ++p) {
+      const Gemm g = make_gemm(a, p);
+      SegIter it = seg_begin(g, G, c);
+      Seg sg;
+      for (; ok && seg_next(g, it, sg); ++seg_idx) {
+        const int ab = seg_idx & 1;
+        if (!mbar_wait(acce_bar(ab), (uint32_t)(((seg_idx >> 1) & 1) ^ 1), abort_flag)) { ok = false; break; }
+        tc_fence_after();                                // the epilogue's tcgen05.ld of this accumulator come first
+        const uint32_t d_tmem = tmem_base + (uint32_t)(ab * NPAD);
+        uint32_t acc = 0u;
+        for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
+          if (!mbar_wait(full_bar(s), par, abort_flag)) { ok = false; break; }
+          const uint64_t da = da0 + (uint64_t)(s * (Cfg::kStageBytes >> 4)), db = da + (uint64_t)(kWBytes >> 4);
+          if (issuer) {
             umma_bf16(d_tmem, da, db, idesc, acc);
 #pragma unroll
             for (int k = 1; k < kTcBlockK / 16; ++k) umma_bf16(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, 1u);
-            acc = 1u;
-            if (s % WGS == WGS - 1) umma_commit(empty_bar(s / WGS));
-            if (++s == STAGES) { s = 0; par ^= 1u; }
+            umma_commit(empty_bar(s));
           }
-          if (ok) umma_commit(accf_bar(ab));
+          acc = 1u;
+          if (++s == STAGES) { s = 0; par ^= 1u; }
         }
+        if (ok && issuer) umma_commit(accf_bar(ab));
       }
-      if (!ok) atomicExch(a.status, 1);
     }
+    if (!ok && issuer) atomicExch(a.status, 1);
   } else if (warp >= 4) {
     // ------------------------------------------------------------ workers (+ epilogue: warps 4..7)
     const int wt = threadIdx.x - 128;              // 0..255
