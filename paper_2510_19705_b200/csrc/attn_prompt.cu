@@ -13,7 +13,7 @@
 // (which put the products into the chain; sixteen softmax warps, or the tiles' exponentials in turns, changed nothing),
 // 284 us this way with one bf16 per weight, 326 us with hi + lo.
 // 320 threads: warps 0-3 / 4-7 = softmax of tile A / B, warp 8 = K / V loader (TMA: a tile per copy and column block;
-// the pages of a tile follow one another in the pool), warp 9 = MMA issue (one lane).  Items come longest first.  Every wait is bounded.
+// the pages of a tile follow one another in the pool), warp 9 = MMA issue (one elected lane).  Items come longest first.  Every wait is bounded.
 #include <algorithm>
 #include "attn_prompt.cuh"
 #include "gemm_tc.cuh"
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
   auto pv_done = [&](int x) { return b0 + 8u * (24 + x); };
   auto o_done = [&](int x) { return b0 + 8u * (26 + x); };           // the last P V (a barrier of its own: the parity wait tells neighbours apart only)
   const uint32_t v_land = b0 + 8u * 28;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int kvh = blockIdx.x % a.nkv;
   const int4 it = a.items[blockIdx.x / a.nkv];
   const int row0 = it.x, ntok = it.y, seq = it.z, pos0 = it.w;
@@ -124,31 +124,29 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
   if (warp == kLoaderWarp) {
     // ------------------------------------------------------------------ loader
     const int *pt = a.page_table + (size_t)seq * a.pages_per_seq;
+    const bool issuer = elect_one();
     bool ok = true;
-    for (int j = 0; j < n && ok; ++j) {
+    auto wait = [&](uint32_t bar, uint32_t parity) { ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag)); return ok; };
+    for (int j = 0; j < n; ++j) {
       const int b = j % kStages, key = j * TK;
-      const uint32_t ph = (uint32_t)((j / kStages) & 1), off = (uint32_t)(lane * kBlk);
+      const uint32_t ph = (uint32_t)((j / kStages) & 1);
       // (rows past the last key belong to nobody: their scores are masked, their V rows zeroed below)
       const int row = ((kvh * a.n_pages + pt[key >> a.page_shift]) << a.page_shift) + (key & ((1 << a.page_shift) - 1));
-      if (lane == 0) {
-        ok = mbar_wait(k_free(b), ph ^ 1u, abort_flag);
-        if (ok) mbar_expect_tx(k_full(b), C::kTile);
+      if (!wait(k_free(b), ph ^ 1u)) break;
+      if (issuer) {
+        mbar_expect_tx(k_full(b), C::kTile);
+#pragma unroll
+        for (int i = 0; i < C::NB; ++i) tma_load_2d(s0 + C::kOffK + b * C::kTile + i * kBlk, &a.k, i * 64, row, k_full(b));
       }
-      ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
-      if (!ok) break;
-      if (lane < C::NB) tma_load_2d(s0 + C::kOffK + b * C::kTile + off, &a.k, lane * 64, row, k_full(b));
       const bool tail = (j + 1) * TK > kv_len;
-      if (lane == 0) {
-        ok = mbar_wait(v_free(b), ph ^ 1u, abort_flag);
-        if (ok) mbar_expect_tx(tail ? v_land : v_full(b), C::kTile);
+      if (!wait(v_free(b), ph ^ 1u)) break;
+      if (issuer) {
+        mbar_expect_tx(tail ? v_land : v_full(b), C::kTile);
+#pragma unroll
+        for (int i = 0; i < C::NB; ++i) tma_load_2d(s0 + C::kOffV + b * C::kTile + i * kBlk, &a.v, i * 64, row, tail ? v_land : v_full(b));
       }
-      ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
-      if (!ok) break;
-      if (lane < C::NB) tma_load_2d(s0 + C::kOffV + b * C::kTile + off, &a.v, lane * 64, row, tail ? v_land : v_full(b));
       if (tail) {                                                    // the last tile: V rows past the last key must be finite (P is 0 there)
-        if (lane == 0) ok = mbar_wait(v_land, 0u, abort_flag);
-        ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
-        if (!ok) break;
+        if (!wait(v_land, 0u)) break;
         const int r0 = kv_len - j * TK;
         for (int i = r0 * 8 * C::NB + lane; i < TK * 8 * C::NB; i += 32) {
           const int r = i / (8 * C::NB), c = i % (8 * C::NB);        // whole rows: the swizzle permutes within a row
@@ -156,7 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive(v_full(b));
+        if (issuer) mbar_arrive(v_full(b));
       }
     }
     if (!ok) {                                                       // copies in flight land before the shared memory goes away
@@ -165,36 +163,39 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
     }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------------ MMA issue
-    if (lane == 0) {
-      const uint32_t id1 = umma_idesc_bf16(TK), id2 = umma_idesc_bf16(HD) | (1u << 16);      // bit 16: B is MN-major
-      auto issue_s = [&](int x, int j) {
-        const uint32_t qb = desc_lo_k(s0 + x * C::kQTile), kb = desc_lo_k(s0 + C::kOffK + (j % kStages) * C::kTile), d = tS(x) + (uint32_t)((j & 1) * TK);
+    const bool issuer = elect_one();
+    const uint32_t id1 = umma_idesc_bf16(TK), id2 = umma_idesc_bf16(HD) | (1u << 16);      // bit 16: B is MN-major
+    auto issue_s = [&](int x, int j) {                               // (the issuer only)
+      const uint32_t qb = desc_lo_k(s0 + x * C::kQTile), kb = desc_lo_k(s0 + C::kOffK + (j % kStages) * C::kTile), d = tS(x) + (uint32_t)((j & 1) * TK);
 #pragma unroll
-        for (int ks = 0; ks < HD / 16; ++ks)
-          umma_ss(d, qb + (ks >> 2) * (kQBlk / 16) + (ks & 3) * 2, kb + (ks >> 2) * (kBlk / 16) + (ks & 3) * 2, id1, ks > 0 ? 1u : 0u);
-        umma_commit(s_full(x, j & 1));
-      };
-      auto k_wait = [&](int j) { return mbar_wait(k_full(j % kStages), (uint32_t)((j / kStages) & 1), abort_flag); };
-      bool ok = true;
-      for (int j = 0; j < min(2, n) && ok; ++j) {                    // the first two key tiles' scores
-        ok = k_wait(j);
-        if (!ok) break;
-        tc_fence_after();
+      for (int ks = 0; ks < HD / 16; ++ks)
+        umma_ss(d, qb + (ks >> 2) * (kQBlk / 16) + (ks & 3) * 2, kb + (ks >> 2) * (kBlk / 16) + (ks & 3) * 2, id1, ks > 0 ? 1u : 0u);
+      umma_commit(s_full(x, j & 1));
+    };
+    auto k_wait = [&](int j) { return mbar_wait(k_full(j % kStages), (uint32_t)((j / kStages) & 1), abort_flag); };
+    bool ok = true;
+    for (int j = 0; j < min(2, n) && ok; ++j) {                      // the first two key tiles' scores
+      ok = k_wait(j);
+      if (!ok) break;
+      tc_fence_after();
+      if (issuer) {
         if (j < nA) issue_s(0, j);
         if (j < nB) issue_s(1, j);
         umma_commit(k_free(j % kStages));
       }
-      for (int j = 0; j < n && ok; ++j) {
-        const uint32_t vb = desc_lo_mn(s0 + C::kOffV + (j % kStages) * C::kTile);
-        ok = mbar_wait(v_full(j % kStages), (uint32_t)((j / kStages) & 1), abort_flag);
-        if (ok && j + 2 < n) ok = k_wait(j + 2);
-        for (int x = 0; x < 2 && ok; ++x) {
-          const int nx = x ? nB : nA;
-          if (j >= nx) continue;
-          ok = mbar_wait(p_ready(x, j & 1), (uint32_t)((j >> 1) & 1), abort_flag);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t d = tO(x), p = tS(x) + (uint32_t)((j & 1) * TK);
+    }
+    for (int j = 0; j < n && ok; ++j) {
+      const uint32_t vb = desc_lo_mn(s0 + C::kOffV + (j % kStages) * C::kTile);
+      ok = mbar_wait(v_full(j % kStages), (uint32_t)((j / kStages) & 1), abort_flag);
+      if (ok && j + 2 < n) ok = k_wait(j + 2);
+      for (int x = 0; x < 2 && ok; ++x) {
+        const int nx = x ? nB : nA;
+        if (j >= nx) continue;
+        ok = mbar_wait(p_ready(x, j & 1), (uint32_t)((j >> 1) & 1), abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d = tO(x), p = tS(x) + (uint32_t)((j & 1) * TK);
+        if (issuer) {
 #pragma unroll
           for (int ks = 0; ks < TK / 16; ++ks) umma_ts(d, p + ks * 16, vb + ks * 128, id2, ks > 0 ? 1u : (j > 0 ? 1u : 0u));
 #pragma unroll
@@ -203,10 +204,10 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
           if (j + 2 < nx) issue_s(x, j + 2);                         // over P(j), after the products that read it
           if (j + 1 == nx) umma_commit(o_done(x));
         }
-        if (ok) {
-          umma_commit(v_free(j % kStages));
-          if (j + 2 < n) umma_commit(k_free((j + 2) % kStages));
-        }
+      }
+      if (ok && issuer) {
+        umma_commit(v_free(j % kStages));
+        if (j + 2 < n) umma_commit(k_free((j + 2) % kStages));
       }
     }
   } else {

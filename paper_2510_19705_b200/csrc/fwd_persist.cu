@@ -384,7 +384,7 @@ __device__ __forceinline__ void ldmatrix_x4_trans(unsigned *r, const void *row_p
 // the GEMM accumulators are idle during this phase).  Rows 32..127 of the A operands are whatever shared memory
 // follows the real rows: their results are never read.  The eight worker warps: per stream (warps 0-3 / 4-7) warp
 // 0 = softmax (the only one whose TMEM lane quarter holds real rows), warp 1 = K tiles (three buffers: a K buffer
-// is free as soon as S is complete), warp 2 = V tiles (two buffers), warp 3 = MMA issue (one lane).  Shared memory:
+// is free as soon as S is complete), warp 2 = V tiles (two buffers), warp 3 = MMA issue (one elected lane).  Shared memory:
 // the weight ring and the attention scratch together (the weight producer does not run ahead over this phase).
 constexpr int kTcaTile = 64, kTcaKBufs = 3, kTcaVBufs = 2;
 constexpr int kTcaTileBytes = 2 * kTcaTile * 128;                 // two 64-column blocks of [64 keys][128 B]
@@ -428,7 +428,7 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
   auto v_full = [&](int s, int b) { return b0 + 8u * (s * 12 + 6 + b); };
   auto v_free = [&](int s, int b) { return b0 + 8u * (s * 12 + 8 + b); };
   auto p_ready = [&](int s, int b) { return b0 + 8u * (s * 12 + 10 + b); };
-  const int warp = wt >> 5, lane = wt & 31, s = warp >> 2, role = warp & 3;
+  const int warp = __shfl_sync(0xFFFFFFFFu, wt >> 5, 0), lane = wt & 31, s = warp >> 2, role = warp & 3;
 #ifdef HSD_PROFILE
   // profiling build: CTA 0's first softmax warp laps its set-up [5], waits for S [6], softmax up to P ready [7] and the
   // item's end [8]; [9] counts the items
@@ -528,13 +528,14 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
   } else if (role == 3) {
-    // ---------------- MMA issue for stream s (one lane)
-    if (lane == 0) {
-      const uint32_t id1 = umma_idesc_bf16(TK), id2 = umma_idesc_bf16(HD) | (1u << 16);     // bit 16: B is MN-major
-      auto issue_s = [&](int t) {                                 // S[t & 1] = Q K_t^T
-        const int b = t % NKB;
-        ok = mbar_wait(k_full(s, b), (uint32_t)((t / NKB) & 1), abort_flag);
-        if (!ok) return;
+    // ---------------- MMA issue for stream s
+    const bool issuer = elect_one();
+    const uint32_t id1 = umma_idesc_bf16(TK), id2 = umma_idesc_bf16(HD) | (1u << 16);       // bit 16: B is MN-major
+    auto issue_s = [&](int t) {                                   // S[t & 1] = Q K_t^T
+      const int b = t % NKB;
+      ok = mbar_wait(k_full(s, b), (uint32_t)((t / NKB) & 1), abort_flag);
+      if (!ok) return;
+      if (issuer) {
 #pragma unroll
         for (int ks = 0; ks < HD / 16; ++ks) {
           const uint64_t da = umma_desc(s0 + (ks >> 2) * 4096 + (ks & 3) * 32);
@@ -542,17 +543,19 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
           umma_bf16(tS + (uint32_t)((t & 1) * 64), da, db, id1, ks > 0 ? 1u : 0u);
         }
         umma_commit(k_free(s, b));                                // S(t) complete = the K buffer is free
-      };
-      if (n_mine > 0) issue_s(0);
-      if (n_mine > 1 && ok) issue_s(1);
-      for (int t = 0; t < n_mine && ok; ++t) {
-        // P(t) is written (so S(t) has been read as well) and V(t) has landed
-        ok = mbar_wait(p_ready(s, t & 1), (uint32_t)((t >> 1) & 1), abort_flag);
-        if (!ok) break;
-        const int vb = t % NVB;
-        ok = mbar_wait(v_full(s, vb), (uint32_t)((t / NVB) & 1), abort_flag);
-        if (!ok) break;
-        tc_fence_after();
+      }
+    };
+    if (n_mine > 0) issue_s(0);
+    if (n_mine > 1 && ok) issue_s(1);
+    for (int t = 0; t < n_mine && ok; ++t) {
+      // P(t) is written (so S(t) has been read as well) and V(t) has landed
+      ok = mbar_wait(p_ready(s, t & 1), (uint32_t)((t >> 1) & 1), abort_flag);
+      if (!ok) break;
+      const int vb = t % NVB;
+      ok = mbar_wait(v_full(s, vb), (uint32_t)((t / NVB) & 1), abort_flag);
+      if (!ok) break;
+      tc_fence_after();
+      if (issuer) {
         const uint32_t p_off = kTcaOffP + (s * 2 + (t & 1)) * 4096;
 #pragma unroll
         for (int ks = 0; ks < TK / 16; ++ks) {
@@ -561,8 +564,8 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
           umma_bf16(tO, da, db, id2, (t > 0 || ks > 0) ? 1u : 0u);
         }
         umma_commit(v_free(s, vb));
-        if (t + 2 < n_mine) issue_s(t + 2);                       // its S buffer (t & 1) was read before P(t) was written
       }
+      if (t + 2 < n_mine) issue_s(t + 2);                         // its S buffer (t & 1) was read before P(t) was written
     }
   } else {
     // ---------------- stream s: softmax (thread = query vector `lane`)

@@ -109,7 +109,7 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
   auto empty_bar = [&](int s) { return bar0 + 8u * (kStages + s); };
   auto accf_bar = [&](int b) { return bar0 + 8u * (2 * kStages + b); };
   auto acce_bar = [&](int b) { return bar0 + 8u * (2 * kStages + 2 + b); };
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
 
@@ -130,34 +130,37 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer (one lane per CTA)
-    if (lane == 0) {
-      int s = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int t = pair; t < n_tiles && ok; t += pairs) {
-        const int mt = t % m_tiles, nt = t / m_tiles;
-        const Half hf = half_of<MODE>(args, nt, (int)rank);
-        const int arow = mt * kBM + (int)rank * 128;
-        for (int kb = 0; kb < KB; ++kb) {
-          if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
+    // ------------------------------------------------------------------ TMA producer (one lane of each CTA issues)
+    const bool issuer = elect_one();
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int t = pair; t < n_tiles && ok; t += pairs) {
+      const int mt = t % m_tiles, nt = t / m_tiles;
+      const Half hf = half_of<MODE>(args, nt, (int)rank);
+      const int arow = mt * kBM + (int)rank * 128;
+      for (int kb = 0; kb < KB; ++kb) {
+        if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
+        if (issuer) {
           const uint32_t dst = s0 + (uint32_t)(s * kStageBytes), bar = map_to_rank(full_bar(s), 0);
           if (rank == 0) mbar_expect_tx(full_bar(s), 2 * kStageBytes);
           tma_load_2d_pair(dst, &args.a, kb * kBK, arow, bar);
           tma_load_2d_pair(dst + kABytes, &args.w[hf.seg], kb * kBK, hf.n0, bar);
           tma_load_2d_pair(dst + kABytes + kBBytes / 2, &args.w[hf.seg], kb * kBK, hf.n0 + 64, bar);
-          if (++s == kStages) { s = 0; ph ^= 1u; }
         }
-      }
-      if (!ok) {                                     // copies still in flight must land before the shared memory goes away
-        const unsigned long long t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 200000ull) {}
+        if (++s == kStages) { s = 0; ph ^= 1u; }
       }
     }
+    if (!ok) {                                       // copies still in flight must land before the shared memory goes away
+      const unsigned long long t0 = globaltimer_ns();
+      while (globaltimer_ns() - t0 < 200000ull) {}
+    }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer (one lane of the leader)
-    if (lane == 0 && rank == 0) {
+    // ------------------------------------------------------------------ MMA issuer (one lane of the leader issues)
+    if (rank == 0) {
+      const bool issuer = elect_one();
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+      const uint64_t da0 = umma_desc(s0);
       int s = 0, ci = 0;
       uint32_t ph = 0;
       bool ok = true;
@@ -168,18 +171,21 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
           if (!ok) break;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + (uint32_t)(ab * kBN);
+          uint32_t acc = 0u;
           for (int kb = k0; kb < k1; ++kb) {
             if (!mbar_wait(full_bar(s), ph, abort_flag)) { ok = false; break; }
             tc_fence_after();
-            const uint32_t wa = s0 + (uint32_t)(s * kStageBytes);
-            const uint64_t da = umma_desc(wa), db = umma_desc(wa + kABytes);
+            const uint64_t da = da0 + (uint64_t)(s * (kStageBytes >> 4)), db = da + (uint64_t)(kABytes >> 4);
+            if (issuer) {
+              umma_bf16_pair(d_tmem, da, db, idesc, acc);
 #pragma unroll
-            for (int k = 0; k < kBK / 16; ++k)
-              umma_bf16_pair(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (kb > k0 || k > 0) ? 1u : 0u);
-            umma_commit_pair(empty_bar(s));
+              for (int k = 1; k < kBK / 16; ++k) umma_bf16_pair(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, 1u);
+              umma_commit_pair(empty_bar(s));
+            }
+            acc = 1u;
             if (++s == kStages) { s = 0; ph ^= 1u; }
           }
-          if (ok) umma_commit_pair(accf_bar(ab));
+          if (ok && issuer) umma_commit_pair(accf_bar(ab));
         }
       }
     }

@@ -7,7 +7,7 @@
 // A stream-K split over all SMs with pieces in global memory took 29.5 us for 14336 x 4096 at 24 rows (117 MB); whole tiles of 104 rows
 // on 138 CTAs take 25.6 us; 4096 x 4096 at 256 rows 49 -> 20 us.
 //
-// 192 threads: warp 0 = TMA producer (one lane), warp 1 = TMEM owner + MMA issuer (one lane), warps 2..5 = epilogue
+// 192 threads: warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer (one elected lane issues), warps 2..5 = epilogue
 // (each reads its own 32-lane quarter of TMEM).  Shared-memory ring of (128 x 64 weight tile + NPAD x 64 activation
 // tile), both K-major with the 128-byte swizzle TMA writes and the UMMA descriptors read.  A CTA's k-blocks are summed in
 // two halves with a TMEM accumulator each, added in fp32 at the end: the tensor core's fp32 accumulation loses about as
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
   auto accf_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + b); };
   auto acce_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + 2 + b); };
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   // S > 1: the cluster's CTAs share tile blockIdx.x / S; S = 1: tiles blockIdx.x, + gridDim.x, ...
   const int rank = S > 1 ? (int)cluster_rank() : 0;
   const int tile0 = S > 1 ? (int)blockIdx.x / S : (int)blockIdx.x, step = S > 1 ? n_tiles : (int)gridDim.x;
@@ -185,21 +185,22 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      const uint64_t policy = l2_policy_evict_first();
-      int s = 0, issued = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      const uint32_t box_bytes = (uint32_t)args.w_box_rows * kTcBlockK * 2;
-      for (int tile = tile0; tile < n_tiles && ok; tile += step) {
-        const TileInfo ti = tile_info(args, tile);
-        const bool second = MODE == GEMM_SWIGLU_T || (args.w_box_rows < args.tile_rows && ti.row0 + args.w_box_rows < args.seg_n[ti.seg]);
-        const CUtensorMap *w0 = &args.w[ti.seg], *w1 = MODE == GEMM_SWIGLU_T ? &args.w[1] : w0;
-        const int row1 = MODE == GEMM_SWIGLU_T ? ti.row0 : ti.row0 + args.w_box_rows;
-        const uint32_t bytes = (second ? 2 : 1) * box_bytes + (uint32_t)args.a_box_rows * kTcBlockK * 2;
-        for (int kb = kb0; kb < kb1; ++kb, ++issued) {
-          if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
-          const uint32_t dst = smem_u32(ring + (size_t)s * Cfg::kStageBytes);
+    const bool issuer = elect_one();
+    const uint64_t policy = l2_policy_evict_first();
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    const uint32_t box_bytes = (uint32_t)args.w_box_rows * kTcBlockK * 2;
+    for (int tile = tile0; tile < n_tiles && ok; tile += step) {
+      const TileInfo ti = tile_info(args, tile);
+      const bool second = MODE == GEMM_SWIGLU_T || (args.w_box_rows < args.tile_rows && ti.row0 + args.w_box_rows < args.seg_n[ti.seg]);
+      const CUtensorMap *w0 = &args.w[ti.seg], *w1 = MODE == GEMM_SWIGLU_T ? &args.w[1] : w0;
+      const int row1 = MODE == GEMM_SWIGLU_T ? ti.row0 : ti.row0 + args.w_box_rows;
+      const uint32_t bytes = (second ? 2 : 1) * box_bytes + (uint32_t)args.a_box_rows * kTcBlockK * 2;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
+        if (issuer) {
+          const uint32_t dst = smem_u32(ring) + (uint32_t)(s * Cfg::kStageBytes);
           mbar_expect_tx(full_bar(s), bytes);
           if (args.stream_weights) {
             tma_load_2d_hint(dst, w0, kb * kTcBlockK, ti.row0, full_bar(s), policy);
@@ -209,47 +210,47 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             if (second) tma_load_2d(dst + box_bytes, w1, kb * kTcBlockK, row1, full_bar(s));
           }
           tma_load_2d(dst + kStageWBytes, &args.a, kb * kTcBlockK, args.row0, full_bar(s));
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
-      if (!ok) {                                   // copies in flight land before the shared memory goes away
-        const unsigned long long t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 200000ull) {}
-      }
+    }
+    if (!ok) {                                   // copies in flight land before the shared memory goes away
+      const unsigned long long t0 = globaltimer_ns();
+      while (globaltimer_ns() - t0 < 200000ull) {}
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(NPAD);
-      int s = 0, ti = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int tile = tile0; tile < n_tiles && ok; tile += step, ++ti) {
-        const int ab = ti % Cfg::kBufs;
-        if (!mbar_wait(acce_bar(ab), (uint32_t)((ti / Cfg::kBufs) & 1) ^ 1u, abort_flag)) break;
-        tc_fence_after();
-        uint32_t d_tmem = tmem_base + (uint32_t)(ab * 2 * NPAD), acc = 0u;
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(full_bar(s), ph, abort_flag)) { ok = false; break; }
-          const uint32_t wa = smem_u32(ring + (size_t)s * Cfg::kStageBytes);
-          const uint64_t da = umma_desc(wa), db = umma_desc(wa + kStageWBytes);
-          if (kb == kb_half) {
-            if (Cfg::kFold) {
-              if (!mbar_wait(acce_bar(1), (uint32_t)(ti & 1) ^ 1u, abort_flag)) { ok = false; break; }
-              tc_fence_after();
-            }
-            d_tmem += NPAD; acc = 0u;
+    const bool issuer = elect_one();
+    const uint32_t idesc = umma_idesc_bf16(NPAD);
+    const uint64_t da0 = umma_desc(smem_u32(ring));
+    int s = 0, ti = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int tile = tile0; tile < n_tiles && ok; tile += step, ++ti) {
+      const int ab = ti % Cfg::kBufs;
+      if (!mbar_wait(acce_bar(ab), (uint32_t)((ti / Cfg::kBufs) & 1) ^ 1u, abort_flag)) break;
+      tc_fence_after();
+      uint32_t d_tmem = tmem_base + (uint32_t)(ab * 2 * NPAD), acc = 0u;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait(full_bar(s), ph, abort_flag)) { ok = false; break; }
+        if (kb == kb_half) {
+          if (Cfg::kFold) {
+            if (!mbar_wait(acce_bar(1), (uint32_t)(ti & 1) ^ 1u, abort_flag)) { ok = false; break; }
+            tc_fence_after();
           }
-#pragma unroll
-          for (int k = 0; k < kTcBlockK / 16; ++k) {
-            umma_bf16(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, acc);
-            acc = 1u;
-          }
-          umma_commit(empty_bar(s));            // the stage is free once these MMAs have read it
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
+          d_tmem += NPAD; acc = 0u;
         }
-        if (ok) umma_commit(accf_bar(ab));      // accumulator complete
+        const uint64_t da = da0 + (uint64_t)(s * (Cfg::kStageBytes >> 4)), db = da + (uint64_t)(kStageWBytes >> 4);
+        if (issuer) {
+          umma_bf16(d_tmem, da, db, idesc, acc);
+#pragma unroll
+          for (int k = 1; k < kTcBlockK / 16; ++k) umma_bf16(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, 1u);
+          umma_commit(empty_bar(s));            // the stage is free once these MMAs have read it
+        }
+        acc = 1u;
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
+      if (ok && issuer) umma_commit(accf_bar(ab));      // accumulator complete
     }
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..5)
