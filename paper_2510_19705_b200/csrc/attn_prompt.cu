@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
     const int *pt = a.page_table + (size_t)seq * a.pages_per_seq;
     const bool issuer = elect_one();
     bool ok = true;
-    auto wait = [&](uint32_t bar, uint32_t parity) { ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag)); return ok; };
+    auto wait = [&](uint32_t bar, uint32_t parity) { ok = mbar_wait_warp(bar, parity, abort_flag); return ok; };
     for (int j = 0; j < n; ++j) {
       const int b = j % kStages, key = j * TK;
       const uint32_t ph = (uint32_t)((j / kStages) & 1);
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
         umma_ss(d, qb + (ks >> 2) * (kQBlk / 16) + (ks & 3) * 2, kb + (ks >> 2) * (kBlk / 16) + (ks & 3) * 2, id1, ks > 0 ? 1u : 0u);
       umma_commit(s_full(x, j & 1));
     };
-    auto k_wait = [&](int j) { return mbar_wait(k_full(j % kStages), (uint32_t)((j / kStages) & 1), abort_flag); };
+    auto k_wait = [&](int j) { return mbar_wait_warp(k_full(j % kStages), (uint32_t)((j / kStages) & 1), abort_flag); };
     bool ok = true;
     for (int j = 0; j < min(2, n) && ok; ++j) {                      // the first two key tiles' scores
       ok = k_wait(j);
@@ -186,12 +186,12 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
     }
     for (int j = 0; j < n && ok; ++j) {
       const uint32_t vb = desc_lo_mn(s0 + C::kOffV + (j % kStages) * C::kTile);
-      ok = mbar_wait(v_full(j % kStages), (uint32_t)((j / kStages) & 1), abort_flag);
+      ok = mbar_wait_warp(v_full(j % kStages), (uint32_t)((j / kStages) & 1), abort_flag);
       if (ok && j + 2 < n) ok = k_wait(j + 2);
       for (int x = 0; x < 2 && ok; ++x) {
         const int nx = x ? nB : nA;
         if (j >= nx) continue;
-        ok = mbar_wait(p_ready(x, j & 1), (uint32_t)((j >> 1) & 1), abort_flag);
+        ok = mbar_wait_warp(p_ready(x, j & 1), (uint32_t)((j >> 1) & 1), abort_flag);
         if (!ok) break;
         tc_fence_after();
         const uint32_t d = tO(x), p = tS(x) + (uint32_t)((j & 1) * TK);

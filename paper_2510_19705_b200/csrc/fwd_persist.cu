@@ -533,7 +533,7 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
     const uint32_t id1 = umma_idesc_bf16(TK), id2 = umma_idesc_bf16(HD) | (1u << 16);       // bit 16: B is MN-major
     auto issue_s = [&](int t) {                                   // S[t & 1] = Q K_t^T
       const int b = t % NKB;
-      ok = mbar_wait(k_full(s, b), (uint32_t)((t / NKB) & 1), abort_flag);
+      ok = mbar_wait_warp(k_full(s, b), (uint32_t)((t / NKB) & 1), abort_flag);
       if (!ok) return;
       if (issuer) {
 #pragma unroll
@@ -549,10 +549,10 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
     if (n_mine > 1 && ok) issue_s(1);
     for (int t = 0; t < n_mine && ok; ++t) {
       // P(t) is written (so S(t) has been read as well) and V(t) has landed
-      ok = mbar_wait(p_ready(s, t & 1), (uint32_t)((t >> 1) & 1), abort_flag);
+      ok = mbar_wait_warp(p_ready(s, t & 1), (uint32_t)((t >> 1) & 1), abort_flag);
       if (!ok) break;
       const int vb = t % NVB;
-      ok = mbar_wait(v_full(s, vb), (uint32_t)((t / NVB) & 1), abort_flag);
+      ok = mbar_wait_warp(v_full(s, vb), (uint32_t)((t / NVB) & 1), abort_flag);
       if (!ok) break;
       tc_fence_after();
       if (issuer) {
@@ -1515,8 +1515,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
   // instruction chain wherever the data is there already: the ring's eight stages at the start of every phase, and
   // phases whose CTA streams more than its share.  So they keep wrapped slot counters and parities in registers instead of
   // dividing a stage count, and tcgen05.fence::after_thread_sync (~0.1 us while MMAs are in flight) is issued only where
-  // another thread's tcgen05 operations must come first (accumulator reuse), not after the wait on TMA data.  A role that
-  // gives up leaves its loops lane by lane: nothing inside them synchronises the warp.
+  // another thread's tcgen05 operations must come first (accumulator reuse), not after the wait on TMA data.
   if (warp == 0) {
     // ------------------------------------------------------------ weight-tile producer (runs ahead)
     const bool issuer = elect_one();
@@ -1530,7 +1529,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
       Seg sg;
       // the tensor-memory attention phase uses the ring's memory: the O projection's tiles wait until it is over
       // (one completion per layer, waited for in every layer, so the parity never is ambiguous)
-      if (TC && (p & 3) == 1 && p < 4 * a.n_run && !mbar_wait(attn_done_bar, (uint32_t)((p >> 2) & 1), abort_flag)) { ok = false; break; }
+      if (TC && (p & 3) == 1 && p < 4 * a.n_run && !mbar_wait_warp(attn_done_bar, (uint32_t)((p >> 2) & 1), abort_flag)) { ok = false; break; }
       if (issuer && built_down(a, p)) ring_pos_sh[(p >> 2) & 15] = (unsigned)s | (par << 8) | ((unsigned)p << 16);   // where the builders' tiles go
       while (ok && seg_next(g, it, sg)) {
         const Tile ti = tile_of(g, sg.tile);
@@ -1540,7 +1539,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
         const int row1 = g.mode == MODE_SWIGLU ? ti.row0 : ti.row0 + kTcBoxRows;
         const uint32_t tx = (second ? 2 : 1) * kBoxBytes;
         for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-          if (!mbar_wait(empty_bar(s), par, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(empty_bar(s), par, abort_flag)) { ok = false; break; }
           if (issuer) {
             const uint32_t dst = smem_u32(ring) + (uint32_t)(s * Cfg::kStageBytes);
             mbar_expect_tx(full_bar(s), tx);
@@ -1576,11 +1575,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
       Seg sg;
       bool have = seg_next(g, it, sg);
       // the operand of phase p is complete once the workers have passed the barrier before it
-      if (!mbar_wait(ready_bar(p & 1), (uint32_t)((p >> 1) & 1), abort_flag)) { ok = false; break; }
+      if (!mbar_wait_warp(ready_bar(p & 1), (uint32_t)((p >> 1) & 1), abort_flag)) { ok = false; break; }
       const bool built = built_down(a, p);
       while (ok && have) {
         for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-          if (!mbar_wait(empty_bar(s), par, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(empty_bar(s), par, abort_flag)) { ok = false; break; }
           if (issuer && !built) {                        // built down projection: the workers fill the tile and arrive
             mbar_expect_tx(full_bar(s), a_bytes);
             tma_load_2d(smem_u32(ring) + (uint32_t)(s * Cfg::kStageBytes) + kWBytes, g.amap, kb * kTcBlockK, 0, full_bar(s));
@@ -1605,12 +1604,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
       Seg sg;
       for (; ok && seg_next(g, it, sg); ++seg_idx) {
         const int ab = seg_idx & 1;
-        if (!mbar_wait(acce_bar(ab), (uint32_t)(((seg_idx >> 1) & 1) ^ 1), abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(acce_bar(ab), (uint32_t)(((seg_idx >> 1) & 1) ^ 1), abort_flag)) { ok = false; break; }
         tc_fence_after();                                // the epilogue's tcgen05.ld of this accumulator come first
         const uint32_t d_tmem = tmem_base + (uint32_t)(ab * NPAD);
         uint32_t acc = 0u;
         for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-          if (!mbar_wait(full_bar(s), par, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(full_bar(s), par, abort_flag)) { ok = false; break; }
           const uint64_t da = da0 + (uint64_t)(s * (Cfg::kStageBytes >> 4)), db = da + (uint64_t)(kWBytes >> 4);
           if (issuer) {
             umma_bf16(d_tmem, da, db, idesc, acc);

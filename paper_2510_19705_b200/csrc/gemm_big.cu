@@ -140,7 +140,7 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
       const Half hf = half_of<MODE>(args, nt, (int)rank);
       const int arow = mt * kBM + (int)rank * 128;
       for (int kb = 0; kb < KB; ++kb) {
-        if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
         if (issuer) {
           const uint32_t dst = s0 + (uint32_t)(s * kStageBytes), bar = map_to_rank(full_bar(s), 0);
           if (rank == 0) mbar_expect_tx(full_bar(s), 2 * kStageBytes);
@@ -167,13 +167,13 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
       for (int t = pair; t < n_tiles && ok; t += pairs) {
         for (int k0 = 0; k0 < KB && ok; k0 += chain, ++ci) {
           const int ab = ci & 1, k1 = min(KB, k0 + chain);
-          ok = mbar_wait(acce_bar(ab), (uint32_t)((ci >> 1) & 1) ^ 1u, abort_flag);
+          ok = mbar_wait_warp(acce_bar(ab), (uint32_t)((ci >> 1) & 1) ^ 1u, abort_flag);
           if (!ok) break;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + (uint32_t)(ab * kBN);
           uint32_t acc = 0u;
           for (int kb = k0; kb < k1; ++kb) {
-            if (!mbar_wait(full_bar(s), ph, abort_flag)) { ok = false; break; }
+            if (!mbar_wait_warp(full_bar(s), ph, abort_flag)) { ok = false; break; }
             tc_fence_after();
             const uint64_t da = da0 + (uint64_t)(s * (kStageBytes >> 4)), db = da + (uint64_t)(kABytes >> 4);
             if (issuer) {

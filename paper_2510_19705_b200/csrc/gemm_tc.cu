@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       const int row1 = MODE == GEMM_SWIGLU_T ? ti.row0 : ti.row0 + args.w_box_rows;
       const uint32_t bytes = (second ? 2 : 1) * box_bytes + (uint32_t)args.a_box_rows * kTcBlockK * 2;
       for (int kb = kb0; kb < kb1; ++kb) {
-        if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
         if (issuer) {
           const uint32_t dst = smem_u32(ring) + (uint32_t)(s * Cfg::kStageBytes);
           mbar_expect_tx(full_bar(s), bytes);
@@ -228,14 +228,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     bool ok = true;
     for (int tile = tile0; tile < n_tiles && ok; tile += step, ++ti) {
       const int ab = ti % Cfg::kBufs;
-      if (!mbar_wait(acce_bar(ab), (uint32_t)((ti / Cfg::kBufs) & 1) ^ 1u, abort_flag)) break;
+      if (!mbar_wait_warp(acce_bar(ab), (uint32_t)((ti / Cfg::kBufs) & 1) ^ 1u, abort_flag)) break;
       tc_fence_after();
       uint32_t d_tmem = tmem_base + (uint32_t)(ab * 2 * NPAD), acc = 0u;
       for (int kb = kb0; kb < kb1; ++kb) {
-        if (!mbar_wait(full_bar(s), ph, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(full_bar(s), ph, abort_flag)) { ok = false; break; }
         if (kb == kb_half) {
           if (Cfg::kFold) {
-            if (!mbar_wait(acce_bar(1), (uint32_t)(ti & 1) ^ 1u, abort_flag)) { ok = false; break; }
+            if (!mbar_wait_warp(acce_bar(1), (uint32_t)(ti & 1) ^ 1u, abort_flag)) { ok = false; break; }
             tc_fence_after();
           }
           d_tmem += NPAD; acc = 0u;

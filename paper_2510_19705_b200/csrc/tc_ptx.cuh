@@ -49,12 +49,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // Pipeline roles (TMA producers, MMA issuers) run with their whole warp: every lane waits, and the lane that elect_one()
 // names issues.  Control flow and descriptors are then uniform over the warp, so the operands of tcgen05 / TMA
 // instructions live in uniform registers; in a branch of one lane they are moved there again for every instruction.
-// Resident operands, M = 128, N = 16, K = 64 with its wait and commit, cycles: one lane 509, whole warp 185 (the four
+// Resident operands, M = 128, N = 16, K = 64 with its wait and commit, cycles: one lane 509, whole warp 217 (the four
 // MMAs alone: 156).  warp_index() is the warp's number as a uniform value.
+// mbar_wait_warp() lets no lane go on before all have seen the phase: a lane that lagged behind the issuing one could
+// otherwise look at a barrier when its parity has come round again, and wait for a phase that is over.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
   return p != 0;
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+  return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag)) != 0;
 }
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0); }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
