@@ -178,8 +178,8 @@ int hsd_create_models(const hsd_model_desc *models, int n_levels, const int32_t 
 
 /* Decode passes of bf16 models fold two finish phases of the verification forward (Algorithm 2's multi-row pass)
  * into their consumers: the q / k / v finish into the attention phase, the gate / up finish into the down
- * projection; and the RMSNorm after each residual projection starts, on CTAs that hold no tile of that
- * projection, as soon as its partial sums are stored instead of after a grid-wide barrier.  fold_qkv = 0 /
+ * projection; and the RMSNorm after each residual projection starts as soon as its partial sums are there instead
+ * of after a grid-wide barrier.  fold_qkv = 0 /
  * fold_gate_up = 0 / early_norm = 0 keeps the separate phase or the barrier; the results are the same sums in
  * the same order either way (a test hook and a tuning knob; all on by default).  Errors: INVALID_ARG. */
 int hsd_set_phase_folding(hsd_ctx *ctx, int fold_qkv, int fold_gate_up, int early_norm);

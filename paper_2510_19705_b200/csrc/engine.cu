@@ -33,7 +33,7 @@ constexpr int kPromptRows = 2304;              // rows of one prompt chunk on th
                                                //   which with 4096-wide outputs make 1.95 rounds of the 74 CTA pairs (eight make 1.73)
 constexpr uint32_t kTraceMagic = 0x48534454u;
 
-constexpr size_t kTcCtrlBytes = 16384 + 256;    // status word (first 256 bytes) + per-tile counters
+constexpr size_t kTcCtrlBytes = 256;            // the status word
 constexpr int kHeadMaps = 17;                   // output-head tensor maps: one per level (<= 16), then the shared head
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -51,7 +51,7 @@ size_t elem_size(int dtype) { return dtype == HSD_BF16 ? 2 : 4; }
 // page table, per-level logits rows, decision scratch, descriptor ring).
 struct ModelLayout {
   size_t cos_tab, sin_tab, k_pool, v_pool, pool_layer_stride, x, h, qkv, q, att, act, partials, hf, tc_scratch,
-      tc_pieces_bytes, tc_pieces2, wmaps_dev, layers_dev, small_layers, attn_counters, prof;
+      tc_pieces_bytes, wmaps_dev, layers_dev, small_layers, prof;
   int partial_rows;
 };
 struct Layout {
@@ -167,28 +167,12 @@ Layout make_layout(const hsd_model_desc *models, int n_models, int n_levels, con
     M.act = take((size_t)L.max_rows * m->d_ff * es);
     M.partials = take((size_t)M.partial_rows * nq * (hd + 2) * 4);
     M.hf = take((size_t)L.max_logit_rows * d * es);
-    // tensor-core GEMM scratch: [status word | per-tile counters (16 KiB)] + split pieces (largest plan)
-    M.tc_pieces_bytes = 0;
-    if (m->dtype == HSD_BF16) {
-      const int sms = device_sm_count();
-      const int npads[5] = {16, 32, 64, 128, 256};
-      const int shapes[5][4] = {{nq * hd, nkv * hd, nkv * hd, d}, {d, 0, 0, nq * hd}, {m->d_ff, m->d_ff, 0, d},
-                                {d, 0, 0, m->d_ff}, {m->vocab, 0, 0, d}};
-      const int modes[5] = {GEMM_STORE_F32, GEMM_ADD_F32, GEMM_SWIGLU_T, GEMM_ADD_F32, GEMM_STORE_T_SCATTER};
-      for (int g = 0; g < 5; ++g)
-        for (int np : npads) {
-          if (shapes[g][3] % kTcBlockK) continue;
-          int nsegs = shapes[g][2] ? 3 : (shapes[g][1] ? 2 : 1);
-          TcGemmPlan pl = tc_plan(shapes[g], nsegs, modes[g], shapes[g][3], np, sms);
-          M.tc_pieces_bytes = std::max(M.tc_pieces_bytes, pl.scratch_bytes);
-        }
-    }
+    // tensor-core scratch: [status word (256 bytes) | split pieces of the one-launch forward]
+    M.tc_pieces_bytes = m->dtype == HSD_BF16 ? fwd_pieces_bytes(d, nq * hd, nkv * hd, m->d_ff, m->vocab, device_sm_count()) : 0;
     M.tc_scratch = take(kTcCtrlBytes + M.tc_pieces_bytes);
-    M.tc_pieces2 = take(M.tc_pieces_bytes);       // second piece buffer (down projection of passes with few rows)
     M.wmaps_dev = take(((size_t)m->n_layers * 7 + kHeadMaps) * sizeof(CUtensorMap));
     M.layers_dev = take((size_t)m->n_layers * sizeof(FwdLayerDev));
     M.small_layers = take(m->dtype == HSD_F32 ? (size_t)m->n_layers * sizeof(SmallLayerDev) : 0);
-    M.attn_counters = take(16384);
     M.prof = take((size_t)device_sm_count() * kFwdProfEvents * 8);
   }
   L.total = off;
@@ -548,6 +532,7 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     a.pages_per_seq = md.pages_per_seq; a.n_pages = md.n_pages; a.eps = md.eps;
     a.wmaps = c->dev<CUtensorMap>(ML.wmaps_dev);
     a.layers = c->dev<FwdLayerDev>(ML.layers_dev);
+    a.k_pool = c->ws + ML.k_pool; a.v_pool = c->ws + ML.v_pool; a.pool_stride = ML.pool_layer_stride;
     a.embed = (const __nv_bfloat16 *)M.embed; a.final_norm = (const __nv_bfloat16 *)c->level_norm[level];
     a.cos_tab = c->dev<float>(ML.cos_tab); a.sin_tab = c->dev<float>(ML.sin_tab);
     a.R = R; a.L = n_logit; a.n_attn = n_attn; a.attn_rows = arows; a.n_splits = n_splits; a.keys_per_split = keys_per_split;
@@ -557,8 +542,8 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     a.h = c->dev<__nv_bfloat16>(ML.h); a.q = c->dev<__nv_bfloat16>(ML.q); a.att = c->dev<__nv_bfloat16>(ML.att);
     a.act = c->dev<__nv_bfloat16>(ML.act); a.hf = c->dev<__nv_bfloat16>(ML.hf);
     a.logits = (__nv_bfloat16 *)(c->ws + L.logits[level]);
-    a.attn_partials = c->dev<float>(ML.partials); a.attn_counters = c->dev<int>(ML.attn_counters);
-    a.pieces = (float *)(c->ws + ML.tc_scratch + kTcCtrlBytes); a.tile_counters = (int *)(c->ws + ML.tc_scratch + 256);
+    a.attn_partials = c->dev<float>(ML.partials);
+    a.pieces[0] = (float *)(c->ws + ML.tc_scratch + kTcCtrlBytes); a.pieces_bytes = ML.tc_pieces_bytes;
     a.grid_counter = c->dev<unsigned>(L.grid_counter); a.status = (int *)(c->ws + c->status_off);
     const int np = tc_npad(std::max(R, n_logit));
     const int pi = np == 16 ? 0 : np == 32 ? 1 : np == 64 ? 2 : 3;
@@ -570,12 +555,11 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     a.fuse_qkv = (one_item_per_seq && !c->no_fuse_qkv) ? 1 : 0;
     // few rows: the SwiGLU finish folds into the down projection (its CTAs build their activation tiles)
     a.fuse_gu = (R <= 4 && !c->no_fuse_gu) ? 1 : 0;
-    // the norms after the residual projections start on otherwise idle CTAs as soon as the pieces are there
+    // the norms after the residual projections start as soon as the pieces are there
     a.early_norm = c->no_early_norm ? 0 : 1;
     // long key ranges: attention work items on tcgen05 / tensor memory (they take their q / k / v from the finish phase)
     a.tc_attn = (tc_capable && keys_per_split >= kTcAttnMinKeys) ? 1 : 0;
     if (a.tc_attn) a.fuse_qkv = 0;
-    a.pieces2 = (float *)(c->ws + ML.tc_pieces2);
     for (int b = 0; b < 4; ++b) a.amap[b] = box_rows <= 16 ? M.amaps_rows[b][box_rows - 1] : M.amaps[b][pi];
     a.prof = nullptr;
 #ifdef HSD_PROFILE
@@ -1037,7 +1021,8 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
   }
   if (cudaMemcpy(c->ws + ml.wmaps_dev, M.wmaps.data(), M.wmaps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(c->ws + ml.layers_dev, ld.data(), ld.size() * sizeof(FwdLayerDev), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemset(c->ws + ml.attn_counters, 0, 16384) != cudaSuccess)
+      cudaMemset(c->ws + ml.tc_scratch + kTcCtrlBytes, 0xFF, ml.tc_pieces_bytes) != cudaSuccess ||
+      cudaMemset(c->ws + ml.partials, 0xFF, (size_t)ml.partial_rows * md.nq * (md.hd + 2) * 4) != cudaSuccess)
     return HSD_E_CUDA;
   M.use_persist = coop_launch_supported() && fwd_persist_supported(md.hd, md.nq / md.nkv) && md.d % 256 == 0 && md.d <= 4096 &&
                   (md.d / kTcBlockM) * 2 <= c->sm_count && md.n_layers <= 64 && (md.page & (md.page - 1)) == 0 && md.page >= 16;
@@ -1232,8 +1217,8 @@ int hsd_generate(hsd_ctx *c, const int32_t *prompt_ids, int batch, int prompt_le
 // Logits of chosen exit layers at every position of one token sequence: the input of the calibration of
 // Section 4.2 (acceptance rates between all candidate drafters).  One pass over the layers with the
 // one-kernel-per-op path; after each chosen layer the shared final norm and output head are applied to all rows.
-int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const int32_t *layers, int n_layers_sel,
-                     void *out_logits, void *stream) {
+static int layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const int32_t *layers, int n_layers_sel, void *out_logits,
+                        void *stream, size_t *partials_used) {
   if (!c || !token_ids || !layers || !out_logits || n_tokens < 1 || n_layers_sel < 1) return HSD_E_INVALID_ARG;
   Model &M = c->models.back();                  // the target's decoder
   const ModelDims &md = M.md;
@@ -1291,6 +1276,8 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
   char *rows_buf = c->dev<char>(ML.partials);
   const size_t row_bytes = (size_t)md.d * es, rows_cap = (size_t)ML.partial_rows * md.nq * (md.hd + 2) * 4 / row_bytes;
   const int layers_cap = tm ? (int)std::min<size_t>(rows_cap / R, (size_t)n_layers_sel) : 0;     // layers whose rows fit the buffer
+  if (M.use_persist)
+    *partials_used = layers_cap ? (size_t)layers_cap * R * row_bytes : (tm ? 0 : (size_t)R * n_splits * md.nq * (md.hd + 2) * 4);
   int held = 0, next = 0;                                 // layers in the buffer; layers normalised so far
   auto flush = [&]() -> int {                             // logits of the layers held: next - held ..
     void *out = (char *)out_logits + (size_t)(next - held) * R * md.V * es;
@@ -1337,7 +1324,15 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
                  (char *)out_logits + (size_t)next * R * md.V * es, rb.lrow_dst));
     ++next;
   }
-  return sync_stream(c);
+  return HSD_OK;
+}
+
+int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const int32_t *layers, int n_layers_sel,
+                     void *out_logits, void *stream) {
+  size_t used = 0;                              // bytes of the partials buffer written: the one-launch forward finds it filled with 0xFF
+  int st = layer_logits(c, token_ids, n_tokens, layers, n_layers_sel, out_logits, stream, &used);
+  if (used && cudaMemsetAsync(c->ws + c->models.back().lay.partials, 0xFF, used, c->stream) != cudaSuccess && !st) st = HSD_E_CUDA;
+  return st ? st : sync_stream(c);
 }
 
 int hsd_set_exit_heads(hsd_ctx *c, const void *const *final_norms, const void *const *lm_heads) {

@@ -5,7 +5,8 @@
 // phase workers, 8..11 = phase workers only.  The 256 worker threads walk the phase program
 //   embed+norm | QKV(+rope, KV append) | attention | O(+residual) | norm | gate/up(+SwiGLU) |
 //   down(+residual) | norm | ... | final norm | output head
-// with a grid barrier between phases.  The weight producer is not tied to the barriers: weights are
+// with a grid barrier before each projection that takes its activations by TMA; the other phases wait for the words they
+// read (kHole).  The weight producer is not tied to the barriers: weights are
 // read-only, so it runs ahead into the next GEMM as far as the ring allows; the activation producer
 // waits for the barrier that completes its operand.  GEMM work is split evenly over the CTAs in
 // (tile, k-block) units; each segment's partial sums go to a piece buffer and the following phase
@@ -14,6 +15,7 @@
 // q / k / v of its own rows, and with at most four rows the down projection's CTAs build their
 // activation tiles from the gate / up pieces in shared memory (warps 5, 7, 9, 11).
 // Every wait (mbarrier, grid barrier) is bounded by wall time and raises a status word.
+#include <type_traits>
 #include "fwd_persist.cuh"
 #include "forward.cuh"
 #include "gemm_tc.cuh"
@@ -113,62 +115,138 @@ __device__ __forceinline__ int unit_owner(int U, int G, int u) {
 // fixed piece order (bit-reproducible; no CTA waits for another inside a GEMM).
 struct Seg { int tile, kb0, kb1; };
 struct SegIter { int tile, kb, left; };        // next k-block (tile, kb) and the k-blocks still to hand out
-// regular: every tile is cut into `parts` equal k-ranges (GEMMs with few tiles: at most 4 pieces per
-// tile, so the consumer can fetch all of them in one batch); otherwise the (tile, k-block) units are
+// regular: every tile is cut into `parts` equal k-ranges (GEMMs with few tiles: at most four pieces per
+// tile, residual projections residual_parts(), so the consumer can fetch all of them in one batch); otherwise the (tile, k-block) units are
 // dealt out evenly (tiles >= CTAs / 2: a tile then spans at most 3 CTAs).
 struct SplitGeom { int U, Gp, pieces_max, parts; };
-__device__ __forceinline__ SplitGeom split_geom(const Gemm &g, int G) {
+// The norm after a residual projection loads a row's pieces in one batch: four of up to 4096 columns.
+__host__ __device__ __forceinline__ int residual_parts(int) { return 4; }
+__host__ __device__ __forceinline__ SplitGeom split_geom(int n_tiles, int KB, int most, int G) {
   SplitGeom sg;
-  sg.U = g.n_tiles * g.KB;
-  if (g.n_tiles * 2 <= G) {
-    sg.parts = min(min(4, G / g.n_tiles), g.KB);
-    sg.Gp = g.n_tiles * sg.parts;
+  sg.U = n_tiles * KB;
+  if (n_tiles * 2 <= G) {
+    const int fit = G / n_tiles < KB ? G / n_tiles : KB;
+    sg.parts = most < fit ? most : fit;
+    sg.Gp = n_tiles * sg.parts;
     sg.pieces_max = sg.parts;
   } else {
     sg.parts = 0;
-    sg.Gp = min(G, sg.U);
+    sg.Gp = G < sg.U ? G : sg.U;
     const int per = sg.U / sg.Gp;
-    sg.pieces_max = (g.KB + per - 1) / per + 1;
+    sg.pieces_max = (KB + per - 1) / per + 1;
   }
   return sg;
 }
-// The divisions happen once, here; seg_next only counts (the pipeline roles call it on their critical path).
-__device__ __forceinline__ SegIter seg_begin(const Gemm &g, int G, int c) {
+__device__ __forceinline__ SplitGeom split_geom(const Gemm &g, int G) {
+  return split_geom(g.n_tiles, g.KB, g.mode == MODE_ADD ? residual_parts(g.seg_n[0]) : 4, G);
+}
+// What one CTA has to do in one kind of projection (0 QKV, 1 O, 2 gate / up, 3 down, 4 head): the same in every layer, so
+// it is worked out once per launch and kept in shared memory (an integer division is ~100 cycles between a phase's barrier
+// and its first load).  piece0: the CTA's piece of its first segment's tile; tiles it starts itself: piece 0.
+struct PhaseGeom { int tile, kb, left, piece0, KB, pieces_max, parts, U, Gp; };
+__device__ __forceinline__ int kind_of(const FwdArgs &a, int p) { return p < 4 * a.n_run ? p & 3 : 4; }
+__device__ __forceinline__ SegIter seg_begin(const PhaseGeom &pg) {
   SegIter it;
-  const SplitGeom sg = split_geom(g, G);
-  it.tile = 0; it.kb = 0; it.left = 0;
-  if (c < sg.Gp) {
-    if (sg.parts) {
-      const int tile = c / sg.parts, part = c - tile * sg.parts;
-      it.tile = tile;
-      it.kb = cta_begin(g.KB, sg.parts, part);
-      it.left = cta_begin(g.KB, sg.parts, part + 1) - it.kb;
-    } else {
-      const int cur = cta_begin(sg.U, sg.Gp, c);
-      it.left = cta_begin(sg.U, sg.Gp, c + 1) - cur;
-      it.tile = cur / g.KB;
-      it.kb = cur - it.tile * g.KB;
-    }
-  }
+  it.tile = pg.tile; it.kb = pg.kb; it.left = pg.left;
   return it;
 }
-__device__ __forceinline__ bool seg_next(const Gemm &g, SegIter &it, Seg &s) {
+__device__ __forceinline__ bool seg_next(const PhaseGeom &pg, SegIter &it, Seg &s) {
   if (it.left <= 0) return false;
-  const int n = min(g.KB - it.kb, it.left);
+  const int n = min(pg.KB - it.kb, it.left);
   s.tile = it.tile; s.kb0 = it.kb; s.kb1 = it.kb + n;
   it.left -= n; it.kb = 0; ++it.tile;
   return true;
 }
-// Pieces of a tile: they belong to consecutive CTAs first_owner .. first_owner + n - 1.
-__device__ __forceinline__ void tile_pieces(const Gemm &g, const SplitGeom &geo, int tile, int &first_owner, int &n) {
-  if (geo.parts) { first_owner = tile * geo.parts; n = geo.parts; return; }
-  first_owner = unit_owner(geo.U, geo.Gp, tile * g.KB);
-  n = unit_owner(geo.U, geo.Gp, tile * g.KB + g.KB - 1) - first_owner + 1;
+__device__ __forceinline__ int piece_of(const PhaseGeom &pg, const Seg &s) { return s.kb0 > 0 ? pg.piece0 : 0; }
+// Pieces of a tile: they belong to consecutive CTAs.
+__device__ __forceinline__ int tile_pieces(const PhaseGeom &pg, int tile) {
+  if (pg.parts) return pg.parts;
+  return unit_owner(pg.U, pg.Gp, tile * pg.KB + pg.KB - 1) - unit_owner(pg.U, pg.Gp, tile * pg.KB) + 1;
 }
-// Phase p is a down projection whose activation tiles are built in place from the gate / up pieces: its own
-// pieces then go to the second buffer (the first is still being read by slower CTAs).
+__device__ __forceinline__ PhaseGeom phase_geom(const Gemm &g, int G, int c) {
+  const SplitGeom sg = split_geom(g, G);
+  PhaseGeom pg;
+  pg.KB = g.KB; pg.pieces_max = sg.pieces_max; pg.parts = sg.parts; pg.U = sg.U; pg.Gp = sg.Gp;
+  pg.tile = pg.kb = pg.left = pg.piece0 = 0;
+  if (c < sg.Gp) {
+    if (sg.parts) {
+      pg.tile = c / sg.parts; pg.piece0 = c - pg.tile * sg.parts;
+      pg.kb = cta_begin(g.KB, sg.parts, pg.piece0);
+      pg.left = cta_begin(g.KB, sg.parts, pg.piece0 + 1) - pg.kb;
+    } else {
+      const int cur = cta_begin(sg.U, sg.Gp, c);
+      pg.left = cta_begin(sg.U, sg.Gp, c + 1) - cur;
+      pg.tile = cur / g.KB;
+      pg.kb = cur - pg.tile * g.KB;
+      pg.piece0 = c - unit_owner(sg.U, sg.Gp, pg.tile * g.KB);
+    }
+  }
+  return pg;
+}
+// Phase p is a down projection whose activation tiles are built in place from the gate / up pieces.
 __device__ __forceinline__ bool built_down(const FwdArgs &a, int p) { return a.fuse_gu && (p & 3) == 3 && p < 4 * a.n_run; }
-__device__ __forceinline__ float *pieces_of(const FwdArgs &a, int p) { return built_down(a, p) ? a.pieces2 : a.pieces; }
+
+// Handing partial sums to the next phase.  A word of the piece and partial buffers that has not been written holds
+// kHole (a NaN no sum is stored as), and its reader takes it as soon as it holds something else: the data is its own flag.  A counter
+// or barrier in between costs a release that waits until every store of the CTA is in L2 (1 to 1.8 us under the weight
+// stream), the flag's way, and then the loads; polling the data costs the loads.  Words are accessed with relaxed
+// single-word semantics and depend on no order among themselves.  The words' writer makes them holes again one phase and
+// at least one grid barrier after their readers (put_holes), and at least one grid barrier before the next ones, so
+// between launches all words are holes.
+constexpr unsigned kHole = 0xFFFFFFFFu;
+__device__ __forceinline__ void put_word(float *p, float v) {
+  const unsigned w = __float_as_uint(v) == kHole ? 0x7FFFFFFFu : __float_as_uint(v);
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(w) : "memory");
+}
+__device__ __forceinline__ void put_hole(float *p) { asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(kHole) : "memory"); }
+__device__ __forceinline__ void put_holes2(float *p) { asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1, %1};" ::"l"(p), "r"(kHole) : "memory"); }
+__device__ __forceinline__ void put_words2(float *p, float x, float y) {
+  const unsigned wx = __float_as_uint(x) == kHole ? 0x7FFFFFFFu : __float_as_uint(x), wy = __float_as_uint(y) == kHole ? 0x7FFFFFFFu : __float_as_uint(y);
+  asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1, %2};" ::"l"(p), "r"(wx), "r"(wy) : "memory");
+}
+__device__ __forceinline__ float get_word(const float *p) {
+  unsigned w;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(p) : "memory");
+  return __uint_as_float(w);
+}
+__device__ __forceinline__ float2 get_words2(const float *p) {
+  unsigned w[2];
+  asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "l"(p) : "memory");
+  return make_float2(__uint_as_float(w[0]), __uint_as_float(w[1]));
+}
+__device__ __forceinline__ float4 get_words4(const float *p) {
+  unsigned w[4];
+  asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(p) : "memory");
+  return make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3]));
+}
+// A thread's N vectors of words: load(i, v[i]) is asked once for all, then again for those that still hold a hole, for 2 s at
+// most (then the CTA gives up: what the caller goes on with is never used).  Asking for all of them again each time made
+// a look at a row's 64 KB of pieces 1.2 us long.
+__device__ __forceinline__ unsigned top(float v) { return __float_as_uint(v); }
+__device__ __forceinline__ unsigned top(const float2 &v) { return max(top(v.x), top(v.y)); }
+__device__ __forceinline__ unsigned top(const float4 &v) { return max(max(top(v.x), top(v.y)), max(top(v.z), top(v.w))); }
+template <int N, class V, class Load> __device__ __forceinline__ void settle_words(V (&v)[N], const Load &load, volatile int *abort_flag) {
+  unsigned long long t0 = 0;
+  for (unsigned it = 1;; ++it) {
+    unsigned seen = 0u;
+#pragma unroll
+    for (int i = 0; i < N; ++i) seen = max(seen, top(v[i]));
+    if (seen != kHole) return;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (top(v[i]) == kHole) load(i);
+    if ((it & 15u) != 0u) continue;
+    if (*abort_flag) return;
+    const unsigned long long now = globaltimer_ns();
+    if (t0 == 0) t0 = now;
+    else if (now - t0 > kWaitLimitNs) { *abort_flag = 1; return; }
+  }
+}
+template <int N, class V, class Load> __device__ __forceinline__ void fetch_words(V (&v)[N], const Load &load, volatile int *abort_flag) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) load(i);
+  settle_words(v, load, abort_flag);
+}
 __device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 2, 256;" ::: "memory"); }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 // barrier of one 128-thread worker group (id 1 = warps 4..7, the epilogue group; id 3 = warps 8..11)
@@ -227,38 +305,16 @@ __device__ __forceinline__ bool grid_barrier(const FwdArgs &a, unsigned &epoch, 
 // ------------------------------------------------------------------------------ RMSNorm phase
 // One row per CTA turn, held in registers (all loads issued before their first use).
 //   src_embed: the row comes from the embedding table (and is copied to x).
-//   pend:      the residual-add projection that ran just before; its split pieces are added to the
-//              row in fixed piece order (x <- x + p_0 + p_1 + ...) and x is written back.
-// Requires d % 4 == 0 and d <= 4096.
-//   pieces_target != 0: the CTA was idle in that projection and has passed no grid barrier since; it waits until
-//              the counter of CTAs that have stored their pieces reaches pieces_target.
-template <int NPAD>
-__device__ __forceinline__ bool norm_phase(const FwdArgs &a, int n_rows, const int *row_list, bool src_embed,
-                                           const Gemm *pend, const float *pend_pieces, const __nv_bfloat16 *gain, __nv_bfloat16 *dst,
-                                           float *red, int wt, unsigned pieces_target, volatile int *abort_flag) {
-  constexpr int MAXV = 4;                                  // float4 slots per thread
-  constexpr int PB = 4;                                    // pieces loaded at a time per slot
+//   pend_pieces: split pieces (np per tile) of the residual-add projection that ran just before; they are added to
+//              the row in fixed piece order (x <- x + p_0 + p_1 + ...) and x is written back.
+// Requires d % 4 == 0 and d <= 1024 MAXV.
+template <int NPAD, int MAXV>                              // MAXV float4 slots per thread: rows of up to 1024 MAXV columns
+__device__ __forceinline__ void norm_phase(const FwdArgs &a, int n_rows, const int *row_list, bool src_embed,
+                                           const float *pend_pieces, int np, const __nv_bfloat16 *gain, __nv_bfloat16 *dst,
+                                           float *red, int wt, volatile int *abort_flag) {
+  constexpr int PB = 16 / MAXV;                            // pieces per slot (residual_parts)
   const int d = a.d, nvec = d >> 2;
-  SplitGeom geo;
-  geo.U = 1; geo.Gp = 1; geo.pieces_max = 1;
-  if (pend) geo = split_geom(*pend, gridDim.x);
-  // rows go to the LAST CTAs of the grid when the norm may start early: those have no tile of the projection
-  const int first = a.early_norm ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
-  if (pieces_target != 0u && first < n_rows) {
-    if (wt == 0) {
-      const unsigned *cnt = a.grid_counter + 16;
-      unsigned long long t0 = 0;
-      for (uint32_t it = 0; (int)(ld_acquire_u32(cnt) - pieces_target) < 0; ++it) {
-        if ((it & 31u) == 31u) {
-          const unsigned long long now = globaltimer_ns();
-          if (t0 == 0) t0 = now;
-          if (*abort_flag || now - t0 > kWaitLimitNs) { *abort_flag = 1; break; }
-        }
-      }
-    }
-    worker_sync();
-    if (*abort_flag) return false;
-  }
+  const int first = (int)(gridDim.x - 1 - blockIdx.x);      // the last CTAs first: they hold no tile of the projection
   for (int i = first; i < n_rows; i += gridDim.x) {
     const int row = row_list ? row_list[i] : i;
     float *xrow = a.x + (size_t)row * d;
@@ -290,26 +346,27 @@ __device__ __forceinline__ bool norm_phase(const FwdArgs &a, int n_rows, const i
       const int iv = wt + 256 * j;
       graw[j] = iv < nvec ? __ldg(reinterpret_cast<const uint2 *>(gain) + iv) : make_uint2(0u, 0u);
     }
-    if (pend) {
+    if (pend_pieces) {
       // every piece of every slot in one batch of loads: the residual projections have at most d / 128
-      // = 32 tiles, so they are always cut the regular way (the launcher checks it), `parts` <= 4
-      // pieces per tile at a fixed stride
-      const int np = geo.parts;
-      float4 t[MAXV][PB];
+      // = 32 tiles, so they are always cut the regular way (the launcher checks it), np <= PB pieces per
+      // tile at a fixed stride
+      float4 t[MAXV * PB];
+      const float *base[MAXV];
 #pragma unroll
       for (int j = 0; j < MAXV; ++j) {
-        const int iv = wt + 256 * j, k = iv << 2, tile = k >> 7, mm = k & 127;
-        const float *base = pend_pieces + ((size_t)tile * np * NPAD + row) * kTcBlockM + mm;
-#pragma unroll
-        for (int pp = 0; pp < PB; ++pp)
-          t[j][pp] = (iv < nvec && pp < np) ? __ldcg(reinterpret_cast<const float4 *>(base + (size_t)pp * NPAD * kTcBlockM))
-                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+        const int k = (wt + 256 * j) << 2;
+        base[j] = pend_pieces + ((size_t)(k >> 7) * np * NPAD + row) * kTcBlockM + (k & 127);
       }
+      fetch_words(t, [&](int i) {
+        const int j = i / PB, pp = i % PB;
+        t[i] = (wt + 256 * j < nvec && pp < np) ? get_words4(base[j] + (size_t)pp * NPAD * kTcBlockM) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }, abort_flag);
 #pragma unroll
       for (int j = 0; j < MAXV; ++j)
 #pragma unroll
         for (int pp = 0; pp < PB; ++pp) {
-          v[j].x += t[j][pp].x; v[j].y += t[j][pp].y; v[j].z += t[j][pp].z; v[j].w += t[j][pp].w;
+          const float4 &e = t[j * PB + pp];
+          v[j].x += e.x; v[j].y += e.y; v[j].z += e.z; v[j].w += e.w;
         }
     }
     float ss = 0.f;
@@ -327,7 +384,7 @@ __device__ __forceinline__ bool norm_phase(const FwdArgs &a, int n_rows, const i
     for (int j = 0; j < MAXV; ++j) {
       const int iv = wt + 256 * j;
       if (iv < nvec) {
-        if (src_embed || pend) reinterpret_cast<float4 *>(xrow)[iv] = v[j];
+        if (src_embed || pend_pieces) reinterpret_cast<float4 *>(xrow)[iv] = v[j];
         const float g0 = __uint_as_float(graw[j].x << 16), g1 = __uint_as_float(graw[j].x & 0xFFFF0000u);
         const float g2 = __uint_as_float(graw[j].y << 16), g3 = __uint_as_float(graw[j].y & 0xFFFF0000u);
         __nv_bfloat162 lo = __floats2bfloat162_rn(v[j].x * inv * g0, v[j].y * inv * g1);
@@ -339,7 +396,6 @@ __device__ __forceinline__ bool norm_phase(const FwdArgs &a, int n_rows, const i
       }
     }
   }
-  return true;
 }
 
 // ------------------------------------------------------------------------------ attention phases
@@ -354,6 +410,14 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gsrc) : "memory");
 }
 
+struct LayerNorms { const __nv_bfloat16 *attn, *mlp; };
+__device__ __forceinline__ FwdLayerDev layer_of(const FwdArgs &a, int l) {
+  FwdLayerDev ly;
+  ly.attn_norm = ly.mlp_norm = nullptr;
+  ly.k_pool = reinterpret_cast<__nv_bfloat16 *>(a.k_pool + a.pool_stride * l);
+  ly.v_pool = reinterpret_cast<__nv_bfloat16 *>(a.v_pool + a.pool_stride * l);
+  return ly;
+}
 struct PageCache { int tag_item, tag_tile; int pg[128]; };   // pg[warp * 16 + j]: page of the warp's j-th sub-tile
 
 __device__ __forceinline__ void mma_bf16_16x8x16(float *c, const unsigned *a, unsigned b0, unsigned b1) {
@@ -683,7 +747,7 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
     const float mm = fmaxf(m_ref, m1);
     const float f0 = m_ref > -INFINITY ? ex2_approx((m_ref - mm) * sc) : 0.f, f1 = m1 > -INFINITY ? ex2_approx((m1 - mm) * sc) : 0.f;
     const float lt = l * f0 + l1 * f1;
-    const bool real = lane < it.nqv;
+    const bool real = lane < it.nqv, wanted = it.key_lo <= it.pos0 + lane / it.group;   // (the merge phase reads a row's splits up to its own position)
     const int r = it.row0 + lane / it.group, hq = it.kvh * it.group + lane % it.group;
     float *dst = a.attn_partials + (((size_t)r * a.nq + hq) * a.n_splits + it.split) * (HD + 2);
     __nv_bfloat16 *adst = a.att + ((size_t)r * a.nq + hq) * HD;
@@ -702,13 +766,13 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
 #pragma unroll
           for (int e = 0; e < 16; e += 2)
             *reinterpret_cast<__nv_bfloat162 *>(adst + c + e) = __floats2bfloat162_rn(o[e] * inv, o[e + 1] * inv);
-        } else {
+        } else if (wanted) {
 #pragma unroll
-          for (int e = 0; e < 16; e += 2) *reinterpret_cast<float2 *>(dst + c + e) = make_float2(o[e], o[e + 1]);
+          for (int e = 0; e < 16; e += 2) put_words2(dst + c + e, o[e], o[e + 1]);
         }
       }
     }
-    if (real && a.n_splits > 1) { dst[HD] = mm * rsqrtf((float)HD); dst[HD + 1] = lt; }   // m in natural-log units, as the merge phase expects
+    if (real && wanted && a.n_splits > 1) put_words2(dst + HD, mm * rsqrtf((float)HD), lt);   // m in natural-log units, as the merge phase expects
     tc_fence_before();
   }
   lap(8);
@@ -851,17 +915,11 @@ __device__ __forceinline__ void attn_tiles_phase(const FwdArgs &a, const FwdLaye
           const int U = qkv_geom[4], Gp = qkv_geom[5], KB = qkv_geom[6];
           n_pieces = unit_owner(U, Gp, tile * KB + KB - 1) - unit_owner(U, Gp, tile * KB) + 1;
         }
-        const float *base = a.pieces + ((size_t)(tile * g_pmax) * NPAD + (row0 + rr)) * kTcBlockM + m;
-        float4 pc4[4][4];                                        // [piece][low 0-3, low 4-7, high 0-3, high 4-7]
-#pragma unroll
-        for (int pp = 0; pp < 4; ++pp) {
-          const float4 *src = reinterpret_cast<const float4 *>(base + pp * pstride);
-          const bool on = pp < n_pieces;
-          pc4[pp][0] = on ? __ldcg(src) : make_float4(0.f, 0.f, 0.f, 0.f);
-          pc4[pp][1] = on ? __ldcg(src + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
-          pc4[pp][2] = on ? __ldcg(src + HALF / 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-          pc4[pp][3] = on ? __ldcg(src + HALF / 4 + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        const float *base = a.pieces[0] + ((size_t)(tile * g_pmax) * NPAD + (row0 + rr)) * kTcBlockM + m;
+        float4 pc4[16];                                          // [piece][low 0-3, low 4-7, high 0-3, high 4-7]
+        fetch_words(pc4, [&](int i) {
+          pc4[i] = (i >> 2) < n_pieces ? get_words4(base + (i >> 2) * pstride + (i & 1) * 4 + ((i >> 1) & 1) * HALF) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }, abort_flag);
         float cs[8], sn[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) { cs[e] = 1.f; sn[e] = 0.f; }
@@ -880,10 +938,10 @@ __device__ __forceinline__ void attn_tiles_phase(const FwdArgs &a, const FwdLaye
         for (int e = 0; e < 8; ++e) { lo[e] = 0.f; hi[e] = 0.f; }
 #pragma unroll
         for (int pp = 0; pp < 4; ++pp) {
-          lo[0] += pc4[pp][0].x; lo[1] += pc4[pp][0].y; lo[2] += pc4[pp][0].z; lo[3] += pc4[pp][0].w;
-          lo[4] += pc4[pp][1].x; lo[5] += pc4[pp][1].y; lo[6] += pc4[pp][1].z; lo[7] += pc4[pp][1].w;
-          hi[0] += pc4[pp][2].x; hi[1] += pc4[pp][2].y; hi[2] += pc4[pp][2].z; hi[3] += pc4[pp][2].w;
-          hi[4] += pc4[pp][3].x; hi[5] += pc4[pp][3].y; hi[6] += pc4[pp][3].z; hi[7] += pc4[pp][3].w;
+          lo[0] += pc4[4 * pp + 0].x; lo[1] += pc4[4 * pp + 0].y; lo[2] += pc4[4 * pp + 0].z; lo[3] += pc4[4 * pp + 0].w;
+          lo[4] += pc4[4 * pp + 1].x; lo[5] += pc4[4 * pp + 1].y; lo[6] += pc4[4 * pp + 1].z; lo[7] += pc4[4 * pp + 1].w;
+          hi[0] += pc4[4 * pp + 2].x; hi[1] += pc4[4 * pp + 2].y; hi[2] += pc4[4 * pp + 2].z; hi[3] += pc4[4 * pp + 2].w;
+          hi[4] += pc4[4 * pp + 3].x; hi[5] += pc4[4 * pp + 3].y; hi[6] += pc4[4 * pp + 3].z; hi[7] += pc4[4 * pp + 3].w;
         }
         unsigned wl[4], wh[4];
 #pragma unroll
@@ -1086,10 +1144,10 @@ __device__ __forceinline__ void attn_tiles_phase(const FwdArgs &a, const FwdLaye
       const int r = row0 + qi / group, hq = kvh * group + qi % group;
       if (a.n_splits == 1) {                                     // the only split: this is the attention output
         *reinterpret_cast<__nv_bfloat162 *>(a.att + ((size_t)r * a.nq + hq) * HD + dd) = __floats2bfloat162_rn(ox / l, oy / l);
-      } else {
+      } else if (key_lo <= pos0 + qi / group) {                  // (the merge phase reads a row's splits up to its own position)
         float *dst = a.attn_partials + (((size_t)r * a.nq + hq) * a.n_splits + split) * (HD + 2);
-        *reinterpret_cast<float2 *>(dst + dd) = make_float2(ox, oy);
-        if (dd == 0) { dst[HD] = mm; dst[HD + 1] = l; }
+        put_words2(dst + dd, ox, oy);
+        if (dd == 0) put_words2(dst + HD, mm, l);
       }
     }
     lap(4);
@@ -1099,7 +1157,7 @@ __device__ __forceinline__ void attn_tiles_phase(const FwdArgs &a, const FwdLaye
 // Phase B: merge the split partials of one (row, head) per HD / 2 threads (two output dimensions each); a single
 // batch of loads.
 template <int HD>
-__device__ __forceinline__ void attn_merge_phase(const FwdArgs &a, const int *row_pos_sh, int wt) {
+__device__ __forceinline__ void attn_merge_phase(const FwdArgs &a, const int *row_pos_sh, int wt, volatile int *abort_flag) {
   constexpr int TPI = HD / 2, PER = 256 / TPI;                    // threads per item, items per CTA turn
   const int g = wt / TPI, dd = (wt % TPI) * 2;
   const int n_items = a.R * a.nq;
@@ -1107,25 +1165,21 @@ __device__ __forceinline__ void attn_merge_phase(const FwdArgs &a, const int *ro
     const int r = it / a.nq;
     const int used = min(a.n_splits, row_pos_sh[r] / a.keys_per_split + 1);   // splits holding keys <= own position
     const float *src = a.attn_partials + (size_t)it * a.n_splits * (HD + 2);
-    float ms[kAttnMaxSplits], ls[kAttnMaxSplits];
-    float2 os[kAttnMaxSplits];
-#pragma unroll
-    for (int s = 0; s < kAttnMaxSplits; ++s) {
-      const bool on = s < used;
-      const float2 ml = on ? __ldcg(reinterpret_cast<const float2 *>(src + s * (HD + 2) + HD)) : make_float2(-INFINITY, 0.f);
-      ms[s] = ml.x; ls[s] = ml.y;
-      os[s] = on ? __ldcg(reinterpret_cast<const float2 *>(src + s * (HD + 2) + dd)) : make_float2(0.f, 0.f);
-    }
+    float2 w[2 * kAttnMaxSplits];                                  // (m, l) and two output dimensions of every split
+    fetch_words(w, [&](int i) {
+      const int sp = i >> 1;
+      w[i] = sp < used ? get_words2(src + sp * (HD + 2) + ((i & 1) ? dd : HD)) : ((i & 1) ? make_float2(0.f, 0.f) : make_float2(-INFINITY, 0.f));
+    }, abort_flag);
     float m = -INFINITY;
 #pragma unroll
-    for (int s = 0; s < kAttnMaxSplits; ++s) m = fmaxf(m, ms[s]);
+    for (int s = 0; s < kAttnMaxSplits; ++s) m = fmaxf(m, w[2 * s].x);
     float l = 0.f, ox = 0.f, oy = 0.f;
 #pragma unroll
     for (int s = 0; s < kAttnMaxSplits; ++s) {
-      const float w = (ms[s] > -INFINITY) ? __expf(ms[s] - m) : 0.f;
-      l += w * ls[s];
-      ox += w * os[s].x;
-      oy += w * os[s].y;
+      const float f = (w[2 * s].x > -INFINITY) ? __expf(w[2 * s].x - m) : 0.f;
+      l += f * w[2 * s].y;
+      ox += f * w[2 * s + 1].x;
+      oy += f * w[2 * s + 1].y;
     }
     *reinterpret_cast<__nv_bfloat162 *>(a.att + (size_t)it * HD + dd) = __floats2bfloat162_rn(ox / l, oy / l);
   }
@@ -1199,11 +1253,42 @@ struct WorkerCtx {
   volatile int *abort_flag, *wait_ok;
   float *staging;
   const int *row_pos_sh, *row_pg_sh;
-  const FwdLayerDev *layers_sh;
   const float *rope_cos_sh, *rope_sin_sh;
+  const PhaseGeom *geom;                         // [5], by kind of projection
   int wt, lane, q, G, c;
   int seg_idx;
 };
+
+// This CTA's words of a projection become holes again (warps 8..11 while the others are in a later projection).
+template <int NPAD>
+__device__ __forceinline__ void put_holes(const FwdArgs &a, const WorkerCtx &w, int kind) {
+  const PhaseGeom &pg = w.geom[kind];
+  SegIter it = seg_begin(pg);
+  Seg sg;
+#pragma unroll 1
+  while (seg_next(pg, it, sg)) {
+    float *mine = a.pieces[kind] + ((size_t)sg.tile * pg.pieces_max + piece_of(pg, sg)) * NPAD * kTcBlockM + (w.wt & 127);
+    for (int r = 0; r < a.R; ++r) put_hole(mine + r * kTcBlockM);
+  }
+}
+// ... and its attention partials: a warp per query vector.
+template <int HD>
+__device__ __forceinline__ void put_partial_holes(const FwdArgs &a, int wt, const int *first_item) {
+  const int group = a.nq / a.nkv, n_work = a.n_attn * a.nkv * a.n_splits;
+  const float inv_group = 1.f / (float)group;
+#pragma unroll 1
+  for (int wi = blockIdx.x; wi < n_work; wi += gridDim.x) {
+    const int unit = wi / a.n_splits, split = wi - unit * a.n_splits, ai = unit / a.nkv, kvh = unit - ai * a.nkv;
+    const int4 it = wi == (int)blockIdx.x ? make_int4(first_item[0], first_item[1], first_item[2], first_item[3]) : a.attn_items[ai];
+    const int key_lo = split * a.keys_per_split;
+    if (key_lo >= it.w + it.y) continue;
+    for (int qi = max(0, key_lo - it.w) * group + ((wt >> 5) & 3); qi < it.y * group; qi += 4) {       // rows from key_lo on wrote theirs
+      const int r = (int)(((float)qi + 0.5f) * inv_group);
+      float *dst = a.attn_partials + (((size_t)(it.x + r) * a.nq + kvh * group + qi - r * group) * a.n_splits + split) * (HD + 2);
+      for (int e = wt & 31; e < HD / 2 + 1; e += 32) put_holes2(dst + 2 * e);
+    }
+  }
+}
 
 // GEMM phase p, epilogue side (warps 4..7): accumulator -> this CTA's piece of the tile.  Group-uniform:
 // a give-up is decided by one thread and shared. 
@@ -1213,17 +1298,14 @@ __device__ __forceinline__ void gemm_epilogue(const FwdArgs &a, WorkerCtx &w, in
   constexpr int CH = PCfg<NPAD>::kChunk;
   const int m = w.q * 32 + w.lane;
 
-    const Gemm g = make_gemm(a, p);
-    const SplitGeom geo = split_geom(g, w.G);
-    SegIter it = seg_begin(g, w.G, w.c);
+    const int kind = kind_of(a, p), rows = kind == 4 ? a.L : a.R;
+    const PhaseGeom &pg = w.geom[kind];
+    const bool keep = a.L > 0 || p != 4 * a.n_run - 1;            // a pass without logits ends here: nobody reads these pieces
+    SegIter it = seg_begin(pg);
     Seg sg;
-    for (; seg_next(g, it, sg); ++w.seg_idx) {
+    for (; seg_next(pg, it, sg); ++w.seg_idx) {
       const int ab = w.seg_idx & 1;
-      // this CTA's piece of the tile (the next phase sums the pieces): worked out while the MMAs run
-      int fo, np_tile;
-      tile_pieces(g, geo, sg.tile, fo, np_tile);
-      const int piece = w.c - fo;
-      float *mine = pieces_of(a, p) + ((size_t)sg.tile * geo.pieces_max + piece) * NPAD * kTcBlockM;
+      float *mine = a.pieces[kind] + ((size_t)sg.tile * pg.pieces_max + piece_of(pg, sg)) * NPAD * kTcBlockM;
       if (w.wt == 0) w.wait_ok[w.seg_idx & 1] = mbar_wait((w.accf_bar0 + 8u * ab), (uint32_t)((w.seg_idx >> 1) & 1), w.abort_flag) ? 1 : 0;
       epi_sync();
       if (!w.wait_ok[w.seg_idx & 1]) return;
@@ -1240,18 +1322,12 @@ __device__ __forceinline__ void gemm_epilogue(const FwdArgs &a, WorkerCtx &w, in
           __syncwarp();
           if (w.lane == 0) mbar_arrive((w.acce_bar0 + 8u * ab));
         }
-        if (c0 < g.rows) {
+        if (c0 < rows && keep) {
 #pragma unroll
           for (int i = 0; i < CH; ++i)
-            if (c0 + i < g.rows) mine[(c0 + i) * kTcBlockM + m] = v[i];
+            if (c0 + i < rows) put_word(mine + (c0 + i) * kTcBlockM + m, v[i]);
         }
       }
-    }
-    // residual projection whose norm starts early: tell the norm's CTAs that this CTA's pieces are in place (the
-    // stores of the 128 epilogue threads are ordered before the release by the group barrier, as in the grid barrier)
-    if (a.early_norm && g.mode == MODE_ADD && w.c < geo.Gp) {
-      epi_sync();
-      if (w.wt == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.grid_counter + 16) : "memory");
     }
   }
 
@@ -1263,14 +1339,13 @@ __device__ __forceinline__ void gemm_epilogue(const FwdArgs &a, WorkerCtx &w, in
 // a warp keeps the loads of its next two stages in flight (DEPTH = 2).
 template <int NPAD, int PB, int DEPTH>
 __device__ __forceinline__ void build_act_stages(const FwdArgs &a, WorkerCtx &w, int p, uint8_t *ring, uint32_t full_bar0,
-                                                 uint32_t empty_bar0, volatile unsigned *ring_pos, const int *bgeom) {
+                                                 uint32_t empty_bar0, volatile unsigned *ring_pos) {
   constexpr int STAGES = PCfg<NPAD>::kStages;
-  // geometry worked out once at kernel start (the same in every layer): this CTA's k-blocks of the down projection
-  // (residual projections: one segment per CTA) and how the gate / up tiles are cut into pieces
-  SegIter it;
-  it.tile = 0; it.kb = bgeom[0]; it.left = bgeom[1];
-  const int g_parts = bgeom[2], g_pmax = bgeom[3];
-  const int KBg = a.d / kTcBlockK, Ug = ((a.ff + kTcBoxRows - 1) / kTcBoxRows) * KBg, Gpg = min(w.G, Ug);
+  // this CTA's k-blocks of the down projection (residual projections: one segment per CTA) and how the gate / up
+  // tiles are cut into pieces
+  const PhaseGeom &pgu = w.geom[2];
+  const SegIter it = seg_begin(w.geom[3]);
+  const int g_parts = pgu.parts, g_pmax = pgu.pieces_max, KBg = pgu.KB, Ug = pgu.U, Gpg = pgu.Gp;
   const float inv_U = 1.f / (float)Ug;
   // unit_owner without an integer division (all quantities < 2^24, so the float quotient is off by one at most)
   auto owner = [&](int u) {
@@ -1294,25 +1369,23 @@ __device__ __forceinline__ void build_act_stages(const FwdArgs &a, WorkerCtx &w,
   const uint32_t par0 = (rp >> 8) & 1u;
   const bool on = r < a.R;
   const size_t pstride = (size_t)NPAD * kTcBlockM;
-  const float *lane_base = a.pieces + (size_t)r * kTcBlockM + c8 * 8;
-  float4 t[DEPTH][PB][4];                                      // [stage in flight][piece][gate 0-3, gate 4-7, up 0-3, up 4-7]
-  auto load = [&](float4 (&dst)[PB][4], int i) {               // pieces of the CTA's stage i (this lane's row and columns)
+  const float *lane_base = a.pieces[2] + (size_t)r * kTcBlockM + c8 * 8;
+  float4 t[DEPTH][PB * 4];                                     // [stage in flight][piece: gate 0-3, gate 4-7, up 0-3, up 4-7]
+  auto load = [&](float4 (&dst)[PB * 4], int i, auto &&take) { // pieces of the CTA's stage i (this lane's row and columns)
     const int kb = it.kb + i;
     int n_pieces = 0;
-    if (i < it.left) n_pieces = g_parts ? g_parts : owner(kb * KBg + KBg - 1) - owner(kb * KBg) + 1;
+    if (i < it.left && on) n_pieces = g_parts ? g_parts : owner(kb * KBg + KBg - 1) - owner(kb * KBg) + 1;
     const float *tbase = lane_base + (size_t)kb * g_pmax * pstride;
+    take([&](int q) {
+      dst[q] = (q >> 2) < n_pieces ? get_words4(tbase + (q >> 2) * pstride + (q & 1) * 4 + ((q >> 1) & 1) * kTcBoxRows) : make_float4(0.f, 0.f, 0.f, 0.f);
+    });
+  };
+  auto ask = [&](auto &&one) {
 #pragma unroll
-    for (int pp = 0; pp < PB; ++pp) {
-      const float4 *src = reinterpret_cast<const float4 *>(tbase + pp * pstride);
-      const bool ld = on && pp < n_pieces;
-      dst[pp][0] = ld ? __ldcg(src) : make_float4(0.f, 0.f, 0.f, 0.f);
-      dst[pp][1] = ld ? __ldcg(src + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
-      dst[pp][2] = ld ? __ldcg(src + kTcBoxRows / 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-      dst[pp][3] = ld ? __ldcg(src + kTcBoxRows / 4 + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    for (int q = 0; q < PB * 4; ++q) one(q);
   };
 #pragma unroll
-  for (int dpt = 0; dpt < DEPTH; ++dpt) load(t[dpt], warp4 + 4 * dpt);
+  for (int dpt = 0; dpt < DEPTH; ++dpt) load(t[dpt], warp4 + 4 * dpt, ask);
 #pragma unroll 1
   for (int i0 = warp4; i0 < it.left; i0 += 4 * DEPTH) {
 #pragma unroll
@@ -1321,6 +1394,8 @@ __device__ __forceinline__ void build_act_stages(const FwdArgs &a, WorkerCtx &w,
       if (i >= it.left) break;
       const int pos = s0 + i, s = pos % STAGES;
       const uint32_t par = par0 ^ (uint32_t)((pos / STAGES) & 1);
+      load(t[dpt], i, [&](auto &&one) { settle_words(t[dpt], one, w.abort_flag); });
+      __syncwarp();
       bool ok = true;                                          // the slot is free once its previous MMAs have retired
       if (w.lane == 0) ok = mbar_wait(empty_bar0 + 8u * s, par, w.abort_flag);
       if (!__shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0)) return;
@@ -1329,10 +1404,10 @@ __device__ __forceinline__ void build_act_stages(const FwdArgs &a, WorkerCtx &w,
       for (int e = 0; e < 8; ++e) { gt[e] = 0.f; up[e] = 0.f; }
 #pragma unroll
       for (int pp = 0; pp < PB; ++pp) {
-        gt[0] += t[dpt][pp][0].x; gt[1] += t[dpt][pp][0].y; gt[2] += t[dpt][pp][0].z; gt[3] += t[dpt][pp][0].w;
-        gt[4] += t[dpt][pp][1].x; gt[5] += t[dpt][pp][1].y; gt[6] += t[dpt][pp][1].z; gt[7] += t[dpt][pp][1].w;
-        up[0] += t[dpt][pp][2].x; up[1] += t[dpt][pp][2].y; up[2] += t[dpt][pp][2].z; up[3] += t[dpt][pp][2].w;
-        up[4] += t[dpt][pp][3].x; up[5] += t[dpt][pp][3].y; up[6] += t[dpt][pp][3].z; up[7] += t[dpt][pp][3].w;
+        gt[0] += t[dpt][4 * pp + 0].x; gt[1] += t[dpt][4 * pp + 0].y; gt[2] += t[dpt][4 * pp + 0].z; gt[3] += t[dpt][4 * pp + 0].w;
+        gt[4] += t[dpt][4 * pp + 1].x; gt[5] += t[dpt][4 * pp + 1].y; gt[6] += t[dpt][4 * pp + 1].z; gt[7] += t[dpt][4 * pp + 1].w;
+        up[0] += t[dpt][4 * pp + 2].x; up[1] += t[dpt][4 * pp + 2].y; up[2] += t[dpt][4 * pp + 2].z; up[3] += t[dpt][4 * pp + 2].w;
+        up[4] += t[dpt][4 * pp + 3].x; up[5] += t[dpt][4 * pp + 3].y; up[6] += t[dpt][4 * pp + 3].z; up[7] += t[dpt][4 * pp + 3].w;
       }
       if (on) {
         unsigned o[4];
@@ -1347,7 +1422,7 @@ __device__ __forceinline__ void build_act_stages(const FwdArgs &a, WorkerCtx &w,
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor core reads the tile through the async proxy
       __syncwarp();
       if (w.lane == 0) mbar_arrive(full_bar0 + 8u * s);
-      load(t[dpt], i + 4 * DEPTH);                               // this buffer's next stage
+      load(t[dpt], i + 4 * DEPTH, ask);                          // this buffer's next stage
     }
   }
 }
@@ -1362,7 +1437,8 @@ __device__ __forceinline__ void gemm_finish(const FwdArgs &a, WorkerCtx &w, int 
   constexpr int PBF = 4;                         // pieces per tile at most (regular: <= 4 parts; dealt units: <= 3)
   constexpr int RB = 8;                          // token rows per unit (two load batches; more units than 2 x CTAs at 24+ rows)
   const Gemm g = make_gemm(a, p);
-  const SplitGeom geo = split_geom(g, w.G);
+  const PhaseGeom &pg = w.geom[kind_of(a, p)];
+  float *const pieces = a.pieces[kind_of(a, p)];
   const int layer = p >> 2;
   const int gidx = w.wt >> 7, gm = w.wt & 127;   // two groups of 128 threads, one unit each at a time
   float *gstage = w.staging + gidx * (kTcBlockM * (RG + 1));
@@ -1375,25 +1451,19 @@ __device__ __forceinline__ void gemm_finish(const FwdArgs &a, WorkerCtx &w, int 
 #pragma unroll 1
     for (int u = w.c + gidx * w.G; u < n_units; u += 2 * w.G) {
       const int tile = u / n_rb, r0 = (u - tile * n_rb) * RB + rh, col = tile * kTcBoxRows + cc;
-      int fo, n_pieces;
-      tile_pieces(g, geo, tile, fo, n_pieces);
-      const float *base = a.pieces + (size_t)tile * geo.pieces_max * NPAD * kTcBlockM + cc;
-      float tg[PBF][RB / 2], tu[PBF][RB / 2];
-#pragma unroll
-      for (int pp = 0; pp < PBF; ++pp)
-#pragma unroll
-        for (int i = 0; i < RB / 2; ++i) {
-          const bool on = pp < n_pieces && r0 + i < g.rows;
-          const float *src = base + ((size_t)pp * NPAD + r0 + i) * kTcBlockM;
-          tg[pp][i] = on ? __ldcg(src) : 0.f;
-          tu[pp][i] = on ? __ldcg(src + kTcBoxRows) : 0.f;
-        }
+      const int n_pieces = tile_pieces(pg, tile);
+      const float *base = pieces + (size_t)tile * pg.pieces_max * NPAD * kTcBlockM + cc;
+      float tw[PBF * RB];                        // [piece][row][gate, up]
+      fetch_words(tw, [&](int q) {
+        const int pp = q / RB, i = (q % RB) >> 1;
+        tw[q] = (pp < n_pieces && r0 + i < g.rows) ? get_word(base + ((size_t)pp * NPAD + r0 + i) * kTcBlockM + (q & 1) * kTcBoxRows) : 0.f;
+      }, w.abort_flag);
       if (col < g.seg_n[0]) {
 #pragma unroll
         for (int i = 0; i < RB / 2; ++i) {
           float gt = 0.f, up = 0.f;
 #pragma unroll
-          for (int pp = 0; pp < PBF; ++pp) { gt += tg[pp][i]; up += tu[pp][i]; }
+          for (int pp = 0; pp < PBF; ++pp) { gt += tw[pp * RB + 2 * i]; up += tw[pp * RB + 2 * i + 1]; }
           if (r0 + i < g.rows) a.act[(size_t)(r0 + i) * a.ff + col] = __float2bfloat16_rn(silu_mul(gt, up));
         }
       }
@@ -1404,18 +1474,18 @@ __device__ __forceinline__ void gemm_finish(const FwdArgs &a, WorkerCtx &w, int 
   for (int u = w.c + gidx * w.G; u < n_units; u += 2 * w.G) {
     const int tile = u / n_rb, r_lo = (u - tile * n_rb) * RB, r_hi = min(g.rows, r_lo + RB);
     const Tile ti = tile_of(g, tile);
-    int fo, n_pieces;
-    tile_pieces(g, geo, tile, fo, n_pieces);
-    const float *base = a.pieces + (size_t)tile * geo.pieces_max * NPAD * kTcBlockM + gm;
+    const int n_pieces = tile_pieces(pg, tile);
+    float *base = pieces + (size_t)tile * pg.pieces_max * NPAD * kTcBlockM + gm;
     const int half = a.hd >> 1, dh = ((ti.row0 + gm) % a.hd) % half;
     const bool rope = (g.mode == MODE_QKV && ti.seg < 2);
-    float tn[PBF][RG], csn[RG], snn[RG];
+    float tn[PBF * RG], csn[RG], snn[RG];
+    auto one = [&](int c0, int q) {
+      const int pp = q / RG, i = q % RG;
+      tn[q] = (pp < n_pieces && c0 + i < r_hi) ? get_word(base + ((size_t)pp * NPAD + c0 + i) * kTcBlockM) : 0.f;
+    };
     auto fetch = [&](int c0) {                   // pieces and rope values of rows c0 .. c0 + RG - 1
 #pragma unroll
-      for (int pp = 0; pp < PBF; ++pp)
-#pragma unroll
-        for (int i = 0; i < RG; ++i)
-          tn[pp][i] = (pp < n_pieces && c0 + i < r_hi) ? __ldcg(base + ((size_t)pp * NPAD + c0 + i) * kTcBlockM) : 0.f;
+      for (int q = 0; q < PBF * RG; ++q) one(c0, q);
 #pragma unroll
       for (int i = 0; i < RG; ++i) {
         csn[i] = 1.f; snn[i] = 0.f;
@@ -1434,15 +1504,22 @@ __device__ __forceinline__ void gemm_finish(const FwdArgs &a, WorkerCtx &w, int 
 #pragma unroll 1
     for (int c0 = r_lo; c0 < r_hi; c0 += RG) {
       float v[RG], cs[RG], sn[RG];
+      settle_words(tn, [&](int q) { one(c0, q); }, w.abort_flag);
+      if (g.mode == MODE_LOGITS) {               // the pass ends here: the words' one reader makes them holes again
+        for (int pp = 0; pp < n_pieces; ++pp)
+#pragma unroll
+          for (int i = 0; i < RG; ++i)
+            if (c0 + i < r_hi) put_hole(base + ((size_t)pp * NPAD + c0 + i) * kTcBlockM);
+      }
 #pragma unroll
       for (int i = 0; i < RG; ++i) {
         v[i] = 0.f;
 #pragma unroll
-        for (int pp = 0; pp < PBF; ++pp) v[i] += tn[pp][i];
+        for (int pp = 0; pp < PBF; ++pp) v[i] += tn[pp * RG + i];
         cs[i] = csn[i]; sn[i] = snn[i];
       }
       if (c0 + RG < r_hi) fetch(c0 + RG);
-      final_store<RG>(a, g, ti, w.layers_sh[layer < a.n_run ? layer : 0], gm, gm, c0, v, gstage, w.row_pos_sh,
+      final_store<RG>(a, g, ti, layer_of(a, layer < a.n_run ? layer : 0), gm, gm, c0, v, gstage, w.row_pos_sh,
                       w.row_pg_sh, cs, sn, 1 + 2 * gidx);
     }
   }
@@ -1468,14 +1545,16 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
   // [16] phase << 16 | parity << 8 | slot of the first stage of built down projection number (layer & 15): the
   // weight producer is at most one ring (8 stages) ahead, so never 16 such phases
   volatile unsigned *ring_pos_sh = reinterpret_cast<volatile unsigned *>(ctl + 928);
-  int *bgeom_sh = reinterpret_cast<int *>(ctl + 944);                    // [4] geometry of the built down projection
-  static_assert((2 * Cfg::kStages + 6) * 8 + (944 + 4) * 4 <= kCtrlBytes - 128, "control area overflow");
+  PhaseGeom *geom_sh = reinterpret_cast<PhaseGeom *>(ctl + 672);          // [5]
+  static_assert(5 * sizeof(PhaseGeom) <= (928 - 672) * 4, "control area overlap");
+  static_assert((2 * Cfg::kStages + 6) * 8 + 944 * 4 <= kCtrlBytes - 128, "control area overflow");
   volatile int *wait_ok = reinterpret_cast<volatile int *>(ctl + 4);   // [2]
   float *red = reinterpret_cast<float *>(ctl + 8);                      // [8]
   PageCache *pcache = reinterpret_cast<PageCache *>(ctl + 16);          // 130 words
   int *row_pos_sh = reinterpret_cast<int *>(ctl + 160);                 // [128] position of each packed row
   int *row_pg_sh = reinterpret_cast<int *>(ctl + 288);                  // [128] KV page holding that position
-  FwdLayerDev *layers_sh = reinterpret_cast<FwdLayerDev *>(ctl + 416);  // [<= kMaxLayersSh] pointer table
+  LayerNorms *norms_sh = reinterpret_cast<LayerNorms *>(ctl + 416);     // [<= kMaxLayersSh] norm gains
+  static_assert(kMaxLayersSh * sizeof(LayerNorms) <= (672 - 416) * 4, "control area overlap");
   long long *dbg_cy = reinterpret_cast<long long *>(reinterpret_cast<uint8_t *>(bars) + kCtrlBytes - 128);   // debug cycle counters [16]
   // cos / sin of the launch's rows (the tables are touched once per layer, so the weight stream would
   // evict them from L2 between uses): [kRopeCacheRows][hd / 2] each, after the attention / staging area
@@ -1504,6 +1583,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
     pcache->tag_tile = -1;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (threadIdx.x >= 128 && threadIdx.x < 133) {
+    const int k = threadIdx.x - 128;
+    geom_sh[k] = phase_geom(make_gemm(a, k < 4 ? k : 4 * a.n_run), G, c);
+  }
   constexpr uint32_t tmem_cols = TC ? 512u : (uint32_t)Cfg::kTmemCols;      // the attention phase takes all of tensor memory
   if (warp == 2) tmem_alloc(smem_u32(tmem_slot), tmem_cols);
   tc_fence_before();
@@ -1525,13 +1608,14 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
     bool ok = true;
     for (int p = 0; p < n_phases && ok; ++p) {
       const Gemm g = make_gemm(a, p);
-      SegIter it = seg_begin(g, G, c);
+      const PhaseGeom &pg = geom_sh[kind_of(a, p)];
+      SegIter it = seg_begin(pg);
       Seg sg;
       // the tensor-memory attention phase uses the ring's memory: the O projection's tiles wait until it is over
       // (one completion per layer, waited for in every layer, so the parity never is ambiguous)
       if (TC && (p & 3) == 1 && p < 4 * a.n_run && !mbar_wait_warp(attn_done_bar, (uint32_t)((p >> 2) & 1), abort_flag)) { ok = false; break; }
       if (issuer && built_down(a, p)) ring_pos_sh[(p >> 2) & 15] = (unsigned)s | (par << 8) | ((unsigned)p << 16);   // where the builders' tiles go
-      while (ok && seg_next(g, it, sg)) {
+      while (ok && seg_next(pg, it, sg)) {
         const Tile ti = tile_of(g, sg.tile);
         const bool second = (g.mode == MODE_SWIGLU) || (ti.row0 + kTcBoxRows < g.seg_n[ti.seg]);
         const CUtensorMap *m0 = g.mode == MODE_SWIGLU ? g.w[0] : g.w[ti.seg];
@@ -1570,10 +1654,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
     bool ok = true;
     const uint32_t a_bytes = (uint32_t)a.a_box_rows * kTcBlockK * 2;
     for (int p = 0; p < n_phases && ok; ++p) {
-      const Gemm g = make_gemm(a, p);
-      SegIter it = seg_begin(g, G, c);
+      const int kind = kind_of(a, p);
+      const CUtensorMap *amap = &a.amap[kind == 1 ? 1 : kind == 3 ? 2 : kind == 4 ? 3 : 0];
+      const PhaseGeom &pg = geom_sh[kind];
+      SegIter it = seg_begin(pg);
       Seg sg;
-      bool have = seg_next(g, it, sg);
+      bool have = seg_next(pg, it, sg);
       // the operand of phase p is complete once the workers have passed the barrier before it
       if (!mbar_wait_warp(ready_bar(p & 1), (uint32_t)((p >> 1) & 1), abort_flag)) { ok = false; break; }
       const bool built = built_down(a, p);
@@ -1582,11 +1668,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
           if (!mbar_wait_warp(empty_bar(s), par, abort_flag)) { ok = false; break; }
           if (issuer && !built) {                        // built down projection: the workers fill the tile and arrive
             mbar_expect_tx(full_bar(s), a_bytes);
-            tma_load_2d(smem_u32(ring) + (uint32_t)(s * Cfg::kStageBytes) + kWBytes, g.amap, kb * kTcBlockK, 0, full_bar(s));
+            tma_load_2d(smem_u32(ring) + (uint32_t)(s * Cfg::kStageBytes) + kWBytes, amap, kb * kTcBlockK, 0, full_bar(s));
           }
           if (++s == STAGES) { s = 0; par ^= 1u; }
         }
-        have = seg_next(g, it, sg);
+        have = seg_next(pg, it, sg);
       }
     }
     if (!ok && issuer) atomicExch(a.status, 1);
@@ -1599,10 +1685,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
     uint32_t par = 0;
     bool ok = true;
     for (int p = 0; p < n_phases && ok; ++p) {
-      const Gemm g = make_gemm(a, p);
-      SegIter it = seg_begin(g, G, c);
+      const PhaseGeom &pg = geom_sh[kind_of(a, p)];
+      SegIter it = seg_begin(pg);
       Seg sg;
-      for (; ok && seg_next(g, it, sg); ++seg_idx) {
+      for (; ok && seg_next(pg, it, sg); ++seg_idx) {
         const int ab = seg_idx & 1;
         if (!mbar_wait_warp(acce_bar(ab), (uint32_t)(((seg_idx >> 1) & 1) ^ 1), abort_flag)) { ok = false; break; }
         tc_fence_after();                                // the epilogue's tcgen05.ld of this accumulator come first
@@ -1636,13 +1722,13 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
     WorkerCtx w;
     w.tmem_base = tmem_base; w.accf_bar0 = accf_bar(0); w.acce_bar0 = acce_bar(0);
     w.abort_flag = abort_flag; w.wait_ok = wait_ok; w.staging = staging;
-    w.row_pos_sh = row_pos_sh; w.row_pg_sh = row_pg_sh; w.layers_sh = layers_sh;
+    w.row_pos_sh = row_pos_sh; w.row_pg_sh = row_pg_sh; w.geom = geom_sh;
     w.rope_cos_sh = rope_cos_sh; w.rope_sin_sh = rope_sin_sh;
     w.wt = wt; w.lane = lane; w.q = q; w.G = G; w.c = c; w.seg_idx = 0;
 
     // ---- phase program
     if (HSD_PROF(a) && wt == 0) a.prof[(size_t)blockIdx.x * kFwdProfEvents] = globaltimer_ns();
-    for (int l = wt; l < a.n_run; l += 256) layers_sh[l] = a.layers[l];
+    for (int l = wt; l < a.n_run; l += 256) { norms_sh[l].attn = a.layers[l].attn_norm; norms_sh[l].mlp = a.layers[l].mlp_norm; }
     if (a.R <= kRopeCacheRows)
       for (int i = wt; i < a.R * (HD / 2); i += 256) {
         const int r = i / (HD / 2), k = i % (HD / 2);
@@ -1661,53 +1747,53 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
       int4 fi = make_int4(0, 0, 0, 0);
       if ((int)blockIdx.x < n_work) fi = a.attn_items[blockIdx.x / (a.n_splits * a.nkv)];
       first_item_sh[0] = fi.x; first_item_sh[1] = fi.y; first_item_sh[2] = fi.z; first_item_sh[3] = fi.w;
-      const Gemm gq = make_gemm(a, 0);
-      const SplitGeom geo = split_geom(gq, G);
-      qkv_geom_sh[0] = (gq.seg_n[0] + kTcBlockM - 1) / kTcBlockM;
-      qkv_geom_sh[1] = qkv_geom_sh[0] + (gq.seg_n[1] + kTcBlockM - 1) / kTcBlockM;
-      qkv_geom_sh[2] = geo.parts; qkv_geom_sh[3] = geo.pieces_max; qkv_geom_sh[4] = geo.U; qkv_geom_sh[5] = geo.Gp; qkv_geom_sh[6] = gq.KB;
-      const Gemm gdn = make_gemm(a, 3);
-      const SplitGeom geo_gu = split_geom(make_gemm(a, 2), G);
-      const SegIter itd = seg_begin(gdn, G, c);
-      bgeom_sh[0] = itd.kb; bgeom_sh[1] = itd.left; bgeom_sh[2] = geo_gu.parts; bgeom_sh[3] = geo_gu.pieces_max;
+      const PhaseGeom &pq = geom_sh[0];
+      qkv_geom_sh[0] = (a.nq * a.hd + kTcBlockM - 1) / kTcBlockM;
+      qkv_geom_sh[1] = qkv_geom_sh[0] + (a.nkv * a.hd + kTcBlockM - 1) / kTcBlockM;
+      qkv_geom_sh[2] = pq.parts; qkv_geom_sh[3] = pq.pieces_max; qkv_geom_sh[4] = pq.U; qkv_geom_sh[5] = pq.Gp; qkv_geom_sh[6] = pq.KB;
     }
     // One step loop, one call site per phase body: the whole per-layer program has to stay resident in
     // the instruction cache (every phase runs once per layer, so code that does not fit is fetched
     // cold through the saturated memory system every single time).
-    //   t = 0                embed + norm                                  -> ready(QKV 0)
-    //   t = 1 + 10 l + s     s: 0 QKV pieces | 1 QKV finish | 2 attention tiles | 3 attention merge -> ready(O)
-    //                           4 O pieces | 5 norm (+O pieces) -> ready(gate/up) | 6 gate/up pieces
-    //                           7 gate/up finish -> ready(down) | 8 down pieces | 9 norm (+down pieces) -> ready(next)
+    //   t = 0                embed + norm, barrier                         -> ready(QKV 0)
+    //   t = 1 + 10 l + s     s: 0 QKV pieces | 1 QKV finish, barrier | 2 attention tiles | 3 attention merge, barrier -> ready(O)
+    //                           4 O pieces | 5 norm (+O pieces), barrier -> ready(gate/up) | 6 gate/up pieces
+    //                           7 gate/up finish, barrier -> ready(down) | 8 down pieces | 9 norm (+down pieces), barrier -> ready(next)
     //   t = 1 + 10 n, + 1    output-head pieces | output-head finish
-    // Steps 1 and 7 are empty (no barrier) when the finish is folded into the phase after it.
+    // Steps 1 and 7 are empty when the finish is folded into the phase after it.  A phase that reads the words of the one
+    // before waits for those words, so there is a grid barrier only before a projection that takes its activations by TMA:
+    // three per layer (five with both finish phases).  Words become holes again under a later projection, behind a barrier
+    // after their last reader and in front of one before their next: QKV, partials and O under gate / up, down under the next
+    // QKV or the head, and so gate / up if folded (otherwise under down).
     const int n_steps = 1 + 10 * a.n_run + (a.L > 0 ? 2 : 0);
     enum { K_EPI, K_FIN, K_ATTN_A, K_ATTN_B, K_NORM, K_NONE };
-    // CTAs with pieces of the two residual projections; pieces stored so far (what the early norm waits for)
-    const unsigned add_ctas_o = (unsigned)min(G, split_geom(make_gemm(a, 1), G).Gp), add_ctas_d = (unsigned)min(G, split_geom(make_gemm(a, 3), G).Gp);
-    unsigned pieces_target = 0u;
 #pragma unroll 1
     for (int t = 0; t < n_steps && alive; ++t) {
       int kind, gp = 0, ready = -1, l = 0;
       bool barrier = true;
       if (t == 0) { kind = K_NORM; ready = 0; }
-      else if (t > 10 * a.n_run) { gp = 4 * a.n_run; kind = (t == 1 + 10 * a.n_run) ? K_EPI : K_FIN; barrier = (kind == K_EPI); }
+      else if (t > 10 * a.n_run) { gp = 4 * a.n_run; kind = (t == 1 + 10 * a.n_run) ? K_EPI : K_FIN; barrier = false; }
       else {
         l = (t - 1) / 10;
         const int sstep = (t - 1) % 10, p = 4 * l;
         switch (sstep) {
-          case 0: kind = K_EPI; gp = p; break;
+          case 0: kind = K_EPI; gp = p; barrier = false; break;
           case 1:                                            // folded into the attention phase when every item stands alone
             if (a.fuse_qkv) { kind = K_NONE; barrier = false; }
             else { kind = K_FIN; gp = p; }
             break;
-          case 2: kind = K_ATTN_A; if (a.n_splits == 1) ready = p + 1; break;       // a single key split needs no merge phase
+          case 2:
+            kind = K_ATTN_A;
+            if (a.n_splits == 1) ready = p + 1;                 // a single key split needs no merge phase
+            else barrier = false;
+            break;
           case 3:
             if (a.n_splits == 1) { kind = K_NONE; barrier = false; }
             else { kind = K_ATTN_B; ready = p + 1; }
             break;
           case 4: kind = K_EPI; gp = p + 1; barrier = !a.early_norm; break;
           case 5: kind = K_NORM; gp = p + 1; ready = p + 2; break;
-          case 6: kind = K_EPI; gp = p + 2; if (a.fuse_gu) ready = p + 3; break;
+          case 6: kind = K_EPI; gp = p + 2; barrier = false; break;
           case 7:                                            // folded into the down projection in passes with few rows
             if (a.fuse_gu) { kind = K_NONE; barrier = false; }
             else { kind = K_FIN; gp = p + 2; ready = p + 3; }
@@ -1722,31 +1808,47 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
       switch (kind) {
         case K_EPI:
           if (built_down(a, gp)) {
-            if (a.gu_pieces_max <= 2) build_act_stages<NPAD, 2, 2>(a, w, gp, ring, full_bar(0), empty_bar(0), ring_pos_sh, bgeom_sh);
-            else build_act_stages<NPAD, 4, 1>(a, w, gp, ring, full_bar(0), empty_bar(0), ring_pos_sh, bgeom_sh);
+            if (a.gu_pieces_max <= 2) build_act_stages<NPAD, 2, 2>(a, w, gp, ring, full_bar(0), empty_bar(0), ring_pos_sh);
+            else build_act_stages<NPAD, 4, 1>(a, w, gp, ring, full_bar(0), empty_bar(0), ring_pos_sh);
           }
           if (is_epi) gemm_epilogue<NPAD>(a, w, gp);
+          else {
+            const int kind = kind_of(a, gp);
+            if (kind == 2) {
+              put_holes<NPAD>(a, w, 0);
+              put_holes<NPAD>(a, w, 1);
+              if (a.n_splits > 1) put_partial_holes<HD>(a, wt, first_item_sh);
+            } else if (kind == 3 ? !a.fuse_gu : (kind == 0 || kind == 4) && gp > 0) {
+              if (kind != 3) put_holes<NPAD>(a, w, 3);
+              if (kind == 3 || a.fuse_gu) put_holes<NPAD>(a, w, 2);
+            }
+          }
+          // (a built down projection takes nothing by TMA but its weights: the activation producer only counts slots)
+          if (a.fuse_gu && gp < 4 * a.n_run && (gp & 3) == 2 && wt == 0) mbar_arrive(ready_bar((gp + 1) & 1));
           break;
         case K_FIN: gemm_finish<NPAD>(a, w, gp); break;
         case K_ATTN_A:
-          attn_tiles_phase<NPAD, HD, TC>(a, layers_sh[l], scratch, pcache, wt, dbg_cy, first_item_sh, qkv_geom_sh, row_pg_sh, rope_cos_sh, rope_sin_sh,
+          attn_tiles_phase<NPAD, HD, TC>(a, layer_of(a, l), scratch, pcache, wt, dbg_cy, first_item_sh, qkv_geom_sh, row_pg_sh, rope_cos_sh, rope_sin_sh,
                                      ring, tmem_base, abort_flag);
           if (TC) {                                               // the ring's memory is the weight producer's again
             worker_sync();
             if (wt == 0) mbar_arrive(attn_done_bar);
           }
           break;
-        case K_ATTN_B: attn_merge_phase<HD>(a, row_pos_sh, wt); break;
+        case K_ATTN_B: attn_merge_phase<HD>(a, row_pos_sh, wt, abort_flag); break;
         case K_NORM: {
           const bool first = (t == 0);
           const bool last = !first && (((t - 1) % 10) == 9) && (l + 1 >= a.n_run);      // final norm over the logit rows
           const bool mid = !first && (((t - 1) % 10) == 5);
-          const Gemm pend = make_gemm(a, first ? 0 : gp);
           const __nv_bfloat16 *gain = first ? a.layers[0].attn_norm
-                                            : (last ? a.final_norm : (mid ? layers_sh[l].mlp_norm : layers_sh[l + 1].attn_norm));
-          if (!first && a.early_norm) pieces_target += mid ? add_ctas_o : add_ctas_d;
-          alive = norm_phase<NPAD>(a, last ? a.L : a.R, last ? a.lrow_src : nullptr, first, first ? nullptr : &pend, pieces_of(a, gp), gain,
-                                   last ? a.hf : a.h, red, wt, (!first && a.early_norm) ? pieces_target : 0u, abort_flag);
+                                            : (last ? a.final_norm : (mid ? norms_sh[l].mlp : norms_sh[l + 1].attn));
+          auto norm = [&](auto slots) {
+            norm_phase<NPAD, decltype(slots)::value>(a, last ? a.L : a.R, last ? a.lrow_src : nullptr, first,
+                                                     first ? nullptr : a.pieces[gp & 3], geom_sh[gp & 3].pieces_max, gain, last ? a.hf : a.h,
+                                                     red, wt, abort_flag);
+          };
+          if (a.d <= 2048) norm(std::integral_constant<int, 2>{});
+          else norm(std::integral_constant<int, 4>{});
           break;
         }
         default: break;
@@ -1827,6 +1929,30 @@ int launch_hd(const FwdArgs &args, int npad, int sm_count, cudaStream_t s) {
 
 }  // namespace
 
+namespace {
+// Piece buffers of the five kinds of projections (QKV, O, gate / up, down, head), one after the other; offsets in floats.
+struct PieceLayout { size_t off[5], total; int gu_pieces_max; };
+PieceLayout piece_layout(int d, int nqd, int nkvd, int ff, int V, int npad, int G) {
+  auto tiles = [](int n) { return (n + kTcBlockM - 1) / kTcBlockM; };
+  const int n_tiles[5] = {tiles(nqd) + 2 * tiles(nkvd), tiles(d), (ff + kTcBoxRows - 1) / kTcBoxRows, tiles(d), tiles(V)};
+  const int K[5] = {d, nqd, d, ff, d};
+  PieceLayout pl;
+  pl.total = 0;
+  for (int g = 0; g < 5; ++g) {
+    const SplitGeom sg = split_geom(n_tiles[g], K[g] / kTcBlockK, g == 1 || g == 3 ? residual_parts(d) : 4, G);
+    if (g == 2) pl.gu_pieces_max = sg.pieces_max;
+    pl.off[g] = pl.total;
+    pl.total += (size_t)n_tiles[g] * sg.pieces_max * npad * kTcBlockM;
+  }
+  return pl;
+}
+}  // namespace
+
+size_t fwd_pieces_bytes(int d, int nqd, int nkvd, int ff, int V, int sm_count) {
+  if (d < kTcBlockK || nqd < kTcBlockK || ff < kTcBlockK) return 0;
+  return piece_layout(d, nqd, nkvd, ff, V, 128, sm_count).total * 4;
+}
+
 int launch_attention_tiles(const FwdArgs &args, __nv_bfloat16 *k_pool, __nv_bfloat16 *v_pool, int sm_count, cudaStream_t s) {
   if (args.fuse_qkv || args.n_splits != 1 || args.n_attn < 1) return HSD_E_INVALID_ARG;
   switch (args.hd) {
@@ -1852,21 +1978,12 @@ int launch_forward_persistent(const FwdArgs &args, int npad, int sm_count, cudaS
   }
   if (args.tc_attn && (args.hd != 128 || args.fuse_qkv)) return HSD_E_INVALID_ARG;
   FwdArgs a = args;
-  {  // pieces per gate / up tile (the device's split_geom, for a grid of sm_count CTAs)
-    const int n_tiles = (a.ff + kTcBoxRows - 1) / kTcBoxRows, KB = a.d / kTcBlockK;
-    if (n_tiles * 2 <= sm_count) a.gu_pieces_max = std::min(std::min(4, sm_count / n_tiles), KB);
-    else {
-      const int U = n_tiles * KB, Gp = std::min(sm_count, U), per = U / Gp;
-      a.gu_pieces_max = (KB + per - 1) / per + 1;
-    }
-    if (a.gu_pieces_max > 4) a.fuse_gu = 0;
-  }
-  {  // CTAs without a tile of the residual projections (the device's split_geom): enough of them for every row?
-    const int n_tiles = (a.d + kTcBlockM - 1) / kTcBlockM;
-    int idle = 0;
-    if (n_tiles * 2 <= sm_count) idle = sm_count - n_tiles * std::min(4, sm_count / n_tiles);   // >= the device's count of idle CTAs
-    a.early_norm = (a.early_norm && a.R <= idle && a.L <= idle) ? 1 : 0;
-  }
+  const PieceLayout pl = piece_layout(a.d, a.nq * a.hd, a.nkv * a.hd, a.ff, a.V, npad, sm_count);
+  if (pl.total * 4 > args.pieces_bytes) return HSD_E_WORKSPACE_TOO_SMALL;
+  for (int g = 0; g < 5; ++g) a.pieces[g] = args.pieces[0] + pl.off[g];
+  a.gu_pieces_max = pl.gu_pieces_max;
+  // (a pass without logits ends with the last down projection, after which no phase could make gate / up's words holes)
+  if (a.gu_pieces_max > 4 || a.L == 0) a.fuse_gu = 0;
   switch (a.hd) {
     case 128: return a.tc_attn ? launch_hd<128, true>(a, npad, sm_count, s) : launch_hd<128, false>(a, npad, sm_count, s);
     case 64: return launch_hd<64, false>(a, npad, sm_count, s);

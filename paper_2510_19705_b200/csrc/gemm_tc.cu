@@ -429,21 +429,6 @@ int tc_make_map(CUtensorMap *map, const void *base, long long rows, long long co
 
 int tc_npad(int rows) { return rows <= 16 ? 16 : rows <= 32 ? 32 : rows <= 64 ? 64 : rows <= 128 ? 128 : 256; }
 
-TcGemmPlan tc_plan(const int *seg_n, int n_segs, int mode, int K, int npad, int sm_count) {
-  TcGemmPlan p;
-  p.kb = K / kTcBlockK;
-  p.n_tiles = 0;
-  if (mode == GEMM_SWIGLU_T) p.n_tiles = (seg_n[0] + kTcBoxRows - 1) / kTcBoxRows;
-  else
-    for (int s = 0; s < n_segs; ++s) p.n_tiles += (seg_n[s] + kTcBlockM - 1) / kTcBlockM;
-  long long U = (long long)p.n_tiles * p.kb;
-  p.grid = (int)std::min<long long>(sm_count, U);
-  long long per = U / p.grid;                     // every CTA gets at least this many k-blocks
-  p.pieces_max = (int)((p.kb + per - 1) / per) + 1;
-  p.scratch_bytes = (size_t)p.n_tiles * p.pieces_max * npad * kTcBlockM * 4 + (size_t)p.n_tiles * 4 + 256;
-  return p;
-}
-
 // Rows of a tile of one matrix on its own: 128, or as many fewer as spread the rows evenly over the rounds the SMs need.
 int tc_tile_rows(int N, int sm_count) {
   if (ceil_div(N, kTcBlockM) * 2 <= sm_count) return kTcBlockM;       // k-blocks are divided: full tiles

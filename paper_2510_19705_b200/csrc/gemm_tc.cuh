@@ -18,12 +18,6 @@ int tc_init();                     // HSD_OK when the tensor-map encoder is avai
 // 2-D bf16 tensor map over a row-major [rows, cols] matrix, box = [box_rows, 64], 128-byte swizzle.
 int tc_make_map(CUtensorMap *map, const void *base, long long rows, long long cols, int box_rows);
 
-// Split of a projection's (tile, k-block) units over the CTAs of the one-launch forward, and the scratch its pieces take.
-struct TcGemmPlan {
-  int n_tiles, kb, grid, pieces_max;
-  size_t scratch_bytes;
-};
-TcGemmPlan tc_plan(const int *seg_n, int n_segs, int mode, int K, int npad, int sm_count);
 int tc_npad(int rows);             // 16, 32, 64, 128 or 256 (rows <= 256)
 
 // Where the q / k / v projection's rows go (GEMM_QKV_T): q rotated -> q; k rotated, v -> their cache pages.

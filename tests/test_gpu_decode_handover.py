@@ -1,0 +1,41 @@
+"""The one-launch forward hands partial sums to the next phase as words that are "not written" until they are: every
+launch has to leave all of them unwritten again, whatever its rows, its phases and the calls before it."""
+import pytest
+import torch
+
+from paper_2510_19705_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+# residual projections cut into 8 parts (width 256, 2048) and 4 (2304); gate / up in equal parts and dealt out
+@pytest.mark.parametrize("d_model,nq,nkv,hd,ff", [(256, 8, 2, 32, 704), (2048, 32, 8, 64, 5632), (2304, 18, 3, 128, 1472)])
+def test_calls_do_not_depend_on_the_calls_before(lib, d_model, nq, nkv, hd, ff):
+    cfg = inputs.model_cfg(3, d_model, nq, nkv, ff, 2000, "bf16", head_dim=hd)
+    w = inputs.make_weights(cfg, 5, device="cuda")
+    tokens = inputs.make_prompts(cfg["vocab"], 1, 40, 9)[0].cuda().contiguous()
+
+    def engine(folded=True):
+        eng = lib.Hsd(cfg, w, (1, 3), (2,), max_batch=6, max_seq=160)
+        if not folded:
+            eng.set_phase_folding(False, False, False)
+        return eng
+
+    def call(eng, kind, n, batch):
+        if kind == "layers":
+            return [eng.layer_logits(tokens[:n], [1, 3])]
+        toks, stats, _ = eng.generate(inputs.make_prompts(cfg["vocab"], batch, n, n).cuda(), 24, n)
+        return [toks, torch.tensor([[s[k] for k in ("calls", "rows", "accepted", "emitted")] for s in stats])]
+
+    # prompts of up to four tokens are a pass without logits of at most three rows; six sequences have more rows than fold
+    calls = [("gen", 24, 1), ("gen", 3, 1), ("layers", 40, 1), ("gen", 100, 6), ("gen", 2, 6), ("layers", 1, 1), ("gen", 24, 1), ("gen", 17, 3)]
+    used, separate = engine(), engine(folded=False)
+    for c in calls:
+        alone = engine()
+        want = call(alone, *c)
+        for eng in (used, separate):
+            for a, b in zip(call(eng, *c), want):
+                assert torch.equal(a, b), c
+        alone.close()
+    used.close()
+    separate.close()
