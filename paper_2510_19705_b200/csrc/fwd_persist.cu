@@ -119,8 +119,10 @@ struct SegIter { int tile, kb, left; };        // next k-block (tile, kb) and th
 // tile, residual projections residual_parts(), so the consumer can fetch all of them in one batch); otherwise the (tile, k-block) units are
 // dealt out evenly (tiles >= CTAs / 2: a tile then spans at most 3 CTAs).
 struct SplitGeom { int U, Gp, pieces_max, parts; };
-// The norm after a residual projection loads a row's pieces in one batch: four of up to 4096 columns.
-__host__ __device__ __forceinline__ int residual_parts(int) { return 4; }
+// The norm after a residual projection holds a row in registers, 16 float4 loads of pieces per thread at a time: 4 pieces
+// of up to 4096 columns or 8 of up to 2048.  Width 2048 in 4 parts left 84 of 148 CTAs without a tile of O and down
+// and put 22 k-blocks of down on each other one: 1B hierarchy, target pass 0.552 ms in 4 parts, 0.518 in 8.
+__host__ __device__ __forceinline__ int residual_parts(int d) { return d <= 2048 ? 8 : 4; }
 __host__ __device__ __forceinline__ SplitGeom split_geom(int n_tiles, int KB, int most, int G) {
   SplitGeom sg;
   sg.U = n_tiles * KB;
