@@ -101,6 +101,8 @@ __global__ void __launch_bounds__(kThreads, 1) prompt_attn_kernel(const __grid_c
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == kMmaWarp) tmem_alloc(smem_u32(&tmem_slot), 512);
+  chain_next();
+  chain_wait();
   if (warp < kLoaderWarp) {
     // Q: thread = query vector; K-major, 128-byte swizzle; vectors past the tile's tokens are zero
     const int x = warp >> 2, row = (warp & 3) * 32 + lane, tok = row / group, g = row - tok * group;
@@ -329,7 +331,7 @@ int launch_t(const PromptAttnArgs &a, cudaStream_t s) {
   static std::atomic<u64> limits{0};
   const int limit = hsd_smem_limit((const void *)prompt_attn_kernel<HD>, Cfg<HD>::kSmem, limits);
   if (limit) return limit;
-  prompt_attn_kernel<HD><<<a.n_items * a.nkv, kThreads, Cfg<HD>::kSmem, s>>>(a);
+  HSD_CUDA_OK(hsd_launch(prompt_attn_kernel<HD>, a.n_items * a.nkv, kThreads, Cfg<HD>::kSmem, s, 0, a.chained, a));
   hsd_count_launches(1);
   return hsd_launch_status();
 }

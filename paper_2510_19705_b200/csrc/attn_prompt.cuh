@@ -14,6 +14,7 @@ struct PromptAttnArgs {
   const int *page_table;
   int nq, nkv, hd, page_shift, pages_per_seq, n_pages;
   int *status;                       // set non-zero if a bounded wait gave up
+  bool chained;                      // part of a chain of kernels (common.cuh)
 };
 
 // tokens of one 128-row query tile: the heads of a KV group sit side by side in it

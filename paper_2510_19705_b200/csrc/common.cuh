@@ -35,6 +35,33 @@ static inline int hsd_smem_limit(const void *kernel, int bytes, std::atomic<u64>
   return HSD_OK;
 }
 
+// A chain of kernels on one stream, each of which may start (and prepare: barriers, tensor memory, the first weights) while
+// the one before it still runs.  Every CTA of such a kernel calls chain_wait() before it touches anything the kernels
+// before it read or wrote: it returns when the one before is complete, which had waited in the same way.  chain_next()
+// lets the next kernel's CTAs come as SMs become free.  A chain begins with a launch of the ordinary kind; in one, both
+// do nothing.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... KA, class... A>
+static inline cudaError_t hsd_launch(void (*kernel)(KA...), int grid, int threads, size_t smem, cudaStream_t s, int cluster, bool chained, A &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (cluster > 0) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = cluster; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (chained) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = at; cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
+}
+
 // SMs of the GPU that measured lines (path choices, unit sizes) refer to; launches ask the device.
 constexpr int kMeasuredSMs = 148;
 

@@ -343,6 +343,7 @@ int gemm(hsd_ctx *c, Model &M, int abuf, const void *A, int R, int K, const Gemm
   a.ldo = (mode == GEMM_SWIGLU_T) ? segs.n[0] : total;
   a.status = (int *)(c->ws + c->status_off);
   a.stream_weights = 1;
+  a.chained = true;                             // (the calls of gemm() follow kernels of their own call)
   if (qkv) a.qkv = *qkv;
   for (int r0 = 0; r0 < R; r0 += 256) {
     a.R = std::min(256, R - r0);
@@ -715,12 +716,14 @@ int forward_prompt(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
   g.q = c->dev<__nv_bfloat16>(ML.q);
   g.nq = md.nq; g.nkv = md.nkv; g.hd = md.hd; g.page = md.page; g.pages_per_seq = md.pages_per_seq; g.n_pages = md.n_pages;
   g.status = (int *)(c->ws + c->status_off);
+  g.chained = true;                             // the kernels after the embedding are a chain
   PromptAttnArgs pa = {};
   pa.q = g.q; pa.att = c->dev<__nv_bfloat16>(ML.att);
   pa.items = (const int4 *)(devp + o_items); pa.n_items = n_items; pa.page_table = g.page_table;
   pa.nq = md.nq; pa.nkv = md.nkv; pa.hd = md.hd; pa.pages_per_seq = md.pages_per_seq; pa.n_pages = md.n_pages;
   while ((1 << pa.page_shift) < md.page) ++pa.page_shift;
   pa.status = g.status;
+  pa.chained = true;
   auto product = [&](int abuf, int K, int wmap0, int n_maps, int mode, int n, void *out, int ldo) {
     g.a = M.amaps[abuf][3];
     for (int i = 0; i < n_maps; ++i) g.w[i] = M.wmaps[(size_t)wmap0 + i];
@@ -733,7 +736,7 @@ int forward_prompt(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
   for (int l = 0; l < n_run; ++l) {
     const void *const *w = &M.lw[(size_t)l * 9];
     const bool last = l == n_run - 1;
-    HSD_TRY(launch_rmsnorm(md, x, w[0], nullptr, R, h, s));
+    HSD_TRY(launch_rmsnorm(md, x, w[0], nullptr, R, h, s, true));
     g.k_pool = (__nv_bfloat16 *)(c->ws + ML.k_pool + ML.pool_layer_stride * l);
     g.v_pool = (__nv_bfloat16 *)(c->ws + ML.v_pool + ML.pool_layer_stride * l);
     g.seg_n[1] = g.seg_n[2] = nkvd;
@@ -743,7 +746,7 @@ int forward_prompt(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     pa.k = M.kvmaps[2 * l]; pa.v = M.kvmaps[2 * l + 1];
     HSD_TRY(launch_prompt_attention(pa, s));
     HSD_TRY(product(1, nqd, l * 7 + 3, 1, BIG_ADD_F32, md.d, x, md.d));
-    HSD_TRY(launch_rmsnorm(md, x, w[5], nullptr, R, h, s));
+    HSD_TRY(launch_rmsnorm(md, x, w[5], nullptr, R, h, s, true));
     HSD_TRY(product(0, md.d, l * 7 + 4, 2, BIG_SWIGLU, md.ff, c->dev<void>(ML.act), md.ff));
     HSD_TRY(product(2, md.ff, l * 7 + 6, 1, BIG_ADD_F32, md.d, x, md.d));
   }
@@ -1273,6 +1276,7 @@ static int layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, cons
   pa.nq = md.nq; pa.nkv = md.nkv; pa.hd = md.hd; pa.pages_per_seq = md.pages_per_seq; pa.n_pages = md.n_pages;
   while ((1 << pa.page_shift) < md.page) ++pa.page_shift;
   pa.status = (int *)(c->ws + c->status_off);
+  pa.chained = true;                            // with tensor cores the kernels after the embedding are a chain
   char *rows_buf = c->dev<char>(ML.partials);
   const size_t row_bytes = (size_t)md.d * es, rows_cap = (size_t)ML.partial_rows * md.nq * (md.hd + 2) * 4 / row_bytes;
   const int layers_cap = tm ? (int)std::min<size_t>(rows_cap / R, (size_t)n_layers_sel) : 0;     // layers whose rows fit the buffer
@@ -1283,7 +1287,7 @@ static int layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, cons
     void *out = (char *)out_logits + (size_t)(next - held) * R * md.V * es;
     BigGemmArgs g = {};
     g.R = held * R; g.K = md.d; g.mode = BIG_LOGITS; g.seg_n[0] = md.V; g.ldo = md.V;
-    g.out_bf16 = (__nv_bfloat16 *)out; g.status = pa.status;
+    g.out_bf16 = (__nv_bfloat16 *)out; g.status = pa.status; g.chained = true;
     g.w[0] = M.wmaps[(size_t)md.n_layers * 7 + kHeadMaps - 1];
     held = 0;
     int st = tc_make_map(&g.a, rows_buf, g.R, md.d, kBigBoxRowsA);
@@ -1293,7 +1297,7 @@ static int layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, cons
   for (int l = 0; l < md.n_layers && next < n_layers_sel; ++l) {
     const void *const *w = &M.lw[(size_t)l * 9];
     void *kp = c->ws + ML.k_pool + ML.pool_layer_stride * l, *vp = c->ws + ML.v_pool + ML.pool_layer_stride * l;
-    HSD_TRY(launch_rmsnorm(md, x, w[0], nullptr, R, h, s));
+    HSD_TRY(launch_rmsnorm(md, x, w[0], nullptr, R, h, s, true));
     HSD_TRY(project_qkv(c, M, l, rb, h, qkv, pt, kp, vp, q));
     if (tm) {
       pa.k = M.kvmaps[2 * l]; pa.v = M.kvmaps[2 * l + 1];
@@ -1303,7 +1307,7 @@ static int layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, cons
     }
     GemmSegs o_segs = {{w[4], nullptr, nullptr}, {md.d, 0, 0}, 1};
     HSD_TRY(gemm(c, M, 1, att, R, md.nq * md.hd, o_segs, l * 7 + 3, GEMM_ADD_F32, x, nullptr, nullptr));
-    HSD_TRY(launch_rmsnorm(md, x, w[5], nullptr, R, h, s));
+    HSD_TRY(launch_rmsnorm(md, x, w[5], nullptr, R, h, s, true));
     GemmSegs gu_segs = {{w[6], w[7], nullptr}, {md.ff, md.ff, 0}, 2};
     HSD_TRY(gemm(c, M, 0, h, R, md.d, gu_segs, l * 7 + 4, GEMM_SWIGLU_T, nullptr, act, nullptr));
     GemmSegs d_segs = {{w[8], nullptr, nullptr}, {md.d, 0, 0}, 1};
@@ -1311,14 +1315,14 @@ static int layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, cons
     if (layers[next] != l + 1) continue;
     // exit after layer l + 1: shared final norm + head on every row
     if (layers_cap > 0) {
-      HSD_TRY(launch_rmsnorm(md, x, M.final_norm, rb.lrow_src, R, rows_buf + (size_t)held * R * row_bytes, s));
+      HSD_TRY(launch_rmsnorm(md, x, M.final_norm, rb.lrow_src, R, rows_buf + (size_t)held * R * row_bytes, s, true));
       ++next;
       if (++held == layers_cap || next == n_layers_sel) HSD_TRY(flush());
       continue;
     }
     // (the normalised rows go to the h buffer, free between two layers and large enough for every row; the
     // buffer of the generation path's final norm holds the few logit rows of a verification only)
-    HSD_TRY(launch_rmsnorm(md, x, M.final_norm, rb.lrow_src, R, h, s));
+    HSD_TRY(launch_rmsnorm(md, x, M.final_norm, rb.lrow_src, R, h, s, true));
     GemmSegs lm_segs = {{M.lm_head, nullptr, nullptr}, {md.V, 0, 0}, 1};
     HSD_TRY(gemm(c, M, 0, h, R, md.d, lm_segs, md.n_layers * 7 + kHeadMaps - 1, GEMM_STORE_T_SCATTER, nullptr,
                  (char *)out_logits + (size_t)next * R * md.V * es, rb.lrow_dst));

@@ -43,6 +43,14 @@ __global__ void __launch_bounds__(256) rmsnorm_vec_kernel(const float *__restric
                                                           const int *__restrict__ src, int d, float eps, __nv_bfloat16 *__restrict__ out) {
   __shared__ float sh[8];
   const int i = blockIdx.x, n4 = d >> 2;
+  uint2 graw[NV];
+#pragma unroll
+  for (int j = 0; j < NV; ++j) {
+    const int k = threadIdx.x + 256 * j;
+    graw[j] = k < n4 ? __ldg(reinterpret_cast<const uint2 *>(gain) + k) : make_uint2(0u, 0u);
+  }
+  chain_next();
+  chain_wait();
   const float4 *row = reinterpret_cast<const float4 *>(x + (size_t)(src ? src[i] : i) * d);
   float4 v[NV];
   float ss = 0.f;
@@ -64,9 +72,9 @@ __global__ void __launch_bounds__(256) rmsnorm_vec_kernel(const float *__restric
   for (int j = 0; j < NV; ++j) {
     const int k = threadIdx.x + 256 * j;
     if (k >= n4) continue;
-    const uint2 graw = __ldg(reinterpret_cast<const uint2 *>(gain) + k);
-    const __nv_bfloat162 a = __floats2bfloat162_rn(v[j].x * inv * __uint_as_float(graw.x << 16), v[j].y * inv * __uint_as_float(graw.x & 0xFFFF0000u));
-    const __nv_bfloat162 b = __floats2bfloat162_rn(v[j].z * inv * __uint_as_float(graw.y << 16), v[j].w * inv * __uint_as_float(graw.y & 0xFFFF0000u));
+    const uint2 g = graw[j];
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v[j].x * inv * __uint_as_float(g.x << 16), v[j].y * inv * __uint_as_float(g.x & 0xFFFF0000u));
+    const __nv_bfloat162 b = __floats2bfloat162_rn(v[j].z * inv * __uint_as_float(g.y << 16), v[j].w * inv * __uint_as_float(g.y & 0xFFFF0000u));
     reinterpret_cast<uint2 *>(out + (size_t)i * d)[k] = make_uint2(*reinterpret_cast<const unsigned *>(&a), *reinterpret_cast<const unsigned *>(&b));
   }
 }
@@ -415,16 +423,15 @@ int launch_embed(const ModelDims &md, const void *embed, const int *tokens, cons
   return hsd_launch_status();
 }
 
-int launch_rmsnorm(const ModelDims &md, const float *x, const void *gain, const int *src, int rows, void *out, cudaStream_t s) {
+int launch_rmsnorm(const ModelDims &md, const float *x, const void *gain, const int *src, int rows, void *out, cudaStream_t s, bool chained) {
   if (rows == 0) return HSD_OK;
   // the vector form wants 8-byte-aligned gains and rows it can hold: 2 / 4 / 8 float4 per thread
   const bool vec = md.dtype == HSD_BF16 && md.d % 4 == 0 && md.d <= 8192 && ((uintptr_t)gain & 7) == 0 && ((uintptr_t)out & 7) == 0 &&
                    ((uintptr_t)x & 15) == 0;
   if (vec) {
     const __nv_bfloat16 *g = (const __nv_bfloat16 *)gain;
-    if (md.d <= 2048) rmsnorm_vec_kernel<2><<<rows, 256, 0, s>>>(x, g, src, md.d, md.eps, (__nv_bfloat16 *)out);
-    else if (md.d <= 4096) rmsnorm_vec_kernel<4><<<rows, 256, 0, s>>>(x, g, src, md.d, md.eps, (__nv_bfloat16 *)out);
-    else rmsnorm_vec_kernel<8><<<rows, 256, 0, s>>>(x, g, src, md.d, md.eps, (__nv_bfloat16 *)out);
+    auto kernel = md.d <= 2048 ? rmsnorm_vec_kernel<2> : md.d <= 4096 ? rmsnorm_vec_kernel<4> : rmsnorm_vec_kernel<8>;
+    HSD_CUDA_OK(hsd_launch(kernel, rows, 256, 0, s, 0, chained, x, g, src, md.d, md.eps, (__nv_bfloat16 *)out));
   } else if (md.dtype == HSD_BF16)
     rmsnorm_kernel<__nv_bfloat16><<<rows, 256, 0, s>>>(x, (const __nv_bfloat16 *)gain, src, md.d, md.eps, (__nv_bfloat16 *)out);
   else

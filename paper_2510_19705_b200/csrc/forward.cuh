@@ -42,7 +42,7 @@ enum GemmMode { GEMM_STORE_F32 = 0, GEMM_ADD_F32 = 1, GEMM_STORE_T_SCATTER = 2, 
 
 int launch_embed(const ModelDims &md, const void *embed, const int *tokens, const RowBatch &rb, float *x, cudaStream_t s);
 // out[i, :] = T(rmsnorm(x[src ? src[i] : i, :]) * gain)
-int launch_rmsnorm(const ModelDims &md, const float *x, const void *gain, const int *src, int rows, void *out, cudaStream_t s);
+int launch_rmsnorm(const ModelDims &md, const float *x, const void *gain, const int *src, int rows, void *out, cudaStream_t s, bool chained = false);
 // SIMT GEMM: A [R, K] (storage type) times the segments' W^T, epilogue by mode.
 //   STORE_F32        out_f32[r, n] = acc                       (ldo = total N)
 //   ADD_F32          out_f32[r, n] += acc                      (residual stream)

@@ -112,6 +112,7 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+  chain_next();
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -139,15 +140,29 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
       const int mt = t % m_tiles, nt = t / m_tiles;
       const Half hf = half_of<MODE>(args, nt, (int)rank);
       const int arow = mt * kBM + (int)rank * 128;
-      for (int kb = 0; kb < KB; ++kb) {
+      auto load_w = [&](int kb, int slot) {
+        const uint32_t dst = s0 + (uint32_t)(slot * kStageBytes) + kABytes, bar = map_to_rank(full_bar(slot), 0);
+        if (rank == 0) mbar_expect_tx(full_bar(slot), 2 * kStageBytes);
+        tma_load_2d_pair(dst, &args.w[hf.seg], kb * kBK, hf.n0, bar);
+        tma_load_2d_pair(dst + kBBytes / 2, &args.w[hf.seg], kb * kBK, hf.n0 + 64, bar);
+      };
+      auto load_a = [&](int kb, int slot) {
+        tma_load_2d_pair(s0 + (uint32_t)(slot * kStageBytes), &args.a, kb * kBK, arow, map_to_rank(full_bar(slot), 0));
+      };
+      int kb = 0;
+      if (t == pair) {                               // the ring's first weights before the wait for the activations
+        kb = min(kStages, KB);
+        if (issuer)
+          for (int i = 0; i < kb; ++i) load_w(i, i);
+        chain_wait();
+        if (issuer)
+          for (int i = 0; i < kb; ++i) load_a(i, i);
+        s = kb;
+        if (s == kStages) { s = 0; ph ^= 1u; }
+      }
+      for (; kb < KB; ++kb) {
         if (!mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
-        if (issuer) {
-          const uint32_t dst = s0 + (uint32_t)(s * kStageBytes), bar = map_to_rank(full_bar(s), 0);
-          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * kStageBytes);
-          tma_load_2d_pair(dst, &args.a, kb * kBK, arow, bar);
-          tma_load_2d_pair(dst + kABytes, &args.w[hf.seg], kb * kBK, hf.n0, bar);
-          tma_load_2d_pair(dst + kABytes + kBBytes / 2, &args.w[hf.seg], kb * kBK, hf.n0 + 64, bar);
-        }
+        if (issuer) { load_a(kb, s); load_w(kb, s); }
         if (++s == kStages) { s = 0; ph ^= 1u; }
       }
     }
@@ -193,6 +208,7 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
     // ------------------------------------------------------------------ epilogue (warps 2..9): thread = token row and half
     // of the tile's columns
     const int q = warp & 3, hw = (warp - 2) >> 2;                       // TMEM lane quarter, column half
+    chain_wait();
     int ci = 0;
     bool ok = true;
     for (int t = pair; t < n_tiles; t += pairs) {
@@ -254,6 +270,7 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..5): thread = token row
     const int q = warp & 3, et = threadIdx.x - 64;
+    chain_wait();
     int ti = 0;
     for (int t = pair; t < n_tiles; t += pairs, ++ti) {
       const int ab = ti & 1;
@@ -375,7 +392,7 @@ int launch_t(const BigGemmArgs &a, int n_tiles, int m_tiles, int sm_count, cudaS
   const int limit = hsd_smem_limit((const void *)gemm_big_kernel<MODE, HD>, kSmemBytes, limits);
   if (limit) return limit;
   const int pairs = std::min(sm_count / 2, n_tiles), KB = a.K / kBK;
-  gemm_big_kernel<MODE, HD><<<2 * pairs, threads_of<MODE>(), kSmemBytes, s>>>(a, n_tiles, m_tiles, KB, chain_blocks(a, KB, sm_count));
+  HSD_CUDA_OK(hsd_launch(gemm_big_kernel<MODE, HD>, 2 * pairs, threads_of<MODE>(), kSmemBytes, s, 0, a.chained, a, n_tiles, m_tiles, KB, chain_blocks(a, KB, sm_count)));
   hsd_count_launches(1);
   return hsd_launch_status();
 }

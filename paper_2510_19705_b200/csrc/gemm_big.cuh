@@ -30,6 +30,7 @@ struct BigGemmArgs {
   __nv_bfloat16 *q, *k_pool, *v_pool;
   int nq, nkv, hd, page, pages_per_seq, n_pages;
   int *status;                         // set non-zero if a bounded wait gave up
+  bool chained;                        // part of a chain of kernels (common.cuh)
 };
 
 constexpr int kBigBoxRowsA = 128;
