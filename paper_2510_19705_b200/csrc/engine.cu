@@ -3,6 +3,7 @@
 // resample -> KV rollback), KV paging, workspace carving, statistics and the decision log.
 #include <stdio.h>
 #include <stdlib.h>
+#include <string.h>
 #include <math.h>
 #include <algorithm>
 #include <new>
@@ -33,7 +34,7 @@ constexpr int kPromptRows = 2304;              // rows of one prompt chunk on th
                                                //   which with 4096-wide outputs make 1.95 rounds of the 74 CTA pairs (eight make 1.73)
 constexpr uint32_t kTraceMagic = 0x48534454u;
 
-constexpr size_t kTcCtrlBytes = 256;            // the status word
+constexpr size_t kResultHead = 256;             // the block a decision's host wait copies: status word, then accepted counts
 constexpr int kHeadMaps = 17;                   // output-head tensor maps: one per level (<= 16), then the shared head
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -55,7 +56,7 @@ struct ModelLayout {
   int partial_rows;
 };
 struct Layout {
-  size_t tokens, page_table, vscratch, n_acc, ring, grid_counter, total;
+  size_t tokens, page_table, vscratch, result, ring, grid_counter, total;
   std::vector<size_t> logits;
   std::vector<int> slots;
   std::vector<ModelLayout> model;
@@ -141,10 +142,10 @@ Layout make_layout(const hsd_model_desc *models, int n_models, int n_levels, con
     L.max_logit_rows = std::max(L.max_logit_rows, B * L.slots[i]);
   }
   L.vscratch = take(verify_scratch_bytes(B, sumT + 1));
-  L.n_acc = take((size_t)B * 4);
-  // a slot holds one pass's descriptors: <= 40 bytes a row, or a prompt chunk's row lists (8 bytes a row) and one 16-byte
+  L.result = take(kResultHead + (size_t)B * 4);
+  // a slot holds one pass's descriptors (<= 40 bytes a row) and those of the decision after it, or a prompt chunk's row lists (8 bytes a row) and one 16-byte
   // item per 32 rows of a sequence (8 heads to a KV group, at most) and per sequence
-  L.ring_slot = align_up(std::max((size_t)L.base_rows * 40 + (size_t)B * 96, (size_t)L.max_rows * 8 + (size_t)(L.max_rows / 32 + B) * 16) + 1024, 256);
+  L.ring_slot = align_up(std::max((size_t)L.base_rows * 40 + (size_t)B * (96 + sizeof(VerifySeq)), (size_t)L.max_rows * 8 + (size_t)(L.max_rows / 32 + B) * 16) + 1024, 256);
   L.ring = take(L.ring_slot * kRingSlots);
   L.grid_counter = take(256);
   L.model.resize(n_models);
@@ -167,9 +168,9 @@ Layout make_layout(const hsd_model_desc *models, int n_models, int n_levels, con
     M.act = take((size_t)L.max_rows * m->d_ff * es);
     M.partials = take((size_t)M.partial_rows * nq * (hd + 2) * 4);
     M.hf = take((size_t)L.max_logit_rows * d * es);
-    // tensor-core scratch: [status word (256 bytes) | split pieces of the one-launch forward]
+    // split pieces of the one-launch forward
     M.tc_pieces_bytes = m->dtype == HSD_BF16 ? fwd_pieces_bytes(d, nq * hd, nkv * hd, m->d_ff, m->vocab, device_sm_count()) : 0;
-    M.tc_scratch = take(kTcCtrlBytes + M.tc_pieces_bytes);
+    M.tc_scratch = take(M.tc_pieces_bytes);
     M.wmaps_dev = take(((size_t)m->n_layers * 7 + kHeadMaps) * sizeof(CUtensorMap));
     M.layers_dev = take((size_t)m->n_layers * sizeof(FwdLayerDev));
     M.small_layers = take(m->dtype == HSD_F32 ? (size_t)m->n_layers * sizeof(SmallLayerDev) : 0);
@@ -184,6 +185,8 @@ struct SeqWork {
   int logit_first;       // first position whose output row is wanted (-1: none); rows up to end - 1
   int slot0;             // destination slot of that first row in the level's logits buffer
 };
+
+struct LogRecord { int level, b; uint32_t serial; int ctx, t, n, fwd_rows, logit_rows; long long logit_row0; const int *tokens; int n_tokens; };
 
 struct TimerPair { cudaEvent_t a, b; int level; };
 
@@ -217,7 +220,10 @@ struct hsd_ctx {
   char *ws;
   // pinned host mirrors
   char *ring_host;
-  int *n_acc_host;
+  int *result_host;                           // [kResultHead / 4 + max_batch]: status word, accepted counts
+  int *token_host;                            // decision log: tokens on their way, [3][max_batch][token_stride]
+  int token_stride;
+  std::vector<LogRecord> pending;             // level-0 records whose tokens have been asked for
   int *page_table_host;
   int ring_next, ring_in_flight;
   // per-sequence state
@@ -237,6 +243,7 @@ struct hsd_ctx {
   int trace_logit_calls, trace_records;
   cudaStream_t stream;
   uint64_t seed;
+  unsigned launch_parity = 0;                 // one-launch bf16 passes so far, modulo 2
   unsigned small_base = 0;                    // barrier arrivals of all one-launch fp32 passes so far
   bool any_tc = false;                        // some model runs kernels with bounded waits (their status word is polled)
   bool no_fuse_qkv = false;                   // keep the QKV finish phase in every pass (hsd_set_phase_folding)
@@ -247,7 +254,6 @@ struct hsd_ctx {
   int sm_count;
   std::vector<const void *> level_head, level_norm;   // output head and final norm gain of each level (the model's own unless set)
   std::vector<uint32_t> coin24;               // per level: kNoCoin, or the IID acceptance probability x 2^24 (ablation)
-  int *status_host;
   size_t status_off;                          // the one status word every tensor-core kernel of the context raises
 
   Model &model_of(int level) { return models[level_model[level]]; }
@@ -257,12 +263,14 @@ struct hsd_ctx {
 
 namespace {
 
-int sync_stream(hsd_ctx *c) {
-  if (c->any_tc &&
-      cudaMemcpyAsync(c->status_host, c->ws + c->status_off, 4, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
+// Waits for the stream; the status word and the first n_counts accepted counts come along.
+int sync_stream(hsd_ctx *c, int n_counts = 0) {
+  if ((c->any_tc || n_counts > 0) &&
+      cudaMemcpyAsync(c->result_host, c->ws + c->status_off, n_counts > 0 ? kResultHead + (size_t)n_counts * 4 : 4, cudaMemcpyDeviceToHost,
+                      c->stream) != cudaSuccess)
     return HSD_E_CUDA;
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) return HSD_E_CUDA;
-  if (c->any_tc && *c->status_host != 0) return HSD_E_DEVICE_TIMEOUT;
+  if (c->any_tc && *c->result_host != 0) return HSD_E_DEVICE_TIMEOUT;
   c->ring_in_flight = 0;
   for (int i = 0; i < c->timers_used; ++i) {
     float ms = 0.f;
@@ -373,8 +381,10 @@ int project_qkv(hsd_ctx *c, Model &M, int layer, const RowBatch &rb, const void 
 }
 
 // One forward pass of level `level` (layers 1..exit) over the given rows; logits of the wanted
-// rows go to the level's logits buffer.  KV of every processed position is (re)written.
-int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
+// rows go to the level's logits buffer.  KV of every processed position is (re)written.  `after`: descriptors of the
+// kernel that follows the pass, uploaded with its own (one copy for both); *after_dev = where they are.
+int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work, const void *after = nullptr, size_t after_bytes = 0,
+            const char **after_dev = nullptr) {
   Model &M = c->model_of(level);
   const ModelDims &md = M.md;
   const Layout &L = c->lay;
@@ -404,8 +414,12 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
   // slot layout: row_seq[R] | row_pos[R] | attn int4[n_attn] | lrow_src[n_logit] | lrow_dst int64[n_logit]
   size_t o_seq = 0, o_pos = align_up(o_seq + (size_t)R * 4, 16), o_attn = align_up(o_pos + (size_t)R * 4, 16),
          o_src = align_up(o_attn + (size_t)n_attn * 16, 16), o_dst = align_up(o_src + (size_t)n_logit * 4, 16),
-         bytes = o_dst + (size_t)n_logit * 8;
+         o_after = align_up(o_dst + (size_t)n_logit * 8, 16), bytes = o_after + after_bytes;
   if (bytes > L.ring_slot) return HSD_E_INVALID_ARG;
+  if (after_bytes) {
+    memcpy(host + o_after, after, after_bytes);
+    *after_dev = devp + o_after;
+  }
   int *row_seq = (int *)(host + o_seq), *row_pos = (int *)(host + o_pos), *lsrc = (int *)(host + o_src);
   int4 *attn = (int4 *)(host + o_attn);
   long long *ldst = (long long *)(host + o_dst);
@@ -544,8 +558,11 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     a.act = c->dev<__nv_bfloat16>(ML.act); a.hf = c->dev<__nv_bfloat16>(ML.hf);
     a.logits = (__nv_bfloat16 *)(c->ws + L.logits[level]);
     a.attn_partials = c->dev<float>(ML.partials);
-    a.pieces[0] = (float *)(c->ws + ML.tc_scratch + kTcCtrlBytes); a.pieces_bytes = ML.tc_pieces_bytes;
-    a.grid_counter = c->dev<unsigned>(L.grid_counter); a.status = (int *)(c->ws + c->status_off);
+    a.pieces[0] = (float *)(c->ws + ML.tc_scratch); a.pieces_bytes = ML.tc_pieces_bytes;
+    // two counters in turn: a launch clears the one the next launch uses
+    a.grid_counter = c->dev<unsigned>(L.grid_counter) + 16 * (c->launch_parity & 1);
+    a.next_counter = c->dev<unsigned>(L.grid_counter) + 16 * (~c->launch_parity & 1);
+    a.status = (int *)(c->ws + c->status_off);
     const int np = tc_npad(std::max(R, n_logit));
     const int pi = np == 16 ? 0 : np == 32 ? 1 : np == 64 ? 2 : 3;
     // few rows: fetch exactly the rows that exist (the MMA still reads `np` rows of the stage; the rest is stale
@@ -573,9 +590,9 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
       HSD_CUDA_OK(cudaMemsetAsync(a.prof, 0, (size_t)c->sm_count * kFwdProfEvents * 8, s));
     }
 #endif
-    HSD_CUDA_OK(cudaMemsetAsync(a.grid_counter, 0, 128, s));
     int stp = launch_forward_persistent(a, np, c->sm_count, s);
     if (stp) return stp;
+    c->launch_parity ^= 1;                      // (not launched: not cleared)
 #ifdef HSD_PROFILE
     if (prof) {
       std::vector<unsigned long long> ev((size_t)c->sm_count * kFwdProfEvents);
@@ -610,7 +627,7 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
     a.tokens = c->dev<int>(L.tokens); a.page_table = c->dev<int>(L.page_table);
     a.x = c->dev<float>(ML.x); a.q = c->dev<float>(ML.q); a.att = c->dev<float>(ML.att); a.act = c->dev<float>(ML.act);
     a.logits = (float *)(c->ws + L.logits[level]);
-    a.counter = c->dev<unsigned>(L.grid_counter) + 48;        // behind the words the bf16 forward clears
+    a.counter = c->dev<unsigned>(L.grid_counter) + 48;        // behind the bf16 forward's two
     a.status = (int *)(c->ws + c->status_off);
     for (int g = 0, l0 = 0; g * kSmallRows < R; l0 += a.L, ++g) {       // (a sequence's rows ascend: its earlier keys are there)
       a.R = std::min(kSmallRows, R - g * kSmallRows); a.L = group_logits[g];
@@ -756,22 +773,23 @@ int forward_prompt(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
 }
 
 // ---------------------------------------------------------------------------- decision log
-int fetch_tokens(hsd_ctx *c, int b, int pos0, int n, std::vector<int32_t> &out) {
-  size_t base = out.size();
-  out.resize(base + n);
+// Asks for n tokens of a sequence; they are at the address returned once the stream has been waited for.  Three places
+// per sequence: 0 = level 0's, 1 = a verification's drafts, 2 = the tokens after its decision.
+int ask_tokens(hsd_ctx *c, int place, int b, int pos0, int n, const int **at) {
+  int *host = c->token_host + ((size_t)place * c->max_batch + b) * c->token_stride;
+  *at = host;
+  if (n > c->token_stride) return HSD_E_INVALID_ARG;
   if (n == 0) return HSD_OK;
-  if (cudaMemcpyAsync(out.data() + base, c->dev<int>(c->lay.tokens) + (size_t)b * c->md.max_seq + pos0, (size_t)n * 4,
-                      cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
-    return HSD_E_CUDA;
-  return cudaStreamSynchronize(c->stream) == cudaSuccess ? HSD_OK : HSD_E_CUDA;
+  return cudaMemcpyAsync(host, c->dev<int>(c->lay.tokens) + (size_t)b * c->md.max_seq + pos0, (size_t)n * 4, cudaMemcpyDeviceToHost, c->stream) == cudaSuccess
+             ? HSD_OK : HSD_E_CUDA;
 }
 
-int trace_write(hsd_ctx *c, int level, int b, uint32_t serial, int ctx_len, int t, int n, int fwd_rows, int logit_rows,
-                long long logit_row0, const std::vector<int32_t> &toks) {
-  if (!c->trace) return HSD_OK;
+int trace_write(hsd_ctx *c, const LogRecord &r) {
   const ModelDims &md = c->md;
+  const int level = r.level, logit_rows = r.logit_rows;
+  const long long logit_row0 = r.logit_row0;
   int has_logits = c->trace_records < c->trace_logit_calls;
-  int32_t hdr[12] = {(int32_t)kTraceMagic, level, b, (int32_t)serial, ctx_len, t, n, fwd_rows, logit_rows, has_logits, md.V,
+  int32_t hdr[12] = {(int32_t)kTraceMagic, level, r.b, (int32_t)r.serial, r.ctx, r.t, r.n, r.fwd_rows, logit_rows, has_logits, md.V,
                      md.dtype};
   std::vector<char> rows;
   if (has_logits) {
@@ -782,9 +800,15 @@ int trace_write(hsd_ctx *c, int level, int b, uint32_t serial, int ctx_len, int 
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return HSD_E_CUDA;
   }
   if (fwrite(hdr, 4, 12, c->trace) != 12) return HSD_E_IO;
-  if (!toks.empty() && fwrite(toks.data(), 4, toks.size(), c->trace) != toks.size()) return HSD_E_IO;
+  if (r.n_tokens > 0 && fwrite(r.tokens, 4, r.n_tokens, c->trace) != (size_t)r.n_tokens) return HSD_E_IO;
   if (has_logits && fwrite(rows.data(), 1, rows.size(), c->trace) != rows.size()) return HSD_E_IO;
   c->trace_records++;
+  return HSD_OK;
+}
+// The pending records of level 0; the stream has been waited for since their tokens were asked for.
+int trace_pending(hsd_ctx *c) {
+  for (const LogRecord &r : c->pending) HSD_TRY(trace_write(c, r));
+  c->pending.clear();
   return HSD_OK;
 }
 
@@ -807,30 +831,32 @@ int run_level0(hsd_ctx *c, const std::vector<int> &act) {
       int start = std::min(c->len_g[b][0], len - 1);
       work.push_back({b, start, len, len - 1, j});
     }
-    HSD_TRY(forward(c, 0, work));
-    char *host, *devp;
-    HSD_TRY(ring_acquire(c, &host, &devp));
-    SampleRow *rows = (SampleRow *)host;
+    std::vector<SampleRow> rows(act.size());
     for (size_t i = 0; i < act.size(); ++i) {
       int b = act[i];
       rows[i].logit_row = (long long)b * L.slots[0] + j;
       rows[i].out_index = (long long)b * c->md.max_seq + c->buf_len[b];
       rows[i].j = j; rows[i].serial = ser[i]; rows[i].seq = b; rows[i].level = 0;
-      c->buf_len[b]++;
     }
-    HSD_CUDA_OK(cudaMemcpyAsync(devp, host, act.size() * sizeof(SampleRow), cudaMemcpyHostToDevice, c->stream));
-    HSD_TRY(launch_draft_sample(c->ws + L.logits[0], c->md.dtype, c->md.V, (const SampleRow *)devp, (int)act.size(), 1, 0,
+    const char *rows_dev = nullptr;
+    HSD_TRY(forward(c, 0, work, rows.data(), rows.size() * sizeof(SampleRow), &rows_dev));
+    for (int b : act) c->buf_len[b]++;
+    HSD_TRY(launch_draft_sample(c->ws + L.logits[0], c->md.dtype, c->md.V, (const SampleRow *)rows_dev, (int)act.size(), 1, 0,
                                 c->seed, c->dev<int>(L.tokens), c->stream));
   }
   for (size_t i = 0; i < act.size(); ++i) {
     hsd_level_stats &st = c->stats[0];
     st.calls++;
     st.emitted += steps;
-    if (c->trace) {
-      std::vector<int32_t> toks;
-      HSD_TRY(fetch_tokens(c, act[i], ctx0[i], steps, toks));
-      HSD_TRY(trace_write(c, 0, act[i], ser[i], ctx0[i], 0, steps, steps, steps, (long long)act[i] * L.slots[0], toks));
+    if (c->trace) {                             // written behind the wait of the verification that follows
+      LogRecord r = {0, act[i], ser[i], ctx0[i], 0, steps, steps, steps, (long long)act[i] * L.slots[0], nullptr, steps};
+      HSD_TRY(ask_tokens(c, 0, act[i], ctx0[i], steps, &r.tokens));
+      c->pending.push_back(r);
     }
+  }
+  if (c->trace && c->n_levels == 1) {
+    HSD_TRY(sync_stream(c));
+    HSD_TRY(trace_pending(c));
   }
   return HSD_OK;
 }
@@ -848,10 +874,7 @@ int run_verify(hsd_ctx *c, int level, const std::vector<int> &act, const std::ve
     work.push_back({b, start, c->buf_len[b], ctx[b] - 1, count[b]});
     t_max = std::max(t_max, t);
   }
-  HSD_TRY(forward(c, level, work));
-  char *host, *devp;
-  HSD_TRY(ring_acquire(c, &host, &devp));
-  VerifySeq *vs = (VerifySeq *)host;
+  std::vector<VerifySeq> vs(act.size());
   std::vector<uint32_t> ser(act.size());
   for (size_t i = 0; i < act.size(); ++i) {
     int b = act[i];
@@ -862,17 +885,21 @@ int run_verify(hsd_ctx *c, int level, const std::vector<int> &act, const std::ve
     vs[i].t = c->buf_len[b] - ctx[b];
     vs[i].serial = ser[i]; vs[i].seq = b; vs[i].level = level;
   }
-  HSD_CUDA_OK(cudaMemcpyAsync(devp, host, act.size() * sizeof(VerifySeq), cudaMemcpyHostToDevice, c->stream));
-  std::vector<std::vector<int32_t>> drafts(c->trace ? act.size() : 0);
-  for (size_t i = 0; i < drafts.size(); ++i) HSD_TRY(fetch_tokens(c, act[i], ctx[act[i]], c->buf_len[act[i]] - ctx[act[i]], drafts[i]));
+  const char *vs_dev = nullptr;
+  HSD_TRY(forward(c, level, work, vs.data(), vs.size() * sizeof(VerifySeq), &vs_dev));
+  std::vector<const int *> drafts(act.size()), after(act.size());
+  if (c->trace)                                 // (the decision writes its final token over one of the drafts)
+    for (size_t i = 0; i < act.size(); ++i) HSD_TRY(ask_tokens(c, 1, act[i], ctx[act[i]], vs[i].t, &drafts[i]));
   HSD_TRY(launch_verify(c->ws + L.logits[level], c->ws + L.logits[level - 1], c->dev<int>(L.tokens), c->md.dtype, c->md.V,
-                        (int)act.size(), t_max, (const VerifySeq *)devp, 0, 0, 0, c->ws + L.vscratch, c->seed, nullptr,
-                        c->dev<int>(L.n_acc), 1, c->stream, c->coin24[level]));
-  HSD_CUDA_OK(cudaMemcpyAsync(c->n_acc_host, c->dev<int>(L.n_acc), act.size() * 4, cudaMemcpyDeviceToHost, c->stream));
-  HSD_TRY(sync_stream(c));
+                        (int)act.size(), t_max, (const VerifySeq *)vs_dev, 0, 0, 0, c->ws + L.vscratch, c->seed, nullptr,
+                        c->dev<int>(L.result + kResultHead), 1, c->stream, c->coin24[level]));
+  if (c->trace)
+    for (size_t i = 0; i < act.size(); ++i) HSD_TRY(ask_tokens(c, 2, act[i], ctx[act[i]], vs[i].t + 1, &after[i]));
+  HSD_TRY(sync_stream(c, (int)act.size()));
+  if (c->trace) HSD_TRY(trace_pending(c));
   hsd_level_stats &st = c->stats[level];
   for (size_t i = 0; i < act.size(); ++i) {
-    int b = act[i], t = c->buf_len[b] - ctx[b], n = c->n_acc_host[i];
+    int b = act[i], t = c->buf_len[b] - ctx[b], n = c->result_host[kResultHead / 4 + i];
     if (n < 0 || n > t) return HSD_E_CUDA;
     // rollback / commit: the buffer keeps x_1..x_n and m; the position of m (and everything the
     // rejected drafts wrote) is valid in no layer group
@@ -885,9 +912,10 @@ int run_verify(hsd_ctx *c, int level, const std::vector<int> &act, const std::ve
     st.accepted += n;
     st.emitted += n + 1;
     if (c->trace) {
-      HSD_TRY(fetch_tokens(c, b, ctx[b] + n, 1, drafts[i]));          // the final token m
-      HSD_TRY(trace_write(c, level, b, ser[i], ctx[b], t, n, work[i].end - work[i].start, t + 1,
-                          (long long)b * L.slots[level] + count[b], drafts[i]));
+      std::vector<int> toks(drafts[i], drafts[i] + t);
+      toks.push_back(after[i][n]);                                    // the final token m
+      HSD_TRY(trace_write(c, LogRecord{level, b, ser[i], ctx[b], t, n, work[i].end - work[i].start, t + 1,
+                                       (long long)b * L.slots[level] + count[b], toks.data(), t + 1}));
     }
     count[b] += n + 1;
   }
@@ -1012,7 +1040,6 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
     for (int p = 0; p < 5 && !st; ++p) st = tc_make_map(&M.amaps[b][p], c->ws + abuf_off[b], arows[b], acols[b], npads[p]);
   for (int b = 0; b < 4 && !st; ++b)
     for (int r = 1; r <= 16 && !st; ++r) st = tc_make_map(&M.amaps_rows[b][r - 1], c->ws + abuf_off[b], arows[b], acols[b], r);
-  if (!st && cudaMemset(c->ws + ml.tc_scratch, 0, kTcCtrlBytes) != cudaSuccess) st = HSD_E_CUDA;
   if (st) return st;
   // tables of the persistent forward: tensor maps and per-layer pointers in device memory
   std::vector<FwdLayerDev> ld(md.n_layers);
@@ -1024,7 +1051,7 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
   }
   if (cudaMemcpy(c->ws + ml.wmaps_dev, M.wmaps.data(), M.wmaps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(c->ws + ml.layers_dev, ld.data(), ld.size() * sizeof(FwdLayerDev), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemset(c->ws + ml.tc_scratch + kTcCtrlBytes, 0xFF, ml.tc_pieces_bytes) != cudaSuccess ||
+      cudaMemset(c->ws + ml.tc_scratch, 0xFF, ml.tc_pieces_bytes) != cudaSuccess ||
       cudaMemset(c->ws + ml.partials, 0xFF, (size_t)ml.partial_rows * md.nq * (md.hd + 2) * 4) != cudaSuccess)
     return HSD_E_CUDA;
   M.use_persist = coop_launch_supported() && fwd_persist_supported(md.hd, md.nq / md.nkv) && md.d % 256 == 0 && md.d <= 4096 &&
@@ -1076,15 +1103,16 @@ int create_ctx(const hsd_model_desc *models, int n_models, const int32_t *exit_l
   c->lay = lay;
   c->ws = (char *)workspace;
   c->coin24.assign(n_levels, kNoCoin);
-  c->ring_host = nullptr; c->n_acc_host = nullptr; c->page_table_host = nullptr; c->status_host = nullptr;
+  c->ring_host = nullptr; c->result_host = nullptr; c->token_host = nullptr; c->page_table_host = nullptr;
+  c->token_stride = lay.slots[n_levels - 1] + 1;          // a verification's drafts and one more
   c->sm_count = device_sm_count();
   c->trace = nullptr; c->trace_logit_calls = 0; c->trace_records = 0;
   c->ring_next = 0; c->ring_in_flight = 0; c->timers_used = 0; c->timers_ok = true; c->stream = nullptr; c->seed = 0;
-  c->status_off = lay.model[0].tc_scratch;
+  c->status_off = lay.result;
   bool ok = cudaMallocHost(&c->ring_host, lay.ring_slot * kRingSlots) == cudaSuccess &&
-            cudaMallocHost(&c->n_acc_host, (size_t)c->max_batch * 4) == cudaSuccess &&
-            cudaMallocHost(&c->page_table_host, (size_t)c->max_batch * lay.pages_per_seq * 4) == cudaSuccess &&
-            cudaMallocHost(&c->status_host, 4) == cudaSuccess;
+            cudaMallocHost(&c->result_host, kResultHead + (size_t)c->max_batch * 4) == cudaSuccess &&
+            cudaMallocHost(&c->token_host, (size_t)3 * c->max_batch * c->token_stride * 4) == cudaSuccess &&
+            cudaMallocHost(&c->page_table_host, (size_t)c->max_batch * lay.pages_per_seq * 4) == cudaSuccess;
   for (int i = 0; i < kTimerPairs; ++i) { c->timers[i].a = nullptr; c->timers[i].b = nullptr; }
   for (int i = 0; ok && i < kTimerPairs; ++i)
     c->timers_ok = c->timers_ok && cudaEventCreate(&c->timers[i].a) == cudaSuccess && cudaEventCreate(&c->timers[i].b) == cudaSuccess;
@@ -1108,7 +1136,7 @@ int create_ctx(const hsd_model_desc *models, int n_models, const int32_t *exit_l
     c->level_norm[i] = c->model_of(i).final_norm;
   }
   c->stats.assign(n_levels, hsd_level_stats{});
-  *c->status_host = 0;
+  *c->result_host = 0;
   *out = c;
   return HSD_OK;
 }
@@ -1176,6 +1204,7 @@ int hsd_generate(hsd_ctx *c, const int32_t *prompt_ids, int batch, int prompt_le
   c->free_pages.clear();
   for (int p = c->lay.n_pages - 1; p >= 0; --p) c->free_pages.push_back(p);
   c->trace_records = 0;
+  c->pending.clear();
   cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
   bool ev = cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess && cudaEventCreate(&e2) == cudaSuccess;
   int st = HSD_OK;
@@ -1422,9 +1451,9 @@ void hsd_destroy(hsd_ctx *c) {
   if (!c) return;
   if (c->trace) fclose(c->trace);
   if (c->ring_host) cudaFreeHost(c->ring_host);
-  if (c->n_acc_host) cudaFreeHost(c->n_acc_host);
+  if (c->result_host) cudaFreeHost(c->result_host);
+  if (c->token_host) cudaFreeHost(c->token_host);
   if (c->page_table_host) cudaFreeHost(c->page_table_host);
-  if (c->status_host) cudaFreeHost(c->status_host);
   for (int i = 0; i < kTimerPairs; ++i) {
     if (c->timers[i].a) cudaEventDestroy(c->timers[i].a);
     if (c->timers[i].b) cudaEventDestroy(c->timers[i].b);

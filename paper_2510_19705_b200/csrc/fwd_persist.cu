@@ -1583,6 +1583,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
     for (int i = 0; i < 16; ++i) ring_pos_sh[i] = 0xFFFFFFFFu;
     pcache->tag_item = -1;
     pcache->tag_tile = -1;
+    if (c == 0) *a.next_counter = 0u;                    // (nobody uses it while this launch runs)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (threadIdx.x >= 128 && threadIdx.x < 133) {

@@ -42,6 +42,7 @@ struct FwdArgs {
   float *pieces[5];                // split pieces of QKV, O, gate / up, down, head: the caller gives the first, the launcher divides it
   size_t pieces_bytes;
   unsigned *grid_counter;          // zero on entry
+  unsigned *next_counter;          // the next launch's counter: cleared
   int *status;                     // set non-zero when a bounded wait gave up
   unsigned long long *prof;        // optional [gridDim][kFwdProfEvents]: barrier arrive / depart times (ns)
   CUtensorMap amap[4];             // activations h, att, act, hf; box rows = row padding of this launch
