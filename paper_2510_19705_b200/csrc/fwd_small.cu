@@ -29,7 +29,8 @@ struct Shared {
   float a[16 * kChunk];                          // rows of the product's left operand
   float inv[kSmallRows];                         // 1 / rms of each row
   int pos[kSmallRows], pg[kSmallRows], tok[kSmallRows];   // position of each row, the page that holds it, its token
-  float m[kWarps], l[kWarps], o[kWarps][128];    // attention: the warps' states
+  float m[kWarps], l[kWarps];
+  __align__(16) float o[kWarps][128];    // attention: the warps' states
   int ok;
 };
 
@@ -57,10 +58,11 @@ __device__ __forceinline__ bool barrier(const SmallFwdArgs &a, unsigned &target,
   return sh.ok != 0;
 }
 
-// acc[r][0 / 1] = row r0 + r of the operand times weight rows w0 / w1, valid in every lane.  The operand's rows: src(r),
-// scaled by inv[r] x gain when gain is given.
+// acc[0][0 / 1] = row r0 + lane_row(lane) of the operand times weight rows w0 / w1.  The operand's rows: src(r),
+// scaled by 1 / rms x gain when gain is given: rows of one chunk are read once, by a warp each, which has the row's scale
+// before it stages it; longer ones need their scales in sh.inv (row_scales).
 template <int RT, class Src>
-__device__ __forceinline__ void product(Shared &sh, const Src &src, const float *gain, int K, int r0, int rows, bool active, const float *w0,
+__device__ __forceinline__ void product(Shared &sh, const Src &src, const float *gain, float eps, int K, int r0, int rows, bool active, const float *w0,
                                         const float *w1, float (*acc)[2]) {
   const int tid = threadIdx.x, lane = tid & 31;
 #pragma unroll
@@ -73,15 +75,39 @@ __device__ __forceinline__ void product(Shared &sh, const Src &src, const float 
       p1 = __ldg(reinterpret_cast<const float4 *>(w1 + kc) + lane);
     }
     __syncthreads();
-    for (int i = tid; i < rows * n4; i += kThreads) {
-      const int r = i / n4, k = i - r * n4;
-      float4 v = __ldcg(reinterpret_cast<const float4 *>(src(r0 + r) + kc) + k);
-      if (gain) {
-        const float4 g = __ldg(reinterpret_cast<const float4 *>(gain + kc) + k);
-        const float s = sh.inv[r0 + r];
-        v = make_float4(v.x * s * g.x, v.y * s * g.y, v.z * s * g.z, v.w * s * g.w);
+    if (gain && K <= kChunk) {
+      constexpr int NV = kChunk / 128;
+      for (int r = tid >> 5; r < rows; r += kWarps) {
+        const float4 *row = reinterpret_cast<const float4 *>(src(r0 + r));
+        float4 v[NV], g[NV];
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+          const int k = lane + 32 * j;
+          v[j] = k < n4 ? __ldcg(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+          g[j] = k < n4 ? __ldg(reinterpret_cast<const float4 *>(gain) + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        float ss = 0.f;
+#pragma unroll
+        for (int j = 0; j < NV; ++j) ss += (v[j].x * v[j].x + v[j].y * v[j].y) + (v[j].z * v[j].z + v[j].w * v[j].w);
+        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, o);
+        const float s = rsqrtf(ss / (float)K + eps);
+#pragma unroll
+        for (int j = 0; j < NV; ++j)
+          if (lane + 32 * j < n4)
+            *reinterpret_cast<float4 *>(sh.a + r * kChunk + 4 * (lane + 32 * j)) =
+                make_float4(v[j].x * s * g[j].x, v[j].y * s * g[j].y, v[j].z * s * g[j].z, v[j].w * s * g[j].w);
       }
-      *reinterpret_cast<float4 *>(sh.a + r * kChunk + 4 * k) = v;
+    } else {
+      for (int i = tid; i < rows * n4; i += kThreads) {
+        const int r = i / n4, k = i - r * n4;
+        float4 v = __ldcg(reinterpret_cast<const float4 *>(src(r0 + r) + kc) + k);
+        if (gain) {
+          const float4 g = __ldg(reinterpret_cast<const float4 *>(gain + kc) + k);
+          const float s = sh.inv[r0 + r];
+          v = make_float4(v.x * s * g.x, v.y * s * g.y, v.z * s * g.z, v.w * s * g.w);
+        }
+        *reinterpret_cast<float4 *>(sh.a + r * kChunk + 4 * k) = v;
+      }
     }
     __syncthreads();
     if (!active) continue;
@@ -101,21 +127,37 @@ __device__ __forceinline__ void product(Shared &sh, const Src &src, const float 
     }
   }
   if (active) {
+    // sums over the lanes; while there are several rows a lane keeps the half its bit selects and gives the other away
+    // (the same additions as a butterfly per value, 12 exchanges instead of 40 for four rows)
+    int n = RT;
 #pragma unroll
-    for (int r = 0; r < RT; ++r) {
-      if (r >= rows) break;
+    for (int o = 16; o > 0; o >>= 1) {
+      if (n > 1) {
+        n >>= 1;
+        const bool up = (lane & o) != 0;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        acc[r][0] += __shfl_xor_sync(0xFFFFFFFFu, acc[r][0], o);
-        acc[r][1] += __shfl_xor_sync(0xFFFFFFFFu, acc[r][1], o);
+        for (int r = 0; r < RT / 2; ++r) {
+          if (r >= n) break;
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const float keep = up ? acc[n + r][e] : acc[r][e], give = up ? acc[r][e] : acc[n + r][e];
+            acc[r][e] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+          }
+        }
+      } else {
+        acc[0][0] += __shfl_xor_sync(0xFFFFFFFFu, acc[0][0], o);
+        acc[0][1] += __shfl_xor_sync(0xFFFFFFFFu, acc[0][1], o);
       }
     }
   }
 }
+// The row whose sums product() leaves in acc[0] of a lane (32 / RT neighbours hold the same).
+template <int RT> __device__ __forceinline__ int lane_row(int lane) { return lane / (32 / RT); }
 
-// 1 / rms of rows 0 .. n - 1, a warp per row (product()'s first barrier comes before the scales are read).
+// 1 / rms of rows 0 .. n - 1 longer than a chunk, a warp per row (product()'s first barrier comes before the scales are read).
 template <class Src> __device__ __forceinline__ void row_scales(Shared &sh, const Src &src, int n, int d, float eps) {
   const int lane = threadIdx.x & 31;
+  if (d <= kChunk) return;
   for (int r = threadIdx.x >> 5; r < n; r += kWarps) {
     const float4 *row = reinterpret_cast<const float4 *>(src(r));
     float ss = 0.f;
@@ -131,7 +173,7 @@ template <class Src> __device__ __forceinline__ void row_scales(Shared &sh, cons
 // A whole product phase: pairs of weight rows dealt to the grid's warps, row tiles of RT; finish(pair, row, v0, v1) is
 // called once per (pair, row), by one lane.
 template <int RT, class Src, class Pair, class Finish>
-__device__ __forceinline__ void product_phase(Shared &sh, const Src &src, const float *gain, int K, int n_rows, int n_pairs, const Pair &pair,
+__device__ __forceinline__ void product_phase(Shared &sh, const Src &src, const float *gain, float eps, int K, int n_rows, int n_pairs, const Pair &pair,
                                               const Finish &finish) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int base = blockIdx.x * kWarps; base < n_pairs; base += gridDim.x * kWarps) {      // uniform over the CTA
@@ -142,36 +184,38 @@ __device__ __forceinline__ void product_phase(Shared &sh, const Src &src, const 
     for (int r0 = 0; r0 < n_rows; r0 += RT) {
       const int rows = min(RT, n_rows - r0);
       float acc[RT][2];
-      product<RT>(sh, src, gain, K, r0, rows, active, w0, w1, acc);
-      if (!active) continue;
-#pragma unroll
-      for (int r = 0; r < RT; ++r)
-        if (r < rows && lane == r) finish(p, r0 + r, acc[r][0], acc[r][1]);
+      product<RT>(sh, src, gain, eps, K, r0, rows, active, w0, w1, acc);
+      // (all rows at once: one lane's finish after the other's is a trip to L2 per row)
+      if (active && lane % (32 / RT) == 0 && lane_row<RT>(lane) < rows) finish(p, r0 + lane_row<RT>(lane), acc[0][0], acc[0][1]);
     }
   }
 }
 
-// Attention of (row, query head) units, a CTA each: lane = key for the scores, lane = output dimension for P V.
-template <int HD> __device__ __forceinline__ void attention_phase(const SmallFwdArgs &a, const SmallLayerDev &ly, Shared &sh) {
-  constexpr int DPL = HD / 32;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, group = a.nq / a.nkv;
+// Attention of (row, query head) units, a CTA each: lane = key for the scores, HD / 4 lanes to a key's values for P V (few
+// instructions: a warp runs this once a layer, and unrolled code for each key comes from beyond the instruction cache).
+// `first`: the thread's cache row in the CTA's first unit, key = thread (the same in every layer: found once).
+__device__ __forceinline__ int cache_row(const SmallFwdArgs &a, int u, int key) {
+  const int r = u / a.nq, kvh = (u - r * a.nq) / (a.nq / a.nkv);
+  return (kvh * a.n_pages + a.page_table[(size_t)a.row_seq[r] * a.pages_per_seq + key / a.page]) * a.page + key % a.page;
+}
+template <int HD> __device__ __forceinline__ void attention_phase(const SmallFwdArgs &a, const SmallLayerDev &ly, Shared &sh, int first) {
+  constexpr int LPR = HD / 4, RPI = 32 / LPR, NI = 32 / RPI, PRE = NI < 8 ? NI : 8;   // lanes of a row, rows at a time
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float scale = rsqrtf((float)HD);
   for (int u = blockIdx.x; u < a.R * a.nq; u += gridDim.x) {
-    const int r = u / a.nq, h = u - r * a.nq, kvh = h / group, n_keys = sh.pos[r] + 1;
-    const int *pt = a.page_table + (size_t)a.row_seq[r] * a.pages_per_seq;
+    const int r = u / a.nq, h = u - r * a.nq, n_keys = sh.pos[r] + 1;
     __syncthreads();                                                 // the previous unit's merge has been read
     if (tid < HD) sh.a[tid] = __ldcg(a.q + ((size_t)r * a.nq + h) * HD + tid);
     __syncthreads();
-    float m = -INFINITY, l = 0.f, o[DPL];
-#pragma unroll
-    for (int e = 0; e < DPL; ++e) o[e] = 0.f;
+    float m = -INFINITY, l = 0.f;
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);                      // four dimensions, of the keys of this lane's group
     for (int k0 = warp * 32; k0 < n_keys; k0 += kWarps * 32) {
       const int key = k0 + lane, nk = min(32, n_keys - k0);
       float s = -INFINITY;
-      size_t row = 0;
+      int row = 0;
       if (lane < nk) {
-        row = ((size_t)kvh * a.n_pages + pt[key / a.page]) * a.page + key % a.page;
-        const float4 *kr = reinterpret_cast<const float4 *>(ly.k_pool + row * HD);
+        row = (u == (int)blockIdx.x && key < kThreads) ? first : cache_row(a, u, key);
+        const float4 *kr = reinterpret_cast<const float4 *>(ly.k_pool + (size_t)row * HD);
         float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int c = 0; c < HD / 4; ++c) {
@@ -180,6 +224,17 @@ template <int HD> __device__ __forceinline__ void attention_phase(const SmallFwd
         }
         s = ((t.x + t.y) + (t.z + t.w)) * scale;
       }
+      auto value = [&](int i) {                                      // of key RPI i + lane / LPR of the tile
+        const int kk = RPI * i + lane / LPR, vr = __shfl_sync(0xFFFFFFFFu, row, kk);
+        return kk < nk ? __ldcg(reinterpret_cast<const float4 *>(ly.v_pool + (size_t)vr * HD) + lane % LPR) : make_float4(0.f, 0.f, 0.f, 0.f);
+      };
+      auto add = [&](int i, float weight, const float4 &v) {
+        const float w = __shfl_sync(0xFFFFFFFFu, weight, RPI * i + lane / LPR);
+        o = make_float4(fmaf(w, v.x, o.x), fmaf(w, v.y, o.y), fmaf(w, v.z, o.z), fmaf(w, v.w, o.w));
+      };
+      float4 pre[PRE];                                               // on their way while the weights are worked out
+#pragma unroll
+      for (int i = 0; i < PRE; ++i) pre[i] = value(i);
       float mx = s;
 #pragma unroll
       for (int x = 16; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, x));
@@ -190,20 +245,21 @@ template <int HD> __device__ __forceinline__ void attention_phase(const SmallFwd
       for (int x = 16; x > 0; x >>= 1) ps += __shfl_xor_sync(0xFFFFFFFFu, ps, x);
       l = l * corr + ps;
       m = mn;
+      o = make_float4(o.x * corr, o.y * corr, o.z * corr, o.w * corr);
 #pragma unroll
-      for (int e = 0; e < DPL; ++e) o[e] *= corr;
-#pragma unroll 8
-      for (int kk = 0; kk < 32; ++kk) {
-        if (kk >= nk) break;
-        const float pk = __shfl_sync(0xFFFFFFFFu, p, kk);
-        const size_t vr = __shfl_sync(0xFFFFFFFFu, row, kk);
-#pragma unroll
-        for (int e = 0; e < DPL; ++e) o[e] = fmaf(pk, __ldcg(ly.v_pool + vr * HD + lane + 32 * e), o[e]);
+      for (int i = 0; i < PRE; ++i) add(i, p, pre[i]);
+#pragma unroll 4
+      for (int i = PRE; i < NI; ++i) {
+        if (RPI * i >= nk) break;
+        add(i, p, value(i));
       }
     }
-    if (lane == 0) { sh.m[warp] = m; sh.l[warp] = l; }
 #pragma unroll
-    for (int e = 0; e < DPL; ++e) sh.o[warp][lane + 32 * e] = o[e];
+    for (int x = LPR; x < 32; x <<= 1)
+      o = make_float4(o.x + __shfl_xor_sync(0xFFFFFFFFu, o.x, x), o.y + __shfl_xor_sync(0xFFFFFFFFu, o.y, x),
+                      o.z + __shfl_xor_sync(0xFFFFFFFFu, o.z, x), o.w + __shfl_xor_sync(0xFFFFFFFFu, o.w, x));
+    if (lane == 0) { sh.m[warp] = m; sh.l[warp] = l; }
+    if (lane < LPR) *reinterpret_cast<float4 *>(&sh.o[warp][4 * lane]) = o;
     __syncthreads();
     if (tid < HD) {                                                  // the warps' states in warp order (the first always holds keys)
       float mm = sh.m[0];
@@ -240,12 +296,14 @@ __global__ void __launch_bounds__(kThreads) fwd_small_kernel(const __grid_consta
     for (int k = tid; k < a.d; k += kThreads) a.x[(size_t)r * a.d + k] = src[k];
   }
   const int nqd = a.nq * HD;
+  int first = 0;
+  if ((int)blockIdx.x < a.R * a.nq && tid <= sh.pos[blockIdx.x / a.nq]) first = cache_row(a, blockIdx.x, tid);
   for (int l = 0; l < a.n_run; ++l) {
     const SmallLayerDev ly = a.layers[l];
     auto xs = [&](int r) { return l == 0 ? a.embed + (size_t)sh.tok[r] * a.d : (const float *)(a.x + (size_t)r * a.d); };
     auto xr = [&](int r) { return (const float *)(a.x + (size_t)r * a.d); };
     row_scales(sh, xs, a.R, a.d, a.eps);
-    product_phase<RT>(sh, xs, ly.w[0], a.d, a.R, (a.nq + 2 * a.nkv) * HALF,
+    product_phase<RT>(sh, xs, ly.w[0], a.eps, a.d, a.R, (a.nq + 2 * a.nkv) * HALF,
                       [&](int p, const float *&w0, const float *&w1) {
                         const int head = p / HALF, c = p - head * HALF;
                         const float *w = head < a.nq ? ly.w[1] + (size_t)head * HD * a.d
@@ -271,22 +329,22 @@ __global__ void __launch_bounds__(kThreads) fwd_small_kernel(const __grid_consta
                         dst[c + HALF] = v1;
                       });
     if (!barrier(a, target, sh)) return;
-    attention_phase<HD>(a, ly, sh);
+    attention_phase<HD>(a, ly, sh, first);
     if (!barrier(a, target, sh)) return;
     auto add = [&](int p, int r, float v0, float v1) {
       float2 *dst = reinterpret_cast<float2 *>(a.x + (size_t)r * a.d + 2 * p);
       const float2 old = __ldcg(dst);
       *dst = make_float2(old.x + v0, old.y + v1);
     };
-    product_phase<RT>(sh, [&](int r) { return (const float *)(a.att + (size_t)r * nqd); }, nullptr, nqd, a.R, a.d / 2,
+    product_phase<RT>(sh, [&](int r) { return (const float *)(a.att + (size_t)r * nqd); }, nullptr, 0.f, nqd, a.R, a.d / 2,
                       [&](int p, const float *&w0, const float *&w1) { w0 = ly.w[4] + (size_t)2 * p * nqd; w1 = w0 + nqd; }, add);
     if (!barrier(a, target, sh)) return;
     row_scales(sh, xr, a.R, a.d, a.eps);
-    product_phase<RT>(sh, xr, ly.w[5], a.d, a.R, a.ff,
+    product_phase<RT>(sh, xr, ly.w[5], a.eps, a.d, a.R, a.ff,
                       [&](int p, const float *&w0, const float *&w1) { w0 = ly.w[6] + (size_t)p * a.d; w1 = ly.w[7] + (size_t)p * a.d; },
                       [&](int p, int r, float g, float u) { a.act[(size_t)r * a.ff + p] = g / (1.f + __expf(-g)) * u; });
     if (!barrier(a, target, sh)) return;
-    product_phase<RT>(sh, [&](int r) { return (const float *)(a.act + (size_t)r * a.ff); }, nullptr, a.ff, a.R, a.d / 2,
+    product_phase<RT>(sh, [&](int r) { return (const float *)(a.act + (size_t)r * a.ff); }, nullptr, 0.f, a.ff, a.R, a.d / 2,
                       [&](int p, const float *&w0, const float *&w1) { w0 = ly.w[8] + (size_t)2 * p * a.ff; w1 = w0 + a.ff; }, add);
     if (l + 1 < a.n_run || a.L > 0)
       if (!barrier(a, target, sh)) return;
@@ -294,7 +352,7 @@ __global__ void __launch_bounds__(kThreads) fwd_small_kernel(const __grid_consta
   if (a.L > 0) {
     auto xl = [&](int r) { return (const float *)(a.x + (size_t)a.lrow_src[r] * a.d); };
     row_scales(sh, xl, a.L, a.d, a.eps);
-    product_phase<RT>(sh, xl, a.final_norm, a.d, a.L, (a.V + 1) / 2,
+    product_phase<RT>(sh, xl, a.final_norm, a.eps, a.d, a.L, (a.V + 1) / 2,
                       [&](int p, const float *&w0, const float *&w1) {
                         w0 = a.lm_head + (size_t)2 * p * a.d;
                         w1 = 2 * p + 1 < a.V ? w0 + a.d : w0;
