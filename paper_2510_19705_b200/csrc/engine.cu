@@ -1124,6 +1124,8 @@ int create_ctx(const hsd_model_desc *models, int n_models, const int32_t *exit_l
     st = init_model(c, c->models[mi], &models[mi], lay.model[mi]);
     c->any_tc = c->any_tc || c->models[mi].use_tc || c->models[mi].use_small;
   }
+  // the buffers are filled on the default stream; a generation may run on one that does not wait for it
+  if (!st && cudaStreamSynchronize(nullptr) != cudaSuccess) st = HSD_E_CUDA;
   if (st) {
     hsd_destroy(c);
     return st;

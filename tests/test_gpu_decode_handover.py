@@ -39,3 +39,19 @@ def test_calls_do_not_depend_on_the_calls_before(lib, d_model, nq, nkv, hd, ff):
         alone.close()
     used.close()
     separate.close()
+
+
+def test_first_pass_on_another_stream_finds_the_buffers_filled(lib):
+    """A context is created on the default stream; its first pass may run on one that does not wait for that stream."""
+    cfg = inputs.model_cfg(3, 256, 8, 2, 704, 2000, "bf16", head_dim=32)
+    w = inputs.make_weights(cfg, 5, device="cuda")
+    prompt = inputs.make_prompts(cfg["vocab"], 1, 24, 24).cuda()
+    torch.cuda.synchronize()
+    side, outs = torch.cuda.Stream(), []
+    for stream in (torch.cuda.current_stream(), side):
+        eng = lib.Hsd(cfg, w, (1, 3), (2,), max_batch=6, max_seq=4096)
+        with torch.cuda.stream(stream):
+            outs.append(eng.generate(prompt, 24, 3)[0])
+        stream.synchronize()
+        eng.close()
+    assert torch.equal(outs[0], outs[1])
