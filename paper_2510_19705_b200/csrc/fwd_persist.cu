@@ -222,12 +222,14 @@ __device__ __forceinline__ float4 get_words4(const float *p) {
   return make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3]));
 }
 // A thread's N vectors of words: load(i, v[i]) is asked once for all, then again for those that still hold a hole, for 2 s at
-// most (then the CTA gives up: what the caller goes on with is never used).  Asking for all of them again each time made
-// a look at a row's 64 KB of pieces 1.2 us long.
+// most or until another CTA has given up (then this one does: what the caller goes on with is never used).  Asking for all of
+// them again each time made a look at a row's 64 KB of pieces 1.2 us long; the status word is looked at every 256 rounds, about
+// 0.2 ms, because the look costs a trip to L2 of its own.
 __device__ __forceinline__ unsigned top(float v) { return __float_as_uint(v); }
 __device__ __forceinline__ unsigned top(const float2 &v) { return max(top(v.x), top(v.y)); }
 __device__ __forceinline__ unsigned top(const float4 &v) { return max(max(top(v.x), top(v.y)), max(top(v.z), top(v.w))); }
-template <int N, class V, class Load> __device__ __forceinline__ void settle_words(V (&v)[N], const Load &load, volatile int *abort_flag) {
+template <int N, class V, class Load>
+__device__ __forceinline__ void settle_words(V (&v)[N], const Load &load, volatile int *abort_flag, const int *status) {
   unsigned long long t0 = 0;
   for (unsigned it = 1;; ++it) {
     unsigned seen = 0u;
@@ -241,15 +243,25 @@ template <int N, class V, class Load> __device__ __forceinline__ void settle_wor
     if (*abort_flag) return;
     const unsigned long long now = globaltimer_ns();
     if (t0 == 0) t0 = now;
-    else if (now - t0 > kWaitLimitNs) { *abort_flag = 1; return; }
+    else if (now - t0 > kWaitLimitNs || ((it & 255u) == 0u && *reinterpret_cast<const volatile int *>(status) != 0)) { *abort_flag = 1; return; }
   }
 }
-template <int N, class V, class Load> __device__ __forceinline__ void fetch_words(V (&v)[N], const Load &load, volatile int *abort_flag) {
+template <int N, class V, class Load>
+__device__ __forceinline__ void fetch_words(V (&v)[N], const Load &load, volatile int *abort_flag, const int *status) {
 #pragma unroll
   for (int i = 0; i < N; ++i) load(i);
-  settle_words(v, load, abort_flag);
+  settle_words(v, load, abort_flag, status);
 }
 __device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 2, 256;" ::: "memory"); }
+// The same barrier with a vote: true in every worker thread if `gone` is in any.  Pipeline roles raise the CTA's flag at any
+// time, so threads that read it one after the other may differ; a thread that left for that reason alone would be missing at
+// the others' next barrier, for good.
+__device__ __forceinline__ bool worker_sync_any(bool gone) {
+  uint32_t any;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 2, 256, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+               : "=r"(any) : "r"(gone ? 1u : 0u) : "memory");
+  return any != 0;
+}
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 // barrier of one 128-thread worker group (id 1 = warps 4..7, the epilogue group; id 3 = warps 8..11)
 __device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
@@ -259,7 +271,8 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
   return v;
 }
 
-// Grid-wide barrier of the worker threads.  `epoch` counts barriers; the counter only grows.
+// Grid-wide barrier of the worker threads; false, in all of them, once a wait of the CTA has given up.  `epoch` counts
+// barriers; the counter only grows.
 // If ready_bar != 0 the spinning thread then releases the activation producer for the next GEMM.
 __device__ __forceinline__ bool grid_barrier(const FwdArgs &a, unsigned &epoch, volatile int *abort_flag, int wt,
                                              uint32_t ready_bar) {
@@ -269,26 +282,25 @@ __device__ __forceinline__ bool grid_barrier(const FwdArgs &a, unsigned &epoch, 
   // The activations this phase wrote with plain stores are read by the next GEMM's TMA loads (async proxy):
   // every writer orders its generic-proxy writes before async-proxy accesses here, ahead of the release.
   if (ready_bar) asm volatile("fence.proxy.async.global;" ::: "memory");
-  worker_sync();
+  if (worker_sync_any(*abort_flag != 0)) return false;
   ++epoch;
-  if (*abort_flag) return false;
+  bool gone = false;
   if (wt == 0) {
     const unsigned target = epoch * gridDim.x;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.grid_counter) : "memory");
     if (HSD_PROF(a) && 2 * epoch + 1 < (unsigned)kFwdProfEvents) a.prof[(size_t)blockIdx.x * kFwdProfEvents + 2 * epoch] = globaltimer_ns();
-    bool ok = true;
     unsigned long long t0 = 0;                       // the clock is read only once the wait has lasted a while
     for (uint32_t it = 0; (int)(ld_acquire_u32(a.grid_counter) - target) < 0; ++it) {
       if ((it & 31u) == 31u) {
         const unsigned long long now = globaltimer_ns();
         if (t0 == 0) t0 = now;
         if (*abort_flag || *reinterpret_cast<volatile int *>(a.status) != 0 || now - t0 > kWaitLimitNs) {
-          ok = false;
+          gone = true;
           break;
         }
       }
     }
-    if (!ok) {
+    if (gone) {
       *abort_flag = 1;
       atomicExch(a.status, 1);
     } else {
@@ -300,8 +312,7 @@ __device__ __forceinline__ bool grid_barrier(const FwdArgs &a, unsigned &epoch, 
       }
     }
   }
-  worker_sync();
-  return *abort_flag == 0;
+  return !worker_sync_any(gone);
 }
 
 // ------------------------------------------------------------------------------ RMSNorm phase
@@ -362,7 +373,7 @@ __device__ __forceinline__ void norm_phase(const FwdArgs &a, int n_rows, const i
       fetch_words(t, [&](int i) {
         const int j = i / PB, pp = i % PB;
         t[i] = (wt + 256 * j < nvec && pp < np) ? get_words4(base[j] + (size_t)pp * NPAD * kTcBlockM) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }, abort_flag);
+      }, abort_flag, a.status);
 #pragma unroll
       for (int j = 0; j < MAXV; ++j)
 #pragma unroll
@@ -484,7 +495,8 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float *o) {
 
 struct TcaItem { int row0, nrows, seq, pos0, kvh, split, key_lo, key_hi, nqv, group; };
 
-__device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 *kpool, const __nv_bfloat16 *vpool, uint8_t *smem,
+// False, in every thread of the CTA, if a wait gave up.
+__device__ __noinline__ bool attn_item_tc(const FwdArgs &a, const __nv_bfloat16 *kpool, const __nv_bfloat16 *vpool, uint8_t *smem,
                                           uint32_t tmem, const TcaItem it, int wt, volatile int *abort_flag, long long *dbg) {
   constexpr int HD = 128, TK = kTcaTile, NKB = kTcaKBufs, NVB = kTcaVBufs;
   const uint32_t s0 = smem_u32(smem), b0 = s0 + kTcaOffBar;
@@ -554,7 +566,7 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
           if (lane == 0) mbar_wait(isk ? k_free(s, b) : v_free(s, b), (uint32_t)(use & 1), abort_flag);
           __syncwarp();
         }
-        if (*abort_flag) break;
+        if (__any_sync(0xFFFFFFFFu, *abort_flag != 0)) break;
         const int key0 = it.key_lo + (2 * t + s) * TK;
         // the tile's four 16-key groups lie in one page each (pages hold >= 16 tokens, key ranges start on multiples of 16)
         int pg = 0;
@@ -723,9 +735,8 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
   // ---- all MMAs of the item are complete once both softmax warps are here; stream 1 hands (O, m, l) to stream 0
   //      through shared memory (over the K buffers), stream 0 writes the item's result
   tc_fence_before();
-  worker_sync();
+  if (worker_sync_any(*abort_flag != 0)) return false;
   tc_fence_after();
-  if (*abort_flag) return;
   if (wt == 0)                                                    // nobody waits on the item's barriers any more: their memory
     for (int i = 0; i < 24; ++i)                                  // goes back to the weight ring / the next item
       asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(b0 + 8u * i) : "memory");
@@ -778,6 +789,7 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
     tc_fence_before();
   }
   lap(8);
+  return true;
 }
 
 // Phase A: warp-level online softmax.  A work item is (attention item, KV head, key split); its keys
@@ -790,8 +802,9 @@ __device__ __noinline__ void attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
 // (rows x group) every warp works on its own sub-tiles; with 17..32 the warps pair up on a sub-tile,
 // one 16-row m-tile each.  At the end the warps' states are merged through shared memory and the
 // split's partial (o, m, l) goes to global memory.
+// False, in every thread, if a wait of a tensor-memory item gave up.
 template <int NPAD, int HD, bool TC>
-__device__ __forceinline__ void attn_tiles_phase(const FwdArgs &a, const FwdLayerDev &lay, uint8_t *scratch, PageCache *pc, int wt, long long *dbg,
+__device__ __forceinline__ bool attn_tiles_phase(const FwdArgs &a, const FwdLayerDev &lay, uint8_t *scratch, PageCache *pc, int wt, long long *dbg,
                                                  const int *first_item, const int *qkv_geom, const int *row_pg_sh, const float *rope_cos_sh,
                                                  const float *rope_sin_sh, uint8_t *tc_smem, uint32_t tmem, volatile int *abort_flag) {
   constexpr int CPR = HD / 8;                      // 16-byte chunks per row
@@ -837,8 +850,7 @@ __device__ __forceinline__ void attn_tiles_phase(const FwdArgs &a, const FwdLaye
       TcaItem ti;
       ti.row0 = row0; ti.nrows = nrows; ti.seq = seq; ti.pos0 = pos0; ti.kvh = kvh; ti.split = split;
       ti.key_lo = key_lo; ti.key_hi = key_hi; ti.nqv = nqv; ti.group = group;
-      attn_item_tc(a, kpool, vpool, tc_smem, tmem, ti, wt, abort_flag, dbg);
-      if (*abort_flag) return;
+      if (!attn_item_tc(a, kpool, vpool, tc_smem, tmem, ti, wt, abort_flag, dbg)) return false;
       continue;
     }
     const int n_sub = (key_hi - key_lo + 15) >> 4;
@@ -921,7 +933,7 @@ __device__ __forceinline__ void attn_tiles_phase(const FwdArgs &a, const FwdLaye
         float4 pc4[16];                                          // [piece][low 0-3, low 4-7, high 0-3, high 4-7]
         fetch_words(pc4, [&](int i) {
           pc4[i] = (i >> 2) < n_pieces ? get_words4(base + (i >> 2) * pstride + (i & 1) * 4 + ((i >> 1) & 1) * HALF) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }, abort_flag);
+        }, abort_flag, a.status);
         float cs[8], sn[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) { cs[e] = 1.f; sn[e] = 0.f; }
@@ -1154,6 +1166,7 @@ __device__ __forceinline__ void attn_tiles_phase(const FwdArgs &a, const FwdLaye
     }
     lap(4);
   }
+  return true;
 }
 
 // Phase B: merge the split partials of one (row, head) per HD / 2 threads (two output dimensions each); a single
@@ -1171,7 +1184,7 @@ __device__ __forceinline__ void attn_merge_phase(const FwdArgs &a, const int *ro
     fetch_words(w, [&](int i) {
       const int sp = i >> 1;
       w[i] = sp < used ? get_words2(src + sp * (HD + 2) + ((i & 1) ? dd : HD)) : ((i & 1) ? make_float2(0.f, 0.f) : make_float2(-INFINITY, 0.f));
-    }, abort_flag);
+    }, abort_flag, a.status);
     float m = -INFINITY;
 #pragma unroll
     for (int s = 0; s < kAttnMaxSplits; ++s) m = fmaxf(m, w[2 * s].x);
@@ -1362,10 +1375,10 @@ __device__ __forceinline__ void build_act_stages(const FwdArgs &a, WorkerCtx &w,
   // ring position (slot, parity of its empty barrier) of the phase's first stage, published by the weight producer
   ring_pos += (p >> 2) & 15;
   unsigned rp = *ring_pos;
-  if ((int)(rp >> 16) != p) {
+  if (!__all_sync(0xFFFFFFFFu, (int)(rp >> 16) == p)) {
     const unsigned long long t0 = globaltimer_ns();
-    while ((int)((rp = *ring_pos) >> 16) != p)
-      if (*w.abort_flag || globaltimer_ns() - t0 > kWaitLimitNs) { *w.abort_flag = 1; return; }
+    while (!__all_sync(0xFFFFFFFFu, (int)((rp = *ring_pos) >> 16) == p))
+      if (__any_sync(0xFFFFFFFFu, *w.abort_flag != 0 || globaltimer_ns() - t0 > kWaitLimitNs)) { *w.abort_flag = 1; return; }
   }
   const int s0 = (int)(rp & 0xFFu), warp4 = w.wt >> 6, r = w.lane >> 3, c8 = w.lane & 7;
   const uint32_t par0 = (rp >> 8) & 1u;
@@ -1396,7 +1409,7 @@ __device__ __forceinline__ void build_act_stages(const FwdArgs &a, WorkerCtx &w,
       if (i >= it.left) break;
       const int pos = s0 + i, s = pos % STAGES;
       const uint32_t par = par0 ^ (uint32_t)((pos / STAGES) & 1);
-      load(t[dpt], i, [&](auto &&one) { settle_words(t[dpt], one, w.abort_flag); });
+      load(t[dpt], i, [&](auto &&one) { settle_words(t[dpt], one, w.abort_flag, a.status); });
       __syncwarp();
       bool ok = true;                                          // the slot is free once its previous MMAs have retired
       if (w.lane == 0) ok = mbar_wait(empty_bar0 + 8u * s, par, w.abort_flag);
@@ -1459,7 +1472,7 @@ __device__ __forceinline__ void gemm_finish(const FwdArgs &a, WorkerCtx &w, int 
       fetch_words(tw, [&](int q) {
         const int pp = q / RB, i = (q % RB) >> 1;
         tw[q] = (pp < n_pieces && r0 + i < g.rows) ? get_word(base + ((size_t)pp * NPAD + r0 + i) * kTcBlockM + (q & 1) * kTcBoxRows) : 0.f;
-      }, w.abort_flag);
+      }, w.abort_flag, a.status);
       if (col < g.seg_n[0]) {
 #pragma unroll
         for (int i = 0; i < RB / 2; ++i) {
@@ -1506,7 +1519,7 @@ __device__ __forceinline__ void gemm_finish(const FwdArgs &a, WorkerCtx &w, int 
 #pragma unroll 1
     for (int c0 = r_lo; c0 < r_hi; c0 += RG) {
       float v[RG], cs[RG], sn[RG];
-      settle_words(tn, [&](int q) { one(c0, q); }, w.abort_flag);
+      settle_words(tn, [&](int q) { one(c0, q); }, w.abort_flag, a.status);
       if (g.mode == MODE_LOGITS) {               // the pass ends here: the words' one reader makes them holes again
         for (int pp = 0; pp < n_pieces; ++pp)
 #pragma unroll
@@ -1605,7 +1618,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
   if (warp == 0) {
     // ------------------------------------------------------------ weight-tile producer (runs ahead)
     const bool issuer = elect_one();
-    int s = 0, n_issued = 0;
+    int s = 0;
     uint32_t par = 1;                                    // parity to wait for on the slot's empty barrier
     const uint64_t w_policy = l2_policy_evict_first();   // weights are read once per pass: first out of L2
     bool ok = true;
@@ -1633,22 +1646,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
             tma_load_2d_hint(dst, m0, kb * kTcBlockK, ti.row0, full_bar(s), w_policy);
             if (second) tma_load_2d_hint(dst + kBoxBytes, m1, kb * kTcBlockK, row1, full_bar(s), w_policy);
           }
-          ++n_issued;
           if (++s == STAGES) { s = 0; par ^= 1u; }
         }
       }
     }
-    if (!ok && issuer) {
-      atomicExch(a.status, 1);
-      // let copies in flight land (bounded): the last min(n_issued, STAGES) slots, newest first
-      uint32_t fpar = par ^ 1u;                          // full-barrier parity of the current round
-      for (int i = 0, sl = s; i < STAGES && i < n_issued; ++i) {
-        if (--sl < 0) { sl = STAGES - 1; fpar ^= 1u; }
-        unsigned long long t0 = globaltimer_ns();
-        while (!mbar_try_wait(full_bar(sl), fpar))
-          if (globaltimer_ns() - t0 > kWaitLimitNs / 4) break;
-      }
-    }
+    if (!ok && issuer) atomicExch(a.status, 1);
   } else if (warp == 1) {
     // ------------------------------------------------------------ activation-tile producer
     const bool issuer = elect_one();
@@ -1831,9 +1833,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
           break;
         case K_FIN: gemm_finish<NPAD>(a, w, gp); break;
         case K_ATTN_A:
-          attn_tiles_phase<NPAD, HD, TC>(a, layer_of(a, l), scratch, pcache, wt, dbg_cy, first_item_sh, qkv_geom_sh, row_pg_sh, rope_cos_sh, rope_sin_sh,
-                                     ring, tmem_base, abort_flag);
-          if (TC) {                                               // the ring's memory is the weight producer's again
+          alive = attn_tiles_phase<NPAD, HD, TC>(a, layer_of(a, l), scratch, pcache, wt, dbg_cy, first_item_sh, qkv_geom_sh, row_pg_sh, rope_cos_sh,
+                                                 rope_sin_sh, ring, tmem_base, abort_flag);
+          if (TC && alive) {                                               // the ring's memory is the weight producer's again
             worker_sync();
             if (wt == 0) mbar_arrive(attn_done_bar);
           }
@@ -1864,8 +1866,13 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (*abort_flag) {                                     // (nobody writes it any more: the same in all threads)
+    if (threadIdx.x == 0) atomicExch(a.status, 1);
+    const unsigned long long t0 = globaltimer_ns();      // copies and MMAs in flight end before their memory goes away
+    while (globaltimer_ns() - t0 < 200000ull) {}
+    __syncthreads();
+  }
   if (warp == 2) tmem_dealloc(tmem_base, tmem_cols);
-  if (threadIdx.x == 0 && *abort_flag) atomicExch(a.status, 1);
 }
 
 // The attention tiles phase as a launch of its own (prompt passes with more rows than the persistent forward takes):

@@ -55,3 +55,36 @@ def test_first_pass_on_another_stream_finds_the_buffers_filled(lib):
         stream.synchronize()
         eng.close()
     assert torch.equal(outs[0], outs[1])
+
+
+def _grid_counters(eng, cfg, max_seq, T, n_levels):
+    """The two barrier counters of a context of one sequence (bf16, head size 32, pages of 16): one line of 64 bytes each."""
+    from paper_2510_19705_b200 import binding
+    up = lambda n: (n + 255) // 256 * 256
+    slots = [sum(T[:i + 1]) + 1 for i in range(n_levels)]
+    parts = [4 * max_seq, 4 * ((max_seq + 15) // 16)] + [s * cfg["vocab"] * 2 for s in slots]
+    parts += [binding.hsd_verify_workspace_bytes(1, sum(T) + 1), 256 + 4, up(128 * 40 + 96 + 40 + 1024) * 48]
+    base = (-eng.workspace.data_ptr()) % 256
+    off = base + sum(up(n) for n in parts)
+    return eng.workspace[off:off + 256].view(torch.int32).view(4, 16)[:2, 0]
+
+
+def test_a_wait_that_runs_out_ends_with_an_error(lib):
+    """Barrier counters far below anything the launch can count up to: the first barrier's waits, and those of the roles behind
+    it, run out after two seconds.  The call reports it, and the GPU goes on."""
+    cfg = inputs.model_cfg(3, 256, 8, 2, 704, 2000, "bf16", head_dim=32)
+    w = inputs.make_weights(cfg, 5, device="cuda")
+    prompt = inputs.make_prompts(cfg["vocab"], 1, 24, 24).cuda()
+    eng = lib.Hsd(cfg, w, (1, 3), (2,), max_batch=1, max_seq=160)
+    want = eng.generate(prompt, 24, 3)[0]
+    counters, sms = _grid_counters(eng, cfg, 160, (2,), 2), torch.cuda.get_device_properties(0).multi_processor_count
+    seen = sorted(counters.tolist())
+    assert seen[0] == 0 and seen[1] > 0 and seen[1] % sms == 0, seen         # these are the counters: cleared, and one pass's arrivals
+    counters.fill_(-2 ** 30)
+    torch.cuda.synchronize()
+    with pytest.raises(lib.HsdError, match="timed out"):
+        eng.generate(prompt, 24, 3)
+    eng.close()
+    eng = lib.Hsd(cfg, w, (1, 3), (2,), max_batch=1, max_seq=160)
+    assert torch.equal(eng.generate(prompt, 24, 3)[0], want)
+    eng.close()
