@@ -14,7 +14,24 @@
 // In decode passes two finish phases fold into their consumer: the attention phase finishes the
 // q / k / v of its own rows, and with at most four rows the down projection's CTAs build their
 // activation tiles from the gate / up pieces in shared memory (warps 5, 7, 9, 11).
-// Every wait (mbarrier, grid barrier) is bounded by wall time and raises a status word.
+// Every wait (mbarrier, grid barrier, words) is bounded by wall time and raises a status word.
+//
+// A parity wait sees a completion of its barrier only until the next one, so every waiter here is one that the next completion
+// cannot do without, and has seen the one before:
+//   full[slot]        MMA issuer: the slot's next tiles come behind empty[slot], which its commit completes
+//   empty[slot]       weight producer, activation producer or builder: the next MMAs need the tile that each of them brings.
+//                     Where the builders bring the activations, the activation producer counts the slots and does not wait:
+//                     nothing there would wait for it.  (It finds its next slot's last completion but one behind it: that one
+//                     came before the last built stage's weights, and those before the down words its next `ready` rests on.)
+//   acc_full[b]       epilogue: the next MMAs come behind acc_empty[b], which its warps complete
+//   acc_empty[b]      MMA issuer: the next epilogue needs its MMAs
+//   ready[kind]       activation producer, in CTAs with tiles of that kind of projection: the next arrival, a layer later, comes
+//                     behind this CTA's epilogue of those tiles.  The other CTAs' producers do not look at it
+// In a tensor-memory attention item, per stream:
+//   k_full, v_full    MMA issuer: the next loads come behind k_free / v_free, which its commits complete
+//   k_free, v_free    loader: the next MMAs need its tile; softmax: they need its P (k_free doubles as "S complete")
+//   p_ready           MMA issuer: the next P needs its S
+// The weight producer's wait for the end of the attention phase has no such tie in CTAs without tiles: it compares a count.
 #include <type_traits>
 #include "fwd_persist.cuh"
 #include "forward.cuh"
@@ -269,6 +286,19 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+
+// A warp's wait for a count in shared memory that only grows.  Looks are 64 ns apart: the softmax warps of the attention phase
+// it waits for issue from the same scheduler.
+__device__ __forceinline__ bool count_wait_warp(const unsigned *count, unsigned want, volatile int *abort_flag) {
+  const unsigned long long t0 = globaltimer_ns();
+  for (;;) {
+    unsigned v;
+    asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(count)) : "memory");
+    if (__all_sync(0xFFFFFFFFu, v >= want)) return true;
+    if (__any_sync(0xFFFFFFFFu, *abort_flag != 0 || globaltimer_ns() - t0 > kWaitLimitNs)) { *abort_flag = 1; return false; }
+    __nanosleep(64);
+  }
 }
 
 // Grid-wide barrier of the worker threads; false, in all of them, once a wait of the CTA has given up.  `epoch` counts
@@ -1551,18 +1581,19 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
   uint8_t *ring = smem;
   uint8_t *scratch = smem + STAGES * Cfg::kStageBytes;
   uint64_t *bars = reinterpret_cast<uint64_t *>(scratch + kScratchBytes);
-  // bars: full[STAGES] | empty[STAGES] | acc_full[2] | acc_empty[2] | ready[2]
-  uint32_t *ctl = reinterpret_cast<uint32_t *>(bars + 2 * STAGES + 6);
+  // bars: full[STAGES] | empty[STAGES] | acc_full[2] | acc_empty[2] | ready[5] (by kind of projection)
+  uint32_t *ctl = reinterpret_cast<uint32_t *>(bars + 2 * STAGES + 9);
   uint32_t *tmem_slot = ctl;
   volatile int *abort_flag = reinterpret_cast<volatile int *>(ctl + 1);
   int *first_item_sh = reinterpret_cast<int *>(ctl + 148);               // [4] this CTA's first attention item
   int *qkv_geom_sh = reinterpret_cast<int *>(ctl + 152);                 // [7] piece geometry of the QKV projection
   // [16] phase << 16 | parity << 8 | slot of the first stage of built down projection number (layer & 15): the
   // weight producer is at most one ring (8 stages) ahead, so never 16 such phases
-  volatile unsigned *ring_pos_sh = reinterpret_cast<volatile unsigned *>(ctl + 928);
+  volatile unsigned *ring_pos_sh = reinterpret_cast<volatile unsigned *>(ctl + 720);
   PhaseGeom *geom_sh = reinterpret_cast<PhaseGeom *>(ctl + 672);          // [5]
-  static_assert(5 * sizeof(PhaseGeom) <= (928 - 672) * 4, "control area overlap");
-  static_assert((2 * Cfg::kStages + 6) * 8 + 944 * 4 <= kCtrlBytes - 128, "control area overflow");
+  static_assert(5 * sizeof(PhaseGeom) <= (720 - 672) * 4, "control area overlap");
+  static_assert((2 * Cfg::kStages + 9) * 8 + 736 * 4 <= kCtrlBytes - 128, "control area overflow");
+  unsigned *attn_done_sh = ctl + 2;                                      // attention phases this CTA is through with (TC)
   volatile int *wait_ok = reinterpret_cast<volatile int *>(ctl + 4);   // [2]
   float *red = reinterpret_cast<float *>(ctl + 8);                      // [8]
   PageCache *pcache = reinterpret_cast<PageCache *>(ctl + 16);          // 130 words
@@ -1581,7 +1612,6 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
   auto accf_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + b); };
   auto acce_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + 2 + b); };
   auto ready_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + 4 + b); };
-  const uint32_t attn_done_bar = smem_u32(dbg_cy + 15);         // the last counter slot (laps use 0..14)
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int G = gridDim.x, c = blockIdx.x;
@@ -1589,10 +1619,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 2); mbar_init(empty_bar(s), 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), 4); mbar_init(ready_bar(b), 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), 4); }
+    for (int k = 0; k < 5; ++k) mbar_init(ready_bar(k), 1);
     *abort_flag = 0;
     for (int i = 0; i < 15; ++i) dbg_cy[i] = 0;
-    mbar_init(attn_done_bar, 1);
+    *attn_done_sh = 0u;
     for (int i = 0; i < 16; ++i) ring_pos_sh[i] = 0xFFFFFFFFu;
     pcache->tag_item = -1;
     pcache->tag_tile = -1;
@@ -1628,8 +1659,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
       SegIter it = seg_begin(pg);
       Seg sg;
       // the tensor-memory attention phase uses the ring's memory: the O projection's tiles wait until it is over
-      // (one completion per layer, waited for in every layer, so the parity never is ambiguous)
-      if (TC && (p & 3) == 1 && p < 4 * a.n_run && !mbar_wait_warp(attn_done_bar, (uint32_t)((p >> 2) & 1), abort_flag)) { ok = false; break; }
+      if (TC && (p & 3) == 1 && p < 4 * a.n_run && !count_wait_warp(attn_done_sh, (unsigned)(p >> 2) + 1u, abort_flag)) { ok = false; break; }
       if (issuer && built_down(a, p)) ring_pos_sh[(p >> 2) & 15] = (unsigned)s | (par << 8) | ((unsigned)p << 16);   // where the builders' tiles go
       while (ok && seg_next(pg, it, sg)) {
         const Tile ti = tile_of(g, sg.tile);
@@ -1662,22 +1692,26 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
       const int kind = kind_of(a, p);
       const CUtensorMap *amap = &a.amap[kind == 1 ? 1 : kind == 3 ? 2 : kind == 4 ? 3 : 0];
       const PhaseGeom &pg = geom_sh[kind];
+      if (pg.left == 0) continue;
+      if (built_down(a, p)) {                            // the workers fill the tiles and arrive
+        s += pg.left;
+        par ^= (uint32_t)(s / STAGES) & 1u;
+        s %= STAGES;
+        continue;
+      }
+      // the operand of phase p is complete once the workers have passed the barrier before it
+      if (!mbar_wait_warp(ready_bar(kind), kind == 4 ? 0u : (uint32_t)((p >> 2) & 1), abort_flag)) { ok = false; break; }
       SegIter it = seg_begin(pg);
       Seg sg;
-      bool have = seg_next(pg, it, sg);
-      // the operand of phase p is complete once the workers have passed the barrier before it
-      if (!mbar_wait_warp(ready_bar(p & 1), (uint32_t)((p >> 1) & 1), abort_flag)) { ok = false; break; }
-      const bool built = built_down(a, p);
-      while (ok && have) {
+      while (ok && seg_next(pg, it, sg)) {
         for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
           if (!mbar_wait_warp(empty_bar(s), par, abort_flag)) { ok = false; break; }
-          if (issuer && !built) {                        // built down projection: the workers fill the tile and arrive
+          if (issuer) {
             mbar_expect_tx(full_bar(s), a_bytes);
             tma_load_2d(smem_u32(ring) + (uint32_t)(s * Cfg::kStageBytes) + kWBytes, amap, kb * kTcBlockK, 0, full_bar(s));
           }
           if (++s == STAGES) { s = 0; par ^= 1u; }
         }
-        have = seg_next(pg, it, sg);
       }
     }
     if (!ok && issuer) atomicExch(a.status, 1);
@@ -1828,16 +1862,15 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
               if (kind == 3 || a.fuse_gu) put_holes<NPAD>(a, w, 2);
             }
           }
-          // (a built down projection takes nothing by TMA but its weights: the activation producer only counts slots)
-          if (a.fuse_gu && gp < 4 * a.n_run && (gp & 3) == 2 && wt == 0) mbar_arrive(ready_bar((gp + 1) & 1));
           break;
         case K_FIN: gemm_finish<NPAD>(a, w, gp); break;
         case K_ATTN_A:
           alive = attn_tiles_phase<NPAD, HD, TC>(a, layer_of(a, l), scratch, pcache, wt, dbg_cy, first_item_sh, qkv_geom_sh, row_pg_sh, rope_cos_sh,
                                                  rope_sin_sh, ring, tmem_base, abort_flag);
           if (TC && alive) {                                               // the ring's memory is the weight producer's again
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // TMA writes next where these threads wrote
             worker_sync();
-            if (wt == 0) mbar_arrive(attn_done_bar);
+            if (wt == 0) asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(smem_u32(attn_done_sh)), "r"((unsigned)l + 1u) : "memory");
           }
           break;
         case K_ATTN_B: attn_merge_phase<HD>(a, row_pos_sh, wt, abort_flag); break;
@@ -1858,7 +1891,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
         }
         default: break;
       }
-      if (barrier && alive) alive = grid_barrier(a, epoch, abort_flag, wt, ready >= 0 ? ready_bar(ready & 1) : 0u);
+      if (barrier && alive) alive = grid_barrier(a, epoch, abort_flag, wt, ready >= 0 ? ready_bar(kind_of(a, ready)) : 0u);
     }
   }
   if (HSD_PROF(a) && blockIdx.x == 0 && threadIdx.x == 128) for (int i = 0; i < 15; ++i) a.prof[940 + i] = (unsigned long long)dbg_cy[i];

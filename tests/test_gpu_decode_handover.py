@@ -57,6 +57,35 @@ def test_first_pass_on_another_stream_finds_the_buffers_filled(lib):
     assert torch.equal(outs[0], outs[1])
 
 
+# k-blocks of a CTA's part of the down projection, with eight parts of width 256 and a ring of eight slots: some without a
+# second one, one turn less one, one, one and one more, several with a remainder
+@pytest.mark.parametrize("blocks_of_8_parts", [7, 8, 11, 56, 64, 72, 136])
+def test_built_down_projections_of_any_length(lib, blocks_of_8_parts):
+    """Passes of up to four rows build the down projection's activations in the ring slots; the activation producer steps over
+    as many slots and takes up the next projection's tiles behind them."""
+    cfg = inputs.model_cfg(3, 256, 8, 2, 64 * blocks_of_8_parts, 2000, "bf16", head_dim=32)
+    w = inputs.make_weights(cfg, 5, device="cuda")
+    prompt, outs = inputs.make_prompts(cfg["vocab"], 1, 24, 24).cuda(), []
+    for folded in (True, False):
+        eng = lib.Hsd(cfg, w, (1, 3), (2,), max_batch=1, max_seq=160)
+        eng.set_phase_folding(True, folded, True)
+        outs.append(eng.generate(prompt, 100, 3)[0])
+        eng.close()
+    assert torch.equal(outs[0], outs[1])
+
+
+def test_thousands_of_passes(lib):
+    """Hand-overs that fail once in a million fail in long runs: 3000 tokens through 48 layers, about 4000 passes, 148 CTAs."""
+    cfg = inputs.model_cfg(48, 256, 8, 2, 1408, 2000, "bf16", head_dim=32)
+    w = inputs.make_weights(cfg, 5, device="cuda")
+    prompt, outs = inputs.make_prompts(cfg["vocab"], 1, 24, 24).cuda(), []
+    eng = lib.Hsd(cfg, w, (8, 48), (2,), max_batch=1, max_seq=3072)
+    for _ in range(2):
+        outs.append(eng.generate(prompt, 3000, 3)[0])
+    eng.close()
+    assert torch.equal(outs[0], outs[1])
+
+
 def _grid_counters(eng, cfg, max_seq, T, n_levels):
     """The two barrier counters of a context of one sequence (bf16, head size 32, pages of 16): one line of 64 bytes each."""
     from paper_2510_19705_b200 import binding
