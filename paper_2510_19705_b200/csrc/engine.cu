@@ -1117,6 +1117,9 @@ int create_ctx(const hsd_model_desc *models, int n_models, const int32_t *exit_l
   for (int i = 0; ok && i < kTimerPairs; ++i)
     c->timers_ok = c->timers_ok && cudaEventCreate(&c->timers[i].a) == cudaSuccess && cudaEventCreate(&c->timers[i].b) == cudaSuccess;
   int st = ok ? HSD_OK : HSD_E_CUDA;
+  // The buffers are filled on the default stream.  Other streams may neither still be writing to the workspace's memory (a
+  // block that an allocator hands on within a stream) nor start a generation before it is filled: both sides wait.
+  if (!st && cudaDeviceSynchronize() != cudaSuccess) st = HSD_E_CUDA;
   if (!st && (cudaMemset(c->ws + c->status_off, 0, 256) != cudaSuccess || cudaMemset(c->ws + lay.grid_counter, 0, 256) != cudaSuccess))
     st = HSD_E_CUDA;
   c->models.resize(n_models);
@@ -1124,7 +1127,6 @@ int create_ctx(const hsd_model_desc *models, int n_models, const int32_t *exit_l
     st = init_model(c, c->models[mi], &models[mi], lay.model[mi]);
     c->any_tc = c->any_tc || c->models[mi].use_tc || c->models[mi].use_small;
   }
-  // the buffers are filled on the default stream; a generation may run on one that does not wait for it
   if (!st && cudaStreamSynchronize(nullptr) != cudaSuccess) st = HSD_E_CUDA;
   if (st) {
     hsd_destroy(c);

@@ -117,3 +117,26 @@ def test_a_wait_that_runs_out_ends_with_an_error(lib):
     eng = lib.Hsd(cfg, w, (1, 3), (2,), max_batch=1, max_seq=160)
     assert torch.equal(eng.generate(prompt, 24, 3)[0], want)
     eng.close()
+
+
+def test_creation_waits_for_work_on_the_memory_it_is_given(lib):
+    """The workspace may be a block whose last user, on a stream the default one does not wait for, is still writing to it."""
+    cfg = inputs.model_cfg(3, 256, 8, 2, 704, 2000, "bf16", head_dim=32)
+    w = inputs.make_weights(cfg, 5, device="cuda")
+    prompt = inputs.make_prompts(cfg["vocab"], 1, 24, 24).cuda()
+    eng = lib.Hsd(cfg, w, (1, 3), (2,), max_batch=6, max_seq=160)
+    want, size = eng.generate(prompt, 24, 3)[0], eng.workspace.numel()
+    eng.close()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        block = torch.empty(size, dtype=torch.uint8, device="cuda")
+        where = block.data_ptr()
+        torch.cuda._sleep(200_000_000)               # about 0.1 s
+        block.zero_()
+        del block
+        eng = lib.Hsd(cfg, w, (1, 3), (2,), max_batch=6, max_seq=160)
+        assert eng.workspace.data_ptr() == where     # the allocator handed the block on
+        got = eng.generate(prompt, 24, 3)[0]
+    torch.cuda.synchronize()
+    assert torch.equal(got, want)
+    eng.close()
