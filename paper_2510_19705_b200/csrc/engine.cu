@@ -1369,6 +1369,8 @@ int hsd_layer_logits(hsd_ctx *c, const int32_t *token_ids, int n_tokens, const i
   size_t used = 0;                              // bytes of the partials buffer written: the one-launch forward finds it filled with 0xFF
   int st = layer_logits(c, token_ids, n_tokens, layers, n_layers_sel, out_logits, stream, &used);
   if (used && cudaMemsetAsync(c->ws + c->models.back().lay.partials, 0xFF, used, c->stream) != cudaSuccess && !st) st = HSD_E_CUDA;
+  // (after an error as well: the next call may come on another stream, and no stale word may be left for it)
+  if (st && used) cudaStreamSynchronize(c->stream);
   return st ? st : sync_stream(c);
 }
 
