@@ -1393,6 +1393,8 @@ int hsd_set_exit_heads(hsd_ctx *c, const void *const *final_norms, const void *c
                           cudaMemcpyHostToDevice) != cudaSuccess)
       st = HSD_E_CUDA;
   }
+  // a copy from pageable memory returns once it is staged, and the next pass may run on a stream that does not wait for it
+  if (!st && cudaStreamSynchronize(nullptr) != cudaSuccess) st = HSD_E_CUDA;
   return st;
 }
 

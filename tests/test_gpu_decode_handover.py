@@ -140,3 +140,22 @@ def test_creation_waits_for_work_on_the_memory_it_is_given(lib):
     torch.cuda.synchronize()
     assert torch.equal(got, want)
     eng.close()
+
+
+def test_heads_are_in_place_for_a_pass_on_another_stream(lib):
+    """New output heads go up on the default stream; the next pass may run on one that does not wait for that stream."""
+    cfg = inputs.model_cfg(3, 256, 8, 2, 704, 2000, "bf16", head_dim=32)
+    w, other = (inputs.make_weights(cfg, seed, device="cuda") for seed in (5, 6))
+    prompt = inputs.make_prompts(cfg["vocab"], 1, 24, 24).cuda()
+    torch.cuda.synchronize()
+    eng, side = lib.Hsd(cfg, w, (1, 3), (2,), max_batch=1, max_seq=160), torch.cuda.Stream()
+    heads, outs = [[None, None], [{"lm_head": other["lm_head"]}, {"lm_head": other["lm_head"]}]], {}
+    for turn in range(6):
+        for i, h in enumerate(heads):
+            eng.set_exit_heads(h)
+            with torch.cuda.stream(side if turn else torch.cuda.current_stream()):
+                got = eng.generate(prompt, 24, 3)[0]
+            torch.cuda.synchronize()
+            assert torch.equal(got, outs.setdefault(i, got)), (turn, i)
+    assert not torch.equal(outs[0], outs[1])
+    eng.close()
