@@ -174,6 +174,7 @@ gemm_big_kernel(const __grid_constant__ BigGemmArgs args, int n_tiles, int m_til
     // ------------------------------------------------------------------ MMA issuer (one lane of the leader issues)
     if (rank == 0) {
       const bool issuer = elect_one();
+      chain_wait();                                  // (the limit of the waits below is for this kernel's own work)
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
       const uint64_t da0 = umma_desc(s0);
       int s = 0, ci = 0;
