@@ -113,3 +113,34 @@ def test_prompt_residual_sums_are_short_chains(seed):
     want = om.last_logits64[0]
     rel = float(np.linalg.norm(rec["logits"][0] - want) / np.linalg.norm(want))
     assert rel < 1.5e-2, rel
+
+
+@pytest.mark.parametrize("hd,nq,nkv,prompt", [(128, 4, 1, 300), (64, 8, 4, 700)])
+def test_chains_of_early_launches_follow_the_work_before_them(hd, nq, nkv, prompt):
+    """The kernels of a prompt and of layer logits start early, one after the other, but not ahead of what was on the stream
+    before the call: tokens and weights that arrive there right before it, behind 50 ms of other work, are the ones it uses."""
+    cfg = inputs.model_cfg(3, 256, nq, nkv, 704, 1024, "bf16", head_dim=hd)
+    w, other = (inputs.make_weights(cfg, seed, device="cuda") for seed in (11, 12))
+    prompts = inputs.make_prompts(cfg["vocab"], 1, prompt, 3).cuda()
+
+    def flat(weights):
+        return [t for k, v in sorted(weights.items()) for t in ([v] if k != "layers" else [l[n] for l in v for n in sorted(l)])]
+
+    def calls(eng, tokens):
+        return eng.layer_logits(tokens[0, :100].contiguous(), [1, 3]), eng.generate(tokens, 16, 5)[0]
+
+    eng = binding.Hsd(cfg, w, (1, 3), (2,), max_batch=1, max_seq=prompt + 64)
+    want = calls(eng, prompts)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        for late in range(2):                        # before the layer logits, before the prompt
+            right = [t.clone() for t in flat(w)]
+            tokens = torch.zeros_like(prompts)
+            for t, o in zip(flat(w), flat(other)):
+                t.copy_(o)
+            torch.cuda._sleep(100_000_000)
+            for t, r in zip(flat(w), right):
+                t.copy_(r)
+            tokens.copy_(prompts)
+            got = calls(eng, tokens) if late == 0 else (want[0], eng.generate(tokens, 16, 5)[0])
+            assert all(torch.equal(a, b) for a, b in zip(got, want)), late
+    eng.close()
