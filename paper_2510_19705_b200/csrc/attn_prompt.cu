@@ -13,7 +13,11 @@
 // (which put the products into the chain; sixteen softmax warps, or the tiles' exponentials in turns, changed nothing),
 // 284 us this way with one bf16 per weight, 326 us with hi + lo.
 // 320 threads: warps 0-3 / 4-7 = softmax of tile A / B, warp 8 = K / V loader (TMA: a tile per copy and column block;
-// the pages of a tile follow one another in the pool), warp 9 = MMA issue (one elected lane).  Items come longest first.  Every wait is bounded.
+// the pages of a tile follow one another in the pool), warp 9 = MMA issue (one elected lane).  Items come longest first.
+// Every wait is bounded, and no waiter can be passed by (a parity wait sees a completion only until the next one): k_full and
+// v_full have their next loads behind k_free / v_free, which the issuer's commits complete; those their next MMAs behind the
+// loader's tiles; s_full, pv_done (looked at only before a rescale) and o_done theirs behind p_ready of all four softmax warps;
+// p_ready its next weights behind the scores.
 #include <algorithm>
 #include "attn_prompt.cuh"
 #include "gemm_tc.cuh"

@@ -143,9 +143,10 @@ Layout make_layout(const hsd_model_desc *models, int n_models, int n_levels, con
   }
   L.vscratch = take(verify_scratch_bytes(B, sumT + 1));
   L.result = take(kResultHead + (size_t)B * 4);
-  // a slot holds one pass's descriptors (<= 40 bytes a row) and those of the decision after it, or a prompt chunk's row lists (8 bytes a row) and one 16-byte
-  // item per 32 rows of a sequence (8 heads to a KV group, at most) and per sequence
-  L.ring_slot = align_up(std::max((size_t)L.base_rows * 40 + (size_t)B * (96 + sizeof(VerifySeq)), (size_t)L.max_rows * 8 + (size_t)(L.max_rows / 32 + B) * 16) + 1024, 256);
+  // a slot holds one pass's descriptors (<= 40 bytes a row) and those of the decision after it, or a prompt chunk's row
+  // lists (8 bytes a row) and one 16-byte item per 32 rows of a sequence (8 heads to a KV group, at most) and per sequence
+  L.ring_slot = align_up(std::max((size_t)L.base_rows * 40 + (size_t)B * (96 + sizeof(VerifySeq)),
+                                  (size_t)L.max_rows * 8 + (size_t)(L.max_rows / 32 + B) * 16) + 1024, 256);
   L.ring = take(L.ring_slot * kRingSlots);
   L.grid_counter = take(256);
   L.model.resize(n_models);
@@ -1046,8 +1047,6 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
   for (int l = 0; l < md.n_layers; ++l) {
     ld[l].attn_norm = (const __nv_bfloat16 *)M.lw[(size_t)l * 9 + 0];
     ld[l].mlp_norm = (const __nv_bfloat16 *)M.lw[(size_t)l * 9 + 5];
-    ld[l].k_pool = (__nv_bfloat16 *)(c->ws + ml.k_pool + ml.pool_layer_stride * l);
-    ld[l].v_pool = (__nv_bfloat16 *)(c->ws + ml.v_pool + ml.pool_layer_stride * l);
   }
   if (cudaMemcpy(c->ws + ml.wmaps_dev, M.wmaps.data(), M.wmaps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(c->ws + ml.layers_dev, ld.data(), ld.size() * sizeof(FwdLayerDev), cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -1061,8 +1060,8 @@ int init_model(hsd_ctx *c, Model &M, const hsd_model_desc *model, const ModelLay
     M.kvmaps.resize((size_t)md.n_layers * 2);
     const long long rows = (long long)md.nkv * md.n_pages * md.page;
     for (int l = 0; l < md.n_layers && !st; ++l) {
-      st = prompt_attn_map(&M.kvmaps[2 * l], ld[l].k_pool, rows, md.hd);
-      if (!st) st = prompt_attn_map(&M.kvmaps[2 * l + 1], ld[l].v_pool, rows, md.hd);
+      st = prompt_attn_map(&M.kvmaps[2 * l], c->ws + ml.k_pool + ml.pool_layer_stride * l, rows, md.hd);
+      if (!st) st = prompt_attn_map(&M.kvmaps[2 * l + 1], c->ws + ml.v_pool + ml.pool_layer_stride * l, rows, md.hd);
     }
   }
   return st;

@@ -5,8 +5,9 @@
 // phase workers, 8..11 = phase workers only.  The 256 worker threads walk the phase program
 //   embed+norm | QKV(+rope, KV append) | attention | O(+residual) | norm | gate/up(+SwiGLU) |
 //   down(+residual) | norm | ... | final norm | output head
-// with a grid barrier before each projection that takes its activations by TMA; the other phases wait for the words they
-// read (kHole).  The weight producer is not tied to the barriers: weights are
+// with a grid barrier before each projection that takes its activations by TMA, and behind a q / k / v finish of its own:
+// the attention phase reads q and the cache, which are plain stores.  The other phases wait for the words they read
+// (kHole).  The weight producer is not tied to the barriers: weights are
 // read-only, so it runs ahead into the next GEMM as far as the ring allows; the activation producer
 // waits for the barrier that completes its operand.  GEMM work is split evenly over the CTAs in
 // (tile, k-block) units; each segment's partial sums go to a piece buffer and the following phase
@@ -69,7 +70,6 @@ template <int NPAD> struct PCfg {
 
 struct Gemm {
   const CUtensorMap *w[3];
-  const CUtensorMap *amap;
   int seg_n[3];
   int n_segs, K, KB, n_tiles, mode, rows;
 };
@@ -82,19 +82,19 @@ __device__ __forceinline__ Gemm make_gemm(const FwdArgs &a, int p) {
   g.n_segs = 1;
   g.rows = a.R;
   if (l >= a.n_run) {                       // output head
-    g.w[0] = a.wmaps + a.lm_map; g.seg_n[0] = a.V; g.amap = &a.amap[3]; g.K = a.d; g.mode = MODE_LOGITS; g.rows = a.L;
+    g.w[0] = a.wmaps + a.lm_map; g.seg_n[0] = a.V; g.K = a.d; g.mode = MODE_LOGITS; g.rows = a.L;
   } else if (j == 0) {
     const CUtensorMap *m = a.wmaps + l * 7;
     g.w[0] = m; g.w[1] = m + 1; g.w[2] = m + 2;
     g.seg_n[0] = a.nq * a.hd; g.seg_n[1] = g.seg_n[2] = a.nkv * a.hd;
-    g.n_segs = 3; g.amap = &a.amap[0]; g.K = a.d; g.mode = MODE_QKV;
+    g.n_segs = 3; g.K = a.d; g.mode = MODE_QKV;
   } else if (j == 1) {
-    g.w[0] = a.wmaps + l * 7 + 3; g.seg_n[0] = a.d; g.amap = &a.amap[1]; g.K = a.nq * a.hd; g.mode = MODE_ADD;
+    g.w[0] = a.wmaps + l * 7 + 3; g.seg_n[0] = a.d; g.K = a.nq * a.hd; g.mode = MODE_ADD;
   } else if (j == 2) {
     g.w[0] = a.wmaps + l * 7 + 4; g.w[1] = a.wmaps + l * 7 + 5; g.seg_n[0] = g.seg_n[1] = a.ff;
-    g.n_segs = 2; g.amap = &a.amap[0]; g.K = a.d; g.mode = MODE_SWIGLU;
+    g.n_segs = 2; g.K = a.d; g.mode = MODE_SWIGLU;
   } else {
-    g.w[0] = a.wmaps + l * 7 + 6; g.seg_n[0] = a.d; g.amap = &a.amap[2]; g.K = a.ff; g.mode = MODE_ADD;
+    g.w[0] = a.wmaps + l * 7 + 6; g.seg_n[0] = a.d; g.K = a.ff; g.mode = MODE_ADD;
   }
   g.KB = g.K / kTcBlockK;
   if (g.mode == MODE_SWIGLU) g.n_tiles = (g.seg_n[0] + kTcBoxRows - 1) / kTcBoxRows;
@@ -133,8 +133,8 @@ __device__ __forceinline__ int unit_owner(int U, int G, int u) {
 struct Seg { int tile, kb0, kb1; };
 struct SegIter { int tile, kb, left; };        // next k-block (tile, kb) and the k-blocks still to hand out
 // regular: every tile is cut into `parts` equal k-ranges (GEMMs with few tiles: at most four pieces per
-// tile, residual projections residual_parts(), so the consumer can fetch all of them in one batch); otherwise the (tile, k-block) units are
-// dealt out evenly (tiles >= CTAs / 2: a tile then spans at most 3 CTAs).
+// tile, residual projections residual_parts(), so the consumer can fetch all of them in one batch);
+// otherwise the (tile, k-block) units are dealt out evenly (tiles >= CTAs / 2: a tile then spans at most 3 CTAs).
 struct SplitGeom { int U, Gp, pieces_max, parts; };
 // The norm after a residual projection holds a row in registers, 16 float4 loads of pieces per thread at a time: 4 pieces
 // of up to 4096 columns or 8 of up to 2048.  Width 2048 in 4 parts left 84 of 148 CTAs without a tile of O and down
@@ -205,9 +205,9 @@ __device__ __forceinline__ PhaseGeom phase_geom(const Gemm &g, int G, int c) {
 // Phase p is a down projection whose activation tiles are built in place from the gate / up pieces.
 __device__ __forceinline__ bool built_down(const FwdArgs &a, int p) { return a.fuse_gu && (p & 3) == 3 && p < 4 * a.n_run; }
 
-// Handing partial sums to the next phase.  A word of the piece and partial buffers that has not been written holds
-// kHole (a NaN no sum is stored as), and its reader takes it as soon as it holds something else: the data is its own flag.  A counter
-// or barrier in between costs a release that waits until every store of the CTA is in L2 (1 to 1.8 us under the weight
+// Handing partial sums to the next phase.  A word of the piece and partial buffers that has not been written holds kHole
+// (a NaN no sum is stored as), and its reader takes it as soon as it holds something else: the data is its own flag.  A
+// counter or barrier in between costs a release that waits until every store of the CTA is in L2 (1 to 1.8 us under the weight
 // stream), the flag's way, and then the loads; polling the data costs the loads.  Words are accessed with relaxed
 // single-word semantics and depend on no order among themselves.  The words' writer makes them holes again one phase and
 // at least one grid barrier after their readers (put_holes), and at least one grid barrier before the next ones, so
@@ -357,7 +357,9 @@ __device__ __forceinline__ void norm_phase(const FwdArgs &a, int n_rows, const i
                                            float *red, int wt, volatile int *abort_flag) {
   constexpr int PB = 16 / MAXV;                            // pieces per slot (residual_parts)
   const int d = a.d, nvec = d >> 2;
-  const int first = (int)(gridDim.x - 1 - blockIdx.x);      // the last CTAs first: they hold no tile of the projection
+  // the last CTAs first: some hold no tile of the projection.  The other rows fall to CTAs that do; their epilogue warps
+  // write the CTA's words before they come here, so no CTA waits for itself
+  const int first = (int)(gridDim.x - 1 - blockIdx.x);
   for (int i = first; i < n_rows; i += gridDim.x) {
     const int row = row_list ? row_list[i] : i;
     float *xrow = a.x + (size_t)row * d;
@@ -453,15 +455,14 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gsrc) : "memory");
 }
 
-struct LayerNorms { const __nv_bfloat16 *attn, *mlp; };
-__device__ __forceinline__ FwdLayerDev layer_of(const FwdArgs &a, int l) {
-  FwdLayerDev ly;
-  ly.attn_norm = ly.mlp_norm = nullptr;
-  ly.k_pool = reinterpret_cast<__nv_bfloat16 *>(a.k_pool + a.pool_stride * l);
-  ly.v_pool = reinterpret_cast<__nv_bfloat16 *>(a.v_pool + a.pool_stride * l);
-  return ly;
+struct LayerCache { __nv_bfloat16 *k_pool, *v_pool; };
+__device__ __forceinline__ LayerCache cache_of(const FwdArgs &a, int l) {
+  LayerCache lc;
+  lc.k_pool = reinterpret_cast<__nv_bfloat16 *>(a.k_pool + a.pool_stride * l);
+  lc.v_pool = reinterpret_cast<__nv_bfloat16 *>(a.v_pool + a.pool_stride * l);
+  return lc;
 }
-struct PageCache { int tag_item, tag_tile; int pg[128]; };   // pg[warp * 16 + j]: page of the warp's j-th sub-tile
+struct PageCache { int tag_item; int pg[128]; };   // pg[warp * 16 + j]: page of the warp's j-th sub-tile
 
 __device__ __forceinline__ void mma_bf16_16x8x16(float *c, const unsigned *a, unsigned b0, unsigned b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -834,7 +835,7 @@ __device__ __noinline__ bool attn_item_tc(const FwdArgs &a, const __nv_bfloat16 
 // split's partial (o, m, l) goes to global memory.
 // False, in every thread, if a wait of a tensor-memory item gave up.
 template <int NPAD, int HD, bool TC>
-__device__ __forceinline__ bool attn_tiles_phase(const FwdArgs &a, const FwdLayerDev &lay, uint8_t *scratch, PageCache *pc, int wt, long long *dbg,
+__device__ __forceinline__ bool attn_tiles_phase(const FwdArgs &a, const LayerCache &lay, uint8_t *scratch, PageCache *pc, int wt, long long *dbg,
                                                  const int *first_item, const int *qkv_geom, const int *row_pg_sh, const float *rope_cos_sh,
                                                  const float *rope_sin_sh, uint8_t *tc_smem, uint32_t tmem, volatile int *abort_flag) {
   constexpr int CPR = HD / 8;                      // 16-byte chunks per row
@@ -1233,7 +1234,7 @@ __device__ __forceinline__ void attn_merge_phase(const FwdArgs &a, const int *ro
 // ------------------------------------------------------------------------------ epilogue stores
 // v[i] = final value of output feature (tile row m) for token row c0 + i.
 template <int CH>
-__device__ __forceinline__ void final_store(const FwdArgs &a, const Gemm &g, const Tile &ti, const FwdLayerDev &lay, int m, int et,
+__device__ __forceinline__ void final_store(const FwdArgs &a, const Gemm &g, const Tile &ti, const LayerCache &lay, int m, int et,
                                             int c0, const float *v, float *staging, const int *rpos, const int *rpg,
                                             const float *cs, const float *sn, int bar_id) {
   const int rows = g.rows;
@@ -1336,45 +1337,44 @@ __device__ __forceinline__ void put_partial_holes(const FwdArgs &a, int wt, cons
 }
 
 // GEMM phase p, epilogue side (warps 4..7): accumulator -> this CTA's piece of the tile.  Group-uniform:
-// a give-up is decided by one thread and shared. 
-
+// a give-up is decided by one thread and shared.
 template <int NPAD>
 __device__ __forceinline__ void gemm_epilogue(const FwdArgs &a, WorkerCtx &w, int p) {
   constexpr int CH = PCfg<NPAD>::kChunk;
   const int m = w.q * 32 + w.lane;
 
-    const int kind = kind_of(a, p), rows = kind == 4 ? a.L : a.R;
-    const PhaseGeom &pg = w.geom[kind];
-    const bool keep = a.L > 0 || p != 4 * a.n_run - 1;            // a pass without logits ends here: nobody reads these pieces
-    SegIter it = seg_begin(pg);
-    Seg sg;
-    for (; seg_next(pg, it, sg); ++w.seg_idx) {
-      const int ab = w.seg_idx & 1;
-      float *mine = a.pieces[kind] + ((size_t)sg.tile * pg.pieces_max + piece_of(pg, sg)) * NPAD * kTcBlockM;
-      if (w.wt == 0) w.wait_ok[w.seg_idx & 1] = mbar_wait((w.accf_bar0 + 8u * ab), (uint32_t)((w.seg_idx >> 1) & 1), w.abort_flag) ? 1 : 0;
-      epi_sync();
-      if (!w.wait_ok[w.seg_idx & 1]) return;
-      tc_fence_after();
-      const uint32_t tbase = w.tmem_base + ((uint32_t)(w.q * 32) << 16) + (uint32_t)(ab * NPAD);
+  const int kind = kind_of(a, p), rows = kind == 4 ? a.L : a.R;
+  const PhaseGeom &pg = w.geom[kind];
+  const bool keep = a.L > 0 || p != 4 * a.n_run - 1;            // a pass without logits ends here: nobody reads these pieces
+  SegIter it = seg_begin(pg);
+  Seg sg;
+  for (; seg_next(pg, it, sg); ++w.seg_idx) {
+    const int ab = w.seg_idx & 1;
+    float *mine = a.pieces[kind] + ((size_t)sg.tile * pg.pieces_max + piece_of(pg, sg)) * NPAD * kTcBlockM;
+    if (w.wt == 0) w.wait_ok[w.seg_idx & 1] = mbar_wait((w.accf_bar0 + 8u * ab), (uint32_t)((w.seg_idx >> 1) & 1), w.abort_flag) ? 1 : 0;
+    epi_sync();
+    if (!w.wait_ok[w.seg_idx & 1]) return;
+    tc_fence_after();
+    const uint32_t tbase = w.tmem_base + ((uint32_t)(w.q * 32) << 16) + (uint32_t)(ab * NPAD);
 #pragma unroll 1
-      for (int c0 = 0; c0 < NPAD; c0 += CH) {
-        float v[CH];
+    for (int c0 = 0; c0 < NPAD; c0 += CH) {
+      float v[CH];
 #pragma unroll
-        for (int j = 0; j < CH / 16; ++j) tmem_ld16(tbase + c0 + j * 16, v + j * 16);
-        tmem_ld_wait();
-        if (c0 + CH >= NPAD) {                   // accumulator fully read: hand it back to the MMA warp
-          tc_fence_before();
-          __syncwarp();
-          if (w.lane == 0) mbar_arrive((w.acce_bar0 + 8u * ab));
-        }
-        if (c0 < rows && keep) {
+      for (int j = 0; j < CH / 16; ++j) tmem_ld16(tbase + c0 + j * 16, v + j * 16);
+      tmem_ld_wait();
+      if (c0 + CH >= NPAD) {                   // accumulator fully read: hand it back to the MMA warp
+        tc_fence_before();
+        __syncwarp();
+        if (w.lane == 0) mbar_arrive((w.acce_bar0 + 8u * ab));
+      }
+      if (c0 < rows && keep) {
 #pragma unroll
-          for (int i = 0; i < CH; ++i)
-            if (c0 + i < rows) put_word(mine + (c0 + i) * kTcBlockM + m, v[i]);
-        }
+        for (int i = 0; i < CH; ++i)
+          if (c0 + i < rows) put_word(mine + (c0 + i) * kTcBlockM + m, v[i]);
       }
     }
   }
+}
 
 // Down projection p of a pass with at most four rows: the worker warps build its activation tiles straight into
 // the ring slots (SwiGLU of the gate / up pieces, summed in piece order; k-block kb of the down projection is tile
@@ -1399,8 +1399,8 @@ __device__ __forceinline__ void build_act_stages(const FwdArgs &a, WorkerCtx &w,
     const int rem = x - q * Ug;
     return rem < 0 ? q - 1 : (rem >= Ug ? q + 1 : q);
   };
-  // builders: the four worker warps that share no scheduler with the weight producer or the MMA issuer (single
-  // threads whose issue rate bounds the phase)
+  // builders: the four worker warps that share no scheduler with the weight producer or the MMA issuer (whose issue rate
+  // bounds the phase)
   if (it.left <= 0 || ((w.wt >> 5) & 1) == 0) return;
   // ring position (slot, parity of its empty barrier) of the phase's first stage, published by the weight producer
   ring_pos += (p >> 2) & 15;
@@ -1564,7 +1564,7 @@ __device__ __forceinline__ void gemm_finish(const FwdArgs &a, WorkerCtx &w, int 
         cs[i] = csn[i]; sn[i] = snn[i];
       }
       if (c0 + RG < r_hi) fetch(c0 + RG);
-      final_store<RG>(a, g, ti, layer_of(a, layer < a.n_run ? layer : 0), gm, gm, c0, v, gstage, w.row_pos_sh,
+      final_store<RG>(a, g, ti, cache_of(a, layer < a.n_run ? layer : 0), gm, gm, c0, v, gstage, w.row_pos_sh,
                       w.row_pg_sh, cs, sn, 1 + 2 * gidx);
     }
   }
@@ -1599,8 +1599,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
   PageCache *pcache = reinterpret_cast<PageCache *>(ctl + 16);          // 130 words
   int *row_pos_sh = reinterpret_cast<int *>(ctl + 160);                 // [128] position of each packed row
   int *row_pg_sh = reinterpret_cast<int *>(ctl + 288);                  // [128] KV page holding that position
-  LayerNorms *norms_sh = reinterpret_cast<LayerNorms *>(ctl + 416);     // [<= kMaxLayersSh] norm gains
-  static_assert(kMaxLayersSh * sizeof(LayerNorms) <= (672 - 416) * 4, "control area overlap");
+  FwdLayerDev *norms_sh = reinterpret_cast<FwdLayerDev *>(ctl + 416);   // [<= kMaxLayersSh] norm gains
+  static_assert(kMaxLayersSh * sizeof(FwdLayerDev) <= (672 - 416) * 4, "control area overlap");
   long long *dbg_cy = reinterpret_cast<long long *>(reinterpret_cast<uint8_t *>(bars) + kCtrlBytes - 128);   // debug cycle counters [16]
   // cos / sin of the launch's rows (the tables are touched once per layer, so the weight stream would
   // evict them from L2 between uses): [kRopeCacheRows][hd / 2] each, after the attention / staging area
@@ -1626,7 +1626,6 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
     *attn_done_sh = 0u;
     for (int i = 0; i < 16; ++i) ring_pos_sh[i] = 0xFFFFFFFFu;
     pcache->tag_item = -1;
-    pcache->tag_tile = -1;
     if (c == 0) *a.next_counter = 0u;                    // (nobody uses it while this launch runs)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1767,7 +1766,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
 
     // ---- phase program
     if (HSD_PROF(a) && wt == 0) a.prof[(size_t)blockIdx.x * kFwdProfEvents] = globaltimer_ns();
-    for (int l = wt; l < a.n_run; l += 256) { norms_sh[l].attn = a.layers[l].attn_norm; norms_sh[l].mlp = a.layers[l].mlp_norm; }
+    for (int l = wt; l < a.n_run; l += 256) norms_sh[l] = a.layers[l];
     if (a.R <= kRopeCacheRows)
       for (int i = wt; i < a.R * (HD / 2); i += 256) {
         const int r = i / (HD / 2), k = i % (HD / 2);
@@ -1800,10 +1799,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
     //                           7 gate/up finish, barrier -> ready(down) | 8 down pieces | 9 norm (+down pieces), barrier -> ready(next)
     //   t = 1 + 10 n, + 1    output-head pieces | output-head finish
     // Steps 1 and 7 are empty when the finish is folded into the phase after it.  A phase that reads the words of the one
-    // before waits for those words, so there is a grid barrier only before a projection that takes its activations by TMA:
-    // three per layer (five with both finish phases).  Words become holes again under a later projection, behind a barrier
-    // after their last reader and in front of one before their next: QKV, partials and O under gate / up, down under the next
-    // QKV or the head, and so gate / up if folded (otherwise under down).
+    // before waits for those words, so there is a grid barrier only before a projection that takes its activations by TMA,
+    // and behind step 1 (its q and cache rows are plain stores): three per layer, five with both finish phases.  Words become
+    // holes again under a later projection, behind a barrier after their last reader and in front of one before their next:
+    // QKV, partials and O under gate / up, down under the next QKV or the head, and so gate / up if folded (otherwise under
+    // down).
     const int n_steps = 1 + 10 * a.n_run + (a.L > 0 ? 2 : 0);
     enum { K_EPI, K_FIN, K_ATTN_A, K_ATTN_B, K_NORM, K_NONE };
 #pragma unroll 1
@@ -1865,7 +1865,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
           break;
         case K_FIN: gemm_finish<NPAD>(a, w, gp); break;
         case K_ATTN_A:
-          alive = attn_tiles_phase<NPAD, HD, TC>(a, layer_of(a, l), scratch, pcache, wt, dbg_cy, first_item_sh, qkv_geom_sh, row_pg_sh, rope_cos_sh,
+          alive = attn_tiles_phase<NPAD, HD, TC>(a, cache_of(a, l), scratch, pcache, wt, dbg_cy, first_item_sh, qkv_geom_sh, row_pg_sh, rope_cos_sh,
                                                  rope_sin_sh, ring, tmem_base, abort_flag);
           if (TC && alive) {                                               // the ring's memory is the weight producer's again
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // TMA writes next where these threads wrote
@@ -1879,7 +1879,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
           const bool last = !first && (((t - 1) % 10) == 9) && (l + 1 >= a.n_run);      // final norm over the logit rows
           const bool mid = !first && (((t - 1) % 10) == 5);
           const __nv_bfloat16 *gain = first ? a.layers[0].attn_norm
-                                            : (last ? a.final_norm : (mid ? norms_sh[l].mlp : norms_sh[l + 1].attn));
+                                            : (last ? a.final_norm : (mid ? norms_sh[l].mlp_norm : norms_sh[l + 1].attn_norm));
           auto norm = [&](auto slots) {
             norm_phase<NPAD, decltype(slots)::value>(a, last ? a.L : a.R, last ? a.lrow_src : nullptr, first,
                                                      first ? nullptr : a.pieces[gp & 3], geom_sh[gp & 3].pieces_max, gain, last ? a.hf : a.h,
@@ -1921,15 +1921,13 @@ __global__ void __launch_bounds__(256, 2) attn_tiles_kernel(const __grid_constan
   __shared__ long long dbg_cy[16];
   if (threadIdx.x == 0) {
     pcache.tag_item = -1;
-    pcache.tag_tile = -1;
     const int n_work = a.n_attn * a.nkv * a.n_splits;
     int4 fi = make_int4(0, 0, 0, 0);
     if ((int)blockIdx.x < n_work) fi = a.attn_items[blockIdx.x / (a.n_splits * a.nkv)];
     first_item_sh[0] = fi.x; first_item_sh[1] = fi.y; first_item_sh[2] = fi.z; first_item_sh[3] = fi.w;
   }
   __syncthreads();
-  FwdLayerDev lay;
-  lay.attn_norm = nullptr; lay.mlp_norm = nullptr; lay.k_pool = k_pool; lay.v_pool = v_pool;
+  const LayerCache lay = {k_pool, v_pool};
   attn_tiles_phase<128, HD, false>(a, lay, scratch, &pcache, (int)threadIdx.x, dbg_cy, first_item_sh, qkv_geom_sh, nullptr, nullptr, nullptr,
                             nullptr, 0u, nullptr);
 }

@@ -10,7 +10,6 @@ namespace hsd {
 
 struct FwdLayerDev {
   const __nv_bfloat16 *attn_norm, *mlp_norm;
-  __nv_bfloat16 *k_pool, *v_pool;
 };
 
 struct FwdArgs {

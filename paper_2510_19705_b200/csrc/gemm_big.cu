@@ -6,7 +6,10 @@
 // both load their own operands and signal the issuing CTA's barrier.  Warp 0 = TMA producer, warp 1 = TMEM owner and
 // (leader) MMA issuer, then the epilogue; six stages; two 256-column accumulators (all of tensor memory), so a tile's epilogue
 // runs under the next tile's MMAs.  Tiles are dealt round-robin with the token tile fastest: the pairs that work at the same
-// time share weight rows, so a weight tile comes from HBM once.  Every wait is bounded.
+// time share weight rows, so a weight tile comes from HBM once.  Every wait is bounded, and no waiter can be passed by (a
+// parity wait sees a completion only until the next one): full[s] has its next loads behind empty[s], which the issuer's commit
+// completes in both CTAs; empty[s] its next MMAs behind the loads of both producers; acc_full its next MMAs behind acc_empty,
+// which every epilogue warp of the pair completes; acc_empty its next epilogue behind the MMAs.
 // The tensor core's fp32 accumulation loses about as much as its chain is long.  Products for the fp32 residual stream cut K
 // into chains (chain_blocks): the accumulators take turns, eight epilogue warps add each chain's sum to their registers under
 // the next chain's MMAs and put the whole sum back into tensor memory for the finish (a finish straight from the 128

@@ -13,7 +13,10 @@
 // two halves with a TMEM accumulator each, added in fp32 at the end: the tensor core's fp32 accumulation loses about as
 // much as its chain is long (relative error against fp64 at K = 4096: 4.4e-6 in one chain, 2.1e-6 in two).  Every
 // wait is bounded by wall time; a wait that gives up raises a flag, every role leaves its loop, TMEM is freed and a
-// status word tells the host.
+// status word tells the host.  No waiter can be passed by (a parity wait sees a completion only until the next one): full[s]
+// has its next loads behind empty[s], which the MMA issuer's commit completes; empty[s] its next MMAs behind the producer's
+// loads; acc_full its next MMAs behind acc_empty, which all four epilogue warps complete; acc_empty its next epilogue behind
+// the MMAs.
 #include <algorithm>
 #include "gemm_tc.cuh"
 #include "tc_ptx.cuh"
