@@ -1,7 +1,7 @@
 // One-launch forward of small fp32 models: a cooperative kernel runs every layer of a pass.
 //
-// Bound by latency: a four-layer pass of width 128 moves 4 MB, but as one launch per operation it took 206 us (39
-// launches of about 5 us); this way 103 us, 5 us a phase.  Here a layer is five phases with a grid barrier after each:
+// Bound by latency: a four-layer pass of width 128 (4.8 rows) moves 4 MB, but as one launch per operation it took 206 us (39
+// launches of about 5 us); this way 68 us, 3.3 us a phase.  Here a layer is five phases with a grid barrier after each:
 //   q / k / v (RMSNorm of the rows in front, rotary embedding and cache append behind), attention, O + residual,
 //   gate / up (RMSNorm in front, SwiGLU behind), down + residual;
 // the last phase is the final norm + output head over the logit rows.  In a product a warp owns two weight rows (rotary
@@ -381,10 +381,15 @@ template <int HD> int launch_hd(const SmallFwdArgs &a, int grid, cudaStream_t s)
 }  // namespace
 
 // Small: where launches and not weights take the time.  8 MB of weights a layer are about 2 us of the phases' loads on
-// 148 SMs; a larger model streams its weights better with the many CTAs of one launch per operation.  At the line (four
-// layers of width 512, 8.1 MB each, a head of 65 MB; ms a pass, launches per operation / this kernel): one row 0.070 / 0.051,
-// 6 rows 0.267 / 0.172, 16 rows 0.111 / 0.114 (one layer), about 45 rows 0.440 / 0.447 (two layers), 100 0.91 / 0.79, a prompt's
-// 128 2.07 / 1.53.
+// 148 SMs; a much larger model streams its weights better with the many CTAs of one launch per operation.  Passes of models of
+// width 512 to 2048 with a vocabulary of 32000 (us, launches per operation / this kernel; 1 row through one layer, about 25
+// through two, about 43 through four, a prompt's 128 through four):
+//   8.4 MB a layer   81 / 63    384 / 215    1056 / 507     2170 / 815       (just on this kernel's side)
+//   16.7             91 / 83    430 / 265    1267 / 679     2700 / 1256
+//   25.2            111 / 113   533 / 435    1424 / 1006    3000 / 1764
+//   45              129 / 145   577 / 518    1693 / 1336    3720 / 2555
+//   180             209 / 295  1203 / 1251   3321 / 3105    7750 / 6680
+// So the line lies on the safe side: up to about 25 MB next to nothing would be slower in this kernel.
 bool fwd_small_supported(const ModelDims &md) {
   const long long layer = ((long long)md.d * md.hd * (2 * md.nq + 2 * md.nkv) + 3ll * md.d * md.ff) * 4;
   return md.dtype == HSD_F32 && (md.hd == 32 || md.hd == 64 || md.hd == 128) && md.d % 4 == 0 && md.ff % 4 == 0 && (md.nq * md.hd) % 4 == 0 &&
