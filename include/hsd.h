@@ -91,16 +91,15 @@ int hsd_verify_level(int level, const void *target_logits, const void *draft_log
  * allocating call (which may synchronise the whole device) is off limits.  hsd_verify_level
  * makes such callers find scratch memory somewhere; this variant brings its own.
  *
- * Same arguments, outputs and results as hsd_verify_level.  The scratch (row statistics, counters
- * and a queue of sequences) lives in a fixed device array of 98,560 bytes inside the library image (every GPU
+ * Same arguments, outputs and results as hsd_verify_level.  The scratch (row statistics)
+ * lives in a fixed device array of 98,560 bytes inside the library image (every GPU
  * that loads the library holds it until the process exits), which bounds the call:
  * batch * (2 t + 1) <= 4096, else HSD_E_TOO_LARGE (exactly 4096 is accepted).
  * The call performs no cudaMalloc / cudaFree and uses no allocating library routine.
  *   - The first call on each device looks up the array's device address and keeps it; make that
  *     first call outside any stream capture.  The kept address does not survive cudaDeviceReset():
  *     do not use this entry point on a device after resetting it.
- *   - All calls share the one array and it keeps whatever the last call left in it.  The counters
- *     and the queue must start at zero and every call clears them on `stream` before its kernel; the statistics
+ *   - All calls share the one array and it keeps whatever the last call left in it: the statistics
  *     are overwritten before they are read.  Two calls that overlap on the GPU -- different streams,
  *     or different host threads -- race on the array: serialise them (one stream, or an event
  *     between them).

@@ -42,47 +42,7 @@ draft_sample_kernel(const T *__restrict__ logits, int V, const SampleRow *__rest
   if (threadIdx.x == 0) out[d.out_index] = tok;
 }
 
-// ------------------------------------------------------------------------------ row statistics
-// grid (2 * t_max + 1, batch).  Block (r, b): r <= t_max -> target row r; else draft row
-// r - t_max - 1.  Writes the row maximum, the integer total S and the weight of the drafted token.
-template <typename T>
-__global__ void __launch_bounds__(kStatThreads)
-row_stats_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, const int32_t *__restrict__ tokens,
-                 int V, int t_max, const VerifySeq *__restrict__ desc, int regular_t, RowStat *__restrict__ stats) {
-  __shared__ float shf[32];
-  __shared__ u64 sh64[33];
-  int b = blockIdx.y, r = blockIdx.x;
-  VerifySeq d;
-  if (desc) d = desc[b];
-  else { d.t = regular_t; d.p_row0 = (long long)b * (regular_t + 1); d.q_row0 = (long long)b * regular_t; d.tok_off = (long long)b * regular_t; }
-  const T *row;
-  int tok = -1;
-  if (r <= t_max) {
-    if (r > d.t) return;
-    row = p_logits + (size_t)(d.p_row0 + r) * V;
-    if (r < d.t) tok = tokens[d.tok_off + r];
-  } else {
-    int j = r - t_max - 1;
-    if (j >= d.t) return;
-    row = q_logits + (size_t)(d.q_row0 + j) * V;
-    tok = tokens[d.tok_off + j];
-  }
-  float m = row_max(row, V, shf);
-  u64 local = 0;
-  for (int k = threadIdx.x; k < V; k += blockDim.x) local += exp_weight(to_f32(row[k]), m);
-  u64 total;
-  block_exclusive_scan(local, sh64, &total);
-  if (threadIdx.x == 0) {
-    RowStat s;
-    s.m = m;
-    s.S = total;
-    s.Ex = (tok >= 0 && tok < V) ? exp_weight(to_f32(row[tok]), m) : 0u;
-    stats[(size_t)b * (2 * t_max + 1) + r] = s;
-  }
-}
-
-// Same statistics with the whole row held in registers: 16-byte loads, one pass over HBM, packed
-// arithmetic.  Needs V a multiple of the vector width, V <= 8 vectors per thread and 16-byte rows.
+// 16 bytes of a row
 template <typename T> struct StatVec;
 template <> struct StatVec<__nv_bfloat16> {
   static constexpr int N = 8;
@@ -99,75 +59,6 @@ template <> struct StatVec<float> {
     f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y); f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
   }
 };
-constexpr int kStatVecPerThread = 8;
-
-template <typename T>
-__global__ void __launch_bounds__(kStatThreads)
-row_stats_vec_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, const int32_t *__restrict__ tokens,
-                     int V, int t_max, const VerifySeq *__restrict__ desc, int regular_t, RowStat *__restrict__ stats) {
-  constexpr int VN = StatVec<T>::N;
-  __shared__ float shf[32];
-  __shared__ u64 sh64[33];
-  int b = blockIdx.y, r = blockIdx.x;
-  VerifySeq d;
-  if (desc) d = desc[b];
-  else { d.t = regular_t; d.p_row0 = (long long)b * (regular_t + 1); d.q_row0 = (long long)b * regular_t; d.tok_off = (long long)b * regular_t; }
-  const T *row;
-  int tok = -1;
-  if (r <= t_max) {
-    if (r > d.t) return;
-    row = p_logits + (size_t)(d.p_row0 + r) * V;
-    if (r < d.t) tok = tokens[d.tok_off + r];
-  } else {
-    int j = r - t_max - 1;
-    if (j >= d.t) return;
-    row = q_logits + (size_t)(d.q_row0 + j) * V;
-    tok = tokens[d.tok_off + j];
-  }
-  const int nvec = V / VN;
-  const uint4 *row4 = reinterpret_cast<const uint4 *>(row);
-  uint4 regs[kStatVecPerThread];
-#pragma unroll
-  for (int j = 0; j < kStatVecPerThread; ++j) {
-    const int iv = threadIdx.x + kStatThreads * j;
-    regs[j] = iv < nvec ? __ldg(row4 + iv) : make_uint4(0u, 0u, 0u, 0u);
-  }
-  float m = -INFINITY;
-#pragma unroll
-  for (int j = 0; j < kStatVecPerThread; ++j) {
-    if ((int)threadIdx.x + kStatThreads * j < nvec) {
-      float f[VN];
-      StatVec<T>::unpack(regs[j], f);
-#pragma unroll
-      for (int e = 0; e < VN; ++e) m = fmaxf(m, f[e]);
-    }
-  }
-  m = block_max(m, shf);
-  u64 local = 0;
-#pragma unroll
-  for (int j = 0; j < kStatVecPerThread; ++j) {
-    if ((int)threadIdx.x + kStatThreads * j < nvec) {
-      float f[VN];
-      StatVec<T>::unpack(regs[j], f);
-#pragma unroll
-      for (int e = 0; e < VN; e += 2) {
-        u32 e0, e1;
-        exp_weight2(f[e], f[e + 1], m, e0, e1);
-        local += (u64)e0 + (u64)e1;
-      }
-    }
-  }
-  u64 total;
-  block_exclusive_scan(local, sh64, &total);
-  if (threadIdx.x == 0) {
-    RowStat s;
-    s.m = m;
-    s.S = total;
-    s.Ex = (tok >= 0 && tok < V) ? exp_weight(to_f32(row[tok]), m) : 0u;
-    stats[(size_t)b * (2 * t_max + 1) + r] = s;
-  }
-}
-
 // ------------------------------------------------------------------------------ decision
 // One block per sequence: accept tests for all positions (each with its own counter-addressed
 // uniform, so the parallel form equals Algorithm 2's sequential loop with break), n = index of the
@@ -193,8 +84,10 @@ decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, in
   if ((int)threadIdx.x < d.t) {
     int j = threadIdx.x;
     RowStat sp = st[j], sq = st[t_max + 1 + j];
-    u64 Pp = fixed_prob(sp.Ex, prob_scale(sp.S));
-    u64 Pq = fixed_prob(sq.Ex, prob_scale(sq.S));
+    const int tok = tokens[d.tok_off + j];
+    const bool in = tok >= 0 && tok < V;
+    u64 Pp = fixed_prob(in ? exp_weight(to_f32(p_logits[(size_t)(d.p_row0 + j) * V + tok]), sp.m) : 0u, prob_scale(sp.S));
+    u64 Pq = fixed_prob(in ? exp_weight(to_f32(q_logits[(size_t)(d.q_row0 + j) * V + tok]), sq.m) : 0u, prob_scale(sq.S));
     u32 U = uniform24(seed, j, d.serial, d.level, PURPOSE_ACCEPT, d.seq);
     bool ok = (((u64)U * Pq) >> 24) < Pp;                 // u < p(x) / q(x)
     if (coin24 != kNoCoin) ok = U < coin24;               // ablation: IID acceptance with a fixed probability
@@ -249,374 +142,279 @@ decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, in
   }
 }
 
-// ------------------------------------------------------------------------------ fused verification
-// Algorithm 2's decision in ONE launch for bf16 rows: statistics of all p and q rows, the accept tests and the
-// final draw.  Persistent grid, one CTA per SM: a producer thread streams the CTA's rows into a shared-memory
-// ring with bulk copies (so HBM latency hides under the other rows' arithmetic, which is what bounds this
-// kernel: ~16 issue slots per logit for the unfused fp32 exp and the 64-bit sums); the 1024 threads take a row
-// into registers, thread 0 refills the slot with the row three items ahead, and the row is reduced to (max,
-// integer total, weight of the drafted token).
-// Rows are dealt round-robin in sequence-major order, so a sequence's rows finish at about the same time on
-// different SMs; the CTA that delivers a sequence's last row (a counter per sequence) takes that sequence's
-// decision while the rows it needs are still in L2.  No CTA ever waits for another.
-constexpr int kFusedConsumers = 1024;
-constexpr int kFusedThreads = kFusedConsumers;
-constexpr int kFusedSlots = 3;
-constexpr int kFusedVecPerThread = 8;                      // 16-byte vectors of a row per thread of a 512-thread group
-constexpr int kFusedMaxV = 512 * kFusedVecPerThread * 8;
-constexpr uint32_t kFusedPiece = 4096;                     // bytes per bulk copy; 32 of them cover the largest row
-using FusedGroup = WholeBlock;
+// ------------------------------------------------------------------------------ statistics of many rows
+// (maximum, integer total) of every row of a verification, rows dealt to a persistent grid of one CTA per SM.  Bound by
+// fp32 issue: the unfused exponential is 15 packed multiplies and adds a pair of logits, 14.1 cycles a warp and logit per
+// scheduler however it is written (microbenchmark), 1.85 us for 32000 logits on an SM; 64 KB from HBM take 1.4 us.  A warp
+// of its own brings the rows into a ring of 32 KB chunks; with a row's first chunk it publishes where the statistics go and
+// the elements in front of and behind the row's 16-byte vectors, so that rows may begin on any element.  GROUPS groups of
+// WARPS warps take the CTA's rows in turn, each with its own barrier, so that one's reductions and waits (0.7 us a row, as
+// much as a row of 2048 logits has of arithmetic) run under the others' exponentials.  A row stays in the ring between its
+// maximum and its sum; rows of more chunks than the ring has come through it twice.
+constexpr uint32_t kRsPiece = 2048;                        // bytes; a chunk is asked for by its first lanes (a single large copy runs at a fraction of an SM's bandwidth)
+constexpr uint32_t kRsBytes = 229376;                      // of the ring
+constexpr int kRsMaxEdge = 16;
 
-struct FusedArgs {
-  const __nv_bfloat16 *p, *q;
-  int32_t *tokens;
-  int V, t_max, batch;
+struct RowStatArgs {
+  const void *p, *q;
+  int V, t_max, batch, regular_t;
   const VerifySeq *desc;
-  int regular_t;
-  u32 regular_serial, regular_level;
   RowStat *stats;
-  unsigned *counters;            // zero on entry: [batch] rows delivered per sequence | queue length | tickets drawn |
-                                 // [batch] queue of sequences ready for their decision (b + 1)
-  u64 seed;
-  int32_t *out_tokens, *out_n;
-  int write_in_place;
-  u32 coin24;
-  int *status;                   // optional: set to 1 if a bounded wait gave up
+};
+struct RsInfo {
+  int stat;                                                // index of the row's statistics, -1: no more rows
+  int n_vec, n_edge;
+  float edge[kRsMaxEdge];
 };
 
-__device__ __forceinline__ VerifySeq fused_seq(const FusedArgs &a, int b) {
-  VerifySeq d;
-  if (a.desc) return a.desc[b];
-  d.t = a.regular_t; d.p_row0 = (long long)b * (a.regular_t + 1); d.q_row0 = (long long)b * a.regular_t;
-  d.tok_off = (long long)b * a.regular_t; d.serial = a.regular_serial; d.seq = b; d.level = a.regular_level;
-  return d;
-}
-
-__device__ __forceinline__ void bulk_load_row(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
+template <typename T> __device__ __forceinline__ uint4 rs_pad();                 // a vector of -inf: weight 0, never the maximum of a row
+template <> __device__ __forceinline__ uint4 rs_pad<float>() { return make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u); }
+template <> __device__ __forceinline__ uint4 rs_pad<__nv_bfloat16>() { return make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u); }
+// maximum of the vectors' elements so far (bf16: of packed pairs, which is exact)
+template <typename T> struct RsMax;
+template <> struct RsMax<float> {
+  float m = -INFINITY;
+  __device__ void take(const uint4 &v) {
+    m = fmaxf(fmaxf(fmaxf(m, __uint_as_float(v.x)), __uint_as_float(v.y)), fmaxf(__uint_as_float(v.z), __uint_as_float(v.w)));
+  }
+  __device__ float get() const { return m; }
+};
+template <> struct RsMax<__nv_bfloat16> {
+  __nv_bfloat162 m = __floats2bfloat162_rn(-INFINITY, -INFINITY);
+  __device__ void take(const uint4 &v) {
+    const __nv_bfloat162 a = __hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&v.x), *reinterpret_cast<const __nv_bfloat162 *>(&v.y));
+    const __nv_bfloat162 b = __hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&v.z), *reinterpret_cast<const __nv_bfloat162 *>(&v.w));
+    m = __hmax2(m, __hmax2(a, b));
+  }
+  __device__ float get() const { return fmaxf(__low2float(m), __high2float(m)); }
+};
 
-// Inverse CDF over weight(i) of the thread's own 32 tokens, as block_inverse_cdf_chunk, except that the walk
-// through the owning thread's chunk is done by warp 0 together: lane i recomputes the weight of the chunk's
-// token i from global memory (weight_at(k)), a warp scan finds the first token whose inclusive sum passes the
-// threshold.  Integer weights, so the recomputed values are the same.
-template <class WeightFn, class WeightAt>
-__device__ __forceinline__ int fused_inverse_cdf(int V, int k0, u32 U, WeightFn weight, WeightAt weight_at, u64 *sh64 /*[34]*/,
-                                                 int *sh_owner) {
-  u64 local = 0;
-#pragma unroll
-  for (int i = 0; i < kChunkTokens; ++i)
-    if (k0 + i < V) local += weight(i);
-  u64 total;
-  const u64 excl = block_exclusive_scan<FusedGroup>(local, sh64, &total);
-  if (total == 0) return -1;                               // uniform
-  const u64 tau = cdf_threshold(U, total);
-  if (tau >= excl && tau < excl + local) {                 // exactly one thread
-    *sh_owner = threadIdx.x;
-    sh64[33] = excl;
-  }
-  FusedGroup::sync();
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x, k = *sh_owner * kChunkTokens + lane;
-    u64 c = k < V ? weight_at(k) : 0ull;
-    for (int o = 1; o < 32; o <<= 1) {
-      const u64 n = __shfl_up_sync(0xFFFFFFFFu, c, o);
-      if (lane >= o) c += n;
-    }
-    const unsigned hit = __ballot_sync(0xFFFFFFFFu, c + sh64[33] > tau && k < V);
-    if (lane == 0) *sh_owner = *sh_owner * kChunkTokens + (__ffs(hit) - 1);
-  }
-  FusedGroup::sync();
-  const int r = *sh_owner;
-  FusedGroup::sync();
-  return r;
-}
-
-// The decision of sequence b (the whole CTA): accept tests on the row statistics, then the final draw from the
-// residual of the first rejected position, or from the last target row.
-__device__ __forceinline__ void fused_decide(const FusedArgs &a, int b, const VerifySeq &d, u64 *sh64, int *sh_int /*[2]*/) {
-  const int tid = threadIdx.x, V = a.V, t_max = a.t_max;
-  const RowStat *st = a.stats + (size_t)b * (2 * t_max + 1);
-  if (tid == 0) sh_int[1] = d.t;
-  FusedGroup::sync();
-  if (tid < d.t) {
-    const int j = tid;
-    const float4 rp = __ldcg(reinterpret_cast<const float4 *>(st + j)), rq = __ldcg(reinterpret_cast<const float4 *>(st + t_max + 1 + j));
-    const RowStat sp = *reinterpret_cast<const RowStat *>(&rp), sq = *reinterpret_cast<const RowStat *>(&rq);
-    const u64 Pp = fixed_prob(sp.Ex, prob_scale(sp.S)), Pq = fixed_prob(sq.Ex, prob_scale(sq.S));
-    const u32 U = uniform24(a.seed, j, d.serial, d.level, PURPOSE_ACCEPT, d.seq);
-    bool ok = (((u64)U * Pq) >> 24) < Pp;                  // u < p(x) / q(x)
-    if (a.coin24 != kNoCoin) ok = U < a.coin24;            // ablation: IID acceptance with a fixed probability
-    if (!ok) atomicMin(&sh_int[1], j);
-  }
-  FusedGroup::sync();
-  const int n = sh_int[1];
-  FusedGroup::sync();                                      // sh_int[1] is reused by the draw
-  const u32 U = uniform24(a.seed, 0, d.serial, d.level, PURPOSE_FINAL, d.seq);
-  const __nv_bfloat16 *prow = a.p + (size_t)(d.p_row0 + n) * V;
-  const float4 rpn = __ldcg(reinterpret_cast<const float4 *>(st + n));
-  const RowStat spn = *reinterpret_cast<const RowStat *>(&rpn);
-  const float mp = spn.m;
-  const int k0 = tid * kChunkTokens;
-  const Chunk32 cp = chunk_load(prow, V, k0);
-  int m_tok = -1;
-  if (n < d.t) {
-    const __nv_bfloat16 *qrow = a.q + (size_t)(d.q_row0 + n) * V;
-    const Chunk32 cq = chunk_load(qrow, V, k0);
-    const float4 rqn = __ldcg(reinterpret_cast<const float4 *>(st + t_max + 1 + n));
-    const RowStat sqn = *reinterpret_cast<const RowStat *>(&rqn);
-    const ProbScale psp = prob_scale(spn.S), psq = prob_scale(sqn.S);
-    const float mq = sqn.m;
-    auto residual = [&](float lp, float lq) {                // both rows' weights in one packed evaluation
-      u32 ep, eq;
-      exp_weight2m(lp, lq, mp, mq, ep, eq);
-      const u64 Pp = fixed_prob(ep, psp), Pq = fixed_prob(eq, psq);
-      return Pp > Pq ? Pp - Pq : 0ull;
-    };
-    m_tok = fused_inverse_cdf(V, k0, U, [&](int i) { return residual(chunk_get(cp, i), chunk_get(cq, i)); },
-                              [&](int k) { return residual(__bfloat162float(prow[k]), __bfloat162float(qrow[k])); }, sh64, &sh_int[1]);
-  }
-  if (m_tok < 0)   // bonus token, or an all-zero residual: draw from the verifier's own row
-    m_tok = fused_inverse_cdf(V, k0, U, [&](int i) { return (u64)exp_weight(chunk_get(cp, i), mp); },
-                              [&](int k) { return (u64)exp_weight(__bfloat162float(prow[k]), mp); }, sh64, &sh_int[1]);
-  if (tid == 0) {
-    a.out_n[b] = n;
-    if (a.write_in_place) a.tokens[d.tok_off + n] = m_tok;
-  }
-  if (a.out_tokens) {
-    for (int j = tid; j <= t_max; j += kFusedConsumers) {
-      int v = -1;
-      if (j < n) v = a.tokens[d.tok_off + j];
-      else if (j == n) v = m_tok;
-      a.out_tokens[(size_t)b * (t_max + 1) + j] = v;
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kFusedThreads, 1) verify_fused_kernel(const __grid_constant__ FusedArgs a) {
-  extern __shared__ uint8_t fused_smem_raw[];
-  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(fused_smem_raw) + 127) & ~(uintptr_t)127);
-  const uint32_t row_bytes = (uint32_t)a.V * 2u, slot_bytes = (row_bytes + 127u) & ~127u;
-  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)kFusedSlots * slot_bytes);   // full[S][2]
-  __shared__ float shf[2][16];
-  __shared__ u64 sh64[34];                   // row phase: [g * 16 + warp]; decisions: the block scan's scratch
-  __shared__ int sh_flag[2];
+template <typename T, int GROUPS, int WARPS, int CHUNK>
+__global__ void __launch_bounds__(32 * (GROUPS * WARPS + 1), 1) row_stats_kernel(const __grid_constant__ RowStatArgs a) {
+  constexpr int kRsRing = (int)kRsBytes / CHUNK, kRsChunkVecs = CHUNK / 16;
+  constexpr uint32_t kRsChunk = CHUNK;
+  static_assert(CHUNK <= 32 * (int)kRsPiece && CHUNK % 16 == 0);
+  extern __shared__ uint8_t rs_smem_raw[];
+  uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(rs_smem_raw) + 127) & ~(uintptr_t)127);
+  // full, per group | empty, per slot of the ring | a row's maxima, per group.  A parity wait tells a barrier's phases apart
+  // only one phase back, so a barrier's phases all belong to one waiter, which waits for each: chunk y of a group completes
+  // barrier y mod kRsRing of that group, and only the producer waits for "empty".
+  __shared__ __align__(8) uint64_t bars[kRsRing * (GROUPS + 1) + GROUPS];
+  __shared__ RsInfo infos[kRsRing];
+  __shared__ int sh_max[GROUPS][2][WARPS];                 // order keys
+  __shared__ u64 sh_sum[GROUPS][2][WARPS];
   __shared__ int sh_abort;
-  const uint32_t bar0 = ptx::smem_u32(bars);
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int rows_per_seq = 2 * a.t_max + 1, n_items = a.batch * rows_per_seq;
-  if (tid == 0) {
-    for (int s = 0; s < 2 * kFusedSlots; ++s) ptx::mbar_init(bar0 + 8u * s, 1);
+  constexpr int ES = (int)sizeof(T), VN = 16 / ES, THREADS = 32 * WARPS;
+  const int lane = threadIdx.x & 31, warp = ptx::warp_index();
+  const uint32_t full0 = ptx::smem_u32(bars), empty = full0 + 8u * kRsRing * GROUPS, ring0 = ptx::smem_u32(ring);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kRsRing * GROUPS; ++s) ptx::mbar_init(full0 + 8u * s, 1);
+    for (int s = 0; s < kRsRing + GROUPS; ++s) ptx::mbar_init(empty + 8u * s, WARPS);
     sh_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   volatile int *abort_flag = &sh_abort;
-  // item i = (sequence b, row r): r <= t_max: target row r (valid if r <= t_b); else draft row r - t_max - 1 (valid if < t_b)
-  auto row_of = [&](int i, VerifySeq &d, int &b, int &r) -> const __nv_bfloat16 * {
-    b = i / rows_per_seq; r = i - b * rows_per_seq;
-    d = fused_seq(a, b);
-    if (r <= a.t_max) return r <= d.t ? a.p + (size_t)(d.p_row0 + r) * a.V : nullptr;
-    const int j = r - a.t_max - 1;
-    return j < d.t ? a.q + (size_t)(d.q_row0 + j) * a.V : nullptr;
-  };
-  // Rows.  The CTA's valid items, numbered k = 0, 1, ..., go to its two groups of 512 threads in turn (group
-  // k & 1) through ring slot k % 3; each group has its own barrier, so one group's reductions and global round
-  // trips run under the other group's arithmetic.  The group that has taken item k out of its slot asks for item
-  // k + 3 (4 KiB bulk copies, one per lane of the group's first warp: a single 64 KB copy runs at a fraction
-  // of an SM's bandwidth).
-  const int grp = tid >> 9, gtid = tid & 511, gwarp = gtid >> 5, bar_id = 1 + grp;
-  auto group_sync = [&]() { asm volatile("bar.sync %0, 512;" ::"r"(bar_id) : "memory"); };
-  // A slot's uses alternate between the groups, and a parity wait tells a barrier's phases apart only one phase
-  // back, so each slot has two "full" barriers used in turn: a barrier's phases then all belong to one group, which
-  // takes them in order.
-  auto full_bar = [&](int k) { return bar0 + 8u * (uint32_t)((k % kFusedSlots) * 2 + ((k / kFusedSlots) & 1)); };
-  int f_idx = blockIdx.x, f_ord = 0;                        // fetch cursor: next item index to look at, valid items passed so far
-  auto fetch_ordinal = [&](int want) {                      // all lanes of a warp; asks for valid item number `want`, if it exists
-    while (f_idx < n_items) {
-      VerifySeq d; int b, r;
-      const __nv_bfloat16 *row = row_of(f_idx, d, b, r);
-      f_idx += gridDim.x;
-      if (!row) continue;
-      if (f_ord++ < want) continue;
-      const int slot = want % kFusedSlots;
-      const uint32_t bar = full_bar(want);
-      if (lane == 0) ptx::mbar_expect_tx(bar, row_bytes);
-      __syncwarp();
-      const uint32_t off = (uint32_t)lane * kFusedPiece;
-      if (off < row_bytes)
-        bulk_load_row(ptx::smem_u32(smem + (size_t)slot * slot_bytes) + off, reinterpret_cast<const uint8_t *>(row) + off,
-                      min(kFusedPiece, row_bytes - off), bar);
-      return;
+  // A row is n_chunks chunks (the last may be empty).  In the ring's order row k of the CTA begins at chunk k passes n_chunks.
+  const int n_chunks = max(1, (int)(((long long)a.V * ES + kRsChunk - 1) / kRsChunk));
+  const bool resident = n_chunks <= kRsRing;
+  const int passes = resident ? 1 : 2;
+  if (warp == GROUPS * WARPS) {
+    // ---- the rows of this CTA, in order
+    chain_wait();
+    chain_next();
+    const int rows_per_seq = 2 * a.t_max + 1, n_items = a.batch * rows_per_seq;
+    uint32_t slot = 0, phase = 0;                          // of the next chunk
+    auto advance = [&]() { if (++slot == kRsRing) { slot = 0; phase ^= 1u; } };
+    uint32_t sent[GROUPS], group = 0;                      // chunks of each group so far (mod kRsRing); the next row's group
+#pragma unroll
+    for (int g = 0; g < GROUPS; ++g) sent[g] = 0;
+    bool ok = true;
+    for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+      const int b = i / rows_per_seq, r = i - b * rows_per_seq;
+      const bool is_p = r <= a.t_max;
+      const int at = is_p ? r : r - a.t_max - 1;
+      long long row0;
+      if (a.desc) {
+        const int t = a.desc[b].t;
+        if (at >= t + (is_p ? 1 : 0)) continue;
+        row0 = is_p ? a.desc[b].p_row0 : a.desc[b].q_row0;
+      } else row0 = (long long)b * (a.regular_t + (is_p ? 1 : 0));
+      const T *row = reinterpret_cast<const T *>(is_p ? a.p : a.q) + (size_t)(row0 + at) * a.V;
+      const uintptr_t lo = reinterpret_cast<uintptr_t>(row), hi = lo + (size_t)a.V * ES;
+      const uintptr_t v0 = min((lo + 15) & ~(uintptr_t)15, hi), v1 = max(hi & ~(uintptr_t)15, v0);   // the whole vectors
+      const size_t bytes = v1 - v0;
+      const int head = (int)(v0 - lo) / ES, n_edge = head + (int)(hi - v1) / ES;
+      uint32_t y = 0;
+#pragma unroll
+      for (int g = 0; g < GROUPS; ++g)
+        if (g == (int)group) y = sent[g];
+      for (int ps = 0; ps < passes && ok; ++ps)
+        for (int c = 0; c < n_chunks; ++c, advance()) {
+          ok = ptx::mbar_wait_warp(empty + 8u * slot, phase ^ 1u, abort_flag);
+          if (!ok) break;
+          if (c == 0) {
+            if (lane == 0) { infos[slot].stat = i; infos[slot].n_vec = (int)(bytes / 16); infos[slot].n_edge = n_edge; }
+            if (lane < n_edge) infos[slot].edge[lane] = to_f32(lane < head ? row[lane] : reinterpret_cast<const T *>(v1)[lane - head]);
+            __syncwarp();
+          }
+          const size_t off = (size_t)c * kRsChunk;
+          const uint32_t n = off < bytes ? (uint32_t)min((size_t)kRsChunk, bytes - off) : 0u, po = (uint32_t)lane * kRsPiece;
+          const uint32_t full = full0 + 8u * (group * kRsRing + y);
+          if (++y == kRsRing) y = 0;
+          if (lane == 0) { if (n) ptx::mbar_expect_tx(full, n); else ptx::mbar_arrive(full); }
+          __syncwarp();
+          if (po < n) bulk_load(ring0 + slot * kRsChunk + po, reinterpret_cast<const void *>(v0 + off + po), min(kRsPiece, n - po), full);
+        }
+#pragma unroll
+      for (int g = 0; g < GROUPS; ++g)
+        if (g == (int)group) sent[g] = y;
+      if (++group == GROUPS) group = 0;
     }
-  };
-  if (tid < 32) {                                           // items 0, 1, 2; afterwards group 0 asks for 3, 5, ..., group 1 for 4, 6, ...
-    for (int k = 0; k < kFusedSlots; ++k) fetch_ordinal(k);
-    f_idx = blockIdx.x; f_ord = 0;                          // group 0's own cursor starts over (its next request is item 3)
+    for (int e = 0; e < GROUPS && ok; ++e) {               // "no more rows", to each group: a row without data, whose other chunks pass by
+      uint32_t y = 0;
+#pragma unroll
+      for (int g = 0; g < GROUPS; ++g)
+        if (g == (int)group) y = sent[g];
+      for (int c = 0; c < passes * n_chunks; ++c, advance()) {
+        ok = ptx::mbar_wait_warp(empty + 8u * slot, phase ^ 1u, abort_flag);
+        if (!ok) break;
+        if (c == 0 && lane == 0) { infos[slot].stat = -1; ptx::mbar_arrive(full0 + 8u * (group * kRsRing + y)); }
+        if (c > 0 && lane < WARPS) ptx::mbar_arrive(empty + 8u * slot);
+        __syncwarp();
+      }
+      if (++group == GROUPS) group = 0;
+    }
+    if (!ok) {
+      // copies already asked for must land before the CTA's shared memory goes away (bounded: 20 us are far longer than one takes)
+      const unsigned long long t0 = ptx::globaltimer_ns();
+      while (ptx::globaltimer_ns() - t0 < 20000ull) {}
+    }
+    return;
   }
-  const int nvec = a.V >> 3;
-  int ord = 0;                                              // valid items of this CTA seen so far
-  unsigned pending_before = 0u, pending_last = 0xFFFFFFFFu; // the row counter's old value of the group's previous item (thread 0 of the group)
-  int pending_b = -1;
-  auto settle = [&]() {                                     // group thread 0: was the previous item its sequence's last row?
-    if (pending_b >= 0 && pending_before == pending_last) {
-      // the sequence is ready for its decision: append it to the queue (entry = b + 1; 0 = not yet written)
-      const unsigned at = atomicAdd(&a.counters[a.batch], 1u);
-      asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.counters + a.batch + 2 + at), "r"((unsigned)pending_b + 1u) : "memory");
-    }
-    pending_b = -1;
+  // ---- the exponentials
+  const int group = warp / WARPS, gwarp = warp - group * WARPS, gtid = gwarp * 32 + lane;
+  const uint32_t maxima = empty + 8u * (kRsRing + group), full = full0 + 8u * kRsRing * group;
+  uint32_t slot = (uint32_t)(group * passes * n_chunks) % kRsRing, y = 0, phase = 0;    // the next chunk: its slot, its barrier and phase
+  const uint32_t others = (uint32_t)((GROUPS - 1) * passes * n_chunks) % kRsRing;      // slots of the other groups' rows in between
+  auto next_slot = [&](uint32_t n) { slot += n; if (slot >= kRsRing) slot -= kRsRing; };
+  auto wait_chunk = [&]() {
+    const bool there = ptx::mbar_wait_warp(full + 8u * y, phase, abort_flag);
+    if (++y == kRsRing) { y = 0; phase ^= 1u; }
+    return there;
   };
-  for (int i = blockIdx.x; i < n_items; i += gridDim.x) {
-    VerifySeq d; int b, r;
-    const __nv_bfloat16 *row = row_of(i, d, b, r);
-    if (!row) continue;
-    const int k = ord++;
-    if ((k & 1) != grp) continue;
-    const int s = k % kFusedSlots;
-    const uint32_t par = (uint32_t)(k / (2 * kFusedSlots)) & 1u;
-    // the drafted token's logit (the group's thread 0 only), asked for before the wait
-    int tok = -1;
-    if (r < d.t) tok = a.tokens[d.tok_off + r];
-    else if (r > a.t_max) tok = a.tokens[d.tok_off + (r - a.t_max - 1)];
-    float l_tok = 0.f;
-    const bool has_tok = tok >= 0 && tok < a.V;
-    if (gtid == 0 && has_tok) l_tok = __bfloat162float(row[tok]);
-    if (lane == 0) ptx::mbar_wait(full_bar(k), par, abort_flag);       // a give-up raises the CTA's abort flag
+  auto chunk_done = [&]() {
     __syncwarp();
-    const uint4 *src = reinterpret_cast<const uint4 *>(smem + (size_t)s * slot_bytes);
-    uint4 regs[kFusedVecPerThread];
+    if (lane == 0) ptx::mbar_arrive(empty + 8u * slot);
+  };
+  // f(vector) for the group's vectors of the chunk that is at hand; `left`: vectors of the row from the chunk's first on
+  auto vectors = [&](int left, auto &&f) {
+    const uint4 *src = reinterpret_cast<const uint4 *>(ring + (size_t)slot * kRsChunk) + gtid;
+#pragma unroll 1
+    for (int j = 0; j < kRsChunkVecs; j += 4 * THREADS) {
+      if (left >= j + 4 * THREADS) {
+        uint4 x[4];
 #pragma unroll
-    for (int j = 0; j < kFusedVecPerThread; ++j) {
-      const int iv = gtid + 512 * j;
-      regs[j] = iv < nvec ? src[iv] : make_uint4(0u, 0u, 0u, 0u);
-    }
-    group_sync();                                           // every thread holds its part of the row: the slot is free
-    if (*abort_flag) break;                                 // uniform over the group: raised before the barrier
-    if (gwarp == 0) fetch_ordinal(k + kFusedSlots);
-    // the row maximum on the packed pairs (the maximum of bf16 values is one of them: exact)
-    __nv_bfloat162 mx2 = __floats2bfloat162_rn(-INFINITY, -INFINITY);
+        for (int e = 0; e < 4; ++e) x[e] = src[j + e * THREADS];
 #pragma unroll
-    for (int j = 0; j < kFusedVecPerThread; ++j) {
-      if (gtid + 512 * j < nvec) {
-        const uint4 r4 = regs[j];
-        mx2 = __hmax2(mx2, *reinterpret_cast<const __nv_bfloat162 *>(&r4.x));
-        mx2 = __hmax2(mx2, *reinterpret_cast<const __nv_bfloat162 *>(&r4.y));
-        mx2 = __hmax2(mx2, *reinterpret_cast<const __nv_bfloat162 *>(&r4.z));
-        mx2 = __hmax2(mx2, *reinterpret_cast<const __nv_bfloat162 *>(&r4.w));
+        for (int e = 0; e < 4; ++e) f(x[e]);
+      } else {
+#pragma unroll 1
+        for (int e = j; e < min(left, j + 4 * THREADS); e += THREADS) f(e + gtid < left ? src[e] : rs_pad<T>());
+        return;
       }
     }
-    float m = fmaxf(__low2float(mx2), __high2float(mx2));
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    if (lane == 0) shf[grp][gwarp] = m;
-    group_sync();
-    m = shf[grp][lane & 15];
-    for (int o = 8; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+  };
+  auto finish = [&](int stat, float m, int k) {            // a warp: the total of the group's row k
+    u64 s = lane < WARPS ? sh_sum[group][k & 1][lane] : 0ull;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    if (lane == 0) { RowStat st; st.m = m; st.S = s; a.stats[stat] = st; }
+  };
+  int last_stat = -1, k = 0;
+  float last_m = 0.f;
+  for (;; ++k) {
+    if (!wait_chunk()) return;
+    const int stat = infos[slot].stat, n_vec = infos[slot].n_vec, n_edge = infos[slot].n_edge;
+    RsMax<T> mx;
+    float edge = -INFINITY;
+    if (stat >= 0) {
+      if (gtid < n_edge) edge = infos[slot].edge[gtid];
+      const uint32_t slot0 = slot;
+      for (int c = 0; c < n_chunks; ++c) {
+        if (c > 0 && !wait_chunk()) return;
+        vectors(n_vec - c * kRsChunkVecs, [&](const uint4 &x) { mx.take(x); });
+        if (!resident) chunk_done();
+        next_slot(1);
+      }
+      if (resident) slot = slot0;
+    } else chunk_done();
+    // the row's maxima and the last row's totals cross the group
+    const int key = __reduce_max_sync(0xFFFFFFFFu, order_key(fmaxf(mx.get(), edge)));
+    if (lane == 0) { sh_max[group][k & 1][gwarp] = key; ptx::mbar_arrive(maxima); }
+    __syncwarp();
+    if (!ptx::mbar_wait_warp(maxima, (uint32_t)k & 1u, abort_flag)) return;
+    if (last_stat >= 0 && gwarp == k % WARPS) finish(last_stat, last_m, k - 1);
+    if (stat < 0) return;
+    const float m = order_value(__reduce_max_sync(0xFFFFFFFFu, sh_max[group][k & 1][lane % WARPS]));
     u64 local = 0;
+    if (n_edge > 0) local += exp_weight(edge, m);
+    for (int c = 0; c < n_chunks; ++c) {
+      if (!resident && !wait_chunk()) return;
+      vectors(n_vec - c * kRsChunkVecs, [&](const uint4 &x) {
+        float f[VN];
+        StatVec<T>::unpack(x, f);
 #pragma unroll
-    for (int j = 0; j < kFusedVecPerThread; ++j) {
-      if (gtid + 512 * j < nvec) {
-        float f[8];
-        StatVec<__nv_bfloat16>::unpack(regs[j], f);
-#pragma unroll
-        for (int e = 0; e < 8; e += 2) {
+        for (int e = 0; e < VN; e += 2) {
           u32 e0, e1;
           exp_weight2(f[e], f[e + 1], m, e0, e1);
           local += (u64)e0 + (u64)e1;
         }
-      }
+      });
+      chunk_done();
+      next_slot(1);
     }
-    for (int o = 16; o > 0; o >>= 1) local += __shfl_xor_sync(0xFFFFFFFFu, local, o);
-    if (lane == 0) sh64[grp * 16 + gwarp] = local;
-    group_sync();
-    if (gtid == 0) {
-      u64 total = 0;
-#pragma unroll
-      for (int w = 0; w < 16; ++w) total += sh64[grp * 16 + w];
-      settle();                                             // the previous item's counter value has long arrived
-      RowStat st;
-      st.m = m; st.S = total; st.Ex = has_tok ? exp_weight(l_tok, m) : 0u;
-      a.stats[(size_t)b * rows_per_seq + r] = st;
-      // the statistics are ordered before the count by the release (and the other rows' statistics before whatever
-      // follows a look at its old value, which happens one item later, by the acquire)
-      asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(pending_before) : "l"(a.counters + b) : "memory");
-      pending_b = b;
-      pending_last = (unsigned)(2 * d.t);                   // 2 t + 1 rows per sequence
-    }
-    // (the next item's first barrier keeps the other threads from overwriting sh64 / shf before thread 0 has read them)
-  }
-  if (gtid == 0) settle();
-  // Decisions.  Taking one where its last row arrives would chain: the CTA that decides delivers its next rows
-  // late, so it is the last arriver of those sequences too.  Instead every CTA, once its rows are done, draws
-  // tickets until all `batch` decisions are handed out; a ticket whose entry is not written yet waits for it
-  // (bounded): the rows it waits for are never this CTA's own.
-  for (;;) {
-    __syncthreads();
-    if (tid == 0) {
-      int b = -1;
-      if (!*abort_flag) {
-        const unsigned t = atomicAdd(&a.counters[a.batch + 1], 1u);
-        if (t < (unsigned)a.batch) {
-          const unsigned *entry = a.counters + a.batch + 2 + t;
-          unsigned v = 0;
-          unsigned long long t0 = 0;
-          for (uint32_t it = 0;; ++it) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(entry) : "memory");
-            if (v != 0u) break;
-            if ((it & 31u) == 31u) {
-              const unsigned long long now = ptx::globaltimer_ns();
-              if (t0 == 0) t0 = now;
-              if (now - t0 > ptx::kWaitLimitNs) { *abort_flag = 1; break; }
-            }
-          }
-          if (v != 0u) b = (int)v - 1;
-        }
-      }
-      sh_flag[0] = b;
-    }
-    __syncthreads();
-    const int b = sh_flag[0];
-    if (b < 0) break;
-    const VerifySeq d = fused_seq(a, b);
-    fused_decide(a, b, d, sh64, sh_flag);
-  }
-  if (tid == 0 && sh_abort) {
-    // copies already asked for must land before the CTA's shared memory goes away (bounded)
-    const unsigned long long t0 = ptx::globaltimer_ns();
-    while (ptx::globaltimer_ns() - t0 < 20000ull) {}      // 20 us: far longer than a row's copy takes
-    if (a.status) atomicExch(a.status, 1);
+    const u64 s = warp_sum54(local);
+    if (lane == 0) sh_sum[group][k & 1][gwarp] = s;
+    last_stat = stat; last_m = m;
+    next_slot(others);
   }
 }
 
 // ------------------------------------------------------------------------------ one cluster per sequence
-// Algorithm 2's decision, or level 0's draw (no drafts: the rule's final draw from the one row), for few sequences: a
-// cluster of C CTAs takes a sequence's 2 t + 1 rows, each CTA the same V / C consecutive tokens of every row.  Bound by
-// latency, not by bytes (t = 3 rows of 32000 bf16 tokens are 0.4 MB): the rows are read once into shared memory, the row
+// Algorithm 2's decision on at most one draft, or level 0's draw (no drafts: the rule's final draw from the one row), for few
+// sequences: a cluster of C CTAs takes a sequence's 2 t + 1 rows, each CTA the same V / C consecutive tokens of every row.  Bound by
+// latency, not by bytes (three rows of 32000 bf16 tokens are 0.2 MB): the rows are read once into shared memory, the row
 // maxima and then the integer totals cross the cluster in one exchange each, every CTA takes the accept tests by itself,
 // and a rejection costs one more exchange for the residual's totals.  No scratch in global memory, nothing to clear.
 // A warp owns consecutive tokens; lane and unit index are interleaved (unit = 4 bytes: a bf16 pair or an fp32 value;
 // 2 bytes when rows of odd length leave bf16 pairs unaligned), so loads are whole lines whatever the row's alignment.
-constexpr int kClThreads = 512, kClWarps = kClThreads / 32, kClMaxRows = 63, kClMaxC = 8;
+constexpr int kClThreads = 512, kClWarps = kClThreads / 32, kClMaxRows = 3, kClMaxC = 8;
 
 template <typename T, int PER> struct ClUnit;              // PER tokens of one load
 template <> struct ClUnit<float, 1> {
   typedef float raw;
   __device__ static void get(float r, float *f) { f[0] = r; }
+  __device__ static raw none() { return -INFINITY; }
 };
 template <> struct ClUnit<__nv_bfloat16, 1> {
   typedef unsigned short raw;
   __device__ static void get(unsigned short r, float *f) { f[0] = __uint_as_float((u32)r << 16); }
+  __device__ static raw none() { return 0xFF80u; }
 };
 template <> struct ClUnit<__nv_bfloat16, 2> {
   typedef u32 raw;
   __device__ static void get(u32 r, float *f) { f[0] = __uint_as_float(r << 16); f[1] = __uint_as_float(r & 0xFFFF0000u); }
+  __device__ static raw none() { return 0xFF80FF80u; }
 };
 
 struct ClusterArgs {
   const void *p, *q;
   int32_t *tokens;
   int V, t_max, seg;             // seg: tokens per CTA, a multiple of 64
-  int staged;                    // rows kept in shared memory; 0: they do not fit and are read again where they are needed
   const VerifySeq *desc;         // verification: per sequence, or null (regular)
   const SampleRow *rows;         // draws: per row, or null (regular)
   int regular_t;                 // draws: rows per sequence
@@ -643,13 +441,56 @@ __device__ __forceinline__ u32 cl_map(const void *p, u32 rank) {
 }
 __device__ __forceinline__ void cl_store(u32 addr, u32 v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 __device__ __forceinline__ void cl_store(u32 addr, u64 v) { asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory"); }
-// fp32 (no NaN) -> signed integer in the same order, and back
-__device__ __forceinline__ int order_key(float f) { const int b = __float_as_int(f); return b ^ ((b >> 31) & 0x7FFFFFFF); }
-__device__ __forceinline__ float order_value(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7FFFFFFF)); }
-// Sum over a warp of values below 2^54.
-__device__ __forceinline__ u64 warp_sum54(u64 v) {
-  const u32 lo = __reduce_add_sync(0xFFFFFFFFu, (u32)v & 0x7FFFFFFu), hi = __reduce_add_sync(0xFFFFFFFFu, (u32)(v >> 27));
-  return ((u64)hi << 27) + lo;
+// Inverse CDF within a CTA whose weights pass the threshold: the warp, then the unit, then the token whose inclusive sum
+// does.  w: the thread's weights, sums: the warps' totals, before: the sum of the CTAs in front.
+template <int NT, int PER, class W, class Emit>
+__device__ __forceinline__ void cl_find_token(const W (&w)[NT], u64 tau, u64 before, const u64 *sums, int k_lane, Emit emit) {
+  constexpr int NU = NT / PER;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  u64 mine = lane < kClWarps ? sums[lane] : 0ull;                  // every warp finds the owning one for itself
+  u64 incl = mine;
+  for (int o = 1; o < 32; o <<= 1) {
+    const u64 v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  const int owner = __ffs(__ballot_sync(0xFFFFFFFFu, before + incl > tau)) - 1;
+  if (warp != owner) return;
+  u64 base = before + __shfl_sync(0xFFFFFFFFu, incl - mine, owner);
+  u64 tot[NU];
+#pragma unroll
+  for (int i = 0; i < NU; ++i) {
+    u64 s = 0;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) s += w[i * PER + e];
+    tot[i] = warp_sum54(s);
+  }
+  bool done = false;
+#pragma unroll
+  for (int i = 0; i < NU; ++i) {
+    if (!done && base + tot[i] > tau) {                            // uniform over the warp
+      done = true;
+      u64 s = 0;
+#pragma unroll
+      for (int e = 0; e < PER; ++e) s += w[i * PER + e];
+      u64 c = s;
+      for (int o = 1; o < 32; o <<= 1) {
+        const u64 v = __shfl_up_sync(0xFFFFFFFFu, c, o);
+        if (lane >= o) c += v;
+      }
+      const int l = __ffs(__ballot_sync(0xFFFFFFFFu, base + c > tau)) - 1;
+      if (lane == l) {
+        u64 run = base + c - s;
+        int k = k_lane + 32 * PER * i;
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+          run += w[i * PER + e];
+          if (run > tau) break;
+          ++k;
+        }
+        emit(k);
+      }
+    } else if (!done) base += tot[i];
+  }
 }
 
 // Shared memory (dynamic): raw units [rows][NU][threads] | wmax int [rows][warps] | wsum u64 [rows + 1][warps]
@@ -687,7 +528,7 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
   const int t = DRAW ? 0 : d.t, n_rows = 2 * t + 1;                           // rows 0..t: p; t + 1 + j: q_j
   raw_t *stage = reinterpret_cast<raw_t *>(cl_smem);
   const size_t max_rows = 2 * (size_t)a.t_max + 1;
-  u64 *wsum = reinterpret_cast<u64 *>(cl_smem + (a.staged ? max_rows * NU * kClThreads * sizeof(raw_t) : 0));   // [rows + 1][warps]
+  u64 *wsum = reinterpret_cast<u64 *>(cl_smem + max_rows * NU * kClThreads * sizeof(raw_t));   // [rows + 1][warps]
   int *wmax = reinterpret_cast<int *>(wsum + (max_rows + 1) * kClWarps);
   auto row_ptr = [&](int r) {
     return r <= t ? reinterpret_cast<const T *>(a.p) + (size_t)(d.p_row0 + r) * a.V
@@ -703,9 +544,7 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
     if (tok >= 0 && tok < a.V) { lp = to_f32(row_ptr(tid)[tok]); lq = to_f32(row_ptr(t + 1 + tid)[tok]); }
   }
   auto unit_of = [&](int r, int i) -> raw_t {                      // a unit of this thread, once more
-    if (a.staged) return stage[((size_t)r * NU + i) * kClThreads + tid];
-    const int k = k_lane + 32 * PER * i;
-    return k < tok_end ? __ldg(reinterpret_cast<const raw_t *>(row_ptr(r) + k)) : raw_t(0);
+    return stage[((size_t)r * NU + i) * kClThreads + tid];
   };
   // weights of a row's units against the row maximum, two tokens j, j + 1 at a time (0 past the CTA's tokens)
   auto weights_of = [&](const raw_t *v, float m, auto &&take) {
@@ -745,7 +584,7 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
 #pragma unroll
           for (int e = 0; e < PER; ++e) m = fmaxf(m, f[e]);
         }
-        if (a.staged) stage[((size_t)(r0 + rr) * NU + i) * kClThreads + tid] = v[rr][i];
+        stage[((size_t)(r0 + rr) * NU + i) * kClThreads + tid] = v[rr][i];
       }
       const int key = __reduce_max_sync(0xFFFFFFFFu, order_key(m));
       if (lane == 0) wmax[(r0 + rr) * kClWarps + warp] = key;
@@ -865,55 +704,13 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
       }
     }
   } else if (tau >= before && tau < before + csum[src][rank]) {
-    u64 mine = lane < kClWarps ? wsum[src * kClWarps + lane] : 0ull;   // every warp finds the owning one for itself
-    u64 incl = mine;
-    for (int o = 1; o < 32; o <<= 1) {
-      const u64 v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    const int owner = __ffs(__ballot_sync(0xFFFFFFFFu, before + incl > tau)) - 1;
-    if (warp == owner) {
-      u64 base = before + __shfl_sync(0xFFFFFFFFu, incl - mine, owner);
-      u64 tot[NU];
-#pragma unroll
-      for (int i = 0; i < NU; ++i) {
-        u64 s = 0;
-#pragma unroll
-        for (int e = 0; e < PER; ++e) s += w[i * PER + e];
-        tot[i] = warp_sum54(s);
+    cl_find_token<NT, PER>(w, tau, before, wsum + src * kClWarps, k_lane, [&](int k) {
+      if (DRAW) a.out_tokens[out_index] = k;
+      else {
+        if (a.write_in_place) a.tokens[d.tok_off + n] = k;
+        if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = k;
       }
-      bool done = false;
-#pragma unroll
-      for (int i = 0; i < NU; ++i) {
-        if (!done && base + tot[i] > tau) {                        // uniform over the warp
-          done = true;
-          u64 s = 0;
-#pragma unroll
-          for (int e = 0; e < PER; ++e) s += w[i * PER + e];
-          u64 c = s;
-          for (int o = 1; o < 32; o <<= 1) {
-            const u64 v = __shfl_up_sync(0xFFFFFFFFu, c, o);
-            if (lane >= o) c += v;
-          }
-          const int l = __ffs(__ballot_sync(0xFFFFFFFFu, base + c > tau)) - 1;
-          if (lane == l) {
-            u64 run = base + c - s;
-            int k = k_lane + 32 * PER * i;
-#pragma unroll
-            for (int e = 0; e < PER; ++e) {
-              run += w[i * PER + e];
-              if (run > tau) break;
-              ++k;
-            }
-            if (DRAW) a.out_tokens[out_index] = k;
-            else {
-              if (a.write_in_place) a.tokens[d.tok_off + n] = k;
-              if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = k;
-            }
-          }
-        } else if (!done) base += tot[i];
-      }
-    }
+    });
   }
   if (!DRAW && rank == 0) {
     if (tid == 0) a.out_n[b] = n;
@@ -921,13 +718,151 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
   }
 }
 
+// The decision of a sequence whose rows' statistics are there (row_stats_stream_kernel, which this kernel follows in a
+// chain): the accept tests by every CTA of the cluster for itself, the residual's weights of the CTA's tokens, one exchange
+// of their totals.  Bound by latency: two gathers, a row of each side and an exchange.  64 sequences of 32000 tokens, two
+// CTAs each: 6 us behind the statistics; a CTA of 1024 threads a sequence, 32 tokens each, took 9.
+template <typename T, int PER, int NT>
+__global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __grid_constant__ ClusterArgs a, const RowStat *stats) {
+  typedef typename ClUnit<T, PER>::raw raw_t;
+  constexpr int NU = NT / PER;
+  __shared__ u64 wsum[2][kClWarps], csum[2][kClMaxC];              // [residual, the verifier's row]
+  __shared__ int sh_n;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const u32 rank = cl_rank(), C = cl_size();
+  const int b = (int)cl_id();
+  cl_arrive();                                                     // (the wait is in front of the first store to a peer)
+  VerifySeq d;
+  if (a.desc) d = a.desc[b];
+  else {
+    d.t = a.regular_t; d.p_row0 = (long long)b * (a.regular_t + 1); d.q_row0 = (long long)b * a.regular_t;
+    d.tok_off = (long long)b * a.regular_t; d.serial = a.regular_serial; d.seq = b; d.level = a.regular_level;
+  }
+  const int t = d.t;
+  const T *p = reinterpret_cast<const T *>(a.p) + (size_t)d.p_row0 * a.V, *q = reinterpret_cast<const T *>(a.q) + (size_t)d.q_row0 * a.V;
+  const RowStat *sp = stats + (size_t)b * (2 * a.t_max + 1), *sq = sp + a.t_max + 1;
+  auto stat = [](const RowStat *s) {
+    const float4 v = __ldcg(reinterpret_cast<const float4 *>(s));
+    return *reinterpret_cast<const RowStat *>(&v);
+  };
+  if (tid == 0) sh_n = t;
+  // the call's inputs are complete when the statistics kernel begins: the drafted tokens' logits come ahead of its end
+  int tok = -1;
+  float lp = 0.f, lq = 0.f;
+  auto drafted = [&](int j) {
+    tok = a.tokens[d.tok_off + j];
+    if (tok >= 0 && tok < a.V) { lp = to_f32(p[(size_t)j * a.V + tok]); lq = to_f32(q[(size_t)j * a.V + tok]); }
+  };
+  if (tid < t) drafted(tid);
+  __syncthreads();
+  chain_wait();
+  chain_next();
+  for (int j = tid; j < t; j += kClThreads) {
+    if (j != tid) drafted(j);
+    const RowStat s = stat(sp + j), r = stat(sq + j);
+    const bool in = tok >= 0 && tok < a.V;
+    const u64 Pp = fixed_prob(in ? exp_weight(lp, s.m) : 0u, prob_scale(s.S)), Pq = fixed_prob(in ? exp_weight(lq, r.m) : 0u, prob_scale(r.S));
+    const u32 U = uniform24(a.seed, j, d.serial, d.level, PURPOSE_ACCEPT, d.seq);
+    bool ok = (((u64)U * Pq) >> 24) < Pp;                          // u < p(x) / q(x)
+    if (a.coin24 != kNoCoin) ok = U < a.coin24;                    // ablation: IID acceptance with a fixed probability
+    if (!ok) atomicMin(&sh_n, j);
+  }
+  __syncthreads();
+  const int n = sh_n, tok0 = (int)rank * a.seg, tok_end = min(a.V, tok0 + a.seg);
+  const int k_lane = tok0 + warp * (32 * NT) + lane * PER;         // first token of unit i: k_lane + 32 PER i
+  const RowStat spn = stat(sp + n);
+  raw_t vp[NU];
+  auto fetch = [&](const T *row, raw_t *v) {                       // -inf past the CTA's tokens: no weight
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      const int k = k_lane + 32 * PER * i;
+      v[i] = k < tok_end ? __ldg(reinterpret_cast<const raw_t *>(row + k)) : ClUnit<T, PER>::none();
+    }
+  };
+  fetch(p + (size_t)n * a.V, vp);
+  u64 w[NT], total = 0;
+  bool running = false;                                            // every CTA of the cluster has started
+  auto exchange = [&](int src, u64 local) {                        // the CTAs' totals -> csum[src], their sum -> total
+    const u64 s = warp_sum54(local);
+    if (lane == 0) wsum[src][warp] = s;
+    __syncthreads();
+    if (!running) cl_wait();
+    running = true;
+    if (warp == 0) {
+      u64 c = lane < kClWarps ? wsum[src][lane] : 0ull;
+      for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
+      if (lane < (int)C) cl_store(cl_map(&csum[src][rank], (u32)lane), c);
+    }
+    cl_sync();
+    total = 0;
+    for (u32 c = 0; c < C; ++c) total += csum[src][c];
+  };
+  int src = 0;
+  if (n < t) {
+    raw_t vq[NU];
+    fetch(q + (size_t)n * a.V, vq);
+    const RowStat sqn = stat(sq + n);
+    const ProbScale psp = prob_scale(spn.S), psq = prob_scale(sqn.S);
+    u64 local = 0;
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      float fp[PER], fq[PER];
+      ClUnit<T, PER>::get(vp[i], fp);
+      ClUnit<T, PER>::get(vq[i], fq);
+#pragma unroll
+      for (int e = 0; e < PER; ++e) {
+        u32 ep, eq;
+        exp_weight2m(fp[e], fq[e], spn.m, sqn.m, ep, eq);
+        const u64 Pp = fixed_prob(ep, psp), Pq = fixed_prob(eq, psq);
+        w[i * PER + e] = Pp > Pq ? Pp - Pq : 0ull;
+        local += w[i * PER + e];
+      }
+    }
+    exchange(0, local);
+  }
+  if (total == 0) {                                                // the bonus token, or an all-zero residual: the verifier's own row
+    src = 1;
+    u64 local = 0;
+    if (n < t) fetch(p + (size_t)n * a.V, vp);                     // (once more, so that the residual need not keep it)
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      float f[PER];
+      ClUnit<T, PER>::get(vp[i], f);
+#pragma unroll
+      for (int e = 0; e < PER; ++e) {
+        w[i * PER + e] = exp_weight(f[e], spn.m);
+        local += w[i * PER + e];
+      }
+    }
+    exchange(1, local);
+  }
+  const u32 U = uniform24(a.seed, 0, d.serial, d.level, PURPOSE_FINAL, d.seq);
+  const u64 tau = cdf_threshold(U, total);
+  u64 before = 0;
+  for (u32 c = 0; c < rank; ++c) before += csum[src][c];
+  auto emit = [&](int k) {
+    if (a.write_in_place) a.tokens[d.tok_off + n] = k;
+    if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = k;
+  };
+  if (total == 0) {                                                // non-finite logits: no token
+    if (rank == 0 && tid == 0) emit(-1);
+  } else if (tau >= before && tau < before + csum[src][rank]) {
+    cl_find_token<NT, PER>(w, tau, before, wsum[src], k_lane, emit);
+  }
+  if (rank == 0) {
+    if (tid == 0) a.out_n[b] = n;
+    if (a.out_tokens)
+      for (int j = tid; j <= a.t_max; j += kClThreads)
+        if (j != n) a.out_tokens[(size_t)b * (a.t_max + 1) + j] = j < n ? a.tokens[d.tok_off + j] : -1;
+  }
+}
+
 // Cluster size, tokens per thread and shared memory of a call with n sequences of at most `rows` rows; false if the rows
 // are too long or too many for this path.
-struct ClusterPlan { int C, NT, per, staged, seg; size_t smem; };
+struct ClusterPlan { int C, NT, per, seg; size_t smem; };
 constexpr size_t kClMaxSmem = 216 * 1024;
 constexpr int kClEights = 14;                     // clusters of eight that run at once (one CTA per SM)
 static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, int rows, bool draw, ClusterPlan *pl) {
-  if (rows > kClMaxRows) return false;
   pl->per = (dtype == HSD_BF16 && V % 2 == 0 && ((uintptr_t)p & 3) == 0 && ((uintptr_t)q & 3) == 0) ? 2 : 1;
   // as many CTAs as run at once (draws: two per SM), of at least 4096 tokens (eight a thread) each: clusters of eight do not fit all SMs
   // (16 of them took two rounds), clusters of four and two do
@@ -942,35 +877,19 @@ static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, 
   pl->NT = seg <= 8 * kClThreads ? 8 : seg <= 16 * kClThreads ? 16 : 32;
   const size_t extra = (size_t)(rows + 1) * kClWarps * 8 + (size_t)rows * kClWarps * 4;
   const size_t stage = (size_t)rows * pl->NT * kClThreads * (dtype == HSD_BF16 ? 2 : 4);
-  pl->staged = stage + extra <= kClMaxSmem;
-  pl->smem = extra + (pl->staged ? stage : 0);
+  pl->smem = extra + stage;
   return true;
 }
-// Where the cluster path is the faster one (us a call on an idle GPU, cluster / other path).  Its time grows with the
-// tokens a CTA goes through, rows x 512 NT, and with the rounds its clusters need; the other paths give every row a CTA
-// of its own.
-//   verification, rows the fused kernel takes: both times from their fits (within 10 % of 140 measured calls: V 64 to
-//     32000, 1 to 128 sequences, t 1 to 16), the cluster path where its own is the smaller by 15 %.  V = 32000
-//     bf16, t = 3: 1 to 8 sequences 12 / 25, 32: 17 / 30, 64: 38 / 35; t = 8: 8 sequences 19 / 26, 16: 36 / 30.  V = 2048,
-//     t = 16: 16 sequences 37 / 25, 64: 37 / 51; t = 8: 4 sequences 21 / 19, 32: 21 / 25.
-//   other rows: statistics and decision kernels, each row read twice by one CTA.  fp32, V = 32001: t = 3 14 / 58, t = 8
-//     30 / 58; V = 9001: t = 3 14 / 15, t = 8 29 / 15; V = 2048: t = 3 11 / 7.  bf16 of odd length, 49999: t = 3 21 / 50, t = 8 55 / 50;
-//     128 sequences at t = 1 (four rounds) 98 / 79, fp32 97 / 82; rows of more than 50000 tokens take the other path so much
-//     longer that rounds do not matter (65536, 128 sequences: 88 / 142).
-//   draws (two CTAs per SM, 16 tokens a thread at most): bf16 32000: 1 row 4.4 / 10.6, 64 rows 6.7 / 11.3 (one CTA per
+// Where the one-launch cluster path is the faster one (us a call in a captured sequence of calls, cluster / other path).
+//   verification: three rows of a long vocabulary a sequence, clusters of four or eight.  t = 1, bf16: V = 32000, 1 sequence 9.3 / 9.9,
+//     4: 10.5 / 10.9, 32 (clusters of four): 12.7 / 12.6, 64 (of two): 19.4 / 18.9; V = 8192, 1: 9.3 / 7.5; V = 49999, 1: 15.2 / 15.5; fp32:
+//     V = 32000, 1: 9.6 / 11.6, V = 8192, 1: 9.6 / 7.8.  More rows cost a CTA 0.9 us each, and the statistics kernel has an SM
+//     for each: t = 3, 1 sequence bf16 11.9 / 10.5, fp32 13.7 / 12.3; t = 8, 8 sequences bf16 19 / 10.6.
+//   draws (two CTAs per SM, 16 tokens a thread at most), other path a CTA a row: bf16 32000: 1 row 4.4 / 10.6, 64 rows 6.7 / 11.3 (one CTA per
 //     SM, 32 tokens a thread: 11.2), 100 rows would take a second round; fp32 32000: 1 row 5.7 / 28, 64 rows 8.6 / 28; 16001:
 //     5.2 / 10.8; 9001 (two CTAs a row): 6.9 / 6.2, 12289 (two) 10.4 / 9.5, (four) 6.3 / 9.5, 2048: 6.8 / 3.9; bf16 2048 (one CTA): 6.7 / 9.8.
-static bool cluster_pays_verify(const ClusterPlan &pl, int dtype, int V, int batch, int rows, bool fused) {
-  const long long work = (long long)pl.seg * rows;
-  if (fused) {
-    const double tokens = 512.0 * pl.NT * rows, rounds = ceil_div(pl.C * batch, kMeasuredSMs);
-    const double cluster_us = rounds * (7.5 + tokens * (pl.NT == 32 ? 2.7e-4 : 2.05e-4));
-    const double fused_us = 17.5 + V * 2.4e-4 + (double)batch * rows * (0.0155 + V * 4e-7);
-    return cluster_us * 1.15 < fused_us;
-  }
-  if (pl.C * batch > 2 * kMeasuredSMs && V <= 50000) return false;
-  if (dtype == HSD_BF16) return work * 5 <= 8ll * V;
-  return V > 20000 ? work <= 4ll * V : work * 5 <= 11ll * V;
+static bool cluster_pays_verify(const ClusterPlan &pl, int V, int batch) {
+  return V > 24000 && pl.NT <= 16 && pl.C >= 4 && pl.C * batch <= kMeasuredSMs;
 }
 static bool cluster_pays_draw(const ClusterPlan &pl, int dtype, int V, int n, bool chunked) {
   if (pl.seg > 4096 && pl.C * n > 2 * kMeasuredSMs) return false;
@@ -997,19 +916,18 @@ template <typename T, int PER, bool DRAW>
 static int launch_cluster_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
   if (pl.NT == 8) return launch_cluster_t<T, PER, 8, DRAW>(a, pl, n, s);
   if (pl.NT == 16) return launch_cluster_t<T, PER, 16, DRAW>(a, pl, n, s);
-  if constexpr (!DRAW) return launch_cluster_t<T, PER, 32, DRAW>(a, pl, n, s);
   return HSD_E_UNSUPPORTED;
 }
 template <bool DRAW>
 static int launch_cluster(ClusterArgs a, const ClusterPlan &pl, int dtype, int n, cudaStream_t s) {
   a.seg = pl.seg;
-  a.staged = pl.staged;
   if (dtype == HSD_F32) return launch_cluster_nt<float, 1, DRAW>(a, pl, n, s);
   return pl.per == 2 ? launch_cluster_nt<__nv_bfloat16, 2, DRAW>(a, pl, n, s) : launch_cluster_nt<__nv_bfloat16, 1, DRAW>(a, pl, n, s);
 }
 
 // ------------------------------------------------------------------------------ host launchers
-// Scratch of one verification call: [counter per sequence (fused kernel)] [RowStat per logits row].
+// Scratch of one verification call: [unused: counters of an earlier kernel, kept so that a workspace laid out for a call is what
+// it was] [RowStat per logits row].
 static size_t verify_counter_bytes(int batch) { return ((size_t)(2 * batch + 2) * 4 + 255) / 256 * 256; }
 size_t verify_scratch_bytes(int batch, int t_max) {
   return verify_counter_bytes(batch) + (size_t)batch * (2 * t_max + 1) * sizeof(RowStat);
@@ -1039,27 +957,7 @@ int launch_draft_sample(const void *logits, int dtype, int V, const SampleRow *d
              : launch_draft_sample_t<float>(logits, V, desc, n_rows, regular_rows, regular_serial, seed, out, s);
 }
 
-template <typename T>
-static int launch_verify_t(const void *p, const void *q, int32_t *tokens, int V, int batch, int t_max,
-                           const VerifySeq *desc, int regular_t, u32 regular_serial, u32 regular_level, RowStat *stats,
-                           u64 seed, int32_t *out_tokens, int32_t *out_n, int write_in_place, cudaStream_t s, u32 coin24) {
-  dim3 grid(2 * t_max + 1, batch);
-  constexpr int VN = StatVec<T>::N;
-  const bool vec_ok = V % VN == 0 && V / VN <= kStatVecPerThread * kStatThreads && ((uintptr_t)p & 15) == 0 &&
-                      (q == nullptr || ((uintptr_t)q & 15) == 0);
-  if (vec_ok)
-    row_stats_vec_kernel<T><<<grid, kStatThreads, 0, s>>>((const T *)p, (const T *)q, tokens, V, t_max, desc, regular_t, stats);
-  else
-    row_stats_kernel<T><<<grid, kStatThreads, 0, s>>>((const T *)p, (const T *)q, tokens, V, t_max, desc, regular_t, stats);
-  if (cudaGetLastError() != cudaSuccess) return HSD_E_CUDA;
-  decide_kernel<T><<<batch, kSampleThreads, 0, s>>>((const T *)p, (const T *)q, tokens, V, t_max, desc, regular_t,
-                                                   regular_serial, regular_level, stats, seed, out_tokens, out_n,
-                                                   write_in_place, coin24);
-  hsd_count_launches(2);
-  return hsd_launch_status();
-}
-
-static int fused_sm_count() {
+static int sm_count() {
   static int sms = 0;
   if (sms == 0) {
     int dev = 0, n = 0;
@@ -1069,50 +967,74 @@ static int fused_sm_count() {
   return sms;
 }
 
+template <typename T, int GROUPS, int WARPS, int CHUNK>
+static int launch_row_stats_t(const RowStatArgs &a, int grid, cudaStream_t s) {
+  constexpr int smem = (int)kRsBytes + 128;
+  static std::atomic<u64> limits{0};
+  const int limit = hsd_smem_limit((const void *)row_stats_kernel<T, GROUPS, WARPS, CHUNK>, smem, limits);
+  if (limit) return limit;
+  HSD_CUDA_OK(hsd_launch(row_stats_kernel<T, GROUPS, WARPS, CHUNK>, grid, 32 * (GROUPS * WARPS + 1), smem, s, 0, true, a));
+  hsd_count_launches(1);
+  return HSD_OK;
+}
+// us a call, GROUPS x WARPS = 1 x 16 / 2 x 8 / 3 x 8 (chunks of 32 KB; 2 x 12 on chunks of 24 KB lies behind 2 x 8):
+//   a row a CTA, 32000: bf16 5.6 / 5.9 / 6.2, fp32 6.9 / 7.4 / 7.7
+//   1088 rows of 32000: bf16 29.7 / 25.3 / 24.6, fp32 35.3 / 32.3 / 32.5; of 2048: bf16 9.6 / 7.0 / 6.9; of 50000, fp32: 57.4 / 57.7 / 58.2
+static int launch_row_stats(const RowStatArgs &a, int dtype, cudaStream_t s) {
+  const long long n_items = (long long)a.batch * (2 * a.t_max + 1);
+  const int grid = (int)std::min<long long>(sm_count(), n_items);
+  if (n_items <= grid)                                     // a row a CTA: all its warps on it
+    return dtype == HSD_F32 ? launch_row_stats_t<float, 1, 16, 32768>(a, grid, s) : launch_row_stats_t<__nv_bfloat16, 1, 16, 32768>(a, grid, s);
+  return dtype == HSD_F32 ? launch_row_stats_t<float, 3, 8, 32768>(a, grid, s) : launch_row_stats_t<__nv_bfloat16, 3, 8, 32768>(a, grid, s);
+}
+
+template <typename T, int PER>
+static int launch_decide_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, const RowStat *stats, cudaStream_t s) {
+  const int grid = n * pl.C;
+  if (pl.NT == 8) HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 8>, grid, kClThreads, 0, s, pl.C, true, a, stats));
+  else if (pl.NT == 16) HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 16>, grid, kClThreads, 0, s, pl.C, true, a, stats));
+  else HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 32>, grid, kClThreads, 0, s, pl.C, true, a, stats));
+  hsd_count_launches(1);
+  return hsd_launch_status();
+}
+
 int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int V, int batch, int t_max,
                   const VerifySeq *desc, int regular_t, u32 regular_serial, u32 regular_level, void *scratch,
                   u64 seed, int32_t *out_tokens, int32_t *out_n, int write_in_place, cudaStream_t s,
                   u32 coin24) {
   if (batch == 0) return HSD_OK;
-  unsigned *counters = (unsigned *)scratch;
   RowStat *stats = (RowStat *)((char *)scratch + verify_counter_bytes(batch));
-  // bf16 rows that a bulk copy can fetch (16-byte multiples) and 1024 threads can hold: one fused launch
-  const size_t slot = ((size_t)V * 2 + 127) / 128 * 128, smem = kFusedSlots * slot + 2 * kFusedSlots * 8 + 128;
-  const bool fused = dtype == HSD_BF16 && V % 8 == 0 && V <= kFusedMaxV && smem <= 220 * 1024 && ((uintptr_t)p & 15) == 0 &&
-                     (q == nullptr || ((uintptr_t)q & 15) == 0) && t_max < kFusedConsumers;
+  ClusterArgs a = {};
+  a.p = p; a.q = q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.desc = desc; a.regular_t = regular_t;
+  a.regular_serial = regular_serial; a.regular_level = regular_level; a.seed = seed; a.out_tokens = out_tokens; a.out_n = out_n;
+  a.write_in_place = write_in_place; a.coin24 = coin24;
   ClusterPlan pl;
-  if (cluster_plan(p, q, dtype, V, batch, 2 * t_max + 1, false, &pl) && cluster_pays_verify(pl, dtype, V, batch, 2 * t_max + 1, fused)) {
-    ClusterArgs a = {};
-    a.p = p; a.q = q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.desc = desc; a.regular_t = regular_t;
-    a.regular_serial = regular_serial; a.regular_level = regular_level; a.seed = seed; a.out_tokens = out_tokens; a.out_n = out_n;
-    a.write_in_place = write_in_place; a.coin24 = coin24;
+  if (2 * t_max + 1 <= kClMaxRows && cluster_plan(p, q, dtype, V, batch, 2 * t_max + 1, false, &pl) && cluster_pays_verify(pl, V, batch))
     return launch_cluster<false>(a, pl, dtype, batch, s);
+  RowStatArgs r = {};
+  r.p = p; r.q = q; r.V = V; r.t_max = t_max; r.batch = batch; r.regular_t = regular_t; r.desc = desc; r.stats = stats;
+  const int st = launch_row_stats(r, dtype, s);
+  if (st) return st;
+  if (cluster_plan(p, q, dtype, V, batch, 1, false, &pl)) {     // a decision reads one row of each side
+    a.seg = pl.seg;
+    if (dtype == HSD_F32) return launch_decide_nt<float, 1>(a, pl, batch, stats, s);
+    return pl.per == 2 ? launch_decide_nt<__nv_bfloat16, 2>(a, pl, batch, stats, s) : launch_decide_nt<__nv_bfloat16, 1>(a, pl, batch, stats, s);
   }
-  if (fused) {
-    static std::atomic<u64> limits{0};
-    const int limit = hsd_smem_limit((const void *)verify_fused_kernel, 220 * 1024, limits);
-    if (limit) return limit;
-    HSD_CUDA_OK(cudaMemsetAsync(counters, 0, verify_counter_bytes(batch), s));
-    FusedArgs a;
-    a.p = (const __nv_bfloat16 *)p; a.q = (const __nv_bfloat16 *)q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.batch = batch;
-    a.desc = desc; a.regular_t = regular_t; a.regular_serial = regular_serial; a.regular_level = regular_level;
-    a.stats = stats; a.counters = counters; a.seed = seed; a.out_tokens = out_tokens; a.out_n = out_n;
-    a.write_in_place = write_in_place; a.coin24 = coin24; a.status = nullptr;
-    const int n_items = batch * (2 * t_max + 1);
-    verify_fused_kernel<<<std::min(fused_sm_count(), n_items), kFusedThreads, smem, s>>>(a);
-    hsd_count_launches(1);
-    return hsd_launch_status();
-  }
-  return dtype == HSD_BF16 ? launch_verify_t<__nv_bfloat16>(p, q, tokens, V, batch, t_max, desc, regular_t, regular_serial,
-                                                            regular_level, stats, seed, out_tokens, out_n, write_in_place, s, coin24)
-                           : launch_verify_t<float>(p, q, tokens, V, batch, t_max, desc, regular_t, regular_serial,
-                                                    regular_level, stats, seed, out_tokens, out_n, write_in_place, s, coin24);
+  // rows of more than 131072 tokens
+  if (dtype == HSD_BF16)
+    decide_kernel<__nv_bfloat16><<<batch, kSampleThreads, 0, s>>>((const __nv_bfloat16 *)p, (const __nv_bfloat16 *)q, tokens, V, t_max, desc, regular_t,
+                                                                  regular_serial, regular_level, stats, seed, out_tokens, out_n, write_in_place, coin24);
+  else
+    decide_kernel<float><<<batch, kSampleThreads, 0, s>>>((const float *)p, (const float *)q, tokens, V, t_max, desc, regular_t,
+                                                          regular_serial, regular_level, stats, seed, out_tokens, out_n, write_in_place, coin24);
+  hsd_count_launches(1);
+  return hsd_launch_status();
 }
 
 // ------------------------------------------------------------------------------ static scratch
 // Scratch for hsd_verify_level_static: lives in the library image, so every GPU that loads the
 // library holds these bytes until the process exits.  One RowStat per logits row of a call.
-constexpr int kStaticStatRows = 4096;                       // 64 KiB of row statistics + 32.25 KiB of counters and queue
+constexpr int kStaticStatRows = 4096;                       // 64 KiB of row statistics behind verify_counter_bytes()
 constexpr size_t kStaticScratchBytes = kStaticStatRows * sizeof(RowStat) + ((2 * kStaticStatRows + 2) * 4 + 255) / 256 * 256;
 static __device__ __align__(256) unsigned char g_static_verify_scratch[kStaticScratchBytes];
 
@@ -1199,8 +1121,7 @@ int hsd_verify_level_static(int level, const void *target_logits, const void *dr
   void *scratch = nullptr;
   int st = hsd::static_scratch_address(&scratch);          // first call on this device looks the symbol up
   if (st) return st;
-  // every RowStat the decision reads is written by the same call first; the per-sequence counters have to start
-  // at zero and are cleared on the stream inside launch_verify (a memset node, no allocation)
+  // every RowStat the decision reads is written by the same call first
   return hsd::launch_verify(target_logits, draft_logits, const_cast<int32_t *>(draft_tokens), dtype, vocab, batch, t,
                             nullptr, t, (u32)call_serial, (u32)level, scratch, seed, out_tokens, out_n_accepted, 0,
                             (cudaStream_t)stream);

@@ -64,10 +64,12 @@ __device__ __forceinline__ void exp_weight2m(float l0, float l1, float m0, float
   x.y = fmaxf(x.y, -32.0f);
   const float log2e = __uint_as_float(0x3FB8AA3Bu);
   const float2 t = __fmul2_rn(x, make_float2(log2e, log2e));
-  const float magic = __uint_as_float(0x4B400000u);        // see exp_weight
+  // see exp_weight; 32 more, an even number, leaves the rounding as it is and j + 32 in the low bits, which a shift puts on
+  // the exponent field: p is in [0.7, 1.5) and the result normal, so adding there is the exact multiplication
+  const float magic = __uint_as_float(0x4B400020u);
   const float2 tm = __fadd2_rn(t, make_float2(magic, magic));
-  const float2 jj = __fadd2_rn(tm, make_float2(-magic, -magic));
-  const float2 f = __fadd2_rn(t, make_float2(-jj.x, -jj.y));
+  const float2 nj = __ffma2_rn(tm, make_float2(-1.0f, -1.0f), make_float2(magic, magic));   // -j, exact
+  const float2 f = __fadd2_rn(t, nj);
   float c = __uint_as_float(0x3AADDD0Au);
   float2 p = make_float2(c, c);
   c = __uint_as_float(0x3C1E7544u); p = __fadd2_rn(__fmul2_rn(p, f), make_float2(c, c));
@@ -75,11 +77,8 @@ __device__ __forceinline__ void exp_weight2m(float l0, float l1, float m0, float
   c = __uint_as_float(0x3E75FCDEu); p = __fadd2_rn(__fmul2_rn(p, f), make_float2(c, c));
   c = __uint_as_float(0x3F317215u); p = __fadd2_rn(__fmul2_rn(p, f), make_float2(c, c));
   p = __fadd2_rn(__fmul2_rn(p, f), make_float2(1.0f, 1.0f));
-  const float2 sc = make_float2(__int_as_float((__float_as_int(tm.x) - 0x4B400000 + 32 + 127) << 23),
-                                __int_as_float((__float_as_int(tm.y) - 0x4B400000 + 32 + 127) << 23));
-  const float2 w = __fmul2_rn(p, sc);
-  e0 = __float2uint_rz(w.x);
-  e1 = __float2uint_rz(w.y);
+  e0 = __float2uint_rz(__uint_as_float(__float_as_uint(p.x) + (__float_as_uint(tm.x) << 23)));
+  e1 = __float2uint_rz(__uint_as_float(__float_as_uint(p.y) + (__float_as_uint(tm.y) << 23)));
 }
 
 // Fixed-point probabilities in units of 2^-40: P = (E * rinv) >> shift.
@@ -97,6 +96,15 @@ __device__ __forceinline__ u64 fixed_prob(u32 E, ProbScale ps) { return ((u64)E 
 // (U * total) >> 24 without overflow (U < 2^24, total < 2^64).
 __device__ __forceinline__ u64 cdf_threshold(u32 U, u64 total) {
   return (u64)U * (total >> 24) + (((u64)U * (total & 0xFFFFFFull)) >> 24);
+}
+
+// fp32 (no NaN) -> signed integer in the same order, and back
+__device__ __forceinline__ int order_key(float f) { const int b = __float_as_int(f); return b ^ ((b >> 31) & 0x7FFFFFFF); }
+__device__ __forceinline__ float order_value(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7FFFFFFF)); }
+// Sum over a warp of values below 2^54.
+__device__ __forceinline__ u64 warp_sum54(u64 v) {
+  const u32 lo = __reduce_add_sync(0xFFFFFFFFu, (u32)v & 0x7FFFFFFu), hi = __reduce_add_sync(0xFFFFFFFFu, (u32)(v >> 27));
+  return ((u64)hi << 27) + lo;
 }
 
 // ---- block-wide reductions over a group of threads: the whole block (blockDim.x a multiple of 32, at most

@@ -155,3 +155,57 @@ def test_cluster_draws_on_a_busy_gpu(lib, dtype, V, B):
     torch.cuda.synchronize()
     for i, x in enumerate(got):
         assert np.array_equal(x.cpu().numpy(), want[i % 4]), i
+
+
+@pytest.mark.parametrize("dtype,V,B,t,shift", [("bf16", 32000, 19, 4, 0), ("fp32", 32001, 14, 6, 0),  # more rows than SMs: two and three groups of warps
+                                               ("bf16", 50000, 16, 5, 0),      # rows of four chunks, CTAs whose third group has no row
+                                               ("bf16", 16385, 9, 8, 3),       # a second chunk of a few elements, rows that begin anywhere
+                                               ("fp32", 57347, 1, 2, 0), ("fp32", 57341, 30, 2, 1),    # one element past the ring, the longest rows in it
+                                               ("bf16", 131080, 2, 1, 0),      # longer than the clusters of the decision take
+                                               ("bf16", 5, 40, 2, 1), ("fp32", 3, 64, 2, 0),   # rows without a whole vector
+                                               ("bf16", 64, 2, 40, 0), ("fp32", 40, 1, 600, 2)])       # more drafts than lanes, than threads
+def test_row_statistics_and_decisions_match_oracle(lib, dtype, V, B, t, shift):
+    def moved(x):                                                      # the same values from element `shift` of a buffer on
+        buf = torch.empty(x.numel() + shift, dtype=x.dtype, device="cuda")
+        buf[shift:] = x.reshape(-1)
+        return buf[shift:].view(x.shape)
+    p, q = inputs.make_accept_logits(B, t, V, seed=V + t, device="cuda", dtype=dtype)
+    p[0, :, V // 2:] = -float("inf")
+    p, q = moved(p), moved(q)
+    x = lib.hsd_draft_sample(q, 5, 0)
+    p_np, q_np, x_np = inputs.logits_to_numpy(p), inputs.logits_to_numpy(q), x.cpu().numpy()
+    for serial in range(2):
+        out, n = lib.hsd_verify_level(1, p, q, x, 23, serial)
+        want_out, want_n = _oracle_verify(1, p_np, q_np, x_np, 23, serial)
+        assert np.array_equal(n.cpu().numpy(), want_n) and np.array_equal(out.cpu().numpy(), want_out)
+
+
+def test_verifications_in_a_captured_graph_and_back_to_back(lib):
+    # each call's kernels start under the end of the one before it; all share one workspace, and a call drafts from the rows
+    # that a kernel of the same stream has just written
+    B, t, V = 24, 3, 32000
+    sets = [inputs.make_accept_logits(B, t, V, seed=s, device="cuda", dtype="bf16") for s in range(3)]
+    p, q = torch.empty_like(sets[0][0]), torch.empty_like(sets[0][1])
+    ws = torch.empty(lib.hsd_verify_workspace_bytes(B, t), dtype=torch.uint8, device="cuda")
+    want = []
+    for i, (pi, qi) in enumerate(sets):
+        x = lib.hsd_draft_sample(qi, 3, i)
+        want.append([v.cpu() for v in lib.hsd_verify_level(1, pi, qi, x, 9, i)])
+
+    def chain():
+        got = []
+        for i in range(12):
+            p.copy_(sets[i % 3][0])
+            q.copy_(sets[i % 3][1])
+            got.append(lib.hsd_verify_level(1, p, q, lib.hsd_draft_sample(q, 3, i % 3), 9, i % 3, workspace=ws))
+        return got
+    runs = [chain()]
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        captured = chain()
+    graph.replay()
+    torch.cuda.synchronize()
+    for got in runs + [captured]:
+        for i, (out, n) in enumerate(got):
+            assert torch.equal(out.cpu(), want[i % 3][0]) and torch.equal(n.cpu(), want[i % 3][1]), i
