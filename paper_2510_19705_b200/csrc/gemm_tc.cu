@@ -177,8 +177,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), 4); }
     *abort_flag = 0;
-    // a wait gives up after two seconds, long after every CTA (one per SM) has started
-    if (args.reset_status && blockIdx.x == 0) *args.status = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), Cfg::kTmemCols);
@@ -220,13 +218,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       };
       int kb = kb0;
       if (tile == tile0) {
+        if (!args.early_weights) chain_wait();
+        // a wait gives up after two seconds, long after every CTA (one per SM) has started
+        if (args.reset_status && blockIdx.x == 0 && issuer) *args.status = 0;
         if (issuer)
           for (int i = 0; i < ahead; ++i) {
             load_w(kb0 + i, i);
-            if (!args.chained) load_a(kb0 + i, i);
+            if (!args.early_weights) load_a(kb0 + i, i);
           }
-        chain_wait();
-        if (issuer && args.chained)
+        if (args.early_weights) chain_wait();
+        if (issuer && args.early_weights)
           for (int i = 0; i < ahead; ++i) load_a(kb0 + i, i);
         kb += ahead; s = ahead;
         if (s == STAGES) { s = 0; ph ^= 1u; }

@@ -32,7 +32,8 @@ struct TcGemmArgs {
   CUtensorMap a;                   // activation map, covers the whole buffer
   int tile_rows = kTcBlockM, w_box_rows = kTcBoxRows;   // weight rows of a tile (<= 128; SWIGLU: 64 gate + 64 up) and of one box of their maps
   int a_box_rows;                  // rows of one box of the activation map (R .. row padding)
-  bool chained = false;            // part of a chain of kernels (common.cuh): the first weights are asked for before the kernel before it is over
+  bool chained = false;            // part of a chain of kernels (common.cuh)
+  bool early_weights = false;      // in a chain: the first weights are asked for before the kernel before is over (which must not write them)
   int stream_weights = 0;          // 1: the weights will not be read again soon (evict-first in L2)
   int reset_status = 0;            // 1: the kernel clears the status word first
   TcQkv qkv;

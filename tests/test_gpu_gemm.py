@@ -59,3 +59,30 @@ def test_gemm_tile_and_cluster_edges(lib, R, N, K):
     # fp32 accumulation: 2^-23 per addition of a chain of K / 32 partial sums of this size, at most
     bound = 2.0 ** -23 * (K / 32) * (A.double().abs() @ W.double().abs().T) + 1e-7
     assert bool(((out - ref).abs() < bound).all())
+
+
+@pytest.mark.parametrize("R,N,K", [(5, 1024, 4096), (24, 14336, 512), (200, 2000, 1024)])
+def test_gemm_calls_back_to_back_see_what_the_stream_wrote_before(lib, R, N, K):
+    # a call starts under the end of the one before it: operands rewritten between calls, a result that is the next operand,
+    # one workspace and one result buffer for all
+    g = torch.Generator(device="cuda").manual_seed(R)
+    A = [torch.randn(R, K, generator=g, device="cuda").to(torch.bfloat16) for _ in range(3)]
+    W = [(torch.randn(N, K, generator=g, device="cuda") * 0.05).to(torch.bfloat16) for _ in range(3)]
+    want = [lib.hsd_gemm_bf16(a, w) for a, w in zip(A, W)]
+    a, w = torch.empty_like(A[0]), torch.empty_like(W[0])
+    out = torch.empty(R, N, device="cuda")
+    ws = torch.empty(lib.hsd_gemm_workspace_bytes(R, N, K) + 256, dtype=torch.uint8, device="cuda")
+    got = []
+    for i in range(24):
+        a.copy_(A[i % 3])
+        w.copy_(W[i % 3])
+        lib.hsd_gemm_bf16(a, w, out=out, workspace=ws, check=False)
+        lib.hsd_gemm_bf16(A[0], W[0], workspace=ws, check=False)
+        got.append(out.clone())
+    assert all(torch.equal(o, want[i % 3]) for i, o in enumerate(got))
+    square = (torch.randn(K, K, generator=g, device="cuda") * 0.02).to(torch.bfloat16)
+    x, y = A[0], A[0]
+    for _ in range(6):
+        x = lib.hsd_gemm_bf16(x, square, check=False).to(torch.bfloat16)
+        y = lib.hsd_gemm_bf16(y, square).to(torch.bfloat16)
+    assert torch.equal(x, y)
