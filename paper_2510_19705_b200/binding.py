@@ -1,18 +1,22 @@
-"""Thin ctypes binding over the C-ABI library (include/hsd.h).
+"""Thin binding over the C-ABI library (include/hsd.h): ctypes, and native functions (native/host_calls.cpp) for the
+calls that take microseconds.
 
 Argument marshalling only: torch supplies device memory and streams, every step of the path runs
 in the library's own CUDA kernels.  There is no CPU fallback: if the shared library has not been
 built, or a call returns an error status, this module raises.
 """
 import ctypes
+import importlib.util
 import os
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libhsd.so")
+HOST_PATH = os.path.join(_HERE, "_host_calls.so")
 HSD_F32, HSD_BF16 = 0, 1
 _lib = None
+_host = None
 
 
 class HsdError(RuntimeError):
@@ -31,6 +35,23 @@ def library():
         _declare_engine(lib)
         _lib = lib
     return _lib
+
+
+def _host_calls():
+    """The native functions (loaded once), bound to the library's entry points."""
+    global _host
+    if _host is None:
+        if not os.path.exists(HOST_PATH):
+            raise HsdError("_host_calls.so is missing: run `python -m paper_2510_19705_b200.build`")
+        lib = library()
+        spec = importlib.util.spec_from_file_location("_host_calls", HOST_PATH)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        mod.init(*(ctypes.cast(f, ctypes.c_void_p).value for f in
+                   (lib.hsd_draft_sample, lib.hsd_verify_workspace_bytes, lib.hsd_verify_level, lib.hsd_gemm_workspace_bytes,
+                    lib.hsd_gemm_bf16, lib.hsd_gemm_status, lib.hsd_strerror)), HsdError)
+        _host = mod
+    return _host
 
 
 def _declare(lib):
@@ -78,12 +99,7 @@ def _stream():
 
 def hsd_draft_sample(logits, seed, call_serial, out_tokens=None):
     """logits [batch, rows, vocab] (CUDA, fp32/bf16) -> int32 tokens [batch, rows]."""
-    batch, rows, vocab = logits.shape
-    if out_tokens is None:
-        out_tokens = torch.empty(batch, rows, dtype=torch.int32, device=logits.device)
-    _check(library().hsd_draft_sample(_dev(logits), batch, rows, vocab, _dtype_code(logits), seed, call_serial,
-                                      _stream(), _dev(out_tokens)))
-    return out_tokens
+    return (_host or _host_calls()).draft_sample(logits, seed, call_serial, out_tokens)
 
 
 def hsd_verify_workspace_bytes(batch, t):
@@ -94,20 +110,8 @@ def hsd_verify_level(level, target_logits, draft_logits, draft_tokens, seed, cal
                      out_tokens=None, out_n_accepted=None):
     """target_logits [batch, t+1, vocab], draft_logits [batch, t, vocab], draft_tokens int32 [batch, t]
     -> (out_tokens int32 [batch, t+1] padded with -1, n_accepted int32 [batch])."""
-    batch, tp1, vocab = target_logits.shape
-    t = tp1 - 1
-    dev = target_logits.device
-    if workspace is None:
-        workspace = torch.empty(max(16, hsd_verify_workspace_bytes(batch, t)), dtype=torch.uint8, device=dev)
-    if out_tokens is None:
-        out_tokens = torch.empty(batch, t + 1, dtype=torch.int32, device=dev)
-    if out_n_accepted is None:
-        out_n_accepted = torch.empty(batch, dtype=torch.int32, device=dev)
-    _check(library().hsd_verify_level(level, _dev(target_logits), _dev(draft_logits) if t > 0 else None,
-                                      _dev(draft_tokens) if t > 0 else None, batch, t, vocab,
-                                      _dtype_code(target_logits), seed, call_serial, _dev(workspace),
-                                      workspace.numel(), _stream(), _dev(out_tokens), _dev(out_n_accepted)))
-    return out_tokens, out_n_accepted
+    return (_host or _host_calls()).verify_level(level, target_logits, draft_logits, draft_tokens, seed, call_serial, workspace,
+                                                 out_tokens, out_n_accepted)
 
 
 def hsd_verify_level_static(level, target_logits, draft_logits, draft_tokens, seed, call_serial, out_tokens,
@@ -461,19 +465,4 @@ def hsd_gemm_workspace_bytes(R, N, K):
 
 def hsd_gemm_bf16(A, W, out=None, workspace=None, check=True):
     """A bf16 [R, K], W bf16 [N, K] (CUDA) -> fp32 [R, N] = A @ W^T on the tensor cores."""
-    lib = library()
-    R, K = A.shape
-    N = W.shape[0]
-    need = hsd_gemm_workspace_bytes(R, N, K)
-    if need == 0:
-        raise HsdError("hsd_gemm_bf16: unsupported shape R=%d N=%d K=%d" % (R, N, K))
-    if workspace is None:
-        workspace = torch.empty(need + 256, dtype=torch.uint8, device=A.device)
-    base = (workspace.data_ptr() + 255) // 256 * 256
-    if out is None:
-        out = torch.empty(R, N, dtype=torch.float32, device=A.device)
-    _check(lib.hsd_gemm_bf16(_dev(A), R, K, _dev(W), N, _dev(out), ctypes.c_void_p(base),
-                             workspace.numel() - (base - workspace.data_ptr()), _stream()))
-    if check:
-        _check(lib.hsd_gemm_status(ctypes.c_void_p(base), _stream()))
-    return out
+    return (_host or _host_calls()).gemm_bf16(A, W, out, workspace, check)

@@ -1,11 +1,14 @@
-"""In-tree build of the C-ABI library (libhsd.so) for sm_100a with nvcc."""
+"""In-tree build of the C-ABI library (libhsd.so) for sm_100a with nvcc, and of the binding's native calls (_host_calls.so)."""
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhsd.so")
+HOST_SRC = os.path.join(HERE, "native", "host_calls.cpp")
+HOST = os.path.join(HERE, "_host_calls.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a", "-Xcompiler", "-fPIC",
          "--cudart", "static", "--expt-extended-lambda", "--expt-relaxed-constexpr"]
@@ -16,11 +19,24 @@ def sources():
 
 
 def needs_build():
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(HOST):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "hsd.h")]
-    return any(os.path.getmtime(d) > t for d in deps)
+    header = os.path.join(HERE, "..", "include", "hsd.h")
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [header]
+    return any(os.path.getmtime(d) > os.path.getmtime(LIB) for d in deps) or \
+        any(os.path.getmtime(d) > os.path.getmtime(HOST) for d in (HOST_SRC, header))
+
+
+def host_command():
+    """g++ command of the binding's native calls: torch's headers and libraries, no device code."""
+    import torch
+    root = os.path.dirname(torch.__file__)
+    lib = os.path.join(root, "lib")
+    cuda = os.path.dirname(os.path.dirname(NVCC))
+    inc = [sysconfig.get_paths()["include"], os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include")]
+    return [os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)] + \
+        ["-isystem" + d for d in inc] + [HOST_SRC, "-o", HOST, "-L" + lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
 
 
 def build(force=False, verbose=False):
@@ -36,12 +52,13 @@ def build(force=False, verbose=False):
         cmd = [NVCC] + FLAGS + extra + (["-Xptxas", "-v"] if verbose else []) + ["-c", src, "-o", obj]
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
         objs.append(obj)
+    procs.append((HOST_SRC, subprocess.Popen(host_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     for src, p in procs:
         out, _ = p.communicate()
         if verbose or p.returncode != 0:
             sys.stderr.write(out)
         if p.returncode != 0:
-            raise RuntimeError("nvcc failed on " + src)
+            raise RuntimeError("the compiler failed on " + src)
     cmd = [NVCC, "-shared", "--cudart", "static", "-gencode", "arch=compute_100a,code=sm_100a", "-o", LIB] + objs
     subprocess.run(cmd, check=True)
     return LIB
