@@ -16,6 +16,8 @@ draft_sample_kernel(const T *__restrict__ logits, int V, const SampleRow *__rest
                     int regular_rows, u32 regular_serial, u64 seed, int32_t *__restrict__ out) {
   __shared__ float shf[32];
   __shared__ u64 sh64[34];
+  chain_wait();
+  chain_next();
   SampleRow d;
   if (desc) {
     d = desc[blockIdx.x];
@@ -511,6 +513,8 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
   const u32 rank = cl_rank(), C = cl_size();
   const int b = (int)cl_id();
   cl_arrive();                                                     // (the wait is in front of the first store to a peer)
+  chain_wait();
+  chain_next();
   VerifySeq d;
   long long out_index = 0;
   u32 uj = 0;
@@ -885,16 +889,18 @@ static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, 
 //     4: 10.5 / 10.9, 32 (clusters of four): 12.7 / 12.6, 64 (of two): 19.4 / 18.9; V = 8192, 1: 9.3 / 7.5; V = 49999, 1: 15.2 / 15.5; fp32:
 //     V = 32000, 1: 9.6 / 11.6, V = 8192, 1: 9.6 / 7.8.  More rows cost a CTA 0.9 us each, and the statistics kernel has an SM
 //     for each: t = 3, 1 sequence bf16 11.9 / 10.5, fp32 13.7 / 12.3; t = 8, 8 sequences bf16 19 / 10.6.
-//   draws (two CTAs per SM, 16 tokens a thread at most), other path a CTA a row: bf16 32000: 1 row 4.4 / 10.6, 64 rows 6.7 / 11.3 (one CTA per
-//     SM, 32 tokens a thread: 11.2), 100 rows would take a second round; fp32 32000: 1 row 5.7 / 28, 64 rows 8.6 / 28; 16001:
-//     5.2 / 10.8; 9001 (two CTAs a row): 6.9 / 6.2, 12289 (two) 10.4 / 9.5, (four) 6.3 / 9.5, 2048: 6.8 / 3.9; bf16 2048 (one CTA): 6.7 / 9.8.
+//   draws (two CTAs per SM, 16 tokens a thread at most), other path a CTA of 1024 threads a row, which has 32 tokens a thread where bf16 rows
+//     allow (`chunked`): while the clusters run in one round, bf16 32000: 1 row 4.0 / 10.2, 64 rows 6.4 / 11.0; 2048: 4.0 / 8.5 to 9.4;
+//     fp32 32000: 4.5 / 26, 64 rows 7.9 / 28; 8000: 4.4 / 6.1; 2048: 4.0 / 3.9.  In more rounds, chunked: 32000, 100 rows 10.5 / 11.1, 148: 13.8 / 11.1
+//     (a row a CTA then), 200: 16.3 / 20.5, 512: 40 / 40, 16000, 512: 20 / 35; others: fp32 11000, 256: 13.8 / 9.9, 24001, 148: 16.7 / 12.9,
+//     32000, 100: 12.5 / 28, 512: 50 / 105; 8000, 512: 13.1 / 15.9; bf16 9001, 256: 14.0 / 12.2, 32001: 26 / 38.
 static bool cluster_pays_verify(const ClusterPlan &pl, int V, int batch) {
   return V > 24000 && pl.NT <= 16 && pl.C >= 4 && pl.C * batch <= kMeasuredSMs;
 }
-static bool cluster_pays_draw(const ClusterPlan &pl, int dtype, int V, int n, bool chunked) {
-  if (pl.seg > 4096 && pl.C * n > 2 * kMeasuredSMs) return false;
-  if (dtype == HSD_BF16 && chunked) return pl.seg <= 4096 || pl.C > 1;
-  return V > (pl.C > 2 ? 12000 : 13000) && pl.C > 1;
+static bool cluster_pays_draw(const ClusterPlan &pl, int V, int n, bool chunked) {
+  if (pl.C * n <= 2 * kMeasuredSMs) return true;
+  if (chunked) return n > kMeasuredSMs || pl.C * n <= 3 * kMeasuredSMs;
+  return V > 26000 || V <= 8192;
 }
 
 template <typename T, int PER, int NT, bool DRAW>
@@ -902,13 +908,7 @@ static int launch_cluster_t(const ClusterArgs &a, const ClusterPlan &pl, int n, 
   static std::atomic<u64> limits{0};
   const int limit = hsd_smem_limit((const void *)cluster_sample_kernel<T, PER, NT, DRAW>, (int)(DRAW ? kClMaxSmem / 2 : kClMaxSmem), limits);
   if (limit) return limit;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n * pl.C); cfg.blockDim = dim3(kClThreads); cfg.dynamicSmemBytes = pl.smem; cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = pl.C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
-  HSD_CUDA_OK(cudaLaunchKernelEx(&cfg, cluster_sample_kernel<T, PER, NT, DRAW>, a));
+  HSD_CUDA_OK(hsd_launch(cluster_sample_kernel<T, PER, NT, DRAW>, n * pl.C, kClThreads, pl.smem, s, pl.C, true, a));
   hsd_count_launches(1);
   return hsd_launch_status();
 }
@@ -936,7 +936,7 @@ size_t verify_scratch_bytes(int batch, int t_max) {
 template <typename T>
 static int launch_draft_sample_t(const void *logits, int V, const SampleRow *desc, int n_rows, int regular_rows,
                                  u32 regular_serial, u64 seed, int32_t *out, cudaStream_t s) {
-  draft_sample_kernel<T><<<n_rows, kSampleThreads, 0, s>>>((const T *)logits, V, desc, regular_rows, regular_serial, seed, out);
+  HSD_CUDA_OK(hsd_launch(draft_sample_kernel<T>, n_rows, kSampleThreads, 0, s, 0, true, (const T *)logits, V, desc, regular_rows, regular_serial, seed, out));
   hsd_count_launches(1);
   return hsd_launch_status();
 }
@@ -946,7 +946,7 @@ int launch_draft_sample(const void *logits, int dtype, int V, const SampleRow *d
   if (n_rows == 0) return HSD_OK;
   ClusterPlan pl;
   if (cluster_plan(logits, nullptr, dtype, V, n_rows, 1, true, &pl) &&
-      cluster_pays_draw(pl, dtype, V, n_rows, V % 8 == 0 && V <= kSampleThreads * kChunkTokens && ((uintptr_t)logits & 15) == 0)) {
+      cluster_pays_draw(pl, V, n_rows, dtype == HSD_BF16 && V % 8 == 0 && V <= kSampleThreads * kChunkTokens && ((uintptr_t)logits & 15) == 0)) {
     ClusterArgs a = {};
     a.p = logits; a.V = V; a.t_max = 0; a.rows = desc; a.regular_t = regular_rows;
     a.regular_serial = regular_serial; a.seed = seed; a.out_tokens = out; a.coin24 = kNoCoin;

@@ -209,3 +209,13 @@ def test_verifications_in_a_captured_graph_and_back_to_back(lib):
     for got in runs + [captured]:
         for i, (out, n) in enumerate(got):
             assert torch.equal(out.cpu(), want[i % 3][0]) and torch.equal(n.cpu(), want[i % 3][1]), i
+
+
+@pytest.mark.parametrize("dtype,V,B", [("bf16", 2048, 3), ("fp32", 513, 300),      # one CTA a row; more rows than run at once
+                                       ("bf16", 32000, 112), ("bf16", 32000, 148), ("fp32", 32001, 75),   # several rounds of clusters, a row a CTA
+                                       ("fp32", 9001, 149), ("bf16", 8190, 297)])
+def test_draws_of_many_rows_match_oracle(lib, dtype, V, B):
+    _, q = inputs.make_accept_logits(B, 1, V, seed=V + B, device="cuda", dtype=dtype)
+    want = _oracle_draft(inputs.logits_to_numpy(q), 41, 2)
+    got = [lib.hsd_draft_sample(q, 41, 2) for _ in range(3)]
+    assert all(np.array_equal(x.cpu().numpy(), want) for x in got)
