@@ -70,3 +70,19 @@ __host__ __device__ static inline int ceil_div(int a, int b) { return (a + b - 1
 // Stored value -> fp32 (bf16 widens exactly).
 __device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
+
+// Row lists of one forward pass: in device memory, or (few rows) in the kernel's own parameters, which saves a small pass
+// the upload in front of it (1.5 us, and 5 us until the kernel behind it starts).
+constexpr int kRowBlob = 1536;
+struct PassRows {
+  const int *row_seq, *row_pos, *lrow_src;   // sequence and position of each row; packed row of each logits row
+  const int4 *attn;                          // work items: (first packed row, rows, sequence, position of first row)
+  const long long *lrow_dst;                 // destination row in the level's logits buffer
+  int in_blob, o_pos, o_attn, o_src, o_dst;  // 1: the lists lie in `blob` (row_seq in front), not at the pointers
+  __align__(16) unsigned char blob[kRowBlob];
+  __device__ __forceinline__ const int *seq() const { return in_blob ? reinterpret_cast<const int *>(blob) : row_seq; }
+  __device__ __forceinline__ const int *pos() const { return in_blob ? reinterpret_cast<const int *>(blob + o_pos) : row_pos; }
+  __device__ __forceinline__ const int *src() const { return in_blob ? reinterpret_cast<const int *>(blob + o_src) : lrow_src; }
+  __device__ __forceinline__ int4 item(int i) const { return in_blob ? reinterpret_cast<const int4 *>(blob + o_attn)[i] : attn[i]; }
+  __device__ __forceinline__ long long dst(int r) const { return in_blob ? reinterpret_cast<const long long *>(blob + o_dst)[r] : lrow_dst[r]; }
+};

@@ -34,7 +34,7 @@ constexpr int kPromptRows = 2304;              // rows of one prompt chunk on th
                                                //   which with 4096-wide outputs make 1.95 rounds of the 74 CTA pairs (eight make 1.73)
 constexpr uint32_t kTraceMagic = 0x48534454u;
 
-constexpr size_t kResultHead = 256;             // the block a decision's host wait copies: status word, then accepted counts
+constexpr size_t kResultHead = 256;             // the block of a decision's results: status word, then accepted counts
 constexpr int kHeadMaps = 17;                   // output-head tensor maps: one per level (<= 16), then the shared head
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -221,10 +221,13 @@ struct hsd_ctx {
   char *ws;
   // pinned host mirrors
   char *ring_host;
-  int *result_host;                           // [kResultHead / 4 + max_batch]: status word, accepted counts
-  int *token_host;                            // decision log: tokens on their way, [3][max_batch][token_stride]
+  // Written by the kernels themselves (mapped), read once the stream has been waited for
+  int *result_host;                           // [kResultHead / 4 + 2 max_batch]: status word, accepted counts, final tokens
+  int *token_host;                            // the latest draws, [max_batch][token_stride]
   int token_stride;
-  std::vector<LogRecord> pending;             // level-0 records whose tokens have been asked for
+  std::vector<int> tokens;                    // decided tokens, [max_batch][max_seq] as on the device (behind the prompt)
+  std::vector<int> drawn_at;                  // [max_batch]: where the latest draws go in it, until a wait has brought them (-1: nowhere)
+  std::vector<LogRecord> pending;             // level-0 records whose tokens the next wait brings
   int *page_table_host;
   int ring_next, ring_in_flight;
   // per-sequence state
@@ -264,11 +267,9 @@ struct hsd_ctx {
 
 namespace {
 
-// Waits for the stream; the status word and the first n_counts accepted counts come along.
-int sync_stream(hsd_ctx *c, int n_counts = 0) {
-  if ((c->any_tc || n_counts > 0) &&
-      cudaMemcpyAsync(c->result_host, c->ws + c->status_off, n_counts > 0 ? kResultHead + (size_t)n_counts * 4 : 4, cudaMemcpyDeviceToHost,
-                      c->stream) != cudaSuccess)
+// Waits for the stream; the status word comes along, unless the kernels of a decision have brought it.
+int sync_stream(hsd_ctx *c, bool decided = false) {
+  if (c->any_tc && !decided && cudaMemcpyAsync(c->result_host, c->ws + c->status_off, 4, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
     return HSD_E_CUDA;
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) return HSD_E_CUDA;
   if (c->any_tc && *c->result_host != 0) return HSD_E_DEVICE_TIMEOUT;
@@ -382,9 +383,10 @@ int project_qkv(hsd_ctx *c, Model &M, int layer, const RowBatch &rb, const void 
 }
 
 // One forward pass of level `level` (layers 1..exit) over the given rows; logits of the wanted
-// rows go to the level's logits buffer.  KV of every processed position is (re)written.  `after`: descriptors of the
-// kernel that follows the pass, uploaded with its own (one copy for both); *after_dev = where they are.
-int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work, const void *after = nullptr, size_t after_bytes = 0,
+// rows go to the level's logits buffer.  KV of every processed position is (re)written.  `after`: n_after descriptors of the
+// kernels that follow the pass.  Few rows and descriptors travel in the kernels' parameters (*after_dev = null); otherwise
+// one upload brings both (*after_dev = where the descriptors are).
+int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work, const void *after = nullptr, int n_after = 0, size_t after_bytes = 0,
             const char **after_dev = nullptr) {
   Model &M = c->model_of(level);
   const ModelDims &md = M.md;
@@ -417,10 +419,6 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work, const void 
          o_src = align_up(o_attn + (size_t)n_attn * 16, 16), o_dst = align_up(o_src + (size_t)n_logit * 4, 16),
          o_after = align_up(o_dst + (size_t)n_logit * 8, 16), bytes = o_after + after_bytes;
   if (bytes > L.ring_slot) return HSD_E_INVALID_ARG;
-  if (after_bytes) {
-    memcpy(host + o_after, after, after_bytes);
-    *after_dev = devp + o_after;
-  }
   int *row_seq = (int *)(host + o_seq), *row_pos = (int *)(host + o_pos), *lsrc = (int *)(host + o_src);
   int4 *attn = (int4 *)(host + o_attn);
   long long *ldst = (long long *)(host + o_dst);
@@ -452,7 +450,20 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work, const void 
   auto item_cost = [&](const int4 &it) { return (long long)(it.w + it.y) * ((it.y * qgroup + 15) / 16); };
   if (M.use_persist && n_attn > 1)
     std::stable_sort(attn, attn + n_attn, [&](const int4 &x, const int4 &y) { return item_cost(x) > item_cost(y); });
-  HSD_CUDA_OK(cudaMemcpyAsync(devp, host, bytes, cudaMemcpyHostToDevice, c->stream));
+  const bool one_launch = (M.use_persist && R <= 128 && n_logit <= 128) || (small && R <= kSmallRows);
+  const bool in_args = one_launch && o_after <= (size_t)kRowBlob && n_after <= kInlineDesc;
+  if (!in_args) {
+    if (after_bytes) memcpy(host + o_after, after, after_bytes);
+    HSD_CUDA_OK(cudaMemcpyAsync(devp, host, bytes, cudaMemcpyHostToDevice, c->stream));
+  }
+  if (after_dev) *after_dev = in_args ? nullptr : devp + o_after;
+  auto pass_rows = [&](PassRows &p) {
+    p.in_blob = in_args;
+    p.o_pos = (int)o_pos; p.o_attn = (int)o_attn; p.o_src = (int)o_src; p.o_dst = (int)o_dst;
+    p.row_seq = (const int *)(devp + o_seq); p.row_pos = (const int *)(devp + o_pos); p.attn = (const int4 *)(devp + o_attn);
+    p.lrow_src = (const int *)(devp + o_src); p.lrow_dst = (const long long *)(devp + o_dst);
+    if (in_args) memcpy(p.blob, host, o_after);
+  };
   st = upload_page_tables(c);
   if (st) return st;
   RowBatch rb;
@@ -553,7 +564,7 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work, const void 
     a.cos_tab = c->dev<float>(ML.cos_tab); a.sin_tab = c->dev<float>(ML.sin_tab);
     a.R = R; a.L = n_logit; a.n_attn = n_attn; a.attn_rows = arows; a.n_splits = n_splits; a.keys_per_split = keys_per_split;
     a.tokens = c->dev<int>(L.tokens); a.page_table = c->dev<int>(L.page_table);
-    a.row_seq = rb.row_seq; a.row_pos = rb.row_pos; a.lrow_src = rb.lrow_src; a.attn_items = rb.attn; a.lrow_dst = rb.lrow_dst;
+    pass_rows(a.rows);
     a.x = c->dev<float>(ML.x);
     a.h = c->dev<__nv_bfloat16>(ML.h); a.q = c->dev<__nv_bfloat16>(ML.q); a.att = c->dev<__nv_bfloat16>(ML.att);
     a.act = c->dev<__nv_bfloat16>(ML.act); a.hf = c->dev<__nv_bfloat16>(ML.hf);
@@ -630,10 +641,11 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work, const void 
     a.logits = (float *)(c->ws + L.logits[level]);
     a.counter = c->dev<unsigned>(L.grid_counter) + 48;        // behind the bf16 forward's two
     a.status = (int *)(c->ws + c->status_off);
+    pass_rows(a.rows);
     for (int g = 0, l0 = 0; g * kSmallRows < R; l0 += a.L, ++g) {       // (a sequence's rows ascend: its earlier keys are there)
       a.R = std::min(kSmallRows, R - g * kSmallRows); a.L = group_logits[g];
-      a.row_seq = rb.row_seq + g * kSmallRows; a.row_pos = rb.row_pos + g * kSmallRows;
-      a.lrow_src = rb.lrow_src + l0; a.lrow_dst = rb.lrow_dst + l0;
+      a.rows.row_seq = rb.row_seq + g * kSmallRows; a.rows.row_pos = rb.row_pos + g * kSmallRows;
+      a.rows.lrow_src = rb.lrow_src + l0; a.rows.lrow_dst = rb.lrow_dst + l0;
       a.base = c->small_base;
       HSD_TRY(launch_forward_small(a, M.small_grid, s));
       c->small_base += fwd_small_arrivals(a.n_run, a.L, M.small_grid);
@@ -660,7 +672,7 @@ int forward(hsd_ctx *c, int level, const std::vector<SeqWork> &work, const void 
       while ((1 << fa.page_shift) < md.page) ++fa.page_shift;
       fa.pages_per_seq = md.pages_per_seq; fa.n_pages = md.n_pages;
       fa.R = R; fa.n_attn = n_attn; fa.attn_rows = arows; fa.n_splits = 1; fa.keys_per_split = keys_per_split;
-      fa.page_table = pt; fa.attn_items = rb.attn; fa.row_seq = rb.row_seq; fa.row_pos = rb.row_pos;
+      fa.page_table = pt; pass_rows(fa.rows);
       fa.q = (__nv_bfloat16 *)q; fa.att = (__nv_bfloat16 *)att; fa.attn_partials = c->dev<float>(ML.partials);
       HSD_TRY(launch_attention_tiles(fa, (__nv_bfloat16 *)kp, (__nv_bfloat16 *)vp, c->sm_count, s));
     } else {
@@ -774,17 +786,6 @@ int forward_prompt(hsd_ctx *c, int level, const std::vector<SeqWork> &work) {
 }
 
 // ---------------------------------------------------------------------------- decision log
-// Asks for n tokens of a sequence; they are at the address returned once the stream has been waited for.  Three places
-// per sequence: 0 = level 0's, 1 = a verification's drafts, 2 = the tokens after its decision.
-int ask_tokens(hsd_ctx *c, int place, int b, int pos0, int n, const int **at) {
-  int *host = c->token_host + ((size_t)place * c->max_batch + b) * c->token_stride;
-  *at = host;
-  if (n > c->token_stride) return HSD_E_INVALID_ARG;
-  if (n == 0) return HSD_OK;
-  return cudaMemcpyAsync(host, c->dev<int>(c->lay.tokens) + (size_t)b * c->md.max_seq + pos0, (size_t)n * 4, cudaMemcpyDeviceToHost, c->stream) == cudaSuccess
-             ? HSD_OK : HSD_E_CUDA;
-}
-
 int trace_write(hsd_ctx *c, const LogRecord &r) {
   const ModelDims &md = c->md;
   const int level = r.level, logit_rows = r.logit_rows;
@@ -806,7 +807,7 @@ int trace_write(hsd_ctx *c, const LogRecord &r) {
   c->trace_records++;
   return HSD_OK;
 }
-// The pending records of level 0; the stream has been waited for since their tokens were asked for.
+// The pending records of level 0; the stream has been waited for since their tokens were drawn.
 int trace_pending(hsd_ctx *c) {
   for (const LogRecord &r : c->pending) HSD_TRY(trace_write(c, r));
   c->pending.clear();
@@ -840,20 +841,22 @@ int run_level0(hsd_ctx *c, const std::vector<int> &act) {
       rows[i].j = j; rows[i].serial = ser[i]; rows[i].seq = b; rows[i].level = 0;
     }
     const char *rows_dev = nullptr;
-    HSD_TRY(forward(c, 0, work, rows.data(), rows.size() * sizeof(SampleRow), &rows_dev));
+    HSD_TRY(forward(c, 0, work, rows.data(), (int)rows.size(), rows.size() * sizeof(SampleRow), &rows_dev));
     for (int b : act) c->buf_len[b]++;
-    HSD_TRY(launch_draft_sample(c->ws + L.logits[0], c->md.dtype, c->md.V, (const SampleRow *)rows_dev, (int)act.size(), 1, 0,
-                                c->seed, c->dev<int>(L.tokens), c->stream));
+    HostMirror mirror;
+    mirror.token = c->token_host;
+    mirror.stride = c->token_stride;
+    HSD_TRY(launch_draft_sample(c->ws + L.logits[0], c->md.dtype, c->md.V, rows_dev ? (const SampleRow *)rows_dev : rows.data(), (int)act.size(), 1, 0,
+                                c->seed, c->dev<int>(L.tokens), c->stream, !rows_dev, mirror));
   }
   for (size_t i = 0; i < act.size(); ++i) {
     hsd_level_stats &st = c->stats[0];
     st.calls++;
     st.emitted += steps;
-    if (c->trace) {                             // written behind the wait of the verification that follows
-      LogRecord r = {0, act[i], ser[i], ctx0[i], 0, steps, steps, steps, (long long)act[i] * L.slots[0], nullptr, steps};
-      HSD_TRY(ask_tokens(c, 0, act[i], ctx0[i], steps, &r.tokens));
-      c->pending.push_back(r);
-    }
+    c->drawn_at[act[i]] = ctx0[i];
+    if (c->trace)                               // written behind the wait of the verification that follows
+      c->pending.push_back(LogRecord{0, act[i], ser[i], ctx0[i], 0, steps, steps, steps, (long long)act[i] * L.slots[0],
+                                     c->token_host + (size_t)act[i] * c->token_stride, steps});
   }
   if (c->trace && c->n_levels == 1) {
     HSD_TRY(sync_stream(c));
@@ -887,21 +890,30 @@ int run_verify(hsd_ctx *c, int level, const std::vector<int> &act, const std::ve
     vs[i].serial = ser[i]; vs[i].seq = b; vs[i].level = level;
   }
   const char *vs_dev = nullptr;
-  HSD_TRY(forward(c, level, work, vs.data(), vs.size() * sizeof(VerifySeq), &vs_dev));
-  std::vector<const int *> drafts(act.size()), after(act.size());
-  if (c->trace)                                 // (the decision writes its final token over one of the drafts)
-    for (size_t i = 0; i < act.size(); ++i) HSD_TRY(ask_tokens(c, 1, act[i], ctx[act[i]], vs[i].t, &drafts[i]));
+  HSD_TRY(forward(c, level, work, vs.data(), (int)vs.size(), vs.size() * sizeof(VerifySeq), &vs_dev));
+  HostMirror mirror;
+  mirror.status = c->result_host;
+  mirror.status_src = (const int *)(c->ws + c->status_off);
+  mirror.n = c->result_host + kResultHead / 4;
+  mirror.token = mirror.n + c->max_batch;
+  for (size_t i = 0; i < act.size(); ++i) mirror.n[i] = -1;       // (nothing is in flight that writes there: the last decision was waited for)
   HSD_TRY(launch_verify(c->ws + L.logits[level], c->ws + L.logits[level - 1], c->dev<int>(L.tokens), c->md.dtype, c->md.V,
-                        (int)act.size(), t_max, (const VerifySeq *)vs_dev, 0, 0, 0, c->ws + L.vscratch, c->seed, nullptr,
-                        c->dev<int>(L.result + kResultHead), 1, c->stream, c->coin24[level]));
-  if (c->trace)
-    for (size_t i = 0; i < act.size(); ++i) HSD_TRY(ask_tokens(c, 2, act[i], ctx[act[i]], vs[i].t + 1, &after[i]));
-  HSD_TRY(sync_stream(c, (int)act.size()));
+                        (int)act.size(), t_max, vs_dev ? (const VerifySeq *)vs_dev : vs.data(), 0, 0, 0, c->ws + L.vscratch, c->seed, nullptr,
+                        c->dev<int>(L.result + kResultHead), 1, c->stream, c->coin24[level], !vs_dev, mirror));
+  HSD_TRY(sync_stream(c, true));
   if (c->trace) HSD_TRY(trace_pending(c));
+  for (int b = 0; b < c->max_batch; ++b)        // the draws since the last wait
+    if (c->drawn_at[b] >= 0) {
+      memcpy(&c->tokens[(size_t)b * c->md.max_seq + c->drawn_at[b]], c->token_host + (size_t)b * c->token_stride, (size_t)c->T[0] * 4);
+      c->drawn_at[b] = -1;
+    }
   hsd_level_stats &st = c->stats[level];
   for (size_t i = 0; i < act.size(); ++i) {
-    int b = act[i], t = c->buf_len[b] - ctx[b], n = c->result_host[kResultHead / 4 + i];
+    int b = act[i], t = c->buf_len[b] - ctx[b], n = mirror.n[i];
     if (n < 0 || n > t) return HSD_E_CUDA;
+    int *toks = &c->tokens[(size_t)b * c->md.max_seq + ctx[b]];
+    const std::vector<int> drafts(toks, toks + t);
+    toks[n] = mirror.token[i];                  // the final token m
     // rollback / commit: the buffer keeps x_1..x_n and m; the position of m (and everything the
     // rejected drafts wrote) is valid in no layer group
     c->buf_len[b] = ctx[b] + n + 1;
@@ -913,10 +925,10 @@ int run_verify(hsd_ctx *c, int level, const std::vector<int> &act, const std::ve
     st.accepted += n;
     st.emitted += n + 1;
     if (c->trace) {
-      std::vector<int> toks(drafts[i], drafts[i] + t);
-      toks.push_back(after[i][n]);                                    // the final token m
+      std::vector<int> decided(drafts);
+      decided.push_back(toks[n]);
       HSD_TRY(trace_write(c, LogRecord{level, b, ser[i], ctx[b], t, n, work[i].end - work[i].start, t + 1,
-                                       (long long)b * L.slots[level] + count[b], toks.data(), t + 1}));
+                                       (long long)b * L.slots[level] + count[b], decided.data(), t + 1}));
     }
     count[b] += n + 1;
   }
@@ -1103,14 +1115,14 @@ int create_ctx(const hsd_model_desc *models, int n_models, const int32_t *exit_l
   c->ws = (char *)workspace;
   c->coin24.assign(n_levels, kNoCoin);
   c->ring_host = nullptr; c->result_host = nullptr; c->token_host = nullptr; c->page_table_host = nullptr;
-  c->token_stride = lay.slots[n_levels - 1] + 1;          // a verification's drafts and one more
+  c->token_stride = lay.slots[n_levels - 1] + 1;          // a level-0 call's draws fit
   c->sm_count = device_sm_count();
   c->trace = nullptr; c->trace_logit_calls = 0; c->trace_records = 0;
   c->ring_next = 0; c->ring_in_flight = 0; c->timers_used = 0; c->timers_ok = true; c->stream = nullptr; c->seed = 0;
   c->status_off = lay.result;
   bool ok = cudaMallocHost(&c->ring_host, lay.ring_slot * kRingSlots) == cudaSuccess &&
-            cudaMallocHost(&c->result_host, kResultHead + (size_t)c->max_batch * 4) == cudaSuccess &&
-            cudaMallocHost(&c->token_host, (size_t)3 * c->max_batch * c->token_stride * 4) == cudaSuccess &&
+            cudaHostAlloc(&c->result_host, kResultHead + (size_t)2 * c->max_batch * 4, cudaHostAllocMapped) == cudaSuccess &&
+            cudaHostAlloc(&c->token_host, (size_t)c->max_batch * c->token_stride * 4, cudaHostAllocMapped) == cudaSuccess &&
             cudaMallocHost(&c->page_table_host, (size_t)c->max_batch * lay.pages_per_seq * 4) == cudaSuccess;
   for (int i = 0; i < kTimerPairs; ++i) { c->timers[i].a = nullptr; c->timers[i].b = nullptr; }
   for (int i = 0; ok && i < kTimerPairs; ++i)
@@ -1208,6 +1220,8 @@ int hsd_generate(hsd_ctx *c, const int32_t *prompt_ids, int batch, int prompt_le
   for (int p = c->lay.n_pages - 1; p >= 0; --p) c->free_pages.push_back(p);
   c->trace_records = 0;
   c->pending.clear();
+  c->tokens.resize((size_t)c->max_batch * c->md.max_seq);
+  c->drawn_at.assign(c->max_batch, -1);
   cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
   bool ev = cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess && cudaEventCreate(&e2) == cudaSuccess;
   int st = HSD_OK;

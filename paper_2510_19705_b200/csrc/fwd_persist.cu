@@ -366,7 +366,7 @@ __device__ __forceinline__ void norm_phase(const FwdArgs &a, int n_rows, const i
     float4 v[MAXV];
     if (src_embed) {
       // an id outside the vocabulary (only possible after non-finite logits) must not become an address
-      const int tok = min(max(a.tokens[(size_t)a.row_seq[row] * a.max_seq + a.row_pos[row]], 0), a.V - 1);
+      const int tok = min(max(a.tokens[(size_t)a.rows.seq()[row] * a.max_seq + a.rows.pos()[row]], 0), a.V - 1);
       const __nv_bfloat16 *erow = a.embed + (size_t)tok * d;
       uint2 raw[MAXV];
 #pragma unroll
@@ -869,7 +869,7 @@ __device__ __forceinline__ bool attn_tiles_phase(const FwdArgs &a, const LayerCa
 #endif
     const int split = wi % a.n_splits, kvh = (wi / a.n_splits) % a.nkv, ai = wi / (a.n_splits * a.nkv);
     const int4 it = wi == (int)blockIdx.x ? make_int4(first_item[0], first_item[1], first_item[2], first_item[3])
-                                          : a.attn_items[ai];   // the CTA's first item was fetched at kernel start
+                                          : a.rows.item(ai);   // the CTA's first item was fetched at kernel start
     const int row0 = it.x, nrows = it.y, seq = it.z, pos0 = it.w;
     const int kv_len = pos0 + nrows;
     const int key_lo = split * a.keys_per_split, key_hi = min(kv_len, key_lo + a.keys_per_split);
@@ -1246,7 +1246,7 @@ __device__ __forceinline__ void final_store(const FwdArgs &a, const Gemm &g, con
 #pragma unroll
       for (int i = 0; i < CH; ++i) {
         const int r = c0 + i;
-        if (r < rows) a.logits[(size_t)a.lrow_dst[r] * a.V + n] = __float2bfloat16_rn(v[i]);
+        if (r < rows) a.logits[(size_t)a.rows.dst(r) * a.V + n] = __float2bfloat16_rn(v[i]);
       }
     }
   } else if (g.mode == MODE_SWIGLU) {
@@ -1325,7 +1325,7 @@ __device__ __forceinline__ void put_partial_holes(const FwdArgs &a, int wt, cons
 #pragma unroll 1
   for (int wi = blockIdx.x; wi < n_work; wi += gridDim.x) {
     const int unit = wi / a.n_splits, split = wi - unit * a.n_splits, ai = unit / a.nkv, kvh = unit - ai * a.nkv;
-    const int4 it = wi == (int)blockIdx.x ? make_int4(first_item[0], first_item[1], first_item[2], first_item[3]) : a.attn_items[ai];
+    const int4 it = wi == (int)blockIdx.x ? make_int4(first_item[0], first_item[1], first_item[2], first_item[3]) : a.rows.item(ai);
     const int key_lo = split * a.keys_per_split;
     if (key_lo >= it.w + it.y) continue;
     for (int qi = max(0, key_lo - it.w) * group + ((wt >> 5) & 3); qi < it.y * group; qi += 4) {       // rows from key_lo on wrote theirs
@@ -1770,20 +1770,20 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
     if (a.R <= kRopeCacheRows)
       for (int i = wt; i < a.R * (HD / 2); i += 256) {
         const int r = i / (HD / 2), k = i % (HD / 2);
-        rope_cos_sh[i] = a.cos_tab[(size_t)a.row_pos[r] * (HD / 2) + k];
-        rope_sin_sh[i] = a.sin_tab[(size_t)a.row_pos[r] * (HD / 2) + k];
+        rope_cos_sh[i] = a.cos_tab[(size_t)a.rows.pos()[r] * (HD / 2) + k];
+        rope_sin_sh[i] = a.sin_tab[(size_t)a.rows.pos()[r] * (HD / 2) + k];
       }
     for (int r = wt; r < a.R; r += 256) {             // per-row facts every layer needs, fetched once
-      const int pos = a.row_pos[r];
+      const int pos = a.rows.pos()[r];
       row_pos_sh[r] = pos;
-      row_pg_sh[r] = a.page_table[(size_t)a.row_seq[r] * a.pages_per_seq + pos / a.page];
+      row_pg_sh[r] = a.page_table[(size_t)a.rows.seq()[r] * a.pages_per_seq + pos / a.page];
     }
     // descriptor of this CTA's first attention work item, kept in shared memory (the same in every layer; a
     // dependent global load at the start of every attention phase otherwise)
     if (wt == 0) {
       const int n_work = a.n_attn * a.nkv * a.n_splits;
       int4 fi = make_int4(0, 0, 0, 0);
-      if ((int)blockIdx.x < n_work) fi = a.attn_items[blockIdx.x / (a.n_splits * a.nkv)];
+      if ((int)blockIdx.x < n_work) fi = a.rows.item(blockIdx.x / (a.n_splits * a.nkv));
       first_item_sh[0] = fi.x; first_item_sh[1] = fi.y; first_item_sh[2] = fi.z; first_item_sh[3] = fi.w;
       const PhaseGeom &pq = geom_sh[0];
       qkv_geom_sh[0] = (a.nq * a.hd + kTcBlockM - 1) / kTcBlockM;
@@ -1881,7 +1881,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_persistent_kernel(const __
           const __nv_bfloat16 *gain = first ? a.layers[0].attn_norm
                                             : (last ? a.final_norm : (mid ? norms_sh[l].mlp_norm : norms_sh[l + 1].attn_norm));
           auto norm = [&](auto slots) {
-            norm_phase<NPAD, decltype(slots)::value>(a, last ? a.L : a.R, last ? a.lrow_src : nullptr, first,
+            norm_phase<NPAD, decltype(slots)::value>(a, last ? a.L : a.R, last ? a.rows.src() : nullptr, first,
                                                      first ? nullptr : a.pieces[gp & 3], geom_sh[gp & 3].pieces_max, gain, last ? a.hf : a.h,
                                                      red, wt, abort_flag);
           };
@@ -1923,7 +1923,7 @@ __global__ void __launch_bounds__(256, 2) attn_tiles_kernel(const __grid_constan
     pcache.tag_item = -1;
     const int n_work = a.n_attn * a.nkv * a.n_splits;
     int4 fi = make_int4(0, 0, 0, 0);
-    if ((int)blockIdx.x < n_work) fi = a.attn_items[blockIdx.x / (a.n_splits * a.nkv)];
+    if ((int)blockIdx.x < n_work) fi = a.rows.item(blockIdx.x / (a.n_splits * a.nkv));
     first_item_sh[0] = fi.x; first_item_sh[1] = fi.y; first_item_sh[2] = fi.z; first_item_sh[3] = fi.w;
   }
   __syncthreads();

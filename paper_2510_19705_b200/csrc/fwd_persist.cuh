@@ -31,9 +31,8 @@ struct FwdArgs {
   int gu_pieces_max;               // pieces per gate / up tile at most (its split geometry; filled in by the launcher)
   int early_norm;                  // 0: a grid barrier between a residual projection and the norm that sums its pieces
   int tc_attn;                     // 1: work items with long key ranges run on tcgen05 / tensor memory (head size 128; needs fuse_qkv = 0)
-  const int *tokens, *page_table, *row_seq, *row_pos, *lrow_src;
-  const int4 *attn_items;          // (first packed row, rows, sequence, position of first row)
-  const long long *lrow_dst;
+  const int *tokens, *page_table;
+  PassRows rows;
   // buffers
   float *x;
   __nv_bfloat16 *h, *q, *att, *act, *hf, *logits;
@@ -58,7 +57,7 @@ bool fwd_persist_supported(int hd, int group);
 size_t fwd_pieces_bytes(int d, int nqd, int nkvd, int ff, int V, int sm_count);   // of the pieces, for passes of up to 128 rows
 int launch_forward_persistent(const FwdArgs &args, int npad, int sm_count, cudaStream_t s);
 // The attention tiles phase alone, one key split per item (args: geometry, R, n_attn, attn_rows, n_splits = 1,
-// keys_per_split, page table, attn_items, q, att; fuse_qkv = 0): the item's rows of `att` are written.
+// keys_per_split, page table, rows, q, att; fuse_qkv = 0): the item's rows of `att` are written.
 int launch_attention_tiles(const FwdArgs &args, __nv_bfloat16 *k_pool, __nv_bfloat16 *v_pool, int sm_count, cudaStream_t s);
 
 }  // namespace hsd

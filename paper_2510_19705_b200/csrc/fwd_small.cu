@@ -196,7 +196,7 @@ __device__ __forceinline__ void product_phase(Shared &sh, const Src &src, const 
 // `first`: the thread's cache row in the CTA's first unit, key = thread (the same in every layer: found once).
 __device__ __forceinline__ int cache_row(const SmallFwdArgs &a, int u, int key) {
   const int r = u / a.nq, kvh = (u - r * a.nq) / (a.nq / a.nkv);
-  return (kvh * a.n_pages + a.page_table[(size_t)a.row_seq[r] * a.pages_per_seq + key / a.page]) * a.page + key % a.page;
+  return (kvh * a.n_pages + a.page_table[(size_t)a.rows.seq()[r] * a.pages_per_seq + key / a.page]) * a.page + key % a.page;
 }
 template <int HD> __device__ __forceinline__ void attention_phase(const SmallFwdArgs &a, const SmallLayerDev &ly, Shared &sh, int first) {
   constexpr int LPR = HD / 4, RPI = 32 / LPR, NI = 32 / RPI, PRE = NI < 8 ? NI : 8;   // lanes of a row, rows at a time
@@ -282,8 +282,8 @@ __global__ void __launch_bounds__(kThreads) fwd_small_kernel(const __grid_consta
   unsigned target = a.base;
   constexpr int HALF = HD / 2;
   if (tid < a.R) {
-    const int seq = a.row_seq[tid];
-    sh.pos[tid] = a.row_pos[tid];
+    const int seq = a.rows.seq()[tid];
+    sh.pos[tid] = a.rows.pos()[tid];
     sh.pg[tid] = a.page_table[(size_t)seq * a.pages_per_seq + sh.pos[tid] / a.page];
     // an id outside the vocabulary (only possible after non-finite logits) must not become an address
     sh.tok[tid] = min(max(a.tokens[(size_t)seq * a.max_seq + sh.pos[tid]], 0), a.V - 1);
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(kThreads) fwd_small_kernel(const __grid_consta
       if (!barrier(a, target, sh)) return;
   }
   if (a.L > 0) {
-    auto xl = [&](int r) { return (const float *)(a.x + (size_t)a.lrow_src[r] * a.d); };
+    auto xl = [&](int r) { return (const float *)(a.x + (size_t)a.rows.src()[r] * a.d); };
     row_scales(sh, xl, a.L, a.d, a.eps);
     product_phase<RT>(sh, xl, a.final_norm, a.eps, a.d, a.L, (a.V + 1) / 2,
                       [&](int p, const float *&w0, const float *&w1) {
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(kThreads) fwd_small_kernel(const __grid_consta
                         w1 = 2 * p + 1 < a.V ? w0 + a.d : w0;
                       },
                       [&](int p, int r, float v0, float v1) {
-                        float *dst = a.logits + (size_t)a.lrow_dst[r] * a.V + 2 * p;
+                        float *dst = a.logits + (size_t)a.rows.dst(r) * a.V + 2 * p;
                         dst[0] = v0;
                         if (2 * p + 1 < a.V) dst[1] = v1;
                       });

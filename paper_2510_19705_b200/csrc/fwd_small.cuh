@@ -13,8 +13,8 @@ struct SmallFwdArgs {
   const SmallLayerDev *layers;       // global memory [n_layers]
   const float *embed, *final_norm, *lm_head, *cos_tab, *sin_tab;
   int R, L;                          // <= kSmallRows
-  const int *tokens, *page_table, *row_seq, *row_pos, *lrow_src;
-  const long long *lrow_dst;
+  const int *tokens, *page_table;
+  PassRows rows;
   float *x, *q, *att, *act, *logits;
   unsigned *counter;                 // counts barrier arrivals, never reset: `base` = its value when the launch starts
   unsigned base;

@@ -10,17 +10,33 @@ namespace hsd {
 
 // ------------------------------------------------------------------------------ draft sampling
 // One block per row: token = inverse-CDF sample of softmax(row) with the purpose-0 uniform.
+// A call's descriptors: n_inline of them here, or all at `desc`, or (both zero) worked out from the regular layout.
+template <typename D> struct DescList {
+  const D *desc;
+  int n_inline;
+  D inl[kInlineDesc];
+  __device__ __forceinline__ bool given() const { return n_inline > 0 || desc; }
+  __device__ __forceinline__ D at(int i) const { return n_inline > 0 ? inl[i] : desc[i]; }
+};
+template <typename D> static DescList<D> desc_list(const D *desc, int n, bool on_host) {
+  DescList<D> l;
+  l.desc = on_host ? nullptr : desc;
+  l.n_inline = on_host ? n : 0;
+  for (int i = 0; i < l.n_inline; ++i) l.inl[i] = desc[i];
+  return l;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kSampleThreads)
-draft_sample_kernel(const T *__restrict__ logits, int V, const SampleRow *__restrict__ desc,
-                    int regular_rows, u32 regular_serial, u64 seed, int32_t *__restrict__ out) {
+draft_sample_kernel(const T *__restrict__ logits, int V, const __grid_constant__ DescList<SampleRow> desc,
+                    int regular_rows, u32 regular_serial, u64 seed, int32_t *__restrict__ out, const HostMirror mirror) {
   __shared__ float shf[32];
   __shared__ u64 sh64[34];
   chain_wait();
   chain_next();
   SampleRow d;
-  if (desc) {
-    d = desc[blockIdx.x];
+  if (desc.given()) {
+    d = desc.at(blockIdx.x);
   } else {
     d.logit_row = blockIdx.x;
     d.out_index = blockIdx.x;
@@ -41,7 +57,10 @@ draft_sample_kernel(const T *__restrict__ logits, int V, const SampleRow *__rest
     float m = row_max(row, V, shf);
     tok = block_inverse_cdf(V, U, [&](int k) { return (u64)exp_weight(to_f32(row[k]), m); }, sh64, nullptr);
   }
-  if (threadIdx.x == 0) out[d.out_index] = tok;
+  if (threadIdx.x == 0) {
+    out[d.out_index] = tok;
+    if (mirror.token) mirror.token[(size_t)d.seq * mirror.stride + d.j] = tok;
+  }
 }
 
 // 16 bytes of a row
@@ -68,14 +87,14 @@ template <> struct StatVec<float> {
 template <typename T>
 __global__ void __launch_bounds__(kSampleThreads)
 decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, int32_t *__restrict__ tokens, int V,
-              int t_max, const VerifySeq *__restrict__ desc, int regular_t, u32 regular_serial, u32 regular_level,
+              int t_max, const __grid_constant__ DescList<VerifySeq> desc, int regular_t, u32 regular_serial, u32 regular_level,
               const RowStat *__restrict__ stats, u64 seed, int32_t *__restrict__ out_tokens /*[B, t_max+1] or null*/,
-              int32_t *__restrict__ out_n /*[B]*/, int write_in_place, u32 coin24) {
+              int32_t *__restrict__ out_n /*[B]*/, int write_in_place, u32 coin24, const HostMirror mirror) {
   __shared__ u64 sh64[34];
   __shared__ int sh_first_reject;
   int b = blockIdx.x;
   VerifySeq d;
-  if (desc) d = desc[b];
+  if (desc.given()) d = desc.at(b);
   else {
     d.t = regular_t; d.p_row0 = (long long)b * (regular_t + 1); d.q_row0 = (long long)b * regular_t;
     d.tok_off = (long long)b * regular_t; d.serial = regular_serial; d.seq = b; d.level = regular_level;
@@ -133,6 +152,8 @@ decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, in
   if (threadIdx.x == 0) {
     out_n[b] = n;
     if (write_in_place) tokens[d.tok_off + n] = m_tok;
+    if (mirror.n) { mirror.n[b] = n; mirror.token[b] = m_tok; }
+    if (mirror.status && b == 0) *mirror.status = __ldcg(mirror.status_src);
   }
   if (out_tokens) {
     for (int j = threadIdx.x; j <= t_max; j += blockDim.x) {
@@ -160,7 +181,7 @@ constexpr int kRsMaxEdge = 16;
 struct RowStatArgs {
   const void *p, *q;
   int V, t_max, batch, regular_t;
-  const VerifySeq *desc;
+  DescList<VerifySeq> desc;
   RowStat *stats;
 };
 struct RsInfo {
@@ -241,10 +262,10 @@ __global__ void __launch_bounds__(32 * (GROUPS * WARPS + 1), 1) row_stats_kernel
       const bool is_p = r <= a.t_max;
       const int at = is_p ? r : r - a.t_max - 1;
       long long row0;
-      if (a.desc) {
-        const int t = a.desc[b].t;
-        if (at >= t + (is_p ? 1 : 0)) continue;
-        row0 = is_p ? a.desc[b].p_row0 : a.desc[b].q_row0;
+      if (a.desc.given()) {
+        const VerifySeq d = a.desc.at(b);
+        if (at >= d.t + (is_p ? 1 : 0)) continue;
+        row0 = is_p ? d.p_row0 : d.q_row0;
       } else row0 = (long long)b * (a.regular_t + (is_p ? 1 : 0));
       const T *row = reinterpret_cast<const T *>(is_p ? a.p : a.q) + (size_t)(row0 + at) * a.V;
       const uintptr_t lo = reinterpret_cast<uintptr_t>(row), hi = lo + (size_t)a.V * ES;
@@ -417,8 +438,9 @@ struct ClusterArgs {
   const void *p, *q;
   int32_t *tokens;
   int V, t_max, seg;             // seg: tokens per CTA, a multiple of 64
-  const VerifySeq *desc;         // verification: per sequence, or null (regular)
-  const SampleRow *rows;         // draws: per row, or null (regular)
+  DescList<VerifySeq> desc;      // verification: per sequence
+  DescList<SampleRow> rows;      // draws: per row
+  HostMirror mirror;
   int regular_t;                 // draws: rows per sequence
   u32 regular_serial, regular_level;
   u64 seed;
@@ -520,11 +542,11 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
   u32 uj = 0;
   if (DRAW) {
     SampleRow s;
-    if (a.rows) s = a.rows[b];
+    if (a.rows.given()) s = a.rows.at(b);
     else { s.logit_row = b; s.out_index = b; s.j = b % a.regular_t; s.seq = b / a.regular_t; s.serial = a.regular_serial; s.level = 0; }
     d.p_row0 = s.logit_row; d.q_row0 = 0; d.tok_off = 0; d.t = 0; d.serial = s.serial; d.seq = s.seq; d.level = s.level;
     out_index = s.out_index; uj = s.j;
-  } else if (a.desc) d = a.desc[b];
+  } else if (a.desc.given()) d = a.desc.at(b);
   else {
     d.t = a.regular_t; d.p_row0 = (long long)b * (a.regular_t + 1); d.q_row0 = (long long)b * a.regular_t;
     d.tok_off = (long long)b * a.regular_t; d.serial = a.regular_serial; d.seq = b; d.level = a.regular_level;
@@ -699,25 +721,27 @@ __global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kerne
   const u64 tau = cdf_threshold(U, total);
   u64 before = 0;
   for (u32 c = 0; c < rank; ++c) before += csum[src][c];
-  if (total == 0) {                                                // non-finite logits: no token
-    if (rank == 0 && tid == 0) {
-      if (DRAW) a.out_tokens[out_index] = -1;
-      else {
-        if (a.write_in_place) a.tokens[d.tok_off + n] = -1;
-        if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = -1;
-      }
+  auto emit = [&](int k) {
+    if (DRAW) {
+      a.out_tokens[out_index] = k;
+      if (a.mirror.token) a.mirror.token[(size_t)d.seq * a.mirror.stride + uj] = k;
+    } else {
+      if (a.write_in_place) a.tokens[d.tok_off + n] = k;
+      if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = k;
+      if (a.mirror.n) a.mirror.token[b] = k;
     }
+  };
+  if (total == 0) {                                                // non-finite logits: no token
+    if (rank == 0 && tid == 0) emit(-1);
   } else if (tau >= before && tau < before + csum[src][rank]) {
-    cl_find_token<NT, PER>(w, tau, before, wsum + src * kClWarps, k_lane, [&](int k) {
-      if (DRAW) a.out_tokens[out_index] = k;
-      else {
-        if (a.write_in_place) a.tokens[d.tok_off + n] = k;
-        if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = k;
-      }
-    });
+    cl_find_token<NT, PER>(w, tau, before, wsum + src * kClWarps, k_lane, emit);
   }
   if (!DRAW && rank == 0) {
-    if (tid == 0) a.out_n[b] = n;
+    if (tid == 0) {
+      a.out_n[b] = n;
+      if (a.mirror.n) a.mirror.n[b] = n;
+      if (a.mirror.status && b == 0) *a.mirror.status = __ldcg(a.mirror.status_src);
+    }
     if (a.out_tokens && tid <= a.t_max && tid != n) a.out_tokens[(size_t)b * (a.t_max + 1) + tid] = tid < n ? tok : -1;
   }
 }
@@ -737,7 +761,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
   const int b = (int)cl_id();
   cl_arrive();                                                     // (the wait is in front of the first store to a peer)
   VerifySeq d;
-  if (a.desc) d = a.desc[b];
+  if (a.desc.given()) d = a.desc.at(b);
   else {
     d.t = a.regular_t; d.p_row0 = (long long)b * (a.regular_t + 1); d.q_row0 = (long long)b * a.regular_t;
     d.tok_off = (long long)b * a.regular_t; d.serial = a.regular_serial; d.seq = b; d.level = a.regular_level;
@@ -847,6 +871,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
   auto emit = [&](int k) {
     if (a.write_in_place) a.tokens[d.tok_off + n] = k;
     if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = k;
+    if (a.mirror.n) a.mirror.token[b] = k;
   };
   if (total == 0) {                                                // non-finite logits: no token
     if (rank == 0 && tid == 0) emit(-1);
@@ -854,7 +879,11 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
     cl_find_token<NT, PER>(w, tau, before, wsum[src], k_lane, emit);
   }
   if (rank == 0) {
-    if (tid == 0) a.out_n[b] = n;
+    if (tid == 0) {
+      a.out_n[b] = n;
+      if (a.mirror.n) a.mirror.n[b] = n;
+      if (a.mirror.status && b == 0) *a.mirror.status = __ldcg(a.mirror.status_src);
+    }
     if (a.out_tokens)
       for (int j = tid; j <= a.t_max; j += kClThreads)
         if (j != n) a.out_tokens[(size_t)b * (a.t_max + 1) + j] = j < n ? a.tokens[d.tok_off + j] : -1;
@@ -934,27 +963,29 @@ size_t verify_scratch_bytes(int batch, int t_max) {
 }
 
 template <typename T>
-static int launch_draft_sample_t(const void *logits, int V, const SampleRow *desc, int n_rows, int regular_rows,
-                                 u32 regular_serial, u64 seed, int32_t *out, cudaStream_t s) {
-  HSD_CUDA_OK(hsd_launch(draft_sample_kernel<T>, n_rows, kSampleThreads, 0, s, 0, true, (const T *)logits, V, desc, regular_rows, regular_serial, seed, out));
+static int launch_draft_sample_t(const void *logits, int V, const DescList<SampleRow> &desc, int n_rows, int regular_rows,
+                                 u32 regular_serial, u64 seed, int32_t *out, cudaStream_t s, const HostMirror &mirror) {
+  HSD_CUDA_OK(hsd_launch(draft_sample_kernel<T>, n_rows, kSampleThreads, 0, s, 0, true, (const T *)logits, V, desc, regular_rows, regular_serial, seed, out, mirror));
   hsd_count_launches(1);
   return hsd_launch_status();
 }
 
 int launch_draft_sample(const void *logits, int dtype, int V, const SampleRow *desc, int n_rows, int regular_rows,
-                        u32 regular_serial, u64 seed, int32_t *out, cudaStream_t s) {
+                        u32 regular_serial, u64 seed, int32_t *out, cudaStream_t s, bool desc_on_host, HostMirror mirror) {
   if (n_rows == 0) return HSD_OK;
+  if (desc_on_host && n_rows > kInlineDesc) return HSD_E_INVALID_ARG;
+  const DescList<SampleRow> list = desc_list(desc, n_rows, desc_on_host);
   ClusterPlan pl;
   if (cluster_plan(logits, nullptr, dtype, V, n_rows, 1, true, &pl) &&
       cluster_pays_draw(pl, V, n_rows, dtype == HSD_BF16 && V % 8 == 0 && V <= kSampleThreads * kChunkTokens && ((uintptr_t)logits & 15) == 0)) {
     ClusterArgs a = {};
-    a.p = logits; a.V = V; a.t_max = 0; a.rows = desc; a.regular_t = regular_rows;
+    a.p = logits; a.V = V; a.t_max = 0; a.rows = list; a.mirror = mirror; a.regular_t = regular_rows;
     a.regular_serial = regular_serial; a.seed = seed; a.out_tokens = out; a.coin24 = kNoCoin;
     return launch_cluster<true>(a, pl, dtype, n_rows, s);
   }
   return dtype == HSD_BF16
-             ? launch_draft_sample_t<__nv_bfloat16>(logits, V, desc, n_rows, regular_rows, regular_serial, seed, out, s)
-             : launch_draft_sample_t<float>(logits, V, desc, n_rows, regular_rows, regular_serial, seed, out, s);
+             ? launch_draft_sample_t<__nv_bfloat16>(logits, V, list, n_rows, regular_rows, regular_serial, seed, out, s, mirror)
+             : launch_draft_sample_t<float>(logits, V, list, n_rows, regular_rows, regular_serial, seed, out, s, mirror);
 }
 
 static int sm_count() {
@@ -1001,18 +1032,20 @@ static int launch_decide_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, 
 int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int V, int batch, int t_max,
                   const VerifySeq *desc, int regular_t, u32 regular_serial, u32 regular_level, void *scratch,
                   u64 seed, int32_t *out_tokens, int32_t *out_n, int write_in_place, cudaStream_t s,
-                  u32 coin24) {
+                  u32 coin24, bool desc_on_host, HostMirror mirror) {
   if (batch == 0) return HSD_OK;
+  if (desc_on_host && batch > kInlineDesc) return HSD_E_INVALID_ARG;
+  const DescList<VerifySeq> list = desc_list(desc, batch, desc_on_host);
   RowStat *stats = (RowStat *)((char *)scratch + verify_counter_bytes(batch));
   ClusterArgs a = {};
-  a.p = p; a.q = q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.desc = desc; a.regular_t = regular_t;
+  a.p = p; a.q = q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.desc = list; a.mirror = mirror; a.regular_t = regular_t;
   a.regular_serial = regular_serial; a.regular_level = regular_level; a.seed = seed; a.out_tokens = out_tokens; a.out_n = out_n;
   a.write_in_place = write_in_place; a.coin24 = coin24;
   ClusterPlan pl;
   if (2 * t_max + 1 <= kClMaxRows && cluster_plan(p, q, dtype, V, batch, 2 * t_max + 1, false, &pl) && cluster_pays_verify(pl, V, batch))
     return launch_cluster<false>(a, pl, dtype, batch, s);
   RowStatArgs r = {};
-  r.p = p; r.q = q; r.V = V; r.t_max = t_max; r.batch = batch; r.regular_t = regular_t; r.desc = desc; r.stats = stats;
+  r.p = p; r.q = q; r.V = V; r.t_max = t_max; r.batch = batch; r.regular_t = regular_t; r.desc = list; r.stats = stats;
   const int st = launch_row_stats(r, dtype, s);
   if (st) return st;
   if (cluster_plan(p, q, dtype, V, batch, 1, false, &pl)) {     // a decision reads one row of each side
@@ -1022,11 +1055,11 @@ int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int 
   }
   // rows of more than 131072 tokens
   if (dtype == HSD_BF16)
-    decide_kernel<__nv_bfloat16><<<batch, kSampleThreads, 0, s>>>((const __nv_bfloat16 *)p, (const __nv_bfloat16 *)q, tokens, V, t_max, desc, regular_t,
-                                                                  regular_serial, regular_level, stats, seed, out_tokens, out_n, write_in_place, coin24);
+    decide_kernel<__nv_bfloat16><<<batch, kSampleThreads, 0, s>>>((const __nv_bfloat16 *)p, (const __nv_bfloat16 *)q, tokens, V, t_max, list, regular_t,
+                                                                  regular_serial, regular_level, stats, seed, out_tokens, out_n, write_in_place, coin24, mirror);
   else
-    decide_kernel<float><<<batch, kSampleThreads, 0, s>>>((const float *)p, (const float *)q, tokens, V, t_max, desc, regular_t,
-                                                          regular_serial, regular_level, stats, seed, out_tokens, out_n, write_in_place, coin24);
+    decide_kernel<float><<<batch, kSampleThreads, 0, s>>>((const float *)p, (const float *)q, tokens, V, t_max, list, regular_t,
+                                                          regular_serial, regular_level, stats, seed, out_tokens, out_n, write_in_place, coin24, mirror);
   hsd_count_launches(1);
   return hsd_launch_status();
 }

@@ -29,8 +29,20 @@ struct __align__(16) RowStat {
 
 size_t verify_scratch_bytes(int batch, int t_max);
 
+// Descriptors of a call: in device memory, or (few of them) in host memory, from where they go into the kernels' parameters.
+constexpr int kInlineDesc = 8;
+// What the kernels write for the host besides their outputs (mapped host memory; all null: nothing).  A draw's token goes to
+// token[seq * stride + j], a verification's final token and accepted count to token[b] and n[b], and status_src's word to status.
+struct HostMirror {
+  int32_t *token = nullptr, *n = nullptr;
+  int *status = nullptr;
+  const int *status_src = nullptr;
+  int stride = 0;
+};
+
+// `desc_on_host`: desc is host memory (at most kInlineDesc of them).
 int launch_draft_sample(const void *logits, int dtype, int V, const SampleRow *desc, int n_rows, int regular_rows,
-                        u32 regular_serial, u64 seed, int32_t *out, cudaStream_t s);
+                        u32 regular_serial, u64 seed, int32_t *out, cudaStream_t s, bool desc_on_host = false, HostMirror mirror = HostMirror());
 
 // coin24 != kNoCoin: the ablation of Appendix "Examining the assumptions": every accept test becomes a biased
 // coin, accepted iff the test's own 24-bit uniform is below coin24 (= acceptance probability x 2^24).
@@ -39,6 +51,6 @@ constexpr u32 kNoCoin = 0xFFFFFFFFu;
 int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int V, int batch, int t_max,
                   const VerifySeq *desc, int regular_t, u32 regular_serial, u32 regular_level, void *scratch,
                   u64 seed, int32_t *out_tokens, int32_t *out_n, int write_in_place, cudaStream_t s,
-                  u32 coin24 = kNoCoin);
+                  u32 coin24 = kNoCoin, bool desc_on_host = false, HostMirror mirror = HostMirror());
 
 }  // namespace hsd
