@@ -407,15 +407,14 @@ __global__ void __launch_bounds__(32 * (GROUPS * WARPS + 1), 1) row_stats_kernel
   }
 }
 
-// ------------------------------------------------------------------------------ one cluster per sequence
-// Algorithm 2's decision on at most one draft, or level 0's draw (no drafts: the rule's final draw from the one row), for few
-// sequences: a cluster of C CTAs takes a sequence's 2 t + 1 rows, each CTA the same V / C consecutive tokens of every row.  Bound by
-// latency, not by bytes (three rows of 32000 bf16 tokens are 0.2 MB): the rows are read once into shared memory, the row
-// maxima and then the integer totals cross the cluster in one exchange each, every CTA takes the accept tests by itself,
-// and a rejection costs one more exchange for the residual's totals.  No scratch in global memory, nothing to clear.
+// ------------------------------------------------------------------------------ clusters
+// Draws, the statistics of few rows and all decisions: a cluster of C CTAs takes a row (a decision: a row of each side), each CTA
+// the same V / C consecutive tokens.  Bound by latency, not by bytes (a row of 32000 bf16 tokens is 64 KB): a CTA's tokens are
+// read once into registers, the maximum and then the integer total cross the cluster in one exchange each.  No scratch in
+// global memory, nothing to clear.
 // A warp owns consecutive tokens; lane and unit index are interleaved (unit = 4 bytes: a bf16 pair or an fp32 value;
 // 2 bytes when rows of odd length leave bf16 pairs unaligned), so loads are whole lines whatever the row's alignment.
-constexpr int kClThreads = 512, kClWarps = kClThreads / 32, kClMaxRows = 3, kClMaxC = 8;
+constexpr int kClThreads = 512, kClWarps = kClThreads / 32, kClMaxC = 8;
 
 template <typename T, int PER> struct ClUnit;              // PER tokens of one load
 template <> struct ClUnit<float, 1> {
@@ -517,232 +516,135 @@ __device__ __forceinline__ void cl_find_token(const W (&w)[NT], u64 tau, u64 bef
   }
 }
 
-// Shared memory (dynamic): raw units [rows][NU][threads] | wmax int [rows][warps] | wsum u64 [rows + 1][warps]
-// DRAW: one row, 32-bit weights, two CTAs per SM.
-template <bool DRAW> struct ClWeight { typedef u64 type; };
-template <> struct ClWeight<true> { typedef u32 type; };
-template <typename T, int PER, int NT, bool DRAW>
-__global__ void __launch_bounds__(kClThreads, DRAW ? 2 : 1) cluster_sample_kernel(const __grid_constant__ ClusterArgs a) {
-  typedef typename ClUnit<T, PER>::raw raw_t;
-  constexpr int NU = NT / PER;                                     // units per thread and row
-  extern __shared__ __align__(16) unsigned char cl_smem[];
-  __shared__ int cmax[kClMaxRows][kClMaxC];                        // row maxima of every CTA of the cluster (order keys)
-  __shared__ u64 csum[kClMaxRows + 1][kClMaxC];                    // row totals; the last entry: the residual
-  __shared__ float row_m[kClMaxRows];
-  __shared__ u64 row_S[kClMaxRows];
-  __shared__ int sh_n;
+// The units of a CTA's part of a row, -inf past its tokens (no weight, never the maximum); their maximum over the cluster; and the
+// sum of a u64 a thread over the cluster, in every CTA (ALL) or in the first, whose parts csum holds.
+template <typename T, int PER, int NU>
+__device__ __forceinline__ void cl_units(const T *row, int k_lane, int tok_end, typename ClUnit<T, PER>::raw (&v)[NU]) {
+#pragma unroll
+  for (int u = 0; u < NU; ++u) {
+    const int k = k_lane + 32 * PER * u;
+    v[u] = k < tok_end ? __ldg(reinterpret_cast<const typename ClUnit<T, PER>::raw *>(row + k)) : ClUnit<T, PER>::none();
+  }
+}
+template <int N> __device__ __forceinline__ float cl_max(const float (&f)[N], int *wmax /*[kClWarps]*/, int *cmax /*[kClMaxC]*/, u32 rank, u32 C) {
+  float m = -INFINITY;
+#pragma unroll
+  for (int e = 0; e < N; ++e) m = fmaxf(m, f[e]);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, key = __reduce_max_sync(0xFFFFFFFFu, order_key(m));
+  if (lane == 0) wmax[warp] = key;
+  __syncthreads();
+  cl_wait();                                                       // every CTA of the cluster has started
+  if (warp == 0) {
+    const int all = __reduce_max_sync(0xFFFFFFFFu, wmax[lane & (kClWarps - 1)]);
+    if (lane < (int)C) cl_store(cl_map(&cmax[rank], (u32)lane), (u32)all);
+  }
+  cl_sync();
+  int top = cmax[0];
+  for (u32 c = 1; c < C; ++c) top = max(top, cmax[c]);
+  return order_value(top);
+}
+template <bool ALL> __device__ __forceinline__ void cl_total(u64 local, u64 *wsum /*[kClWarps]*/, u64 *csum /*[kClMaxC]*/, u32 rank, u32 C) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u64 s = warp_sum54(local);
+  if (lane == 0) wsum[warp] = s;
+  __syncthreads();
+  if (warp == 0) {
+    u64 t = lane < kClWarps ? wsum[lane] : 0ull;
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+    if (lane < (ALL ? (int)C : 1)) cl_store(cl_map(&csum[rank], (u32)lane), t);
+  }
+  cl_sync();
+}
+
+// Level 0's draw: token = inverse-CDF sample of softmax(row) with the purpose-0 uniform.  Two CTAs per SM.
+template <typename T, int PER, int NT>
+__global__ void __launch_bounds__(kClThreads, 2) cluster_draw_kernel(const __grid_constant__ ClusterArgs a) {
+  constexpr int NU = NT / PER;
+  __shared__ int wmax[kClWarps], cmax[kClMaxC];                    // order keys
+  __shared__ u64 wsum[kClWarps], csum[kClMaxC];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const u32 rank = cl_rank(), C = cl_size();
   const int b = (int)cl_id();
   cl_arrive();                                                     // (the wait is in front of the first store to a peer)
   chain_wait();
   chain_next();
-  VerifySeq d;
-  long long out_index = 0;
-  u32 uj = 0;
-  if (DRAW) {
-    SampleRow s;
-    if (a.rows.given()) s = a.rows.at(b);
-    else { s.logit_row = b; s.out_index = b; s.j = b % a.regular_t; s.seq = b / a.regular_t; s.serial = a.regular_serial; s.level = 0; }
-    d.p_row0 = s.logit_row; d.q_row0 = 0; d.tok_off = 0; d.t = 0; d.serial = s.serial; d.seq = s.seq; d.level = s.level;
-    out_index = s.out_index; uj = s.j;
-  } else if (a.desc.given()) d = a.desc.at(b);
-  else {
-    d.t = a.regular_t; d.p_row0 = (long long)b * (a.regular_t + 1); d.q_row0 = (long long)b * a.regular_t;
-    d.tok_off = (long long)b * a.regular_t; d.serial = a.regular_serial; d.seq = b; d.level = a.regular_level;
-  }
-  const int t = DRAW ? 0 : d.t, n_rows = 2 * t + 1;                           // rows 0..t: p; t + 1 + j: q_j
-  raw_t *stage = reinterpret_cast<raw_t *>(cl_smem);
-  const size_t max_rows = 2 * (size_t)a.t_max + 1;
-  u64 *wsum = reinterpret_cast<u64 *>(cl_smem + max_rows * NU * kClThreads * sizeof(raw_t));   // [rows + 1][warps]
-  int *wmax = reinterpret_cast<int *>(wsum + (max_rows + 1) * kClWarps);
-  auto row_ptr = [&](int r) {
-    return r <= t ? reinterpret_cast<const T *>(a.p) + (size_t)(d.p_row0 + r) * a.V
-                  : reinterpret_cast<const T *>(a.q) + (size_t)(d.q_row0 + r - t - 1) * a.V;
-  };
+  SampleRow d;
+  if (a.rows.given()) d = a.rows.at(b);
+  else { d.logit_row = b; d.out_index = b; d.j = b % a.regular_t; d.seq = b / a.regular_t; d.serial = a.regular_serial; d.level = 0; }
   const int tok0 = (int)rank * a.seg, tok_end = min(a.V, tok0 + a.seg);
   const int k_lane = tok0 + warp * (32 * NT) + lane * PER;         // first token of unit i: k_lane + 32 PER i
-  // the drafted tokens' logits (every CTA takes the accept tests for itself)
-  float lp = 0.f, lq = 0.f;
-  int tok = -1;
-  if (tid < t) {
-    tok = a.tokens[d.tok_off + tid];
-    if (tok >= 0 && tok < a.V) { lp = to_f32(row_ptr(tid)[tok]); lq = to_f32(row_ptr(t + 1 + tid)[tok]); }
+  typename ClUnit<T, PER>::raw v[NU];
+  cl_units<T, PER, NU>(reinterpret_cast<const T *>(a.p) + (size_t)d.logit_row * a.V, k_lane, tok_end, v);
+  float f[NT];
+#pragma unroll
+  for (int u = 0; u < NU; ++u) ClUnit<T, PER>::get(v[u], f + u * PER);
+  const float m = cl_max(f, wmax, cmax, rank, C);
+  u32 w[NT];
+  u64 local = 0, total = 0, before = 0;
+#pragma unroll
+  for (int e = 0; e < NT; e += 2) {
+    exp_weight2(f[e], f[e + 1], m, w[e], w[e + 1]);
+    local += (u64)w[e] + (u64)w[e + 1];
   }
-  auto unit_of = [&](int r, int i) -> raw_t {                      // a unit of this thread, once more
-    return stage[((size_t)r * NU + i) * kClThreads + tid];
-  };
-  // weights of a row's units against the row maximum, two tokens j, j + 1 at a time (0 past the CTA's tokens)
-  auto weights_of = [&](const raw_t *v, float m, auto &&take) {
-    float f[NT];
-#pragma unroll
-    for (int i = 0; i < NU; ++i) ClUnit<T, PER>::get(v[i], f + i * PER);
-#pragma unroll
-    for (int j = 0; j < NT; j += 2) {
-      u32 e0, e1;
-      exp_weight2(f[j], f[j + 1], m, e0, e1);
-      take(j, k_lane + 32 * PER * (j / PER) < tok_end ? e0 : 0u, k_lane + 32 * PER * ((j + 1) / PER) < tok_end ? e1 : 0u);
-    }
-  };
-  // ---- rows into shared memory (own slots: no barrier between the write and the later reads) and the row maxima
-  constexpr int RB = NU <= 4 ? 8 : (NU <= 8 ? 4 : (NU <= 16 ? 2 : 1));   // rows fetched at a time
-  for (int r0 = 0; r0 < n_rows; r0 += RB) {
-    raw_t v[RB][NU];
-#pragma unroll
-    for (int rr = 0; rr < RB; ++rr) {
-      const T *row = row_ptr(min(r0 + rr, n_rows - 1));
-#pragma unroll
-      for (int i = 0; i < NU; ++i) {
-        const int k = k_lane + 32 * PER * i;
-        v[rr][i] = k < tok_end ? __ldg(reinterpret_cast<const raw_t *>(row + k)) : raw_t(0);
-      }
-    }
-#pragma unroll
-    for (int rr = 0; rr < RB; ++rr) {
-      if (r0 + rr >= n_rows) break;
-      float m = -INFINITY;
-#pragma unroll
-      for (int i = 0; i < NU; ++i) {
-        const int k = k_lane + 32 * PER * i;
-        float f[PER];
-        ClUnit<T, PER>::get(v[rr][i], f);
-        if (k < tok_end) {                                         // (PER = 2: V is even)
-#pragma unroll
-          for (int e = 0; e < PER; ++e) m = fmaxf(m, f[e]);
-        }
-        stage[((size_t)(r0 + rr) * NU + i) * kClThreads + tid] = v[rr][i];
-      }
-      const int key = __reduce_max_sync(0xFFFFFFFFu, order_key(m));
-      if (lane == 0) wmax[(r0 + rr) * kClWarps + warp] = key;
-    }
+  cl_total<true>(local, wsum, csum, rank, C);
+  for (u32 c = 0; c < C; ++c) {
+    if (c < rank) before += csum[c];
+    total += csum[c];
   }
-  __syncthreads();
-  cl_wait();                                                       // every CTA of the cluster has started
-  for (int r = warp; r < n_rows; r += kClWarps) {
-    const int key = __reduce_max_sync(0xFFFFFFFFu, wmax[r * kClWarps + (lane & (kClWarps - 1))]);
-    if (lane < (int)C) cl_store(cl_map(&cmax[r][rank], (u32)lane), (u32)key);
-  }
-  cl_sync();
-  if (tid < n_rows) {
-    int key = cmax[tid][0];
-    for (u32 c = 1; c < C; ++c) key = max(key, cmax[tid][c]);
-    row_m[tid] = order_value(key);
-  }
-  __syncthreads();
-  // ---- integer totals
-  for (int r0 = 0; r0 < n_rows; r0 += RB) {
-    raw_t v[RB][NU];
-#pragma unroll
-    for (int rr = 0; rr < RB; ++rr)
-#pragma unroll
-      for (int i = 0; i < NU; ++i) v[rr][i] = unit_of(min(r0 + rr, n_rows - 1), i);
-#pragma unroll
-    for (int rr = 0; rr < RB; ++rr) {
-      if (r0 + rr >= n_rows) break;
-      const float m = row_m[r0 + rr];
-      u64 local = 0;
-      weights_of(v[rr], m, [&](int, u32 e0, u32 e1) { local += (u64)e0 + (u64)e1; });
-      const u64 s = warp_sum54(local);
-      if (lane == 0) wsum[(r0 + rr) * kClWarps + warp] = s;
-    }
-  }
-  __syncthreads();
-  auto publish = [&](int r) {                                      // a warp: total of wsum row r -> every CTA's csum
-    u64 s = lane < kClWarps ? wsum[r * kClWarps + lane] : 0ull;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-    if (lane < (int)C) cl_store(cl_map(&csum[r][rank], (u32)lane), s);
-  };
-  for (int r = warp; r < n_rows; r += kClWarps) publish(r);
-  cl_sync();
-  if (tid < n_rows) {
-    u64 S = 0;
-    for (u32 c = 0; c < C; ++c) S += csum[tid][c];
-    row_S[tid] = S;
-  }
-  __syncthreads();
-  // ---- accept tests (t <= 31: one warp), n = first rejection
-  if (!DRAW && warp == 0) {
-    bool ok = true;
-    if (lane < t) {
-      const u32 ep = (tok >= 0 && tok < a.V) ? exp_weight(lp, row_m[lane]) : 0u, eq = (tok >= 0 && tok < a.V) ? exp_weight(lq, row_m[t + 1 + lane]) : 0u;
-      const u64 Pp = fixed_prob(ep, prob_scale(row_S[lane])), Pq = fixed_prob(eq, prob_scale(row_S[t + 1 + lane]));
-      const u32 U = uniform24(a.seed, lane, d.serial, d.level, PURPOSE_ACCEPT, d.seq);
-      ok = (((u64)U * Pq) >> 24) < Pp;                             // u < p(x) / q(x)
-      if (a.coin24 != kNoCoin) ok = U < a.coin24;                  // ablation: IID acceptance with a fixed probability
-    }
-    const unsigned rejected = __ballot_sync(0xFFFFFFFFu, !ok);
-    if (lane == 0) sh_n = rejected ? __ffs(rejected) - 1 : t;
-  }
-  if (!DRAW) __syncthreads();
-  const int n = DRAW ? 0 : sh_n;
-  // ---- the final draw's weights: the residual of row n, or row t itself
-  typename ClWeight<DRAW>::type w[NT];
-  int src = n;                                                     // row of wsum / csum that holds the totals of w
-  u64 total = row_S[n];
-  const float mp = row_m[n];
-  auto row_weights = [&]() {
-    raw_t v[NU];
-#pragma unroll
-    for (int i = 0; i < NU; ++i) v[i] = unit_of(n, i);
-    weights_of(v, mp, [&](int j, u32 e0, u32 e1) { w[j] = e0; w[j + 1] = e1; });
-  };
-  if (!DRAW && n < t) {
-    const float mq = row_m[t + 1 + n];
-    const ProbScale psp = prob_scale(row_S[n]), psq = prob_scale(row_S[t + 1 + n]);
-    u64 local = 0;
-#pragma unroll
-    for (int i = 0; i < NU; ++i) {
-      const int k = k_lane + 32 * PER * i;
-      float fp[PER], fq[PER];
-      ClUnit<T, PER>::get(unit_of(n, i), fp);
-      ClUnit<T, PER>::get(unit_of(t + 1 + n, i), fq);
-#pragma unroll
-      for (int e = 0; e < PER; ++e) {
-        u32 ep, eq;
-        exp_weight2m(fp[e], fq[e], mp, mq, ep, eq);
-        const u64 Pp = fixed_prob(ep, psp), Pq = fixed_prob(eq, psq);
-        w[i * PER + e] = (k < tok_end && Pp > Pq) ? Pp - Pq : 0ull;
-        local += w[i * PER + e];
-      }
-    }
-    const u64 s = warp_sum54(local);
-    if (lane == 0) wsum[n_rows * kClWarps + warp] = s;
-    __syncthreads();
-    if (warp == 0) publish(n_rows);
-    cl_sync();
-    total = 0;
-    for (u32 c = 0; c < C; ++c) total += csum[n_rows][c];
-    if (total != 0) src = n_rows;
-    else total = row_S[n];                                         // an all-zero residual: draw from the verifier's own row
-  }
-  if (DRAW || src == n) row_weights();
-  // ---- inverse CDF: the CTA, then the warp, then the unit, then the token whose inclusive sum passes the threshold
-  const u32 U = uniform24(a.seed, uj, d.serial, d.level, DRAW ? PURPOSE_DRAFT : PURPOSE_FINAL, d.seq);
-  const u64 tau = cdf_threshold(U, total);
-  u64 before = 0;
-  for (u32 c = 0; c < rank; ++c) before += csum[src][c];
+  const u64 tau = cdf_threshold(uniform24(a.seed, d.j, d.serial, d.level, PURPOSE_DRAFT, d.seq), total);
   auto emit = [&](int k) {
-    if (DRAW) {
-      a.out_tokens[out_index] = k;
-      if (a.mirror.token) a.mirror.token[(size_t)d.seq * a.mirror.stride + uj] = k;
-    } else {
-      if (a.write_in_place) a.tokens[d.tok_off + n] = k;
-      if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = k;
-      if (a.mirror.n) a.mirror.token[b] = k;
-    }
+    a.out_tokens[d.out_index] = k;
+    if (a.mirror.token) a.mirror.token[(size_t)d.seq * a.mirror.stride + d.j] = k;
   };
   if (total == 0) {                                                // non-finite logits: no token
     if (rank == 0 && tid == 0) emit(-1);
-  } else if (tau >= before && tau < before + csum[src][rank]) {
-    cl_find_token<NT, PER>(w, tau, before, wsum + src * kClWarps, k_lane, emit);
+  } else if (tau >= before && tau < before + csum[rank]) {
+    cl_find_token<NT, PER>(w, tau, before, wsum, k_lane, emit);
   }
-  if (!DRAW && rank == 0) {
-    if (tid == 0) {
-      a.out_n[b] = n;
-      if (a.mirror.n) a.mirror.n[b] = n;
-      if (a.mirror.status && b == 0) *a.mirror.status = __ldcg(a.mirror.status_src);
-    }
-    if (a.out_tokens && tid <= a.t_max && tid != n) a.out_tokens[(size_t)b * (a.t_max + 1) + tid] = tid < n ? tok : -1;
+}
+
+// The statistics of few rows: a cluster a row, each CTA consecutive tokens of it in registers; the maximum and the total cross the
+// cluster in one exchange each.  7 rows of 32000 bf16 tokens: 3.3 us (a CTA a row that takes them through its ring: 5.8).
+template <typename T, int PER, int NT>
+__global__ void __launch_bounds__(kClThreads, 2) cluster_stats_kernel(const __grid_constant__ RowStatArgs a, int seg) {
+  constexpr int NU = NT / PER;
+  __shared__ int wmax[kClWarps], cmax[kClMaxC];                    // order keys
+  __shared__ u64 wsum[kClWarps], csum[kClMaxC];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const u32 rank = cl_rank(), C = cl_size();
+  cl_arrive();                                                     // (the wait is in front of the first store to a peer)
+  chain_wait();
+  chain_next();
+  const int rows_per_seq = 2 * a.t_max + 1, i = (int)cl_id(), b = i / rows_per_seq, r = i - b * rows_per_seq;
+  const bool is_p = r <= a.t_max;
+  const int at = is_p ? r : r - a.t_max - 1;
+  long long row0 = (long long)b * (a.regular_t + (is_p ? 1 : 0));
+  if (a.desc.given()) {
+    const VerifySeq d = a.desc.at(b);
+    if (at >= d.t + (is_p ? 1 : 0)) return;                        // the whole cluster
+    row0 = is_p ? d.p_row0 : d.q_row0;
+  }
+  const T *row = reinterpret_cast<const T *>(is_p ? a.p : a.q) + (size_t)(row0 + at) * a.V;
+  const int tok0 = (int)rank * seg, tok_end = min(a.V, tok0 + seg), k_lane = tok0 + warp * (32 * NT) + lane * PER;
+  typename ClUnit<T, PER>::raw v[NU];
+  cl_units<T, PER, NU>(row, k_lane, tok_end, v);
+  float f[NT];
+#pragma unroll
+  for (int u = 0; u < NU; ++u) ClUnit<T, PER>::get(v[u], f + u * PER);
+  const float m = cl_max(f, wmax, cmax, rank, C);
+  u64 local = 0;
+#pragma unroll
+  for (int e = 0; e < NT; e += 2) {
+    u32 e0, e1;
+    exp_weight2(f[e], f[e + 1], m, e0, e1);
+    local += (u64)e0 + (u64)e1;
+  }
+  cl_total<false>(local, wsum, csum, rank, C);
+  if (rank == 0 && tid == 0) {
+    RowStat st;
+    st.m = m; st.S = 0;
+    for (u32 c = 0; c < C; ++c) st.S += csum[c];
+    a.stats[i] = st;
   }
 }
 
@@ -890,68 +792,51 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
   }
 }
 
-// Cluster size, tokens per thread and shared memory of a call with n sequences of at most `rows` rows; false if the rows
-// are too long or too many for this path.
-struct ClusterPlan { int C, NT, per, seg; size_t smem; };
-constexpr size_t kClMaxSmem = 216 * 1024;
+// Cluster size, tokens a thread and tokens a CTA of a call with n clusters; false if the rows are too long.  `two`: two CTAs per SM.
+struct ClusterPlan { int C, NT, per, seg; };
 constexpr int kClEights = 14;                     // clusters of eight that run at once (one CTA per SM)
-static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, int rows, bool draw, ClusterPlan *pl) {
+static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, bool two, ClusterPlan *pl) {
   pl->per = (dtype == HSD_BF16 && V % 2 == 0 && ((uintptr_t)p & 3) == 0 && ((uintptr_t)q & 3) == 0) ? 2 : 1;
-  // as many CTAs as run at once (draws: two per SM), of at least 4096 tokens (eight a thread) each: clusters of eight do not fit all SMs
+  // as many CTAs as run at once, of at least 4096 tokens (eight a thread) each: clusters of eight do not fit all SMs
   // (16 of them took two rounds), clusters of four and two do
   int C = 1;
-  while (C < kClMaxC && V > C * 4096 && 2 * C * n <= (C == 4 ? 8 * kClEights : draw ? 2 * kMeasuredSMs : kMeasuredSMs)) C *= 2;
-  const int most = (draw ? 16 : 32) * kClThreads;
+  while (C < kClMaxC && V > C * 4096 && 2ll * C * n <= (C == 4 ? 8 * kClEights : two ? 2 * kMeasuredSMs : kMeasuredSMs)) C *= 2;
+  const int most = (two ? 16 : 32) * kClThreads;
   while (C < kClMaxC && ceil_div(V, C) > most - 64) C *= 2;
   const int seg = ceil_div(ceil_div(V, C), 64) * 64;
   if (seg > most) return false;
   pl->C = C;
   pl->seg = seg;
   pl->NT = seg <= 8 * kClThreads ? 8 : seg <= 16 * kClThreads ? 16 : 32;
-  const size_t extra = (size_t)(rows + 1) * kClWarps * 8 + (size_t)rows * kClWarps * 4;
-  const size_t stage = (size_t)rows * pl->NT * kClThreads * (dtype == HSD_BF16 ? 2 : 4);
-  pl->smem = extra + stage;
   return true;
 }
-// Where the one-launch cluster path is the faster one (us a call in a captured sequence of calls, cluster / other path).
-//   verification: three rows of a long vocabulary a sequence, clusters of four or eight.  t = 1, bf16: V = 32000, 1 sequence 9.3 / 9.9,
-//     4: 10.5 / 10.9, 32 (clusters of four): 12.7 / 12.6, 64 (of two): 19.4 / 18.9; V = 8192, 1: 9.3 / 7.5; V = 49999, 1: 15.2 / 15.5; fp32:
-//     V = 32000, 1: 9.6 / 11.6, V = 8192, 1: 9.6 / 7.8.  More rows cost a CTA 0.9 us each, and the statistics kernel has an SM
-//     for each: t = 3, 1 sequence bf16 11.9 / 10.5, fp32 13.7 / 12.3; t = 8, 8 sequences bf16 19 / 10.6.
+// Where clusters are the faster ones (us a call in a row of calls, clusters / other path).
+//   statistics (the whole verification), while the clusters run in one round: 32000 bf16, 7 rows 8.4 / 10.8, 66 rows 10.1 / 11.5, 88 rows (in
+//     two rounds) 12.9 / 11.5; fp32, 7 rows 9.2 / 12.9, 66: 11.1 / 13.3, 88: 13.8 / 13.5; 16000 bf16, 132 rows 10.1 / 10.0, 176 (two) 11.9 / 11.6; 2048:
+//     8.0 / 8.0, 176 rows 8.8 / 8.7; 45001 bf16, 33 rows 13.5 / 16.1, 44 (two) 16.4 / 16.2.
 //   draws (two CTAs per SM, 16 tokens a thread at most), other path a CTA of 1024 threads a row, which has 32 tokens a thread where bf16 rows
-//     allow (`chunked`): while the clusters run in one round, bf16 32000: 1 row 4.0 / 10.2, 64 rows 6.4 / 11.0; 2048: 4.0 / 8.5 to 9.4;
-//     fp32 32000: 4.5 / 26, 64 rows 7.9 / 28; 8000: 4.4 / 6.1; 2048: 4.0 / 3.9.  In more rounds, chunked: 32000, 100 rows 10.5 / 11.1, 148: 13.8 / 11.1
-//     (a row a CTA then), 200: 16.3 / 20.5, 512: 40 / 40, 16000, 512: 20 / 35; others: fp32 11000, 256: 13.8 / 9.9, 24001, 148: 16.7 / 12.9,
-//     32000, 100: 12.5 / 28, 512: 50 / 105; 8000, 512: 13.1 / 15.9; bf16 9001, 256: 14.0 / 12.2, 32001: 26 / 38.
-static bool cluster_pays_verify(const ClusterPlan &pl, int V, int batch) {
-  return V > 24000 && pl.NT <= 16 && pl.C >= 4 && pl.C * batch <= kMeasuredSMs;
-}
+//     allow (`chunked`): while the clusters run in one round, bf16 32000: 1 row 4.0 / 10.2, 64 rows 5.8 / 11.0; 2048: 3.8 / 8.5 to 9.4;
+//     fp32 32000: 4.1 / 26, 64 rows 6.6 / 28; 8000: 4.1 / 6.1; 2048: 3.9 / 3.9.  In more rounds, chunked: 32000, 100 rows 9.4 / 11.1, 148: 12.5 / 11.1
+//     (a row a CTA then), 200: 14.6 / 20.5, 512: 37 / 40, 16000, 512: 18 / 35; others: fp32 9001, 256: 12 / 9.1, 16000, 256: 11 / 16.9 (two CTAs a row),
+//     20000, 148: 13.4 / 10.7, 32000, 100: 10.2 / 28, 512: 41 / 105; 8000, 512: 10.7 / 15.9; bf16 32001, 256: 21 / 38.
+static bool cluster_pays_stats(const ClusterPlan &pl, long long rows) { return pl.C * rows <= 2 * kMeasuredSMs; }
 static bool cluster_pays_draw(const ClusterPlan &pl, int V, int n, bool chunked) {
   if (pl.C * n <= 2 * kMeasuredSMs) return true;
   if (chunked) return n > kMeasuredSMs || pl.C * n <= 3 * kMeasuredSMs;
-  return V > 26000 || V <= 8192;
+  return V > 26000 || V <= 8192 || (V > 13500 && pl.C == 2);
 }
 
-template <typename T, int PER, int NT, bool DRAW>
-static int launch_cluster_t(const ClusterArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
-  static std::atomic<u64> limits{0};
-  const int limit = hsd_smem_limit((const void *)cluster_sample_kernel<T, PER, NT, DRAW>, (int)(DRAW ? kClMaxSmem / 2 : kClMaxSmem), limits);
-  if (limit) return limit;
-  HSD_CUDA_OK(hsd_launch(cluster_sample_kernel<T, PER, NT, DRAW>, n * pl.C, kClThreads, pl.smem, s, pl.C, true, a));
+template <typename T, int PER>
+static int launch_cluster_draw_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
+  if (pl.NT == 8) HSD_CUDA_OK(hsd_launch(cluster_draw_kernel<T, PER, 8>, n * pl.C, kClThreads, 0, s, pl.C, true, a));
+  else HSD_CUDA_OK(hsd_launch(cluster_draw_kernel<T, PER, 16>, n * pl.C, kClThreads, 0, s, pl.C, true, a));
   hsd_count_launches(1);
   return hsd_launch_status();
 }
-template <typename T, int PER, bool DRAW>
-static int launch_cluster_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
-  if (pl.NT == 8) return launch_cluster_t<T, PER, 8, DRAW>(a, pl, n, s);
-  if (pl.NT == 16) return launch_cluster_t<T, PER, 16, DRAW>(a, pl, n, s);
-  return HSD_E_UNSUPPORTED;
-}
-template <bool DRAW>
-static int launch_cluster(ClusterArgs a, const ClusterPlan &pl, int dtype, int n, cudaStream_t s) {
+static int launch_cluster_draw(ClusterArgs a, const ClusterPlan &pl, int dtype, int n, cudaStream_t s) {
   a.seg = pl.seg;
-  if (dtype == HSD_F32) return launch_cluster_nt<float, 1, DRAW>(a, pl, n, s);
-  return pl.per == 2 ? launch_cluster_nt<__nv_bfloat16, 2, DRAW>(a, pl, n, s) : launch_cluster_nt<__nv_bfloat16, 1, DRAW>(a, pl, n, s);
+  if (dtype == HSD_F32) return launch_cluster_draw_nt<float, 1>(a, pl, n, s);
+  return pl.per == 2 ? launch_cluster_draw_nt<__nv_bfloat16, 2>(a, pl, n, s) : launch_cluster_draw_nt<__nv_bfloat16, 1>(a, pl, n, s);
 }
 
 // ------------------------------------------------------------------------------ host launchers
@@ -976,12 +861,12 @@ int launch_draft_sample(const void *logits, int dtype, int V, const SampleRow *d
   if (desc_on_host && n_rows > kInlineDesc) return HSD_E_INVALID_ARG;
   const DescList<SampleRow> list = desc_list(desc, n_rows, desc_on_host);
   ClusterPlan pl;
-  if (cluster_plan(logits, nullptr, dtype, V, n_rows, 1, true, &pl) &&
+  if (cluster_plan(logits, nullptr, dtype, V, n_rows, true, &pl) &&
       cluster_pays_draw(pl, V, n_rows, dtype == HSD_BF16 && V % 8 == 0 && V <= kSampleThreads * kChunkTokens && ((uintptr_t)logits & 15) == 0)) {
     ClusterArgs a = {};
     a.p = logits; a.V = V; a.t_max = 0; a.rows = list; a.mirror = mirror; a.regular_t = regular_rows;
     a.regular_serial = regular_serial; a.seed = seed; a.out_tokens = out; a.coin24 = kNoCoin;
-    return launch_cluster<true>(a, pl, dtype, n_rows, s);
+    return launch_cluster_draw(a, pl, dtype, n_rows, s);
   }
   return dtype == HSD_BF16
              ? launch_draft_sample_t<__nv_bfloat16>(logits, V, list, n_rows, regular_rows, regular_serial, seed, out, s, mirror)
@@ -1011,8 +896,20 @@ static int launch_row_stats_t(const RowStatArgs &a, int grid, cudaStream_t s) {
 // us a call, GROUPS x WARPS = 1 x 16 / 2 x 8 / 3 x 8 (chunks of 32 KB; 2 x 12 on chunks of 24 KB lies behind 2 x 8):
 //   a row a CTA, 32000: bf16 5.6 / 5.9 / 6.2, fp32 6.9 / 7.4 / 7.7
 //   1088 rows of 32000: bf16 29.7 / 25.3 / 24.6, fp32 35.3 / 32.3 / 32.5; of 2048: bf16 9.6 / 7.0 / 6.9; of 50000, fp32: 57.4 / 57.7 / 58.2
+template <typename T, int PER>
+static int launch_cluster_stats(const RowStatArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
+  if (pl.NT == 8) HSD_CUDA_OK(hsd_launch(cluster_stats_kernel<T, PER, 8>, n * pl.C, kClThreads, 0, s, pl.C, true, a, pl.seg));
+  else HSD_CUDA_OK(hsd_launch(cluster_stats_kernel<T, PER, 16>, n * pl.C, kClThreads, 0, s, pl.C, true, a, pl.seg));
+  hsd_count_launches(1);
+  return HSD_OK;
+}
 static int launch_row_stats(const RowStatArgs &a, int dtype, cudaStream_t s) {
   const long long n_items = (long long)a.batch * (2 * a.t_max + 1);
+  ClusterPlan pl;
+  if (n_items <= 2 * kMeasuredSMs && cluster_plan(a.p, a.q, dtype, a.V, (int)n_items, true, &pl) && cluster_pays_stats(pl, n_items)) {
+    if (dtype == HSD_F32) return launch_cluster_stats<float, 1>(a, pl, (int)n_items, s);
+    return pl.per == 2 ? launch_cluster_stats<__nv_bfloat16, 2>(a, pl, (int)n_items, s) : launch_cluster_stats<__nv_bfloat16, 1>(a, pl, (int)n_items, s);
+  }
   const int grid = (int)std::min<long long>(sm_count(), n_items);
   if (n_items <= grid)                                     // a row a CTA: all its warps on it
     return dtype == HSD_F32 ? launch_row_stats_t<float, 1, 16, 32768>(a, grid, s) : launch_row_stats_t<__nv_bfloat16, 1, 16, 32768>(a, grid, s);
@@ -1042,13 +939,11 @@ int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int 
   a.regular_serial = regular_serial; a.regular_level = regular_level; a.seed = seed; a.out_tokens = out_tokens; a.out_n = out_n;
   a.write_in_place = write_in_place; a.coin24 = coin24;
   ClusterPlan pl;
-  if (2 * t_max + 1 <= kClMaxRows && cluster_plan(p, q, dtype, V, batch, 2 * t_max + 1, false, &pl) && cluster_pays_verify(pl, V, batch))
-    return launch_cluster<false>(a, pl, dtype, batch, s);
   RowStatArgs r = {};
   r.p = p; r.q = q; r.V = V; r.t_max = t_max; r.batch = batch; r.regular_t = regular_t; r.desc = list; r.stats = stats;
   const int st = launch_row_stats(r, dtype, s);
   if (st) return st;
-  if (cluster_plan(p, q, dtype, V, batch, 1, false, &pl)) {     // a decision reads one row of each side
+  if (cluster_plan(p, q, dtype, V, batch, false, &pl)) {
     a.seg = pl.seg;
     if (dtype == HSD_F32) return launch_decide_nt<float, 1>(a, pl, batch, stats, s);
     return pl.per == 2 ? launch_decide_nt<__nv_bfloat16, 2>(a, pl, batch, stats, s) : launch_decide_nt<__nv_bfloat16, 1>(a, pl, batch, stats, s);
