@@ -167,3 +167,18 @@ def test_pairwise_alpha_of_extreme_logits(lib, V, dtype):
     p = torch.softmax(z - z.max(-1, keepdim=True).values, -1)
     want = torch.stack([torch.minimum(p[i:i + 1], p).sum(-1).mean(-1) for i in range(4)])
     assert torch.equal(got, got.T) and (got - want).abs().max() < 1e-5, (got, want)
+
+
+@pytest.mark.parametrize("dtype,L,R,V", [(torch.bfloat16, 5, 20, 4001), (torch.bfloat16, 24, 30, 2048), (torch.float32, 18, 200, 8192)])
+def test_rates_of_calls_back_to_back(lib, dtype, L, R, V):
+    # the kernels of a call start under the end of the one before it, and read logits that the stream has just written
+    g = torch.Generator(device="cuda").manual_seed(L)
+    sets = [(torch.randn(L, R, V, generator=g, device="cuda") * 3).to(dtype) for _ in range(3)]
+    want = [lib.hsd_pairwise_alpha(x).clone() for x in sets]
+    x = torch.empty_like(sets[0])
+    got = []
+    for i in range(12):
+        x.copy_(sets[i % 3])
+        got.append(lib.hsd_pairwise_alpha(x))
+        lib.hsd_pairwise_alpha(sets[(i + 1) % 3])
+    assert all(torch.equal(a, want[i % 3]) for i, a in enumerate(got))
