@@ -379,7 +379,10 @@ int launch_alpha_t(const T *logits, long long model_stride, int L, int R, int V,
          : L <= 16 ? launch_pairs<T, VEC, 512>(logits, model_stride, L, R, V, p, stats, partials, s)
                    : launch_pairs<T, VEC, 256>(logits, model_stride, L, R, V, p, stats, partials, s);
   if (st) return st;
-  HSD_CUDA_OK(hsd_launch(alpha_reduce_kernel, p.n_pairs > 0 ? min(p.n_pairs, 4 * kMeasuredSMs) : 1, kAlphaThreads, 0, s, 0, true, partials, L, R * p.n_units, R,
+  // (behind more than two waves of pairs the reduction's waiting CTAs take the last wave's places: 32 models x 256 x 32000 571 us
+  // early, 568 not, 32 x 16 54.1 / 52.8; 5 x 20 x 17001, one wave and a half, 18.7 / 21.9)
+  const bool early = p.n_units * R <= 2 * (L <= 8 ? 3 : 2) * kMeasuredSMs;
+  HSD_CUDA_OK(hsd_launch(alpha_reduce_kernel, p.n_pairs > 0 ? min(p.n_pairs, 4 * kMeasuredSMs) : 1, kAlphaThreads, 0, s, 0, early, partials, L, R * p.n_units, R,
                          alpha));
   hsd_count_launches(p.n_pairs > 0 ? 3 : 2);
   return hsd_launch_status();
