@@ -449,24 +449,37 @@ int tc_make_map(CUtensorMap *map, const void *base, long long rows, long long co
 
 int tc_npad(int rows) { return rows <= 16 ? 16 : rows <= 32 ? 32 : rows <= 64 ? 64 : rows <= 128 ? 128 : 256; }
 
-// Rows of a tile of one matrix on its own: 128, or as many fewer as spread the rows evenly over the rounds the SMs need.
-int tc_tile_rows(int N, int sm_count) {
-  if (ceil_div(N, kTcBlockM) * 2 <= sm_count) return kTcBlockM;       // k-blocks are divided: full tiles
-  const int rounds = ceil_div(N, kTcBlockM * sm_count);
-  return std::min(kTcBlockM, ceil_div(ceil_div(N, rounds * sm_count), 8) * 8);
+namespace {
+// CTAs a tile's k-blocks are divided over: 2, 4 or (few tiles) 8 while full tiles alone leave half the SMs idle.  The division
+// does not depend on the number of rows, so neither does a row's result.  48 clusters of three or 16 of eight do not run at
+// once (6144 x 4096 at 128 rows: 36 us in threes, 25 us in pairs), 74 of two, 32 of four and 14 of eight do.
+int split_of(int full_tiles, int K, int sm_count) {
+  int S = 1;
+  while (S < (full_tiles <= 14 ? 8 : 4) && full_tiles * S * 2 <= sm_count && S * 2 <= K / kTcBlockK) S *= 2;
+  return S;
+}
+}  // namespace
+
+// Rows of a tile of one matrix on its own: 128, or as many fewer as spread N evenly over the rounds the SMs need or, with the
+// k-blocks divided, over the clusters that run at once (the same sums: a row's result does not change).  Of up to 32 token rows
+// full tiles are as fast (5632 x 2048: 8.0 and 8.1 us at 16) and leave SMs on which the next launch starts; of more a CTA's
+// activations and finish count: 64 / 128 / 200 rows of 5632 x 2048 11.2 / 14.6 / 19.0 -> 9.3 / 11.4 / 15.8 us, of 2048 x 5632
+// 10.2 / 12.3 / 16.9 -> 10.0 / 11.4 / 15.6, of 1024 x 4096 7.9 / 9.6 / 13.0 -> 7.5 / 9.0 / 11.7.
+int tc_tile_rows(int N, int K, int R, int sm_count) {
+  const int S = split_of(ceil_div(N, kTcBlockM), K, sm_count);
+  if (S > 1 && R <= 32) return kTcBlockM;
+  const int at_once = S == 2 ? 74 : S == 4 ? 32 : S == 8 ? 14 : sm_count, rounds = ceil_div(N, kTcBlockM * at_once);
+  return std::min(kTcBlockM, ceil_div(ceil_div(N, rounds * at_once), 8) * 8);
 }
 
 int launch_gemm_tc(const TcGemmArgs &args, int sm_count, cudaStream_t s) {
   if (args.R < 1 || args.R > 256 || args.K < kTcBlockK || args.K % kTcBlockK != 0) return HSD_E_UNSUPPORTED;
-  int n_tiles = 0;
-  if (args.mode == GEMM_SWIGLU_T) n_tiles = ceil_div(args.seg_n[0], kTcBoxRows);
-  else
-    for (int i = 0; i < args.n_segs; ++i) n_tiles += ceil_div(args.seg_n[i], args.tile_rows);
-  // k-blocks divided over 2, 4 or (few tiles) 8 CTAs while the tiles alone leave half the SMs idle; the division does not
-  // depend on the number of rows, so neither does a row's result.  48 clusters of three or 16 of eight do not run at
-  // once (6144 x 4096 at 128 rows: 36 us in threes, 25 us in pairs), 74 of two and 32 of four do.
-  int S = 1;
-  while (S < (n_tiles <= 14 ? 8 : 4) && n_tiles * S * 2 <= sm_count && S * 2 <= args.K / kTcBlockK) S *= 2;
+  int n_tiles = 0, full_tiles = 0;
+  for (int i = 0; i < (args.mode == GEMM_SWIGLU_T ? 1 : args.n_segs); ++i) {
+    n_tiles += ceil_div(args.seg_n[i], args.mode == GEMM_SWIGLU_T ? kTcBoxRows : args.tile_rows);
+    full_tiles += ceil_div(args.seg_n[i], args.mode == GEMM_SWIGLU_T ? kTcBoxRows : kTcBlockM);
+  }
+  const int S = split_of(full_tiles, args.K, sm_count);
   const int grid = S > 1 ? n_tiles * S : std::min(n_tiles, sm_count);
   switch (tc_npad(args.R)) {
     case 16: return launch_mode<16>(args, n_tiles, S, grid, s);

@@ -46,7 +46,7 @@ struct TcGemmArgs {
   int ldo;
   int *status;                     // device word: set non-zero if a bounded wait gave up
 };
-int tc_tile_rows(int N, int sm_count);
+int tc_tile_rows(int N, int K, int R, int sm_count);
 int launch_gemm_tc(const TcGemmArgs &args, int sm_count, cudaStream_t s);
 
 }  // namespace hsd

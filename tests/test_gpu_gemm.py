@@ -61,6 +61,22 @@ def test_gemm_tile_and_cluster_edges(lib, R, N, K):
     assert bool(((out - ref).abs() < bound).all())
 
 
+@pytest.mark.parametrize("R", [33, 129])
+@pytest.mark.parametrize("N,K", [(7, 64),              # a tile of 8 rows
+                                 (250, 576), (1025, 1024), (1792, 512),     # clusters of eight: tiles of 24, 80 and 128 rows
+                                 (1793, 512), (2048, 1088), (4097, 256),    # of four
+                                 (4737, 192), (5632, 320), (9472, 128)])    # of two
+def test_gemm_of_more_rows_takes_narrower_tiles_of_the_same_sums(lib, R, N, K):
+    g = torch.Generator().manual_seed(R + N + K)
+    A = torch.randn(R, K, generator=g).to(torch.bfloat16).cuda()
+    W = (torch.randn(N, K, generator=g) * 0.05).to(torch.bfloat16).cuda()
+    out = lib.hsd_gemm_bf16(A, W)
+    few = torch.cat([lib.hsd_gemm_bf16(A[r:r + 32].contiguous(), W) for r in range(0, R, 32)])     # full tiles
+    assert torch.equal(out, few)                          # the k-blocks are divided alike, whatever the rows of a tile
+    bound = 2.0 ** -23 * (K / 32) * (A.double().abs() @ W.double().abs().T) + 1e-7
+    assert bool(((out.double() - A.double() @ W.double().T).abs() < bound).all())
+
+
 @pytest.mark.parametrize("R,N,K", [(5, 1024, 4096), (24, 14336, 512), (200, 2000, 1024)])
 def test_gemm_calls_back_to_back_see_what_the_stream_wrote_before(lib, R, N, K):
     # a call starts under the end of the one before it: operands rewritten between calls, a result that is the next operand,
