@@ -38,8 +38,9 @@ static inline int hsd_smem_limit(const void *kernel, int bytes, std::atomic<u64>
 // A chain of kernels on one stream, each of which may start (and prepare: barriers, tensor memory, the first weights) while
 // the one before it still runs.  Every CTA of such a kernel calls chain_wait() before it touches anything the kernels
 // before it read or wrote: it returns when the one before is complete, which had waited in the same way.  chain_next()
-// lets the next kernel's CTAs come as SMs become free.  A chain begins with a launch of the ordinary kind; in one, both
-// do nothing.
+// lets the next kernel's CTAs come as SMs become free.  The first kernel of a public call may itself start early, behind
+// whatever is on the stream; after a launch of the ordinary kind both do nothing.  A kernel whose successor reads inputs of the
+// call ahead of its own wait calls chain_next() behind its chain_wait().
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... KA, class... A>

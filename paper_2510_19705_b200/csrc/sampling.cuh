@@ -107,54 +107,29 @@ __device__ __forceinline__ u64 warp_sum54(u64 v) {
   return ((u64)hi << 27) + lo;
 }
 
-// ---- block-wide reductions over a group of threads: the whole block (blockDim.x a multiple of 32, at most
-// 1024), or the first N threads of a block that has other warps besides (named barrier ID).
-struct WholeBlock {
-  __device__ static __forceinline__ void sync() { __syncthreads(); }
-  __device__ static __forceinline__ int threads() { return blockDim.x; }
-};
-template <int ID, int N> struct FirstThreads {
-  __device__ static __forceinline__ void sync() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
-  __device__ static __forceinline__ int threads() { return N; }
-};
-
-template <class G = WholeBlock>
+// ---- block-wide reductions (blockDim.x a multiple of 32, at most 1024)
 __device__ __forceinline__ float block_max(float v, float *sh /*[32]*/) {
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-  int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = G::threads() >> 5;
-  G::sync();
+  int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (int)blockDim.x >> 5;
+  __syncthreads();
   if (l == 0) sh[w] = v;
-  G::sync();
+  __syncthreads();
   float r = (l < nw) ? sh[l] : -INFINITY;
   for (int o = 16; o > 0; o >>= 1) r = fmaxf(r, __shfl_xor_sync(0xFFFFFFFFu, r, o));
   return r;
 }
 
-// Sum of one u64 per thread; every thread gets the total.
-template <class G = WholeBlock>
-__device__ __forceinline__ u64 block_sum(u64 v, u64 *sh /*[33]*/) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = G::threads() >> 5;
-  G::sync();
-  if (l == 0) sh[w] = v;
-  G::sync();
-  u64 r = (l < nw) ? sh[l] : 0ull;
-  for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, o);
-  return r;
-}
-
 // Exclusive prefix sum of one u64 per thread in thread order; *total receives the block sum.
-template <class G = WholeBlock>
 __device__ __forceinline__ u64 block_exclusive_scan(u64 v, u64 *sh /*[33]*/, u64 *total) {
-  int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = G::threads() >> 5;
+  int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (int)blockDim.x >> 5;
   u64 inc = v;
   for (int o = 1; o < 32; o <<= 1) {
     u64 n = __shfl_up_sync(0xFFFFFFFFu, inc, o);
     if (l >= o) inc += n;
   }
-  G::sync();
+  __syncthreads();
   if (l == 31) sh[w] = inc;
-  G::sync();
+  __syncthreads();
   if (w == 0) {
     u64 t = (l < nw) ? sh[l] : 0ull, ti = t;
     for (int o = 1; o < 32; o <<= 1) {
@@ -164,7 +139,7 @@ __device__ __forceinline__ u64 block_exclusive_scan(u64 v, u64 *sh /*[33]*/, u64
     if (l < nw) sh[l] = ti - t;          // exclusive warp offsets
     if (l == 31) sh[32] = ti;            // block total
   }
-  G::sync();
+  __syncthreads();
   *total = sh[32];
   return sh[w] + inc - v;
 }
@@ -236,18 +211,18 @@ __device__ __forceinline__ float chunk_max(const Chunk32 &c, int V, int k0) {
 }
 // Inverse CDF over weights weight(i) of the thread's own 32 tokens (i = local index, compile-time in the
 // unrolled loops).  Same result as block_inverse_cdf with the same weights.
-template <class G = WholeBlock, class WeightFn>
+template <class WeightFn>
 __device__ __forceinline__ int block_inverse_cdf_chunk(int V, int k0, u32 U, WeightFn weight, u64 *sh64 /*[34]*/, u64 *total_out) {
   u64 local = 0;
 #pragma unroll
   for (int i = 0; i < kChunkTokens; ++i)
     if (k0 + i < V) local += weight(i);
   u64 total;
-  u64 excl = block_exclusive_scan<G>(local, sh64, &total);
+  u64 excl = block_exclusive_scan(local, sh64, &total);
   if (total_out) *total_out = total;
   int *result = reinterpret_cast<int *>(&sh64[33]);
   if (threadIdx.x == 0) *result = -1;
-  G::sync();
+  __syncthreads();
   if (total != 0) {
     u64 tau = cdf_threshold(U, total);
     if (tau >= excl && tau < excl + local) {
@@ -262,9 +237,9 @@ __device__ __forceinline__ int block_inverse_cdf_chunk(int V, int k0, u32 U, Wei
       }
     }
   }
-  G::sync();
+  __syncthreads();
   int r = *result;
-  G::sync();
+  __syncthreads();
   return r;
 }
 
