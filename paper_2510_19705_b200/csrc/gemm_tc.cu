@@ -5,7 +5,7 @@
 // shared memory and are added across the cluster in rank order (bit-reproducible): no pieces in global memory, no
 // counters.  With enough tiles to occupy the GPU a CTA takes whole tiles, and the next tile's weights stream in under a tile's finish.
 // A stream-K split over all SMs with pieces in global memory took 29.5 us for 14336 x 4096 at 24 rows (117 MB); whole tiles of 104 rows
-// on 138 CTAs take 25.6 us; 4096 x 4096 at 256 rows 49 -> 20 us.
+// on 138 CTAs take 25.6 us (22.5 started early); 4096 x 4096 at 256 rows 49 -> 20 us.
 //
 // 192 threads: warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer (one elected lane issues), warps 2..5 = epilogue
 // (each reads its own 32-lane quarter of TMEM).  Shared-memory ring of (128 x 64 weight tile + NPAD x 64 activation
