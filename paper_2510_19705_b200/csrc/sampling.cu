@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(32 * (GROUPS * WARPS + 1), 1) row_stats_kernel
     return;
   }
   // ---- the exponentials
+  chain_wait();                                            // (the limit of the waits below is for this kernel's own work)
   const int group = warp / WARPS, gwarp = warp - group * WARPS, gtid = gwarp * 32 + lane;
   const uint32_t maxima = empty + 8u * (kRsRing + group), full = full0 + 8u * kRsRing * group;
   uint32_t slot = (uint32_t)(group * passes * n_chunks) % kRsRing, y = 0, phase = 0;    // the next chunk: its slot, its barrier and phase

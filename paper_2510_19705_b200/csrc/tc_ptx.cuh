@@ -7,7 +7,10 @@
 namespace hsd {
 namespace ptx {
 
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;    // every device-side wait gives up after 2 s
+#ifndef HSD_WAIT_LIMIT_NS
+#define HSD_WAIT_LIMIT_NS 2000000000ull                        // (a test of the waits builds with a shorter one)
+#endif
+constexpr unsigned long long kWaitLimitNs = HSD_WAIT_LIMIT_NS; // every device-side wait gives up after 2 s
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
