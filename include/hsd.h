@@ -73,6 +73,8 @@ int hsd_draft_sample(const void *logits, int batch, int rows, int vocab, int dty
  *                  16-byte aligned; contents on entry are ignored, on exit unspecified
  *   out_tokens     device [batch, t+1] int32: x_1..x_n, m, then -1 padding
  *   out_n_accepted device [batch] int32: n
+ * A device-side wait that gives up after its two seconds (a GPU taken away meanwhile, say) leaves n = -1 and -1 for every
+ * token of the sequences it concerns; hsd_generate returns DEVICE_TIMEOUT.
  * Errors: INVALID_ARG, WORKSPACE_TOO_SMALL, CUDA.  Asynchronous on `stream`.
  */
 size_t hsd_verify_workspace_bytes(int batch, int t);

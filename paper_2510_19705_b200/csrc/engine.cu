@@ -898,7 +898,7 @@ int run_verify(hsd_ctx *c, int level, const std::vector<int> &act, const std::ve
   mirror.status_src = (const int *)(c->ws + c->status_off);
   mirror.n = c->result_host + kResultHead / 4;
   mirror.token = mirror.n + c->max_batch;
-  for (size_t i = 0; i < act.size(); ++i) mirror.n[i] = -1;       // (nothing is in flight that writes there: the last decision was waited for)
+  for (size_t i = 0; i < act.size(); ++i) mirror.n[i] = -2;       // (nothing is in flight that writes there: the last decision was waited for)
   HSD_TRY(launch_verify(c->ws + L.logits[level], c->ws + L.logits[level - 1], c->dev<int>(L.tokens), c->md.dtype, c->md.V,
                         (int)act.size(), t_max, vs_dev ? (const VerifySeq *)vs_dev : vs.data(), 0, 0, 0, c->ws + L.vscratch, c->seed, nullptr,
                         c->dev<int>(L.result + kResultHead), 1, c->stream, c->coin24[level], !vs_dev, mirror));
@@ -912,6 +912,7 @@ int run_verify(hsd_ctx *c, int level, const std::vector<int> &act, const std::ve
   hsd_level_stats &st = c->stats[level];
   for (size_t i = 0; i < act.size(); ++i) {
     int b = act[i], t = c->buf_len[b] - ctx[b], n = mirror.n[i];
+    if (n == kNoDecision) return HSD_E_DEVICE_TIMEOUT;
     if (n < 0 || n > t) return HSD_E_CUDA;
     int *toks = &c->tokens[(size_t)b * c->md.max_seq + ctx[b]];
     const std::vector<int> drafts(toks, toks + t);

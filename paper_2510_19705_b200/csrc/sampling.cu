@@ -91,7 +91,7 @@ decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, in
               const RowStat *__restrict__ stats, u64 seed, int32_t *__restrict__ out_tokens /*[B, t_max+1] or null*/,
               int32_t *__restrict__ out_n /*[B]*/, int write_in_place, u32 coin24, const HostMirror mirror) {
   __shared__ u64 sh64[34];
-  __shared__ int sh_first_reject;
+  __shared__ int sh_first_reject, sh_none;
   int b = blockIdx.x;
   VerifySeq d;
   if (desc.given()) d = desc.at(b);
@@ -100,11 +100,12 @@ decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, in
     d.tok_off = (long long)b * regular_t; d.serial = regular_serial; d.seq = b; d.level = regular_level;
   }
   const RowStat *st = stats + (size_t)b * (2 * t_max + 1);
-  if (threadIdx.x == 0) sh_first_reject = d.t;
+  if (threadIdx.x == 0) { sh_first_reject = d.t; sh_none = 0; }
   __syncthreads();
   if ((int)threadIdx.x < d.t) {
     int j = threadIdx.x;
     RowStat sp = st[j], sq = st[t_max + 1 + j];
+    if (sp.S == kNoStat || sq.S == kNoStat) sh_none = 1;
     const int tok = tokens[d.tok_off + j];
     const bool in = tok >= 0 && tok < V;
     u64 Pp = fixed_prob(in ? exp_weight(to_f32(p_logits[(size_t)(d.p_row0 + j) * V + tok]), sp.m) : 0u, prob_scale(sp.S));
@@ -116,6 +117,7 @@ decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, in
   }
   __syncthreads();
   int n = sh_first_reject;
+  const bool none = sh_none || st[n].S == kNoStat;             // (what the marks give stays within the row and the buffers)
   u32 U = uniform24(seed, 0, d.serial, d.level, PURPOSE_FINAL, d.seq);
   const T *prow = p_logits + (size_t)(d.p_row0 + n) * V;
   float mp = st[n].m;
@@ -149,16 +151,18 @@ decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, in
   }
   if (!fast && m_tok < 0)   // bonus token, or an all-zero residual: draw from the verifier's own row
     m_tok = block_inverse_cdf(V, U, [&](int k) { return (u64)exp_weight(to_f32(prow[k]), mp); }, sh64, nullptr);
+  if (none) m_tok = -1;
+  const int n_out = none ? kNoDecision : n;
   if (threadIdx.x == 0) {
-    out_n[b] = n;
+    out_n[b] = n_out;
     if (write_in_place) tokens[d.tok_off + n] = m_tok;
-    if (mirror.n) { mirror.n[b] = n; mirror.token[b] = m_tok; }
+    if (mirror.n) { mirror.n[b] = n_out; mirror.token[b] = m_tok; }
     if (mirror.status && b == 0) *mirror.status = __ldcg(mirror.status_src);
   }
   if (out_tokens) {
     for (int j = threadIdx.x; j <= t_max; j += blockDim.x) {
       int v = -1;
-      if (j < n) v = tokens[d.tok_off + j];
+      if (j < n_out) v = tokens[d.tok_off + j];
       else if (j == n) v = m_tok;
       out_tokens[(size_t)b * (t_max + 1) + j] = v;
     }
@@ -215,6 +219,13 @@ template <> struct RsMax<__nv_bfloat16> {
   }
   __device__ float get() const { return fmaxf(__low2float(m), __high2float(m)); }
 };
+
+// A warp's wait gave up: the mark on every row of its CTA (one that gets its statistics all the same may keep either).
+__device__ __noinline__ void give_up(RowStat *stats, long long n_items) {
+  RowStat st;
+  st.m = 0.f; st.S = kNoStat;
+  for (long long i = blockIdx.x + (long long)(threadIdx.x & 31) * gridDim.x; i < n_items; i += 32ll * gridDim.x) stats[i] = st;
+}
 
 template <typename T, int GROUPS, int WARPS, int CHUNK>
 __global__ void __launch_bounds__(32 * (GROUPS * WARPS + 1), 1) row_stats_kernel(const __grid_constant__ RowStatArgs a) {
@@ -361,7 +372,7 @@ __global__ void __launch_bounds__(32 * (GROUPS * WARPS + 1), 1) row_stats_kernel
   int last_stat = -1, k = 0;
   float last_m = 0.f;
   for (;; ++k) {
-    if (!wait_chunk()) return;
+    if (!wait_chunk()) goto gave_up;
     const int stat = infos[slot].stat, n_vec = infos[slot].n_vec, n_edge = infos[slot].n_edge;
     RsMax<T> mx;
     float edge = -INFINITY;
@@ -369,7 +380,7 @@ __global__ void __launch_bounds__(32 * (GROUPS * WARPS + 1), 1) row_stats_kernel
       if (gtid < n_edge) edge = infos[slot].edge[gtid];
       const uint32_t slot0 = slot;
       for (int c = 0; c < n_chunks; ++c) {
-        if (c > 0 && !wait_chunk()) return;
+        if (c > 0 && !wait_chunk()) goto gave_up;
         vectors(n_vec - c * kRsChunkVecs, [&](const uint4 &x) { mx.take(x); });
         if (!resident) chunk_done();
         next_slot(1);
@@ -380,14 +391,14 @@ __global__ void __launch_bounds__(32 * (GROUPS * WARPS + 1), 1) row_stats_kernel
     const int key = __reduce_max_sync(0xFFFFFFFFu, order_key(fmaxf(mx.get(), edge)));
     if (lane == 0) { sh_max[group][k & 1][gwarp] = key; ptx::mbar_arrive(maxima); }
     __syncwarp();
-    if (!ptx::mbar_wait_warp(maxima, (uint32_t)k & 1u, abort_flag)) return;
+    if (!ptx::mbar_wait_warp(maxima, (uint32_t)k & 1u, abort_flag)) goto gave_up;
     if (last_stat >= 0 && gwarp == k % WARPS) finish(last_stat, last_m, k - 1);
     if (stat < 0) return;
     const float m = order_value(__reduce_max_sync(0xFFFFFFFFu, sh_max[group][k & 1][lane % WARPS]));
     u64 local = 0;
     if (n_edge > 0) local += exp_weight(edge, m);
     for (int c = 0; c < n_chunks; ++c) {
-      if (!resident && !wait_chunk()) return;
+      if (!resident && !wait_chunk()) goto gave_up;
       vectors(n_vec - c * kRsChunkVecs, [&](const uint4 &x) {
         float f[VN];
         StatVec<T>::unpack(x, f);
@@ -406,6 +417,8 @@ __global__ void __launch_bounds__(32 * (GROUPS * WARPS + 1), 1) row_stats_kernel
     last_stat = stat; last_m = m;
     next_slot(others);
   }
+gave_up:
+  give_up(a.stats, (long long)a.batch * (2 * a.t_max + 1));
 }
 
 // ------------------------------------------------------------------------------ clusters
@@ -654,12 +667,14 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_stats_kernel(const __gr
 // of their totals.  Bound by latency: two gathers, a row of each side and an exchange.  Few
 // sequences of 32000 tokens: 5.8 us behind the statistics; 64 of them, two CTAs each: 11.  Sums of four tokens instead of weights
 // in registers, two CTAs an SM: 11 and 8.4.  The first positions' statistics kept in shared memory: 0.3 us more.
-template <typename T, int PER, int NT>
+// MARKS: the statistics may be marks; looking for them costs 0.1 us (one sequence of three drafts: 7.39, with them 7.49), which
+// cluster_stats_kernel, without a bounded wait, spares.
+template <typename T, int PER, int NT, bool MARKS>
 __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __grid_constant__ ClusterArgs a, const RowStat *stats) {
   typedef typename ClUnit<T, PER>::raw raw_t;
   constexpr int NU = NT / PER;
   __shared__ u64 wsum[2][kClWarps], csum[2][kClMaxC];              // [residual, the verifier's row]
-  __shared__ int sh_n;
+  __shared__ int sh_n, sh_none;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const u32 rank = cl_rank(), C = cl_size();
   const int b = (int)cl_id();
@@ -677,7 +692,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
     const float4 v = __ldcg(reinterpret_cast<const float4 *>(s));
     return *reinterpret_cast<const RowStat *>(&v);
   };
-  if (tid == 0) sh_n = t;
+  if (tid == 0) { sh_n = t; sh_none = 0; }
   // the call's inputs are complete when the statistics kernel begins: the drafted tokens' logits come ahead of its end
   int tok = -1;
   float lp = 0.f, lq = 0.f;
@@ -692,6 +707,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
   for (int j = tid; j < t; j += kClThreads) {
     if (j != tid) drafted(j);
     const RowStat s = stat(sp + j), r = stat(sq + j);
+    if (MARKS && (s.S == kNoStat || r.S == kNoStat)) sh_none = 1;
     const bool in = tok >= 0 && tok < a.V;
     const u64 Pp = fixed_prob(in ? exp_weight(lp, s.m) : 0u, prob_scale(s.S)), Pq = fixed_prob(in ? exp_weight(lq, r.m) : 0u, prob_scale(r.S));
     const u32 U = uniform24(a.seed, j, d.serial, d.level, PURPOSE_ACCEPT, d.seq);
@@ -703,6 +719,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
   const int n = sh_n, tok0 = (int)rank * a.seg, tok_end = min(a.V, tok0 + a.seg);
   const int k_lane = tok0 + warp * (32 * NT) + lane * PER;         // first token of unit i: k_lane + 32 PER i
   const RowStat spn = stat(sp + n);
+  if (MARKS && tid == 0 && spn.S == kNoStat) sh_none = 1;
   raw_t vp[NU];
   auto fetch = [&](const T *row, raw_t *v) {                       // -inf past the CTA's tokens: no weight
 #pragma unroll
@@ -768,6 +785,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
     }
     exchange(1, local);
   }
+  if (MARKS && sh_none) total = 0;                                 // (what the marks gave so far stays within the row and the buffers)
   const u32 U = uniform24(a.seed, 0, d.serial, d.level, PURPOSE_FINAL, d.seq);
   const u64 tau = cdf_threshold(U, total);
   u64 before = 0;
@@ -777,20 +795,21 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
     if (a.out_tokens) a.out_tokens[(size_t)b * (a.t_max + 1) + n] = k;
     if (a.mirror.n) a.mirror.token[b] = k;
   };
-  if (total == 0) {                                                // non-finite logits: no token
+  if (total == 0) {                                                // non-finite logits or no statistics: no token
     if (rank == 0 && tid == 0) emit(-1);
   } else if (tau >= before && tau < before + csum[src][rank]) {
     cl_find_token<NT, PER>(w, tau, before, wsum[src], k_lane, emit);
   }
   if (rank == 0) {
+    const int n_out = MARKS && sh_none ? kNoDecision : n;
     if (tid == 0) {
-      a.out_n[b] = n;
-      if (a.mirror.n) a.mirror.n[b] = n;
+      a.out_n[b] = n_out;
+      if (a.mirror.n) a.mirror.n[b] = n_out;
       if (a.mirror.status && b == 0) *a.mirror.status = __ldcg(a.mirror.status_src);
     }
     if (a.out_tokens)
       for (int j = tid; j <= a.t_max; j += kClThreads)
-        if (j != n) a.out_tokens[(size_t)b * (a.t_max + 1) + j] = j < n ? a.tokens[d.tok_off + j] : -1;
+        if (j != n) a.out_tokens[(size_t)b * (a.t_max + 1) + j] = j < n_out ? a.tokens[d.tok_off + j] : -1;
   }
 }
 
@@ -905,27 +924,47 @@ static int launch_cluster_stats(const RowStatArgs &a, const ClusterPlan &pl, int
   hsd_count_launches(1);
   return HSD_OK;
 }
-static int launch_row_stats(const RowStatArgs &a, int dtype, cudaStream_t s) {
+// *marks: the statistics may be marks (kNoStat)
+static int launch_row_stats(const RowStatArgs &a, int dtype, cudaStream_t s, bool *marks) {
   const long long n_items = (long long)a.batch * (2 * a.t_max + 1);
   ClusterPlan pl;
   if (n_items <= 2 * kMeasuredSMs && cluster_plan(a.p, a.q, dtype, a.V, (int)n_items, true, &pl) && cluster_pays_stats(pl, n_items)) {
     if (dtype == HSD_F32) return launch_cluster_stats<float, 1>(a, pl, (int)n_items, s);
     return pl.per == 2 ? launch_cluster_stats<__nv_bfloat16, 2>(a, pl, (int)n_items, s) : launch_cluster_stats<__nv_bfloat16, 1>(a, pl, (int)n_items, s);
   }
+  *marks = true;
   const int grid = (int)std::min<long long>(sm_count(), n_items);
   if (n_items <= grid)                                     // a row a CTA: all its warps on it
     return dtype == HSD_F32 ? launch_row_stats_t<float, 1, 16, 32768>(a, grid, s) : launch_row_stats_t<__nv_bfloat16, 1, 16, 32768>(a, grid, s);
   return dtype == HSD_F32 ? launch_row_stats_t<float, 3, 8, 32768>(a, grid, s) : launch_row_stats_t<__nv_bfloat16, 3, 8, 32768>(a, grid, s);
 }
 
-template <typename T, int PER>
+template <typename T, int PER, bool MARKS>
 static int launch_decide_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, const RowStat *stats, cudaStream_t s) {
   const int grid = n * pl.C;
-  if (pl.NT == 8) HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 8>, grid, kClThreads, 0, s, pl.C, true, a, stats));
-  else if (pl.NT == 16) HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 16>, grid, kClThreads, 0, s, pl.C, true, a, stats));
-  else HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 32>, grid, kClThreads, 0, s, pl.C, true, a, stats));
+  if (pl.NT == 8) HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 8, MARKS>, grid, kClThreads, 0, s, pl.C, true, a, stats));
+  else if (pl.NT == 16) HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 16, MARKS>, grid, kClThreads, 0, s, pl.C, true, a, stats));
+  else HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 32, MARKS>, grid, kClThreads, 0, s, pl.C, true, a, stats));
   hsd_count_launches(1);
   return hsd_launch_status();
+}
+
+template <typename T> static int launch_decide_long(const ClusterArgs &a, int batch, const RowStat *stats, cudaStream_t s) {
+  decide_kernel<T><<<batch, kSampleThreads, 0, s>>>((const T *)a.p, (const T *)a.q, a.tokens, a.V, a.t_max, a.desc, a.regular_t, a.regular_serial,
+                                                    a.regular_level, stats, a.seed, a.out_tokens, a.out_n, a.write_in_place, a.coin24, a.mirror);
+  hsd_count_launches(1);
+  return hsd_launch_status();
+}
+template <bool MARKS> static int launch_decide(const ClusterArgs &a, const ClusterPlan &pl, int dtype, int batch, const RowStat *stats, cudaStream_t s) {
+  if (dtype == HSD_F32) return launch_decide_nt<float, 1, MARKS>(a, pl, batch, stats, s);
+  return pl.per == 2 ? launch_decide_nt<__nv_bfloat16, 2, MARKS>(a, pl, batch, stats, s) : launch_decide_nt<__nv_bfloat16, 1, MARKS>(a, pl, batch, stats, s);
+}
+static int launch_decisions(ClusterArgs a, int dtype, int batch, const RowStat *stats, bool marks, cudaStream_t s) {
+  ClusterPlan pl;
+  if (!cluster_plan(a.p, a.q, dtype, a.V, batch, false, &pl))      // rows of more than 131072 tokens
+    return dtype == HSD_BF16 ? launch_decide_long<__nv_bfloat16>(a, batch, stats, s) : launch_decide_long<float>(a, batch, stats, s);
+  a.seg = pl.seg;
+  return marks ? launch_decide<true>(a, pl, dtype, batch, stats, s) : launch_decide<false>(a, pl, dtype, batch, stats, s);
 }
 
 int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int V, int batch, int t_max,
@@ -936,29 +975,16 @@ int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int 
   if (desc_on_host && batch > kInlineDesc) return HSD_E_INVALID_ARG;
   const DescList<VerifySeq> list = desc_list(desc, batch, desc_on_host);
   RowStat *stats = (RowStat *)((char *)scratch + verify_counter_bytes(batch));
+  RowStatArgs r = {};
+  r.p = p; r.q = q; r.V = V; r.t_max = t_max; r.batch = batch; r.regular_t = regular_t; r.desc = list; r.stats = stats;
+  bool marks = false;
+  const int st = launch_row_stats(r, dtype, s, &marks);
+  if (st) return st;
   ClusterArgs a = {};
   a.p = p; a.q = q; a.tokens = tokens; a.V = V; a.t_max = t_max; a.desc = list; a.mirror = mirror; a.regular_t = regular_t;
   a.regular_serial = regular_serial; a.regular_level = regular_level; a.seed = seed; a.out_tokens = out_tokens; a.out_n = out_n;
   a.write_in_place = write_in_place; a.coin24 = coin24;
-  ClusterPlan pl;
-  RowStatArgs r = {};
-  r.p = p; r.q = q; r.V = V; r.t_max = t_max; r.batch = batch; r.regular_t = regular_t; r.desc = list; r.stats = stats;
-  const int st = launch_row_stats(r, dtype, s);
-  if (st) return st;
-  if (cluster_plan(p, q, dtype, V, batch, false, &pl)) {
-    a.seg = pl.seg;
-    if (dtype == HSD_F32) return launch_decide_nt<float, 1>(a, pl, batch, stats, s);
-    return pl.per == 2 ? launch_decide_nt<__nv_bfloat16, 2>(a, pl, batch, stats, s) : launch_decide_nt<__nv_bfloat16, 1>(a, pl, batch, stats, s);
-  }
-  // rows of more than 131072 tokens
-  if (dtype == HSD_BF16)
-    decide_kernel<__nv_bfloat16><<<batch, kSampleThreads, 0, s>>>((const __nv_bfloat16 *)p, (const __nv_bfloat16 *)q, tokens, V, t_max, list, regular_t,
-                                                                  regular_serial, regular_level, stats, seed, out_tokens, out_n, write_in_place, coin24, mirror);
-  else
-    decide_kernel<float><<<batch, kSampleThreads, 0, s>>>((const float *)p, (const float *)q, tokens, V, t_max, list, regular_t,
-                                                          regular_serial, regular_level, stats, seed, out_tokens, out_n, write_in_place, coin24, mirror);
-  hsd_count_launches(1);
-  return hsd_launch_status();
+  return launch_decisions(a, dtype, batch, stats, marks, s);
 }
 
 // ------------------------------------------------------------------------------ static scratch

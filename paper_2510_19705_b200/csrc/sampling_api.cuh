@@ -24,8 +24,10 @@ struct VerifySeq {
 
 struct __align__(16) RowStat {
   float m;     // row maximum
-  u64 S;       // sum of the integer weights
+  u64 S;       // sum of the integer weights (< 2^63), or kNoStat
 };
+constexpr u64 kNoStat = ~0ull;     // a bounded wait gave up: the row has no statistics, and its sequence no decision:
+constexpr int kNoDecision = -1;    // the accepted count then, and every token
 
 size_t verify_scratch_bytes(int batch, int t_max);
 
