@@ -81,7 +81,7 @@ alpha_stats_kernel(const T *__restrict__ logits, long long model_stride, int R, 
   __shared__ float shm[kAlphaThreads / 32], shs[kAlphaThreads / 32];
   chain_wait();
   chain_next();                                                       // (behind the wait: the pairs' first logits are read ahead of theirs)
-  const int l = blockIdx.x / R, r = blockIdx.x - l * R;
+  const int r = blockIdx.x, l = blockIdx.y;                           // (positions x models may pass 2^31)
   const T *row = logits + (size_t)l * model_stride + (size_t)r * V;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int N = VEC ? AlphaVec<T>::N : 1, U = 4;
@@ -372,7 +372,7 @@ int launch_alpha_t(const T *logits, long long model_stride, int L, int R, int V,
   const AlphaPlan p = alpha_plan(L, R, V);
   float2 *stats = (float2 *)((char *)ws + p.stats_off);
   float *partials = (float *)((char *)ws + p.partials_off);
-  HSD_CUDA_OK(hsd_launch(alpha_stats_kernel<T, VEC>, R * L, kAlphaThreads, 0, s, 0, true, logits, model_stride, R, V, stats));
+  HSD_CUDA_OK(hsd_launch(alpha_stats_kernel<T, VEC>, dim3(R, L), kAlphaThreads, 0, s, 0, true, logits, model_stride, R, V, stats));
   int st = HSD_OK;
   if (p.n_pairs > 0)
     st = L <= 8    ? launch_pairs<T, VEC, 1024>(logits, model_stride, L, R, V, p, stats, partials, s)

@@ -44,9 +44,9 @@ static inline int hsd_smem_limit(const void *kernel, int bytes, std::atomic<u64>
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... KA, class... A>
-static inline cudaError_t hsd_launch(void (*kernel)(KA...), int grid, int threads, size_t smem, cudaStream_t s, int cluster, bool chained, A &&...args) {
+static inline cudaError_t hsd_launch(void (*kernel)(KA...), dim3 grid, int threads, size_t smem, cudaStream_t s, int cluster, bool chained, A &&...args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
   cudaLaunchAttribute at[2];
   int n = 0;
   if (cluster > 0) {

@@ -182,3 +182,21 @@ def test_rates_of_calls_back_to_back(lib, dtype, L, R, V):
         got.append(lib.hsd_pairwise_alpha(x))
         lib.hsd_pairwise_alpha(sets[(i + 1) % 3])
     assert all(torch.equal(a, want[i % 3]) for i, a in enumerate(got))
+
+
+def test_more_rows_of_all_models_than_fit_one_grid_dimension(lib):
+    # 8 models x (2^28 + 3) positions of two tokens: 2^31 rows; 8.6 GB of logits, 47 GB of workspace
+    L, R, split = 8, 2 ** 28 + 3, 2 ** 27
+    a = torch.tensor([[0.25 * l, 1.0] for l in range(L)], device="cuda").to(torch.bfloat16)
+    b = torch.tensor([[-1.0, 0.5 * l] for l in range(L)], device="cuda").to(torch.bfloat16)
+    x = torch.empty(L, R, 2, dtype=torch.bfloat16, device="cuda")
+    x[:, :split] = a[:, None]
+    x[:, split:] = b[:, None]
+    got = lib.hsd_pairwise_alpha(x).cpu()
+    want = torch.zeros(L, L, dtype=torch.float64)
+    for rows, share in ((a, split / R), (b, 1 - split / R)):
+        p = torch.softmax(rows.cpu().double(), -1)
+        want += share * torch.minimum(p[:, None], p[None]).sum(-1)
+    assert (got - want).abs().max() < 1e-5                            # fp32 softmax and sums of two tokens
+    del x
+    torch.cuda.empty_cache()
