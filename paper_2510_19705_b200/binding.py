@@ -11,9 +11,11 @@ import os
 
 import torch
 
+from . import build
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libhsd.so")
-HOST_PATH = os.path.join(_HERE, "_host_calls.so")
+HOST_PATH = build.host_path()
 HSD_F32, HSD_BF16 = 0, 1
 _lib = None
 _host = None
@@ -42,7 +44,7 @@ def _host_calls():
     global _host
     if _host is None:
         if not os.path.exists(HOST_PATH):
-            raise HsdError("_host_calls.so is missing: run `python -m paper_2510_19705_b200.build`")
+            raise HsdError(os.path.basename(HOST_PATH) + " is missing: run `python -m paper_2510_19705_b200.build`")
         lib = library()
         spec = importlib.util.spec_from_file_location("_host_calls", HOST_PATH)
         mod = importlib.util.module_from_spec(spec)

@@ -28,8 +28,9 @@ def _torch():
 
 
 def host_path():
-    """The binding's native calls (None without torch)."""
-    return os.path.join(HERE, "_host_calls.so") if _torch() else None
+    """The binding's native calls, built against this Python and this torch (None without torch)."""
+    torch = _torch()
+    return torch and os.path.join(HERE, "_host_calls.%s.torch-%s.so" % (sysconfig.get_config_var("SOABI"), torch.__version__))
 
 
 def _older(target, deps):

@@ -1,4 +1,4 @@
-"""The C-ABI library is built by nvcc alone; the binding's native calls come after it."""
+"""The C-ABI library is built by nvcc alone; the binding's native calls come after it and belong to one Python and one torch."""
 import os
 import shutil
 import stat
@@ -38,3 +38,12 @@ def test_the_library_is_built_without_torch(tmp_path):
 def test_the_library_is_there_when_the_native_calls_cannot_be_built(tmp_path, compiler):
     r, built = _build(tmp_path, "from paper_2510_19705_b200 import build\nbuild.build()", CXX=compiler)
     assert r.returncode != 0 and built == ["libhsd.so"]
+
+
+def test_native_calls_of_another_torch_are_not_taken(monkeypatch):
+    import torch
+    build.build()
+    here = build.host_path()
+    assert os.path.exists(here) and not build.needs_build()
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert build.host_path() != here and build.needs_build()
