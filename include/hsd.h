@@ -94,7 +94,7 @@ int hsd_verify_level(int level, const void *target_logits, const void *draft_log
  * makes such callers find scratch memory somewhere; this variant brings its own.
  *
  * Same arguments, outputs and results as hsd_verify_level.  The scratch (row statistics)
- * lives in a fixed device array of 98,560 bytes inside the library image (every GPU
+ * lives in a fixed device array of 65,536 bytes inside the library image (every GPU
  * that loads the library holds it until the process exits), which bounds the call:
  * batch * (2 t + 1) <= 4096, else HSD_E_TOO_LARGE (exactly 4096 is accepted).
  * The call performs no cudaMalloc / cudaFree and uses no allocating library routine.

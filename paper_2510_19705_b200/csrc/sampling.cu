@@ -861,11 +861,9 @@ static int launch_cluster_draw(ClusterArgs a, const ClusterPlan &pl, int dtype, 
 }
 
 // ------------------------------------------------------------------------------ host launchers
-// Scratch of one verification call: [unused: counters of an earlier kernel, kept so that a workspace laid out for a call is what
-// it was] [RowStat per logits row].
-static size_t verify_counter_bytes(int batch) { return ((size_t)(2 * batch + 2) * 4 + 255) / 256 * 256; }
+// Scratch of one verification call: a RowStat per logits row, at its front.  (The rest is room that callers' buffers have always had.)
 size_t verify_scratch_bytes(int batch, int t_max) {
-  return verify_counter_bytes(batch) + (size_t)batch * (2 * t_max + 1) * sizeof(RowStat);
+  return ((size_t)(2 * batch + 2) * 4 + 255) / 256 * 256 + (size_t)batch * (2 * t_max + 1) * sizeof(RowStat);
 }
 
 template <typename T>
@@ -974,7 +972,7 @@ int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int 
   if (batch == 0) return HSD_OK;
   if (desc_on_host && batch > kInlineDesc) return HSD_E_INVALID_ARG;
   const DescList<VerifySeq> list = desc_list(desc, batch, desc_on_host);
-  RowStat *stats = (RowStat *)((char *)scratch + verify_counter_bytes(batch));
+  RowStat *stats = (RowStat *)scratch;
   RowStatArgs r = {};
   r.p = p; r.q = q; r.V = V; r.t_max = t_max; r.batch = batch; r.regular_t = regular_t; r.desc = list; r.stats = stats;
   bool marks = false;
@@ -990,9 +988,8 @@ int launch_verify(const void *p, const void *q, int32_t *tokens, int dtype, int 
 // ------------------------------------------------------------------------------ static scratch
 // Scratch for hsd_verify_level_static: lives in the library image, so every GPU that loads the
 // library holds these bytes until the process exits.  One RowStat per logits row of a call.
-constexpr int kStaticStatRows = 4096;                       // 64 KiB of row statistics behind verify_counter_bytes()
-constexpr size_t kStaticScratchBytes = kStaticStatRows * sizeof(RowStat) + ((2 * kStaticStatRows + 2) * 4 + 255) / 256 * 256;
-static __device__ __align__(256) unsigned char g_static_verify_scratch[kStaticScratchBytes];
+constexpr int kStaticStatRows = 4096;
+static __device__ RowStat g_static_verify_scratch[kStaticStatRows];
 
 // In host code the array's name is only a stand-in for the symbol, not a device address: the
 // address has to be asked for, once per device, with that device current.  The answer is kept per
