@@ -183,8 +183,8 @@ __device__ __forceinline__ void alpha_block(const float *pi, const float *pj, in
 // shared memory TILE at a time as probabilities [model][token] (double-buffered: the next tile's logits are fetched under
 // this tile's minima).  A warp owns one pair of 8-model blocks, or two diagonal blocks (about as much work), and the tokens
 // lane + 32 slice, ...; with fewer blocks than warps the warps share a pair and split the tokens.
-// 32 models x 256 positions x 32000 tokens: 478 us here + 97 us of statistics; one pair per lane, two shared-memory loads
-// per pair and token, took 5021 + 176 us.
+// 32 models x 256 positions x 32000 tokens: 478 us here + 97 us of statistics, each alone (a call 566 to 571); one pair per lane,
+// two shared-memory loads per pair and token, took 5021 + 176 us.
 // All 256 threads stage, so TILE x models is constant: 256 tokens of up to 32 models, 512 of 16, 1024 of 8.  (256 tokens of
 // two models keep 16 threads busy: 2 x 256 x 32000 in fp32 153 us, this way 70.)
 template <typename T, bool VEC, int TILE>

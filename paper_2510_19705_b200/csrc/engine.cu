@@ -1461,7 +1461,7 @@ int hsd_gemm_bf16(const void *A, int R, int K, const void *W, int N, float *out,
   a.status = (int *)workspace;
   a.reset_status = 1;
   // Launched early behind whatever is on the stream, so that a call's launch, barriers and tensor memory hide under the end of
-  // the call before: 24 rows, 14336 x 4096 25.4 -> 22.5 us, 4096 x 4096 12.4 -> 10.0.  Weights ahead of the wait as well would give
+  // the call before: 24 rows, 14336 x 4096 25.4 -> 22.5 us (23.2 on the slowest box), 4096 x 4096 12.4 -> 10.0.  Weights ahead of the wait as well would give
   // 21.7 and 9.9, but here the kernel before may be the one that writes them.
   a.chained = true;
   return launch_gemm_tc(a, sms, (cudaStream_t)stream);

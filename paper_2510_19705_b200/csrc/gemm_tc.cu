@@ -5,7 +5,7 @@
 // shared memory and are added across the cluster in rank order (bit-reproducible): no pieces in global memory, no
 // counters.  With enough tiles to occupy the GPU a CTA takes whole tiles, and the next tile's weights stream in under a tile's finish.
 // A stream-K split over all SMs with pieces in global memory took 29.5 us for 14336 x 4096 at 24 rows (117 MB); whole tiles of 104 rows
-// on 138 CTAs take 25.6 us (22.5 started early); 4096 x 4096 at 256 rows 49 -> 20 us.
+// on 138 CTAs take 25.6 us (22.5 to 23.2 started early, over five boxes); 4096 x 4096 at 256 rows 49 -> 20 us.
 //
 // 192 threads: warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer (one elected lane issues), warps 2..5 = epilogue
 // (each reads its own 32-lane quarter of TMEM).  Shared-memory ring of (128 x 64 weight tile + NPAD x 64 activation
@@ -452,7 +452,8 @@ int tc_npad(int rows) { return rows <= 16 ? 16 : rows <= 32 ? 32 : rows <= 64 ? 
 namespace {
 // CTAs a tile's k-blocks are divided over: 2, 4 or (few tiles) 8 while full tiles alone leave half the SMs idle.  The division
 // does not depend on the number of rows, so neither does a row's result.  48 clusters of three or 16 of eight do not run at
-// once (6144 x 4096 at 128 rows: 36 us in threes, 25 us in pairs), 74 of two, 32 of four and 14 of eight do.
+// once (6144 x 4096 at 128 rows: 36 us in threes, 25 us in pairs), 74 of two, 32 of four and 14 of eight do (on the GPU that
+// was measured: speed only).
 int split_of(int full_tiles, int K, int sm_count) {
   int S = 1;
   while (S < (full_tiles <= 14 ? 8 : 4) && full_tiles * S * 2 <= sm_count && S * 2 <= K / kTcBlockK) S *= 2;

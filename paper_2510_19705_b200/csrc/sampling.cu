@@ -8,8 +8,6 @@
 
 namespace hsd {
 
-// ------------------------------------------------------------------------------ draft sampling
-// One block per row: token = inverse-CDF sample of softmax(row) with the purpose-0 uniform.
 // A call's descriptors: n_inline of them here, or all at `desc`, or (both zero) worked out from the regular layout.
 template <typename D> struct DescList {
   const D *desc;
@@ -26,6 +24,8 @@ template <typename D> static DescList<D> desc_list(const D *desc, int n, bool on
   return l;
 }
 
+// ------------------------------------------------------------------------------ draft sampling
+// One block per row: token = inverse-CDF sample of softmax(row) with the purpose-0 uniform.
 template <typename T>
 __global__ void __launch_bounds__(kSampleThreads)
 draft_sample_kernel(const T *__restrict__ logits, int V, const __grid_constant__ DescList<SampleRow> desc,
@@ -80,7 +80,8 @@ template <> struct StatVec<float> {
     f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y); f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
   }
 };
-// ------------------------------------------------------------------------------ decision
+
+// ------------------------------------------------------------------------------ decision, vocabularies past 131072 tokens
 // One block per sequence: accept tests for all positions (each with its own counter-addressed
 // uniform, so the parallel form equals Algorithm 2's sequential loop with break), n = index of the
 // first rejection, then the final draw from the residual of row n (n < t) or from target row t.
@@ -122,24 +123,7 @@ decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, in
   const T *prow = p_logits + (size_t)(d.p_row0 + n) * V;
   float mp = st[n].m;
   int m_tok = -1;
-  const bool fast = sizeof(T) == 2 && chunk_layout_ok(prow, V, blockDim.x) &&
-                    (n >= d.t || chunk_layout_ok(q_logits + (size_t)(d.q_row0 + n) * V, V, blockDim.x));
-  if (fast) {
-    const int k0 = threadIdx.x * kChunkTokens;
-    const Chunk32 cp = chunk_load(reinterpret_cast<const __nv_bfloat16 *>(prow), V, k0);
-    if (n < d.t) {
-      const Chunk32 cq = chunk_load(reinterpret_cast<const __nv_bfloat16 *>(q_logits + (size_t)(d.q_row0 + n) * V), V, k0);
-      const float mq = st[t_max + 1 + n].m;
-      const ProbScale psp = prob_scale(st[n].S), psq = prob_scale(st[t_max + 1 + n].S);
-      m_tok = block_inverse_cdf_chunk(V, k0, U, [&](int i) {
-        u64 Pp = fixed_prob(exp_weight(chunk_get(cp, i), mp), psp);
-        u64 Pq = fixed_prob(exp_weight(chunk_get(cq, i), mq), psq);
-        return Pp > Pq ? Pp - Pq : 0ull;
-      }, sh64, nullptr);
-    }
-    if (m_tok < 0)
-      m_tok = block_inverse_cdf_chunk(V, k0, U, [&](int i) { return (u64)exp_weight(chunk_get(cp, i), mp); }, sh64, nullptr);
-  } else if (n < d.t) {
+  if (n < d.t) {
     const T *qrow = q_logits + (size_t)(d.q_row0 + n) * V;
     float mq = st[t_max + 1 + n].m;
     ProbScale psp = prob_scale(st[n].S), psq = prob_scale(st[t_max + 1 + n].S);
@@ -149,7 +133,7 @@ decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, in
       return Pp > Pq ? Pp - Pq : 0ull;
     }, sh64, nullptr);
   }
-  if (!fast && m_tok < 0)   // bonus token, or an all-zero residual: draw from the verifier's own row
+  if (m_tok < 0)   // bonus token, or an all-zero residual: draw from the verifier's own row
     m_tok = block_inverse_cdf(V, U, [&](int k) { return (u64)exp_weight(to_f32(prow[k]), mp); }, sh64, nullptr);
   if (none) m_tok = -1;
   const int n_out = none ? kNoDecision : n;
@@ -179,7 +163,10 @@ decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, in
 // much as a row of 2048 logits has of arithmetic) run under the others' exponentials.  A row stays in the ring between its
 // maximum and its sum; rows of more chunks than the ring has come through it twice.
 constexpr uint32_t kRsPiece = 2048;                        // bytes; a chunk is asked for by its first lanes (a single large copy runs at a fraction of an SM's bandwidth)
-constexpr uint32_t kRsBytes = 229376;                      // of the ring
+constexpr uint32_t kRsChunk = 32768;
+constexpr int kRsRing = 7, kRsChunkVecs = kRsChunk / 16;
+constexpr uint32_t kRsBytes = kRsRing * kRsChunk;          // of the ring
+static_assert(kRsChunk <= 32 * kRsPiece);
 constexpr int kRsMaxEdge = 16;
 
 struct RowStatArgs {
@@ -227,11 +214,8 @@ __device__ __noinline__ void give_up(RowStat *stats, long long n_items) {
   for (long long i = blockIdx.x + (long long)(threadIdx.x & 31) * gridDim.x; i < n_items; i += 32ll * gridDim.x) stats[i] = st;
 }
 
-template <typename T, int GROUPS, int WARPS, int CHUNK>
+template <typename T, int GROUPS, int WARPS>
 __global__ void __launch_bounds__(32 * (GROUPS * WARPS + 1), 1) row_stats_kernel(const __grid_constant__ RowStatArgs a) {
-  constexpr int kRsRing = (int)kRsBytes / CHUNK, kRsChunkVecs = CHUNK / 16;
-  constexpr uint32_t kRsChunk = CHUNK;
-  static_assert(CHUNK <= 32 * (int)kRsPiece && CHUNK % 16 == 0);
   extern __shared__ uint8_t rs_smem_raw[];
   uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(rs_smem_raw) + 127) & ~(uintptr_t)127);
   // full, per group | empty, per slot of the ring | a row's maxima, per group.  A parity wait tells a barrier's phases apart
@@ -424,8 +408,8 @@ gave_up:
 // ------------------------------------------------------------------------------ clusters
 // Draws, the statistics of few rows and all decisions: a cluster of C CTAs takes a row (a decision: a row of each side), each CTA
 // the same V / C consecutive tokens.  Bound by latency, not by bytes (a row of 32000 bf16 tokens is 64 KB): a CTA's tokens are
-// read once into registers, the maximum and then the integer total cross the cluster in one exchange each.  No scratch in
-// global memory, nothing to clear.
+// read once into registers, the maximum and then the integer total cross the cluster in one exchange each.  Draws need no
+// scratch in global memory; statistics and decisions meet in the RowStats there.
 // A warp owns consecutive tokens; lane and unit index are interleaved (unit = 4 bytes: a bf16 pair or an fp32 value;
 // 2 bytes when rows of odd length leave bf16 pairs unaligned), so loads are whole lines whatever the row's alignment.
 constexpr int kClThreads = 512, kClWarps = kClThreads / 32, kClMaxC = 8;
@@ -667,6 +651,7 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_stats_kernel(const __gr
 // of their totals.  Bound by latency: two gathers, a row of each side and an exchange.  Few
 // sequences of 32000 tokens: 5.8 us behind the statistics; 64 of them, two CTAs each: 11.  Sums of four tokens instead of weights
 // in registers, two CTAs an SM: 11 and 8.4.  The first positions' statistics kept in shared memory: 0.3 us more.
+// 32 tokens a thread (calls whose clusters are of one or two CTAs): their 64-bit weights go past 128 registers, 84 to 144 bytes spill.
 // MARKS: the statistics may be marks; looking for them costs 0.1 us (one sequence of three drafts: 7.39, with them 7.49), which
 // cluster_stats_kernel, without a bounded wait, spares.
 template <typename T, int PER, int NT, bool MARKS>
@@ -815,7 +800,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
 
 // Cluster size, tokens a thread and tokens a CTA of a call with n clusters; false if the rows are too long.  `two`: two CTAs per SM.
 struct ClusterPlan { int C, NT, per, seg; };
-constexpr int kClEights = 14;                     // clusters of eight that run at once (one CTA per SM)
+constexpr int kClEights = 14;                     // clusters of eight that run at once (one CTA per SM) on the GPU that was measured: speed only
 static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, bool two, ClusterPlan *pl) {
   pl->per = (dtype == HSD_BF16 && V % 2 == 0 && ((uintptr_t)p & 3) == 0 && ((uintptr_t)q & 3) == 0) ? 2 : 1;
   // as many CTAs as run at once, of at least 4096 tokens (eight a thread) each: clusters of eight do not fit all SMs
@@ -902,19 +887,16 @@ static int sm_count() {
   return sms;
 }
 
-template <typename T, int GROUPS, int WARPS, int CHUNK>
+template <typename T, int GROUPS, int WARPS>
 static int launch_row_stats_t(const RowStatArgs &a, int grid, cudaStream_t s) {
   constexpr int smem = (int)kRsBytes + 128;
   static std::atomic<u64> limits{0};
-  const int limit = hsd_smem_limit((const void *)row_stats_kernel<T, GROUPS, WARPS, CHUNK>, smem, limits);
+  const int limit = hsd_smem_limit((const void *)row_stats_kernel<T, GROUPS, WARPS>, smem, limits);
   if (limit) return limit;
-  HSD_CUDA_OK(hsd_launch(row_stats_kernel<T, GROUPS, WARPS, CHUNK>, grid, 32 * (GROUPS * WARPS + 1), smem, s, 0, true, a));
+  HSD_CUDA_OK(hsd_launch(row_stats_kernel<T, GROUPS, WARPS>, grid, 32 * (GROUPS * WARPS + 1), smem, s, 0, true, a));
   hsd_count_launches(1);
   return HSD_OK;
 }
-// us a call, GROUPS x WARPS = 1 x 16 / 2 x 8 / 3 x 8 (chunks of 32 KB; 2 x 12 on chunks of 24 KB lies behind 2 x 8):
-//   a row a CTA, 32000: bf16 5.6 / 5.9 / 6.2, fp32 6.9 / 7.4 / 7.7
-//   1088 rows of 32000: bf16 29.7 / 25.3 / 24.6, fp32 35.3 / 32.3 / 32.5; of 2048: bf16 9.6 / 7.0 / 6.9; of 50000, fp32: 57.4 / 57.7 / 58.2
 template <typename T, int PER>
 static int launch_cluster_stats(const RowStatArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
   if (pl.NT == 8) HSD_CUDA_OK(hsd_launch(cluster_stats_kernel<T, PER, 8>, n * pl.C, kClThreads, 0, s, pl.C, true, a, pl.seg));
@@ -922,6 +904,9 @@ static int launch_cluster_stats(const RowStatArgs &a, const ClusterPlan &pl, int
   hsd_count_launches(1);
   return HSD_OK;
 }
+// us a call, GROUPS x WARPS = 1 x 16 / 2 x 8 / 3 x 8 (chunks of 32 KB; the middle one and 2 x 12 on chunks of 24 KB, behind it, are not built):
+//   a row a CTA, 32000: bf16 5.6 / 5.9 / 6.2, fp32 6.9 / 7.4 / 7.7
+//   1088 rows of 32000: bf16 29.7 / 25.3 / 24.6, fp32 35.3 / 32.3 / 32.5; of 2048: bf16 9.6 / 7.0 / 6.9; of 50000, fp32: 57.4 / 57.7 / 58.2
 // *marks: the statistics may be marks (kNoStat)
 static int launch_row_stats(const RowStatArgs &a, int dtype, cudaStream_t s, bool *marks) {
   const long long n_items = (long long)a.batch * (2 * a.t_max + 1);
@@ -933,8 +918,8 @@ static int launch_row_stats(const RowStatArgs &a, int dtype, cudaStream_t s, boo
   *marks = true;
   const int grid = (int)std::min<long long>(sm_count(), n_items);
   if (n_items <= grid)                                     // a row a CTA: all its warps on it
-    return dtype == HSD_F32 ? launch_row_stats_t<float, 1, 16, 32768>(a, grid, s) : launch_row_stats_t<__nv_bfloat16, 1, 16, 32768>(a, grid, s);
-  return dtype == HSD_F32 ? launch_row_stats_t<float, 3, 8, 32768>(a, grid, s) : launch_row_stats_t<__nv_bfloat16, 3, 8, 32768>(a, grid, s);
+    return dtype == HSD_F32 ? launch_row_stats_t<float, 1, 16>(a, grid, s) : launch_row_stats_t<__nv_bfloat16, 1, 16>(a, grid, s);
+  return dtype == HSD_F32 ? launch_row_stats_t<float, 3, 8>(a, grid, s) : launch_row_stats_t<__nv_bfloat16, 3, 8>(a, grid, s);
 }
 
 template <typename T, int PER, bool MARKS>

@@ -16,7 +16,7 @@ extern "C" int occupy(unsigned long long ns, void *stream) {
 // A verification (statistics at the front of `scratch`) whose statistics are computed by grids without their loader warps: the
 // computing warps' waits run out, nothing is in flight.
 template <typename T, int GROUPS, int WARPS> static int without_loaders(const hsd::RowStatArgs &r, int grid, cudaStream_t s) {
-  const auto kernel = hsd::row_stats_kernel<T, GROUPS, WARPS, 32768>;
+  const auto kernel = hsd::row_stats_kernel<T, GROUPS, WARPS>;
   const int smem = (int)hsd::kRsBytes + 128;
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return -1;
   kernel<<<grid, 32 * GROUPS * WARPS, smem, s>>>(r);
