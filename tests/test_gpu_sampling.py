@@ -121,8 +121,8 @@ def test_bad_arguments_are_rejected(lib):
                                          ("bf16", 32000, 14, 2), ("bf16", 32000, 15, 2),    # clusters of eight / of four
                                          ("bf16", 65538, 1, 1),      # 32 tokens a thread
                                          ("bf16", 1536, 2, 31),      # the most rows a sequence can have here
-                                         ("bf16", 512, 128, 16),     # one CTA a sequence, its 33 rows read twice, not staged
-                                         ("bf16", 2048, 16, 16), ("bf16", 2048, 64, 8),     # the fused kernel's side of the line, the clusters'
+                                         ("bf16", 512, 128, 16),     # one CTA a sequence, 33 rows each
+                                         ("bf16", 2048, 16, 16), ("bf16", 2048, 64, 8),     # statistics of many short rows
                                          ("bf16", 30001, 2, 1), ("fp32", 32769, 1, 8), ("fp32", 24001, 40, 1), ("bf16", 9000, 2, 0)])
 def test_cluster_decisions_match_oracle(lib, dtype, V, B, t):
     p, q = inputs.make_accept_logits(B, t, V, seed=V + 7 * t, device="cuda", dtype=dtype)
@@ -157,13 +157,19 @@ def test_cluster_draws_on_a_busy_gpu(lib, dtype, V, B):
         assert np.array_equal(x.cpu().numpy(), want[i % 4]), i
 
 
-@pytest.mark.parametrize("dtype,V,B,t,shift", [("bf16", 32000, 19, 4, 0), ("fp32", 32001, 14, 6, 0),  # more rows than SMs: two and three groups of warps
+# The ring of the streaming statistics takes 229376 bytes; up to 148 rows one group of warps a CTA, three past that; where a
+# cluster a row fits two rounds, clusters take the rows instead.
+@pytest.mark.parametrize("dtype,V,B,t,shift", [("bf16", 32000, 19, 4, 0), ("fp32", 32001, 14, 6, 0),  # more rows than SMs
                                                ("bf16", 50000, 16, 5, 0),      # rows of four chunks, CTAs whose third group has no row
                                                ("bf16", 16385, 9, 8, 3),       # a second chunk of a few elements, rows that begin anywhere
-                                               ("fp32", 57347, 1, 2, 0), ("fp32", 57341, 30, 2, 1),    # one element past the ring, the longest rows in it
-                                               ("bf16", 131080, 2, 1, 0),      # longer than the clusters of the decision take
-                                               ("bf16", 5, 40, 2, 1), ("fp32", 3, 64, 2, 0),   # rows without a whole vector
-                                               ("bf16", 64, 2, 40, 0), ("fp32", 40, 1, 600, 2)])       # more drafts than lanes, than threads
+                                               ("fp32", 57341, 30, 2, 1), ("fp32", 57345, 25, 3, 1),   # the longest rows in the ring; one element past it: twice through
+                                               ("bf16", 114700, 31, 2, 3),     # twice through the ring, three groups, rows that begin anywhere
+                                               ("fp32", 60000, 17, 2, 2),      # ... one group
+                                               ("fp32", 57347, 1, 2, 0),       # clusters
+                                               ("bf16", 131080, 2, 1, 0), ("fp32", 131081, 2, 1, 1),   # longer than the clusters of the decision take
+                                               ("bf16", 5, 60, 2, 1), ("fp32", 3, 64, 2, 0),   # rows without a whole vector
+                                               ("bf16", 5, 40, 2, 1), ("bf16", 64, 2, 40, 0),  # clusters; more drafts than lanes
+                                               ("fp32", 40, 1, 600, 2)])       # more drafts than threads, on the ring
 def test_row_statistics_and_decisions_match_oracle(lib, dtype, V, B, t, shift):
     def moved(x):                                                      # the same values from element `shift` of a buffer on
         buf = torch.empty(x.numel() + shift, dtype=x.dtype, device="cuda")
@@ -219,3 +225,65 @@ def test_draws_of_many_rows_match_oracle(lib, dtype, V, B):
     want = _oracle_draft(inputs.logits_to_numpy(q), 41, 2)
     got = [lib.hsd_draft_sample(q, 41, 2) for _ in range(3)]
     assert all(np.array_equal(x.cpu().numpy(), want) for x in got)
+
+
+def _without_weight(kind, row):
+    """A row of no finite weight."""
+    row.fill_(float("nan") if kind == "nan" else -float("inf"))
+    if kind == "+inf":
+        row.normal_()
+        row[row.numel() // 3] = float("inf")
+
+
+@pytest.mark.parametrize("kind", ["-inf", "nan", "+inf"])
+@pytest.mark.parametrize("dtype,V,B", [("bf16", 2048, 3), ("fp32", 32001, 5),      # clusters
+                                       ("bf16", 32000, 148), ("fp32", 9001, 149)])  # a CTA a row, in chunks and not
+def test_draws_of_rows_without_weight_give_no_token(lib, dtype, V, B, kind):
+    _, q = inputs.make_accept_logits(B, 1, V, seed=V, device="cuda", dtype=dtype)
+    want = _oracle_draft(inputs.logits_to_numpy(q), 3, 0)
+    for b in (0, B - 1):
+        _without_weight(kind, q[b, 0])
+        want[b] = -1
+    assert np.array_equal(lib.hsd_draft_sample(q, 3, 0).cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("kind", ["-inf", "nan", "+inf"])
+@pytest.mark.parametrize("dtype,V,B,t", [("bf16", 2048, 3, 2), ("fp32", 32001, 4, 3),          # statistics by clusters
+                                         ("bf16", 32000, 20, 2), ("fp32", 9001, 49, 3),        # streamed, one group and three
+                                         ("fp32", 57345, 30, 2), ("bf16", 131080, 6, 1)])      # twice through the ring; a CTA a decision
+def test_verifications_of_rows_without_weight(lib, dtype, V, B, t, kind):
+    p, q = inputs.make_accept_logits(B, t, V, seed=V, device="cuda", dtype=dtype)
+    q[:2] = p[:2, :t]                                                  # every draft accepted
+    x = lib.hsd_draft_sample(q, 5, 0)
+    for j in range(t):
+        x[2, j] = p[2, j].float().argmax()
+    p_np, q_np, x_np = inputs.logits_to_numpy(p), inputs.logits_to_numpy(q), x.cpu().numpy()
+    # sequence 0: no weight in its last draft's target row: the draft is rejected and nothing can be drawn.  Sequence 1: in the bonus
+    # row.  Sequence 2: in every draft row: q(x) = 0, every draft with weight in the target row is accepted.  For the oracle the first
+    # is a target row with all its weight on another token.
+    _without_weight(kind, p[0, t - 1])
+    p_np[0, t - 1] = -np.inf
+    p_np[0, t - 1, (x_np[0, t - 1] + 1) % V] = 0.0
+    _without_weight(kind, p[1, t])
+    for j in range(t):
+        _without_weight(kind, q[2, j])
+        q_np[2, j] = -np.inf
+        q_np[2, j, (x_np[2, j] + 1) % V] = 0.0
+    for serial in range(2):
+        out, n = lib.hsd_verify_level(1, p, q, x, 23, serial)
+        want_out, want_n = _oracle_verify(1, p_np, q_np, x_np, 23, serial)
+        assert want_n[:3].tolist() == [t - 1, t, t]
+        want_out[0, t - 1] = want_out[1, t] = -1
+        assert np.array_equal(n.cpu().numpy(), want_n) and np.array_equal(out.cpu().numpy(), want_out)
+
+
+def test_nan_logits_weigh_nothing(lib):
+    p, q = inputs.make_accept_logits(9, 2, 32001, seed=2, device="cuda", dtype="bf16")
+    p[:, :, 5::7] = float("nan")
+    q[:, :, 3::11] = float("nan")
+    x = lib.hsd_draft_sample(q, 5, 0)
+    p_np, q_np = (np.where(np.isnan(a), -np.inf, a) for a in (inputs.logits_to_numpy(p), inputs.logits_to_numpy(q)))
+    assert np.array_equal(x.cpu().numpy(), _oracle_draft(q_np, 5, 0))
+    out, n = lib.hsd_verify_level(1, p, q, x, 23, 0)
+    want_out, want_n = _oracle_verify(1, p_np, q_np, x.cpu().numpy(), 23, 0)
+    assert np.array_equal(n.cpu().numpy(), want_n) and np.array_equal(out.cpu().numpy(), want_out)
