@@ -25,7 +25,10 @@ template <typename D> static DescList<D> desc_list(const D *desc, int n, bool on
 }
 
 // ------------------------------------------------------------------------------ draft sampling
-// One block per row: token = inverse-CDF sample of softmax(row) with the purpose-0 uniform.
+// One block per row: token = inverse-CDF sample of softmax(row) with the purpose-0 uniform.  The kernel behind it does not start
+// early: its CTAs would take the places that this one's last round frees, two on some SMs and none on others.  200 / 297 / 2000
+// fp32 rows of 128256 tokens in a row of calls: 81 / 144 / 744 us; with early starts 115 / 174 / 835, half of that because the
+// descriptor was kept in registers through the row.
 template <typename T>
 __global__ void __launch_bounds__(kSampleThreads)
 draft_sample_kernel(const T *__restrict__ logits, int V, const __grid_constant__ DescList<SampleRow> desc,
@@ -33,20 +36,24 @@ draft_sample_kernel(const T *__restrict__ logits, int V, const __grid_constant__
   __shared__ float shf[32];
   __shared__ u64 sh64[34];
   chain_wait();
-  chain_next();
-  SampleRow d;
-  if (desc.given()) {
-    d = desc.at(blockIdx.x);
-  } else {
+  auto descriptor = [&]() {
+    SampleRow d;
+    if (desc.given()) return desc.at(blockIdx.x);
     d.logit_row = blockIdx.x;
     d.out_index = blockIdx.x;
     d.j = blockIdx.x % regular_rows;
     d.seq = blockIdx.x / regular_rows;
     d.serial = regular_serial;
     d.level = 0;
+    return d;
+  };
+  const T *row;
+  u32 U;
+  {
+    const SampleRow d = descriptor();
+    row = logits + (size_t)d.logit_row * V;
+    U = uniform24(seed, d.j, d.serial, d.level, PURPOSE_DRAFT, d.seq);
   }
-  const T *row = logits + (size_t)d.logit_row * V;
-  u32 U = uniform24(seed, d.j, d.serial, d.level, PURPOSE_DRAFT, d.seq);
   int tok;
   if (sizeof(T) == 2 && chunk_layout_ok(row, V, blockDim.x)) {
     const int k0 = threadIdx.x * kChunkTokens;
@@ -58,6 +65,7 @@ draft_sample_kernel(const T *__restrict__ logits, int V, const __grid_constant__
     tok = block_inverse_cdf(V, U, [&](int k) { return (u64)exp_weight(to_f32(row[k]), m); }, sh64, nullptr);
   }
   if (threadIdx.x == 0) {
+    const SampleRow d = descriptor();
     out[d.out_index] = tok;
     if (mirror.token) mirror.token[(size_t)d.seq * mirror.stride + d.j] = tok;
   }
