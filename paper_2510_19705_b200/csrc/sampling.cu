@@ -420,7 +420,7 @@ gave_up:
 // scratch in global memory; statistics and decisions meet in the RowStats there.
 // A warp owns consecutive tokens; lane and unit index are interleaved (unit = 4 bytes: a bf16 pair or an fp32 value;
 // 2 bytes when rows of odd length leave bf16 pairs unaligned), so loads are whole lines whatever the row's alignment.
-constexpr int kClThreads = 512, kClWarps = kClThreads / 32, kClMaxC = 8;
+constexpr int kClThreads = 512, kClMaxC = 8;
 
 template <typename T, int PER> struct ClUnit;              // PER tokens of one load
 template <> struct ClUnit<float, 1> {
@@ -472,11 +472,11 @@ __device__ __forceinline__ void cl_store(u32 addr, u32 v) { asm volatile("st.sha
 __device__ __forceinline__ void cl_store(u32 addr, u64 v) { asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory"); }
 // Inverse CDF within a CTA whose weights pass the threshold: the warp, then the unit, then the token whose inclusive sum
 // does.  w: the thread's weights, sums: the warps' totals, before: the sum of the CTAs in front.
-template <int NT, int PER, class W, class Emit>
+template <int WARPS, int NT, int PER, class W, class Emit>
 __device__ __forceinline__ void cl_find_token(const W (&w)[NT], u64 tau, u64 before, const u64 *sums, int k_lane, Emit emit) {
   constexpr int NU = NT / PER;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  u64 mine = lane < kClWarps ? sums[lane] : 0ull;                  // every warp finds the owning one for itself
+  u64 mine = lane < WARPS ? sums[lane] : 0ull;                  // every warp finds the owning one for itself
   u64 incl = mine;
   for (int o = 1; o < 32; o <<= 1) {
     const u64 v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
@@ -532,7 +532,7 @@ __device__ __forceinline__ void cl_units(const T *row, int k_lane, int tok_end, 
     v[u] = k < tok_end ? __ldg(reinterpret_cast<const typename ClUnit<T, PER>::raw *>(row + k)) : ClUnit<T, PER>::none();
   }
 }
-template <int N> __device__ __forceinline__ float cl_max(const float (&f)[N], int *wmax /*[kClWarps]*/, int *cmax /*[kClMaxC]*/, u32 rank, u32 C) {
+template <int WARPS, int N> __device__ __forceinline__ float cl_max(const float (&f)[N], int *wmax /*[WARPS]*/, int *cmax /*[kClMaxC]*/, u32 rank, u32 C) {
   float m = -INFINITY;
 #pragma unroll
   for (int e = 0; e < N; ++e) m = fmaxf(m, f[e]);
@@ -541,7 +541,7 @@ template <int N> __device__ __forceinline__ float cl_max(const float (&f)[N], in
   __syncthreads();
   cl_wait();                                                       // every CTA of the cluster has started
   if (warp == 0) {
-    const int all = __reduce_max_sync(0xFFFFFFFFu, wmax[lane & (kClWarps - 1)]);
+    const int all = __reduce_max_sync(0xFFFFFFFFu, wmax[lane & (WARPS - 1)]);
     if (lane < (int)C) cl_store(cl_map(&cmax[rank], (u32)lane), (u32)all);
   }
   cl_sync();
@@ -549,13 +549,13 @@ template <int N> __device__ __forceinline__ float cl_max(const float (&f)[N], in
   for (u32 c = 1; c < C; ++c) top = max(top, cmax[c]);
   return order_value(top);
 }
-template <bool ALL> __device__ __forceinline__ void cl_total(u64 local, u64 *wsum /*[kClWarps]*/, u64 *csum /*[kClMaxC]*/, u32 rank, u32 C) {
+template <int WARPS, bool ALL> __device__ __forceinline__ void cl_total(u64 local, u64 *wsum /*[WARPS]*/, u64 *csum /*[kClMaxC]*/, u32 rank, u32 C) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u64 s = warp_sum54(local);
   if (lane == 0) wsum[warp] = s;
   __syncthreads();
   if (warp == 0) {
-    u64 t = lane < kClWarps ? wsum[lane] : 0ull;
+    u64 t = lane < WARPS ? wsum[lane] : 0ull;
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
     if (lane < (ALL ? (int)C : 1)) cl_store(cl_map(&csum[rank], (u32)lane), t);
   }
@@ -563,11 +563,11 @@ template <bool ALL> __device__ __forceinline__ void cl_total(u64 local, u64 *wsu
 }
 
 // Level 0's draw: token = inverse-CDF sample of softmax(row) with the purpose-0 uniform.  Two CTAs per SM.
-template <typename T, int PER, int NT>
-__global__ void __launch_bounds__(kClThreads, 2) cluster_draw_kernel(const __grid_constant__ ClusterArgs a) {
-  constexpr int NU = NT / PER;
-  __shared__ int wmax[kClWarps], cmax[kClMaxC];                    // order keys
-  __shared__ u64 wsum[kClWarps], csum[kClMaxC];
+template <typename T, int PER, int NT, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) cluster_draw_kernel(const __grid_constant__ ClusterArgs a) {
+  constexpr int NU = NT / PER, WARPS = THREADS / 32;
+  __shared__ int wmax[WARPS], cmax[kClMaxC];                    // order keys
+  __shared__ u64 wsum[WARPS], csum[kClMaxC];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const u32 rank = cl_rank(), C = cl_size();
   const int b = (int)cl_id();
@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_draw_kernel(const __gri
   float f[NT];
 #pragma unroll
   for (int u = 0; u < NU; ++u) ClUnit<T, PER>::get(v[u], f + u * PER);
-  const float m = cl_max(f, wmax, cmax, rank, C);
+  const float m = cl_max<WARPS>(f, wmax, cmax, rank, C);
   u32 w[NT];
   u64 local = 0, total = 0, before = 0;
 #pragma unroll
@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_draw_kernel(const __gri
     exp_weight2(f[e], f[e + 1], m, w[e], w[e + 1]);
     local += (u64)w[e] + (u64)w[e + 1];
   }
-  cl_total<true>(local, wsum, csum, rank, C);
+  cl_total<WARPS, true>(local, wsum, csum, rank, C);
   for (u32 c = 0; c < C; ++c) {
     if (c < rank) before += csum[c];
     total += csum[c];
@@ -605,17 +605,17 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_draw_kernel(const __gri
   if (total == 0) {                                                // non-finite logits: no token
     if (rank == 0 && tid == 0) emit(-1);
   } else if (tau >= before && tau < before + csum[rank]) {
-    cl_find_token<NT, PER>(w, tau, before, wsum, k_lane, emit);
+    cl_find_token<WARPS, NT, PER>(w, tau, before, wsum, k_lane, emit);
   }
 }
 
 // The statistics of few rows: a cluster a row, each CTA consecutive tokens of it in registers; the maximum and the total cross the
 // cluster in one exchange each.  7 rows of 32000 bf16 tokens: 3.3 us (a CTA a row that takes them through its ring: 5.8).
-template <typename T, int PER, int NT>
-__global__ void __launch_bounds__(kClThreads, 2) cluster_stats_kernel(const __grid_constant__ RowStatArgs a, int seg) {
-  constexpr int NU = NT / PER;
-  __shared__ int wmax[kClWarps], cmax[kClMaxC];                    // order keys
-  __shared__ u64 wsum[kClWarps], csum[kClMaxC];
+template <typename T, int PER, int NT, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) cluster_stats_kernel(const __grid_constant__ RowStatArgs a, int seg) {
+  constexpr int NU = NT / PER, WARPS = THREADS / 32;
+  __shared__ int wmax[WARPS], cmax[kClMaxC];                    // order keys
+  __shared__ u64 wsum[WARPS], csum[kClMaxC];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const u32 rank = cl_rank(), C = cl_size();
   cl_arrive();                                                     // (the wait is in front of the first store to a peer)
@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_stats_kernel(const __gr
   float f[NT];
 #pragma unroll
   for (int u = 0; u < NU; ++u) ClUnit<T, PER>::get(v[u], f + u * PER);
-  const float m = cl_max(f, wmax, cmax, rank, C);
+  const float m = cl_max<WARPS>(f, wmax, cmax, rank, C);
   u64 local = 0;
 #pragma unroll
   for (int e = 0; e < NT; e += 2) {
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_stats_kernel(const __gr
     exp_weight2(f[e], f[e + 1], m, e0, e1);
     local += (u64)e0 + (u64)e1;
   }
-  cl_total<false>(local, wsum, csum, rank, C);
+  cl_total<WARPS, false>(local, wsum, csum, rank, C);
   if (rank == 0 && tid == 0) {
     RowStat st;
     st.m = m; st.S = 0;
@@ -662,11 +662,11 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_stats_kernel(const __gr
 // 32 tokens a thread (calls whose clusters are of one or two CTAs): their 64-bit weights go past 128 registers, 84 to 144 bytes spill.
 // MARKS: the statistics may be marks; looking for them costs 0.1 us (one sequence of three drafts: 7.39, with them 7.49), which
 // cluster_stats_kernel, without a bounded wait, spares.
-template <typename T, int PER, int NT, bool MARKS>
-__global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __grid_constant__ ClusterArgs a, const RowStat *stats) {
+template <typename T, int PER, int NT, int THREADS, bool MARKS>
+__global__ void __launch_bounds__(THREADS, kClThreads / THREADS) cluster_decide_kernel(const __grid_constant__ ClusterArgs a, const RowStat *stats) {
   typedef typename ClUnit<T, PER>::raw raw_t;
-  constexpr int NU = NT / PER;
-  __shared__ u64 wsum[2][kClWarps], csum[2][kClMaxC];              // [residual, the verifier's row]
+  constexpr int NU = NT / PER, WARPS = THREADS / 32;
+  __shared__ u64 wsum[2][WARPS], csum[2][kClMaxC];              // [residual, the verifier's row]
   __shared__ int sh_n, sh_none;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const u32 rank = cl_rank(), C = cl_size();
@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
   __syncthreads();
   chain_wait();
   chain_next();
-  for (int j = tid; j < t; j += kClThreads) {
+  for (int j = tid; j < t; j += THREADS) {
     if (j != tid) drafted(j);
     const RowStat s = stat(sp + j), r = stat(sq + j);
     if (MARKS && (s.S == kNoStat || r.S == kNoStat)) sh_none = 1;
@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
     if (!running) cl_wait();
     running = true;
     if (warp == 0) {
-      u64 c = lane < kClWarps ? wsum[src][lane] : 0ull;
+      u64 c = lane < WARPS ? wsum[src][lane] : 0ull;
       for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
       if (lane < (int)C) cl_store(cl_map(&csum[src][rank], (u32)lane), c);
     }
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
   if (total == 0) {                                                // non-finite logits or no statistics: no token
     if (rank == 0 && tid == 0) emit(-1);
   } else if (tau >= before && tau < before + csum[src][rank]) {
-    cl_find_token<NT, PER>(w, tau, before, wsum[src], k_lane, emit);
+    cl_find_token<WARPS, NT, PER>(w, tau, before, wsum[src], k_lane, emit);
   }
   if (rank == 0) {
     const int n_out = MARKS && sh_none ? kNoDecision : n;
@@ -801,13 +801,14 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_decide_kernel(const __g
       if (a.mirror.status && b == 0) *a.mirror.status = __ldcg(a.mirror.status_src);
     }
     if (a.out_tokens)
-      for (int j = tid; j <= a.t_max; j += kClThreads)
+      for (int j = tid; j <= a.t_max; j += THREADS)
         if (j != n) a.out_tokens[(size_t)b * (a.t_max + 1) + j] = j < n_out ? a.tokens[d.tok_off + j] : -1;
   }
 }
 
-// Cluster size, tokens a thread and tokens a CTA of a call with n clusters; false if the rows are too long.  `two`: two CTAs per SM.
-struct ClusterPlan { int C, NT, per, seg; };
+// Cluster size, tokens a thread, tokens and threads of a CTA of a call with n clusters; false if the rows are too long.  `two`: 1024
+// threads' worth of CTAs per SM (decisions: 512).
+struct ClusterPlan { int C, NT, per, seg, threads; };
 constexpr int kClEights = 14;                     // clusters of eight that run at once (one CTA per SM) on the GPU that was measured: speed only
 static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, bool two, ClusterPlan *pl) {
   pl->per = (dtype == HSD_BF16 && V % 2 == 0 && ((uintptr_t)p & 3) == 0 && ((uintptr_t)q & 3) == 0) ? 2 : 1;
@@ -821,10 +822,14 @@ static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, 
   if (seg > most) return false;
   pl->C = C;
   pl->seg = seg;
-  pl->NT = seg <= 8 * kClThreads ? 8 : seg <= 16 * kClThreads ? 16 : 32;
+  // rows of up to 1024 and 2048 tokens, eight a thread: fewer warps to meet, more rows on an SM
+  pl->threads = seg <= 1024 ? 128 : seg <= 2048 ? 256 : kClThreads;
+  pl->NT = seg <= 8 * pl->threads ? 8 : seg <= 16 * pl->threads ? 16 : 32;
   return true;
 }
-// Where clusters are the faster ones (us a call in a row of calls, clusters / other path).
+// Where clusters are the faster ones (us a call in a row of calls, clusters / other path).  Rows of up to 2048 tokens, in CTAs of 128 or
+// 256 threads: always.  Against CTAs of 512 threads and, past two rounds of them, the other path: verifications, bf16, 513 tokens, 1 x 3 8.1 ->
+// 7.2, 64 x 8 13.8 -> 10.9, 2000 x 1 104 -> 40; 2048, 64 x 8 12.4 -> 10.8; draws of 513, 1 row 3.5 -> 3.05, 2000 27 -> 8.6, of 2048 3.2 -> 2.8, 24.4 -> 13.3.
 //   statistics (the whole verification), while the clusters run in one round: 32000 bf16, 7 rows 8.4 / 10.8, 66 rows 10.1 / 11.5, 88 rows (in
 //     two rounds) 12.9 / 11.5; fp32, 7 rows 9.2 / 12.9, 66: 11.1 / 13.3, 88: 13.8 / 13.5; 16000 bf16, 132 rows 10.1 / 10.0, 176 (two) 11.9 / 11.6; 2048:
 //     8.0 / 8.0, 176 rows 8.8 / 8.7; 45001 bf16, 33 rows 13.5 / 16.1, 44 (two) 16.4 / 16.2.
@@ -833,17 +838,21 @@ static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, 
 //     fp32 32000: 4.1 / 26, 64 rows 6.6 / 28; 8000: 4.1 / 6.1; 2048: 3.9 / 3.9.  In more rounds, chunked: 32000, 100 rows 9.4 / 11.1, 148: 12.5 / 11.1
 //     (a row a CTA then), 200: 14.6 / 20.5, 512: 37 / 40, 16000, 512: 18 / 35; others: fp32 9001, 256: 12 / 9.1, 16000, 256: 11 / 16.9 (two CTAs a row),
 //     20000, 148: 13.4 / 10.7, 32000, 100: 10.2 / 28, 512: 41 / 105; 8000, 512: 10.7 / 15.9; bf16 32001, 256: 21 / 38.
-static bool cluster_pays_stats(const ClusterPlan &pl, long long rows) { return pl.C * rows <= 2 * kMeasuredSMs; }
+static bool cluster_pays_stats(const ClusterPlan &pl, long long rows) { return pl.threads < kClThreads || pl.C * rows <= 2 * kMeasuredSMs; }
 static bool cluster_pays_draw(const ClusterPlan &pl, int V, int n, bool chunked) {
-  if (pl.C * n <= 2 * kMeasuredSMs) return true;
+  if (pl.threads < kClThreads || pl.C * n <= 2 * kMeasuredSMs) return true;
   if (chunked) return n > kMeasuredSMs || pl.C * n <= 3 * kMeasuredSMs;
   return V > 26000 || V <= 8192 || (V > 13500 && pl.C == 2);
 }
 
 template <typename T, int PER>
 static int launch_cluster_draw_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
-  if (pl.NT == 8) HSD_CUDA_OK(hsd_launch(cluster_draw_kernel<T, PER, 8>, n * pl.C, kClThreads, 0, s, pl.C, true, a));
-  else HSD_CUDA_OK(hsd_launch(cluster_draw_kernel<T, PER, 16>, n * pl.C, kClThreads, 0, s, pl.C, true, a));
+  const int grid = n * pl.C;
+  auto go = [&](auto kernel, int threads) { return hsd_launch(kernel, grid, threads, 0, s, pl.C, true, a); };
+  HSD_CUDA_OK(pl.threads == 128   ? go(cluster_draw_kernel<T, PER, 8, 128>, 128)
+              : pl.threads == 256 ? go(cluster_draw_kernel<T, PER, 8, 256>, 256)
+              : pl.NT == 8        ? go(cluster_draw_kernel<T, PER, 8, kClThreads>, kClThreads)
+                                  : go(cluster_draw_kernel<T, PER, 16, kClThreads>, kClThreads));
   hsd_count_launches(1);
   return hsd_launch_status();
 }
@@ -907,8 +916,12 @@ static int launch_row_stats_t(const RowStatArgs &a, int grid, cudaStream_t s) {
 }
 template <typename T, int PER>
 static int launch_cluster_stats(const RowStatArgs &a, const ClusterPlan &pl, int n, cudaStream_t s) {
-  if (pl.NT == 8) HSD_CUDA_OK(hsd_launch(cluster_stats_kernel<T, PER, 8>, n * pl.C, kClThreads, 0, s, pl.C, true, a, pl.seg));
-  else HSD_CUDA_OK(hsd_launch(cluster_stats_kernel<T, PER, 16>, n * pl.C, kClThreads, 0, s, pl.C, true, a, pl.seg));
+  const int grid = n * pl.C;
+  auto go = [&](auto kernel, int threads) { return hsd_launch(kernel, grid, threads, 0, s, pl.C, true, a, pl.seg); };
+  HSD_CUDA_OK(pl.threads == 128   ? go(cluster_stats_kernel<T, PER, 8, 128>, 128)
+              : pl.threads == 256 ? go(cluster_stats_kernel<T, PER, 8, 256>, 256)
+              : pl.NT == 8        ? go(cluster_stats_kernel<T, PER, 8, kClThreads>, kClThreads)
+                                  : go(cluster_stats_kernel<T, PER, 16, kClThreads>, kClThreads));
   hsd_count_launches(1);
   return HSD_OK;
 }
@@ -919,7 +932,7 @@ static int launch_cluster_stats(const RowStatArgs &a, const ClusterPlan &pl, int
 static int launch_row_stats(const RowStatArgs &a, int dtype, cudaStream_t s, bool *marks) {
   const long long n_items = (long long)a.batch * (2 * a.t_max + 1);
   ClusterPlan pl;
-  if (n_items <= 2 * kMeasuredSMs && cluster_plan(a.p, a.q, dtype, a.V, (int)n_items, true, &pl) && cluster_pays_stats(pl, n_items)) {
+  if (n_items <= 0x7FFFFFFFll / kClMaxC && cluster_plan(a.p, a.q, dtype, a.V, (int)n_items, true, &pl) && cluster_pays_stats(pl, n_items)) {
     if (dtype == HSD_F32) return launch_cluster_stats<float, 1>(a, pl, (int)n_items, s);
     return pl.per == 2 ? launch_cluster_stats<__nv_bfloat16, 2>(a, pl, (int)n_items, s) : launch_cluster_stats<__nv_bfloat16, 1>(a, pl, (int)n_items, s);
   }
@@ -933,9 +946,14 @@ static int launch_row_stats(const RowStatArgs &a, int dtype, cudaStream_t s, boo
 template <typename T, int PER, bool MARKS>
 static int launch_decide_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, const RowStat *stats, cudaStream_t s) {
   const int grid = n * pl.C;
-  if (pl.NT == 8) HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 8, MARKS>, grid, kClThreads, 0, s, pl.C, true, a, stats));
-  else if (pl.NT == 16) HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 16, MARKS>, grid, kClThreads, 0, s, pl.C, true, a, stats));
-  else HSD_CUDA_OK(hsd_launch(cluster_decide_kernel<T, PER, 32, MARKS>, grid, kClThreads, 0, s, pl.C, true, a, stats));
+  auto go = [&](auto kernel, int threads) { return hsd_launch(kernel, grid, threads, 0, s, pl.C, true, a, stats); };
+  cudaError_t e;
+  if (!MARKS && pl.threads == 128) e = go(cluster_decide_kernel<T, PER, 8, 128, false>, 128);    // (such rows' statistics are the clusters')
+  else if (!MARKS && pl.threads == 256 && pl.NT == 8) e = go(cluster_decide_kernel<T, PER, 8, 256, false>, 256);
+  else if (pl.NT == 8) e = go(cluster_decide_kernel<T, PER, 8, kClThreads, MARKS>, kClThreads);
+  else if (pl.NT == 16) e = go(cluster_decide_kernel<T, PER, 16, kClThreads, MARKS>, kClThreads);
+  else e = go(cluster_decide_kernel<T, PER, 32, kClThreads, MARKS>, kClThreads);
+  HSD_CUDA_OK(e);
   hsd_count_launches(1);
   return hsd_launch_status();
 }

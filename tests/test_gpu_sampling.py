@@ -157,8 +157,8 @@ def test_cluster_draws_on_a_busy_gpu(lib, dtype, V, B):
         assert np.array_equal(x.cpu().numpy(), want[i % 4]), i
 
 
-# The ring of the streaming statistics takes 229376 bytes; up to 148 rows one group of warps a CTA, three past that; where a
-# cluster a row fits two rounds, clusters take the rows instead.
+# Rows of up to 2048 tokens are taken by CTAs of 128 or 256 threads, longer ones by clusters where a cluster a row fits two rounds, else by
+# the streaming kernel: its ring holds 229376 bytes; up to 148 rows one group of warps a CTA, three past that.
 @pytest.mark.parametrize("dtype,V,B,t,shift", [("bf16", 32000, 19, 4, 0), ("fp32", 32001, 14, 6, 0),  # more rows than SMs
                                                ("bf16", 50000, 16, 5, 0),      # rows of four chunks, CTAs whose third group has no row
                                                ("bf16", 16385, 9, 8, 3),       # a second chunk of a few elements, rows that begin anywhere
@@ -167,9 +167,10 @@ def test_cluster_draws_on_a_busy_gpu(lib, dtype, V, B):
                                                ("fp32", 60000, 17, 2, 2),      # ... one group
                                                ("fp32", 57347, 1, 2, 0),       # clusters
                                                ("bf16", 131080, 2, 1, 0), ("fp32", 131081, 2, 1, 1),   # longer than the clusters of the decision take
-                                               ("bf16", 5, 60, 2, 1), ("fp32", 3, 64, 2, 0),   # rows without a whole vector
-                                               ("bf16", 5, 40, 2, 1), ("bf16", 64, 2, 40, 0),  # clusters; more drafts than lanes
-                                               ("fp32", 40, 1, 600, 2)])       # more drafts than threads, on the ring
+                                               ("bf16", 5, 60, 2, 1), ("fp32", 3, 64, 2, 0), ("bf16", 64, 2, 40, 0),     # 128 threads; more drafts than lanes,
+                                               ("fp32", 40, 1, 600, 2), ("bf16", 1024, 170, 3, 0), ("fp32", 1024, 3, 2, 1),   # ... than threads; every token
+                                               ("bf16", 1025, 90, 3, 1), ("fp32", 1025, 2, 1, 0), ("bf16", 2048, 33, 4, 0),    # 256 threads
+                                               ("bf16", 2049, 100, 1, 1), ("fp32", 2049, 60, 2, 0)])     # the shortest rows on the ring
 def test_row_statistics_and_decisions_match_oracle(lib, dtype, V, B, t, shift):
     def moved(x):                                                      # the same values from element `shift` of a buffer on
         buf = torch.empty(x.numel() + shift, dtype=x.dtype, device="cuda")
@@ -218,6 +219,7 @@ def test_verifications_in_a_captured_graph_and_back_to_back(lib):
 
 
 @pytest.mark.parametrize("dtype,V,B", [("bf16", 2048, 3), ("fp32", 513, 300),      # one CTA a row; more rows than run at once
+                                       ("bf16", 1024, 2400), ("fp32", 1024, 5), ("bf16", 1025, 301), ("fp32", 2048, 3), ("fp32", 2049, 3),    # 128, 256, 512 threads
                                        ("bf16", 32000, 112), ("bf16", 32000, 148), ("fp32", 32001, 75),   # several rounds of clusters, a row a CTA
                                        ("fp32", 9001, 149), ("bf16", 8190, 297)])
 def test_draws_of_many_rows_match_oracle(lib, dtype, V, B):
