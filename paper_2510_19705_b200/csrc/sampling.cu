@@ -89,12 +89,14 @@ template <> struct StatVec<float> {
   }
 };
 
-// ------------------------------------------------------------------------------ decision, vocabularies past 131072 tokens
+// ------------------------------------------------------------------------------ decision by a CTA: vocabularies past 131072 tokens, many sequences
 // One block per sequence: accept tests for all positions (each with its own counter-addressed
 // uniform, so the parallel form equals Algorithm 2's sequential loop with break), n = index of the
 // first rejection, then the final draw from the residual of row n (n < t) or from target row t.
-template <typename T>
-__global__ void __launch_bounds__(kSampleThreads)
+// Launched in the ordinary way: started early, beside the streaming statistics' shared memory, it would have no first-level cache to
+// read its rows through (16 sequences of 8 drafts, 151936 tokens: 336 us instead of 136).
+template <typename T, int CTAS>
+__global__ void __launch_bounds__(kSampleThreads, CTAS)
 decide_kernel(const T *__restrict__ p_logits, const T *__restrict__ q_logits, int32_t *__restrict__ tokens, int V,
               int t_max, const __grid_constant__ DescList<VerifySeq> desc, int regular_t, u32 regular_serial, u32 regular_level,
               const RowStat *__restrict__ stats, u64 seed, int32_t *__restrict__ out_tokens /*[B, t_max+1] or null*/,
@@ -824,12 +826,15 @@ static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, 
   pl->seg = seg;
   // rows of up to 1024 and 2048 tokens, eight a thread: fewer warps to meet, more rows on an SM
   pl->threads = seg <= 1024 ? 128 : seg <= 2048 ? 256 : kClThreads;
+  // decisions of more sequences than SMs: two CTAs a SM, of 16 or 32 tokens a thread (us a verification of 4000 bf16 tokens, 512 / 256
+  // threads: 148 x 1 10.3 / 10.8, 200 x 1 15.5 / 12.2, 2000 x 3 151 / 118; 8000: 200 x 1 19.3 / 17.0, 2000 x 3 196 / 165)
+  if (!two && n > kMeasuredSMs && seg <= 8192 && pl->threads == kClThreads) pl->threads = 256;
   pl->NT = seg <= 8 * pl->threads ? 8 : seg <= 16 * pl->threads ? 16 : 32;
   return true;
 }
 // Where clusters are the faster ones (us a call in a row of calls, clusters / other path).  Rows of up to 2048 tokens, in CTAs of 128 or
-// 256 threads: always.  Against CTAs of 512 threads and, past two rounds of them, the other path: verifications, bf16, 513 tokens, 1 x 3 8.1 ->
-// 7.2, 64 x 8 13.8 -> 10.9, 2000 x 1 104 -> 40; 2048, 64 x 8 12.4 -> 10.8; draws of 513, 1 row 3.5 -> 3.05, 2000 27 -> 8.6, of 2048 3.2 -> 2.8, 24.4 -> 13.3.
+// 256 threads: always.  Against CTAs of 512 threads and, past two rounds of them, the other path: verifications, bf16, 513 tokens, 1 x 3 8.3 ->
+// 7.1, 64 x 8 13.9 -> 9.0, 2000 x 1 103 -> 32; 2048, 64 x 8 12.4 -> 10.5; draws of 513, 1 row 3.5 -> 3.05, 2000 27 -> 8.6, of 2048 3.2 -> 2.8, 24.4 -> 13.3.
 //   statistics (the whole verification), while the clusters run in one round: 32000 bf16, 7 rows 8.4 / 10.8, 66 rows 10.1 / 11.5, 88 rows (in
 //     two rounds) 12.9 / 11.5; fp32, 7 rows 9.2 / 12.9, 66: 11.1 / 13.3, 88: 13.8 / 13.5; 16000 bf16, 132 rows 10.1 / 10.0, 176 (two) 11.9 / 11.6; 2048:
 //     8.0 / 8.0, 176 rows 8.8 / 8.7; 45001 bf16, 33 rows 13.5 / 16.1, 44 (two) 16.4 / 16.2.
@@ -839,6 +844,13 @@ static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, 
 //     (a row a CTA then), 200: 14.6 / 20.5, 512: 37 / 40, 16000, 512: 18 / 35; others: fp32 9001, 256: 12 / 9.1, 16000, 256: 11 / 16.9 (two CTAs a row),
 //     20000, 148: 13.4 / 10.7, 32000, 100: 10.2 / 28, 512: 41 / 105; 8000, 512: 10.7 / 15.9; bf16 32001, 256: 21 / 38.
 static bool cluster_pays_stats(const ClusterPlan &pl, long long rows) { return pl.threads < kClThreads || pl.C * rows <= 2 * kMeasuredSMs; }
+//   decisions of more sequences than SMs by decide_kernel, two CTAs of 1024 threads a SM that read their rows through the first-level
+//     cache (the whole verification, clusters / decide_kernel): 12000 bf16 200 x 1 25.0 / 25.5; 16385, 200 x 0 29.7 / 16.9, 2000 x 3 655 / 293;
+//     24000, 149 x 3 42.3 / 44.5, 300 x 0 36 / 25, 2000 x 3 472 / 343, fp32 300 x 0 47 / 31, 2000 x 3 581 / 413; 32000 bf16, 300 x 1 60 / 66, fp32 50 / 90.  Up
+//     to 8192 tokens against 256 threads: fp32 8000, 200 x 1 20.7 / 22.5, 300 x 0 19.0 / 16.3, 600 x 3 68 / 64, bf16 600 x 3 52.8 / 56.8.
+static bool cta_pays_decide(int dtype, int V, int n) {
+  return V <= 8192 ? dtype == HSD_F32 && V > 4096 && n > 2 * kMeasuredSMs : V <= 24576 && n > kMeasuredSMs;
+}
 static bool cluster_pays_draw(const ClusterPlan &pl, int V, int n, bool chunked) {
   if (pl.threads < kClThreads || pl.C * n <= 2 * kMeasuredSMs) return true;
   if (chunked) return n > kMeasuredSMs || pl.C * n <= 3 * kMeasuredSMs;
@@ -950,6 +962,8 @@ static int launch_decide_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, 
   cudaError_t e;
   if (!MARKS && pl.threads == 128) e = go(cluster_decide_kernel<T, PER, 8, 128, false>, 128);    // (such rows' statistics are the clusters')
   else if (!MARKS && pl.threads == 256 && pl.NT == 8) e = go(cluster_decide_kernel<T, PER, 8, 256, false>, 256);
+  else if (pl.threads == 256 && pl.NT == 16) e = go(cluster_decide_kernel<T, PER, 16, 256, MARKS>, 256);
+  else if (pl.threads == 256 && pl.NT == 32) e = go(cluster_decide_kernel<T, PER, 32, 256, MARKS>, 256);
   else if (pl.NT == 8) e = go(cluster_decide_kernel<T, PER, 8, kClThreads, MARKS>, kClThreads);
   else if (pl.NT == 16) e = go(cluster_decide_kernel<T, PER, 16, kClThreads, MARKS>, kClThreads);
   else e = go(cluster_decide_kernel<T, PER, 32, kClThreads, MARKS>, kClThreads);
@@ -958,8 +972,8 @@ static int launch_decide_nt(const ClusterArgs &a, const ClusterPlan &pl, int n, 
   return hsd_launch_status();
 }
 
-template <typename T> static int launch_decide_long(const ClusterArgs &a, int batch, const RowStat *stats, cudaStream_t s) {
-  decide_kernel<T><<<batch, kSampleThreads, 0, s>>>((const T *)a.p, (const T *)a.q, a.tokens, a.V, a.t_max, a.desc, a.regular_t, a.regular_serial,
+template <typename T, int CTAS> static int launch_decide_long(const ClusterArgs &a, int batch, const RowStat *stats, cudaStream_t s) {
+  decide_kernel<T, CTAS><<<batch, kSampleThreads, 0, s>>>((const T *)a.p, (const T *)a.q, a.tokens, a.V, a.t_max, a.desc, a.regular_t, a.regular_serial,
                                                     a.regular_level, stats, a.seed, a.out_tokens, a.out_n, a.write_in_place, a.coin24, a.mirror);
   hsd_count_launches(1);
   return hsd_launch_status();
@@ -971,7 +985,9 @@ template <bool MARKS> static int launch_decide(const ClusterArgs &a, const Clust
 static int launch_decisions(ClusterArgs a, int dtype, int batch, const RowStat *stats, bool marks, cudaStream_t s) {
   ClusterPlan pl;
   if (!cluster_plan(a.p, a.q, dtype, a.V, batch, false, &pl))      // rows of more than 131072 tokens
-    return dtype == HSD_BF16 ? launch_decide_long<__nv_bfloat16>(a, batch, stats, s) : launch_decide_long<float>(a, batch, stats, s);
+    return dtype == HSD_BF16 ? launch_decide_long<__nv_bfloat16, 1>(a, batch, stats, s) : launch_decide_long<float, 1>(a, batch, stats, s);
+  if (cta_pays_decide(dtype, a.V, batch))
+    return dtype == HSD_BF16 ? launch_decide_long<__nv_bfloat16, 2>(a, batch, stats, s) : launch_decide_long<float, 2>(a, batch, stats, s);
   a.seg = pl.seg;
   return marks ? launch_decide<true>(a, pl, dtype, batch, stats, s) : launch_decide<false>(a, pl, dtype, batch, stats, s);
 }

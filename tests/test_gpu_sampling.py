@@ -289,3 +289,17 @@ def test_nan_logits_weigh_nothing(lib):
     out, n = lib.hsd_verify_level(1, p, q, x, 23, 0)
     want_out, want_n = _oracle_verify(1, p_np, q_np, x.cpu().numpy(), 23, 0)
     assert np.array_equal(n.cpu().numpy(), want_n) and np.array_equal(out.cpu().numpy(), want_out)
+
+
+@pytest.mark.parametrize("dtype,V,B,t", [("bf16", 2049, 149, 1), ("fp32", 4096, 150, 1), ("bf16", 4098, 149, 2), ("bf16", 8192, 149, 1),   # 256 threads
+                                         ("fp32", 4097, 297, 1), ("bf16", 8193, 149, 2), ("fp32", 24576, 149, 1),     # a CTA of 1024
+                                         ("bf16", 24577, 149, 1)])                                                    # clusters of two
+def test_decisions_of_more_sequences_than_sms_match_oracle(lib, dtype, V, B, t):
+    p, q = inputs.make_accept_logits(B, t, V, seed=V + B, device="cuda", dtype=dtype)
+    p[0, :, V // 2:] = -float("inf")
+    q[1] = p[1, :t]                                                    # an all-zero residual, if it comes to one; else the bonus row
+    x = lib.hsd_draft_sample(q, 5, 0)
+    p_np, q_np, x_np = inputs.logits_to_numpy(p), inputs.logits_to_numpy(q), x.cpu().numpy()
+    out, n = lib.hsd_verify_level(1, p, q, x, 23, 0)
+    want_out, want_n = _oracle_verify(1, p_np, q_np, x_np, 23, 0)
+    assert np.array_equal(n.cpu().numpy(), want_n) and np.array_equal(out.cpu().numpy(), want_out)

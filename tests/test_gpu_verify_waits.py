@@ -49,9 +49,9 @@ def test_the_kernel_in_front_may_take_its_time(lib, waits, dtype, V, B, t):
     assert torch.equal(out, want[0]) and torch.equal(n, want[1])
 
 
-# decisions by clusters of several sizes; by a CTA a sequence (vocabularies past 131072)
+# decisions by clusters of several sizes, of 256 threads; by a CTA a sequence (many sequences, vocabularies past 131072)
 @pytest.mark.parametrize("groups", [1, 3])
-@pytest.mark.parametrize("dtype,V,B,t", [("bf16", 2048, 3, 2), ("bf16", 32000, 60, 2), ("fp32", 32001, 2, 0), ("bf16", 131080, 2, 1), ("fp32", 131073, 1, 1)])
+@pytest.mark.parametrize("dtype,V,B,t", [("bf16", 2050, 3, 2), ("bf16", 32000, 60, 2), ("fp32", 32001, 2, 0), ("bf16", 5000, 149, 1), ("fp32", 20000, 150, 1), ("bf16", 131080, 2, 1), ("fp32", 131073, 1, 1)])
 def test_a_wait_that_runs_out_is_reported(lib, waits, dtype, V, B, t, groups):
     p, q, x, _, out, n = _inputs(lib, B, t, V, dtype, 3)
     # statistics that a call before left behind: any would give a plausible decision
