@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) cluster_draw_kernel(c
 // The statistics of few rows: a cluster a row, each CTA consecutive tokens of it in registers; the maximum and the total cross the
 // cluster in one exchange each.  7 rows of 32000 bf16 tokens: 3.3 us (a CTA a row that takes them through its ring: 5.8).
 template <typename T, int PER, int NT, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) cluster_stats_kernel(const __grid_constant__ RowStatArgs a, int seg) {
+__global__ void __launch_bounds__(THREADS, (NT == 32 ? 512 : 1024) / THREADS) cluster_stats_kernel(const __grid_constant__ RowStatArgs a, int seg) {
   constexpr int NU = NT / PER, WARPS = THREADS / 32;
   __shared__ int wmax[WARPS], cmax[kClMaxC];                    // order keys
   __shared__ u64 wsum[WARPS], csum[kClMaxC];
@@ -843,7 +843,12 @@ static bool cluster_plan(const void *p, const void *q, int dtype, int V, int n, 
 //     fp32 32000: 4.1 / 26, 64 rows 6.6 / 28; 8000: 4.1 / 6.1; 2048: 3.9 / 3.9.  In more rounds, chunked: 32000, 100 rows 9.4 / 11.1, 148: 12.5 / 11.1
 //     (a row a CTA then), 200: 14.6 / 20.5, 512: 37 / 40, 16000, 512: 18 / 35; others: fp32 9001, 256: 12 / 9.1, 16000, 256: 11 / 16.9 (two CTAs a row),
 //     20000, 148: 13.4 / 10.7, 32000, 100: 10.2 / 28, 512: 41 / 105; 8000, 512: 10.7 / 15.9; bf16 32001, 256: 21 / 38.
-static bool cluster_pays_stats(const ClusterPlan &pl, long long rows) { return pl.threads < kClThreads || pl.C * rows <= 2 * kMeasuredSMs; }
+//   Rows of more than 65536 tokens (clusters of eight, 32 tokens a thread, one CTA an SM), up to four rounds: 128256 bf16, 1 row 22.4 -> 9, 16 rows
+//     26.5 -> 14.6, 48 rows 31.6 -> 21 to 24; 70001, 56 rows as fast, 64 34.6 -> 36.3.
+static bool cluster_plan_stats(const RowStatArgs &a, int dtype, int rows, ClusterPlan *pl) {
+  if (cluster_plan(a.p, a.q, dtype, a.V, rows, true, pl)) return pl->threads < kClThreads || (long long)pl->C * rows <= 2 * kMeasuredSMs;
+  return rows <= 4 * kClEights && cluster_plan(a.p, a.q, dtype, a.V, rows, false, pl);
+}
 //   decisions of more sequences than SMs by decide_kernel, two CTAs of 1024 threads a SM that read their rows through the first-level
 //     cache (the whole verification, clusters / decide_kernel): 12000 bf16 200 x 1 25.0 / 25.5; 16385, 200 x 0 29.7 / 16.9, 2000 x 3 655 / 293;
 //     24000, 149 x 3 42.3 / 44.5, 300 x 0 36 / 25, 2000 x 3 472 / 343, fp32 300 x 0 47 / 31, 2000 x 3 581 / 413; 32000 bf16, 300 x 1 60 / 66, fp32 50 / 90.  Up
@@ -933,7 +938,8 @@ static int launch_cluster_stats(const RowStatArgs &a, const ClusterPlan &pl, int
   HSD_CUDA_OK(pl.threads == 128   ? go(cluster_stats_kernel<T, PER, 8, 128>, 128)
               : pl.threads == 256 ? go(cluster_stats_kernel<T, PER, 8, 256>, 256)
               : pl.NT == 8        ? go(cluster_stats_kernel<T, PER, 8, kClThreads>, kClThreads)
-                                  : go(cluster_stats_kernel<T, PER, 16, kClThreads>, kClThreads));
+              : pl.NT == 16       ? go(cluster_stats_kernel<T, PER, 16, kClThreads>, kClThreads)
+                                  : go(cluster_stats_kernel<T, PER, 32, kClThreads>, kClThreads));
   hsd_count_launches(1);
   return HSD_OK;
 }
@@ -944,7 +950,7 @@ static int launch_cluster_stats(const RowStatArgs &a, const ClusterPlan &pl, int
 static int launch_row_stats(const RowStatArgs &a, int dtype, cudaStream_t s, bool *marks) {
   const long long n_items = (long long)a.batch * (2 * a.t_max + 1);
   ClusterPlan pl;
-  if (n_items <= 0x7FFFFFFFll / kClMaxC && cluster_plan(a.p, a.q, dtype, a.V, (int)n_items, true, &pl) && cluster_pays_stats(pl, n_items)) {
+  if (n_items <= 0x7FFFFFFFll / kClMaxC && cluster_plan_stats(a, dtype, (int)n_items, &pl)) {
     if (dtype == HSD_F32) return launch_cluster_stats<float, 1>(a, pl, (int)n_items, s);
     return pl.per == 2 ? launch_cluster_stats<__nv_bfloat16, 2>(a, pl, (int)n_items, s) : launch_cluster_stats<__nv_bfloat16, 1>(a, pl, (int)n_items, s);
   }

@@ -166,6 +166,8 @@ def test_cluster_draws_on_a_busy_gpu(lib, dtype, V, B):
                                                ("bf16", 114700, 31, 2, 3),     # twice through the ring, three groups, rows that begin anywhere
                                                ("fp32", 60000, 17, 2, 2),      # ... one group
                                                ("fp32", 57347, 1, 2, 0),       # clusters
+                                               ("bf16", 65537, 11, 2, 1), ("fp32", 128256, 4, 3, 0), ("bf16", 131072, 8, 3, 0), ("fp32", 131072, 19, 1, 1),   # 32 tokens a
+                                                                               # thread of a cluster up to 56 rows, the ring past them
                                                ("bf16", 131080, 2, 1, 0), ("fp32", 131081, 2, 1, 1),   # longer than the clusters of the decision take
                                                ("bf16", 5, 60, 2, 1), ("fp32", 3, 64, 2, 0), ("bf16", 64, 2, 40, 0),     # 128 threads; more drafts than lanes,
                                                ("fp32", 40, 1, 600, 2), ("bf16", 1024, 170, 3, 0), ("fp32", 1024, 3, 2, 1),   # ... than threads; every token
