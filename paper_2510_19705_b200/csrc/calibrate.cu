@@ -5,8 +5,8 @@
 //   1. alpha_stats_kernel:   per (model, position): reference exponent and sum of exp (fp32, fixed order, one read of the row)
 //   2. alpha_pairs_kernel:   per (position, <= 4096-token unit): every pair's sum of minima over the unit -> one partial per pair
 //   3. alpha_reduce_kernel:  per pair: the partials of all positions and units added in fixed order in fp64
-// The three are a chain of early launches, which itself starts under the end of what is on the stream: 100 positions of 24 models
-// over 2048 tokens 30 us (36 as ordinary launches), 20 of 5 over 17001 19 (24).
+// The three are a chain of launches, early where it pays, which itself starts under the end of what is on the stream: 100 positions
+// of 24 models over 2048 tokens 30 us (36 as ordinary launches), 20 of 5 over 17001 17 (18).
 // Deterministic (no atomics).  Model pairs are enumerated i < j, pair index = i L - i (i + 1) / 2 + (j - i - 1).
 #include <cuda_bf16.h>
 #include <math.h>
@@ -356,13 +356,13 @@ AlphaPlan alpha_plan(int L, int R, int V) {
 }
 
 template <typename T, bool VEC, int TILE>
-int launch_pairs(const T *logits, long long model_stride, int L, int R, int V, const AlphaPlan &p, const float2 *stats, float *partials, cudaStream_t s) {
+int launch_pairs(const T *logits, long long model_stride, int L, int R, int V, const AlphaPlan &p, const float2 *stats, float *partials, bool early, cudaStream_t s) {
   const int lpad = (L + 7) / 8 * 8;
   const size_t smem = (2 * (size_t)lpad * (TILE + 8) + 8 * 64) * sizeof(float);
   static std::atomic<u64> limits{0};
   const int limit = hsd_smem_limit((const void *)alpha_pairs_kernel<T, VEC, TILE>, 100 * 1024, limits);
   if (limit) return limit;
-  HSD_CUDA_OK(hsd_launch(alpha_pairs_kernel<T, VEC, TILE>, p.n_units * R, kAlphaThreads, smem, s, 0, true, logits, model_stride, L, R, V, p.unit, p.n_units,
+  HSD_CUDA_OK(hsd_launch(alpha_pairs_kernel<T, VEC, TILE>, p.n_units * R, kAlphaThreads, smem, s, 0, early, logits, model_stride, L, R, V, p.unit, p.n_units,
                          stats, partials));
   return HSD_OK;
 }
@@ -373,16 +373,21 @@ int launch_alpha_t(const T *logits, long long model_stride, int L, int R, int V,
   float2 *stats = (float2 *)((char *)ws + p.stats_off);
   float *partials = (float *)((char *)ws + p.partials_off);
   HSD_CUDA_OK(hsd_launch(alpha_stats_kernel<T, VEC>, dim3(R, L), kAlphaThreads, 0, s, 0, true, logits, model_stride, R, V, stats));
+  // CTAs that start early are packed on the SMs that the kernel before leaves first.  That costs more than the early start gives where
+  // there are no more of them than SMs (a CTA's own time then counts), unless both kernels' fit side by side, and, for more than eight
+  // models, in the reduction (us as ordinary launches / all early / this way: 32 models x 8 x 2048 13.2 / 16.6 / 12.6, x 32000 30.0 /
+  // 33.4 / 29.2; fp32 32 x 8 x 8192 14.6 / 19.1 / 14.3; 8 x 20 x 2048 8.2 / 8.5 / 7.7; 10 x 1 x 2048 8.1 / 7.0 / 7.0; behind many waves, 32 x
+  // 256 x 32000, the reduction takes the last one's places: 571 early, 568 not).
+  const long long n_ctas = (long long)p.n_units * R;
+  const bool fit = (long long)L * R + n_ctas <= kMeasuredSMs, pairs_early = fit || n_ctas > kMeasuredSMs,
+             reduce_early = fit || (pairs_early && L <= 8 && n_ctas <= 6 * kMeasuredSMs);
   int st = HSD_OK;
   if (p.n_pairs > 0)
-    st = L <= 8    ? launch_pairs<T, VEC, 1024>(logits, model_stride, L, R, V, p, stats, partials, s)
-         : L <= 16 ? launch_pairs<T, VEC, 512>(logits, model_stride, L, R, V, p, stats, partials, s)
-                   : launch_pairs<T, VEC, 256>(logits, model_stride, L, R, V, p, stats, partials, s);
+    st = L <= 8    ? launch_pairs<T, VEC, 1024>(logits, model_stride, L, R, V, p, stats, partials, pairs_early, s)
+         : L <= 16 ? launch_pairs<T, VEC, 512>(logits, model_stride, L, R, V, p, stats, partials, pairs_early, s)
+                   : launch_pairs<T, VEC, 256>(logits, model_stride, L, R, V, p, stats, partials, pairs_early, s);
   if (st) return st;
-  // (behind more than two waves of pairs the reduction's waiting CTAs take the last wave's places: 32 models x 256 x 32000 571 us
-  // early, 568 not, 32 x 16 54.1 / 52.8; 5 x 20 x 17001, one wave and a half, 18.7 / 21.9)
-  const bool early = p.n_units * R <= 2 * (L <= 8 ? 3 : 2) * kMeasuredSMs;
-  HSD_CUDA_OK(hsd_launch(alpha_reduce_kernel, p.n_pairs > 0 ? min(p.n_pairs, 4 * kMeasuredSMs) : 1, kAlphaThreads, 0, s, 0, early, partials, L, R * p.n_units, R,
+  HSD_CUDA_OK(hsd_launch(alpha_reduce_kernel, p.n_pairs > 0 ? min(p.n_pairs, 4 * kMeasuredSMs) : 1, kAlphaThreads, 0, s, 0, reduce_early, partials, L, R * p.n_units, R,
                          alpha));
   hsd_count_launches(p.n_pairs > 0 ? 3 : 2);
   return hsd_launch_status();
