@@ -209,9 +209,9 @@ alpha_pairs_kernel(const T *__restrict__ logits, long long model_stride, int L, 
     const bool far = __float_as_int(v.y) < 0;
     st[tid] = make_float4(far ? 1.f : kLog2e, v.x, tid < L ? 1.f / fabsf(v.y) : 0.f, 0.f);
   };
-  // bf16: the first logits are asked for ahead of the statistics' end (24 models x 256 x 32000 434 us instead of 451; fp32, with
-  // twice the registers for them, 538 instead of 531)
-  constexpr bool AHEAD = sizeof(T) == 2;
+  // bf16 in vectors: the first logits are asked for ahead of the statistics' end (24 models x 256 x 32000 434 us instead of 451; fp32,
+  // with twice the registers for them, 538 instead of 531; single bf16 logits, 16 x 256 x 13001, 152 instead of 147)
+  constexpr bool AHEAD = sizeof(T) == 2 && VEC;
   if constexpr (!AHEAD) { load_stats(); __syncthreads(); }
   // staging: TPM threads per model; vector i of a thread = tokens (TPM i + tid % TPM) N ..
   constexpr int N = VEC ? AlphaVec<T>::N : 1, TPM = TILE / 32, NV = 32 / N;
