@@ -15,6 +15,8 @@ vp, i32, u64 = ctypes.c_void_p, ctypes.c_int, ctypes.c_uint64
 
 @pytest.fixture(scope="module")
 def waits(tmp_path_factory):
+    if not os.path.exists(build.NVCC):
+        pytest.skip("no nvcc")
     out = str(tmp_path_factory.mktemp("native") / "verify_waits.so")
     src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "native", "verify_waits.cu")
     subprocess.run([build.NVCC] + build.FLAGS + ["-DHSD_WAIT_LIMIT_NS=1000000ull", "-shared", "-o", out, src], check=True)
